@@ -125,8 +125,11 @@ def prepare(case, seed):
             Wg[:n_gate] = -case["gamma"] * 1.1 * torch.log(torch.arange(1, n_gate + 1, device="cuda", dtype=torch.float32))
     s.update(x=x.to(adt), Wg=Wg, Wnoise=normal(S.wg_elems, std=d ** -0.5))
     s["noise"] = normal(S.logits_elems) if train else torch.zeros(S.logits_elems, device="cuda")
-    s.update(W1=normal(n, d, h, std=d ** -0.5, dtype=adt), b1=torch.zeros(n, h, device="cuda", dtype=adt),
-             W2=normal(n, h, d, std=h ** -0.5, dtype=adt), b2=torch.zeros(n, d, device="cuda", dtype=adt))
+    # biases 0 as in the workloads, but those of a model in training (the optimiser divides a gradient by its own size, so
+    # that a bias of 0 would become nothing but the sign of a sum that may be close to 0)
+    std_b = 0.02 if kind == "layer" else 0.0
+    s.update(W1=normal(n, d, h, std=d ** -0.5, dtype=adt), b1=normal(n, h, std=std_b, dtype=adt),
+             W2=normal(n, h, d, std=h ** -0.5, dtype=adt), b2=normal(n, d, std=std_b, dtype=adt))
     s.update(y=empty(T, d, dtype=adt), ws=B.empty_bytes(max(S.ws_bytes, S.ws_fwd_bytes, S.ws_bwd_bytes if train else 0)))
     if kind != "balanced":
         s.update(losses=empty(2), importance=empty(n), load=empty(S.load_elems), counts=empty(n, dtype=torch.int32),
@@ -216,3 +219,128 @@ def tolerance(case):
     if case["act"] == "f32":
         return {"rel": 1e-5, "max": 1e-4}
     return {"rel": 1e-2, "max": 0.6}
+
+
+def exact(case, seed):
+    """The results of `run` on these inputs in 64 bits: the layer's equations in plain torch, experts one after the other
+    and differentiated by hand, the gate differentiated by autograd. Whole numbers (counts, masks, row lists) are left out:
+    a routing decision between logits closer than float's resolution may fall the other way here."""
+    s = prepare(case, seed)
+    T, d, h, n, k, a, k1, b, k2 = (case[q] for q in ("T", "d", "h", "n", "k", "a", "k1", "b", "k2"))
+    kind, f64, dev = case["kind"], torch.float64, "cuda"
+    train = kind != "forward"
+    x = s["x"].to(f64).requires_grad_(train)
+    Wg = s["Wg"].to(f64).requires_grad_(train)
+    Wn = s["Wnoise"].to(f64).requires_grad_(train and kind != "balanced")
+    noise = s["noise"].to(f64)
+
+    def cv2(v):
+        return v.var(unbiased=False) / v.mean() ** 2
+
+    def noisy_gate(x_, Wg_, Wn_, eps, kk):
+        """gates and columns of the kk kept experts, P(x, i) of every column"""
+        cols = Wg_.shape[1]
+        clean, sigma = x_ @ Wg_, torch.nn.functional.softplus(x_ @ Wn_, threshold=700.0)
+        H = clean + eps.view(-1, cols) * sigma
+        top, idx = H.topk(min(kk + 1, cols), dim=1)
+        if kk < cols:
+            kept = torch.zeros_like(H, dtype=torch.bool).scatter_(1, idx[:, :kk], True)
+            P = torch.special.ndtr((clean - torch.where(kept, top[:, kk:kk + 1], top[:, kk - 1:kk])) / sigma)
+        else:
+            P = torch.ones_like(H)
+        return torch.softmax(top[:, :kk], dim=1), idx[:, :kk], P
+
+    out = {}
+    if kind == "balanced":  # rows: expert-major, every expert's m most probable tokens in ascending order
+        m = T * k // n
+        probs = torch.softmax(x @ Wg.view(d, n), dim=1)
+        tok = probs.detach().topk(m, dim=0).indices.sort(dim=0).values.t().reshape(-1)
+        expert = torch.arange(n, device=dev).repeat_interleave(m)
+        mask = torch.zeros(T, n, device=dev, dtype=f64)
+        mask[tok, expert] = 1.0
+        above = (probs.detach() > s["thr"].to(f64)).to(f64)
+        gate = probs[tok, expert] / (probs * mask).sum(1)[tok]
+        loss = ((above - mask) * (probs - s["thr"].to(f64))).sum()
+        bounds = [e * m for e in range(n + 1)]
+        out.update(loss=loss.detach().view(1), probs=probs.detach(), dthr=m - above.sum(0))
+    else:
+        if a:
+            lp, wp = T * a, d * a
+            g_p, i_p, P_p = noisy_gate(x, Wg[:wp].view(d, a), Wn[:wp].view(d, a), noise[:lp], k1)
+            slot_of, group = torch.arange(T * k1, device=dev), i_p.reshape(-1)
+            parts, load_i = [], []
+            for i in range(a):
+                rows = slot_of[group == i]
+                w = slice(wp + i * d * b, wp + (i + 1) * d * b)
+                g, c, P = noisy_gate(x[rows // k1], Wg[w].view(d, b), Wn[w].view(d, b), noise[lp:].view(T * k1, b)[rows], k2)
+                parts.append((rows, g, c + i * b))
+                load_i.append(P.sum(0))
+            order = torch.cat([p[0] for p in parts]).argsort()
+            G = (g_p.reshape(-1, 1) * torch.cat([p[1] for p in parts])[order]).reshape(T, k)
+            idx = torch.cat([p[2] for p in parts])[order].reshape(T, k)
+            load_p, load_i = P_p.sum(0), torch.stack(load_i)
+            sizes = torch.bincount(group, minlength=a).to(f64)
+            load_h = (load_p.view(a, 1) * load_i / sizes.clamp(min=1.0).view(a, 1)).reshape(-1)
+            load = torch.cat([load_h, load_p, load_i.reshape(-1), sizes])
+        else:
+            G, idx, P = noisy_gate(x, Wg.view(d, n), Wn.view(d, n), noise, k)
+            load_h = load = P.sum(0)
+        imp = torch.zeros(n, device=dev, dtype=f64).index_add(0, idx.reshape(-1), G.reshape(-1))
+        losses = torch.stack([0.1 * cv2(imp), 0.1 * cv2(load_h)])
+        loss = losses.sum()
+        order = idx.reshape(-1).argsort(stable=True)
+        tok, gate = order // k, G.reshape(-1)[order]
+        bounds = [0] + torch.bincount(idx.reshape(-1), minlength=n).cumsum(0).tolist()
+        out.update(losses=losses.detach(), importance=imp.detach(), load=load.detach())
+    xd, g = x.detach(), gate.detach().view(-1, 1)
+    W = [s[q] for q in ("W1", "b1", "W2", "b2")]
+
+    def expert_forward(e):
+        w1, b1, w2, b2 = (w[e].to(f64) for w in W)
+        xe = xd[tok[bounds[e]:bounds[e + 1]]]
+        he = torch.relu(xe @ w1 + b1)
+        return xe, he, w1, w2, he @ w2 + b2
+
+    ys = torch.cat([expert_forward(e)[4] for e in range(n) if bounds[e] < bounds[e + 1]])
+    y = torch.zeros(T, d, device=dev, dtype=f64).index_add(0, tok, g * ys)
+    out["y"] = y
+    if not train:
+        return {q: out.get(q) for q in ("y", "losses", "importance", "load", "counts")}
+    dY = s["dY"].to(f64)
+    dy = dY
+    if kind == "layer":
+        bits = (s["keep"].view(T, d // 8, 1) >> torch.arange(8, device=dev, dtype=torch.uint8)) & 1
+        keep, sig = bits.view(T, d).to(f64) / (1.0 - DROP_PROB), torch.sigmoid(y)
+        out["y"], dy = xd + keep * sig, dY * keep * sig * (1.0 - sig)
+    gdt = f64 if n * d * h < 2 ** 28 else torch.float32  # 64-bit sums held in 32 bits where they would fill the card
+    grads = {q: torch.zeros(s[q].shape, device=dev, dtype=gdt) for q in ("dW1", "db1", "dW2", "db2")}
+    dx, dgate = torch.zeros_like(xd), (dy[tok] * ys).sum(1)
+    for e in range(n):
+        rows = slice(bounds[e], bounds[e + 1])
+        if bounds[e] == bounds[e + 1]:
+            continue
+        xe, he, w1, w2, _ = expert_forward(e)
+        de = g[rows] * dy[tok[rows]]
+        dz = (de @ w2.t()) * (he > 0)
+        grads["dW1"][e], grads["db1"][e], grads["dW2"][e], grads["db2"][e] = xe.t() @ dz, dz.sum(0), he.t() @ de, de.sum(0)
+        dx.index_add_(0, tok[rows], dz @ w1.t())
+    (loss + (gate * dgate).sum()).backward()
+    out.update(grads, dX=dx + x.grad + (dY if kind == "layer" else 0.0), dWg=Wg.grad.view(-1))
+    if kind == "balanced":
+        return {q: out.get(q) for q in ("y", "loss", "probs", "mask_bits", "tok_of_row", "thr_counts", "dX", "dWg", "dW1", "db1",
+                                        "dW2", "db2", "dthr")}
+    out["dWnoise"] = Wn.grad.view(-1)
+    if kind == "step":
+        return {q: out.get(q) for q in ("y", "losses", "importance", "load", "counts", "dX", "dWg", "dWnoise", "dW1", "db1",
+                                        "dW2", "db2")}
+    rows, cols, full = [], [], []  # the first optimiser step: factored second moments, full ones for the biases
+    for wq, bq in (("W1", "b1"), ("W2", "b2")):
+        gw, gb = grads["d" + wq].to(f64), grads["d" + bq].to(f64)
+        r, c, v = ((1.0 - BETA2) * (gw ** 2).mean(2), (1.0 - BETA2) * (gw ** 2).mean(1), (1.0 - BETA2) * gb ** 2)
+        vh = r.unsqueeze(2) * c.unsqueeze(1) / r.mean(1).clamp(min=1e-300).view(n, 1, 1) / (1.0 - BETA2)
+        out[wq] = s[wq].to(f64) - LR * gw / (vh.sqrt() + EPS)
+        out[bq] = s[bq].to(f64) - LR * gb / ((v / (1.0 - BETA2)).sqrt() + EPS)
+        rows.append(r), cols.append(c), full.append(v)
+    out["adam"] = torch.cat([q.reshape(-1) for q in (rows[0], cols[0], rows[1], cols[1], full[0], full[1])])
+    return {q: out.get(q) for q in ("y", "losses", "importance", "load", "counts", "dX", "dWg", "dWnoise", "W1", "b1", "W2", "b2",
+                                    "adam")}
