@@ -243,13 +243,15 @@ struct LossesBwdWs {
     }
 };
 
+int64_t gate_weight_grads_part(const Dims &D, int64_t cols);  // floats of scratch of gate_weight_grads
+
 struct GateBwdWs {
-    float *dclean, *draw, *partials, *dX_sec, *partials_s;
+    float *dlogit, *dlogit_s, *partials, *dX_sec, *partials_s;  // dlogit rows: (clean | raw noise) columns
     void *dsplit, *wsplit, *dsplit_s, *wsplit_s, *xs_p;
     bool tc, tc_hier;
     HierIdxWs H;
     GateBwdWs(Carver &cv, const Dims &D) : H(cv, D) {
-        dclean = draw = partials = dX_sec = partials_s = nullptr;
+        dlogit = dlogit_s = partials = dX_sec = partials_s = nullptr;
         dsplit = wsplit = dsplit_s = wsplit_s = xs_p = nullptr;
         if (D.hier) dX_sec = cv.take<float>(D.T * D.k1 * D.d);
         tc = !D.hier && tc_gate_bwd_supported(D.act, (int32_t)D.d, (int32_t)D.n);
@@ -267,8 +269,13 @@ struct GateBwdWs {
             wsplit = cv.take<bf16>(D.d * 6 * D.n);
             partials = cv.take<float>(tc_gate_bwd_partials(D.T, (int32_t)D.d, (int32_t)D.n));
         } else {
-            dclean = cv.take<float>(D.logits);
-            draw = cv.take<float>(D.logits);
+            const int64_t n1 = D.hier ? D.a : D.n, P1 = D.T * D.k1;
+            dlogit = cv.take<float>(D.T * 2 * n1);
+            partials = cv.take<float>(gate_weight_grads_part(D, 2 * n1));
+            if (D.hier) {
+                dlogit_s = cv.take<float>(P1 * 2 * D.b);
+                partials_s = cv.take<float>(simt_wgrad_splits(D.d, 2 * D.b, (int32_t)D.a, P1) * D.a * D.d * 2 * D.b);
+            }
         }
     }
 };
@@ -419,13 +426,13 @@ int32_t do_expert_ffn(const moe_config *c, const Dims &D, const void *xs, const 
         return launch_tc_ffn(*c, xs, offsets, W1, b1, W2, b2, hid, ys, w.tc, status_word(ws_base), st, first_only, relu_bits);
     SimtGemm g = base_gemm(D);  // hid = relu(xs.W1 + b1)
     g.A = xs; g.B = W1; g.C = hid; g.bias = b1; g.relu = 1;
-    g.sa_i = D.d; g.sa_k = 1; g.sb_k = D.h; g.sb_j = 1; g.sc_i = D.h; g.sc_j = 1;
+    g.sa_i = D.d; g.sa_k = 1; g.sb_k = D.h; g.sb_j = 1; g.sc_i = D.h;
     g.mode = 0; g.offsets = offsets; g.nseg = (int32_t)D.n; g.M = D.R; g.N = D.h; g.K = D.d; g.b_e = D.d * D.h;
     MOE_TRY(launch_simt_gemm(g, w.tile_prefix, st));
     if (first_only) return MOE_OK;
     g = base_gemm(D);  // ys = hid.W2 + b2
     g.A = hid; g.B = W2; g.C = ys; g.bias = b2;
-    g.sa_i = D.h; g.sa_k = 1; g.sb_k = D.d; g.sb_j = 1; g.sc_i = D.d; g.sc_j = 1;
+    g.sa_i = D.h; g.sa_k = 1; g.sb_k = D.d; g.sb_j = 1; g.sc_i = D.d;
     g.mode = 0; g.offsets = offsets; g.nseg = (int32_t)D.n; g.M = D.R; g.N = D.d; g.K = D.h; g.b_e = D.h * D.d;
     return launch_simt_gemm(g, w.tile_prefix, st);
 }
@@ -472,23 +479,23 @@ int32_t do_expert_ffn_bwd(const moe_config *c, const Dims &D, const void *xs, co
     MOE_TRY(launch_segment_colsum(dys, D.act, offsets, n, D.R, (int32_t)D.d, db2, w.colsum, w.tile_prefix, st));
     SimtGemm g = base_gemm(D);  // dW2[e] = hid_e^T . dys_e
     g.A = hid; g.B = dys; g.C = dW2;
-    g.sa_i = 1; g.sa_k = D.h; g.sb_k = D.d; g.sb_j = 1; g.sc_i = D.d; g.sc_j = 1;
+    g.sa_i = 1; g.sa_k = D.h; g.sb_k = D.d; g.sb_j = 1; g.sc_i = D.d;
     g.mode = 1; g.offsets = offsets; g.nseg = n; g.M = D.h; g.N = D.d; g.c_e = D.h * D.d;
     MOE_TRY(launch_simt_gemm(g, w.tile_prefix, st));
     g = base_gemm(D);  // dz = (dys . W2[e]^T) * [hid > 0]
     g.A = dys; g.B = W2; g.C = w.dz; g.mask = hid;
-    g.sa_i = D.d; g.sa_k = 1; g.sb_k = 1; g.sb_j = D.d; g.sc_i = D.h; g.sc_j = 1;
+    g.sa_i = D.d; g.sa_k = 1; g.sb_k = 1; g.sb_j = D.d; g.sc_i = D.h;
     g.mode = 0; g.offsets = offsets; g.nseg = n; g.M = D.R; g.N = D.h; g.K = D.d; g.b_e = D.h * D.d;
     MOE_TRY(launch_simt_gemm(g, w.tile_prefix, st));
     MOE_TRY(launch_segment_colsum(w.dz, D.act, offsets, n, D.R, (int32_t)D.h, db1, w.colsum, w.tile_prefix, st));
     g = base_gemm(D);  // dW1[e] = xs_e^T . dz_e
     g.A = xs; g.B = w.dz; g.C = dW1;
-    g.sa_i = 1; g.sa_k = D.d; g.sb_k = D.h; g.sb_j = 1; g.sc_i = D.h; g.sc_j = 1;
+    g.sa_i = 1; g.sa_k = D.d; g.sb_k = D.h; g.sb_j = 1; g.sc_i = D.h;
     g.mode = 1; g.offsets = offsets; g.nseg = n; g.M = D.d; g.N = D.h; g.c_e = D.d * D.h;
     MOE_TRY(launch_simt_gemm(g, w.tile_prefix, st));
     g = base_gemm(D);  // dxs = dz . W1[e]^T
     g.A = w.dz; g.B = W1; g.C = dxs;
-    g.sa_i = D.h; g.sa_k = 1; g.sb_k = 1; g.sb_j = D.h; g.sc_i = D.d; g.sc_j = 1;
+    g.sa_i = D.h; g.sa_k = 1; g.sb_k = 1; g.sb_j = D.h; g.sc_i = D.d;
     g.mode = 0; g.offsets = offsets; g.nseg = n; g.M = D.R; g.N = D.d; g.K = D.h; g.b_e = D.d * D.h;
     return launch_simt_gemm(g, w.tile_prefix, st);
 }
@@ -505,25 +512,28 @@ int32_t do_losses_bwd(const moe_config *c, const Dims &D, const float *importanc
     return launch_load_h_bwd(load, w.dload_h, (int32_t)D.a, (int32_t)D.b, dload, st);
 }
 
-// dW = x^T . dlogit [d, n];  dX (+)= dlogit . W^T [T, d]
-int32_t gate_weight_grads(const Dims &D, const void *x, const float *dlogit, const float *W, int64_t n,
-                          float *dW, float *dX, bool accumulate, cudaStream_t st) {
+// dW = x^T . dlogit [d, n], dX = dlogit . W^T [T, d], with dlogit [T, cols] (cols = n, or 2n columns of [W_g | W_noise], whose
+// two halves then are W / W2 and dW / dW2)
+int32_t gate_weight_grads(const Dims &D, const void *x, const float *dlogit, const float *W, const float *W2, int64_t n,
+                          float *dW, float *dW2, float *dX, float *part, cudaStream_t st) {
+    const int64_t cols = W2 ? 2 * n : n;
     SimtGemm g;
     memset(&g, 0, sizeof(g));
     g.a_row_div = 1;
     g.ta = D.act == MOE_BF16 ? G_BF16 : G_F32; g.tb = G_F32; g.tc = G_F32;
-    g.A = x; g.B = dlogit; g.C = dW;
-    g.sa_i = 1; g.sa_k = D.d; g.sb_k = n; g.sb_j = 1; g.sc_i = n; g.sc_j = 1;
-    g.mode = 1; g.offsets = nullptr; g.nseg = 1; g.M = D.d; g.N = n; g.K = D.T;
-    MOE_TRY(launch_simt_gemm(g, nullptr, st));
+    g.A = x; g.B = dlogit; g.C = dW; g.C2 = dW2; g.c_split = n;
+    g.sa_i = 1; g.sa_k = D.d; g.sb_k = cols; g.sb_j = 1; g.sc_i = n;
+    g.mode = 1; g.offsets = nullptr; g.nseg = 1; g.M = D.d; g.N = cols; g.K = D.T;
+    MOE_TRY(launch_simt_gemm(g, nullptr, st, part));
     memset(&g, 0, sizeof(g));
     g.a_row_div = 1;
     g.ta = g.tb = g.tc = G_F32;
-    g.A = dlogit; g.B = W; g.C = dX; g.accumulate = accumulate ? 1 : 0;
-    g.sa_i = n; g.sa_k = 1; g.sb_k = 1; g.sb_j = n; g.sc_i = D.d; g.sc_j = 1;
-    g.mode = 0; g.offsets = nullptr; g.nseg = 1; g.M = D.T; g.N = D.d; g.K = n;
+    g.A = dlogit; g.B = W; g.B2 = W2; g.b_split = n; g.b_k_contiguous = 1; g.C = dX;
+    g.sa_i = cols; g.sa_k = 1; g.sb_k = 1; g.sb_j = n; g.sc_i = D.d;
+    g.mode = 0; g.offsets = nullptr; g.nseg = 1; g.M = D.T; g.N = D.d; g.K = cols;
     return launch_simt_gemm(g, nullptr, st);
 }
+int64_t gate_weight_grads_part(const Dims &D, int64_t cols) { return simt_wgrad_splits(D.d, cols, 1, D.T) * D.d * cols; }
 
 int32_t do_gate_bwd(const moe_config *c, const Dims &D, const void *x, const float *Wg, const float *Wnoise,
                     const float *noise, const float *clean, const float *raw_noise, const int32_t *topk_idx,
@@ -535,20 +545,18 @@ int32_t do_gate_bwd(const moe_config *c, const Dims &D, const void *x, const flo
         const int64_t P1 = D.T * D.k1, lp = D.T * D.a, wp = D.d * D.a;
         const float *g_p = gates + D.T * D.k, *g_s = g_p + P1;
         float *dg_p = dgates + D.T * D.k, *dg_s = dg_p + P1;
-        float *dc_p = w.dclean, *dr_p = w.draw, *dc_s = w.dclean + lp, *dr_s = w.draw + lp;
         MOE_TRY(w.H.build(D, topk_idx, st));
         MOE_TRY(launch_hier_gate_product_bwd(gates, dgates, D.T, (int32_t)D.k1, (int32_t)D.k2, st));
         if (w.tc_hier) {
             // both levels on the tensor cores: split logit gradients (the secondary ones written in the
             // order sorted by primary group), grouped products, then the slots' rows are added per token
             MOE_TRY(launch_gate_logit_grads(noise, clean, raw_noise, w.H.idx_p, g_p, kth_vals, kth_idx, dg_p, dload,
-                                            nullptr, D.T, (int32_t)D.a, (int32_t)D.k1, nullptr, nullptr, w.dsplit,
-                                            nullptr, st));
+                                            nullptr, D.T, (int32_t)D.a, (int32_t)D.k1, nullptr, w.dsplit, nullptr, st));
             MOE_TRY(launch_tc_gate_bwd(x, D.T, (int32_t)D.d, (int32_t)D.a, Wg, Wnoise, w.dsplit, w.wsplit, w.partials,
                                        dWg, dWnoise, dX_gate, status_word(ws_base), st, D.flags));
             MOE_TRY(launch_gate_logit_grads(noise + lp, clean + lp, raw_noise + lp, w.H.idx_s, g_s, kth_vals + 2 * D.T,
                                             kth_idx + 2 * D.T, dg_s, dload + D.a, w.H.idx_p, P1, (int32_t)D.b,
-                                            (int32_t)D.k2, nullptr, nullptr, w.dsplit_s, w.H.inv_perm_p, st));
+                                            (int32_t)D.k2, nullptr, w.dsplit_s, w.H.inv_perm_p, st));
             MOE_TRY(launch_dispatch_rows(x, D.act, D.T, (int32_t)D.k1, (int32_t)D.d, w.H.inv_perm_p, w.xs_p, st));
             MOE_TRY(launch_tc_hier_secondary_bwd(w.xs_p, w.dsplit_s, w.wsplit_s, Wg + wp, Wnoise + wp, w.H.offsets_p,
                                                  w.H.tile_prefix, (int32_t)D.a, P1, (int32_t)D.d, (int32_t)D.b,
@@ -559,44 +567,36 @@ int32_t do_gate_bwd(const moe_config *c, const Dims &D, const void *x, const flo
         }
         // primary gate (Eq. 12: G_primary), rows = tokens
         MOE_TRY(launch_gate_logit_grads(noise, clean, raw_noise, w.H.idx_p, g_p, kth_vals, kth_idx, dg_p, dload,
-                                        nullptr, D.T, (int32_t)D.a, (int32_t)D.k1, dc_p, dr_p, nullptr, nullptr, st));
-        MOE_TRY(gate_weight_grads(D, x, dc_p, Wg, D.a, dWg, dX_gate, false, st));
-        MOE_TRY(gate_weight_grads(D, x, dr_p, Wnoise, D.a, dWnoise, dX_gate, true, st));
+                                        nullptr, D.T, (int32_t)D.a, (int32_t)D.k1, w.dlogit, nullptr, nullptr, st));
+        MOE_TRY(gate_weight_grads(D, x, w.dlogit, Wg, Wnoise, D.a, dWg, dWnoise, dX_gate, w.partials, st));
         // secondary gates G_i, rows = slots (t, s1); dLoad_i of the row's group
         MOE_TRY(launch_gate_logit_grads(noise + lp, clean + lp, raw_noise + lp, w.H.idx_s, g_s, kth_vals + 2 * D.T,
                                         kth_idx + 2 * D.T, dg_s, dload + D.a, w.H.idx_p, P1, (int32_t)D.b,
-                                        (int32_t)D.k2, dc_s, dr_s, nullptr, nullptr, st));
-        for (int part = 0; part < 2; ++part) {
-            const float *dl = part == 0 ? dc_s : dr_s;
-            const float *W = (part == 0 ? Wg : Wnoise) + wp;
-            float *dW = (part == 0 ? dWg : dWnoise) + wp;
-            SimtGemm g;  // dW_s[i] = sum over the slots of group i of x[token]^T . dlogit[slot]
-            memset(&g, 0, sizeof(g));
-            g.ta = D.act == MOE_BF16 ? G_BF16 : G_F32; g.tb = G_F32; g.tc = G_F32;
-            g.A = x; g.B = dl; g.C = dW;
-            g.sa_i = 1; g.sa_k = D.d; g.sb_k = D.b; g.sb_j = 1; g.sc_i = D.b; g.sc_j = 1;
-            g.mode = 1; g.offsets = w.H.offsets_p; g.nseg = (int32_t)D.a; g.M = D.d; g.N = D.b; g.c_e = D.d * D.b;
-            g.a_row_index = w.H.perm_p; g.a_row_div = (int32_t)D.k1; g.b_row_index = w.H.perm_p;
-            MOE_TRY(launch_simt_gemm(g, w.H.tile_prefix, st));
-            memset(&g, 0, sizeof(g));  // dX_sec[slot] (+)= dlogit[slot] . W_s[group]^T
-            g.ta = g.tb = g.tc = G_F32;
-            g.A = dl; g.B = W; g.C = w.dX_sec; g.accumulate = part;
-            g.sa_i = D.b; g.sa_k = 1; g.sb_k = 1; g.sb_j = D.b; g.sc_i = D.d; g.sc_j = 1;
-            g.mode = 0; g.offsets = w.H.offsets_p; g.nseg = (int32_t)D.a; g.M = P1; g.N = D.d; g.K = D.b;
-            g.b_e = D.d * D.b;
-            g.a_row_index = w.H.perm_p; g.a_row_div = 1; g.c_row_index = w.H.perm_p;
-            MOE_TRY(launch_simt_gemm(g, w.H.tile_prefix, st));
-        }
+                                        (int32_t)D.k2, w.dlogit_s, nullptr, nullptr, st));
+        SimtGemm g;  // dW_s[i] = sum over the slots of group i of x[token]^T . dlogit[slot]
+        memset(&g, 0, sizeof(g));
+        g.ta = D.act == MOE_BF16 ? G_BF16 : G_F32; g.tb = G_F32; g.tc = G_F32;
+        g.A = x; g.B = w.dlogit_s; g.C = dWg + wp; g.C2 = dWnoise + wp; g.c_split = D.b;
+        g.sa_i = 1; g.sa_k = D.d; g.sb_k = 2 * D.b; g.sb_j = 1; g.sc_i = D.b;
+        g.mode = 1; g.offsets = w.H.offsets_p; g.nseg = (int32_t)D.a; g.M = D.d; g.N = 2 * D.b; g.K = P1; g.c_e = D.d * D.b;
+        g.a_row_index = w.H.perm_p; g.a_row_div = (int32_t)D.k1; g.b_row_index = w.H.perm_p;
+        MOE_TRY(launch_simt_gemm(g, w.H.tile_prefix, st, w.partials_s));
+        memset(&g, 0, sizeof(g));  // dX_sec[slot] = dlogit[slot] . [W_g | W_noise]_s[group]^T
+        g.ta = g.tb = g.tc = G_F32;
+        g.A = w.dlogit_s; g.B = Wg + wp; g.B2 = Wnoise + wp; g.b_split = D.b; g.b_k_contiguous = 1; g.C = w.dX_sec;
+        g.sa_i = 2 * D.b; g.sa_k = 1; g.sb_k = 1; g.sb_j = D.b; g.sc_i = D.d;
+        g.mode = 0; g.offsets = w.H.offsets_p; g.nseg = (int32_t)D.a; g.M = P1; g.N = D.d; g.K = 2 * D.b;
+        g.b_e = D.d * D.b;
+        g.a_row_index = w.H.perm_p; g.a_row_div = 1; g.c_row_index = w.H.perm_p;
+        MOE_TRY(launch_simt_gemm(g, w.H.tile_prefix, st));
         return launch_add_slot_rows(w.dX_sec, D.T, (int32_t)D.k1, (int32_t)D.d, dX_gate, st);
     }
     MOE_TRY(launch_gate_logit_grads(noise, clean, raw_noise, topk_idx, gates, kth_vals, kth_idx, dgates, dload,
-                                    nullptr, D.T, (int32_t)D.n, (int32_t)D.k, w.dclean, w.draw, w.dsplit, nullptr,
-                                    st));
+                                    nullptr, D.T, (int32_t)D.n, (int32_t)D.k, w.dlogit, w.dsplit, nullptr, st));
     if (w.tc)
         return launch_tc_gate_bwd(x, D.T, (int32_t)D.d, (int32_t)D.n, Wg, Wnoise, w.dsplit, w.wsplit, w.partials, dWg,
                                   dWnoise, dX_gate, status_word(ws_base), st, D.flags);
-    MOE_TRY(gate_weight_grads(D, x, w.dclean, Wg, D.n, dWg, dX_gate, false, st));
-    return gate_weight_grads(D, x, w.draw, Wnoise, D.n, dWnoise, dX_gate, true, st);
+    return gate_weight_grads(D, x, w.dlogit, Wg, Wnoise, D.n, dWg, dWnoise, dX_gate, w.partials, st);
 }
 
 }  // namespace
@@ -980,6 +980,7 @@ int32_t moe_query_balanced_sizes(const moe_config *cfg, moe_balanced_sizes *out)
         cv.take<bf16>((int64_t)cfg->T * 3 * cfg->n); cv.take<bf16>((int64_t)cfg->d * 3 * cfg->n);
         cv.take<float>(tc_gate_bwd_partials(cfg->T, cfg->d, cfg->n / 2 > 0 ? cfg->n / 2 : 1));
         cv.take<float>((int64_t)cfg->T * cfg->n);
+        cv.take<float>(gate_weight_grads_part(dims_of(cfg), cfg->n));
     });
     out->ws_bytes = kWsHeader + (fwd > bwd ? fwd : bwd);
     return MOE_OK;
@@ -1048,14 +1049,14 @@ int32_t moe_gate_balanced_bwd(const moe_config *cfg, const void *x, const float 
         return launch_tc_gate_bwd(x, D.T, (int32_t)D.d, half, Wg, Wg + half, dsplit, wsplit, partials, dWg, dWg + half, dX_gate,
                                   status_word(ws), st, D.flags, (int32_t)D.n);
     }
-    float *dc = cv.take<float>(D.T * D.n);
+    float *dc = cv.take<float>(D.T * D.n), *part = cv.take<float>(gate_weight_grads_part(D, D.n));
     MOE_TRY(launch_balanced_gate_bwd(probs, mask_bits, den, thresholds, tok_ptr, tok_rows, dG_row, thr_counts, w_batchwise,
                                      D.T, (int32_t)D.n, (int32_t)(D.R / D.n), dc, nullptr, dthresholds, st));
     if (D.T == 0) {
         MOE_CUDA(cudaMemsetAsync(dWg, 0, sizeof(float) * D.d * D.n, st));
         return MOE_OK;
     }
-    return gate_weight_grads(D, x, dc, Wg, D.n, dWg, dX_gate, false, st);
+    return gate_weight_grads(D, x, dc, Wg, nullptr, D.n, dWg, nullptr, dX_gate, part, st);
 }
 
 int32_t moe_dispatch_balanced_bwd(const moe_config *cfg, const void *dxs, const int32_t *tok_ptr,

@@ -18,8 +18,7 @@ __global__ void __launch_bounds__(256) gate_logit_grads_kernel(
     const float *__restrict__ noise, const float *__restrict__ clean, const float *__restrict__ raw,
     const int32_t *__restrict__ idx, const float *__restrict__ gates, const float *__restrict__ kth_vals,
     const int32_t *__restrict__ kth_idx, const float *__restrict__ dgates, const float *__restrict__ dload,
-    const int32_t *__restrict__ dload_row_group, int64_t rows, int32_t n, int32_t k, float *__restrict__ dclean,
-    float *__restrict__ draw, bf16 *__restrict__ dsplit, const int32_t *__restrict__ split_row_index) {
+    const int32_t *__restrict__ dload_row_group, int64_t rows, int32_t n, int32_t k, float *__restrict__ dlogit, bf16 *__restrict__ dsplit, const int32_t *__restrict__ split_row_index) {
     const int lane = threadIdx.x & 31;
     const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (row >= rows) return;
@@ -80,8 +79,8 @@ __global__ void __launch_bounds__(256) gate_logit_grads_kernel(
                 v -= __bfloat162float(b);
             }
         } else {
-            dclean[row * n + j] = dc;
-            draw[row * n + j] = dr;
+            dlogit[row * 2 * n + j] = dc;
+            dlogit[row * 2 * n + n + j] = dr;
         }
     };
 
@@ -235,7 +234,7 @@ __global__ void __launch_bounds__(256) gate_logit_grads_pairs_kernel(
 int32_t launch_gate_logit_grads(const float *noise, const float *clean, const float *raw, const int32_t *idx,
                                 const float *gates, const float *kth_vals, const int32_t *kth_idx,
                                 const float *dgates, const float *dload, const int32_t *dload_row_group,
-                                int64_t rows, int32_t n, int32_t k, float *dclean, float *draw, void *dsplit,
+                                int64_t rows, int32_t n, int32_t k, float *dlogit, void *dsplit,
                                 const int32_t *split_row_index, cudaStream_t st) {
     if (rows == 0) return MOE_OK;
     const unsigned grid = (unsigned)cdiv(rows, 8);
@@ -260,7 +259,7 @@ int32_t launch_gate_logit_grads(const float *noise, const float *clean, const fl
     }
 #define MOE_LOGIT_GRADS(NV)                                                                                          \
     gate_logit_grads_kernel<NV><<<grid, 256, 0, st>>>(noise, clean, raw, idx, gates, kth_vals, kth_idx, dgates, dload, \
-                                                      dload_row_group, rows, n, k, dclean, draw, (bf16 *)dsplit,      \
+                                                      dload_row_group, rows, n, k, dlogit, (bf16 *)dsplit,      \
                                                       split_row_index)
     if (n <= 32) MOE_LOGIT_GRADS(1);
     else if (n <= 64) MOE_LOGIT_GRADS(2);

@@ -180,21 +180,21 @@ int32_t launch_add_gathered(float *dgates, const int32_t *topk_idx, const float 
                             cudaStream_t st);
 
 // ----------------------------------------------------------------------------- gate backward (gate_bwd.cu)
-// dclean, draw [rows, n] from the saved gate tensors; dload_row_stride = 0 broadcasts dload [n].
+// dlogit [rows, 2n] = (dclean | draw) from the saved gate tensors, or (dsplit given) its three-term bf16 split.
 int32_t launch_gate_logit_grads(const float *noise, const float *clean, const float *raw, const int32_t *idx,
                                 const float *gates, const float *kth_vals, const int32_t *kth_idx,
                                 const float *dgates, const float *dload, const int32_t *dload_row_group,
-                                int64_t rows, int32_t n, int32_t k, float *dclean, float *draw, void *dsplit,
+                                int64_t rows, int32_t n, int32_t k, float *dlogit, void *dsplit,
                                 const int32_t *split_row_index, cudaStream_t st);
 
 // ----------------------------------------------------------------------------- SIMT grouped GEMM (gemm_simt.cu)
 enum GemmType { G_F32 = 0, G_BF16 = 1 };
 struct SimtGemm {
-    // C(i,j) = epilogue( sum_kk A(i,kk) * B(kk,j) ), element strides in elements.
+    // C(i,j) = epilogue( sum_kk A(i,kk) * B(kk,j) ), strides in elements; one index of A and of B is contiguous, j of C is.
     const void *A, *B;
     void *C;
     int32_t ta, tb, tc;  // GemmType of A, B, C
-    int64_t sa_i, sa_k, sb_k, sb_j, sc_i, sc_j;
+    int64_t sa_i, sa_k, sb_k, sb_j, sc_i;
     // mode 0: output rows follow the segments (M_e = count_e, K fixed); A, C advance by rows,
     //         B by expert (b_e). mode 1: contraction over the segment rows (K_e = count_e);
     //         A, B advance by rows (their k index), C by expert (c_e).
@@ -206,7 +206,14 @@ struct SimtGemm {
     const void *bias;  // [nseg, N] of type tc, or nullptr
     int32_t relu;      // 1: max(.,0)
     const void *mask;  // mode 0: same shape/type as C; result multiplied by [mask > 0]
-    int32_t accumulate;  // 1: C += (float C only)
+    // a second matrix continues B / C along its contiguous index from b_split / c_split on (same strides): the two gating
+    // matrices [W_g | W_noise] and their gradients. b_k_contiguous: B's contraction index is the contiguous one (needed
+    // where both strides are 1)
+    const void *B2;
+    void *C2;
+    int64_t b_split, c_split;
+    int32_t b_k_contiguous;
+    const int32_t *row_count;  // mode 0 without segments: number of rows, read on the device (at most M)
     // optional row gathers through a permutation: mode 0: A row i reads row a_row_index[i] / a_row_div
     // and C row i is written at c_row_index[i]; mode 1: the contraction index r reads A row
     // a_row_index[r] / a_row_div and B row b_row_index[r].
@@ -215,7 +222,10 @@ struct SimtGemm {
     const int32_t *b_row_index;
     const int32_t *c_row_index;
 };
-int32_t launch_simt_gemm(const SimtGemm &g, int32_t *tile_prefix, cudaStream_t st);
+// Mode 1 over segments: K is the number of rows of all segments. part: simt_wgrad_splits(M, N, nseg, K) * nseg * M * N
+// floats let a product with few tiles be cut along its contraction (float results only)
+int32_t simt_wgrad_splits(int64_t M, int64_t N, int32_t nseg, int64_t K);
+int32_t launch_simt_gemm(const SimtGemm &g, int32_t *tile_prefix, cudaStream_t st, float *part = nullptr);
 // out[e, j] = sum over the rows of segment e of in[r, j]   (out, in of the act type)
 int64_t colsum_ws_floats(int64_t R, int32_t n, int32_t N);
 int32_t launch_segment_colsum(const void *in, int32_t act, const int32_t *offsets, int32_t nseg, int64_t R,
