@@ -12,9 +12,9 @@ namespace moe {
 //   2. per expert, exclusive scan of the chunk histograms -> chunk bases,
 //      totals -> counts                                                   (dispatch_scan_chunks)
 //   3. exclusive scan of counts -> offsets                                (dispatch_scan_experts)
-//   4. one warp per chunk walks its slots in order, 32 at a time; equal experts inside a group
-//      of 32 are ranked with match_any, across groups with a shared-memory cursor per expert
-//                                                                          (dispatch_rank)
+//   4. per chunk the slots are ranked, 32 per warp with match_any, across the warps with a
+//      shared-memory cursor per expert                                     (dispatch_rank)
+// A single chunk needs only step 4, a moderate number of histogram entries only 1 and 4 (see launch_dispatch_index).
 // Integer atomics only (order-independent results); the permutation is unique and bit-exact.
 // ------------------------------------------------------------------------------------------
 constexpr int CH = 1024;  // slots per chunk
@@ -107,41 +107,116 @@ __global__ void __launch_bounds__(1024) dispatch_scan_experts_kernel(const int32
     if (threadIdx.x == 0) offsets[n] = carry;
 }
 
-__global__ void __launch_bounds__(32) dispatch_rank_kernel(const int32_t *__restrict__ topk_idx, int64_t R,
-                                                           int32_t n, const int32_t *__restrict__ chunk_base,
-                                                           const int32_t *__restrict__ offsets,
-                                                           int32_t *__restrict__ perm,
-                                                           int32_t *__restrict__ inv_perm) {
+// exclusive scan over the block of one value per thread (1024 threads); total: sum over the block
+__device__ __forceinline__ int32_t block_scan_1024(int32_t v, int32_t *sh /* [32] */, int32_t *total) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    int32_t inc = v;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int32_t o = __shfl_up_sync(0xffffffffu, inc, off);
+        if (lane >= off) inc += o;
+    }
+    __syncthreads();  // sh may still be read from an earlier call
+    if (lane == 31) sh[w] = inc;
+    __syncthreads();
+    const int32_t sw = sh[lane];
+    int32_t si = sw;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int32_t o = __shfl_up_sync(0xffffffffu, si, off);
+        if (lane >= off) si += o;
+    }
+    *total = __shfl_sync(0xffffffffu, si, 31);
+    return __shfl_sync(0xffffffffu, si - sw, w) + inc - v;
+}
+
+// Where the sorted rows of a chunk's slots start, per expert (cursor[e], shared memory), found by one of
+//   RANK_ONE    the only chunk: counted here, no other kernel
+//   RANK_FEW    from the chunks' histograms: every block adds the chunks before its own and scans the totals (n <= 1024)
+//   RANK_MANY   from the scanned chunk bases and offsets
+// Then 32 warps take 32 slots each: equal experts inside a warp are ranked with match_any, the warps advance the cursors one
+// after the other. (One warp walking the 32 groups with the loads on its critical path took 16 us per chunk, this takes 4.)
+enum RankFrom { RANK_ONE, RANK_FEW, RANK_MANY };
+template <int FROM>
+__global__ void __launch_bounds__(1024) dispatch_rank_kernel(const int32_t *__restrict__ topk_idx, int64_t R, int32_t n,
+                                                             const int32_t *__restrict__ chunk_table, int32_t nchunks,
+                                                             int32_t *__restrict__ counts, int32_t *__restrict__ offsets,
+                                                             int32_t *__restrict__ perm, int32_t *__restrict__ inv_perm) {
     extern __shared__ int32_t cursor[];  // next sorted row of each expert for this chunk
-    const int lane = threadIdx.x;
-    const int32_t *base = chunk_base + (int64_t)blockIdx.x * n;
-    for (int e = lane; e < n; e += 32) cursor[e] = offsets[e] + base[e];
-    __syncwarp();
-    const int64_t p0 = (int64_t)blockIdx.x * CH;
-    for (int i = 0; i < CH; i += 32) {
-        const int64_t p = p0 + i + lane;
-        const bool live = p < R;
-        int32_t e = live ? topk_idx[p] : -1;
-        MOE_BOUNDS_NOTE(!live || (uint32_t)e < (uint32_t)n);
-        if ((uint32_t)e >= (uint32_t)n) e = -1;
-        const unsigned peers = __match_any_sync(0xffffffffu, e);
-        const int rank = __popc(peers & ((1u << lane) - 1u));
-        const int leader = __ffs(peers) - 1;
-        int32_t start = 0;
-        if (e >= 0 && lane == leader) {
+    __shared__ int32_t sh[32];
+    __shared__ int32_t part_total[1024], part_before[1024];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t p = (int64_t)blockIdx.x * CH + tid;
+    const bool live = p < R;
+    int32_t e = live ? topk_idx[p] : -1;
+    MOE_BOUNDS_NOTE(!live || (uint32_t)e < (uint32_t)n);
+    if ((uint32_t)e >= (uint32_t)n) e = -1;
+    if (FROM == RANK_MANY) {
+        const int32_t *base = chunk_table + (int64_t)blockIdx.x * n;
+        for (int32_t q = tid; q < n; q += 1024) cursor[q] = offsets[q] + base[q];
+    } else if (FROM == RANK_FEW) {
+        // thread (group, expert) adds its group's share of the chunks, the groups are then added per expert
+        int32_t width = 32;
+        while (width < n) width <<= 1;
+        const int32_t q = tid & (width - 1), group = tid / width, groups = 1024 / width;
+        int32_t total = 0, before = 0;
+        if (q < n) {
+#pragma unroll 8
+            for (int32_t c = group; c < nchunks; c += groups) {
+                const int32_t v = chunk_table[(int64_t)c * n + q];
+                total += v;
+                before += c < (int32_t)blockIdx.x ? v : 0;
+            }
+        }
+        part_total[tid] = total;
+        part_before[tid] = before;
+        __syncthreads();
+        total = before = 0;
+        if (tid < n)
+            for (int32_t g = 0; g < groups; ++g) { total += part_total[g * width + tid]; before += part_before[g * width + tid]; }
+        int32_t all;
+        const int32_t excl = block_scan_1024(total, sh, &all);
+        if (tid < n) {
+            cursor[tid] = excl + before;
+            if (blockIdx.x == 0) { counts[tid] = total; offsets[tid] = excl; }
+        }
+        if (tid == 0 && blockIdx.x == 0) offsets[n] = all;
+    } else {
+        for (int32_t q = tid; q < n; q += 1024) cursor[q] = 0;
+    }
+    const unsigned peers = __match_any_sync(0xffffffffu, e);
+    const int rank = __popc(peers & ((1u << lane) - 1u)), leader = __ffs(peers) - 1;
+    int32_t start = 0;
+    const int busy_warps = (int)min((int64_t)32, (R - (int64_t)blockIdx.x * CH + 31) / 32);
+    for (int w = 0; w < busy_warps; ++w) {
+        __syncthreads();
+        if (warp == w && e >= 0 && lane == leader) {
             start = cursor[e];
             cursor[e] = start + __popc(peers);
         }
-        start = __shfl_sync(0xffffffffu, start, leader);
-        if (e >= 0) {
-            const int32_t r = start + rank;
-            MOE_BOUNDS_NOTE((uint32_t)r < (uint32_t)R);
-            perm[r] = (int32_t)p;
-            inv_perm[p] = r;
-        } else if (live) {
-            inv_perm[p] = -1;  // expert id outside [0, n): the slot is dropped; the row movers skip negative rows
+    }
+    start = __shfl_sync(0xffffffffu, start, leader);
+    if (FROM == RANK_ONE) {  // the cursors hold the counts now: scan them, then shift the ranks by their expert's offset
+        __syncthreads();
+        int32_t carry = 0;
+        for (int32_t q0 = 0; q0 < n; q0 += 1024) {
+            const int32_t q = q0 + tid, v = q < n ? cursor[q] : 0;
+            int32_t all;
+            const int32_t excl = carry + block_scan_1024(v, sh, &all);
+            if (q < n) { counts[q] = v; offsets[q] = excl; cursor[q] = excl; }
+            carry += all;
         }
-        __syncwarp();
+        if (tid == 0) offsets[n] = carry;
+        __syncthreads();
+        if (e >= 0) start += cursor[e];
+    }
+    if (e >= 0) {
+        const int32_t r = start + rank;
+        MOE_BOUNDS_NOTE((uint32_t)r < (uint32_t)R);
+        perm[r] = (int32_t)p;
+        inv_perm[p] = r;
+    } else if (live) {
+        inv_perm[p] = -1;  // expert id outside [0, n): the slot is dropped; the row movers skip negative rows
     }
 }
 
@@ -153,13 +228,26 @@ int32_t launch_dispatch_index(const int32_t *topk_idx, int64_t R, int32_t n, int
         MOE_CUDA(cudaMemsetAsync(offsets, 0, sizeof(int32_t) * (n + 1), st));
         return MOE_OK;
     }
-    dispatch_hist_kernel<<<nchunks, 256, n * sizeof(int32_t), st>>>(topk_idx, R, n, scratch);
+    const size_t sh = n * sizeof(int32_t);
+    // one chunk: one launch. Up to 64 Ki histogram entries every block can afford to read them all (128 chunks x 256
+    // experts: 1.5 us), which saves the two scans' launches.
+    if (nchunks == 1 && n <= 8192) {
+        dispatch_rank_kernel<RANK_ONE><<<1, 1024, sh, st>>>(topk_idx, R, n, nullptr, 1, counts, offsets, perm, inv_perm);
+        MOE_LAUNCHED();
+        return MOE_OK;
+    }
+    dispatch_hist_kernel<<<nchunks, 256, sh, st>>>(topk_idx, R, n, scratch);
     MOE_LAUNCHED();
+    if (n <= 1024 && (int64_t)nchunks * n <= 65536) {
+        dispatch_rank_kernel<RANK_FEW><<<nchunks, 1024, sh, st>>>(topk_idx, R, n, scratch, nchunks, counts, offsets, perm, inv_perm);
+        MOE_LAUNCHED();
+        return MOE_OK;
+    }
     dispatch_scan_chunks_kernel<<<(unsigned)cdiv(n, 32), 1024, 0, st>>>(scratch, nchunks, n, counts);
     MOE_LAUNCHED();
     dispatch_scan_experts_kernel<<<1, 1024, 0, st>>>(counts, n, offsets);
     MOE_LAUNCHED();
-    dispatch_rank_kernel<<<nchunks, 32, n * sizeof(int32_t), st>>>(topk_idx, R, n, scratch, offsets, perm, inv_perm);
+    dispatch_rank_kernel<RANK_MANY><<<nchunks, 1024, sh, st>>>(topk_idx, R, n, scratch, nchunks, counts, offsets, perm, inv_perm);
     MOE_LAUNCHED();
     return MOE_OK;
 }
