@@ -15,6 +15,7 @@ namespace {
 // p = softmax(c) per row: exponentials and their sum in double (largest logit subtracted), one rounding to float.
 __global__ void __launch_bounds__(256) bal_softmax_kernel(const float *__restrict__ c, int64_t T, int32_t n,
                                                           float *__restrict__ p) {
+    wait_previous_kernel();
     const int lane = threadIdx.x & 31;
     const int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (t >= T) return;
@@ -33,6 +34,7 @@ __global__ void __launch_bounds__(256) bal_softmax_kernel(const float *__restric
 // out [cols, rows] = in [rows, cols]^T, 32 x 32 tiles
 __global__ void __launch_bounds__(256) bal_transpose_kernel(const float *__restrict__ in, int64_t rows, int32_t cols,
                                                             float *__restrict__ out) {
+    wait_previous_kernel();
     __shared__ float tile[32][33];
     const int64_t r0 = (int64_t)blockIdx.x * 32;
     const int32_t c0 = blockIdx.y * 32;
@@ -51,6 +53,7 @@ __global__ void __launch_bounds__(256) bal_transpose_kernel(const float *__restr
 __global__ void __launch_bounds__(1024) bal_select_kernel(const float *__restrict__ pT, int64_t T, int32_t n, int32_t m,
                                                           int32_t words, int32_t *__restrict__ tok_of_row,
                                                           uint32_t *__restrict__ mask_bits) {
+    wait_previous_kernel();
     __shared__ int32_t hist[256];
     __shared__ int32_t warp_gt[32], warp_eq[32];
     __shared__ uint32_t s_prefix;
@@ -125,6 +128,7 @@ __global__ void __launch_bounds__(256) bal_token_kernel(const float *__restrict_
                                                         const float *__restrict__ thr, int64_t T, int32_t n, int32_t words,
                                                         float *__restrict__ den, int32_t *__restrict__ cnt,
                                                         int32_t *__restrict__ thr_counts, double *__restrict__ loss_part) {
+    wait_previous_kernel();
     extern __shared__ int32_t s_cnt[];  // [n] threshold-mask counts of this block
     __shared__ double s_loss[8];
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
@@ -165,6 +169,7 @@ __global__ void __launch_bounds__(256) bal_token_kernel(const float *__restrict_
 
 __global__ void __launch_bounds__(256) bal_loss_final_kernel(const double *__restrict__ part, int64_t nparts,
                                                              float *__restrict__ loss) {
+    wait_previous_kernel();
     __shared__ double sh[256];
     double s = 0.0;
     for (int64_t i = threadIdx.x; i < nparts; i += 256) s += part[i];
@@ -190,6 +195,7 @@ __global__ void __launch_bounds__(256) bal_fill_kernel(const int32_t *__restrict
                                                        const int32_t *__restrict__ tok_ptr, int64_t R, int32_t n, int32_t m,
                                                        int32_t words, int32_t *__restrict__ tok_rows,
                                                        int32_t *__restrict__ offsets) {
+    wait_previous_kernel();
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r <= n) offsets[r] = (int32_t)(r * m);
     if (r >= R) return;
@@ -208,6 +214,7 @@ template <typename XT> struct V16 {
 template <typename XT>
 __global__ void __launch_bounds__(256) bal_gather_kernel(const XT *__restrict__ x, const int32_t *__restrict__ tok_of_row,
                                                          int64_t R, int64_t T, int32_t d, XT *__restrict__ xs) {
+    wait_previous_kernel();
     const int lane = threadIdx.x & 31;
     const int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (r >= R) return;
@@ -225,6 +232,7 @@ __global__ void __launch_bounds__(256) bal_combine_kernel(const XT *__restrict__
                                                           const float *__restrict__ den, const int32_t *__restrict__ tok_ptr,
                                                           const int32_t *__restrict__ tok_rows, int64_t T, int64_t R,
                                                           int32_t n, int32_t m, int32_t d, XT *__restrict__ y) {
+    wait_previous_kernel();
     constexpr int VN = V16<XT>::N;
     const int lane = threadIdx.x & 31;
     const int64_t t = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -259,6 +267,7 @@ __global__ void __launch_bounds__(256) bal_combine_bwd_kernel(const XT *__restri
                                                               const int32_t *__restrict__ tok_of_row, int64_t R, int64_t T,
                                                               int32_t n, int32_t m, int32_t d, float *__restrict__ dG_row,
                                                               XT *__restrict__ dys) {
+    wait_previous_kernel();
     constexpr int VN = V16<XT>::N;
     const int lane = threadIdx.x & 31;
     const int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -292,6 +301,7 @@ __global__ void __launch_bounds__(256) bal_gate_bwd_kernel(const float *__restri
                                                            const float *__restrict__ dG_row, float w, int64_t T, int32_t n,
                                                            int32_t m, int32_t words, float *__restrict__ dc,
                                                            bf16 *__restrict__ dsplit) {
+    wait_previous_kernel();
     const int lane = threadIdx.x & 31;
     const int64_t t = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (t >= T) return;
@@ -337,6 +347,7 @@ __global__ void __launch_bounds__(256) bal_gate_bwd_kernel(const float *__restri
 
 __global__ void bal_dthr_kernel(const int32_t *__restrict__ thr_counts, int32_t n, int32_t m, float w,
                                 float *__restrict__ dthr) {
+    wait_previous_kernel();
     const int32_t j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < n) dthr[j] = -w * (float)(thr_counts[j] - m);
 }
@@ -347,6 +358,7 @@ __global__ void __launch_bounds__(256) bal_dispatch_bwd_kernel(const XT *__restr
                                                                const int32_t *__restrict__ tok_rows,
                                                                const float *__restrict__ dX_gate, int64_t T, int64_t R,
                                                                int32_t d, XT *__restrict__ dX) {
+    wait_previous_kernel();
     constexpr int VN = V16<XT>::N;
     const int lane = threadIdx.x & 31;
     const int64_t t = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -402,19 +414,19 @@ int32_t launch_balanced_gate(const void *x, int32_t act, int64_t T, int32_t d, i
     }
     // logits by the fixed fma chain (one matrix: the projection kernel's second one is absent)
     MOE_TRY(launch_projection(x, act, T, d, n, Wg, nullptr, logits, nullptr, nullptr, 0, nullptr, 1, nullptr, st));
-    bal_softmax_kernel<<<(unsigned)cdiv(T, 8), 256, 0, st>>>(logits, T, n, probs);
+    launch_kernel(bal_softmax_kernel, (unsigned)cdiv(T, 8), 256, 0, st, logits, T, n, probs);
     MOE_LAUNCHED();
-    bal_transpose_kernel<<<dim3((unsigned)cdiv(T, 32), (unsigned)cdiv(n, 32)), 256, 0, st>>>(probs, T, n, pT);
+    launch_kernel(bal_transpose_kernel, dim3((unsigned)cdiv(T, 32), (unsigned)cdiv(n, 32)), 256, 0, st, probs, T, n, pT);
     MOE_LAUNCHED();
-    bal_select_kernel<<<(unsigned)n, 1024, 0, st>>>(pT, T, n, m, words, tok_of_row, mask_bits);
+    launch_kernel(bal_select_kernel, (unsigned)n, 1024, 0, st, pT, T, n, m, words, tok_of_row, mask_bits);
     MOE_LAUNCHED();
-    bal_token_kernel<<<(unsigned)cdiv(T, 8), 256, n * sizeof(int32_t), st>>>(probs, mask_bits, thr, T, n, words, den, cnt,
+    launch_kernel(bal_token_kernel, (unsigned)cdiv(T, 8), 256, n * sizeof(int32_t), st, probs, mask_bits, thr, T, n, words, den, cnt,
                                                                              thr_counts, loss_part);
     MOE_LAUNCHED();
-    bal_loss_final_kernel<<<1, 256, 0, st>>>(loss_part, cdiv(T, 8), loss);
+    launch_kernel(bal_loss_final_kernel, 1, 256, 0, st, loss_part, cdiv(T, 8), loss);
     MOE_LAUNCHED();
     MOE_TRY(launch_exclusive_scan(cnt, (int32_t)T, tok_ptr, st, tile_sums));
-    bal_fill_kernel<<<(unsigned)cdiv(R > n ? R : n + 1, 256) + 1, 256, 0, st>>>(tok_of_row, mask_bits, tok_ptr, R, n, m, words,
+    launch_kernel(bal_fill_kernel, (unsigned)cdiv(R > n ? R : n + 1, 256) + 1, 256, 0, st, tok_of_row, mask_bits, tok_ptr, R, n, m, words,
                                                                                 tok_rows, offsets);
     MOE_LAUNCHED();
     return MOE_OK;
@@ -423,8 +435,8 @@ int32_t launch_balanced_gate(const void *x, int32_t act, int64_t T, int32_t d, i
 int32_t launch_balanced_gather(const void *x, int32_t act, const int32_t *tok_of_row, int64_t R, int64_t T, int32_t d,
                                void *xs, cudaStream_t st) {
     if (R == 0) return MOE_OK;
-    if (act == MOE_BF16) bal_gather_kernel<bf16><<<(unsigned)cdiv(R, 8), 256, 0, st>>>((const bf16 *)x, tok_of_row, R, T, d, (bf16 *)xs);
-    else bal_gather_kernel<float><<<(unsigned)cdiv(R, 8), 256, 0, st>>>((const float *)x, tok_of_row, R, T, d, (float *)xs);
+    if (act == MOE_BF16) launch_kernel(bal_gather_kernel<bf16>, (unsigned)cdiv(R, 8), 256, 0, st, (const bf16 *)x, tok_of_row, R, T, d, (bf16 *)xs);
+    else launch_kernel(bal_gather_kernel<float>, (unsigned)cdiv(R, 8), 256, 0, st, (const float *)x, tok_of_row, R, T, d, (float *)xs);
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -434,9 +446,9 @@ int32_t launch_balanced_combine(const void *ys, int32_t act, const float *p, con
                                 cudaStream_t st) {
     if (T == 0) return MOE_OK;
     if (act == MOE_BF16)
-        bal_combine_kernel<bf16><<<(unsigned)cdiv(T, 8), 256, 0, st>>>((const bf16 *)ys, p, den, tok_ptr, tok_rows, T, R, n, m, d, (bf16 *)y);
+        launch_kernel(bal_combine_kernel<bf16>, (unsigned)cdiv(T, 8), 256, 0, st, (const bf16 *)ys, p, den, tok_ptr, tok_rows, T, R, n, m, d, (bf16 *)y);
     else
-        bal_combine_kernel<float><<<(unsigned)cdiv(T, 8), 256, 0, st>>>((const float *)ys, p, den, tok_ptr, tok_rows, T, R, n, m, d, (float *)y);
+        launch_kernel(bal_combine_kernel<float>, (unsigned)cdiv(T, 8), 256, 0, st, (const float *)ys, p, den, tok_ptr, tok_rows, T, R, n, m, d, (float *)y);
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -446,9 +458,9 @@ int32_t launch_balanced_combine_bwd(const void *dY, const void *ys, int32_t act,
                                     float *dG_row, void *dys, cudaStream_t st) {
     if (R == 0) return MOE_OK;
     if (act == MOE_BF16)
-        bal_combine_bwd_kernel<bf16><<<(unsigned)cdiv(R, 8), 256, 0, st>>>((const bf16 *)dY, (const bf16 *)ys, p, den, tok_of_row, R, T, n, m, d, dG_row, (bf16 *)dys);
+        launch_kernel(bal_combine_bwd_kernel<bf16>, (unsigned)cdiv(R, 8), 256, 0, st, (const bf16 *)dY, (const bf16 *)ys, p, den, tok_of_row, R, T, n, m, d, dG_row, (bf16 *)dys);
     else
-        bal_combine_bwd_kernel<float><<<(unsigned)cdiv(R, 8), 256, 0, st>>>((const float *)dY, (const float *)ys, p, den, tok_of_row, R, T, n, m, d, dG_row, (float *)dys);
+        launch_kernel(bal_combine_bwd_kernel<float>, (unsigned)cdiv(R, 8), 256, 0, st, (const float *)dY, (const float *)ys, p, den, tok_of_row, R, T, n, m, d, dG_row, (float *)dys);
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -459,11 +471,11 @@ int32_t launch_balanced_gate_bwd(const float *p, const uint32_t *mask_bits, cons
                                  void *dsplit, float *dthr, cudaStream_t st) {
     const int32_t words = (n + 31) / 32;
     if (T > 0) {
-        bal_gate_bwd_kernel<<<(unsigned)cdiv(T, 8), 256, 0, st>>>(p, mask_bits, den, thr, tok_ptr, tok_rows, dG_row, w, T, n, m, words, dc,
+        launch_kernel(bal_gate_bwd_kernel, (unsigned)cdiv(T, 8), 256, 0, st, p, mask_bits, den, thr, tok_ptr, tok_rows, dG_row, w, T, n, m, words, dc,
                                                                   (bf16 *)dsplit);
         MOE_LAUNCHED();
     }
-    bal_dthr_kernel<<<(unsigned)cdiv(n, 256), 256, 0, st>>>(thr_counts, n, T > 0 ? m : 0, w, dthr);
+    launch_kernel(bal_dthr_kernel, (unsigned)cdiv(n, 256), 256, 0, st, thr_counts, n, T > 0 ? m : 0, w, dthr);
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -472,9 +484,9 @@ int32_t launch_balanced_dispatch_bwd(const void *dxs, int32_t act, const int32_t
                                      const float *dX_gate, int64_t T, int64_t R, int32_t d, void *dX, cudaStream_t st) {
     if (T == 0) return MOE_OK;
     if (act == MOE_BF16)
-        bal_dispatch_bwd_kernel<bf16><<<(unsigned)cdiv(T, 8), 256, 0, st>>>((const bf16 *)dxs, tok_ptr, tok_rows, dX_gate, T, R, d, (bf16 *)dX);
+        launch_kernel(bal_dispatch_bwd_kernel<bf16>, (unsigned)cdiv(T, 8), 256, 0, st, (const bf16 *)dxs, tok_ptr, tok_rows, dX_gate, T, R, d, (bf16 *)dX);
     else
-        bal_dispatch_bwd_kernel<float><<<(unsigned)cdiv(T, 8), 256, 0, st>>>((const float *)dxs, tok_ptr, tok_rows, dX_gate, T, R, d, (float *)dX);
+        launch_kernel(bal_dispatch_bwd_kernel<float>, (unsigned)cdiv(T, 8), 256, 0, st, (const float *)dxs, tok_ptr, tok_rows, dX_gate, T, R, d, (float *)dX);
     MOE_LAUNCHED();
     return MOE_OK;
 }

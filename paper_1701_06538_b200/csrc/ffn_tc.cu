@@ -477,6 +477,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    wait_previous_kernel();  // barriers and tensor memory are set up while the previous kernel drains
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
@@ -962,6 +963,7 @@ grouped_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     cluster_sync_all();  // both CTAs' barriers exist before anything is signalled across the pair
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    wait_previous_kernel();  // barriers and tensor memory are set up while the previous kernel drains
 
     // K rows past the segment end in stage s's A and B tiles (two 64-column chunks each, the B tile directly behind the
     // A tile) := 0. Zeroing A alone would do for finite data (0 x finite = 0); B as well keeps a non-finite value of the
@@ -1452,7 +1454,7 @@ template <int KIND> int32_t launch(const CUtensorMap &tmA, const CUtensorMap &tm
     }
     if (max_tiles <= 0) return MOE_OK;
     const unsigned grid = (unsigned)imin(max_tiles, sm_count());
-    grouped_gemm_kernel<KIND><<<grid, NTHREADS, SMEM_BYTES, st>>>(tmA, tmB, p);
+    launch_kernel(grouped_gemm_kernel<KIND>, grid, NTHREADS, SMEM_BYTES, st, tmA, tmB, p);
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -1470,7 +1472,7 @@ int32_t launch_acc_wgrad(const CUtensorMap &tmA, const CUtensorMap &tmB, const G
     }
     if (max_tiles <= 0) return MOE_OK;
     const unsigned grid = (unsigned)imin(max_tiles, sm_count());
-    grouped_gemm_kernel<WGRAD, true><<<grid, NTHREADS, SMEM_ACC_BYTES, st>>>(tmA, tmB, p);
+    launch_kernel((grouped_gemm_kernel<WGRAD, true>), grid, NTHREADS, SMEM_ACC_BYTES, st, tmA, tmB, p);
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -1484,11 +1486,13 @@ int32_t launch2(const CUtensorMap &tmA, const CUtensorMap &tmB, const GemmParams
     static int max_clusters = 0;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = 2; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+    cudaLaunchAttribute attrs[2];
+    attrs[0].id = cudaLaunchAttributeClusterDimension;
+    attrs[0].val.clusterDim.x = 2; attrs[0].val.clusterDim.y = 1; attrs[0].val.clusterDim.z = 1;
+    attrs[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // as launch_kernel
+    attrs[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.blockDim = dim3(NTHREADS2); cfg.dynamicSmemBytes = SMEM2_BYTES; cfg.stream = st;
-    cfg.attrs = &attr; cfg.numAttrs = 1;
+    cfg.attrs = attrs; cfg.numAttrs = 2;
     if (!max_clusters) {
         MOE_CUDA(cudaFuncSetAttribute(grouped_gemm2_kernel<KIND, MASKT>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM2_BYTES));
         cfg.gridDim = dim3(2 * (sm_count() / 2));
@@ -1533,6 +1537,7 @@ static bool use_two_cta(int64_t R, int32_t nseg, int32_t flags) {
 __global__ void __launch_bounds__(1024) tile_table_kernel(const int32_t *__restrict__ offsets, int32_t n, int32_t tm,
                                                           int32_t max_m, int32_t *__restrict__ tile_prefix,
                                                           int4 *__restrict__ info, int32_t *__restrict__ counter) {
+    wait_previous_kernel();
     __shared__ int32_t warp_sum[32];
     __shared__ int32_t carry;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -1592,7 +1597,7 @@ static int32_t *tile_counter_of(int32_t *tile_prefix, int32_t nseg, int64_t R) {
 }
 static int32_t launch_tile_table(const int32_t *offsets, int32_t nseg, int32_t tm, int64_t R, int32_t *tile_prefix,
                                  cudaStream_t st, int32_t *counter = nullptr) {
-    tile_table_kernel<<<1, 1024, 0, st>>>(offsets, nseg, tm, (int32_t)(cdiv(R, tm) + nseg), tile_prefix,
+    launch_kernel(tile_table_kernel, 1, 1024, 0, st, offsets, nseg, tm, (int32_t)(cdiv(R, tm) + nseg), tile_prefix,
                                           tile_info_of(tile_prefix, nseg), counter);
     MOE_LAUNCHED();
     return MOE_OK;
@@ -1606,6 +1611,7 @@ static int32_t launch_tile_table(const int32_t *offsets, int32_t nseg, int32_t t
 __global__ void __launch_bounds__(256) colsum_blocks_final_kernel(const float *__restrict__ part, int32_t N,
                                                                   const int32_t *__restrict__ tile_prefix, int32_t G,
                                                                   bf16 *__restrict__ out) {
+    wait_previous_kernel();
     __shared__ float4 sh[16][16];
     const int32_t e = blockIdx.x, q = threadIdx.x >> 4, cl = threadIdx.x & 15;
     const int32_t j = blockIdx.y * 64 + cl * 4;  // N is a multiple of 64
@@ -1651,7 +1657,7 @@ int32_t tc_row_gemm(const void *A, const void *W, bool transposed, const int32_t
     }
     auto finish = [&](int32_t rc, int32_t G) -> int32_t {
         if (rc != MOE_OK || !colsum_out) return rc;
-        colsum_blocks_final_kernel<<<dim3((unsigned)nseg, (unsigned)cdiv(N, 64)), 256, 0, st>>>(colsum_part, N, tile_prefix, G,
+        launch_kernel(colsum_blocks_final_kernel, dim3((unsigned)nseg, (unsigned)cdiv(N, 64)), 256, 0, st, colsum_part, N, tile_prefix, G,
                                                                                                    (bf16 *)colsum_out);
         MOE_LAUNCHED();
         return MOE_OK;
@@ -1700,6 +1706,7 @@ int32_t tc_row_gemm(const void *A, const void *W, bool transposed, const int32_t
 constexpr int SCHED_MAX_SEG = 8192;
 __global__ void __launch_bounds__(256) wgrad_schedule_kernel(const int32_t *__restrict__ offsets, int32_t n,
                                                              int4 *__restrict__ seg, int32_t *__restrict__ counter) {
+    wait_previous_kernel();
     __shared__ int32_t cnt[SCHED_MAX_SEG];
     for (int32_t e = threadIdx.x; e < n; e += blockDim.x) cnt[e] = offsets[e + 1] - offsets[e];
     __syncthreads();
@@ -1727,7 +1734,7 @@ int32_t tc_wgrad_gemm(const void *A, const void *B, const int32_t *offsets, int3
             p.sched_counter = sched_ws;
             p.sched_table = reinterpret_cast<const int4 *>(sched_ws + 4);
             p.sched_group = (int32_t)(cdiv(M, 256) * cdiv(N, BN));
-            wgrad_schedule_kernel<<<(unsigned)cdiv(nseg, 256), 256, 0, st>>>(offsets, nseg, reinterpret_cast<int4 *>(sched_ws + 4),
+            launch_kernel(wgrad_schedule_kernel, (unsigned)cdiv(nseg, 256), 256, 0, st, offsets, nseg, reinterpret_cast<int4 *>(sched_ws + 4),
                                                                           sched_ws);
             MOE_LAUNCHED();
         }
@@ -1761,6 +1768,7 @@ int32_t launch_tc_ffn(const moe_config &c, const void *xs, const int32_t *offset
 __global__ void __launch_bounds__(256) split_weights_kernel(const float *__restrict__ Wg,
                                                             const float *__restrict__ Wn, int32_t d, int32_t n,
                                                             bf16 *__restrict__ wsplit, int32_t ldw) {
+    wait_previous_kernel();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int32_t n2 = 2 * n;
     if (i >= (int64_t)d * n2) return;
@@ -1779,6 +1787,7 @@ __global__ void __launch_bounds__(256) reduce_partials_kernel(const float *__res
                                                               int64_t part_stride, int32_t d, int32_t n,
                                                               float *__restrict__ dWg, float *__restrict__ dWn,
                                                               int32_t ldw) {
+    wait_previous_kernel();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int32_t n2 = 2 * n;
     const int64_t total = (int64_t)d * n2;
@@ -1835,7 +1844,7 @@ int32_t launch_tc_gate_bwd(const void *x, int64_t T, int32_t d, int32_t n, const
         MOE_CUDA(cudaMemsetAsync(dWn, 0, sizeof(float) * d * n, st));
         return MOE_OK;
     }
-    split_weights_kernel<<<(unsigned)cdiv((int64_t)d * n2, 256), 256, 0, st>>>(Wg, Wn, d, n, (bf16 *)wsplit, ldw > 0 ? ldw : n);
+    launch_kernel(split_weights_kernel, (unsigned)cdiv((int64_t)d * n2, 256), 256, 0, st, Wg, Wn, d, n, (bf16 *)wsplit, ldw > 0 ? ldw : n);
     MOE_LAUNCHED();
     int32_t nr, rows;
     gate_bwd_split(T, d, n, &nr, &rows);
@@ -1849,7 +1858,7 @@ int32_t launch_tc_gate_bwd(const void *x, int64_t T, int32_t d, int32_t n, const
         p.rows_per_seg = rows; p.segs_per_term = nr; p.b_term_chunks = n2 / 64;
         p.sub_kb0 = GB_ROWS_HI / BK; p.sub_kb = GB_ROWS_LO / BK; p.interleave = 3;
         MOE_TRY(launch_acc_wgrad(tmA, tmB, p, (int64_t)p.nseg * cdiv(d, BM) * cdiv(n2, BN), st));
-        reduce_partials_kernel<<<(unsigned)cdiv((int64_t)d * n2, 256), 256, 0, st>>>(partials, 3 * nr, (int64_t)d * n2, d, n, dWg, dWn,
+        launch_kernel(reduce_partials_kernel, (unsigned)cdiv((int64_t)d * n2, 256), 256, 0, st, partials, 3 * nr, (int64_t)d * n2, d, n, dWg, dWn,
                                                                                      ldw > 0 ? ldw : n);
         MOE_LAUNCHED();
     }
@@ -1932,7 +1941,7 @@ int32_t launch_tc_hier_secondary_bwd(const void *xs_p, const void *dsplit_s, voi
                                      int64_t P1, int32_t d, int32_t b, float *partials, float *dWg_s, float *dWn_s,
                                      float *dX_sec, int32_t *status, cudaStream_t st) {
     const int32_t n2 = 2 * b;
-    split_weights_kernel<<<(unsigned)cdiv((int64_t)a * d * n2, 256), 256, 0, st>>>(Wg_s, Wn_s, a * d, b, (bf16 *)wsplit_s, b);
+    launch_kernel(split_weights_kernel, (unsigned)cdiv((int64_t)a * d * n2, 256), 256, 0, st, Wg_s, Wn_s, a * d, b, (bf16 *)wsplit_s, b);
     MOE_LAUNCHED();
     {   // dW_s[i] = sum over the slots of group i of x[token]^T . dlogit[slot], one partial per precision term
         CUtensorMap tmA, tmB;
@@ -1942,7 +1951,7 @@ int32_t launch_tc_hier_secondary_bwd(const void *xs_p, const void *dsplit_s, voi
         p.offsets = offsets_p; p.nseg = 3 * a; p.off_mod = a; p.b_term_chunks = n2 / 64;
         p.M = d; p.N = n2; p.R = P1; p.out_f32 = partials; p.status = status;
         MOE_TRY(launch<WGRAD>(tmA, tmB, p, (int64_t)p.nseg * cdiv(d, BM) * cdiv(n2, BN), st));
-        reduce_partials_kernel<<<dim3((unsigned)cdiv((int64_t)d * n2, 256), (unsigned)a), 256, 0, st>>>(
+        launch_kernel(reduce_partials_kernel, dim3((unsigned)cdiv((int64_t)d * n2, 256), (unsigned)a), 256, 0, st, 
             partials, 3, (int64_t)a * d * n2, d, b, dWg_s, dWn_s, b);
         MOE_LAUNCHED();
     }
@@ -1983,6 +1992,7 @@ int32_t launch_tc_ffn_bwd(const moe_config &c, const void *xs, const void *hid, 
 // kernel simply returns once the limit has passed and leaves MOE_ERR_TIMEOUT in the status word.
 // ------------------------------------------------------------------------------------------
 __global__ void debug_wait_kernel(int32_t *status, unsigned long long limit_ns) {
+    wait_previous_kernel();
     __shared__ __align__(8) unsigned long long bar;
     __shared__ int abort_flag;
     abort_flag = 0;
@@ -1992,7 +2002,7 @@ __global__ void debug_wait_kernel(int32_t *status, unsigned long long limit_ns) 
 }
 
 int32_t launch_debug_wait(int32_t *status, unsigned long long limit_ns, cudaStream_t st) {
-    debug_wait_kernel<<<1, 1, 0, st>>>(status, limit_ns);
+    launch_kernel(debug_wait_kernel, 1, 1, 0, st, status, limit_ns);
     MOE_LAUNCHED();
     return MOE_OK;
 }

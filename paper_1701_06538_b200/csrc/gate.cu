@@ -46,6 +46,7 @@ __global__ void __launch_bounds__(256) gate_select_kernel(const float *__restric
                                                           const int32_t *__restrict__ row_count,
                                                           const int2 *__restrict__ row_span,
                                                           const int2 *__restrict__ chain_list) {
+    wait_previous_kernel();
     const int lane = threadIdx.x & 31;
     int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     // row_span (with a row list): {first chain entry, number of candidate columns} of a listed row whose other
@@ -130,7 +131,7 @@ int32_t launch_gate_select(const float *clean, const float *raw, const float *no
     if (rows == 0) return MOE_OK;
     const unsigned grid = (unsigned)cdiv(rows, 8);
 #define MOE_SELECT(KL)                                                                                                 \
-    gate_select_kernel<KL><<<grid, 256, 0, st>>>(clean, raw, noise, rows, n, k, idx, gates, kth_vals, kth_idx, row_list, \
+    launch_kernel(gate_select_kernel<KL>, grid, 256, 0, st, clean, raw, noise, rows, n, k, idx, gates, kth_vals, kth_idx, row_list, \
                                                  row_count, (const int2 *)row_span, (const int2 *)chain_list)
     if (k <= 2) MOE_SELECT(3);
     else if (k <= 4) MOE_SELECT(5);
@@ -155,6 +156,7 @@ int32_t launch_gate_select(const float *clean, const float *raw, const float *no
 __global__ void __launch_bounds__(256) split_gate_weights_kernel(const float *__restrict__ Wg,
                                                                  const float *__restrict__ Wn, int32_t d, int32_t n,
                                                                  bf16 *__restrict__ wsplit) {
+    wait_previous_kernel();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int32_t n2 = 2 * n;
     if (i >= (int64_t)d * n2) return;
@@ -171,6 +173,7 @@ __global__ void __launch_bounds__(256) split_gate_weights_kernel(const float *__
 // one warp per column of [W_g | W_noise]; blockIdx.y = group (stacked [groups, d, n] matrices)
 __global__ void __launch_bounds__(256) gate_col_norms_kernel(const float *__restrict__ Wg, const float *__restrict__ Wn,
                                                              int32_t d, int32_t n, float *__restrict__ wnorm) {
+    wait_previous_kernel();
     const int lane = threadIdx.x & 31;
     const int32_t j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (j >= 2 * n) return;
@@ -187,6 +190,7 @@ __global__ void __launch_bounds__(256) gate_col_norms_kernel(const float *__rest
 template <typename XT>
 __global__ void __launch_bounds__(256) row_norms_kernel(const XT *__restrict__ x, int64_t T, int32_t d,
                                                         float *__restrict__ xnorm) {
+    wait_previous_kernel();
     const int lane = threadIdx.x & 31;
     const int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (t >= T) return;
@@ -269,6 +273,7 @@ __global__ void __launch_bounds__(128) gate_screen_rows_kernel(const float *__re
                                                                int32_t *__restrict__ unsafe_count,
                                                                const int32_t *__restrict__ perm, int32_t kdiv,
                                                                const int32_t *__restrict__ group_of) {
+    wait_previous_kernel();
     __shared__ __align__(16) float tile[4][3][32 * SCREEN_PITCH];
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
     const int64_t s0 = ((int64_t)blockIdx.x * 4 + wp) * 32;  // first sorted row of this warp
@@ -443,6 +448,7 @@ __global__ void __launch_bounds__(256) gate_candidates_kernel(const float *__res
                                                               int32_t *__restrict__ full_list, int32_t kdiv,
                                                               const int32_t *__restrict__ group_of, int32_t k,
                                                               int2 *__restrict__ unsafe_span) {
+    wait_previous_kernel();
     // unsafe_span[i] = {first entry of the row's chains in chain_list, number of candidate columns}, or {0, -1}
     // where the repeated selection has to look at every column
     const int lane = threadIdx.x & 31;
@@ -520,6 +526,7 @@ __global__ void __launch_bounds__(128) gate_chain_kernel(const XT *__restrict__ 
                                                          const int32_t *__restrict__ chain_count,
                                                          float *__restrict__ clean, float *__restrict__ raw,
                                                          int32_t kdiv) {
+    wait_previous_kernel();
     // entry {output row, row of Wt}: the token is output row / kdiv, the column code is Wt row mod 2n (grouped gates
     // keep one [2n, d] block of Wt per group)
     __shared__ __align__(16) uint8_t stage[4][2][32 * CHAIN_PITCH];
@@ -597,6 +604,7 @@ __global__ void __launch_bounds__(128) gate_chain_kernel(const XT *__restrict__ 
 // Wt[c, q] = [W_g | W_noise][q, c]
 __global__ void __launch_bounds__(256) gate_transpose_weights_kernel(const float *__restrict__ Wg, const float *__restrict__ Wn,
                                                                      int32_t d, int32_t n, float *__restrict__ Wt) {
+    wait_previous_kernel();
     __shared__ float tile[32][33];
     Wg += (int64_t)blockIdx.z * d * n; Wn += (int64_t)blockIdx.z * d * n; Wt += (int64_t)blockIdx.z * 2 * n * d;  // group
     const int q0 = blockIdx.x * 32, c0 = blockIdx.y * 32;  // 2n and d are multiples of 32 on this path
@@ -613,10 +621,10 @@ int32_t launch_gate_chains(const void *x, int32_t act, int32_t d, int32_t n, con
                            const int32_t *chain_count, float *clean, float *raw, cudaStream_t st, int32_t kdiv) {
     const unsigned grid = 148 * 16;
     if (act == MOE_BF16)
-        gate_chain_kernel<bf16><<<grid, 128, 0, st>>>((const bf16 *)x, d, n, Wt, (const int2 *)chain_list, chain_count, clean,
+        launch_kernel(gate_chain_kernel<bf16>, grid, 128, 0, st, (const bf16 *)x, d, n, Wt, (const int2 *)chain_list, chain_count, clean,
                                                       raw, kdiv);
     else
-        gate_chain_kernel<float><<<grid, 128, 0, st>>>((const float *)x, d, n, Wt, (const int2 *)chain_list, chain_count, clean,
+        launch_kernel(gate_chain_kernel<float>, grid, 128, 0, st, (const float *)x, d, n, Wt, (const int2 *)chain_list, chain_count, clean,
                                                        raw, kdiv);
     MOE_LAUNCHED();
     return MOE_OK;
@@ -626,17 +634,17 @@ int32_t launch_gate_screen_prepare(const void *x, int32_t act, int64_t T, int32_
                                    const float *Wn, void *wsplit, float *wnorm, float *xnorm,
                                    int32_t *unsafe_count, float *wt, cudaStream_t st, int32_t groups, bool with_xnorm) {
     // groups > 1: Wg, Wn are stacks [groups, d, n]; wsplit [3][groups * d][2n], wnorm [groups][2n], wt [groups][2n][d]
-    gate_transpose_weights_kernel<<<dim3((unsigned)(d / 32), (unsigned)(2 * n / 32), (unsigned)groups), 256, 0, st>>>(Wg, Wn, d, n,
+    launch_kernel(gate_transpose_weights_kernel, dim3((unsigned)(d / 32), (unsigned)(2 * n / 32), (unsigned)groups), 256, 0, st, Wg, Wn, d, n,
                                                                                                                       wt);
     MOE_LAUNCHED();
-    split_gate_weights_kernel<<<(unsigned)cdiv((int64_t)groups * d * 2 * n, 256), 256, 0, st>>>(Wg, Wn, groups * d, n,
+    launch_kernel(split_gate_weights_kernel, (unsigned)cdiv((int64_t)groups * d * 2 * n, 256), 256, 0, st, Wg, Wn, groups * d, n,
                                                                                                   (bf16 *)wsplit);
     MOE_LAUNCHED();
-    gate_col_norms_kernel<<<dim3((unsigned)cdiv(2 * n, 8), (unsigned)groups), 256, 0, st>>>(Wg, Wn, d, n, wnorm);
+    launch_kernel(gate_col_norms_kernel, dim3((unsigned)cdiv(2 * n, 8), (unsigned)groups), 256, 0, st, Wg, Wn, d, n, wnorm);
     MOE_LAUNCHED();
     if (with_xnorm) {
-        if (act == MOE_BF16) row_norms_kernel<bf16><<<(unsigned)cdiv(T, 8), 256, 0, st>>>((const bf16 *)x, T, d, xnorm);
-        else row_norms_kernel<float><<<(unsigned)cdiv(T, 8), 256, 0, st>>>((const float *)x, T, d, xnorm);
+        if (act == MOE_BF16) launch_kernel(row_norms_kernel<bf16>, (unsigned)cdiv(T, 8), 256, 0, st, (const bf16 *)x, T, d, xnorm);
+        else launch_kernel(row_norms_kernel<float>, (unsigned)cdiv(T, 8), 256, 0, st, (const float *)x, T, d, xnorm);
         MOE_LAUNCHED();
     }
     MOE_CUDA(cudaMemsetAsync(unsafe_count, 0, 4 * sizeof(int32_t), st));  // rows to re-select, chains, full-chain rows
@@ -661,12 +669,12 @@ int32_t launch_gate_screen(const float *cr, const float *noise, const float *xno
 #define MOE_SCREEN_KL(KL)                                                                                              \
     do {                                                                                                               \
         if (v16)                                                                                                       \
-            gate_screen_rows_kernel<KL, true><<<grid, 128, 0, st>>>(cr, noise, xnorm, wnorm, theta, T, n,                   \
+            launch_kernel((gate_screen_rows_kernel<KL, true>), grid, 128, 0, st, cr, noise, xnorm, wnorm, theta, T, n,                   \
                                                                     k, idx, gates, clean, raw, kth_vals, kth_idx,      \
                                                                     unsafe_list, unsafe_low, unsafe_count, perm, kdiv, \
                                                                     group_of);                                         \
         else                                                                                                           \
-            gate_screen_rows_kernel<KL, false><<<grid, 128, 0, st>>>(cr, noise, xnorm, wnorm, theta, T,                     \
+            launch_kernel((gate_screen_rows_kernel<KL, false>), grid, 128, 0, st, cr, noise, xnorm, wnorm, theta, T,                     \
                                                                      n, k, idx, gates, clean, raw, kth_vals, kth_idx,  \
                                                                      unsafe_list, unsafe_low, unsafe_count, perm,      \
                                                                      kdiv, group_of);                                  \
@@ -676,7 +684,7 @@ int32_t launch_gate_screen(const float *cr, const float *noise, const float *xno
     else MOE_SCREEN_KL(MOE_MAX_K + 2);
 #undef MOE_SCREEN_KL
     MOE_LAUNCHED();
-    gate_candidates_kernel<<<148 * 4, 256, 0, st>>>(clean, raw, noise, xnorm, wnorm, theta, n, unsafe_list, unsafe_low,
+    launch_kernel(gate_candidates_kernel, 148 * 4, 256, 0, st, clean, raw, noise, xnorm, wnorm, theta, n, unsafe_list, unsafe_low,
                                                     unsafe_count, (int2 *)chain_list, full_list, kdiv, group_of, k,
                                                     (int2 *)unsafe_span);
     MOE_LAUNCHED();
@@ -687,6 +695,7 @@ int32_t launch_gate_screen(const float *cr, const float *noise, const float *xno
 __global__ void hier_merge_kernel(int64_t total, int32_t k1, int32_t k2, int32_t b, const int32_t *idx_p,
                                   const float *g_p, const int32_t *idx_s, const float *g_s, int32_t *topk_idx,
                                   float *gates) {
+    wait_previous_kernel();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // over T*k1*k2
     if (i >= total) return;
     const int64_t p1 = i / k2;  // t*k1 + s1
@@ -699,7 +708,7 @@ int32_t launch_hier_merge(int64_t T, int32_t k1, int32_t k2, int32_t b, const in
                           cudaStream_t st) {
     const int64_t total = T * k1 * k2;
     if (total == 0) return MOE_OK;
-    hier_merge_kernel<<<(unsigned)cdiv(total, 256), 256, 0, st>>>(total, k1, k2, b, idx_p, g_p, idx_s, g_s,
+    launch_kernel(hier_merge_kernel, (unsigned)cdiv(total, 256), 256, 0, st, total, k1, k2, b, idx_p, g_p, idx_s, g_s,
                                                                     topk_idx, gates);
     MOE_LAUNCHED();
     return MOE_OK;

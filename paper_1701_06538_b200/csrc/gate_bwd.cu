@@ -19,6 +19,7 @@ __global__ void __launch_bounds__(256) gate_logit_grads_kernel(
     const int32_t *__restrict__ idx, const float *__restrict__ gates, const float *__restrict__ kth_vals,
     const int32_t *__restrict__ kth_idx, const float *__restrict__ dgates, const float *__restrict__ dload,
     const int32_t *__restrict__ dload_row_group, int64_t rows, int32_t n, int32_t k, float *__restrict__ dlogit, bf16 *__restrict__ dsplit, const int32_t *__restrict__ split_row_index) {
+    wait_previous_kernel();
     const int lane = threadIdx.x & 31;
     const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (row >= rows) return;
@@ -143,6 +144,7 @@ __global__ void __launch_bounds__(256) gate_logit_grads_pairs_kernel(
     const int32_t *__restrict__ kth_idx, const float *__restrict__ dgates, const float *__restrict__ dload,
     const int32_t *__restrict__ dload_row_group, int64_t rows, int32_t n, int32_t k, bf16 *__restrict__ dsplit,
     const int32_t *__restrict__ split_row_index) {
+    wait_previous_kernel();
     const int lane = threadIdx.x & 31;
     const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (row >= rows) return;
@@ -240,7 +242,7 @@ int32_t launch_gate_logit_grads(const float *noise, const float *clean, const fl
     const unsigned grid = (unsigned)cdiv(rows, 8);
     if (dsplit && n % 32 == 0 && n <= 256) {  // the tensor-core path: paired columns
 #define MOE_LOGIT_PAIRS_KS(NVP, KS)                                                                                      \
-    gate_logit_grads_pairs_kernel<NVP, KS><<<grid, 256, 0, st>>>(noise, clean, raw, idx, gates, kth_vals, kth_idx, dgates, \
+    launch_kernel((gate_logit_grads_pairs_kernel<NVP, KS>), grid, 256, 0, st, noise, clean, raw, idx, gates, kth_vals, kth_idx, dgates, \
                                                                  dload, dload_row_group, rows, n, k, (bf16 *)dsplit,      \
                                                                  split_row_index)
 #define MOE_LOGIT_PAIRS(NVP)                                \
@@ -258,7 +260,7 @@ int32_t launch_gate_logit_grads(const float *noise, const float *clean, const fl
         return MOE_OK;
     }
 #define MOE_LOGIT_GRADS(NV)                                                                                          \
-    gate_logit_grads_kernel<NV><<<grid, 256, 0, st>>>(noise, clean, raw, idx, gates, kth_vals, kth_idx, dgates, dload, \
+    launch_kernel(gate_logit_grads_kernel<NV>, grid, 256, 0, st, noise, clean, raw, idx, gates, kth_vals, kth_idx, dgates, dload, \
                                                       dload_row_group, rows, n, k, dlogit, (bf16 *)dsplit,      \
                                                       split_row_index)
     if (n <= 32) MOE_LOGIT_GRADS(1);

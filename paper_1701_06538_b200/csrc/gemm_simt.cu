@@ -61,6 +61,7 @@ struct SimtRun {
 // instead and counts as zero.
 template <typename TA, typename TB, typename TC, bool VEC, bool AK, bool BJ, int BM, int BN, int TM, int TN, int BK>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN), TM * TN >= 64 ? 3 : TM * TN >= 32 ? 4 : 8) simt_gemm_kernel(const __grid_constant__ SimtRun run) {
+    wait_previous_kernel();
     constexpr int NTX = BN / TN, NTY = BM / TM, NT = NTX * NTY;
     constexpr int LDA = BM + 4, LDB = BN + 4;
     constexpr int QA = BM * BK / 4 / NT, QB = BN * BK / 4 / NT;  // quads a thread stages per K block
@@ -341,6 +342,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), TM * TN >= 64 ? 3 : TM 
 
 // C (and C2) = the slices' partial results added in double, in slice order
 __global__ void __launch_bounds__(256) simt_reduce_kernel(const __grid_constant__ SimtRun run) {
+    wait_previous_kernel();
     const SimtGemm &g = run.g;
     const int64_t per = g.M * g.N, total = per * g.nseg;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -391,10 +393,10 @@ static int32_t simt_launch(SimtRun &run, int32_t *tile_prefix, cudaStream_t st) 
     }
     if (grid.y > 65535 || grid.z > 65535) return MOE_ERR_UNSUPPORTED;
     run.tile_prefix = tile_prefix;
-    simt_gemm_kernel<TA, TB, TC, VEC, AK, BJ, BM, BN, TM, TN, BK><<<grid, (BM / TM) * (BN / TN), 0, st>>>(run);
+    launch_kernel((simt_gemm_kernel<TA, TB, TC, VEC, AK, BJ, BM, BN, TM, TN, BK>), grid, (BM / TM) * (BN / TN), 0, st, run);
     MOE_LAUNCHED();
     if (run.part) {
-        simt_reduce_kernel<<<(unsigned)cdiv(g.M * g.N * g.nseg, 256), 256, 0, st>>>(run);
+        launch_kernel(simt_reduce_kernel, (unsigned)cdiv(g.M * g.N * g.nseg, 256), 256, 0, st, run);
         MOE_LAUNCHED();
     }
     return MOE_OK;
@@ -479,6 +481,7 @@ __global__ void __launch_bounds__(256) colsum_partial_kernel(const XT *__restric
                                                              const int32_t *__restrict__ offsets, int32_t nseg,
                                                              int32_t N, const int32_t *__restrict__ tile_prefix,
                                                              float *__restrict__ part) {
+    wait_previous_kernel();
     constexpr int V = 16 / sizeof(XT);
     __shared__ float sh[8][32 * V];
     const int32_t b = blockIdx.x;
@@ -535,6 +538,7 @@ template <typename XT>
 __global__ void __launch_bounds__(256) colsum_final_kernel(const float *__restrict__ part, int32_t N,
                                                            const int32_t *__restrict__ tile_prefix,
                                                            XT *__restrict__ out) {
+    wait_previous_kernel();
     __shared__ float sh[8][32];
     const int32_t e = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int32_t j = blockIdx.y * 32 + lane;
@@ -568,13 +572,13 @@ int32_t launch_segment_colsum(const void *in, int32_t act, const int32_t *offset
     dim3 g1((unsigned)(cdiv(R, CS_ROWS) + nseg), (unsigned)cdiv(N, vcols));
     dim3 g2((unsigned)nseg, (unsigned)cdiv(N, 32));
     if (act == MOE_BF16) {
-        colsum_partial_kernel<bf16><<<g1, 256, 0, st>>>((const bf16 *)in, offsets, nseg, N, tile_prefix, scratch);
+        launch_kernel(colsum_partial_kernel<bf16>, g1, 256, 0, st, (const bf16 *)in, offsets, nseg, N, tile_prefix, scratch);
         MOE_LAUNCHED();
-        colsum_final_kernel<bf16><<<g2, 256, 0, st>>>(scratch, N, tile_prefix, (bf16 *)out);
+        launch_kernel(colsum_final_kernel<bf16>, g2, 256, 0, st, scratch, N, tile_prefix, (bf16 *)out);
     } else {
-        colsum_partial_kernel<float><<<g1, 256, 0, st>>>((const float *)in, offsets, nseg, N, tile_prefix, scratch);
+        launch_kernel(colsum_partial_kernel<float>, g1, 256, 0, st, (const float *)in, offsets, nseg, N, tile_prefix, scratch);
         MOE_LAUNCHED();
-        colsum_final_kernel<float><<<g2, 256, 0, st>>>(scratch, N, tile_prefix, (float *)out);
+        launch_kernel(colsum_final_kernel<float>, g2, 256, 0, st, scratch, N, tile_prefix, (float *)out);
     }
     MOE_LAUNCHED();
     return MOE_OK;

@@ -7,6 +7,7 @@ namespace moe {
 // idx_p[t, s1] = group of primary slot s1; idx_s[p, s2] = expert inside that group
 __global__ void hier_split_idx_kernel(const int32_t *__restrict__ topk_idx, int64_t total, int32_t k2, int32_t a,
                                       int32_t b, int32_t *__restrict__ idx_p, int32_t *__restrict__ idx_s) {
+    wait_previous_kernel();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // over T*k1*k2
     if (i >= total) return;
     int32_t id = topk_idx[i];
@@ -20,7 +21,7 @@ int32_t launch_hier_split_idx(const int32_t *topk_idx, int64_t T, int32_t k1, in
                               int32_t *idx_p, int32_t *idx_s, cudaStream_t st) {
     const int64_t total = T * k1 * k2;
     if (total == 0) return MOE_OK;
-    hier_split_idx_kernel<<<(unsigned)cdiv(total, 256), 256, 0, st>>>(topk_idx, total, k2, a, b, idx_p, idx_s);
+    launch_kernel(hier_split_idx_kernel, (unsigned)cdiv(total, 256), 256, 0, st, topk_idx, total, k2, a, b, idx_p, idx_s);
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -30,6 +31,7 @@ __global__ void __launch_bounds__(256) segment_sum_kernel(const float *__restric
                                                           const int32_t *__restrict__ perm,
                                                           const int32_t *__restrict__ offsets, int32_t nseg,
                                                           float *__restrict__ out) {
+    wait_previous_kernel();
     const int lane = threadIdx.x & 31;
     const int32_t e = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (e >= nseg) return;
@@ -42,7 +44,7 @@ __global__ void __launch_bounds__(256) segment_sum_kernel(const float *__restric
 
 int32_t launch_segment_sum(const float *vals, const int32_t *perm, const int32_t *offsets, int32_t nseg, float *out,
                            cudaStream_t st) {
-    segment_sum_kernel<<<(unsigned)cdiv(nseg, 8), 256, 0, st>>>(vals, perm, offsets, nseg, out);
+    launch_kernel(segment_sum_kernel, (unsigned)cdiv(nseg, 8), 256, 0, st, vals, perm, offsets, nseg, out);
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -59,6 +61,7 @@ __global__ void __launch_bounds__(256) grouped_load_partial_kernel(
     const int32_t *__restrict__ idx_s, const float *__restrict__ clean, const float *__restrict__ raw,
     const float *__restrict__ kth_vals, const int32_t *__restrict__ perm, const int32_t *__restrict__ offsets,
     const int32_t *__restrict__ tile_prefix, int32_t nseg, int32_t n, int32_t k, int32_t CW, float *__restrict__ part) {
+    wait_previous_kernel();
     __shared__ float red[256];
     const int32_t b = blockIdx.x;
     if (b >= tile_prefix[nseg]) return;
@@ -96,6 +99,7 @@ __global__ void __launch_bounds__(256) grouped_load_partial_kernel(
 __global__ void __launch_bounds__(256) grouped_reduce_kernel(const float *__restrict__ part,
                                                              const int32_t *__restrict__ tile_prefix, int32_t n,
                                                              float *__restrict__ out) {
+    wait_previous_kernel();
     const int32_t e = blockIdx.x;
     const int32_t j = blockIdx.y * 256 + threadIdx.x;
     if (j >= n) return;
@@ -110,10 +114,10 @@ int32_t launch_grouped_load(const int32_t *idx_s, const float *clean, const floa
     MOE_TRY(launch_tile_prefix(offsets, nseg, GS_ROWS, tile_prefix, st));
     int32_t CW = 1;
     while (CW < n && CW < 256) CW <<= 1;
-    grouped_load_partial_kernel<<<(unsigned)(cdiv(rows, GS_ROWS) + nseg), 256, 0, st>>>(
+    launch_kernel(grouped_load_partial_kernel, (unsigned)(cdiv(rows, GS_ROWS) + nseg), 256, 0, st, 
         idx_s, clean, raw, kth_vals, perm, offsets, tile_prefix, nseg, n, k, CW, scratch);
     MOE_LAUNCHED();
-    grouped_reduce_kernel<<<dim3((unsigned)nseg, (unsigned)cdiv(n, 256)), 256, 0, st>>>(scratch, tile_prefix, n, out);
+    launch_kernel(grouped_reduce_kernel, dim3((unsigned)nseg, (unsigned)cdiv(n, 256)), 256, 0, st, scratch, tile_prefix, n, out);
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -121,6 +125,7 @@ int32_t launch_grouped_load(const int32_t *idx_s, const float *clean, const floa
 // Load_H[i,j] = Load_primary[i] * Load_i[j] / |X^(i)|  (Eq. 14); a group nobody selected gets 0.
 // load layout: [a*b] Load_H | [a] Load_primary | [a*b] Load_i | [a] |X^(i)|
 __global__ void load_h_kernel(float *__restrict__ load, const int32_t *__restrict__ counts_p, int32_t a, int32_t b) {
+    wait_previous_kernel();
     const int32_t i = blockIdx.x;
     const float *load_p = load + (int64_t)a * b, *load_s = load_p + a;
     float *cnt = load + 2 * (int64_t)a * b + a;
@@ -131,7 +136,7 @@ __global__ void load_h_kernel(float *__restrict__ load, const int32_t *__restric
 }
 
 int32_t launch_load_h(float *load, const int32_t *counts_p, int32_t a, int32_t b, cudaStream_t st) {
-    load_h_kernel<<<a, 128, 0, st>>>(load, counts_p, a, b);
+    launch_kernel(load_h_kernel, a, 128, 0, st, load, counts_p, a, b);
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -141,6 +146,7 @@ int32_t launch_load_h(float *load, const int32_t *counts_p, int32_t a, int32_t b
 __global__ void __launch_bounds__(128) load_h_bwd_kernel(const float *__restrict__ load,
                                                          const float *__restrict__ dload_h, int32_t a, int32_t b,
                                                          float *__restrict__ dload) {
+    wait_previous_kernel();
     __shared__ double red[128];
     const int32_t i = blockIdx.x;
     const float *load_p = load + (int64_t)a * b, *load_s = load_p + a, *cnt = load + 2 * (int64_t)a * b + a;
@@ -162,7 +168,7 @@ __global__ void __launch_bounds__(128) load_h_bwd_kernel(const float *__restrict
 
 int32_t launch_load_h_bwd(const float *load, const float *dload_h, int32_t a, int32_t b, float *dload,
                           cudaStream_t st) {
-    load_h_bwd_kernel<<<a, 128, 0, st>>>(load, dload_h, a, b, dload);
+    launch_kernel(load_h_bwd_kernel, a, 128, 0, st, load, dload_h, a, b, dload);
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -171,6 +177,7 @@ int32_t launch_load_h_bwd(const float *load, const float *dload_h, int32_t a, in
 // gates / dgates layout: [T, k] product | [T, k1] primary | [T, k1, k2] secondary
 __global__ void hier_gate_product_bwd_kernel(const float *__restrict__ gates, float *__restrict__ dgates, int64_t P1,
                                              int32_t k2, int64_t Tk) {
+    wait_previous_kernel();
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // slot (t, s1)
     if (p >= P1) return;
     const float *g_p = gates + Tk, *g_s = g_p + P1;
@@ -188,7 +195,7 @@ int32_t launch_hier_gate_product_bwd(const float *gates, float *dgates, int64_t 
                                      cudaStream_t st) {
     const int64_t P1 = T * k1;
     if (P1 == 0) return MOE_OK;
-    hier_gate_product_bwd_kernel<<<(unsigned)cdiv(P1, 256), 256, 0, st>>>(gates, dgates, P1, k2, T * k1 * k2);
+    launch_kernel(hier_gate_product_bwd_kernel, (unsigned)cdiv(P1, 256), 256, 0, st, gates, dgates, P1, k2, T * k1 * k2);
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -196,6 +203,7 @@ int32_t launch_hier_gate_product_bwd(const float *gates, float *dgates, int64_t 
 // dX_gate[t] += sum_s1 dX_sec[t*k1 + s1]   (both float, [.., d])
 __global__ void add_slot_rows_kernel(const float *__restrict__ dX_sec, int64_t total, int32_t k1, int32_t d,
                                      float *__restrict__ dX_gate) {
+    wait_previous_kernel();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // over T*d
     if (i >= total) return;
     const int64_t t = i / d, q = i % d;
@@ -207,7 +215,7 @@ __global__ void add_slot_rows_kernel(const float *__restrict__ dX_sec, int64_t t
 int32_t launch_add_slot_rows(const float *dX_sec, int64_t T, int32_t k1, int32_t d, float *dX_gate, cudaStream_t st) {
     const int64_t total = T * d;
     if (total == 0) return MOE_OK;
-    add_slot_rows_kernel<<<(unsigned)cdiv(total, 256), 256, 0, st>>>(dX_sec, total, k1, d, dX_gate);
+    launch_kernel(add_slot_rows_kernel, (unsigned)cdiv(total, 256), 256, 0, st, dX_sec, total, k1, d, dX_gate);
     MOE_LAUNCHED();
     return MOE_OK;
 }

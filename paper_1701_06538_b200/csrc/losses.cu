@@ -23,6 +23,7 @@ __global__ void __launch_bounds__(256) level_sums_kernel(const int32_t *__restri
                                                          const float *__restrict__ kth_vals, int64_t rows, int32_t n,
                                                          int32_t k, int32_t CW, float *__restrict__ part_imp,
                                                          float *__restrict__ part_load) {
+    wait_previous_kernel();
     __shared__ float red_i[256], red_l[256];
     const int cw = threadIdx.x % CW, tl = threadIdx.x / CW, TL = 256 / CW;
     const int64_t per = (rows + gridDim.x - 1) / gridDim.x;
@@ -66,6 +67,7 @@ __global__ void __launch_bounds__(256) level_sums_rows_kernel(const int32_t *__r
                                                               const float *__restrict__ kth_vals, int64_t rows,
                                                               int32_t n, int32_t k, float *__restrict__ part_imp,
                                                               float *__restrict__ part_load) {
+    wait_previous_kernel();
     __shared__ float red[2][8][32 * NV];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t per = (rows + gridDim.x - 1) / gridDim.x;
@@ -122,6 +124,7 @@ __global__ void __launch_bounds__(256) level_reduce_kernel(const float *__restri
                                                            const float *__restrict__ part_load, int32_t chunks,
                                                            int32_t n, float *__restrict__ importance,
                                                            float *__restrict__ load) {
+    wait_previous_kernel();
     __shared__ double red[2][8][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int32_t j = blockIdx.x * 32 + lane;
@@ -168,13 +171,13 @@ int32_t launch_level_sums(const int32_t *idx, const float *gates, const float *c
     int32_t CW = 1;
     while (CW < n && CW < 256) CW <<= 1;
     float *part_imp = scratch, *part_load = scratch + (int64_t)chunks * n;
-    if (n <= 32) level_sums_rows_kernel<1><<<chunks, 256, 0, st>>>(idx, gates, clean, raw, kth_vals, rows, n, k, part_imp, part_load);
-    else if (n <= 64) level_sums_rows_kernel<2><<<chunks, 256, 0, st>>>(idx, gates, clean, raw, kth_vals, rows, n, k, part_imp, part_load);
-    else if (n <= 128) level_sums_rows_kernel<4><<<chunks, 256, 0, st>>>(idx, gates, clean, raw, kth_vals, rows, n, k, part_imp, part_load);
-    else if (n <= 256) level_sums_rows_kernel<8><<<chunks, 256, 0, st>>>(idx, gates, clean, raw, kth_vals, rows, n, k, part_imp, part_load);
-    else level_sums_kernel<<<chunks, 256, 0, st>>>(idx, gates, clean, raw, kth_vals, rows, n, k, CW, part_imp, part_load);
+    if (n <= 32) launch_kernel(level_sums_rows_kernel<1>, chunks, 256, 0, st, idx, gates, clean, raw, kth_vals, rows, n, k, part_imp, part_load);
+    else if (n <= 64) launch_kernel(level_sums_rows_kernel<2>, chunks, 256, 0, st, idx, gates, clean, raw, kth_vals, rows, n, k, part_imp, part_load);
+    else if (n <= 128) launch_kernel(level_sums_rows_kernel<4>, chunks, 256, 0, st, idx, gates, clean, raw, kth_vals, rows, n, k, part_imp, part_load);
+    else if (n <= 256) launch_kernel(level_sums_rows_kernel<8>, chunks, 256, 0, st, idx, gates, clean, raw, kth_vals, rows, n, k, part_imp, part_load);
+    else launch_kernel(level_sums_kernel, chunks, 256, 0, st, idx, gates, clean, raw, kth_vals, rows, n, k, CW, part_imp, part_load);
     MOE_LAUNCHED();
-    level_reduce_kernel<<<(unsigned)cdiv(n, 32), 256, 0, st>>>(part_imp, part_load, chunks, n, importance_out,
+    launch_kernel(level_reduce_kernel, (unsigned)cdiv(n, 32), 256, 0, st, part_imp, part_load, chunks, n, importance_out,
                                                                  load_out);
     MOE_LAUNCHED();
     return MOE_OK;
@@ -211,6 +214,7 @@ __device__ Moments block_moments(const float *v, int32_t m, double *sh) {
 
 __global__ void __launch_bounds__(256) cv2_kernel(const float *importance, int32_t n_imp, const float *load,
                                                   int32_t n_load, float w_imp, float w_load, float *losses) {
+    wait_previous_kernel();
     __shared__ double sh[256];
     Moments a = block_moments(importance, n_imp, sh);
     Moments b = block_moments(load, n_load, sh);
@@ -222,13 +226,14 @@ __global__ void __launch_bounds__(256) cv2_kernel(const float *importance, int32
 
 int32_t launch_cv2(const float *importance, int32_t n_imp, const float *load, int32_t n_load, float w_imp,
                    float w_load, float *losses, cudaStream_t st) {
-    cv2_kernel<<<1, 256, 0, st>>>(importance, n_imp, load, n_load, w_imp, w_load, losses);
+    launch_kernel(cv2_kernel, 1, 256, 0, st, importance, n_imp, load, n_load, w_imp, w_load, losses);
     MOE_LAUNCHED();
     return MOE_OK;
 }
 
 // out[i] = scale * dCV^2/dv_i
 __global__ void __launch_bounds__(256) cv2_grad_kernel(const float *v, int32_t m, float scale, float *out) {
+    wait_previous_kernel();
     __shared__ double sh[256];
     Moments a = block_moments(v, m, sh);
     const double c = 2.0 / ((double)m * a.mu * a.mu);
@@ -238,6 +243,7 @@ __global__ void __launch_bounds__(256) cv2_grad_kernel(const float *v, int32_t m
 
 // dgates[p] += dimp[topk_idx[p]]; an expert id outside [0, n) adds nothing
 __global__ void add_gathered_kernel(float *dgates, const int32_t *topk_idx, const float *dimp, int64_t R, int32_t n) {
+    wait_previous_kernel();
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= R) return;
     const int32_t e = topk_idx[p];
@@ -246,7 +252,7 @@ __global__ void add_gathered_kernel(float *dgates, const int32_t *topk_idx, cons
 }
 
 int32_t launch_cv2_grad(const float *v, int32_t m, float scale, float *out, cudaStream_t st) {
-    cv2_grad_kernel<<<1, 256, 0, st>>>(v, m, scale, out);
+    launch_kernel(cv2_grad_kernel, 1, 256, 0, st, v, m, scale, out);
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -254,7 +260,7 @@ int32_t launch_cv2_grad(const float *v, int32_t m, float scale, float *out, cuda
 int32_t launch_add_gathered(float *dgates, const int32_t *topk_idx, const float *dimp, int64_t R, int32_t n,
                             cudaStream_t st) {
     if (R == 0) return MOE_OK;
-    add_gathered_kernel<<<(unsigned)cdiv(R, 256), 256, 0, st>>>(dgates, topk_idx, dimp, R, n);
+    launch_kernel(add_gathered_kernel, (unsigned)cdiv(R, 256), 256, 0, st, dgates, topk_idx, dimp, R, n);
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -262,12 +268,12 @@ int32_t launch_add_gathered(float *dgates, const int32_t *topk_idx, const float 
 int32_t launch_losses_bwd_flat(const float *importance, const float *load, int32_t n, const int32_t *topk_idx,
                                int64_t R, float w_imp, float w_load, float *dgates, float *dload, float *dimp_tmp,
                                cudaStream_t st) {
-    cv2_grad_kernel<<<1, 256, 0, st>>>(importance, n, w_imp, dimp_tmp);
+    launch_kernel(cv2_grad_kernel, 1, 256, 0, st, importance, n, w_imp, dimp_tmp);
     MOE_LAUNCHED();
-    cv2_grad_kernel<<<1, 256, 0, st>>>(load, n, w_load, dload);
+    launch_kernel(cv2_grad_kernel, 1, 256, 0, st, load, n, w_load, dload);
     MOE_LAUNCHED();
     if (R > 0) {
-        add_gathered_kernel<<<(unsigned)cdiv(R, 256), 256, 0, st>>>(dgates, topk_idx, dimp_tmp, R, n);
+        launch_kernel(add_gathered_kernel, (unsigned)cdiv(R, 256), 256, 0, st, dgates, topk_idx, dimp_tmp, R, n);
         MOE_LAUNCHED();
     }
     return MOE_OK;

@@ -26,6 +26,7 @@ template <typename XT>
 __global__ void __launch_bounds__(256) adam_averages_kernel(const XT *__restrict__ g, int32_t rows, int32_t cols,
                                                             float beta2, float *__restrict__ row_avg,
                                                             float *__restrict__ colpart) {
+    wait_previous_kernel();
     constexpr int VN = Vec<XT>::N;
     __shared__ float warp_rows[8][RB];
     const int32_t e = blockIdx.y, rb = blockIdx.x, nrb = gridDim.x;
@@ -86,6 +87,7 @@ __global__ void __launch_bounds__(256) adam_columns_kernel(const float *__restri
                                                            int32_t cols, float beta2, float *__restrict__ col_avg,
                                                            const float *__restrict__ row_avg,
                                                            float *__restrict__ row_mean) {
+    wait_previous_kernel();
     __shared__ double part[256];
     const int32_t e = blockIdx.y;
     const int32_t j = blockIdx.x * 256 + threadIdx.x;
@@ -125,6 +127,7 @@ __global__ void __launch_bounds__(256) adam_update_kernel(XT *__restrict__ W, co
                                                           const float *__restrict__ col_avg,
                                                           const float *__restrict__ row_mean, float lr,
                                                           float inv_correction, float eps) {
+    wait_previous_kernel();
     constexpr int VN = Vec<XT>::N;
     const int32_t e = blockIdx.y;
     const float rm = row_mean[e];
@@ -163,6 +166,7 @@ template <typename XT>
 __global__ void __launch_bounds__(256) adam_vector_kernel(XT *__restrict__ b, const XT *__restrict__ g, int64_t count,
                                                           float *__restrict__ v, float lr, float beta2,
                                                           float inv_correction, float eps) {
+    wait_previous_kernel();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= count) return;
     const float gi = to_f32(g[i]);
@@ -177,12 +181,12 @@ int32_t adam_matrix(XT *W, const XT *g, int32_t n, int32_t rows, int32_t cols, f
     const int32_t nrb = (int32_t)cdiv(rows, RB);
     const int nvec = cols / (int)(16 / sizeof(XT));
     const unsigned threads = (unsigned)imin(256, cdiv(nvec, 32) * 32);
-    adam_averages_kernel<XT><<<dim3((unsigned)nrb, (unsigned)n), threads, 0, st>>>(g, rows, cols, beta2, row_avg, colpart);
+    launch_kernel(adam_averages_kernel<XT>, dim3((unsigned)nrb, (unsigned)n), threads, 0, st, g, rows, cols, beta2, row_avg, colpart);
     MOE_LAUNCHED();
-    adam_columns_kernel<<<dim3((unsigned)cdiv(cols, 256), (unsigned)n), 256, 0, st>>>(colpart, nrb, rows, cols, beta2, col_avg, row_avg,
+    launch_kernel(adam_columns_kernel, dim3((unsigned)cdiv(cols, 256), (unsigned)n), 256, 0, st, colpart, nrb, rows, cols, beta2, col_avg, row_avg,
                                                                                      row_mean);
     MOE_LAUNCHED();
-    adam_update_kernel<XT><<<dim3((unsigned)cdiv(rows, UR), (unsigned)n), 256, 0, st>>>(W, g, rows, cols, row_avg, col_avg,
+    launch_kernel(adam_update_kernel<XT>, dim3((unsigned)cdiv(rows, UR), (unsigned)n), 256, 0, st, W, g, rows, cols, row_avg, col_avg,
                                                                                        row_mean, lr, inv_correction, eps);
     MOE_LAUNCHED();
     return MOE_OK;
@@ -207,16 +211,16 @@ int32_t launch_expert_adam(int32_t act, int32_t n, int32_t d, int32_t h, void *W
     if (act == MOE_BF16) {
         MOE_TRY(adam_matrix<bf16>((bf16 *)W1, (const bf16 *)dW1, n, d, h, r1, c1, lr, beta2, inv_correction, eps, colpart, row_mean, st));
         MOE_TRY(adam_matrix<bf16>((bf16 *)W2, (const bf16 *)dW2, n, h, d, r2, c2, lr, beta2, inv_correction, eps, colpart, row_mean, st));
-        adam_vector_kernel<bf16><<<gb1, 256, 0, st>>>((bf16 *)b1, (const bf16 *)db1, (int64_t)n * h, vb1, lr, beta2, inv_correction, eps);
+        launch_kernel(adam_vector_kernel<bf16>, gb1, 256, 0, st, (bf16 *)b1, (const bf16 *)db1, (int64_t)n * h, vb1, lr, beta2, inv_correction, eps);
         MOE_LAUNCHED();
-        adam_vector_kernel<bf16><<<gb2, 256, 0, st>>>((bf16 *)b2, (const bf16 *)db2, (int64_t)n * d, vb2, lr, beta2, inv_correction, eps);
+        launch_kernel(adam_vector_kernel<bf16>, gb2, 256, 0, st, (bf16 *)b2, (const bf16 *)db2, (int64_t)n * d, vb2, lr, beta2, inv_correction, eps);
         MOE_LAUNCHED();
     } else {
         MOE_TRY(adam_matrix<float>((float *)W1, (const float *)dW1, n, d, h, r1, c1, lr, beta2, inv_correction, eps, colpart, row_mean, st));
         MOE_TRY(adam_matrix<float>((float *)W2, (const float *)dW2, n, h, d, r2, c2, lr, beta2, inv_correction, eps, colpart, row_mean, st));
-        adam_vector_kernel<float><<<gb1, 256, 0, st>>>((float *)b1, (const float *)db1, (int64_t)n * h, vb1, lr, beta2, inv_correction, eps);
+        launch_kernel(adam_vector_kernel<float>, gb1, 256, 0, st, (float *)b1, (const float *)db1, (int64_t)n * h, vb1, lr, beta2, inv_correction, eps);
         MOE_LAUNCHED();
-        adam_vector_kernel<float><<<gb2, 256, 0, st>>>((float *)b2, (const float *)db2, (int64_t)n * d, vb2, lr, beta2, inv_correction, eps);
+        launch_kernel(adam_vector_kernel<float>, gb2, 256, 0, st, (float *)b2, (const float *)db2, (int64_t)n * d, vb2, lr, beta2, inv_correction, eps);
         MOE_LAUNCHED();
     }
     return MOE_OK;

@@ -23,6 +23,7 @@ int64_t dispatch_ws_elems(int64_t R, int32_t n) { return cdiv(R, CH) * (int64_t)
 
 __global__ void __launch_bounds__(256) dispatch_hist_kernel(const int32_t *__restrict__ topk_idx, int64_t R,
                                                             int32_t n, int32_t *__restrict__ chunk_hist) {
+    wait_previous_kernel();
     extern __shared__ int32_t sh[];
     for (int e = threadIdx.x; e < n; e += blockDim.x) sh[e] = 0;
     __syncthreads();
@@ -43,6 +44,7 @@ __global__ void __launch_bounds__(256) dispatch_hist_kernel(const int32_t *__res
 __global__ void __launch_bounds__(1024) dispatch_scan_chunks_kernel(int32_t *__restrict__ chunk_hist,
                                                                     int32_t nchunks, int32_t n,
                                                                     int32_t *__restrict__ counts) {
+    wait_previous_kernel();
     __shared__ int32_t part[32][33];
     const int el = threadIdx.x & 31, cl = threadIdx.x >> 5;
     const int32_t e = blockIdx.x * 32 + el;
@@ -72,6 +74,7 @@ __global__ void __launch_bounds__(1024) dispatch_scan_chunks_kernel(int32_t *__r
 
 __global__ void __launch_bounds__(1024) dispatch_scan_experts_kernel(const int32_t *__restrict__ counts, int32_t n,
                                                                      int32_t *__restrict__ offsets) {
+    wait_previous_kernel();
     __shared__ int32_t warp_sum[32];
     __shared__ int32_t carry;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -142,6 +145,7 @@ __global__ void __launch_bounds__(1024) dispatch_rank_kernel(const int32_t *__re
                                                              const int32_t *__restrict__ chunk_table, int32_t nchunks,
                                                              int32_t *__restrict__ counts, int32_t *__restrict__ offsets,
                                                              int32_t *__restrict__ perm, int32_t *__restrict__ inv_perm) {
+    wait_previous_kernel();
     extern __shared__ int32_t cursor[];  // next sorted row of each expert for this chunk
     __shared__ int32_t sh[32];
     __shared__ int32_t part_total[1024], part_before[1024];
@@ -232,22 +236,22 @@ int32_t launch_dispatch_index(const int32_t *topk_idx, int64_t R, int32_t n, int
     // one chunk: one launch. Up to 64 Ki histogram entries every block can afford to read them all (128 chunks x 256
     // experts: 1.5 us), which saves the two scans' launches.
     if (nchunks == 1 && n <= 8192) {
-        dispatch_rank_kernel<RANK_ONE><<<1, 1024, sh, st>>>(topk_idx, R, n, nullptr, 1, counts, offsets, perm, inv_perm);
+        launch_kernel(dispatch_rank_kernel<RANK_ONE>, 1, 1024, sh, st, topk_idx, R, n, nullptr, 1, counts, offsets, perm, inv_perm);
         MOE_LAUNCHED();
         return MOE_OK;
     }
-    dispatch_hist_kernel<<<nchunks, 256, sh, st>>>(topk_idx, R, n, scratch);
+    launch_kernel(dispatch_hist_kernel, nchunks, 256, sh, st, topk_idx, R, n, scratch);
     MOE_LAUNCHED();
     if (n <= 1024 && (int64_t)nchunks * n <= 65536) {
-        dispatch_rank_kernel<RANK_FEW><<<nchunks, 1024, sh, st>>>(topk_idx, R, n, scratch, nchunks, counts, offsets, perm, inv_perm);
+        launch_kernel(dispatch_rank_kernel<RANK_FEW>, nchunks, 1024, sh, st, topk_idx, R, n, scratch, nchunks, counts, offsets, perm, inv_perm);
         MOE_LAUNCHED();
         return MOE_OK;
     }
-    dispatch_scan_chunks_kernel<<<(unsigned)cdiv(n, 32), 1024, 0, st>>>(scratch, nchunks, n, counts);
+    launch_kernel(dispatch_scan_chunks_kernel, (unsigned)cdiv(n, 32), 1024, 0, st, scratch, nchunks, n, counts);
     MOE_LAUNCHED();
-    dispatch_scan_experts_kernel<<<1, 1024, 0, st>>>(counts, n, offsets);
+    launch_kernel(dispatch_scan_experts_kernel, 1, 1024, 0, st, counts, n, offsets);
     MOE_LAUNCHED();
-    dispatch_rank_kernel<RANK_MANY><<<nchunks, 1024, sh, st>>>(topk_idx, R, n, scratch, nchunks, counts, offsets, perm, inv_perm);
+    launch_kernel(dispatch_rank_kernel<RANK_MANY>, nchunks, 1024, sh, st, topk_idx, R, n, scratch, nchunks, counts, offsets, perm, inv_perm);
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -278,6 +282,7 @@ __device__ __forceinline__ int32_t block_sum_1024(int32_t v, int32_t *sh /* [32]
 }
 __global__ void __launch_bounds__(1024) scan_tile_sums_kernel(const int32_t *__restrict__ counts, int32_t n,
                                                               int32_t *__restrict__ tile_sums) {
+    wait_previous_kernel();
     __shared__ int32_t sh[32];
     const int4 v = scan_tile_load(counts, n, blockIdx.x * SCAN_TILE + threadIdx.x * 4);
     const int32_t total = block_sum_1024(v.x + v.y + v.z + v.w, sh);
@@ -286,6 +291,7 @@ __global__ void __launch_bounds__(1024) scan_tile_sums_kernel(const int32_t *__r
 __global__ void __launch_bounds__(1024) scan_tiles_kernel(const int32_t *__restrict__ counts, int32_t n,
                                                           const int32_t *__restrict__ tile_sums,
                                                           int32_t *__restrict__ offsets) {
+    wait_previous_kernel();
     __shared__ int32_t sh[32];
     __shared__ int32_t warp_excl[32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -330,13 +336,13 @@ __global__ void __launch_bounds__(1024) scan_tiles_kernel(const int32_t *__restr
 int32_t launch_exclusive_scan(const int32_t *counts, int32_t n, int32_t *out, cudaStream_t st, int32_t *tile_sums) {
     if (n > 8192 && tile_sums) {
         const unsigned tiles = (unsigned)cdiv(n + 1, SCAN_TILE);  // position n (the total) falls into a tile as well
-        scan_tile_sums_kernel<<<tiles, 1024, 0, st>>>(counts, n, tile_sums);
+        launch_kernel(scan_tile_sums_kernel, tiles, 1024, 0, st, counts, n, tile_sums);
         MOE_LAUNCHED();
-        scan_tiles_kernel<<<tiles, 1024, 0, st>>>(counts, n, tile_sums, out);
+        launch_kernel(scan_tiles_kernel, tiles, 1024, 0, st, counts, n, tile_sums, out);
         MOE_LAUNCHED();
         return MOE_OK;
     }
-    dispatch_scan_experts_kernel<<<1, 1024, 0, st>>>(counts, n, out);
+    launch_kernel(dispatch_scan_experts_kernel, 1, 1024, 0, st, counts, n, out);
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -344,6 +350,7 @@ int32_t launch_exclusive_scan(const int32_t *counts, int32_t n, int32_t *out, cu
 // tile_prefix[e] = number of bm-row tiles of the segments before e (tile_prefix[n] = total)
 __global__ void __launch_bounds__(1024) tile_prefix_kernel(const int32_t *__restrict__ offsets, int32_t n,
                                                            int32_t bm, int32_t *__restrict__ tile_prefix) {
+    wait_previous_kernel();
     __shared__ int32_t warp_sum[32];
     __shared__ int32_t carry;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -380,7 +387,7 @@ __global__ void __launch_bounds__(1024) tile_prefix_kernel(const int32_t *__rest
 }
 
 int32_t launch_tile_prefix(const int32_t *offsets, int32_t n, int32_t bm, int32_t *tile_prefix, cudaStream_t st) {
-    tile_prefix_kernel<<<1, 1024, 0, st>>>(offsets, n, bm, tile_prefix);
+    launch_kernel(tile_prefix_kernel, 1, 1024, 0, st, offsets, n, bm, tile_prefix);
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -400,6 +407,7 @@ template <typename XT>
 __global__ void __launch_bounds__(256) dispatch_rows_kernel(const XT *__restrict__ x, int64_t T, int32_t k,
                                                             int32_t d, const int32_t *__restrict__ inv_perm,
                                                             XT *__restrict__ xs) {
+    wait_previous_kernel();
     constexpr int VN = 16 / sizeof(XT);
     const int lane = threadIdx.x & 31;
     const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -428,9 +436,9 @@ int32_t launch_dispatch_rows(const void *x, int32_t act, int64_t T, int32_t k, i
     if (T == 0) return MOE_OK;
     const unsigned grid = (unsigned)imin(cdiv(T, 8), 148 * 16);
     if (act == MOE_BF16)
-        dispatch_rows_kernel<bf16><<<grid, 256, 0, st>>>((const bf16 *)x, T, k, d, inv_perm, (bf16 *)xs);
+        launch_kernel(dispatch_rows_kernel<bf16>, grid, 256, 0, st, (const bf16 *)x, T, k, d, inv_perm, (bf16 *)xs);
     else
-        dispatch_rows_kernel<float><<<grid, 256, 0, st>>>((const float *)x, T, k, d, inv_perm, (float *)xs);
+        launch_kernel(dispatch_rows_kernel<float>, grid, 256, 0, st, (const float *)x, T, k, d, inv_perm, (float *)xs);
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -462,6 +470,7 @@ __global__ void __launch_bounds__(256, LAYER ? 3 : 1) combine_kernel(const XT *_
                                                       const int32_t *__restrict__ inv_perm, int64_t T, int32_t k,
                                                       int32_t d, XT *__restrict__ y, const XT *__restrict__ xres,
                                                       const uint8_t *__restrict__ keep, float keep_scale) {
+    wait_previous_kernel();
     constexpr int VN = 16 / sizeof(XT);
     const int lane = threadIdx.x & 31;
     const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -525,10 +534,10 @@ int32_t launch_combine(const void *ys, int32_t act, const float *gates, const in
     const unsigned grid = (unsigned)imin(cdiv(T, 8), 148 * 16);
 #define MOE_CALL_L(KT, VB, L)                                                                                         \
     if (act == MOE_BF16)                                                                                              \
-        combine_kernel<bf16, KT, VB, L><<<grid, 256, 0, st>>>((const bf16 *)ys, gates, inv_perm, T, k, d, (bf16 *)y,  \
+        launch_kernel((combine_kernel<bf16, KT, VB, L>), grid, 256, 0, st, (const bf16 *)ys, gates, inv_perm, T, k, d, (bf16 *)y,  \
                                                               (const bf16 *)xres, keep, keep_scale);                  \
     else                                                                                                              \
-        combine_kernel<float, KT, VB, L><<<grid, 256, 0, st>>>((const float *)ys, gates, inv_perm, T, k, d, (float *)y, \
+        launch_kernel((combine_kernel<float, KT, VB, L>), grid, 256, 0, st, (const float *)ys, gates, inv_perm, T, k, d, (float *)y, \
                                                                (const float *)xres, keep, keep_scale)
 #define MOE_CALL(KT, VB)                     \
     if (keep) { MOE_CALL_L(KT, VB, true); }  \
@@ -550,6 +559,7 @@ __global__ void __launch_bounds__(256, LAYER ? 3 : 1) combine_bwd_kernel(const X
                                                           int32_t k, int32_t d, float *__restrict__ dgates,
                                                           XT *__restrict__ dys, const uint8_t *__restrict__ keep,
                                                           float keep_scale) {
+    wait_previous_kernel();
     constexpr int VN = 16 / sizeof(XT);
     const int lane = threadIdx.x & 31;
     const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -631,10 +641,10 @@ int32_t launch_combine_bwd(const void *dY, const void *ys, int32_t act, const fl
     const unsigned grid = (unsigned)imin(cdiv(T, 8), 148 * 16);
 #define MOE_CALL_L(KT, VB, L)                                                                                            \
     if (act == MOE_BF16)                                                                                                 \
-        combine_bwd_kernel<bf16, KT, VB, L><<<grid, 256, 0, st>>>((const bf16 *)dY, (const bf16 *)ys, gates, inv_perm, T, \
+        launch_kernel((combine_bwd_kernel<bf16, KT, VB, L>), grid, 256, 0, st, (const bf16 *)dY, (const bf16 *)ys, gates, inv_perm, T, \
                                                                    k, d, dgates, (bf16 *)dys, keep, keep_scale);          \
     else                                                                                                                 \
-        combine_bwd_kernel<float, KT, VB, L><<<grid, 256, 0, st>>>((const float *)dY, (const float *)ys, gates, inv_perm, \
+        launch_kernel((combine_bwd_kernel<float, KT, VB, L>), grid, 256, 0, st, (const float *)dY, (const float *)ys, gates, inv_perm, \
                                                                     T, k, d, dgates, (float *)dys, keep, keep_scale)
 #define MOE_CALL(KT, VB)                     \
     if (keep) { MOE_CALL_L(KT, VB, true); }  \
@@ -654,6 +664,7 @@ __global__ void __launch_bounds__(256) dispatch_bwd_kernel(const XT *__restrict_
                                                            int32_t k, int32_t d, const float *add,
                                                            float *out_f32, XT *__restrict__ out_act,
                                                            const XT *__restrict__ add_act) {
+    wait_previous_kernel();
     constexpr int VN = 16 / sizeof(XT);
     const int lane = threadIdx.x & 31;
     const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -733,10 +744,10 @@ int32_t launch_dispatch_bwd(const void *dxs, int32_t act, const int32_t *inv_per
     const unsigned grid = (unsigned)imin(cdiv(T, 8), 148 * 16);
 #define MOE_CALL(KT, VB)                                                                                              \
     if (act == MOE_BF16)                                                                                              \
-        dispatch_bwd_kernel<bf16, KT, VB><<<grid, 256, 0, st>>>((const bf16 *)dxs, inv_perm, T, k, d, add_f32, out_f32, \
+        launch_kernel((dispatch_bwd_kernel<bf16, KT, VB>), grid, 256, 0, st, (const bf16 *)dxs, inv_perm, T, k, d, add_f32, out_f32, \
                                                                  (bf16 *)out_act, (const bf16 *)add_act);              \
     else                                                                                                              \
-        dispatch_bwd_kernel<float, KT, VB><<<grid, 256, 0, st>>>((const float *)dxs, inv_perm, T, k, d, add_f32,       \
+        launch_kernel((dispatch_bwd_kernel<float, KT, VB>), grid, 256, 0, st, (const float *)dxs, inv_perm, T, k, d, add_f32,       \
                                                                   out_f32, (float *)out_act, (const float *)add_act)
     MOE_DISPATCH_KT(k, MOE_CALL);
 #undef MOE_CALL
