@@ -38,7 +38,7 @@ constexpr int A_BYTES = BM * BK * 2;  // 16 KiB
 constexpr int B_BYTES = BN * BK * 2;  // 32 KiB
 constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
 constexpr int EPI_STAGE_BYTES = 8 * 4096;  // per epilogue warp: a 32 x 128 B slab for float output
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /*alignment slack*/ + 256 /*barriers*/ + EPI_STAGE_BYTES;
+constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /*alignment slack*/ + 1024 /*barriers; the boxes behind them are 1024-byte aligned*/ + EPI_STAGE_BYTES;
 constexpr int TMEM_COLS = 512;
 constexpr int NTHREADS = 320;   // TMA warp, MMA warp, 8 epilogue warps
 constexpr int NTHREADS2 = 384;  // two-CTA kernel: + one warp that fixes the ragged K tail of the wgrad ahead of the MMAs, + the tile scheduler warp
@@ -274,7 +274,6 @@ __device__ __forceinline__ void pack32_mode(const uint32_t (&v)[32], const uint4
     for (int j = 0; j < 16; ++j) {
         float x0 = __uint_as_float(v[2 * j]), x1 = __uint_as_float(v[2 * j + 1]);
         if (BIAS) { x0 += __uint_as_float(bw[j] << 16); x1 += __uint_as_float(bw[j] & 0xffff0000u); }
-        if (RELU) { x0 = fmaxf(x0, 0.0f); x1 = fmaxf(x1, 0.0f); }
         if (MASK) {
             if (!(__uint_as_float(mw[j] << 16) > 0.0f)) x0 = 0.0f;
             if (!(__uint_as_float(mw[j] & 0xffff0000u) > 0.0f)) x1 = 0.0f;
@@ -283,21 +282,30 @@ __device__ __forceinline__ void pack32_mode(const uint32_t (&v)[32], const uint4
             if (!((keep_word >> (2 * j)) & 1u)) x0 = 0.0f;
             if (!((keep_word >> (2 * j + 1)) & 1u)) x1 = 0.0f;
         }
-        const __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);
+        __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);
+        if (RELU) h = __hmax2(h, __float2bfloat162_rn(0.0f));  // rounding keeps the sign: the same value as max before rounding
         out[j] = *reinterpret_cast<const uint32_t *>(&h);
     }
 }
-// one bit per packed value: set where the stored bf16 value is greater than zero
+// one bit per packed value: set where the stored bf16 value is greater than zero. The pairs' comparison masks are collected
+// as bit j (element 2j) and bit 16 + j (element 2j + 1), two instructions a pair, and interleaved once at the end.
+__device__ __forceinline__ uint32_t spread_bits(uint32_t x) {  // bit i of the low half -> bit 2 i
+    x = (x | (x << 8)) & 0x00ff00ffu;
+    x = (x | (x << 4)) & 0x0f0f0f0fu;
+    x = (x | (x << 2)) & 0x33333333u;
+    return (x | (x << 1)) & 0x55555555u;
+}
 __device__ __forceinline__ uint32_t positive_bits(const uint4 (&packed)[4]) {
-    const uint32_t *pw = reinterpret_cast<const uint32_t *>(packed);
-    uint32_t word = 0u;
+    const __nv_bfloat162 *pw = reinterpret_cast<const __nv_bfloat162 *>(packed);
+    const __nv_bfloat162 zero = __float2bfloat162_rn(0.0f);
+    uint32_t even = 0u, odd = 0u;  // two chains
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-        const uint32_t lo = pw[j] & 0xffffu, hi = pw[j] >> 16;
-        word |= (uint32_t)(lo != 0u && !(lo & 0x8000u)) << (2 * j);
-        word |= (uint32_t)(hi != 0u && !(hi & 0x8000u)) << (2 * j + 1);
+    for (int j = 0; j < 16; j += 2) {
+        even |= __hgt2_mask(pw[j], zero) & (0x00010001u << j);
+        odd |= __hgt2_mask(pw[j + 1], zero) & (0x00010001u << (j + 1));
     }
-    return word;
+    const uint32_t all = even | odd;
+    return spread_bits(all & 0xffffu) | (spread_bits(all >> 16) << 1);
 }
 // mode: bit 0 bias, bit 1 ReLU, bit 2 mask, bit 3 mask as bits (the combinations the layer uses are specialised)
 __device__ __forceinline__ void pack32(int mode, const uint32_t (&v)[32], const uint4 (&bias_raw)[4],
@@ -318,21 +326,140 @@ __device__ __forceinline__ void pack32(int mode, const uint32_t (&v)[32], const 
     }
 }
 
-// The bias values of one warp's 128 output columns are fetched before the warp waits for its accumulator (the load
-// latency used to sit between the tensor-memory load and the arithmetic of every 32-column piece): lane l < 16 holds
-// the 16-byte piece l; piece 4 * ci + q, q = 0..3, of the ci-th 32-column piece is handed to every lane by shuffles.
-__device__ __forceinline__ uint4 bias_slice_load(const bf16 *bias, int64_t row_off, int32_t col_first, int32_t N, int lane) {
-    uint4 v = make_uint4(0, 0, 0, 0);
-    if (bias && lane < 16 && col_first + lane * 8 < N) v = *reinterpret_cast<const uint4 *>(bias + row_off + col_first + lane * 8);
-    return v;
-}
-__device__ __forceinline__ void bias_slice_piece(const uint4 &mine, int ci, uint4 (&out)[4]) {
+// The bias values of a 64-column box, the same for every lane (broadcast loads). They are fetched one box ahead: the
+// first box's before the warp waits for its accumulator.
+__device__ __forceinline__ void bias_load(const bf16 *bias, uint4 (&out)[2][4]) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        out[q].x = __shfl_sync(0xffffffffu, mine.x, 4 * ci + q);
-        out[q].y = __shfl_sync(0xffffffffu, mine.y, 4 * ci + q);
-        out[q].z = __shfl_sync(0xffffffffu, mine.z, 4 * ci + q);
-        out[q].w = __shfl_sync(0xffffffffu, mine.w, 4 * ci + q);
+    for (int q = 0; q < 8; ++q) out[q >> 2][q & 3] = reinterpret_cast<const uint4 *>(bias)[q];
+}
+
+// One [32 rows][64 columns] box of an output tile, by one warp (a lane owns a row): tensor memory -> bias / ReLU / mask ->
+// bf16 -> global memory. With eight epilogue warps an SM sub-partition has two to hide the latencies of this chain, so a
+// box is taken whole: both 32-column loads are in flight together and everything behind them has twice the independent
+// work (with 32-column steps the epilogue of a 256 x 256 tile took 8500 cycles, against 4900 of tensor work at K = 512).
+// Whole boxes leave as bulk tensor stores through the warp's 4 KiB of shared memory (rows of 128 bytes, 16-byte pieces
+// swizzled by row); boxes cut by a segment end as guarded row stores. MASKT: the box holds the mask values on entry.
+// release() hands the accumulator back; it is called once the box is in registers.
+struct BoxArgs {
+    const CUtensorMap *tm_out;
+    uint8_t *box;
+    uint32_t taddr;             // tensor-memory address of the box
+    int64_t out_off, row0;      // output row of lane 0 is row0 of the matrix that starts at element out_off
+    int32_t rows_valid, col0;
+    int32_t map_row;            // the same row in the output's tensor map
+    int64_t colsum_row;
+    const bf16 *next_bias;      // of the warp's next box, or nullptr
+    uint2 keep;                 // mask bits
+    bool have_acc, wait_box;    // wait_box: an earlier store may still be reading the box
+};
+template <bool MASKT, typename Release>
+__device__ __forceinline__ void epilogue_box(const GemmParams &p, int pack_mode, int lane, const BoxArgs &b, uint4 (&bias)[2][4],
+                                             Release release) {
+    uint32_t v[2][32];
+    if (b.have_acc) {
+        tc_ld_32x32(b.taddr, v[0]);
+        tc_ld_32x32(b.taddr + 32, v[1]);
+        tc_ld_wait();
+        release();
+    } else {
+#pragma unroll
+        for (int j = 0; j < 64; ++j) v[j >> 5][j & 31] = 0u;
+    }
+    if (p.out_f32) {  // 128-byte row segments: lane l moves piece l % 8 of row 4 * i + l / 8
+        const int my_piece = lane & 7, my_sub = lane >> 3;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                *reinterpret_cast<uint4 *>(b.box + lane * 128 + ((q ^ (lane & 7)) << 4)) =
+                    make_uint4(v[u][4 * q], v[u][4 * q + 1], v[u][4 * q + 2], v[u][4 * q + 3]);
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int row = 4 * i + my_sub;
+                if (row < b.rows_valid)
+                    *reinterpret_cast<uint4 *>(p.out_f32 + b.out_off + (b.row0 + row) * p.N + b.col0 + 32 * u + my_piece * 4) =
+                        *reinterpret_cast<const uint4 *>(b.box + row * 128 + ((my_piece ^ (row & 7)) << 4));
+            }
+            __syncwarp();
+        }
+        return;
+    }
+    const bool row_ok = lane < b.rows_valid, staged = p.tma_out && b.rows_valid >= 32;
+    const int64_t out_row = b.row0 + lane;
+    uint8_t *mine = b.box + lane * 128;
+    uint4 packed[2][4];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        uint4 mask_raw[4];
+        if (MASKT) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) mask_raw[q] = *reinterpret_cast<const uint4 *>(mine + (((u * 4 + q) ^ (lane & 7)) << 4));
+        } else if (p.mask && row_ok) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) mask_raw[q] = reinterpret_cast<const uint4 *>(p.mask + out_row * p.N + b.col0 + 32 * u)[q];
+        }
+        pack32(pack_mode, v[u], bias[u], mask_raw, packed[u], u ? b.keep.y : b.keep.x);
+    }
+    if (b.next_bias) bias_load(b.next_bias, bias);
+    if (p.bits_out && row_ok)
+        *reinterpret_cast<uint2 *>(p.bits_out + out_row * (p.N >> 5) + (b.col0 >> 5)) =
+            make_uint2(positive_bits(packed[0]), positive_bits(packed[1]));
+    if (staged) {
+        if (!MASKT && b.wait_box) {
+            if (lane == 0) tma_store_wait_read();
+            __syncwarp();
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) *reinterpret_cast<uint4 *>(mine + ((q ^ (lane & 7)) << 4)) = packed[q >> 2][q & 3];
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) {
+            tma_store_2d(b.tm_out, smem_u32(b.box), b.col0, b.map_row);
+            tma_store_commit();
+        }
+        if (p.colsum_part) {
+            // sums of the box's columns over its 32 rows: a lane reads its two columns down the rows (one 4-byte word a
+            // row, conflict free), half the instructions of a butterfly over registers
+            float s0 = 0.0f, s1 = 0.0f, u0 = 0.0f, u1 = 0.0f;
+            const uint8_t *word = b.box + (lane & 3) * 4;
+#pragma unroll 8
+            for (int r = 0; r < 32; r += 2) {
+                const uint32_t w0 = *reinterpret_cast<const uint32_t *>(word + r * 128 + (((lane >> 2) ^ (r & 7)) << 4));
+                const uint32_t w1 = *reinterpret_cast<const uint32_t *>(word + (r + 1) * 128 + (((lane >> 2) ^ ((r + 1) & 7)) << 4));
+                s0 += __uint_as_float(w0 << 16); s1 += __uint_as_float(w0 & 0xffff0000u);
+                u0 += __uint_as_float(w1 << 16); u1 += __uint_as_float(w1 & 0xffff0000u);
+            }
+            *reinterpret_cast<float2 *>(p.colsum_part + b.colsum_row * p.N + b.col0 + 2 * lane) = make_float2(s0 + u0, s1 + u1);
+            __syncwarp();  // read before the next box overwrites this one
+        }
+        return;
+    }
+    if (row_ok) {
+        uint4 *dst = reinterpret_cast<uint4 *>(p.out + b.out_off + out_row * p.N + b.col0);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) st_global_32B(dst + 2 * q, packed[q >> 1][2 * (q & 1)], packed[q >> 1][2 * (q & 1) + 1]);
+    }
+    if (p.colsum_part) {  // sums of the rounded values, rows past the segment end count as 0; the whole warp: shuffles
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            float a[32];
+            const uint32_t *pw = reinterpret_cast<const uint32_t *>(packed[u]);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+                a[2 * j] = row_ok ? __uint_as_float(pw[j] << 16) : 0.0f;
+                a[2 * j + 1] = row_ok ? __uint_as_float(pw[j] & 0xffff0000u) : 0.0f;
+            }
+            p.colsum_part[b.colsum_row * p.N + b.col0 + 32 * u + lane] = warp_column_sums(a, lane);
+        }
+    }
+}
+// mask bits of a row's 128 columns from col0 on (two boxes), as far as the row has them
+__device__ __forceinline__ void keep_load(const GemmParams &p, int64_t row, int32_t col0, uint2 (&keep)[2]) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        keep[u] = make_uint2(0u, 0u);
+        if (col0 + 64 * u < p.N) keep[u] = *reinterpret_cast<const uint2 *>(p.bits_in + row * (p.N >> 5) + ((col0 + 64 * u) >> 5));
     }
 }
 
@@ -444,7 +571,7 @@ template <int KIND, int TM> struct TileIter {
 template <int KIND, bool ACC = false>
 __global__ void __launch_bounds__(NTHREADS, 1)
 grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                    const GemmParams p) {
+                    const __grid_constant__ CUtensorMap tmO, const GemmParams p) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;  // 1024-B aligned for the 128-B swizzle
     uint8_t *smem = smem_raw + (base - smem_u32(smem_raw));
@@ -646,97 +773,48 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 __syncwarp();  // the sums are read before the next tile overwrites them
                 continue;
             }
-            const int half_w = (warp - 2) >> 2;
-            const uint4 bias_mine = bias_slice_load(p.bias, (int64_t)t.e * p.N, t.n0 + half_w * (BN / 2), p.N, lane);
-            if (have_acc) {
+            // Two warps share each quarter of the accumulator's rows and take two boxes of 64 columns each.
+            const int half = (warp - 2) >> 2;
+            const int32_t first = t.n0 + half * (BN / 2);
+            const int boxes = min(2, max(0, (p.N - first) / 64));  // N is a multiple of 64
+            BoxArgs b;
+            b.tm_out = &tmO;
+            b.box = smem + STAGES * STAGE_BYTES + 1024 + (warp - 2) * 4096;
+            b.out_off = KIND == WGRAD ? (int64_t)t.e * p.M * p.N : 0;
+            b.row0 = (KIND == WGRAD ? t.m0 : t.row0) + quarter * 32;
+            b.rows_valid = (KIND == WGRAD ? p.M : t.row_end) - (int32_t)b.row0;
+            b.map_row = (int32_t)b.row0 + (KIND == WGRAD ? t.e * p.M : 0);
+            b.colsum_row = t.mt * 4 + quarter;
+            b.have_acc = have_acc;
+            b.wait_box = true;
+            uint4 bias[2][4];
+            const bf16 *bias_at = p.bias ? p.bias + (int64_t)t.e * p.N + first : nullptr;
+            if (bias_at && boxes > 0) bias_load(bias_at, bias);
+            uint2 keep[2] = {make_uint2(0u, 0u), make_uint2(0u, 0u)};
+            if (p.bits_in && lane < b.rows_valid) keep_load(p, b.row0 + lane, first, keep);
+            if (have_acc) {  // (the loads above are in flight while the warp waits for its accumulator)
                 ok = mbar_wait(tfull_bar(acc), acc_ph, abort_flag, p.status);
                 if (!ok) break;
                 tc_fence_after();
             }
-            // Two warps share each quarter of the accumulator's rows and take half of its columns each.
-            // A thread owns one row. bf16 results are stored straight from registers (64 B per thread and
-            // step); float results (128 B per row and step) go through a swizzled shared-memory slab so that
-            // the stores are whole 128-byte row segments: lane l moves piece l % 8 of row 4 * i + l / 8.
-            const int half = (warp - 2) >> 2;
-            uint8_t *stage_o = smem + STAGES * STAGE_BYTES + 256 + (warp - 2) * 4096;
-            int64_t tile_row0;   // first output row of this warp's 32 rows
-            int32_t rows_valid;  // how many of them exist
-            int64_t out_off = 0;
-            if (KIND == WGRAD) {
-                out_off = (int64_t)t.e * p.M * p.N;
-                tile_row0 = t.m0 + quarter * 32;
-                rows_valid = p.M - (int32_t)tile_row0;
-            } else {
-                tile_row0 = (int64_t)t.row0 + quarter * 32;
-                rows_valid = t.row_end - (int32_t)tile_row0;
-            }
-            const int my_piece = lane & 7, my_sub = lane >> 3;
-            const bool row_ok = lane < rows_valid;
-            const int64_t out_row = tile_row0 + lane;
-            for (int c = half * (BN / 64); c < (half + 1) * (BN / 64); ++c) {
-                const int col0 = t.n0 + c * 32;
-                if (col0 >= p.N) break;
-                uint32_t v[32];
-                if (have_acc) {
-                    tc_ld_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + c * 32, v);
-                    tc_ld_wait();
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) v[j] = 0u;
-                }
-                uint4 bias_raw[4];
-                if (p.bias) bias_slice_piece(bias_mine, c - half * (BN / 64), bias_raw);  // whole warp: shuffles
-                if (p.out_f32) {
-#pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        *reinterpret_cast<uint4 *>(stage_o + lane * 128 + ((q ^ (lane & 7)) << 4)) =
-                            make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-                    __syncwarp();
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const int row = 4 * i + my_sub;
-                        if (row < rows_valid)
-                            *reinterpret_cast<uint4 *>(p.out_f32 + out_off + (tile_row0 + row) * p.N + col0 + my_piece * 4) =
-                                *reinterpret_cast<const uint4 *>(stage_o + row * 128 + ((my_piece ^ (row & 7)) << 4));
-                    }
-                    __syncwarp();
-                } else if (row_ok || p.colsum_part) {  // with column sums the whole warp takes part (shuffles)
-                    uint4 packed[4];
-                    uint4 mask_raw[4];
-                    if (p.mask && row_ok) {
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            mask_raw[q] = reinterpret_cast<const uint4 *>(p.mask + out_row * p.N + col0)[q];
-                    }
-                    uint32_t keep_word = 0u;
-                    if (p.bits_in && row_ok) keep_word = p.bits_in[out_row * (p.N >> 5) + (col0 >> 5)];
-                    pack32(pack_mode, v, bias_raw, mask_raw, packed, keep_word);
-                    if (p.bits_out && row_ok) p.bits_out[out_row * (p.N >> 5) + (col0 >> 5)] = positive_bits(packed);
-                    if (row_ok) {
-                        uint4 *dst = reinterpret_cast<uint4 *>(p.out + out_off + out_row * p.N + col0);
-                        st_global_32B(dst, packed[0], packed[1]);  // two full 32-byte sectors per row piece
-                        st_global_32B(dst + 2, packed[2], packed[3]);
-                    }
-                    if (p.colsum_part) {  // sums of the rounded values, rows past the segment end count as 0
-                        float a[32];
-                        const uint32_t *pw = reinterpret_cast<const uint32_t *>(packed);
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            a[2 * j] = row_ok ? __uint_as_float(pw[j] << 16) : 0.0f;
-                            a[2 * j + 1] = row_ok ? __uint_as_float(pw[j] & 0xffff0000u) : 0.0f;
-                        }
-                        const float sum = warp_column_sums(a, lane);
-                        p.colsum_part[(int64_t)(t.mt * 4 + quarter) * p.N + col0 + lane] = sum;
-                    }
-                }
-            }
-            if (have_acc) {
+            auto release = [&]() {  // the warp's part of the accumulator is in registers: the buffer goes back
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(tempty_bar(acc));
+            };
+            for (int u = 0; u < boxes; ++u) {
+                b.col0 = first + 64 * u;
+                b.taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + half * (BN / 2) + 64 * u;
+                b.next_bias = bias_at && u + 1 < boxes ? bias_at + 64 : nullptr;
+                b.keep = u ? keep[1] : keep[0];
+                epilogue_box<false>(p, pack_mode, lane, b, bias, [&]() { if (u + 1 == boxes) release(); });
+            }
+            if (have_acc) {
+                if (boxes == 0) release();
                 if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
             }
         }
+        if (p.tma_out && lane == 0) tma_store_wait_all();  // no bulk store may outlive the CTA's shared memory
     }
 
     tc_fence_before();
@@ -911,7 +989,6 @@ grouped_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     // staging (row GEMMs: two such blocks, a warp's two output boxes of a tile pass through the same 4 KiB one after
     // the other; the sixth stage took a seventh off the time the MMA thread waited for operands at 16 K blocks per tile)
     constexpr int NST = (KIND == WGRAD || !MASKT) ? 6 : 5;  // the mask tile needs the 64 KiB region, everything else 32 KiB
-    constexpr bool ONE_BOX = KIND != WGRAD && !MASKT;       // row GEMM without a mask tile: one staging box per warp
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *smem = smem_raw + (base - smem_u32(smem_raw));
@@ -950,7 +1027,7 @@ grouped_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
         asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&tmB) : "memory");
         if (MASKT) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmM) : "memory");
-        if (KIND != WGRAD) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmO) : "memory");
+        if (p.tma_out) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmO) : "memory");
     }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32((const void *)tmem_slot)),
@@ -1167,7 +1244,6 @@ grouped_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
         // ------------------------------------------------------------------ epilogue (warps 2..9, both CTAs)
         const int quarter = warp & 3, half = (warp - 2) >> 2;
         const int pack_mode = p.bits_in ? 8 : (p.bias ? 1 : 0) | (p.relu ? 2 : 0) | (p.mask ? 4 : 0);
-        uint8_t *stage_o = smem + NST * STAGE2_BYTES + (warp - 2) * 4096;
         uint32_t mask_ph = 0;
         int acc = 0;
         uint32_t acc_ph = 0;
@@ -1179,30 +1255,22 @@ grouped_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
             const bool have_acc = t.kblocks > 0;
             ++trace_tile;
             if (warp == 2 && lane == 0) TILE_TRACE_SET(2, trace_tile, 0, TILE_CLOCK());
-            const uint4 bias_mine = bias_slice_load(p.bias, (int64_t)t.e * p.N, t.n0 + half * (BN / 2), p.N, lane);
-            long long tr_ld = 0, tr_st = 0, tr_pack = 0;
-            int64_t tile_row0, out_off = 0;
-            int32_t rows_valid;
-            if (KIND == WGRAD) {
-                out_off = (int64_t)t.e * p.M * p.N;
-                tile_row0 = t.m0 + 128 * (int)rank + quarter * 32;
-                rows_valid = p.M - (int32_t)tile_row0;
-            } else {
-                tile_row0 = (int64_t)t.row0 + 128 * (int)rank + quarter * 32;
-                rows_valid = t.row_end - (int32_t)tile_row0;
-            }
-            const int my_piece = lane & 7, my_sub = lane >> 3;
-            const bool row_ok = lane < rows_valid;
-            const int64_t out_row = tile_row0 + lane;
-            uint4 keep4 = make_uint4(0, 0, 0, 0);  // the mask bits of this thread's row for the warp's four 32-column pieces
-            if (p.bits_in && row_ok) {
-                const uint32_t *kw = p.bits_in + out_row * (p.N >> 5) + ((t.n0 + half * (BN / 2)) >> 5);
-                const int left = (p.N - (t.n0 + half * (BN / 2))) >> 5;  // words that exist in this row from here on
-                if (left > 0) keep4.x = kw[0];
-                if (left > 1) keep4.y = kw[1];
-                if (left > 2) keep4.z = kw[2];
-                if (left > 3) keep4.w = kw[3];
-            }
+            const int32_t first = t.n0 + half * (BN / 2);
+            const int boxes = min(2, max(0, (p.N - first) / 64));  // N is a multiple of 64
+            BoxArgs b;
+            b.tm_out = &tmO;
+            b.out_off = KIND == WGRAD ? (int64_t)t.e * p.M * p.N : 0;
+            b.row0 = (KIND == WGRAD ? t.m0 : t.row0) + 128 * (int)rank + quarter * 32;
+            b.rows_valid = (KIND == WGRAD ? p.M : t.row_end) - (int32_t)b.row0;
+            b.map_row = (int32_t)b.row0 + (KIND == WGRAD ? t.e * p.M : 0);
+            b.colsum_row = (t.mt * 2 + (int)rank) * 4 + quarter;
+            b.have_acc = have_acc;
+            b.wait_box = true;
+            uint4 bias[2][4];
+            const bf16 *bias_at = p.bias ? p.bias + (int64_t)t.e * p.N + first : nullptr;
+            if (bias_at && boxes > 0) bias_load(bias_at, bias);
+            uint2 keep[2] = {make_uint2(0u, 0u), make_uint2(0u, 0u)};
+            if (p.bits_in && lane < b.rows_valid) keep_load(p, b.row0 + lane, first, keep);
             if (have_acc) {  // (the loads above are in flight while the warp waits for its accumulator)
                 ok = mbar_wait(tfull_bar(acc), acc_ph, abort_flag, p.status);
                 if (!ok) break;
@@ -1214,120 +1282,35 @@ grouped_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                 if (!ok) break;
                 mask_ph ^= 1u;
             }
-            // Whole 32-row pieces go out as bulk tensor stores: each lane writes its row's 64-byte pieces into the
-            // warp's own rows of a [128][64] block (the place the mask values were just read from, for MASKT), and one
-            // lane stores each finished [32][64] box. Ragged pieces (segment end) use the guarded row stores.
-            const bool staged = KIND != WGRAD && p.tma_out && !p.out_f32 && rows_valid >= 32;
-            const int mrow = quarter * 32 + lane;
-            if (staged && !MASKT) {  // the previous tile's boxes must have been read out of shared memory
-                if (lane == 0) tma_store_wait_read();
-                __syncwarp();
-            }
-            for (int c = half * (BN / 64); c < (half + 1) * (BN / 64); ++c) {
-                const int col0 = t.n0 + c * 32;
-                if (col0 >= p.N) break;
-                uint32_t v[32];
-                if (have_acc) {
-                    const long long tl0 = TILE_CLOCK();
-                    tc_ld_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + c * 32, v);
-                    tc_ld_wait();
-                    tr_ld += TILE_CLOCK() - tl0;
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) v[j] = 0u;
-                }
-                uint4 bias_raw[4];
-                if (p.bias) bias_slice_piece(bias_mine, c - half * (BN / 64), bias_raw);  // whole warp: shuffles
-                if (p.out_f32) {
-#pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        *reinterpret_cast<uint4 *>(stage_o + lane * 128 + ((q ^ (lane & 7)) << 4)) =
-                            make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-                    __syncwarp();
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const int row = 4 * i + my_sub;
-                        if (row < rows_valid)
-                            *reinterpret_cast<uint4 *>(p.out_f32 + out_off + (tile_row0 + row) * p.N + col0 + my_piece * 4) =
-                                *reinterpret_cast<const uint4 *>(stage_o + row * 128 + ((my_piece ^ (row & 7)) << 4));
-                    }
-                    __syncwarp();
-                } else if (row_ok || p.colsum_part) {  // with column sums the whole warp takes part (shuffles)
-                    uint4 packed[4];
-                    uint4 mask_raw[4];
-                    if (MASKT) {  // from the tile in shared memory: row = this thread's row, 16-B pieces swizzled by row
-                        const uint8_t *mrow_p = smem + NST * STAGE2_BYTES + (c >> 1) * 16384 + mrow * 128;
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            mask_raw[q] = *reinterpret_cast<const uint4 *>(mrow_p + ((((c & 1) * 4 + q) ^ (mrow & 7)) << 4));
-                    } else if (p.mask && row_ok) {
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            mask_raw[q] = reinterpret_cast<const uint4 *>(p.mask + out_row * p.N + col0)[q];
-                    }
-                    const long long tp0 = TILE_CLOCK();
-                    const int ci = c - half * (BN / 64);
-                    pack32(pack_mode, v, bias_raw, mask_raw, packed, ci == 0 ? keep4.x : ci == 1 ? keep4.y : ci == 2 ? keep4.z : keep4.w);
-                    if (p.bits_out && row_ok) p.bits_out[out_row * (p.N >> 5) + (col0 >> 5)] = positive_bits(packed);
-                    tr_pack += TILE_CLOCK() - tp0;
-                    if (staged) {
-                        // with one box per warp (two [128][64] blocks, one per column half) the second box of a tile
-                        // goes where the first one was: its bulk store must have read the box out first
-                        uint8_t *blk = smem + NST * STAGE2_BYTES + (ONE_BOX ? half : (c >> 1)) * 16384;
-                        if (ONE_BOX && (c & 3) == 2) {
-                            if (lane == 0) tma_store_wait_read();
-                            __syncwarp();
-                        }
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            *reinterpret_cast<uint4 *>(blk + mrow * 128 + ((((c & 1) * 4 + q) ^ (mrow & 7)) << 4)) = packed[q];
-                        if (c & 1) {  // the box of 64 columns is complete
-                            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                            __syncwarp();
-                            if (lane == 0) {
-                                tma_store_2d(&tmO, smem_u32(blk + quarter * 4096), t.n0 + (c >> 1) * 64, (int)tile_row0);
-                                tma_store_commit();
-                            }
-                        }
-                    } else if (row_ok) {
-                        const long long ts0 = TILE_CLOCK();
-                        uint4 *dst = reinterpret_cast<uint4 *>(p.out + out_off + out_row * p.N + col0);
-                        st_global_32B(dst, packed[0], packed[1]);  // two full 32-byte sectors per row piece
-                        st_global_32B(dst + 2, packed[2], packed[3]);
-                        tr_st += TILE_CLOCK() - ts0;
-                    }
-                    if (p.colsum_part) {  // sums of the rounded values, rows past the segment end count as 0
-                        float a[32];
-                        const uint32_t *pw = reinterpret_cast<const uint32_t *>(packed);
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            a[2 * j] = row_ok ? __uint_as_float(pw[j] << 16) : 0.0f;
-                            a[2 * j + 1] = row_ok ? __uint_as_float(pw[j] & 0xffff0000u) : 0.0f;
-                        }
-                        const float sum = warp_column_sums(a, lane);
-                        p.colsum_part[(int64_t)((t.mt * 2 + (int)rank) * 4 + quarter) * p.N + col0 + lane] = sum;
-                    }
-                }
-            }
-            if (have_acc) {
+            auto release = [&]() {  // the warp's part of the accumulator is in registers: the buffer goes back
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive_leader_relaxed(tempty_bar(acc));
+            };
+            for (int u = 0; u < boxes; ++u) {
+                b.col0 = first + 64 * u;
+                b.taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + half * (BN / 2) + 64 * u;
+                b.box = smem + NST * STAGE2_BYTES + (MASKT ? (2 * half + u) * 16384 + quarter * 4096 : (warp - 2) * 4096);
+                b.next_bias = bias_at && u + 1 < boxes ? bias_at + 64 : nullptr;
+                b.keep = u ? keep[1] : keep[0];
+                epilogue_box<MASKT>(p, pack_mode, lane, b, bias, [&]() { if (u + 1 == boxes) release(); });
+            }
+            if (have_acc) {
+                if (boxes == 0) release();
                 if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
             }
             if (warp == 2 && lane == 0) {
                 TILE_TRACE_SET(2, trace_tile, 2, TILE_CLOCK());
-                TILE_TRACE_SET(2, trace_tile, 3, tr_ld); TILE_TRACE_SET(2, trace_tile, 4, tr_st); TILE_TRACE_SET(2, trace_tile, 5, tr_pack);
             }
             if (MASKT) {  // the next mask tile may land once this warp's boxes have been read out
                 __syncwarp();
                 if (lane == 0) {
-                    if (staged) tma_store_wait_read();
+                    tma_store_wait_read();
                     mbar_arrive(mempty_bar);
                 }
             }
         }
-        if (KIND != WGRAD && lane == 0) tma_store_wait_all();  // no bulk store may outlive the CTA's shared memory
+        if (lane == 0) tma_store_wait_all();  // no bulk store may outlive the CTA's shared memory
     }
 
     tc_fence_before();
@@ -1400,6 +1383,13 @@ int32_t map_weight_kmajor(CUtensorMap *tm, const void *p, int64_t n, int64_t N, 
     return make_map(tm, p, 3, dims, str, box);
 }
 
+// bf16 output rows as [32][64] boxes
+int32_t map_out_boxes(CUtensorMap *tm, const void *p, int64_t rows, int64_t cols) {
+    const uint64_t dims[2] = {(uint64_t)cols, (uint64_t)rows}, str[1] = {(uint64_t)cols * 2};
+    const uint32_t box[2] = {64, 32};
+    return make_map(tm, p, 2, dims, str, box);
+}
+
 GemmParams default_params() {
     GemmParams p;
     memset(&p, 0, sizeof(p));
@@ -1444,8 +1434,9 @@ template <int KIND, int TM> int32_t complete_params(GemmParams &q, int64_t max_t
 }
 
 template <int KIND> int32_t launch(const CUtensorMap &tmA, const CUtensorMap &tmB, const GemmParams &p_in,
-                                   int64_t max_tiles, cudaStream_t st) {
+                                   int64_t max_tiles, cudaStream_t st, const CUtensorMap *tmO = nullptr) {
     GemmParams p = p_in;
+    p.tma_out = tmO != nullptr;
     MOE_TRY((complete_params<KIND, BM>(p, max_tiles)));
     static bool configured = false;
     if (!configured) {
@@ -1454,7 +1445,7 @@ template <int KIND> int32_t launch(const CUtensorMap &tmA, const CUtensorMap &tm
     }
     if (max_tiles <= 0) return MOE_OK;
     const unsigned grid = (unsigned)imin(max_tiles, sm_count());
-    launch_kernel(grouped_gemm_kernel<KIND>, grid, NTHREADS, SMEM_BYTES, st, tmA, tmB, p);
+    launch_kernel(grouped_gemm_kernel<KIND>, grid, NTHREADS, SMEM_BYTES, st, tmA, tmB, tmO ? *tmO : tmA, p);
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -1472,7 +1463,7 @@ int32_t launch_acc_wgrad(const CUtensorMap &tmA, const CUtensorMap &tmB, const G
     }
     if (max_tiles <= 0) return MOE_OK;
     const unsigned grid = (unsigned)imin(max_tiles, sm_count());
-    launch_kernel((grouped_gemm_kernel<WGRAD, true>), grid, NTHREADS, SMEM_ACC_BYTES, st, tmA, tmB, p);
+    launch_kernel((grouped_gemm_kernel<WGRAD, true>), grid, NTHREADS, SMEM_ACC_BYTES, st, tmA, tmB, tmA, p);
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -1679,13 +1670,8 @@ int32_t tc_row_gemm(const void *A, const void *W, bool transposed, const int32_t
         p.sched_group = (int32_t)cdiv(N, BN);
         MOE_TRY(launch_tile_table(offsets, nseg, 256, R, tile_prefix, st, p.sched_counter));
         const int64_t max_tiles2 = (cdiv(R, 256) + nseg) * cdiv(N, BN);
-        CUtensorMap tmO;  // output rows as [32][64] boxes
-        {
-            const uint64_t dims[2] = {(uint64_t)N, (uint64_t)R};
-            const uint64_t str[1] = {(uint64_t)N * 2};
-            const uint32_t box[2] = {64, 32};
-            MOE_TRY(make_map(&tmO, out, 2, dims, str, box));
-        }
+        CUtensorMap tmO;
+        MOE_TRY(map_out_boxes(&tmO, out, R, N));
         if (transposed && mask && !bits_in) {  // the ReLU-mask rows come in as TMA tiles
             CUtensorMap tmM;
             MOE_TRY(map_rows_kmajor(&tmM, mask, R, N));
@@ -1698,7 +1684,9 @@ int32_t tc_row_gemm(const void *A, const void *W, bool transposed, const int32_t
     else MOE_TRY(map_weight_mnmajor(&tmB, W, nseg, K, N));
     MOE_TRY(launch_tile_table(offsets, nseg, BM, R, tile_prefix, st));
     const int64_t max_tiles = (cdiv(R, BM) + nseg) * cdiv(N, BN);
-    return finish(transposed ? launch<ROW_BK>(tmA, tmB, p, max_tiles, st) : launch<ROW_BMN>(tmA, tmB, p, max_tiles, st), 4);
+    CUtensorMap tmO;
+    MOE_TRY(map_out_boxes(&tmO, out, R, N));
+    return finish(transposed ? launch<ROW_BK>(tmA, tmB, p, max_tiles, st, &tmO) : launch<ROW_BMN>(tmA, tmB, p, max_tiles, st, &tmO), 4);
 }
 
 // Order in which the two-CTA weight-gradient GEMM hands out its tiles: seg[r] = {e, first row, end row, 0} for the
@@ -1727,6 +1715,8 @@ int32_t tc_wgrad_gemm(const void *A, const void *B, const int32_t *offsets, int3
     GemmParams p = default_params();
     p.offsets = offsets; p.nseg = nseg; p.M = M; p.N = N; p.R = R;
     p.out = (bf16 *)out; p.status = status;
+    CUtensorMap tmO;  // the experts' matrices as one tall matrix (a 32-row box never straddles two: M is a multiple of 64)
+    MOE_TRY(map_out_boxes(&tmO, out, (int64_t)nseg * M, N));
     if (use_two_cta(R, nseg, flags) && M >= 256) {  // SM pairs: 256 x 256 tiles, each CTA stages half of A and half of B
         MOE_TRY(map_rows_mnmajor(&tmA, A, R > 0 ? R : 1, M, 2));
         MOE_TRY(map_rows_mnmajor(&tmB, B, R > 0 ? R : 1, N, 2));
@@ -1738,11 +1728,11 @@ int32_t tc_wgrad_gemm(const void *A, const void *B, const int32_t *offsets, int3
                                                                           sched_ws);
             MOE_LAUNCHED();
         }
-        return launch2<WGRAD>(tmA, tmB, p, (int64_t)nseg * cdiv(M, 256) * cdiv(N, BN), st);
+        return launch2<WGRAD>(tmA, tmB, p, (int64_t)nseg * cdiv(M, 256) * cdiv(N, BN), st, nullptr, &tmO);
     }
     MOE_TRY(map_rows_mnmajor(&tmA, A, R > 0 ? R : 1, M, BM / 64));
     MOE_TRY(map_rows_mnmajor(&tmB, B, R > 0 ? R : 1, N, BN / 64));
-    return launch<WGRAD>(tmA, tmB, p, (int64_t)nseg * cdiv(M, BM) * cdiv(N, BN), st);
+    return launch<WGRAD>(tmA, tmB, p, (int64_t)nseg * cdiv(M, BM) * cdiv(N, BN), st, &tmO);
 }
 
 int32_t launch_tc_ffn(const moe_config &c, const void *xs, const int32_t *offsets, const void *W1, const void *b1,
