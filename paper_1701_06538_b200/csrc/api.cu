@@ -168,13 +168,26 @@ struct DispatchWs {
     DispatchWs(Carver &cv, const Dims &D) { scratch = cv.take<int32_t>(dispatch_ws_elems(D.R, (int32_t)D.n)); }
 };
 
+// The segment plan of a call's expert products, in the workspace. Forward: tiles of the row products (SIMT: of every height
+// it may pick). Backward: those of the bias gradients' column sums, the order of the weight gradients' tiles.
+SegmentPlan make_plan(const moe_config *c, const Dims &D, int32_t *ws, bool backward) {
+    SegmentPlan p = plan_at(ws, D.R, D.n);
+    if (tc_ffn_supported(*c)) {
+        p.bm[0] = tc_row_tile(D.R, (int32_t)D.n, D.flags);
+        if (backward && p.bm[0] != COLSUM_ROWS) p.bm[1] = COLSUM_ROWS;
+        if (!backward || !tc_wgrad_sorted(*c)) p.sched = nullptr;
+    } else {
+        p.bm[0] = 64; p.bm[1] = 32; p.bm[2] = backward ? COLSUM_ROWS : 16;
+        p.info = p.sched = nullptr;
+    }
+    return p;
+}
+
 struct FfnWs {
-    int32_t *tile_prefix;
-    void *tc;
+    int32_t *plan;
     void *hid;  // MOE_FLAG_RECOMPUTE_HID: the hidden activations live here instead of in a buffer that is kept
-    FfnWs(Carver &cv, const Dims &D, const moe_config *c) {
-        tile_prefix = cv.take<int32_t>(D.n + 1);
-        tc = tc_ffn_supported(*c) ? cv.take_bytes(tc_ffn_ws_bytes(*c)) : nullptr;
+    FfnWs(Carver &cv, const Dims &D) {
+        plan = cv.take<int32_t>(plan_ints(D.R, D.n));
         hid = (D.flags & MOE_FLAG_RECOMPUTE_HID) ? cv.take_bytes(D.R * D.h * (int64_t)D.esz) : nullptr;
     }
 };
@@ -221,11 +234,9 @@ struct LossesWs {
 
 struct FfnBwdWs {
     void *dz;
-    int32_t *tile_prefix;
     float *colsum;
     FfnBwdWs(Carver &cv, const Dims &D) {
         dz = cv.take_bytes(D.R * D.h * (int64_t)D.esz);
-        tile_prefix = cv.take<int32_t>(tc_tile_ws_ints(D.R, D.n));  // prefix + tile table of the row GEMMs
         int64_t cs = colsum_ws_floats(D.R, (int32_t)D.n, (int32_t)(D.h > D.d ? D.h : D.d));
         if (D.act == MOE_BF16) {  // the tensor-core path sums dz's columns per 32-row block in the GEMM epilogue
             const int64_t cs_tc = tc_colsum_part_floats(D.R, (int32_t)D.n, (int32_t)D.h);
@@ -320,9 +331,13 @@ struct Ctx {
 };
 
 struct BwdWs {
-    float *dgates, *dload, *dX_gate;
+    float *dgates, *dload, *dX_gate, *dimp, *dload_h;
     void *dys, *dxs;
+    int32_t *plan;
     BwdWs(Carver &cv, const Dims &D) {
+        plan = cv.take<int32_t>(plan_ints(D.R, D.n));
+        dimp = cv.take<float>(D.n);
+        dload_h = D.hier ? cv.take<float>(D.n) : nullptr;
         dgates = cv.take<float>(D.gates);
         dload = cv.take<float>(D.dload);
         dX_gate = cv.take<float>(D.T * D.d);
@@ -338,13 +353,16 @@ int32_t do_gate(const moe_config *c, const Dims &D, const void *x, const float *
                 const float *noise, int32_t *topk_idx, float *gates, float *clean, float *raw_noise,
                 float *kth_vals, int32_t *kth_idx, void *ws_base, Carver &cv, cudaStream_t st) {
     GateWs w(cv, D);
+    // the status word of the workspace is cleared by the first kernel
+    int32_t *status = status_word(ws_base);
+    if (D.T == 0) MOE_TRY(reset_status(ws_base, st));
     // One gate over n1 columns with top-k1 (the flat gate, or the primary gate of the hierarchical layer).
     // With bf16 activations the routing is screened on the tensor cores and only the tokens whose order is
     // not provably that of the fixed fma chain are redone with the chain; otherwise the chain does all rows.
     auto first_gate = [&](int32_t n1, int32_t k1, int32_t *idx_out, float *gates_out) -> int32_t {
         if (w.screen) {
             MOE_TRY(launch_gate_screen_prepare(x, D.act, D.T, (int32_t)D.d, n1, Wg, Wnoise, w.wsplit, w.wnorm, w.xnorm,
-                                               w.unsafe_count, w.wt, st));
+                                               w.unsafe_count, w.wt, st, 1, true, status));
             MOE_TRY(launch_tc_gate_fwd(x, D.T, (int32_t)D.d, n1, w.wsplit, w.cr, status_word(ws_base), st));
             MOE_TRY(launch_gate_screen(w.cr, noise, w.xnorm, w.wnorm, (int32_t)D.d, D.T, n1, k1, idx_out, gates_out,
                                        clean, raw_noise, kth_vals, kth_idx, w.unsafe_list, w.unsafe_low, w.unsafe_count,
@@ -358,7 +376,7 @@ int32_t do_gate(const moe_config *c, const Dims &D, const void *x, const float *
                                       w.unsafe_list, w.unsafe_count, w.unsafe_span, w.chain_list);
         }
         MOE_TRY(launch_projection(x, D.act, D.T, (int32_t)D.d, n1, Wg, Wnoise, clean, raw_noise, nullptr, 0, nullptr, 1,
-                                  nullptr, st));
+                                  nullptr, st, nullptr, status));
         return launch_gate_select(clean, raw_noise, noise, D.T, n1, k1, idx_out, gates_out, kth_vals, kth_idx, st);
     };
     if (!D.hier) return first_gate((int32_t)D.n, (int32_t)D.k, topk_idx, gates);
@@ -413,38 +431,43 @@ SimtGemm base_gemm(const Dims &D) {
 }
 
 // hid == nullptr (only with MOE_FLAG_RECOMPUTE_HID): the hidden activations stay in the workspace.
-// first_only: only hid = relu(xs.W1 + b1) is computed (ys is not touched).
+// first_only: only hid = relu(xs.W1 + b1) is computed (ys is not touched). ready: a plan made already (with the row tiles
+// of the forward pass); else it is made here, which also clears the status word.
 int32_t do_expert_ffn(const moe_config *c, const Dims &D, const void *xs, const int32_t *offsets, const void *W1,
                       const void *b1, const void *W2, const void *b2, void *hid, void *ys, void *ws_base,
                       Carver &cv, cudaStream_t st, bool first_only = false, void **hid_used = nullptr,
-                      uint32_t *relu_bits = nullptr) {
-    FfnWs w(cv, D, c);
+                      uint32_t *relu_bits = nullptr, const SegmentPlan *ready = nullptr) {
+    FfnWs w(cv, D);
     if (!hid) hid = w.hid;
     if (!hid) return MOE_ERR_INVALID_ARG;
     if (hid_used) *hid_used = hid;
-    if (w.tc)
-        return launch_tc_ffn(*c, xs, offsets, W1, b1, W2, b2, hid, ys, w.tc, status_word(ws_base), st, first_only, relu_bits);
+    const SegmentPlan plan = ready ? *ready : make_plan(c, D, w.plan, false);
+    if (!ready) MOE_TRY(launch_segment_plan(plan, offsets, (int32_t)D.n, D.R, status_word(ws_base), st));
+    if (tc_ffn_supported(*c))
+        return launch_tc_ffn(*c, xs, offsets, W1, b1, W2, b2, hid, ys, plan, status_word(ws_base), st, first_only, relu_bits);
+    int32_t *scratch = ready ? w.plan : nullptr;  // a backward plan may lack the tile height picked here
     SimtGemm g = base_gemm(D);  // hid = relu(xs.W1 + b1)
     g.A = xs; g.B = W1; g.C = hid; g.bias = b1; g.relu = 1;
     g.sa_i = D.d; g.sa_k = 1; g.sb_k = D.h; g.sb_j = 1; g.sc_i = D.h;
     g.mode = 0; g.offsets = offsets; g.nseg = (int32_t)D.n; g.M = D.R; g.N = D.h; g.K = D.d; g.b_e = D.d * D.h;
-    MOE_TRY(launch_simt_gemm(g, w.tile_prefix, st));
+    MOE_TRY(launch_simt_gemm(g, scratch, st, nullptr, &plan));
     if (first_only) return MOE_OK;
     g = base_gemm(D);  // ys = hid.W2 + b2
     g.A = hid; g.B = W2; g.C = ys; g.bias = b2;
     g.sa_i = D.h; g.sa_k = 1; g.sb_k = D.d; g.sb_j = 1; g.sc_i = D.d;
     g.mode = 0; g.offsets = offsets; g.nseg = (int32_t)D.n; g.M = D.R; g.N = D.d; g.K = D.h; g.b_e = D.h * D.d;
-    return launch_simt_gemm(g, w.tile_prefix, st);
+    return launch_simt_gemm(g, scratch, st, nullptr, &plan);
 }
 
 int32_t do_losses(const moe_config *c, const Dims &D, const int32_t *topk_idx, const float *gates,
                   const float *clean, const float *raw_noise, const float *kth_vals, float *importance, float *load,
-                  float *losses, const int32_t *perm, const int32_t *offsets, Carver &cv, cudaStream_t st) {
+                  float *losses, const int32_t *perm, const int32_t *offsets, Carver &cv, cudaStream_t st,
+                  const LossOut &copy = LossOut{}) {
     LossesWs w(cv, D);
     if (!D.hier) {
-        MOE_TRY(launch_level_sums(topk_idx, gates, clean, raw_noise, kth_vals, D.T, (int32_t)D.n, (int32_t)D.k,
-                                  importance, load, w.scratch, st));
-        return launch_cv2(importance, (int32_t)D.n, load, (int32_t)D.n, c->w_importance, c->w_load, losses, st);
+        const LossFinal fin = {c->w_importance, c->w_load, losses, copy};
+        return launch_level_sums(topk_idx, gates, clean, raw_noise, kth_vals, D.T, (int32_t)D.n, (int32_t)D.k, importance, load,
+                                 w.scratch, st, &fin);
     }
     // Eq. 13: Importance_H = batch sum of the product gates per expert (ordered sum over each expert's rows)
     if (!perm) {
@@ -464,52 +487,58 @@ int32_t do_losses(const moe_config *c, const Dims &D, const int32_t *topk_idx, c
                                 (int32_t)D.a, D.T * D.k1, (int32_t)D.b, (int32_t)D.k2, load_s, w.grouped,
                                 w.H.tile_prefix, st));
     MOE_TRY(launch_load_h(load, w.H.counts_p, (int32_t)D.a, (int32_t)D.b, st));
-    return launch_cv2(importance, (int32_t)ab, load, (int32_t)ab, c->w_importance, c->w_load, losses, st);
+    return launch_cv2(importance, (int32_t)ab, load, (int32_t)ab, c->w_importance, c->w_load, losses, st, copy);
 }
 
 int32_t do_expert_ffn_bwd(const moe_config *c, const Dims &D, const void *xs, const void *hid, const void *dys,
                           const int32_t *offsets, const void *W1, const void *W2, void *dxs, void *dW1, void *db1,
-                          void *dW2, void *db2, void *ws_base, Carver &cv, cudaStream_t st,
+                          void *dW2, void *db2, void *ws_base, Carver &cv, cudaStream_t st, const SegmentPlan &plan,
                           const uint32_t *relu_bits = nullptr) {
     FfnBwdWs w(cv, D);
     const int32_t n = (int32_t)D.n;
     if (tc_ffn_supported(*c))
-        return launch_tc_ffn_bwd(*c, xs, hid, dys, offsets, W1, W2, dxs, dW1, db1, dW2, db2, w.dz, w.colsum,
-                                 w.tile_prefix, status_word(ws_base), st, relu_bits);
-    MOE_TRY(launch_segment_colsum(dys, D.act, offsets, n, D.R, (int32_t)D.d, db2, w.colsum, w.tile_prefix, st));
+        return launch_tc_ffn_bwd(*c, xs, hid, dys, offsets, W1, W2, dxs, dW1, db1, dW2, db2, w.dz, w.colsum, plan,
+                                 status_word(ws_base), st, relu_bits);
+    MOE_TRY(launch_segment_colsum(dys, D.act, offsets, n, D.R, (int32_t)D.d, db2, w.colsum, plan.prefix_of(COLSUM_ROWS), st));
     SimtGemm g = base_gemm(D);  // dW2[e] = hid_e^T . dys_e
     g.A = hid; g.B = dys; g.C = dW2;
     g.sa_i = 1; g.sa_k = D.h; g.sb_k = D.d; g.sb_j = 1; g.sc_i = D.d;
     g.mode = 1; g.offsets = offsets; g.nseg = n; g.M = D.h; g.N = D.d; g.c_e = D.h * D.d;
-    MOE_TRY(launch_simt_gemm(g, w.tile_prefix, st));
+    MOE_TRY(launch_simt_gemm(g, nullptr, st, nullptr, &plan));
     g = base_gemm(D);  // dz = (dys . W2[e]^T) * [hid > 0]
     g.A = dys; g.B = W2; g.C = w.dz; g.mask = hid;
     g.sa_i = D.d; g.sa_k = 1; g.sb_k = 1; g.sb_j = D.d; g.sc_i = D.h;
     g.mode = 0; g.offsets = offsets; g.nseg = n; g.M = D.R; g.N = D.h; g.K = D.d; g.b_e = D.h * D.d;
-    MOE_TRY(launch_simt_gemm(g, w.tile_prefix, st));
-    MOE_TRY(launch_segment_colsum(w.dz, D.act, offsets, n, D.R, (int32_t)D.h, db1, w.colsum, w.tile_prefix, st));
+    MOE_TRY(launch_simt_gemm(g, nullptr, st, nullptr, &plan));
+    MOE_TRY(launch_segment_colsum(w.dz, D.act, offsets, n, D.R, (int32_t)D.h, db1, w.colsum, plan.prefix_of(COLSUM_ROWS), st));
     g = base_gemm(D);  // dW1[e] = xs_e^T . dz_e
     g.A = xs; g.B = w.dz; g.C = dW1;
     g.sa_i = 1; g.sa_k = D.d; g.sb_k = D.h; g.sb_j = 1; g.sc_i = D.h;
     g.mode = 1; g.offsets = offsets; g.nseg = n; g.M = D.d; g.N = D.h; g.c_e = D.d * D.h;
-    MOE_TRY(launch_simt_gemm(g, w.tile_prefix, st));
+    MOE_TRY(launch_simt_gemm(g, nullptr, st, nullptr, &plan));
     g = base_gemm(D);  // dxs = dz . W1[e]^T
     g.A = w.dz; g.B = W1; g.C = dxs;
     g.sa_i = D.h; g.sa_k = 1; g.sb_k = 1; g.sb_j = D.h; g.sc_i = D.d;
     g.mode = 0; g.offsets = offsets; g.nseg = n; g.M = D.R; g.N = D.d; g.K = D.h; g.b_e = D.d * D.h;
-    return launch_simt_gemm(g, w.tile_prefix, st);
+    return launch_simt_gemm(g, nullptr, st, nullptr, &plan);
+}
+
+int32_t expert_ffn_bwd_stage(const moe_config *c, const Dims &D, const void *xs, const void *hid, const void *dys,
+                             const int32_t *offsets, const void *W1, const void *W2, void *dxs, void *dW1, void *db1, void *dW2,
+                             void *db2, void *ws, Carver &cv, cudaStream_t st, const uint32_t *relu_bits) {
+    const SegmentPlan plan = make_plan(c, D, cv.take<int32_t>(plan_ints(D.R, D.n)), true);
+    MOE_TRY(launch_segment_plan(plan, offsets, (int32_t)D.n, D.R, status_word(ws), st));
+    return do_expert_ffn_bwd(c, D, xs, hid, dys, offsets, W1, W2, dxs, dW1, db1, dW2, db2, ws, cv, st, plan, relu_bits);
 }
 
 int32_t do_losses_bwd(const moe_config *c, const Dims &D, const float *importance, const float *load,
                       const int32_t *topk_idx, float *dgates, float *dload, Carver &cv, cudaStream_t st) {
     LossesBwdWs w(cv, D);
-    if (!D.hier)
-        return launch_losses_bwd_flat(importance, load, (int32_t)D.n, topk_idx, D.R, c->w_importance, c->w_load,
-                                      dgates, dload, w.dimp, st);
-    MOE_TRY(launch_cv2_grad(importance, (int32_t)D.n, c->w_importance, w.dimp, st));
+    const Cv2Job jobs[2] = {{importance, (int32_t)D.n, c->w_importance, w.dimp},
+                            {load, (int32_t)D.n, c->w_load, D.hier ? w.dload_h : dload}};  // load[0 : n] is Load_H there
+    MOE_TRY(launch_cv2_grads(jobs, st));
     MOE_TRY(launch_add_gathered(dgates, topk_idx, w.dimp, D.R, (int32_t)D.n, st));
-    MOE_TRY(launch_cv2_grad(load, (int32_t)D.n, c->w_load, w.dload_h, st));  // load[0 : a*b] is Load_H
-    return launch_load_h_bwd(load, w.dload_h, (int32_t)D.a, (int32_t)D.b, dload, st);
+    return D.hier ? launch_load_h_bwd(load, w.dload_h, (int32_t)D.a, (int32_t)D.b, dload, st) : MOE_OK;
 }
 
 // dW = x^T . dlogit [d, n], dX = dlogit . W^T [T, d], with dlogit [T, cols] (cols = n, or 2n columns of [W_g | W_noise], whose
@@ -636,9 +665,9 @@ int32_t moe_query_sizes(const moe_config *cfg, moe_sizes *out) {
     out->kth_elems = D.kth; out->wg_elems = D.wg; out->load_elems = D.load; out->dload_elems = D.dload;
     const int64_t s_gate = measure([&](Carver &cv) { GateWs w(cv, D); (void)w; });
     const int64_t s_disp = measure([&](Carver &cv) { DispatchWs w(cv, D); (void)w; });
-    const int64_t s_ffn = measure([&](Carver &cv) { FfnWs w(cv, D, cfg); (void)w; });
+    const int64_t s_ffn = measure([&](Carver &cv) { FfnWs w(cv, D); (void)w; });
     const int64_t s_loss = measure([&](Carver &cv) { LossesWs w(cv, D); (void)w; });
-    const int64_t s_fbwd = measure([&](Carver &cv) { FfnBwdWs w(cv, D); (void)w; });
+    const int64_t s_fbwd = measure([&](Carver &cv) { cv.take<int32_t>(plan_ints(D.R, D.n)); FfnBwdWs w(cv, D); (void)w; });
     const int64_t s_lbwd = measure([&](Carver &cv) { LossesBwdWs w(cv, D); (void)w; });
     const int64_t s_gbwd = measure([&](Carver &cv) { GateBwdWs w(cv, D); (void)w; });
     int64_t fwd = s_gate;
@@ -648,7 +677,7 @@ int32_t moe_query_sizes(const moe_config *cfg, moe_sizes *out) {
     int64_t stage_bwd = s_fbwd;
     if (s_lbwd > stage_bwd) stage_bwd = s_lbwd;
     if (s_gbwd > stage_bwd) stage_bwd = s_gbwd;
-    const int64_t s_fbwd_recompute = measure([&](Carver &cv) { FfnBwdWs w(cv, D); FfnWs f(cv, D, cfg); (void)w; (void)f; });
+    const int64_t s_fbwd_recompute = measure([&](Carver &cv) { FfnBwdWs w(cv, D); FfnWs f(cv, D); (void)w; (void)f; });
     if ((D.flags & MOE_FLAG_RECOMPUTE_HID) && s_fbwd_recompute > stage_bwd) stage_bwd = s_fbwd_recompute;
     out->adam_state_elems = D.n * (3 * D.d + 3 * D.h);
     out->ws_adam_bytes = kWsHeader + ((adam_ws_floats((int32_t)D.n, (int32_t)D.d, (int32_t)D.h) * 4 + 255) & ~(int64_t)255);
@@ -716,7 +745,6 @@ int32_t moe_gate(const moe_config *cfg, const void *x, const float *Wg, const fl
     const Dims D = dims_of(cfg);
     Carver cv(ws);
     cv.take_bytes(kWsHeader);
-    MOE_TRY(reset_status(ws, as_stream(stream)));
     return do_gate(cfg, D, x, Wg, Wnoise, noise, topk_idx, gates, clean, raw_noise, kth_vals, kth_idx, ws, cv,
                    as_stream(stream));
 }
@@ -740,7 +768,6 @@ int32_t moe_expert_ffn(const moe_config *cfg, const void *xs, const int32_t *off
     const Dims D = dims_of(cfg);
     Carver cv(ws);
     cv.take_bytes(kWsHeader);
-    MOE_TRY(reset_status(ws, as_stream(stream)));
     return do_expert_ffn(cfg, D, xs, offsets, W1, b1, W2, b2, hid, ys, ws, cv, as_stream(stream));
 }
 
@@ -753,7 +780,6 @@ int32_t moe_expert_ffn_bits(const moe_config *cfg, const void *xs, const int32_t
     const Dims D = dims_of(cfg);
     Carver cv(ws);
     cv.take_bytes(kWsHeader);
-    MOE_TRY(reset_status(ws, as_stream(stream)));
     return do_expert_ffn(cfg, D, xs, offsets, W1, b1, W2, b2, hid, ys, ws, cv, as_stream(stream), false, nullptr, relu_bits);
 }
 
@@ -766,9 +792,7 @@ int32_t moe_expert_ffn_bwd_bits(const moe_config *cfg, const void *xs, const voi
     const Dims D = dims_of(cfg);
     Carver cv(ws);
     cv.take_bytes(kWsHeader);
-    MOE_TRY(reset_status(ws, as_stream(stream)));
-    return do_expert_ffn_bwd(cfg, D, xs, hid, dys, offsets, W1, W2, dxs, dW1, db1, dW2, db2, ws, cv, as_stream(stream),
-                             relu_bits);
+    return expert_ffn_bwd_stage(cfg, D, xs, hid, dys, offsets, W1, W2, dxs, dW1, db1, dW2, db2, ws, cv, as_stream(stream), relu_bits);
 }
 
 int32_t moe_combine(const moe_config *cfg, const void *ys, const float *gates, const int32_t *inv_perm, void *y,
@@ -806,9 +830,7 @@ int32_t moe_expert_ffn_bwd(const moe_config *cfg, const void *xs, const void *hi
     const Dims D = dims_of(cfg);
     Carver cv(ws);
     cv.take_bytes(kWsHeader);
-    MOE_TRY(reset_status(ws, as_stream(stream)));
-    return do_expert_ffn_bwd(cfg, D, xs, hid, dys, offsets, W1, W2, dxs, dW1, db1, dW2, db2, ws, cv,
-                             as_stream(stream));
+    return expert_ffn_bwd_stage(cfg, D, xs, hid, dys, offsets, W1, W2, dxs, dW1, db1, dW2, db2, ws, cv, as_stream(stream), nullptr);
 }
 
 int32_t moe_dispatch_bwd(const moe_config *cfg, const void *dxs, const int32_t *inv_perm, float *dX_expert,
@@ -855,7 +877,6 @@ static int32_t forward_impl(const moe_config *cfg, const void *x, const float *W
     const Dims D = dims_of(cfg);
     cudaStream_t st = as_stream(stream);
     Ctx C(ctx, D, tc_ffn_supported(*cfg));
-    MOE_TRY(reset_status(ws, st));
     auto fresh = [&]() { Carver cv(ws); cv.take_bytes(kWsHeader); return cv; };
     { Carver cv = fresh();
       MOE_TRY(do_gate(cfg, D, x, Wg, Wnoise, noise, C.topk_idx, C.gates, C.clean, C.raw_noise, C.kth_vals,
@@ -869,11 +890,8 @@ static int32_t forward_impl(const moe_config *cfg, const void *x, const float *W
                            keep_bits ? x : nullptr, keep_bits, keep_bits ? 1.0f / (1.0f - drop_prob) : 1.0f));
     { Carver cv = fresh();
       MOE_TRY(do_losses(cfg, D, C.topk_idx, C.gates, C.clean, C.raw_noise, C.kth_vals, C.importance, C.load,
-                        C.losses, C.perm, C.offsets, cv, st)); }
-    MOE_CUDA(cudaMemcpyAsync(losses, C.losses, 2 * sizeof(float), cudaMemcpyDeviceToDevice, st));
-    MOE_CUDA(cudaMemcpyAsync(importance, C.importance, D.n * sizeof(float), cudaMemcpyDeviceToDevice, st));
-    MOE_CUDA(cudaMemcpyAsync(load, C.load, D.load * sizeof(float), cudaMemcpyDeviceToDevice, st));
-    MOE_CUDA(cudaMemcpyAsync(counts, C.counts, D.n * sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
+                        C.losses, C.perm, C.offsets, cv, st,
+                        LossOut{losses, importance, load, counts, C.counts, (int32_t)D.n, (int32_t)D.load})); }
     return MOE_OK;
 }
 
@@ -904,27 +922,32 @@ static int32_t backward_impl(const moe_config *cfg, const void *dY, const void *
     const Dims D = dims_of(cfg);
     cudaStream_t st = as_stream(stream);
     Ctx C(const_cast<void *>(ctx), D, tc_ffn_supported(*cfg));
-    MOE_TRY(reset_status(ws, st));
     Carver base(ws);
     base.take_bytes(kWsHeader);
     BwdWs B(base, D);
     auto fresh = [&]() { return base; };  // stage scratch starts after the tensors that live across stages
+    // everything that depends on the routing alone in one launch: the segment plan, the gradients of the balancing losses
+    // (load[0 : n] is Load_H in the hierarchical layer), the status word
+    const SegmentPlan plan = make_plan(cfg, D, B.plan, true);
+    const Cv2Job jobs[2] = {{C.importance, (int32_t)D.n, cfg->w_importance, B.dimp},
+                            {C.load, (int32_t)D.n, cfg->w_load, D.hier ? B.dload_h : B.dload}};
+    MOE_TRY(launch_segment_plan(plan, C.offsets, (int32_t)D.n, D.R, status_word(ws), st, jobs));
+    if (D.hier) MOE_TRY(launch_load_h_bwd(C.load, B.dload_h, (int32_t)D.a, (int32_t)D.b, B.dload, st));
     MOE_TRY(launch_combine_bwd(dY, C.ys, D.act, C.gates, C.inv_perm, D.T, (int32_t)D.k, (int32_t)D.d, B.dgates,
-                               B.dys, st, keep_bits, keep_bits ? 1.0f / (1.0f - drop_prob) : 1.0f));
+                               B.dys, st, keep_bits, keep_bits ? 1.0f / (1.0f - drop_prob) : 1.0f, C.topk_idx, B.dimp,
+                               (int32_t)D.n));
     { Carver cv = fresh();
       const void *hid = C.hid;
       if (!hid) {  // MOE_FLAG_RECOMPUTE_HID: the forward kept no hidden activations; the first GEMM is run again
           FfnBwdWs skip(cv, D);  // the expert backward's own scratch comes first, the recomputed tensor behind it
           (void)skip;
           void *again = nullptr;
-          MOE_TRY(do_expert_ffn(cfg, D, C.xs, C.offsets, W1, b1, W2, b2, nullptr, nullptr, ws, cv, st, true, &again));
+          MOE_TRY(do_expert_ffn(cfg, D, C.xs, C.offsets, W1, b1, W2, b2, nullptr, nullptr, ws, cv, st, true, &again, nullptr, &plan));
           hid = again;
           cv = fresh();
       }
       MOE_TRY(do_expert_ffn_bwd(cfg, D, C.xs, hid, B.dys, C.offsets, W1, W2, B.dxs, dW1, db1, dW2, db2, ws, cv,
-                                st, C.relu_bits)); }
-    { Carver cv = fresh();
-      MOE_TRY(do_losses_bwd(cfg, D, C.importance, C.load, C.topk_idx, B.dgates, B.dload, cv, st)); }
+                                st, plan, C.relu_bits)); }
     { Carver cv = fresh();
       MOE_TRY(do_gate_bwd(cfg, D, x, Wg, Wnoise, noise, C.clean, C.raw_noise, C.topk_idx, C.gates, C.kth_vals,
                           C.kth_idx, B.dgates, B.dload, dWg, dWnoise, B.dX_gate, ws, cv, st)); }

@@ -1511,8 +1511,6 @@ bool tc_ffn_supported(const moe_config &c) {
     return c.act == MOE_BF16 && c.d % 64 == 0 && c.h % 64 == 0 && c.d >= 64 && c.h >= 64;
 }
 
-int64_t tc_tile_ws_ints(int64_t R, int64_t nseg);
-int64_t tc_ffn_ws_bytes(const moe_config &c) { return (tc_tile_ws_ints((int64_t)c.T * c.k, c.n) * 4 + 255) & ~255ll; }
 
 // The 256-row tiles of the two-CTA kernel pay off when the average segment fills them.
 static bool use_two_cta(int64_t R, int32_t nseg, int32_t flags) {
@@ -1527,7 +1525,7 @@ static bool use_two_cta(int64_t R, int32_t nseg, int32_t flags) {
 // the last tile carry segment -1. One block.
 __global__ void __launch_bounds__(1024) tile_table_kernel(const int32_t *__restrict__ offsets, int32_t n, int32_t tm,
                                                           int32_t max_m, int32_t *__restrict__ tile_prefix,
-                                                          int4 *__restrict__ info, int32_t *__restrict__ counter) {
+                                                          int4 *__restrict__ info) {
     wait_previous_kernel();
     __shared__ int32_t warp_sum[32];
     __shared__ int32_t carry;
@@ -1563,7 +1561,6 @@ __global__ void __launch_bounds__(1024) tile_table_kernel(const int32_t *__restr
         __syncthreads();
     }
     if (threadIdx.x == 0) tile_prefix[n] = carry;
-    if (threadIdx.x == 0 && counter) *counter = 0;  // run-time tile counter of the GEMM that follows
     __syncthreads();  // the prefix (global memory, this block's own writes) is complete
     const int32_t total = carry;
     for (int32_t mt = threadIdx.x; mt < max_m; mt += 1024) {
@@ -1582,14 +1579,10 @@ int64_t tc_tile_ws_ints(int64_t R, int64_t nseg) { return ((nseg + 1 + 3) & ~(in
 static int4 *tile_info_of(int32_t *tile_prefix, int32_t nseg) {
     return reinterpret_cast<int4 *>(tile_prefix + ((nseg + 1 + 3) & ~3));
 }
-// the int32 behind the last record of a table of tm = 256-row tiles (the table is sized for 128-row tiles)
-static int32_t *tile_counter_of(int32_t *tile_prefix, int32_t nseg, int64_t R) {
-    return reinterpret_cast<int32_t *>(tile_info_of(tile_prefix, nseg) + cdiv(R, 256) + nseg);
-}
 static int32_t launch_tile_table(const int32_t *offsets, int32_t nseg, int32_t tm, int64_t R, int32_t *tile_prefix,
-                                 cudaStream_t st, int32_t *counter = nullptr) {
+                                 cudaStream_t st) {
     launch_kernel(tile_table_kernel, 1, 1024, 0, st, offsets, nseg, tm, (int32_t)(cdiv(R, tm) + nseg), tile_prefix,
-                                          tile_info_of(tile_prefix, nseg), counter);
+                                          tile_info_of(tile_prefix, nseg));
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -1639,7 +1632,7 @@ int64_t tc_colsum_part_floats(int64_t R, int32_t nseg, int32_t N) { return (cdiv
 // and reduced into colsum_out [nseg, N]; colsum_part needs tc_colsum_part_floats(R, nseg, N) floats
 int32_t tc_row_gemm(const void *A, const void *W, bool transposed, const int32_t *offsets, int32_t nseg, int64_t R,
                     int32_t N, int32_t K, void *out, const void *bias, const void *mask, int relu,
-                    int32_t *tile_prefix, int32_t *status, cudaStream_t st, int32_t flags,
+                    const SegmentPlan &plan, int counter, int32_t *status, cudaStream_t st, int32_t flags,
                     float *colsum_part = nullptr, void *colsum_out = nullptr, uint32_t *bits_out = nullptr,
                     const uint32_t *bits_in = nullptr) {
     if (R == 0) {
@@ -1648,7 +1641,7 @@ int32_t tc_row_gemm(const void *A, const void *W, bool transposed, const int32_t
     }
     auto finish = [&](int32_t rc, int32_t G) -> int32_t {
         if (rc != MOE_OK || !colsum_out) return rc;
-        launch_kernel(colsum_blocks_final_kernel, dim3((unsigned)nseg, (unsigned)cdiv(N, 64)), 256, 0, st, colsum_part, N, tile_prefix, G,
+        launch_kernel(colsum_blocks_final_kernel, dim3((unsigned)nseg, (unsigned)cdiv(N, 64)), 256, 0, st, colsum_part, N, plan.prefix[0], G,
                                                                                                    (bf16 *)colsum_out);
         MOE_LAUNCHED();
         return MOE_OK;
@@ -1656,7 +1649,7 @@ int32_t tc_row_gemm(const void *A, const void *W, bool transposed, const int32_t
     CUtensorMap tmA, tmB;
     MOE_TRY(map_rows_kmajor(&tmA, A, R, K));
     GemmParams p = default_params();
-    p.offsets = offsets; p.tile_prefix = tile_prefix; p.tile_info = tile_info_of(tile_prefix, nseg);
+    p.offsets = offsets; p.tile_prefix = plan.prefix[0]; p.tile_info = plan.info;
     p.nseg = nseg; p.M = 0; p.N = N; p.K = K; p.R = R;
     p.out = (bf16 *)out; p.bias = (const bf16 *)bias; p.mask = (const bf16 *)mask; p.relu = relu; p.status = status;
     p.bits_out = bits_out; p.bits_in = bits_in;
@@ -1665,10 +1658,9 @@ int32_t tc_row_gemm(const void *A, const void *W, bool transposed, const int32_t
     if (use_two_cta(R, nseg, flags)) {  // segments long enough to fill 256-row tiles: SM pairs
         if (transposed) MOE_TRY(map_weight_kmajor_half(&tmB, W, nseg, N, K));
         else MOE_TRY(map_weight_mnmajor_half(&tmB, W, nseg, K, N));
-        p.sched_counter = tile_counter_of(tile_prefix, nseg, R);  // tiles handed out at run time
+        p.sched_counter = plan.counters + counter;  // tiles handed out at run time
         p.sched_table = p.tile_info;
         p.sched_group = (int32_t)cdiv(N, BN);
-        MOE_TRY(launch_tile_table(offsets, nseg, 256, R, tile_prefix, st, p.sched_counter));
         const int64_t max_tiles2 = (cdiv(R, 256) + nseg) * cdiv(N, BN);
         CUtensorMap tmO;
         MOE_TRY(map_out_boxes(&tmO, out, R, N));
@@ -1682,35 +1674,16 @@ int32_t tc_row_gemm(const void *A, const void *W, bool transposed, const int32_t
     }
     if (transposed) MOE_TRY(map_weight_kmajor(&tmB, W, nseg, N, K));
     else MOE_TRY(map_weight_mnmajor(&tmB, W, nseg, K, N));
-    MOE_TRY(launch_tile_table(offsets, nseg, BM, R, tile_prefix, st));
     const int64_t max_tiles = (cdiv(R, BM) + nseg) * cdiv(N, BN);
     CUtensorMap tmO;
     MOE_TRY(map_out_boxes(&tmO, out, R, N));
     return finish(transposed ? launch<ROW_BK>(tmA, tmB, p, max_tiles, st, &tmO) : launch<ROW_BMN>(tmA, tmB, p, max_tiles, st, &tmO), 4);
 }
 
-// Order in which the two-CTA weight-gradient GEMM hands out its tiles: seg[r] = {e, first row, end row, 0} for the
-// segment of rank r by descending size (equal sizes by index), and the tile counter reset. One thread per segment.
-constexpr int SCHED_MAX_SEG = 8192;
-__global__ void __launch_bounds__(256) wgrad_schedule_kernel(const int32_t *__restrict__ offsets, int32_t n,
-                                                             int4 *__restrict__ seg, int32_t *__restrict__ counter) {
-    wait_previous_kernel();
-    __shared__ int32_t cnt[SCHED_MAX_SEG];
-    for (int32_t e = threadIdx.x; e < n; e += blockDim.x) cnt[e] = offsets[e + 1] - offsets[e];
-    __syncthreads();
-    const int32_t e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e == 0) *counter = 0;
-    if (e >= n) return;
-    const int32_t mine = cnt[e];
-    int32_t rank = 0;
-    for (int32_t o = 0; o < n; ++o) rank += (cnt[o] > mine || (cnt[o] == mine && o < e)) ? 1 : 0;
-    seg[rank] = make_int4(e, offsets[e], offsets[e + 1], 0);
-}
-
 // dW[e] [M, N] = A_e^T . B_e, contraction over the rows of segment e; A [R, M], B [R, N].
-// sched_ws: 4 + 4 * nseg ints (16-byte aligned) for the run-time tile order of the two-CTA kernel, or nullptr.
+// plan.sched (if made): the two-CTA kernel hands its tiles out at run time, longest segments first.
 int32_t tc_wgrad_gemm(const void *A, const void *B, const int32_t *offsets, int32_t nseg, int64_t R, int32_t M,
-                      int32_t N, void *out, int32_t *status, cudaStream_t st, int32_t flags, int32_t *sched_ws) {
+                      int32_t N, void *out, int32_t *status, cudaStream_t st, int32_t flags, const SegmentPlan &plan, int counter) {
     CUtensorMap tmA, tmB;
     GemmParams p = default_params();
     p.offsets = offsets; p.nseg = nseg; p.M = M; p.N = N; p.R = R;
@@ -1720,13 +1693,10 @@ int32_t tc_wgrad_gemm(const void *A, const void *B, const int32_t *offsets, int3
     if (use_two_cta(R, nseg, flags) && M >= 256) {  // SM pairs: 256 x 256 tiles, each CTA stages half of A and half of B
         MOE_TRY(map_rows_mnmajor(&tmA, A, R > 0 ? R : 1, M, 2));
         MOE_TRY(map_rows_mnmajor(&tmB, B, R > 0 ? R : 1, N, 2));
-        if (sched_ws && nseg > 1 && nseg <= SCHED_MAX_SEG) {  // tiles of unequal length: longest first, handed out at run time
-            p.sched_counter = sched_ws;
-            p.sched_table = reinterpret_cast<const int4 *>(sched_ws + 4);
+        if (plan.sched) {
+            p.sched_counter = plan.counters + counter;
+            p.sched_table = plan.sched;
             p.sched_group = (int32_t)(cdiv(M, 256) * cdiv(N, BN));
-            launch_kernel(wgrad_schedule_kernel, (unsigned)cdiv(nseg, 256), 256, 0, st, offsets, nseg, reinterpret_cast<int4 *>(sched_ws + 4),
-                                                                          sched_ws);
-            MOE_LAUNCHED();
         }
         return launch2<WGRAD>(tmA, tmB, p, (int64_t)nseg * cdiv(M, 256) * cdiv(N, BN), st, nullptr, &tmO);
     }
@@ -1735,15 +1705,19 @@ int32_t tc_wgrad_gemm(const void *A, const void *B, const int32_t *offsets, int3
     return launch<WGRAD>(tmA, tmB, p, (int64_t)nseg * cdiv(M, BM) * cdiv(N, BN), st, &tmO);
 }
 
+int32_t tc_row_tile(int64_t R, int32_t nseg, int32_t flags) { return use_two_cta(R, nseg, flags) ? 256 : BM; }
+bool tc_wgrad_sorted(const moe_config &c) {
+    return use_two_cta((int64_t)c.T * c.k, c.n, c.flags) && c.n > 1 && c.n <= PLAN_MAX_SORTED;
+}
+
 int32_t launch_tc_ffn(const moe_config &c, const void *xs, const int32_t *offsets, const void *W1, const void *b1,
-                      const void *W2, const void *b2, void *hid, void *ys, void *ws, int32_t *status_word,
+                      const void *W2, const void *b2, void *hid, void *ys, const SegmentPlan &plan, int32_t *status_word,
                       cudaStream_t st, bool first_only, uint32_t *relu_bits) {
     const int64_t R = (int64_t)c.T * c.k;
-    int32_t *tile_prefix = static_cast<int32_t *>(ws);
-    MOE_TRY(tc_row_gemm(xs, W1, false, offsets, c.n, R, c.h, c.d, hid, b1, nullptr, 1, tile_prefix, status_word, st, c.flags,
-                        nullptr, nullptr, relu_bits));
+    MOE_TRY(tc_row_gemm(xs, W1, false, offsets, c.n, R, c.h, c.d, hid, b1, nullptr, 1, plan, first_only ? PLAN_ROWS_AGAIN : PLAN_ROWS_A,
+                        status_word, st, c.flags, nullptr, nullptr, relu_bits));
     if (first_only) return MOE_OK;
-    return tc_row_gemm(hid, W2, false, offsets, c.n, R, c.d, c.h, ys, b2, nullptr, 0, tile_prefix, status_word, st, c.flags);
+    return tc_row_gemm(hid, W2, false, offsets, c.n, R, c.d, c.h, ys, b2, nullptr, 0, plan, PLAN_ROWS_B, status_word, st, c.flags);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1964,16 +1938,16 @@ int32_t launch_tc_hier_secondary_bwd(const void *xs_p, const void *dsplit_s, voi
 
 int32_t launch_tc_ffn_bwd(const moe_config &c, const void *xs, const void *hid, const void *dys,
                           const int32_t *offsets, const void *W1, const void *W2, void *dxs, void *dW1, void *db1,
-                          void *dW2, void *db2, void *dz, float *colsum, int32_t *tile_prefix, int32_t *status_word,
+                          void *dW2, void *db2, void *dz, float *colsum, const SegmentPlan &plan, int32_t *status_word,
                           cudaStream_t st, const uint32_t *relu_bits) {
     const int64_t R = (int64_t)c.T * c.k;
-    MOE_TRY(launch_segment_colsum(dys, c.act, offsets, c.n, R, c.d, db2, colsum, tile_prefix, st));
-    MOE_TRY(tc_wgrad_gemm(hid, dys, offsets, c.n, R, c.h, c.d, dW2, status_word, st, c.flags, tile_prefix));
+    MOE_TRY(launch_segment_colsum(dys, c.act, offsets, c.n, R, c.d, db2, colsum, plan.prefix_of(COLSUM_ROWS), st));
+    MOE_TRY(tc_wgrad_gemm(hid, dys, offsets, c.n, R, c.h, c.d, dW2, status_word, st, c.flags, plan, PLAN_WGRAD_A));
     // db1 = column sums of dz, formed in the epilogue of the GEMM that produces dz
-    MOE_TRY(tc_row_gemm(dys, W2, true, offsets, c.n, R, c.h, c.d, dz, nullptr, hid, 0, tile_prefix, status_word, st, c.flags, colsum, db1,
-                        nullptr, relu_bits));
-    MOE_TRY(tc_wgrad_gemm(xs, dz, offsets, c.n, R, c.d, c.h, dW1, status_word, st, c.flags, tile_prefix));
-    return tc_row_gemm(dz, W1, true, offsets, c.n, R, c.d, c.h, dxs, nullptr, nullptr, 0, tile_prefix, status_word, st, c.flags);
+    MOE_TRY(tc_row_gemm(dys, W2, true, offsets, c.n, R, c.h, c.d, dz, nullptr, hid, 0, plan, PLAN_ROWS_A, status_word, st, c.flags,
+                        colsum, db1, nullptr, relu_bits));
+    MOE_TRY(tc_wgrad_gemm(xs, dz, offsets, c.n, R, c.d, c.h, dW1, status_word, st, c.flags, plan, PLAN_WGRAD_B));
+    return tc_row_gemm(dz, W1, true, offsets, c.n, R, c.d, c.h, dxs, nullptr, nullptr, 0, plan, PLAN_ROWS_B, status_word, st, c.flags);
 }
 
 // ------------------------------------------------------------------------------------------

@@ -17,14 +17,14 @@ namespace moe {
 int32_t launch_projection(const void *x, int32_t act, int64_t M, int32_t d, int32_t n0, const float *W0,
                           const float *W1, float *out0, float *out1, const int32_t *offsets, int32_t nseg,
                           const int32_t *perm, int32_t kdiv, int32_t *tile_prefix, cudaStream_t st,
-                          const int32_t *row_count) {
+                          const int32_t *row_count, int32_t *clear) {
     SimtGemm g;  // rows x [W0 | W1] (W1 == nullptr: one matrix only)
     memset(&g, 0, sizeof(g));
     g.ta = act == MOE_BF16 ? G_BF16 : G_F32; g.tb = g.tc = G_F32;
     g.A = x; g.B = W0; g.B2 = W1; g.C = out0; g.C2 = W1 ? out1 : nullptr; g.b_split = g.c_split = n0;
     g.sa_i = d; g.sa_k = 1; g.sb_k = n0; g.sb_j = 1; g.sc_i = n0;
     g.mode = 0; g.offsets = offsets; g.nseg = nseg; g.M = M; g.N = W1 ? 2 * n0 : n0; g.K = d; g.b_e = (int64_t)d * n0;
-    g.a_row_index = perm; g.a_row_div = kdiv; g.c_row_index = perm; g.row_count = row_count;
+    g.a_row_index = perm; g.a_row_div = kdiv; g.c_row_index = perm; g.row_count = row_count; g.clear = clear;
     return launch_simt_gemm(g, tile_prefix, st);
 }
 
@@ -603,8 +603,13 @@ __global__ void __launch_bounds__(128) gate_chain_kernel(const XT *__restrict__ 
 
 // Wt[c, q] = [W_g | W_noise][q, c]
 __global__ void __launch_bounds__(256) gate_transpose_weights_kernel(const float *__restrict__ Wg, const float *__restrict__ Wn,
-                                                                     int32_t d, int32_t n, float *__restrict__ Wt) {
+                                                                     int32_t d, int32_t n, float *__restrict__ Wt,
+                                                                     int32_t *__restrict__ counters, int32_t *__restrict__ clear) {
     wait_previous_kernel();
+    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) {  // rows to re-select, chains, full-chain rows; the status word
+        if (threadIdx.x < 4) counters[threadIdx.x] = 0;
+        if (threadIdx.x == 4 && clear) *clear = 0;
+    }
     __shared__ float tile[32][33];
     Wg += (int64_t)blockIdx.z * d * n; Wn += (int64_t)blockIdx.z * d * n; Wt += (int64_t)blockIdx.z * 2 * n * d;  // group
     const int q0 = blockIdx.x * 32, c0 = blockIdx.y * 32;  // 2n and d are multiples of 32 on this path
@@ -632,10 +637,11 @@ int32_t launch_gate_chains(const void *x, int32_t act, int32_t d, int32_t n, con
 
 int32_t launch_gate_screen_prepare(const void *x, int32_t act, int64_t T, int32_t d, int32_t n, const float *Wg,
                                    const float *Wn, void *wsplit, float *wnorm, float *xnorm,
-                                   int32_t *unsafe_count, float *wt, cudaStream_t st, int32_t groups, bool with_xnorm) {
+                                   int32_t *unsafe_count, float *wt, cudaStream_t st, int32_t groups, bool with_xnorm,
+                                   int32_t *clear) {
     // groups > 1: Wg, Wn are stacks [groups, d, n]; wsplit [3][groups * d][2n], wnorm [groups][2n], wt [groups][2n][d]
     launch_kernel(gate_transpose_weights_kernel, dim3((unsigned)(d / 32), (unsigned)(2 * n / 32), (unsigned)groups), 256, 0, st, Wg, Wn, d, n,
-                                                                                                                      wt);
+                                                                                                                      wt, unsafe_count, clear);
     MOE_LAUNCHED();
     launch_kernel(split_gate_weights_kernel, (unsigned)cdiv((int64_t)groups * d * 2 * n, 256), 256, 0, st, Wg, Wn, groups * d, n,
                                                                                                   (bf16 *)wsplit);
@@ -647,7 +653,6 @@ int32_t launch_gate_screen_prepare(const void *x, int32_t act, int64_t T, int32_
         else launch_kernel(row_norms_kernel<float>, (unsigned)cdiv(T, 8), 256, 0, st, (const float *)x, T, d, xnorm);
         MOE_LAUNCHED();
     }
-    MOE_CUDA(cudaMemsetAsync(unsafe_count, 0, 4 * sizeof(int32_t), st));  // rows to re-select, chains, full-chain rows
     return MOE_OK;
 }
 

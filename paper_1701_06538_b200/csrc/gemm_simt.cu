@@ -52,6 +52,7 @@ struct SimtRun {
     const int32_t *tile_prefix;
     int32_t vec_c;       // four elements along a row of C can be stored at once
     int32_t splits;      // mode 1: the contraction range of a segment is cut into this many slices
+    const SegmentPlan *plan;  // host side: tile prefixes made already, or nullptr
     float *part;         // splits > 1: [splits][nseg][M][N] partial results instead of C
 };
 
@@ -71,6 +72,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), TM * TN >= 64 ? 3 : TM 
     __shared__ __align__(16) float As[2][BK * LDA];
     __shared__ __align__(16) float Bs[2][BK * LDB];
     const SimtGemm &g = run.g;
+    if (g.clear && threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0) *g.clear = 0;
     const int tid = threadIdx.x, tx = tid % NTX, ty = tid / NTX;
 
     int64_t m0, m_end, kbeg, kend;
@@ -380,11 +382,15 @@ static bool quad_aligned(const void *p, int32_t t) { return (reinterpret_cast<ui
 template <typename TA, typename TB, typename TC, bool VEC, bool AK, bool BJ, int BM, int BN, int TM, int TN, int BK>
 static int32_t simt_launch(SimtRun &run, int32_t *tile_prefix, cudaStream_t st) {
     const SimtGemm &g = run.g;
+    const int32_t *ready = g.mode == 0 && g.offsets && run.plan ? run.plan->prefix_of(BM) : nullptr;
     dim3 grid;
     if (g.mode == 0) {
         int64_t tiles = cdiv(g.M, BM);
         if (g.offsets) {
-            MOE_TRY(launch_tile_prefix(g.offsets, g.nseg, BM, tile_prefix, st));
+            if (!ready) {
+                if (!tile_prefix) return MOE_ERR_WORKSPACE;
+                MOE_TRY(launch_tile_prefix(g.offsets, g.nseg, BM, tile_prefix, st));
+            }
             tiles += g.nseg;
         }
         grid = dim3((unsigned)tiles, (unsigned)cdiv(g.N, BN), 1);
@@ -392,7 +398,7 @@ static int32_t simt_launch(SimtRun &run, int32_t *tile_prefix, cudaStream_t st) 
         grid = dim3((unsigned)cdiv(g.M, BM), (unsigned)cdiv(g.N, BN), (unsigned)(g.nseg * run.splits));
     }
     if (grid.y > 65535 || grid.z > 65535) return MOE_ERR_UNSUPPORTED;
-    run.tile_prefix = tile_prefix;
+    run.tile_prefix = ready ? ready : tile_prefix;
     launch_kernel((simt_gemm_kernel<TA, TB, TC, VEC, AK, BJ, BM, BN, TM, TN, BK>), grid, (BM / TM) * (BN / TN), 0, st, run);
     MOE_LAUNCHED();
     if (run.part) {
@@ -428,8 +434,9 @@ static int32_t simt_pick_tile(SimtRun &run, bool vec, int32_t *tile_prefix, cuda
 }
 
 // part: simt_wgrad_splits(M, N, nseg, rows) * nseg * M * N floats (mode 1, float results), or nullptr: no slices
-int32_t launch_simt_gemm(const SimtGemm &g_in, int32_t *tile_prefix, cudaStream_t st, float *part) {
+int32_t launch_simt_gemm(const SimtGemm &g_in, int32_t *tile_prefix, cudaStream_t st, float *part, const SegmentPlan *plan) {
     SimtRun run;
+    run.plan = plan;
     run.g = g_in;
     SimtGemm &g = run.g;
     if (!g.offsets) g.nseg = 1;
@@ -470,7 +477,7 @@ int32_t launch_simt_gemm(const SimtGemm &g_in, int32_t *tile_prefix, cudaStream_
 // Column sums per segment (bias gradients): partial sums over tiles of 128 rows, then an ordered
 // pass over each segment's tiles. Deterministic.
 // ------------------------------------------------------------------------------------------
-constexpr int CS_ROWS = 128;
+constexpr int CS_ROWS = COLSUM_ROWS;
 int64_t colsum_ws_floats(int64_t R, int32_t n, int32_t N) { return (cdiv(R, CS_ROWS) + n) * (int64_t)N + 64; }
 
 // One block per 128-row tile and per slab of 32 * V columns (V = elements of a 16-byte vector): lane l owns V adjacent
@@ -566,8 +573,7 @@ __global__ void __launch_bounds__(256) colsum_final_kernel(const float *__restri
 }
 
 int32_t launch_segment_colsum(const void *in, int32_t act, const int32_t *offsets, int32_t nseg, int64_t R,
-                              int32_t N, void *out, float *scratch, int32_t *tile_prefix, cudaStream_t st) {
-    MOE_TRY(launch_tile_prefix(offsets, nseg, CS_ROWS, tile_prefix, st));
+                              int32_t N, void *out, float *scratch, const int32_t *tile_prefix, cudaStream_t st) {
     const int vcols = act == MOE_BF16 ? 256 : 128;  // columns per block of the partial sums: 32 lanes x one 16-byte vector
     dim3 g1((unsigned)(cdiv(R, CS_ROWS) + nseg), (unsigned)cdiv(N, vcols));
     dim3 g2((unsigned)nseg, (unsigned)cdiv(N, 32));

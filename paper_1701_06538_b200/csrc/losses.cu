@@ -4,6 +4,7 @@
 #include <math_constants.h>
 
 #include "moe_internal.cuh"
+#include "moments.cuh"
 
 namespace moe {
 
@@ -22,8 +23,9 @@ __global__ void __launch_bounds__(256) level_sums_kernel(const int32_t *__restri
                                                          const float *__restrict__ raw,
                                                          const float *__restrict__ kth_vals, int64_t rows, int32_t n,
                                                          int32_t k, int32_t CW, float *__restrict__ part_imp,
-                                                         float *__restrict__ part_load) {
+                                                         float *__restrict__ part_load, int32_t *__restrict__ ticket) {
     wait_previous_kernel();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *ticket = 0;  // of level_reduce_kernel
     __shared__ float red_i[256], red_l[256];
     const int cw = threadIdx.x % CW, tl = threadIdx.x / CW, TL = 256 / CW;
     const int64_t per = (rows + gridDim.x - 1) / gridDim.x;
@@ -66,8 +68,9 @@ __global__ void __launch_bounds__(256) level_sums_rows_kernel(const int32_t *__r
                                                               const float *__restrict__ raw,
                                                               const float *__restrict__ kth_vals, int64_t rows,
                                                               int32_t n, int32_t k, float *__restrict__ part_imp,
-                                                              float *__restrict__ part_load) {
+                                                              float *__restrict__ part_load, int32_t *__restrict__ ticket) {
     wait_previous_kernel();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *ticket = 0;  // of level_reduce_kernel
     __shared__ float red[2][8][32 * NV];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t per = (rows + gridDim.x - 1) / gridDim.x;
@@ -118,14 +121,29 @@ __global__ void __launch_bounds__(256) level_sums_rows_kernel(const int32_t *__r
     }
 }
 
+// the two losses (Eq. 7, 11), by one block of 256 threads; `losses` and, if given, a second copy
+__device__ __forceinline__ void cv2_block(const float *importance, int32_t n_imp, const float *load, int32_t n_load, float w_imp,
+                                          float w_load, float *losses, float *losses2, double *sh) {
+    const Moments a = block_moments(importance, n_imp, sh), b = block_moments(load, n_load, sh);
+    if (threadIdx.x == 0) {
+        const float l0 = (float)((double)w_imp * a.var / (a.mu * a.mu)), l1 = (float)((double)w_load * b.var / (b.mu * b.mu));
+        losses[0] = l0; losses[1] = l1;
+        if (losses2) { losses2[0] = l0; losses2[1] = l1; }
+    }
+}
+
 // Importance / Load = the blocks' partial sums added in double. A block takes 32 columns; its eight warps each add an
-// eighth of the chunks (in ascending order, eight loads in flight), the eight sums are then added in warp order.
+// eighth of the chunks (in ascending order, eight loads in flight), the eight sums are then added in warp order. With
+// fin.losses set, the block that finishes last (counted by `ticket`) also forms the two losses from the complete vectors,
+// and the copies in fin.copy are written along the way.
 __global__ void __launch_bounds__(256) level_reduce_kernel(const float *__restrict__ part_imp,
                                                            const float *__restrict__ part_load, int32_t chunks,
-                                                           int32_t n, float *__restrict__ importance,
-                                                           float *__restrict__ load) {
+                                                           int32_t n, float *importance, float *load,
+                                                           const LossFinal fin, int32_t *ticket) {
     wait_previous_kernel();
     __shared__ double red[2][8][32];
+    __shared__ double sh[256];
+    __shared__ int last;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int32_t j = blockIdx.x * 32 + lane;
     const int32_t per = (chunks + 7) / 8, c0 = w * per, c1 = min(c0 + per, chunks);
@@ -156,89 +174,79 @@ __global__ void __launch_bounds__(256) level_reduce_kernel(const float *__restri
         for (int q = 0; q < 8; ++q) { a += red[0][q][lane]; b += red[1][q][lane]; }
         if (importance) importance[j] = (float)a;
         if (load) load[j] = (float)b;
+        if (fin.copy.importance) fin.copy.importance[j] = (float)a;
+        if (fin.copy.load) fin.copy.load[j] = (float)b;
+        if (fin.copy.counts) fin.copy.counts[j] = fin.copy.counts_src[j];
     }
+    if (!fin.losses) return;
+    __threadfence();  // this block's sums, before its ticket
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(ticket, 1) == (int)gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    cv2_block(importance, n, load, n, fin.w_imp, fin.w_load, fin.losses, fin.copy.losses, sh);
 }
 
 int32_t launch_level_sums(const int32_t *idx, const float *gates, const float *clean, const float *raw,
                           const float *kth_vals, int64_t rows, int32_t n, int32_t k, float *importance_out,
-                          float *load_out, float *scratch, cudaStream_t st) {
+                          float *load_out, float *scratch, cudaStream_t st, const LossFinal *fin_in) {
+    LossFinal fin = {};
+    if (fin_in) fin = *fin_in;
     if (rows == 0) {
         if (importance_out) MOE_CUDA(cudaMemsetAsync(importance_out, 0, sizeof(float) * n, st));
         if (load_out) MOE_CUDA(cudaMemsetAsync(load_out, 0, sizeof(float) * n, st));
-        return MOE_OK;
+        return fin_in ? launch_cv2(importance_out, n, load_out, n, fin.w_imp, fin.w_load, fin.losses, st, fin.copy) : MOE_OK;
     }
     const int32_t chunks = level_chunks(rows);
     int32_t CW = 1;
     while (CW < n && CW < 256) CW <<= 1;
     float *part_imp = scratch, *part_load = scratch + (int64_t)chunks * n;
-    if (n <= 32) launch_kernel(level_sums_rows_kernel<1>, chunks, 256, 0, st, idx, gates, clean, raw, kth_vals, rows, n, k, part_imp, part_load);
-    else if (n <= 64) launch_kernel(level_sums_rows_kernel<2>, chunks, 256, 0, st, idx, gates, clean, raw, kth_vals, rows, n, k, part_imp, part_load);
-    else if (n <= 128) launch_kernel(level_sums_rows_kernel<4>, chunks, 256, 0, st, idx, gates, clean, raw, kth_vals, rows, n, k, part_imp, part_load);
-    else if (n <= 256) launch_kernel(level_sums_rows_kernel<8>, chunks, 256, 0, st, idx, gates, clean, raw, kth_vals, rows, n, k, part_imp, part_load);
-    else launch_kernel(level_sums_kernel, chunks, 256, 0, st, idx, gates, clean, raw, kth_vals, rows, n, k, CW, part_imp, part_load);
+    int32_t *ticket = reinterpret_cast<int32_t *>(part_load + (int64_t)chunks * n);
+    if (n <= 32) launch_kernel(level_sums_rows_kernel<1>, chunks, 256, 0, st, idx, gates, clean, raw, kth_vals, rows, n, k, part_imp, part_load, ticket);
+    else if (n <= 64) launch_kernel(level_sums_rows_kernel<2>, chunks, 256, 0, st, idx, gates, clean, raw, kth_vals, rows, n, k, part_imp, part_load, ticket);
+    else if (n <= 128) launch_kernel(level_sums_rows_kernel<4>, chunks, 256, 0, st, idx, gates, clean, raw, kth_vals, rows, n, k, part_imp, part_load, ticket);
+    else if (n <= 256) launch_kernel(level_sums_rows_kernel<8>, chunks, 256, 0, st, idx, gates, clean, raw, kth_vals, rows, n, k, part_imp, part_load, ticket);
+    else launch_kernel(level_sums_kernel, chunks, 256, 0, st, idx, gates, clean, raw, kth_vals, rows, n, k, CW, part_imp, part_load, ticket);
     MOE_LAUNCHED();
     launch_kernel(level_reduce_kernel, (unsigned)cdiv(n, 32), 256, 0, st, part_imp, part_load, chunks, n, importance_out,
-                                                                 load_out);
+                  load_out, fin, ticket);
     MOE_LAUNCHED();
     return MOE_OK;
 }
 
-// ---- CV^2 = population variance / mean^2, and its gradient 2/(m mu^2) ((v_i - mu) - Var/mu) ----
-struct Moments { double mu, var; };
-
-__device__ Moments block_moments(const float *v, int32_t m, double *sh) {
-    double s = 0.0;
-    for (int32_t i = threadIdx.x; i < m; i += blockDim.x) s += (double)v[i];
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    for (int off = blockDim.x / 2; off > 0; off >>= 1) {
-        if (threadIdx.x < off) sh[threadIdx.x] += sh[threadIdx.x + off];
-        __syncthreads();
-    }
-    const double mu = sh[0] / m;
-    __syncthreads();
-    double q = 0.0;
-    for (int32_t i = threadIdx.x; i < m; i += blockDim.x) { double dv = (double)v[i] - mu; q += dv * dv; }
-    sh[threadIdx.x] = q;
-    __syncthreads();
-    for (int off = blockDim.x / 2; off > 0; off >>= 1) {
-        if (threadIdx.x < off) sh[threadIdx.x] += sh[threadIdx.x + off];
-        __syncthreads();
-    }
-    Moments r;
-    r.mu = mu;
-    r.var = sh[0] / m;
-    __syncthreads();
-    return r;
-}
-
+// the losses of vectors that are complete already, and the copies of everything
 __global__ void __launch_bounds__(256) cv2_kernel(const float *importance, int32_t n_imp, const float *load,
-                                                  int32_t n_load, float w_imp, float w_load, float *losses) {
+                                                  int32_t n_load, float w_imp, float w_load, float *losses, const LossOut copy) {
     wait_previous_kernel();
     __shared__ double sh[256];
-    Moments a = block_moments(importance, n_imp, sh);
-    Moments b = block_moments(load, n_load, sh);
-    if (threadIdx.x == 0) {
-        losses[0] = (float)((double)w_imp * a.var / (a.mu * a.mu));
-        losses[1] = (float)((double)w_load * b.var / (b.mu * b.mu));
-    }
+    cv2_block(importance, n_imp, load, n_load, w_imp, w_load, losses, copy.losses, sh);
+    if (copy.importance)
+        for (int32_t i = threadIdx.x; i < copy.n; i += 256) copy.importance[i] = importance[i];
+    if (copy.counts)
+        for (int32_t i = threadIdx.x; i < copy.n; i += 256) copy.counts[i] = copy.counts_src[i];
+    if (copy.load)
+        for (int32_t i = threadIdx.x; i < copy.n_load; i += 256) copy.load[i] = load[i];
 }
 
 int32_t launch_cv2(const float *importance, int32_t n_imp, const float *load, int32_t n_load, float w_imp,
-                   float w_load, float *losses, cudaStream_t st) {
-    launch_kernel(cv2_kernel, 1, 256, 0, st, importance, n_imp, load, n_load, w_imp, w_load, losses);
+                   float w_load, float *losses, cudaStream_t st, const LossOut &copy) {
+    launch_kernel(cv2_kernel, 1, 256, 0, st, importance, n_imp, load, n_load, w_imp, w_load, losses, copy);
     MOE_LAUNCHED();
     return MOE_OK;
 }
 
-// out[i] = scale * dCV^2/dv_i
-__global__ void __launch_bounds__(256) cv2_grad_kernel(const float *v, int32_t m, float scale, float *out) {
+struct Cv2Pair { Cv2Job job[2]; };
+__global__ void __launch_bounds__(1024) cv2_grads_kernel(const Cv2Pair pair) {  // one block per vector
     wait_previous_kernel();
-    __shared__ double sh[256];
-    Moments a = block_moments(v, m, sh);
-    const double c = 2.0 / ((double)m * a.mu * a.mu);
-    for (int32_t i = threadIdx.x; i < m; i += blockDim.x)
-        out[i] = (float)((double)scale * c * (((double)v[i] - a.mu) - a.var / a.mu));
+    __shared__ double sh[1024];
+    cv2_grad_block(pair.job[blockIdx.x], sh);
+}
+
+int32_t launch_cv2_grads(const Cv2Job *jobs, cudaStream_t st) {
+    launch_kernel(cv2_grads_kernel, 2, 1024, 0, st, Cv2Pair{{jobs[0], jobs[1]}});
+    MOE_LAUNCHED();
+    return MOE_OK;
 }
 
 // dgates[p] += dimp[topk_idx[p]]; an expert id outside [0, n) adds nothing
@@ -251,31 +259,11 @@ __global__ void add_gathered_kernel(float *dgates, const int32_t *topk_idx, cons
     if ((uint32_t)e < (uint32_t)n) dgates[p] += dimp[e];
 }
 
-int32_t launch_cv2_grad(const float *v, int32_t m, float scale, float *out, cudaStream_t st) {
-    launch_kernel(cv2_grad_kernel, 1, 256, 0, st, v, m, scale, out);
-    MOE_LAUNCHED();
-    return MOE_OK;
-}
-
 int32_t launch_add_gathered(float *dgates, const int32_t *topk_idx, const float *dimp, int64_t R, int32_t n,
                             cudaStream_t st) {
     if (R == 0) return MOE_OK;
     launch_kernel(add_gathered_kernel, (unsigned)cdiv(R, 256), 256, 0, st, dgates, topk_idx, dimp, R, n);
     MOE_LAUNCHED();
-    return MOE_OK;
-}
-
-int32_t launch_losses_bwd_flat(const float *importance, const float *load, int32_t n, const int32_t *topk_idx,
-                               int64_t R, float w_imp, float w_load, float *dgates, float *dload, float *dimp_tmp,
-                               cudaStream_t st) {
-    launch_kernel(cv2_grad_kernel, 1, 256, 0, st, importance, n, w_imp, dimp_tmp);
-    MOE_LAUNCHED();
-    launch_kernel(cv2_grad_kernel, 1, 256, 0, st, load, n, w_load, dload);
-    MOE_LAUNCHED();
-    if (R > 0) {
-        launch_kernel(add_gathered_kernel, (unsigned)cdiv(R, 256), 256, 0, st, dgates, topk_idx, dimp_tmp, R, n);
-        MOE_LAUNCHED();
-    }
     return MOE_OK;
 }
 

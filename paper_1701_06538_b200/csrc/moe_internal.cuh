@@ -111,7 +111,7 @@ static const int64_t kWsHeader = 256;
 int32_t launch_projection(const void *x, int32_t act, int64_t M, int32_t d, int32_t n0, const float *W0,
                           const float *W1, float *out0, float *out1, const int32_t *offsets, int32_t nseg,
                           const int32_t *perm, int32_t kdiv, int32_t *tile_prefix, cudaStream_t st,
-                          const int32_t *row_count = nullptr);
+                          const int32_t *row_count = nullptr, int32_t *clear = nullptr);
 // Noisy logits, top-k, masked softmax for `rows` rows of n columns.
 int32_t launch_gate_select(const float *clean, const float *raw, const float *noise, int64_t rows, int32_t n,
                            int32_t k, int32_t *idx, float *gates, float *kth_vals, int32_t *kth_idx,
@@ -121,7 +121,7 @@ int32_t launch_gate_select(const float *clean, const float *raw, const float *no
 int32_t launch_gate_screen_prepare(const void *x, int32_t act, int64_t T, int32_t d, int32_t n, const float *Wg,
                                    const float *Wn, void *wsplit, float *wnorm, float *xnorm,
                                    int32_t *unsafe_count, float *wt /* [2n, d]: columns as rows */, cudaStream_t st,
-                                   int32_t groups = 1, bool with_xnorm = true);
+                                   int32_t groups = 1, bool with_xnorm = true, int32_t *clear = nullptr);
 int32_t launch_gate_screen(const float *cr, const float *noise, const float *xnorm, const float *wnorm, int32_t d,
                            int64_t T, int32_t n, int32_t k, int32_t *idx, float *gates, float *clean, float *raw,
                            float *kth_vals, int32_t *kth_idx, int32_t *unsafe_list, float *unsafe_low,
@@ -156,7 +156,9 @@ int32_t launch_combine(const void *ys, int32_t act, const float *gates, const in
                        const uint8_t *keep = nullptr, float keep_scale = 1.0f);
 int32_t launch_combine_bwd(const void *dY, const void *ys, int32_t act, const float *gates,
                            const int32_t *inv_perm, int64_t T, int32_t k, int32_t d, float *dgates, void *dys,
-                           cudaStream_t st, const uint8_t *keep = nullptr, float keep_scale = 1.0f);
+                           cudaStream_t st, const uint8_t *keep = nullptr, float keep_scale = 1.0f,
+                           const int32_t *topk_idx = nullptr, const float *dimp = nullptr, int32_t n = 0);
+// (dimp [n]: the gradient of the Importance loss, added to the gate gradients of the experts in topk_idx)
 // out_f32 = sum_s dxs[inv_perm[t*k+s]] (+ add_f32 if given); written as float or, if out_act
 // is given instead, rounded to the act type.
 int32_t launch_dispatch_bwd(const void *dxs, int32_t act, const int32_t *inv_perm, int64_t T, int32_t k,
@@ -165,19 +167,48 @@ int32_t launch_dispatch_bwd(const void *dxs, int32_t act, const int32_t *inv_per
 // tile_prefix[e] = sum_{e' < e} ceil(count_e' / bm), e = 0..n
 int32_t launch_tile_prefix(const int32_t *offsets, int32_t n, int32_t bm, int32_t *tile_prefix, cudaStream_t st);
 
+// ----------------------------------------------------------------------------- per-call segment plan (plan.cu)
+constexpr int PLAN_COUNTERS = 8, PLAN_MAX_SORTED = 8192;
+// run-time tile counters of a plan, by the GEMM that uses them
+enum PlanCounter { PLAN_ROWS_A = 0, PLAN_ROWS_B = 1, PLAN_WGRAD_A = 2, PLAN_WGRAD_B = 3, PLAN_ROWS_AGAIN = 4 };
+struct SegmentPlan {
+    int32_t *prefix[3];  // [n + 1] number of tiles of bm[i] rows in the segments before
+    int32_t bm[3];       // 0: prefix not made
+    int4 *info;          // a record per tile of prefix[0], or nullptr: {segment or -1, first row, segment end, 0}
+    int4 *sched;         // {segment, first row, end row, 0} in descending size, or nullptr
+    int32_t *counters;   // [PLAN_COUNTERS], zeroed
+    const int32_t *prefix_of(int32_t height) const {
+        for (int i = 0; i < 3; ++i)
+            if (bm[i] == height) return prefix[i];
+        return nullptr;
+    }
+};
+struct Cv2Job { const float *v; int32_t m; float scale; float *out; };  // out = scale * dCV^2(v)/dv
+int64_t plan_ints(int64_t R, int64_t n);
+SegmentPlan plan_at(int32_t *ws, int64_t R, int64_t n);
+int32_t launch_segment_plan(const SegmentPlan &plan, const int32_t *offsets, int32_t n, int64_t R, int32_t *status,
+                            cudaStream_t st, const Cv2Job *jobs = nullptr /* two */);
+
 // ----------------------------------------------------------------------------- losses (losses.cu)
+// where the fused forward wants second copies of the stage's results (nullptr: none), and of the expert counts
+struct LossOut {
+    float *losses, *importance, *load;
+    int32_t *counts;
+    const int32_t *counts_src;
+    int32_t n, n_load;  // lengths of importance / counts and of load
+};
+struct LossFinal { float w_imp, w_load; float *losses; LossOut copy; };
 int64_t losses_ws_floats(int64_t rows, int32_t n);
 // Partial column sums over rows of the gate mass (importance) and of P(x, i) (load).
 // flat / primary level: seg == nullptr. Secondary level: rows are slots p, grouped through
 // perm/offsets (sorted row r -> slot perm[r]); sums are per segment: load_out [nseg, n].
 int32_t launch_level_sums(const int32_t *idx, const float *gates, const float *clean, const float *raw,
                           const float *kth_vals, int64_t rows, int32_t n, int32_t k, float *importance_out,
-                          float *load_out, float *scratch, cudaStream_t st);
+                          float *load_out, float *scratch, cudaStream_t st, const LossFinal *fin = nullptr);
+// (fin: the two losses as well, in the same launches; importance_out and load_out are both wanted then)
 int32_t launch_cv2(const float *importance, int32_t n_imp, const float *load, int32_t n_load, float w_imp,
-                   float w_load, float *losses, cudaStream_t st);
-int32_t launch_losses_bwd_flat(const float *importance, const float *load, int32_t n, const int32_t *topk_idx,
-                               int64_t R, float w_imp, float w_load, float *dgates, float *dload, float *dimp_tmp,
-                               cudaStream_t st);
+                   float w_load, float *losses, cudaStream_t st, const LossOut &copy);
+int32_t launch_cv2_grads(const Cv2Job *jobs /* two */, cudaStream_t st);
 
 // ----------------------------------------------------------------------------- hierarchical pieces (hier.cu)
 int32_t launch_hier_split_idx(const int32_t *topk_idx, int64_t T, int32_t k1, int32_t k2, int32_t a, int32_t b,
@@ -194,7 +225,6 @@ int32_t launch_load_h_bwd(const float *load, const float *dload_h, int32_t a, in
 int32_t launch_hier_gate_product_bwd(const float *gates, float *dgates, int64_t T, int32_t k1, int32_t k2,
                                      cudaStream_t st);
 int32_t launch_add_slot_rows(const float *dX_sec, int64_t T, int32_t k1, int32_t d, float *dX_gate, cudaStream_t st);
-int32_t launch_cv2_grad(const float *v, int32_t m, float scale, float *out, cudaStream_t st);
 int32_t launch_add_gathered(float *dgates, const int32_t *topk_idx, const float *dimp, int64_t R, int32_t n,
                             cudaStream_t st);
 
@@ -232,6 +262,7 @@ struct SimtGemm {
     void *C2;
     int64_t b_split, c_split;
     int32_t b_k_contiguous;
+    int32_t *clear;            // status word, cleared if given
     const int32_t *row_count;  // mode 0 without segments: number of rows, read on the device (at most M)
     // optional row gathers through a permutation: mode 0: A row i reads row a_row_index[i] / a_row_div
     // and C row i is written at c_row_index[i]; mode 1: the contraction index r reads A row
@@ -244,18 +275,21 @@ struct SimtGemm {
 // Mode 1 over segments: K is the number of rows of all segments. part: simt_wgrad_splits(M, N, nseg, K) * nseg * M * N
 // floats let a product with few tiles be cut along its contraction (float results only)
 int32_t simt_wgrad_splits(int64_t M, int64_t N, int32_t nseg, int64_t K);
-int32_t launch_simt_gemm(const SimtGemm &g, int32_t *tile_prefix, cudaStream_t st, float *part = nullptr);
+int32_t launch_simt_gemm(const SimtGemm &g, int32_t *tile_prefix, cudaStream_t st, float *part = nullptr,
+                         const SegmentPlan *plan = nullptr);  // plan: tile prefixes made already (heights 16 / 32 / 64)
 // out[e, j] = sum over the rows of segment e of in[r, j]   (out, in of the act type)
 int64_t colsum_ws_floats(int64_t R, int32_t n, int32_t N);
 int32_t launch_segment_colsum(const void *in, int32_t act, const int32_t *offsets, int32_t nseg, int64_t R,
-                              int32_t N, void *out, float *scratch, int32_t *tile_prefix, cudaStream_t st);
+                              int32_t N, void *out, float *scratch, const int32_t *tile_prefix, cudaStream_t st);
+constexpr int COLSUM_ROWS = 128;  // height of the tiles of tile_prefix
 
 // ----------------------------------------------------------------------------- tensor-core experts (ffn_tc.cu)
 bool tc_ffn_supported(const moe_config &c);
-int64_t tc_ffn_ws_bytes(const moe_config &c);
+int32_t tc_row_tile(int64_t R, int32_t nseg, int32_t flags);  // tile height of the row GEMMs: what plan.bm[0] has to be
+bool tc_wgrad_sorted(const moe_config &c);                    // the weight gradients want plan.sched
 // first_only: only hid = relu(xs.W1 + b1) (the recomputation of the hidden activations in the backward pass)
 int32_t launch_tc_ffn(const moe_config &c, const void *xs, const int32_t *offsets, const void *W1, const void *b1,
-                      const void *W2, const void *b2, void *hid, void *ys, void *ws, int32_t *status_word,
+                      const void *W2, const void *b2, void *hid, void *ys, const SegmentPlan &plan, int32_t *status_word,
                       cudaStream_t st, bool first_only = false, uint32_t *relu_bits = nullptr);
 // relu_bits [R, h / 32]: one bit per hidden activation (set where hid > 0), written by the first expert GEMM if given;
 // the backward then masks dz with these bits instead of reading hid again as a mask (16 times less traffic)
@@ -310,7 +344,7 @@ int64_t tc_tile_ws_ints(int64_t R, int64_t nseg);  // int32s of a [nseg + 1] til
 int64_t tc_colsum_part_floats(int64_t R, int32_t nseg, int32_t N);  // scratch of the fused bias-gradient sums
 int32_t launch_tc_ffn_bwd(const moe_config &c, const void *xs, const void *hid, const void *dys,
                           const int32_t *offsets, const void *W1, const void *W2, void *dxs, void *dW1, void *db1,
-                          void *dW2, void *db2, void *dz, float *colsum, int32_t *tile_prefix, int32_t *status_word,
+                          void *dW2, void *db2, void *dz, float *colsum, const SegmentPlan &plan, int32_t *status_word,
                           cudaStream_t st, const uint32_t *relu_bits = nullptr);
 
 }  // namespace moe

@@ -558,7 +558,8 @@ __global__ void __launch_bounds__(256, LAYER ? 3 : 1) combine_bwd_kernel(const X
                                                           const int32_t *__restrict__ inv_perm, int64_t T,
                                                           int32_t k, int32_t d, float *__restrict__ dgates,
                                                           XT *__restrict__ dys, const uint8_t *__restrict__ keep,
-                                                          float keep_scale) {
+                                                          float keep_scale, const int32_t *__restrict__ topk_idx,
+                                                          const float *__restrict__ dimp, int32_t n) {
     wait_previous_kernel();
     constexpr int VN = 16 / sizeof(XT);
     const int lane = threadIdx.x & 31;
@@ -566,6 +567,11 @@ __global__ void __launch_bounds__(256, LAYER ? 3 : 1) combine_bwd_kernel(const X
     const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
     const int nvec = d / VN;
     for (int64_t t = warp; t < T; t += nwarps) {
+        float imp = 0.0f;  // lane s: what the Importance loss adds to slot s (loaded beside the rows, used at the end)
+        if (dimp && lane < k) {
+            const int32_t e = topk_idx[t * k + lane];
+            if ((uint32_t)e < (uint32_t)n) imp = dimp[e];
+        }
         int64_t rowo[KT];
         float g[KT], dot[KT];
         bool valid[KT];
@@ -628,7 +634,8 @@ __global__ void __launch_bounds__(256, LAYER ? 3 : 1) combine_bwd_kernel(const X
                 float v = dot[s];
 #pragma unroll
                 for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-                if (lane == 0) dgates[t * k + s] = valid[s] ? v : 0.0f;
+                const float imp_s = __shfl_sync(0xffffffffu, imp, s);
+                if (lane == 0) dgates[t * k + s] = (valid[s] ? v : 0.0f) + imp_s;
             }
         }
     }
@@ -636,16 +643,17 @@ __global__ void __launch_bounds__(256, LAYER ? 3 : 1) combine_bwd_kernel(const X
 
 int32_t launch_combine_bwd(const void *dY, const void *ys, int32_t act, const float *gates,
                            const int32_t *inv_perm, int64_t T, int32_t k, int32_t d, float *dgates, void *dys,
-                           cudaStream_t st, const uint8_t *keep, float keep_scale) {
+                           cudaStream_t st, const uint8_t *keep, float keep_scale, const int32_t *topk_idx,
+                           const float *dimp, int32_t n) {
     if (T == 0) return MOE_OK;
     const unsigned grid = (unsigned)imin(cdiv(T, 8), 148 * 16);
 #define MOE_CALL_L(KT, VB, L)                                                                                            \
     if (act == MOE_BF16)                                                                                                 \
         launch_kernel((combine_bwd_kernel<bf16, KT, VB, L>), grid, 256, 0, st, (const bf16 *)dY, (const bf16 *)ys, gates, inv_perm, T, \
-                                                                   k, d, dgates, (bf16 *)dys, keep, keep_scale);          \
+                                                                   k, d, dgates, (bf16 *)dys, keep, keep_scale, topk_idx, dimp, n);          \
     else                                                                                                                 \
         launch_kernel((combine_bwd_kernel<float, KT, VB, L>), grid, 256, 0, st, (const float *)dY, (const float *)ys, gates, inv_perm, \
-                                                                    T, k, d, dgates, (float *)dys, keep, keep_scale)
+                                                                    T, k, d, dgates, (float *)dys, keep, keep_scale, topk_idx, dimp, n)
 #define MOE_CALL(KT, VB)                     \
     if (keep) { MOE_CALL_L(KT, VB, true); }  \
     else { MOE_CALL_L(KT, VB, false); }
