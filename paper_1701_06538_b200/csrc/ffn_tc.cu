@@ -566,8 +566,8 @@ template <int KIND, int TM> struct TileIter {
 // into sub-blocks of p.sub_kb0 / p.sub_kb K blocks (first term / other terms). Each sub-block is accumulated in TMEM on
 // its own (an fp32 tensor-core accumulator truncates, and a long run of same-sign terms loses low bits: 128 rows keep
 // that below 1e-5), handed to the epilogue like a tile, and added there, with rounding to nearest, to running sums in
-// shared memory (32 rows x 128 columns of floats per warp, 16-byte units swizzled by row); the sums go to global memory
-// once per tile. Two stages of operands make room for the 128 KiB of sums.
+// registers (a lane's row of the warp's 128 columns); the sums go to global memory once per tile. (With the sums in shared
+// memory, which left room for two operand stages, a K block took 1850 cycles: the latency of its loads.)
 template <int KIND, bool ACC = false>
 __global__ void __launch_bounds__(NTHREADS, 1)
 grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -575,7 +575,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;  // 1024-B aligned for the 128-B swizzle
     uint8_t *smem = smem_raw + (base - smem_u32(smem_raw));
-    constexpr int NST = ACC ? 2 : STAGES;
+    constexpr int NST = STAGES;
     const uint32_t bars = base + NST * STAGE_BYTES;
     auto full_bar = [&](int s) { return bars + 8u * s; };
     auto empty_bar = [&](int s) { return bars + 8u * (NST + s); };
@@ -727,12 +727,15 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         Tile t;
         while (ok && it.next(t)) {
             const bool have_acc = t.kblocks > 0;
-            if (ACC) {
+            if constexpr (ACC) {
+                // a lane's row of the warp's 128 columns: the running sums stay in registers
                 const int half_a = (warp - 2) >> 2;
-                uint8_t *sums = smem + NST * STAGE_BYTES + 256 + (warp - 2) * 16384;  // [32 rows][32 x 16 B], unit ^ row
+                float sums[4][32];
+#pragma unroll
+                for (int i = 0; i < 128; ++i) sums[i >> 5][i & 31] = 0.0f;
                 const int sub = t.e < p.segs_term0 ? p.sub_kb0 : p.sub_kb;
                 const int nsub = (t.kblocks + sub - 1) / sub;
-                for (int sb = 0; sb < nsub && ok; ++sb) {
+                for (int sb = 0; sb < nsub; ++sb) {
                     ok = mbar_wait(tfull_bar(acc), acc_ph, abort_flag, p.status);
                     if (!ok) break;
                     tc_fence_after();
@@ -741,36 +744,38 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                         uint32_t v[32];
                         tc_ld_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + (half_a * 4 + cl) * 32, v);
                         tc_ld_wait();
-#pragma unroll
-                        for (int q = 0; q < 8; ++q) {
-                            float4 *cell = reinterpret_cast<float4 *>(sums + lane * 512 + ((((cl * 8 + q) ^ lane) & 31) << 4));
-                            float4 a = make_float4(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]),
-                                                   __uint_as_float(v[4 * q + 2]), __uint_as_float(v[4 * q + 3]));
-                            if (sb > 0) {
-                                const float4 o = *cell;
-                                a.x += o.x; a.y += o.y; a.z += o.z; a.w += o.w;
-                            }
-                            *cell = a;
+                        if (cl == 3) {  // the accumulator is read: it goes back before the last additions
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(tempty_bar(acc));
                         }
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) sums[cl][j] += __uint_as_float(v[j]);
                     }
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(tempty_bar(acc));
                     if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
                 }
                 if (!ok) break;
-                // the warp's 32 x 128 sums to global memory, one 512-byte row segment per instruction
+                // to global memory by way of the warp's 4 KiB: lane l moves piece l % 8 of row 4 * i + l / 8
+                uint8_t *slab = smem + NST * STAGE_BYTES + 1024 + (warp - 2) * 4096;
                 const int64_t row0 = (int64_t)t.m0 + quarter * 32;
-                float *dst = p.out_f32 + (int64_t)t.e * p.M * p.N + row0 * p.N + t.n0 + half_a * 128 + lane * 4;
-                if (t.n0 + half_a * 128 + lane * 4 < p.N) {
-                    for (int i = 0; i < 32; ++i) {
-                        if (row0 + i >= p.M) break;
-                        float4 val = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                        if (nsub > 0) val = *reinterpret_cast<const float4 *>(sums + i * 512 + (((lane ^ i) & 31) << 4));
-                        *reinterpret_cast<float4 *>(dst + (int64_t)i * p.N) = val;
+                float *dst = p.out_f32 + (int64_t)t.e * p.M * p.N + row0 * p.N + t.n0 + half_a * 128 + (lane & 7) * 4;
+#pragma unroll
+                for (int cl = 0; cl < 4; ++cl) {
+                    if (t.n0 + half_a * 128 + cl * 32 >= p.N) break;
+#pragma unroll
+                    for (int q = 0; q < 8; ++q)
+                        *reinterpret_cast<float4 *>(slab + lane * 128 + ((q ^ (lane & 7)) << 4)) =
+                            make_float4(sums[cl][4 * q], sums[cl][4 * q + 1], sums[cl][4 * q + 2], sums[cl][4 * q + 3]);
+                    __syncwarp();
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int row = 4 * i + (lane >> 3);
+                        if (row0 + row < p.M)
+                            *reinterpret_cast<float4 *>(dst + (int64_t)row * p.N + cl * 32) =
+                                *reinterpret_cast<const float4 *>(slab + row * 128 + (((lane & 7) ^ (row & 7)) << 4));
                     }
+                    __syncwarp();
                 }
-                __syncwarp();  // the sums are read before the next tile overwrites them
                 continue;
             }
             // Two warps share each quarter of the accumulator's rows and take two boxes of 64 columns each.
@@ -1450,20 +1455,19 @@ template <int KIND> int32_t launch(const CUtensorMap &tmA, const CUtensorMap &tm
     return MOE_OK;
 }
 
-// The sub-block accumulating wgrad (float output): two operand stages + 128 KiB of running sums
-constexpr int SMEM_ACC_BYTES = 2 * STAGE_BYTES + 1024 + 256 + 8 * 16384;
+// The sub-block accumulating wgrad (float output)
 int32_t launch_acc_wgrad(const CUtensorMap &tmA, const CUtensorMap &tmB, const GemmParams &p_in, int64_t max_tiles,
                          cudaStream_t st) {
     GemmParams p = p_in;
     MOE_TRY((complete_params<WGRAD, BM>(p, max_tiles)));
     static bool configured = false;
     if (!configured) {
-        MOE_CUDA(cudaFuncSetAttribute(grouped_gemm_kernel<WGRAD, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_ACC_BYTES));
+        MOE_CUDA(cudaFuncSetAttribute(grouped_gemm_kernel<WGRAD, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
         configured = true;
     }
     if (max_tiles <= 0) return MOE_OK;
     const unsigned grid = (unsigned)imin(max_tiles, sm_count());
-    launch_kernel((grouped_gemm_kernel<WGRAD, true>), grid, NTHREADS, SMEM_ACC_BYTES, st, tmA, tmB, tmA, p);
+    launch_kernel((grouped_gemm_kernel<WGRAD, true>), grid, NTHREADS, SMEM_BYTES, st, tmA, tmB, tmA, p);
     MOE_LAUNCHED();
     return MOE_OK;
 }
