@@ -45,6 +45,9 @@ constexpr int NTHREADS2 = 384;  // two-CTA kernel: + one warp that fixes the rag
 constexpr unsigned long long WAIT_LIMIT_NS = 2000000000ull;
 
 enum Kind { ROW_BMN = 0, ROW_BK = 1, WGRAD = 2 };
+// What the epilogue does with an accumulator, fixed at compile time (a run-time choice kept every variant's registers and
+// code in one kernel: 950 cycles for the 32 conversions of a box without any option)
+enum Epilogue { EPI_PLAIN = 0, EPI_BIAS = 1, EPI_RELU = 2, EPI_MASK = 4, EPI_BITS = 8, EPI_F32 = 16 };
 
 constexpr int MAX_TERMS = 8;
 
@@ -264,9 +267,10 @@ __device__ __forceinline__ float warp_column_sums(float (&a)[32], int lane) {
 // Epilogue arithmetic of one thread's 32 accumulator columns: bias, ReLU, ReLU mask, rounding to bf16. The three
 // options are template parameters so that the loop body has no branches (with run-time flags every element pair became
 // its own basic block and the chain add -> max -> convert ran serially, 16 times).
-template <bool BIAS, bool RELU, bool MASK, bool BITS = false>
-__device__ __forceinline__ void pack32_mode(const uint32_t (&v)[32], const uint4 (&bias_raw)[4], const uint4 (&mask_raw)[4],
-                                            uint4 (&packed)[4], uint32_t keep_word = 0u) {
+template <int EPI>
+__device__ __forceinline__ void pack32(const uint32_t (&v)[32], const uint4 (&bias_raw)[4], const uint4 (&mask_raw)[4],
+                                            uint4 (&packed)[4], uint32_t keep_word) {
+    constexpr bool BIAS = EPI & EPI_BIAS, RELU = EPI & EPI_RELU, MASK = EPI & EPI_MASK, BITS = EPI & EPI_BITS;
     const uint32_t *bw = reinterpret_cast<const uint32_t *>(bias_raw);
     const uint32_t *mw = reinterpret_cast<const uint32_t *>(mask_raw);
     uint32_t *out = reinterpret_cast<uint32_t *>(packed);
@@ -307,25 +311,6 @@ __device__ __forceinline__ uint32_t positive_bits(const uint4 (&packed)[4]) {
     const uint32_t all = even | odd;
     return spread_bits(all & 0xffffu) | (spread_bits(all >> 16) << 1);
 }
-// mode: bit 0 bias, bit 1 ReLU, bit 2 mask, bit 3 mask as bits (the combinations the layer uses are specialised)
-__device__ __forceinline__ void pack32(int mode, const uint32_t (&v)[32], const uint4 (&bias_raw)[4],
-                                       const uint4 (&mask_raw)[4], uint4 (&packed)[4], uint32_t keep_word = 0u) {
-    if (mode & 8) {
-        pack32_mode<false, false, false, true>(v, bias_raw, mask_raw, packed, keep_word);
-        return;
-    }
-    switch (mode) {
-        case 0: pack32_mode<false, false, false>(v, bias_raw, mask_raw, packed); break;
-        case 1: pack32_mode<true, false, false>(v, bias_raw, mask_raw, packed); break;
-        case 3: pack32_mode<true, true, false>(v, bias_raw, mask_raw, packed); break;
-        case 4: pack32_mode<false, false, true>(v, bias_raw, mask_raw, packed); break;
-        case 2: pack32_mode<false, true, false>(v, bias_raw, mask_raw, packed); break;
-        case 5: pack32_mode<true, false, true>(v, bias_raw, mask_raw, packed); break;
-        case 6: pack32_mode<false, true, true>(v, bias_raw, mask_raw, packed); break;
-        default: pack32_mode<true, true, true>(v, bias_raw, mask_raw, packed); break;
-    }
-}
-
 // The bias values of a 64-column box, the same for every lane (broadcast loads). They are fetched one box ahead: the
 // first box's before the warp waits for its accumulator.
 __device__ __forceinline__ void bias_load(const bf16 *bias, uint4 (&out)[2][4]) {
@@ -352,8 +337,8 @@ struct BoxArgs {
     uint2 keep;                 // mask bits
     bool have_acc, wait_box;    // wait_box: an earlier store may still be reading the box
 };
-template <bool MASKT, typename Release>
-__device__ __forceinline__ void epilogue_box(const GemmParams &p, int pack_mode, int lane, const BoxArgs &b, uint4 (&bias)[2][4],
+template <int EPI, bool MASKT, typename Release>
+__device__ __forceinline__ void epilogue_box(const GemmParams &p, int lane, const BoxArgs &b, uint4 (&bias)[2][4],
                                              Release release) {
     uint32_t v[2][32];
     if (b.have_acc) {
@@ -365,7 +350,7 @@ __device__ __forceinline__ void epilogue_box(const GemmParams &p, int pack_mode,
 #pragma unroll
         for (int j = 0; j < 64; ++j) v[j >> 5][j & 31] = 0u;
     }
-    if (p.out_f32) {  // 128-byte row segments: lane l moves piece l % 8 of row 4 * i + l / 8
+    if constexpr (EPI & EPI_F32) {  // 128-byte row segments: lane l moves piece l % 8 of row 4 * i + l / 8
         const int my_piece = lane & 7, my_sub = lane >> 3;
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
@@ -384,7 +369,7 @@ __device__ __forceinline__ void epilogue_box(const GemmParams &p, int pack_mode,
             __syncwarp();
         }
         return;
-    }
+    } else {
     const bool row_ok = lane < b.rows_valid, staged = p.tma_out && b.rows_valid >= 32;
     const int64_t out_row = b.row0 + lane;
     uint8_t *mine = b.box + lane * 128;
@@ -395,14 +380,14 @@ __device__ __forceinline__ void epilogue_box(const GemmParams &p, int pack_mode,
         if (MASKT) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) mask_raw[q] = *reinterpret_cast<const uint4 *>(mine + (((u * 4 + q) ^ (lane & 7)) << 4));
-        } else if (p.mask && row_ok) {
+        } else if ((EPI & EPI_MASK) && row_ok) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) mask_raw[q] = reinterpret_cast<const uint4 *>(p.mask + out_row * p.N + b.col0 + 32 * u)[q];
         }
-        pack32(pack_mode, v[u], bias[u], mask_raw, packed[u], u ? b.keep.y : b.keep.x);
+        pack32<EPI>(v[u], bias[u], mask_raw, packed[u], u ? b.keep.y : b.keep.x);
     }
-    if (b.next_bias) bias_load(b.next_bias, bias);
-    if (p.bits_out && row_ok)
+    if ((EPI & EPI_BIAS) && b.next_bias) bias_load(b.next_bias, bias);
+    if ((EPI & EPI_RELU) && p.bits_out && row_ok)
         *reinterpret_cast<uint2 *>(p.bits_out + out_row * (p.N >> 5) + (b.col0 >> 5)) =
             make_uint2(positive_bits(packed[0]), positive_bits(packed[1]));
     if (staged) {
@@ -418,7 +403,7 @@ __device__ __forceinline__ void epilogue_box(const GemmParams &p, int pack_mode,
             tma_store_2d(b.tm_out, smem_u32(b.box), b.col0, b.map_row);
             tma_store_commit();
         }
-        if (p.colsum_part) {
+        if ((EPI & (EPI_MASK | EPI_BITS)) && p.colsum_part) {
             // sums of the box's columns over its 32 rows: a lane reads its two columns down the rows (one 4-byte word a
             // row, conflict free), half the instructions of a butterfly over registers
             float s0 = 0.0f, s1 = 0.0f, u0 = 0.0f, u1 = 0.0f;
@@ -440,7 +425,7 @@ __device__ __forceinline__ void epilogue_box(const GemmParams &p, int pack_mode,
 #pragma unroll
         for (int q = 0; q < 4; ++q) st_global_32B(dst + 2 * q, packed[q >> 1][2 * (q & 1)], packed[q >> 1][2 * (q & 1) + 1]);
     }
-    if (p.colsum_part) {  // sums of the rounded values, rows past the segment end count as 0; the whole warp: shuffles
+    if ((EPI & (EPI_MASK | EPI_BITS)) && p.colsum_part) {  // sums of the rounded values, rows past the segment end count as 0; the whole warp: shuffles
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             float a[32];
@@ -452,6 +437,7 @@ __device__ __forceinline__ void epilogue_box(const GemmParams &p, int pack_mode,
             }
             p.colsum_part[b.colsum_row * p.N + b.col0 + 32 * u + lane] = warp_column_sums(a, lane);
         }
+    }
     }
 }
 // mask bits of a row's 128 columns from col0 on (two boxes), as far as the row has them
@@ -568,7 +554,7 @@ template <int KIND, int TM> struct TileIter {
 // that below 1e-5), handed to the epilogue like a tile, and added there, with rounding to nearest, to running sums in
 // registers (a lane's row of the warp's 128 columns); the sums go to global memory once per tile. (With the sums in shared
 // memory, which left room for two operand stages, a K block took 1850 cycles: the latency of its loads.)
-template <int KIND, bool ACC = false>
+template <int KIND, int EPI, bool ACC = false>
 __global__ void __launch_bounds__(NTHREADS, 1)
 grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ CUtensorMap tmO, const GemmParams p) {
@@ -719,7 +705,6 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     } else {
         // ------------------------------------------------------------------ epilogue (warps 2..9)
         const int quarter = warp & 3;  // TMEM lanes 32*quarter .. 32*quarter + 31 belong to this warp
-        const int pack_mode = p.bits_in ? 8 : (p.bias ? 1 : 0) | (p.relu ? 2 : 0) | (p.mask ? 4 : 0);
         int acc = 0;
         uint32_t acc_ph = 0;
         bool ok = true;
@@ -793,10 +778,10 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             b.have_acc = have_acc;
             b.wait_box = true;
             uint4 bias[2][4];
-            const bf16 *bias_at = p.bias ? p.bias + (int64_t)t.e * p.N + first : nullptr;
-            if (bias_at && boxes > 0) bias_load(bias_at, bias);
+            const bf16 *bias_at = (EPI & EPI_BIAS) ? p.bias + (int64_t)t.e * p.N + first : nullptr;
+            if ((EPI & EPI_BIAS) && boxes > 0) bias_load(bias_at, bias);
             uint2 keep[2] = {make_uint2(0u, 0u), make_uint2(0u, 0u)};
-            if (p.bits_in && lane < b.rows_valid) keep_load(p, b.row0 + lane, first, keep);
+            if ((EPI & EPI_BITS) && lane < b.rows_valid) keep_load(p, b.row0 + lane, first, keep);
             if (have_acc) {  // (the loads above are in flight while the warp waits for its accumulator)
                 ok = mbar_wait(tfull_bar(acc), acc_ph, abort_flag, p.status);
                 if (!ok) break;
@@ -810,9 +795,9 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             for (int u = 0; u < boxes; ++u) {
                 b.col0 = first + 64 * u;
                 b.taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + half * (BN / 2) + 64 * u;
-                b.next_bias = bias_at && u + 1 < boxes ? bias_at + 64 : nullptr;
+                b.next_bias = (EPI & EPI_BIAS) && u + 1 < boxes ? bias_at + 64 : nullptr;
                 b.keep = u ? keep[1] : keep[0];
-                epilogue_box<false>(p, pack_mode, lane, b, bias, [&]() { if (u + 1 == boxes) release(); });
+                epilogue_box<EPI, false>(p, lane, b, bias, [&]() { if (u + 1 == boxes) release(); });
             }
             if (have_acc) {
                 if (boxes == 0) release();
@@ -984,7 +969,7 @@ template <int KIND> struct PairTiles {
 
 // MASKT: the ReLU mask of the dgrad GEMM is not read row by row from global memory by the epilogue but
 // fetched as a 128 x 256 tile by TMA (one stage fewer in exchange for the 64 KiB it occupies).
-template <int KIND, bool MASKT>
+template <int KIND, int EPI, bool MASKT>
 __global__ void __launch_bounds__(NTHREADS2, 1)
 grouped_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                      const __grid_constant__ CUtensorMap tmM, const __grid_constant__ CUtensorMap tmO,
@@ -1248,7 +1233,6 @@ grouped_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     } else {
         // ------------------------------------------------------------------ epilogue (warps 2..9, both CTAs)
         const int quarter = warp & 3, half = (warp - 2) >> 2;
-        const int pack_mode = p.bits_in ? 8 : (p.bias ? 1 : 0) | (p.relu ? 2 : 0) | (p.mask ? 4 : 0);
         uint32_t mask_ph = 0;
         int acc = 0;
         uint32_t acc_ph = 0;
@@ -1272,10 +1256,10 @@ grouped_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
             b.have_acc = have_acc;
             b.wait_box = true;
             uint4 bias[2][4];
-            const bf16 *bias_at = p.bias ? p.bias + (int64_t)t.e * p.N + first : nullptr;
-            if (bias_at && boxes > 0) bias_load(bias_at, bias);
+            const bf16 *bias_at = (EPI & EPI_BIAS) ? p.bias + (int64_t)t.e * p.N + first : nullptr;
+            if ((EPI & EPI_BIAS) && boxes > 0) bias_load(bias_at, bias);
             uint2 keep[2] = {make_uint2(0u, 0u), make_uint2(0u, 0u)};
-            if (p.bits_in && lane < b.rows_valid) keep_load(p, b.row0 + lane, first, keep);
+            if ((EPI & EPI_BITS) && lane < b.rows_valid) keep_load(p, b.row0 + lane, first, keep);
             if (have_acc) {  // (the loads above are in flight while the warp waits for its accumulator)
                 ok = mbar_wait(tfull_bar(acc), acc_ph, abort_flag, p.status);
                 if (!ok) break;
@@ -1296,9 +1280,9 @@ grouped_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                 b.col0 = first + 64 * u;
                 b.taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + half * (BN / 2) + 64 * u;
                 b.box = smem + NST * STAGE2_BYTES + (MASKT ? (2 * half + u) * 16384 + quarter * 4096 : (warp - 2) * 4096);
-                b.next_bias = bias_at && u + 1 < boxes ? bias_at + 64 : nullptr;
+                b.next_bias = (EPI & EPI_BIAS) && u + 1 < boxes ? bias_at + 64 : nullptr;
                 b.keep = u ? keep[1] : keep[0];
-                epilogue_box<MASKT>(p, pack_mode, lane, b, bias, [&]() { if (u + 1 == boxes) release(); });
+                epilogue_box<EPI, MASKT>(p, lane, b, bias, [&]() { if (u + 1 == boxes) release(); });
             }
             if (have_acc) {
                 if (boxes == 0) release();
@@ -1438,21 +1422,36 @@ template <int KIND, int TM> int32_t complete_params(GemmParams &q, int64_t max_t
     return MOE_OK;
 }
 
+template <int KIND, int EPI> int32_t launch_as(const CUtensorMap &tmA, const CUtensorMap &tmB, const GemmParams &p, unsigned grid,
+                                               cudaStream_t st, const CUtensorMap &tmO) {
+    static bool configured = false;
+    if (!configured) {
+        MOE_CUDA(cudaFuncSetAttribute(grouped_gemm_kernel<KIND, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
+        configured = true;
+    }
+    if (grid == 0) return MOE_OK;
+    launch_kernel(grouped_gemm_kernel<KIND, EPI>, grid, NTHREADS, SMEM_BYTES, st, tmA, tmB, tmO, p);
+    MOE_LAUNCHED();
+    return MOE_OK;
+}
 template <int KIND> int32_t launch(const CUtensorMap &tmA, const CUtensorMap &tmB, const GemmParams &p_in,
                                    int64_t max_tiles, cudaStream_t st, const CUtensorMap *tmO = nullptr) {
     GemmParams p = p_in;
     p.tma_out = tmO != nullptr;
     MOE_TRY((complete_params<KIND, BM>(p, max_tiles)));
-    static bool configured = false;
-    if (!configured) {
-        MOE_CUDA(cudaFuncSetAttribute(grouped_gemm_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
-        configured = true;
+    const unsigned grid = max_tiles > 0 ? (unsigned)imin(max_tiles, sm_count()) : 0u;
+    const CUtensorMap &out = tmO ? *tmO : tmA;
+    if (p.out_f32) return launch_as<KIND, EPI_F32>(tmA, tmB, p, grid, st, out);
+    if constexpr (KIND == ROW_BMN) {
+        if (p.relu) return launch_as<KIND, EPI_BIAS | EPI_RELU>(tmA, tmB, p, grid, st, out);
+        return launch_as<KIND, EPI_BIAS>(tmA, tmB, p, grid, st, out);
+    } else {
+        if constexpr (KIND == ROW_BK) {
+            if (p.bits_in) return launch_as<KIND, EPI_BITS>(tmA, tmB, p, grid, st, out);
+            if (p.mask) return launch_as<KIND, EPI_MASK>(tmA, tmB, p, grid, st, out);
+        }
+        return launch_as<KIND, EPI_PLAIN>(tmA, tmB, p, grid, st, out);
     }
-    if (max_tiles <= 0) return MOE_OK;
-    const unsigned grid = (unsigned)imin(max_tiles, sm_count());
-    launch_kernel(grouped_gemm_kernel<KIND>, grid, NTHREADS, SMEM_BYTES, st, tmA, tmB, tmO ? *tmO : tmA, p);
-    MOE_LAUNCHED();
-    return MOE_OK;
 }
 
 // The sub-block accumulating wgrad (float output)
@@ -1462,19 +1461,19 @@ int32_t launch_acc_wgrad(const CUtensorMap &tmA, const CUtensorMap &tmB, const G
     MOE_TRY((complete_params<WGRAD, BM>(p, max_tiles)));
     static bool configured = false;
     if (!configured) {
-        MOE_CUDA(cudaFuncSetAttribute(grouped_gemm_kernel<WGRAD, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
+        MOE_CUDA(cudaFuncSetAttribute(grouped_gemm_kernel<WGRAD, EPI_F32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
         configured = true;
     }
     if (max_tiles <= 0) return MOE_OK;
     const unsigned grid = (unsigned)imin(max_tiles, sm_count());
-    launch_kernel((grouped_gemm_kernel<WGRAD, true>), grid, NTHREADS, SMEM_BYTES, st, tmA, tmB, tmA, p);
+    launch_kernel((grouped_gemm_kernel<WGRAD, EPI_F32, true>), grid, NTHREADS, SMEM_BYTES, st, tmA, tmB, tmA, p);
     MOE_LAUNCHED();
     return MOE_OK;
 }
 
-template <int KIND, bool MASKT = false>
-int32_t launch2(const CUtensorMap &tmA, const CUtensorMap &tmB, const GemmParams &p_in, int64_t max_tiles,
-                cudaStream_t st, const CUtensorMap *tmM = nullptr, const CUtensorMap *tmO = nullptr) {
+template <int KIND, int EPI, bool MASKT = false>
+int32_t launch2_as(const CUtensorMap &tmA, const CUtensorMap &tmB, const GemmParams &p_in, int64_t max_tiles,
+                   cudaStream_t st, const CUtensorMap *tmM, const CUtensorMap *tmO) {
     GemmParams p = p_in;
     p.tma_out = tmO != nullptr;
     MOE_TRY((complete_params<KIND, 256>(p, max_tiles)));
@@ -1489,10 +1488,10 @@ int32_t launch2(const CUtensorMap &tmA, const CUtensorMap &tmB, const GemmParams
     cfg.blockDim = dim3(NTHREADS2); cfg.dynamicSmemBytes = SMEM2_BYTES; cfg.stream = st;
     cfg.attrs = attrs; cfg.numAttrs = 2;
     if (!max_clusters) {
-        MOE_CUDA(cudaFuncSetAttribute(grouped_gemm2_kernel<KIND, MASKT>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM2_BYTES));
+        MOE_CUDA(cudaFuncSetAttribute((grouped_gemm2_kernel<KIND, EPI, MASKT>), cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM2_BYTES));
         cfg.gridDim = dim3(2 * (sm_count() / 2));
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, grouped_gemm2_kernel<KIND, MASKT>, &cfg) != cudaSuccess || n <= 0) return MOE_ERR_CUDA;
+        if (cudaOccupancyMaxActiveClusters(&n, (grouped_gemm2_kernel<KIND, EPI, MASKT>), &cfg) != cudaSuccess || n <= 0) return MOE_ERR_CUDA;
         max_clusters = n;
     }
     if (max_tiles <= 0) return MOE_OK;
@@ -1504,9 +1503,27 @@ int32_t launch2(const CUtensorMap &tmA, const CUtensorMap &tmB, const GemmParams
     }
 #endif
     cfg.gridDim = dim3(2 * (unsigned)imin(max_tiles, max_clusters));
-    MOE_CUDA(cudaLaunchKernelEx(&cfg, grouped_gemm2_kernel<KIND, MASKT>, tmA, tmB, tmM ? *tmM : tmA, tmO ? *tmO : tmA, p));
+    MOE_CUDA(cudaLaunchKernelEx(&cfg, (grouped_gemm2_kernel<KIND, EPI, MASKT>), tmA, tmB, tmM ? *tmM : tmA, tmO ? *tmO : tmA, p));
     MOE_LAUNCHED();
     return MOE_OK;
+}
+
+template <int KIND>
+int32_t launch2(const CUtensorMap &tmA, const CUtensorMap &tmB, const GemmParams &p, int64_t max_tiles, cudaStream_t st,
+                const CUtensorMap *tmM = nullptr, const CUtensorMap *tmO = nullptr) {
+    if constexpr (KIND != WGRAD) {
+        if (p.out_f32) return launch2_as<KIND, EPI_F32>(tmA, tmB, p, max_tiles, st, tmM, tmO);
+    }
+    if constexpr (KIND == ROW_BMN) {
+        if (p.relu) return launch2_as<KIND, EPI_BIAS | EPI_RELU>(tmA, tmB, p, max_tiles, st, tmM, tmO);
+        return launch2_as<KIND, EPI_BIAS>(tmA, tmB, p, max_tiles, st, tmM, tmO);
+    } else {
+        if constexpr (KIND == ROW_BK) {
+            if (p.bits_in) return launch2_as<KIND, EPI_BITS>(tmA, tmB, p, max_tiles, st, tmM, tmO);
+            if (p.mask) return launch2_as<KIND, EPI_MASK, true>(tmA, tmB, p, max_tiles, st, tmM, tmO);  // mask rows as TMA tiles
+        }
+        return launch2_as<KIND, EPI_PLAIN>(tmA, tmB, p, max_tiles, st, tmM, tmO);
+    }
 }
 
 }  // namespace
@@ -1671,7 +1688,7 @@ int32_t tc_row_gemm(const void *A, const void *W, bool transposed, const int32_t
         if (transposed && mask && !bits_in) {  // the ReLU-mask rows come in as TMA tiles
             CUtensorMap tmM;
             MOE_TRY(map_rows_kmajor(&tmM, mask, R, N));
-            return finish(launch2<ROW_BK, true>(tmA, tmB, p, max_tiles2, st, &tmM, &tmO), 8);
+            return finish(launch2<ROW_BK>(tmA, tmB, p, max_tiles2, st, &tmM, &tmO), 8);
         }
         return finish(transposed ? launch2<ROW_BK>(tmA, tmB, p, max_tiles2, st, nullptr, &tmO)
                                  : launch2<ROW_BMN>(tmA, tmB, p, max_tiles2, st, nullptr, &tmO), 8);
