@@ -13,6 +13,9 @@ namespace moe {
 namespace {
 
 // p = softmax(c) per row: exponentials and their sum in double (largest logit subtracted), one rounding to float.
+// NV > 0: a row of at most 32 * NV columns stays in registers with its exponentials (the double exponential is what bounds this
+// kernel: 43 us when each was evaluated twice, 32768 x 256); NV = 0: any width, evaluated again.
+template <int NV>
 __global__ void __launch_bounds__(256) bal_softmax_kernel(const float *__restrict__ c, int64_t T, int32_t n,
                                                           float *__restrict__ p) {
     wait_previous_kernel();
@@ -21,14 +24,37 @@ __global__ void __launch_bounds__(256) bal_softmax_kernel(const float *__restric
     if (t >= T) return;
     const float *row = c + t * n;
     float mx = -CUDART_INF_F;
-    for (int32_t j = lane; j < n; j += 32) mx = fmaxf(mx, row[j]);
+    float v[NV > 0 ? NV : 1];
+    if (NV > 0) {
+#pragma unroll
+        for (int u = 0; u < NV; ++u) v[u] = lane + 32 * u < n ? row[lane + 32 * u] : -CUDART_INF_F;
+#pragma unroll
+        for (int u = 0; u < NV; ++u) mx = fmaxf(mx, v[u]);
+    } else {
+        for (int32_t j = lane; j < n; j += 32) mx = fmaxf(mx, row[j]);
+    }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
     double s = 0.0;
-    for (int32_t j = lane; j < n; j += 32) s += exp((double)row[j] - (double)mx);
+    double e[NV > 0 ? NV : 1];
+    if (NV > 0) {
+#pragma unroll
+        for (int u = 0; u < NV; ++u) {
+            e[u] = lane + 32 * u < n ? exp((double)v[u] - (double)mx) : 0.0;
+            s += e[u];
+        }
+    } else {
+        for (int32_t j = lane; j < n; j += 32) s += exp((double)row[j] - (double)mx);
+    }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    for (int32_t j = lane; j < n; j += 32) p[t * n + j] = (float)(exp((double)row[j] - (double)mx) / s);
+    if (NV > 0) {
+#pragma unroll
+        for (int u = 0; u < NV; ++u)
+            if (lane + 32 * u < n) p[t * n + lane + 32 * u] = (float)(e[u] / s);
+    } else {
+        for (int32_t j = lane; j < n; j += 32) p[t * n + j] = (float)(exp((double)row[j] - (double)mx) / s);
+    }
 }
 
 // out [cols, rows] = in [rows, cols]^T, 32 x 32 tiles
@@ -49,7 +75,10 @@ __global__ void __launch_bounds__(256) bal_transpose_kernel(const float *__restr
 // Batchwise mask of one expert (block = column i of p, given transposed: col [T]): the m largest values, equal values to
 // the lower token. Radix select of the m-th largest key (the bit patterns of non-negative floats order like the
 // values), then an order-preserving compaction: tok_of_row[i * m + q] = q-th kept token, and the expert's bit is set
-// in the token's mask words.
+// in the token's mask words. What bounds it is the latency of six sweeps over the column, so every sweep keeps eight loads
+// per thread in flight; a warp owns a contiguous run of tokens in the compaction, so that its place in the list needs one
+// scan over the warps. (One load at a time, a serial digit search and four barriers per 1024 tokens: 90 us at 32768 x 256.)
+constexpr int SEL_BATCH = 8;
 __global__ void __launch_bounds__(1024) bal_select_kernel(const float *__restrict__ pT, int64_t T, int32_t n, int32_t m,
                                                           int32_t words, int32_t *__restrict__ tok_of_row,
                                                           uint32_t *__restrict__ mask_bits) {
@@ -57,7 +86,7 @@ __global__ void __launch_bounds__(1024) bal_select_kernel(const float *__restric
     __shared__ int32_t hist[256];
     __shared__ int32_t warp_gt[32], warp_eq[32];
     __shared__ uint32_t s_prefix;
-    __shared__ int32_t s_need, s_base_sel, s_base_eq;
+    __shared__ int32_t s_need;
     const int32_t i = blockIdx.x;
     const uint32_t *col = reinterpret_cast<const uint32_t *>(pT + (int64_t)i * T);
     const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
@@ -67,63 +96,85 @@ __global__ void __launch_bounds__(1024) bal_select_kernel(const float *__restric
         if (tid < 256) hist[tid] = 0;
         __syncthreads();
         const uint32_t prefix = s_prefix;
-        for (int64_t t = tid; t < T; t += 1024) {
-            const uint32_t key = col[t];
-            if ((key & known) == prefix) atomicAdd(&hist[(key >> shift) & 0xFFu], 1);
+        for (int64_t t0 = tid; t0 < T; t0 += 1024 * SEL_BATCH) {
+            uint32_t key[SEL_BATCH];
+#pragma unroll
+            for (int u = 0; u < SEL_BATCH; ++u) key[u] = t0 + 1024 * u < T ? col[t0 + 1024 * u] : 0u;
+#pragma unroll
+            for (int u = 0; u < SEL_BATCH; ++u)
+                if (t0 + 1024 * u < T && (key[u] & known) == prefix) atomicAdd(&hist[(key[u] >> shift) & 0xFFu], 1);
         }
         __syncthreads();
-        if (tid == 0) {  // from the largest digit down: the digit that holds the need-th largest key
-            int32_t need = s_need;
-            int d = 255;
-            for (; d > 0; --d) {
-                if (hist[d] >= need) break;
-                need -= hist[d];
+        if (wp == 0) {  // the digit that holds the need-th largest key: lane l holds the digits 255 - 8 l .. 248 - 8 l
+            const int32_t need = s_need;
+            int32_t h[8], sum = 0;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) { h[q] = hist[255 - 8 * lane - q]; sum += h[q]; }
+            int32_t inc = sum;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int32_t o = __shfl_up_sync(0xffffffffu, inc, off);
+                if (lane >= off) inc += o;
             }
-            s_need = need;
-            s_prefix = prefix | ((uint32_t)d << shift);
+            int32_t before = inc - sum;  // keys with a larger digit than this lane's first
+            if (before < need && need <= inc) {
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    if (before < need && need <= before + h[q]) {
+                        s_need = need - before;
+                        s_prefix = prefix | ((uint32_t)(255 - 8 * lane - q) << shift);
+                    }
+                    before += h[q];
+                }
+            }
         }
         known |= 0xFFu << shift;
         __syncthreads();
     }
     const uint32_t kth = s_prefix;    // the m-th largest key
     const int32_t take_eq = s_need;   // how many of the keys equal to it are kept (the first ones in token order)
-    if (tid == 0) { s_base_sel = 0; s_base_eq = 0; }
+    const int64_t run = ((T + 31) / 32 + 31) / 32 * 32, t_first = wp * run, t_last = min(T, t_first + run);
+    int32_t gt = 0, eq = 0;
+    for (int64_t t0 = t_first + lane; t0 < t_last; t0 += 32 * SEL_BATCH) {
+        uint32_t key[SEL_BATCH];
+#pragma unroll
+        for (int u = 0; u < SEL_BATCH; ++u) key[u] = t0 + 32 * u < t_last ? col[t0 + 32 * u] : 0u;
+#pragma unroll
+        for (int u = 0; u < SEL_BATCH; ++u)
+            if (t0 + 32 * u < t_last) { gt += key[u] > kth; eq += key[u] == kth; }
+    }
+    gt = __reduce_add_sync(0xffffffffu, gt);
+    eq = __reduce_add_sync(0xffffffffu, eq);
+    if (lane == 0) { warp_gt[wp] = gt; warp_eq[wp] = eq; }
     __syncthreads();
-    for (int64_t t0 = 0; t0 < T; t0 += 1024) {
-        const int64_t t = t0 + tid;
-        const uint32_t key = t < T ? col[t] : 0u;
-        const bool gt = t < T && key > kth, eq = t < T && key == kth;
-        const uint32_t b_eq = __ballot_sync(0xffffffffu, eq);
-        if (lane == 0) warp_eq[wp] = __popc(b_eq);
-        __syncthreads();
-        int32_t eq_before = s_base_eq;
-        for (int w = 0; w < wp; ++w) eq_before += warp_eq[w];
-        const bool keep = gt || (eq && eq_before + __popc(b_eq & ((1u << lane) - 1u)) < take_eq);
-        const uint32_t b_keep = __ballot_sync(0xffffffffu, keep);
-        if (lane == 0) warp_gt[wp] = __popc(b_keep);
-        __syncthreads();
-        if (keep) {
-            int32_t pos = s_base_sel;
-            for (int w = 0; w < wp; ++w) pos += warp_gt[w];
-            pos += __popc(b_keep & ((1u << lane) - 1u));
-            if (pos < m) {  // always true: exactly m keys are kept
-                tok_of_row[(int64_t)i * m + pos] = (int32_t)t;
+    int32_t eq_base = __reduce_add_sync(0xffffffffu, lane < wp ? warp_eq[lane] : 0);  // in the warps before
+    int32_t pos = __reduce_add_sync(0xffffffffu, lane < wp ? warp_gt[lane] : 0) + min(eq_base, take_eq);
+    for (int64_t t00 = t_first; t00 < t_last; t00 += 32 * SEL_BATCH) {
+        uint32_t key[SEL_BATCH];
+#pragma unroll
+        for (int u = 0; u < SEL_BATCH; ++u) key[u] = t00 + 32 * u + lane < t_last ? col[t00 + 32 * u + lane] : 0u;
+#pragma unroll
+        for (int u = 0; u < SEL_BATCH; ++u) {
+            const int64_t t = t00 + 32 * u + lane;
+            const bool is_eq = t < t_last && key[u] == kth;
+            const uint32_t below = (1u << lane) - 1u, b_eq = __ballot_sync(0xffffffffu, is_eq);
+            const bool keep = (t < t_last && key[u] > kth) || (is_eq && eq_base + __popc(b_eq & below) < take_eq);
+            const uint32_t b_keep = __ballot_sync(0xffffffffu, keep);
+            const int32_t at = pos + __popc(b_keep & below);
+            if (keep && at < m) {  // at < m always: exactly m keys are kept
+                tok_of_row[(int64_t)i * m + at] = (int32_t)t;
                 atomicOr(&mask_bits[t * words + (i >> 5)], 1u << (i & 31));
             }
+            eq_base += __popc(b_eq);
+            pos += __popc(b_keep);
         }
-        __syncthreads();
-        if (tid == 0) {
-            int32_t a = 0, b = 0;
-            for (int w = 0; w < 32; ++w) { a += warp_gt[w]; b += warp_eq[w]; }
-            s_base_sel += a;
-            s_base_eq += b;
-        }
-        __syncthreads();
     }
 }
 
 // Per token (one warp): den = sum of p over the kept experts, cnt = how many keep it, the token's part of L_batchwise
-// (Eq. 20), and the per-expert counts of the threshold mask. Block partials of the loss go to loss_part.
+// (Eq. 20), and the per-expert counts of the threshold mask. Block partials of the loss go to loss_part. A warp takes eight
+// tokens, so that a block clears and adds up its n counts once per 64 tokens.
+constexpr int TOK_PER_WARP = 8;
 __global__ void __launch_bounds__(256) bal_token_kernel(const float *__restrict__ p, const uint32_t *__restrict__ mask_bits,
                                                         const float *__restrict__ thr, int64_t T, int32_t n, int32_t words,
                                                         float *__restrict__ den, int32_t *__restrict__ cnt,
@@ -134,10 +185,13 @@ __global__ void __launch_bounds__(256) bal_token_kernel(const float *__restrict_
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
     for (int32_t j = threadIdx.x; j < n; j += blockDim.x) s_cnt[j] = 0;
     __syncthreads();
-    const int64_t t = (int64_t)blockIdx.x * 8 + wp;
-    double d = 0.0, l = 0.0;
-    int32_t c = 0;
-    if (t < T) {
+    double loss = 0.0;
+    for (int q = 0; q < TOK_PER_WARP; ++q) {
+        const int64_t t = ((int64_t)blockIdx.x * 8 + wp) * TOK_PER_WARP + q;
+        if (t >= T) break;
+        double d = 0.0, l = 0.0;
+        int32_t c = 0;
+#pragma unroll 4
         for (int32_t j = lane; j < n; j += 32) {
             const float pj = p[t * n + j];
             const bool mb = (mask_bits[t * words + (j >> 5)] >> (j & 31)) & 1u;
@@ -146,17 +200,16 @@ __global__ void __launch_bounds__(256) bal_token_kernel(const float *__restrict_
             if (mt) atomicAdd(&s_cnt[j], 1);
             if (mt != mb) l += (mt ? 1.0 : -1.0) * ((double)pj - (double)thr[j]);
         }
-    }
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        d += __shfl_xor_sync(0xffffffffu, d, off);
-        l += __shfl_xor_sync(0xffffffffu, l, off);
-        c += __shfl_xor_sync(0xffffffffu, c, off);
+        for (int off = 16; off > 0; off >>= 1) {
+            d += __shfl_xor_sync(0xffffffffu, d, off);
+            l += __shfl_xor_sync(0xffffffffu, l, off);
+            c += __shfl_xor_sync(0xffffffffu, c, off);
+        }
+        if (lane == 0) { den[t] = (float)d; cnt[t] = c; }
+        loss += l;
     }
-    if (lane == 0) {
-        if (t < T) { den[t] = (float)d; cnt[t] = c; }
-        s_loss[wp] = l;
-    }
+    if (lane == 0) s_loss[wp] = loss;
     __syncthreads();
     for (int32_t j = threadIdx.x; j < n; j += blockDim.x)
         if (s_cnt[j]) atomicAdd(&thr_counts[j], s_cnt[j]);
@@ -223,7 +276,15 @@ __global__ void __launch_bounds__(256) bal_gather_kernel(const XT *__restrict__ 
     const int nvec = d / V16<XT>::N;
     const uint4 *src = reinterpret_cast<const uint4 *>(x + (int64_t)t * d);
     uint4 *dst = reinterpret_cast<uint4 *>(xs + r * d);
-    for (int v = lane; v < nvec; v += 32) dst[v] = src[v];
+    for (int v0 = lane; v0 < nvec; v0 += 128) {
+        uint4 val[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (v0 + 32 * u < nvec) val[u] = src[v0 + 32 * u];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (v0 + 32 * u < nvec) dst[v0 + 32 * u] = val[u];
+    }
 }
 
 // y[t] = sum over the rows of token t (ascending expert) of p[t, e] / den[t] * ys[row]   (Eq. 1 with the gates of Eq. 16)
@@ -402,7 +463,7 @@ int32_t launch_balanced_gate(const void *x, int32_t act, int64_t T, int32_t d, i
     Carver cv(ws);
     float *pT = cv.take<float>(T * n);
     int32_t *cnt = cv.take<int32_t>(T);
-    double *loss_part = cv.take<double>(cdiv(T, 8));
+    double *loss_part = cv.take<double>(cdiv(T, 8));  // one per block of the token kernel, at most
     int32_t *tile_sums = cv.take<int32_t>(cdiv(T + 1, 4096));
     MOE_CUDA(cudaMemsetAsync(mask_bits, 0, sizeof(uint32_t) * T * words, st));
     MOE_CUDA(cudaMemsetAsync(thr_counts, 0, sizeof(int32_t) * n, st));
@@ -414,16 +475,18 @@ int32_t launch_balanced_gate(const void *x, int32_t act, int64_t T, int32_t d, i
     }
     // logits by the fixed fma chain (one matrix: the projection kernel's second one is absent)
     MOE_TRY(launch_projection(x, act, T, d, n, Wg, nullptr, logits, nullptr, nullptr, 0, nullptr, 1, nullptr, st));
-    launch_kernel(bal_softmax_kernel, (unsigned)cdiv(T, 8), 256, 0, st, logits, T, n, probs);
+    if (n <= 128) launch_kernel(bal_softmax_kernel<4>, (unsigned)cdiv(T, 8), 256, 0, st, logits, T, n, probs);
+    else if (n <= 256) launch_kernel(bal_softmax_kernel<8>, (unsigned)cdiv(T, 8), 256, 0, st, logits, T, n, probs);
+    else launch_kernel(bal_softmax_kernel<0>, (unsigned)cdiv(T, 8), 256, 0, st, logits, T, n, probs);
     MOE_LAUNCHED();
     launch_kernel(bal_transpose_kernel, dim3((unsigned)cdiv(T, 32), (unsigned)cdiv(n, 32)), 256, 0, st, probs, T, n, pT);
     MOE_LAUNCHED();
     launch_kernel(bal_select_kernel, (unsigned)n, 1024, 0, st, pT, T, n, m, words, tok_of_row, mask_bits);
     MOE_LAUNCHED();
-    launch_kernel(bal_token_kernel, (unsigned)cdiv(T, 8), 256, n * sizeof(int32_t), st, probs, mask_bits, thr, T, n, words, den, cnt,
+    launch_kernel(bal_token_kernel, (unsigned)cdiv(T, 8 * TOK_PER_WARP), 256, n * sizeof(int32_t), st, probs, mask_bits, thr, T, n, words, den, cnt,
                                                                              thr_counts, loss_part);
     MOE_LAUNCHED();
-    launch_kernel(bal_loss_final_kernel, 1, 256, 0, st, loss_part, cdiv(T, 8), loss);
+    launch_kernel(bal_loss_final_kernel, 1, 256, 0, st, loss_part, cdiv(T, 8 * TOK_PER_WARP), loss);
     MOE_LAUNCHED();
     MOE_TRY(launch_exclusive_scan(cnt, (int32_t)T, tok_ptr, st, tile_sums));
     launch_kernel(bal_fill_kernel, (unsigned)cdiv(R > n ? R : n + 1, 256) + 1, 256, 0, st, tok_of_row, mask_bits, tok_ptr, R, n, m, words,
