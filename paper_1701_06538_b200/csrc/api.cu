@@ -235,8 +235,11 @@ struct LossesWs {
 struct FfnBwdWs {
     void *dz;
     float *colsum;
+    uint32_t *bits;  // MOE_FLAG_RECOMPUTE_HID on the tensor cores: the mask bits that the recomputation writes
     FfnBwdWs(Carver &cv, const Dims &D) {
         dz = cv.take_bytes(D.R * D.h * (int64_t)D.esz);
+        const bool tc = D.act == MOE_BF16 && D.d % 64 == 0 && D.h % 64 == 0;
+        bits = tc && (D.flags & MOE_FLAG_RECOMPUTE_HID) ? cv.take<uint32_t>(D.R * (D.h / 32)) : nullptr;
         int64_t cs = colsum_ws_floats(D.R, (int32_t)D.n, (int32_t)(D.h > D.d ? D.h : D.d));
         if (D.act == MOE_BF16) {  // the tensor-core path sums dz's columns per 32-row block in the GEMM epilogue
             const int64_t cs_tc = tc_colsum_part_floats(D.R, (int32_t)D.n, (int32_t)D.h);
@@ -938,16 +941,17 @@ static int32_t backward_impl(const moe_config *cfg, const void *dY, const void *
                                (int32_t)D.n));
     { Carver cv = fresh();
       const void *hid = C.hid;
+      uint32_t *bits = C.relu_bits;
       if (!hid) {  // MOE_FLAG_RECOMPUTE_HID: the forward kept no hidden activations; the first GEMM is run again
-          FfnBwdWs skip(cv, D);  // the expert backward's own scratch comes first, the recomputed tensor behind it
-          (void)skip;
+          FfnBwdWs own(cv, D);  // the expert backward's own scratch comes first, the recomputed tensor behind it
           void *again = nullptr;
-          MOE_TRY(do_expert_ffn(cfg, D, C.xs, C.offsets, W1, b1, W2, b2, nullptr, nullptr, ws, cv, st, true, &again, nullptr, &plan));
+          bits = own.bits;
+          MOE_TRY(do_expert_ffn(cfg, D, C.xs, C.offsets, W1, b1, W2, b2, nullptr, nullptr, ws, cv, st, true, &again, bits, &plan));
           hid = again;
           cv = fresh();
       }
       MOE_TRY(do_expert_ffn_bwd(cfg, D, C.xs, hid, B.dys, C.offsets, W1, W2, B.dxs, dW1, db1, dW2, db2, ws, cv,
-                                st, plan, C.relu_bits)); }
+                                st, plan, bits)); }
     { Carver cv = fresh();
       MOE_TRY(do_gate_bwd(cfg, D, x, Wg, Wnoise, noise, C.clean, C.raw_noise, C.topk_idx, C.gates, C.kth_vals,
                           C.kth_idx, B.dgates, B.dload, dWg, dWnoise, B.dX_gate, ws, cv, st)); }
