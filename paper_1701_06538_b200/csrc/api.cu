@@ -177,7 +177,8 @@ SegmentPlan make_plan(const moe_config *c, const Dims &D, int32_t *ws, bool back
         if (backward && p.bm[0] != COLSUM_ROWS) p.bm[1] = COLSUM_ROWS;
         if (!backward || !tc_wgrad_sorted(*c)) p.sched = nullptr;
     } else {
-        p.bm[0] = 64; p.bm[1] = 32; p.bm[2] = backward ? COLSUM_ROWS : 16;
+        p.bm[0] = 64; p.bm[1] = 32; p.bm[2] = 16;
+        if (backward) p.bm[3] = COLSUM_ROWS;
         p.info = p.sched = nullptr;
     }
     return p;
@@ -448,18 +449,17 @@ int32_t do_expert_ffn(const moe_config *c, const Dims &D, const void *xs, const 
     if (!ready) MOE_TRY(launch_segment_plan(plan, offsets, (int32_t)D.n, D.R, status_word(ws_base), st));
     if (tc_ffn_supported(*c))
         return launch_tc_ffn(*c, xs, offsets, W1, b1, W2, b2, hid, ys, plan, status_word(ws_base), st, first_only, relu_bits);
-    int32_t *scratch = ready ? w.plan : nullptr;  // a backward plan may lack the tile height picked here
     SimtGemm g = base_gemm(D);  // hid = relu(xs.W1 + b1)
     g.A = xs; g.B = W1; g.C = hid; g.bias = b1; g.relu = 1;
     g.sa_i = D.d; g.sa_k = 1; g.sb_k = D.h; g.sb_j = 1; g.sc_i = D.h;
     g.mode = 0; g.offsets = offsets; g.nseg = (int32_t)D.n; g.M = D.R; g.N = D.h; g.K = D.d; g.b_e = D.d * D.h;
-    MOE_TRY(launch_simt_gemm(g, scratch, st, nullptr, &plan));
+    MOE_TRY(launch_simt_gemm(g, nullptr, st, nullptr, &plan));
     if (first_only) return MOE_OK;
     g = base_gemm(D);  // ys = hid.W2 + b2
     g.A = hid; g.B = W2; g.C = ys; g.bias = b2;
     g.sa_i = D.h; g.sa_k = 1; g.sb_k = D.d; g.sb_j = 1; g.sc_i = D.d;
     g.mode = 0; g.offsets = offsets; g.nseg = (int32_t)D.n; g.M = D.R; g.N = D.d; g.K = D.h; g.b_e = D.h * D.d;
-    return launch_simt_gemm(g, scratch, st, nullptr, &plan);
+    return launch_simt_gemm(g, nullptr, st, nullptr, &plan);
 }
 
 int32_t do_losses(const moe_config *c, const Dims &D, const int32_t *topk_idx, const float *gates,

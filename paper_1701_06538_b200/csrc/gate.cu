@@ -28,6 +28,9 @@ int32_t launch_projection(const void *x, int32_t act, int64_t M, int32_t d, int3
     return launch_simt_gemm(g, tile_prefix, st);
 }
 
+// rows that a block of 256 threads takes: a thread per column as far as that goes
+__host__ __device__ __forceinline__ int select_rows_per_block(int32_t n) { return n <= 64 ? 4 : n <= 128 ? 2 : 1; }
+
 // ------------------------------------------------------------------------------------------
 // Noisy logits H = clean + noise * softplus(raw) (Eq. 4), KeepTopK (Eq. 5) and the softmax over
 // the kept entries (Eq. 3). One warp per row. Each lane keeps the k+1 best of its columns in a
@@ -35,7 +38,10 @@ int32_t launch_projection(const void *x, int32_t act, int64_t M, int32_t d, int3
 // over the list heads then produce the global order. Lowest index wins ties everywhere.
 // softplus is evaluated in double and rounded once, H by one fused multiply-add.
 // ------------------------------------------------------------------------------------------
-template <int KL>  // length of the per-lane sorted lists, >= k + 1
+// STAGED (n > 32, all rows): the noisy logits of the block's rows are formed first, one column per thread and step, and parked
+// in shared memory for the row's warp. The softplus in double is a chain of 3000 cycles, and a warp that walks a wide row
+// alone goes through it n / 32 times (1019 rows of 256 columns: 14 us).
+template <int KL, bool STAGED>  // KL: length of the per-lane sorted lists, >= k + 1
 __global__ void __launch_bounds__(256) gate_select_kernel(const float *__restrict__ clean,
                                                           const float *__restrict__ raw,
                                                           const float *__restrict__ noise, int64_t rows, int32_t n,
@@ -47,8 +53,21 @@ __global__ void __launch_bounds__(256) gate_select_kernel(const float *__restric
                                                           const int2 *__restrict__ row_span,
                                                           const int2 *__restrict__ chain_list) {
     wait_previous_kernel();
-    const int lane = threadIdx.x & 31;
-    int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    extern __shared__ float staged[];  // [rows of the block][n]
+    const int lane = threadIdx.x & 31, rpb = STAGED ? select_rows_per_block(n) : blockDim.x >> 5;
+    int64_t row = (int64_t)blockIdx.x * rpb + (threadIdx.x >> 5);
+    auto noisy = [](float c, float r, float e) {
+        const double rd = (double)r;
+        const float sigma = (float)(fmax(rd, 0.0) + log1p(exp(-fabs(rd))));
+        const float v = fmaf(e, sigma, c);
+        return v == v ? v : -CUDART_INF_F;  // a NaN logit ranks last: the selection stays total, indices stay in [0, n)
+    };
+    if (STAGED) {
+        const int64_t first = (int64_t)blockIdx.x * rpb * n, total = min((int64_t)rpb * n, rows * n - first);
+        for (int i = threadIdx.x; i < total; i += 256) staged[i] = noisy(clean[first + i], raw[first + i], noise[first + i]);
+        __syncthreads();
+        if ((int)(threadIdx.x >> 5) >= rpb) return;
+    }
     // row_span (with a row list): {first chain entry, number of candidate columns} of a listed row whose other
     // columns are known to rank below k + 1, so only the candidates are looked at; {., -1}: every column
     int32_t cand_base = 0, cand_total = -1;
@@ -68,10 +87,7 @@ __global__ void __launch_bounds__(256) gate_select_kernel(const float *__restric
     for (int32_t q = lane; q < visits; q += 32) {
         // a candidate's column is the code of its first chain entry (the clean one), modulo the group's block of 2n
         const int32_t j = cand_total >= 0 ? chain_list[cand_base + 2 * q].y % (2 * n) : q;
-        const double rd = (double)r[j];
-        const float sigma = (float)(fmax(rd, 0.0) + log1p(exp(-fabs(rd))));
-        float v = fmaf(e[j], sigma, c[j]);
-        if (!(v == v)) v = -CUDART_INF_F;  // a NaN logit ranks last: the selection stays total, indices stay in [0, n)
+        float v = STAGED ? staged[(threadIdx.x >> 5) * n + j] : noisy(c[j], r[j], e[j]);
         int32_t id = j;
         bool shifting = false;
 #pragma unroll
@@ -129,13 +145,22 @@ int32_t launch_gate_select(const float *clean, const float *raw, const float *no
                            cudaStream_t st, const int32_t *row_list, const int32_t *row_count, const void *row_span,
                            const void *chain_list) {
     if (rows == 0) return MOE_OK;
-    const unsigned grid = (unsigned)cdiv(rows, 8);
-#define MOE_SELECT(KL)                                                                                                 \
-    launch_kernel(gate_select_kernel<KL>, grid, 256, 0, st, clean, raw, noise, rows, n, k, idx, gates, kth_vals, kth_idx, row_list, \
-                                                 row_count, (const int2 *)row_span, (const int2 *)chain_list)
+    const bool stage = n > 32 && !row_list;
+    const int rpb = stage ? select_rows_per_block(n) : 8;
+    const unsigned grid = (unsigned)cdiv(rows, rpb);
+    const size_t sh = stage ? sizeof(float) * rpb * n : 0;  // at most 32 KiB
+#define MOE_SELECT_AS(KL, STAGED)                                                                                        \
+    launch_kernel((gate_select_kernel<KL, STAGED>), grid, 256, sh, st, clean, raw, noise, rows, n, k, idx, gates, kth_vals, \
+                  kth_idx, row_list, row_count, (const int2 *)row_span, (const int2 *)chain_list)
+#define MOE_SELECT(KL)                        \
+    do {                                      \
+        if (stage) MOE_SELECT_AS(KL, true);   \
+        else MOE_SELECT_AS(KL, false);        \
+    } while (0)
     if (k <= 2) MOE_SELECT(3);
     else if (k <= 4) MOE_SELECT(5);
     else MOE_SELECT(MOE_MAX_K + 1);
+#undef MOE_SELECT_AS
 #undef MOE_SELECT
     MOE_LAUNCHED();
     return MOE_OK;

@@ -412,7 +412,7 @@ static int32_t simt_launch(SimtRun &run, int32_t *tile_prefix, cudaStream_t st) 
 // outputs per thread the better, as long as the blocks spread over the chip: 64 x 128 tiles (8 x 8 outputs per thread)
 // from six blocks per SM on (32768 tokens x 512 features x 256 columns: 186 us = 46 TFLOP/s, with 64 x 64 tiles 213);
 // 64 x 64 tiles (8 x 4) from two per SM on (the 16-expert float layer with 4170 rows: 46 us per product, with 64 x 128
-// tiles 58); else 32 x 32 tiles (4 x 4), and for the projection of few tokens 16 x 16 (2 x 2, K blocks of 64), where a
+// tiles 58); else 32 x 32 tiles (4 x 4), and where even those leave SMs idle 16 x 16 (2 x 2, K blocks of 64): there a
 // block's time is the latency of one chain and its loads (24 tokens x 512 features x 64 columns: 9 us; one 128 x 64
 // tile: 40).
 template <typename TA, typename TB, typename TC, bool AK, bool BJ>
@@ -428,9 +428,8 @@ static int32_t simt_pick_tile(SimtRun &run, bool vec, int32_t *tile_prefix, cuda
         return simt_launch<TA, TB, TC, true, AK, BJ, 64, 128, 8, 8, 16>(run, tile_prefix, st);
     if (blocks(64, 64) >= 2 * 148 && !short_rows && !(run.part && g.N <= 32))
         return simt_launch<TA, TB, TC, true, AK, BJ, 64, 64, 8, 4, 16>(run, tile_prefix, st);
-    if (!AK || !BJ || blocks(32, 32) >= 148) return simt_launch<TA, TB, TC, true, AK, BJ, 32, 32, 4, 4, 32>(run, tile_prefix, st);
-    if constexpr (AK && BJ) return simt_launch<TA, TB, TC, true, AK, BJ, 16, 16, 2, 2, 64>(run, tile_prefix, st);
-    return MOE_OK;
+    if (blocks(32, 32) >= 148) return simt_launch<TA, TB, TC, true, AK, BJ, 32, 32, 4, 4, 32>(run, tile_prefix, st);
+    return simt_launch<TA, TB, TC, true, AK, BJ, 16, 16, 2, 2, 64>(run, tile_prefix, st);
 }
 
 // part: simt_wgrad_splits(M, N, nseg, rows) * nseg * M * N floats (mode 1, float results), or nullptr: no slices

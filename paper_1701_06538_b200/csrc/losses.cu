@@ -10,7 +10,8 @@ namespace moe {
 
 constexpr int LCHUNKS_MAX = 148 * 4;
 
-static inline int32_t level_chunks(int64_t rows) { return (int32_t)imin(cdiv(rows, 32), LCHUNKS_MAX); }
+// a row per warp until the chip is full: the normal-CDF evaluations of a row are one long latency chain per lane
+static inline int32_t level_chunks(int64_t rows) { return (int32_t)imin(cdiv(rows, 8), LCHUNKS_MAX); }
 int64_t losses_ws_floats(int64_t rows, int32_t n) { return 2 * (int64_t)level_chunks(rows) * n + 64; }
 
 __device__ __forceinline__ float softplus_f(float r) { return fmaxf(r, 0.0f) + log1pf(expf(-fabsf(r))); }
@@ -142,7 +143,7 @@ __global__ void __launch_bounds__(256) level_reduce_kernel(const float *__restri
                                                            const LossFinal fin, int32_t *ticket) {
     wait_previous_kernel();
     __shared__ double red[2][8][32];
-    __shared__ double sh[256];
+    __shared__ double sh[32];
     __shared__ int last;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int32_t j = blockIdx.x * 32 + lane;
@@ -219,7 +220,7 @@ int32_t launch_level_sums(const int32_t *idx, const float *gates, const float *c
 __global__ void __launch_bounds__(256) cv2_kernel(const float *importance, int32_t n_imp, const float *load,
                                                   int32_t n_load, float w_imp, float w_load, float *losses, const LossOut copy) {
     wait_previous_kernel();
-    __shared__ double sh[256];
+    __shared__ double sh[32];
     cv2_block(importance, n_imp, load, n_load, w_imp, w_load, losses, copy.losses, sh);
     if (copy.importance)
         for (int32_t i = threadIdx.x; i < copy.n; i += 256) copy.importance[i] = importance[i];
@@ -239,7 +240,7 @@ int32_t launch_cv2(const float *importance, int32_t n_imp, const float *load, in
 struct Cv2Pair { Cv2Job job[2]; };
 __global__ void __launch_bounds__(1024) cv2_grads_kernel(const Cv2Pair pair) {  // one block per vector
     wait_previous_kernel();
-    __shared__ double sh[1024];
+    __shared__ double sh[32];
     cv2_grad_block(pair.job[blockIdx.x], sh);
 }
 

@@ -168,17 +168,17 @@ int32_t launch_dispatch_bwd(const void *dxs, int32_t act, const int32_t *inv_per
 int32_t launch_tile_prefix(const int32_t *offsets, int32_t n, int32_t bm, int32_t *tile_prefix, cudaStream_t st);
 
 // ----------------------------------------------------------------------------- per-call segment plan (plan.cu)
-constexpr int PLAN_COUNTERS = 8, PLAN_MAX_SORTED = 8192;
+constexpr int PLAN_HEIGHTS = 4, PLAN_COUNTERS = 8, PLAN_MAX_SORTED = 8192;
 // run-time tile counters of a plan, by the GEMM that uses them
 enum PlanCounter { PLAN_ROWS_A = 0, PLAN_ROWS_B = 1, PLAN_WGRAD_A = 2, PLAN_WGRAD_B = 3, PLAN_ROWS_AGAIN = 4 };
 struct SegmentPlan {
-    int32_t *prefix[3];  // [n + 1] number of tiles of bm[i] rows in the segments before
-    int32_t bm[3];       // 0: prefix not made
+    int32_t *prefix[PLAN_HEIGHTS];  // [n + 1] number of tiles of bm[i] rows in the segments before
+    int32_t bm[PLAN_HEIGHTS];       // 0: prefix not made
     int4 *info;          // a record per tile of prefix[0], or nullptr: {segment or -1, first row, segment end, 0}
     int4 *sched;         // {segment, first row, end row, 0} in descending size, or nullptr
     int32_t *counters;   // [PLAN_COUNTERS], zeroed
     const int32_t *prefix_of(int32_t height) const {
-        for (int i = 0; i < 3; ++i)
+        for (int i = 0; i < PLAN_HEIGHTS; ++i)
             if (bm[i] == height) return prefix[i];
         return nullptr;
     }

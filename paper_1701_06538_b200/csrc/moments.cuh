@@ -8,30 +8,29 @@ namespace moe {
 
 struct Moments { double mu, var; };
 
-// sh: blockDim.x doubles (a power of two)
+// sum over the block (whole warps) of one value per thread, returned to every thread; sh: 32 doubles
+__device__ __forceinline__ double block_sum(double v, double *sh) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    __syncthreads();  // sh may still be read from an earlier call
+    if (lane == 0) sh[w] = v;
+    __syncthreads();
+    v = lane < (int)(blockDim.x >> 5) ? sh[lane] : 0.0;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    return v;
+}
+
 __device__ __forceinline__ Moments block_moments(const float *v, int32_t m, double *sh) {
     double s = 0.0;
     for (int32_t i = threadIdx.x; i < m; i += blockDim.x) s += (double)__ldcg(v + i);
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    for (int off = blockDim.x / 2; off > 0; off >>= 1) {
-        if (threadIdx.x < off) sh[threadIdx.x] += sh[threadIdx.x + off];
-        __syncthreads();
-    }
-    const double mu = sh[0] / m;
-    __syncthreads();
+    const double mu = block_sum(s, sh) / m;
     double q = 0.0;
     for (int32_t i = threadIdx.x; i < m; i += blockDim.x) { double dv = (double)__ldcg(v + i) - mu; q += dv * dv; }
-    sh[threadIdx.x] = q;
-    __syncthreads();
-    for (int off = blockDim.x / 2; off > 0; off >>= 1) {
-        if (threadIdx.x < off) sh[threadIdx.x] += sh[threadIdx.x + off];
-        __syncthreads();
-    }
     Moments r;
     r.mu = mu;
-    r.var = sh[0] / m;
-    __syncthreads();
+    r.var = block_sum(q, sh) / m;
     return r;
 }
 

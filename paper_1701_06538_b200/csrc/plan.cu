@@ -1,5 +1,5 @@
 // What the kernels of one call need to know about the expert segments, worked out once per call by one launch: tile prefixes
-// for up to three tile heights, the tile records and the run-time counters of the tensor-core GEMMs, the segments in
+// for up to four tile heights, the tile records and the run-time counters of the tensor-core GEMMs, the segments in
 // descending size (weight gradients hand out their longest tiles first), and in the backward pass the gradients of the two
 // balancing losses with respect to Importance and Load. Each is the work of one block; as launches of their own they were
 // nine of the 23 of a small backward pass, 2 to 4 us each.
@@ -49,16 +49,16 @@ __device__ int32_t tile_prefix_block(const int32_t *offsets, int32_t n, int32_t 
     return carry;
 }
 
-// blocks 0..2: tile prefixes (0: the records, the counters and the status word as well); 3, 4: loss gradients; from 5 on:
+// blocks 0..3: tile prefixes (0: the records, the counters and the status word as well); 4, 5: loss gradients; from 6 on:
 // 1024 segments each of the order by size
 __global__ void __launch_bounds__(1024) segment_plan_kernel(const __grid_constant__ PlanArgs a) {
     wait_previous_kernel();
     __shared__ int32_t sh[32];
-    __shared__ double moments[1024];
+    __shared__ double moments[32];
     __shared__ int32_t cnt[PLAN_MAX_SORTED];
     const int32_t *offsets = a.offsets;
     const int32_t n = a.n;
-    if (blockIdx.x < 3) {
+    if (blockIdx.x < PLAN_HEIGHTS) {
         const int which = blockIdx.x;
         if (which == 0) {
             if (threadIdx.x < PLAN_COUNTERS && a.plan.counters) a.plan.counters[threadIdx.x] = 0;
@@ -78,13 +78,13 @@ __global__ void __launch_bounds__(1024) segment_plan_kernel(const __grid_constan
             }
             a.plan.info[mt] = make_int4(lo, offsets[lo] + (mt - prefix[lo]) * bm, offsets[lo + 1], 0);
         }
-    } else if (blockIdx.x < 5) {
-        const Cv2Job &job = a.cv2[blockIdx.x - 3];
+    } else if (blockIdx.x < PLAN_HEIGHTS + 2) {
+        const Cv2Job &job = a.cv2[blockIdx.x - PLAN_HEIGHTS];
         if (job.v) cv2_grad_block(job, moments);
     } else if (a.plan.sched) {  // rank by descending size, equal sizes by index
         for (int32_t e = threadIdx.x; e < n; e += 1024) cnt[e] = offsets[e + 1] - offsets[e];
         __syncthreads();
-        const int32_t e = (blockIdx.x - 5) * 1024 + threadIdx.x;
+        const int32_t e = (blockIdx.x - PLAN_HEIGHTS - 2) * 1024 + threadIdx.x;
         if (e >= n) return;
         const int32_t mine = cnt[e];
         int32_t rank = 0;
@@ -96,12 +96,12 @@ __global__ void __launch_bounds__(1024) segment_plan_kernel(const __grid_constan
 }  // namespace
 
 static int64_t align4(int64_t v) { return (v + 3) & ~(int64_t)3; }
-int64_t plan_ints(int64_t R, int64_t n) { return 3 * align4(n + 1) + 4 * (cdiv(R, 128) + n + 1) + 4 * n + PLAN_COUNTERS; }
+int64_t plan_ints(int64_t R, int64_t n) { return PLAN_HEIGHTS * align4(n + 1) + 4 * (cdiv(R, 128) + n + 1) + 4 * n + PLAN_COUNTERS; }
 
 SegmentPlan plan_at(int32_t *ws, int64_t R, int64_t n) {
     SegmentPlan p;
-    for (int i = 0; i < 3; ++i) { p.prefix[i] = ws + i * align4(n + 1); p.bm[i] = 0; }
-    p.info = reinterpret_cast<int4 *>(ws + 3 * align4(n + 1));
+    for (int i = 0; i < PLAN_HEIGHTS; ++i) { p.prefix[i] = ws + i * align4(n + 1); p.bm[i] = 0; }
+    p.info = reinterpret_cast<int4 *>(ws + PLAN_HEIGHTS * align4(n + 1));
     p.sched = p.info + cdiv(R, 128) + n + 1;
     p.counters = reinterpret_cast<int32_t *>(p.sched + n);
     return p;
@@ -114,7 +114,7 @@ int32_t launch_segment_plan(const SegmentPlan &plan, const int32_t *offsets, int
     a.max_m = plan.info && plan.bm[0] ? (int32_t)(cdiv(R, plan.bm[0]) + n) : 0;
     a.cv2[0] = jobs ? jobs[0] : Cv2Job{nullptr, 0, 0.0f, nullptr};
     a.cv2[1] = jobs ? jobs[1] : Cv2Job{nullptr, 0, 0.0f, nullptr};
-    const unsigned blocks = plan.sched ? 5u + (unsigned)cdiv(n, 1024) : jobs ? 5u : 3u;
+    const unsigned blocks = PLAN_HEIGHTS + (plan.sched ? 2u + (unsigned)cdiv(n, 1024) : jobs ? 2u : 0u);
     launch_kernel(segment_plan_kernel, blocks, 1024, 0, st, a);
     MOE_LAUNCHED();
     return MOE_OK;
