@@ -1612,38 +1612,57 @@ static int32_t launch_tile_table(const int32_t *offsets, int32_t nseg, int32_t t
 // A thread block takes 64 columns of one segment: 16 column lanes (four adjacent columns each, 16-byte loads) by 16 row
 // lanes; row lane q takes the blocks b = b0 + q, b0 + q + 16, ... (eight loads in flight: the largest expert of a skewed
 // batch has over a thousand blocks and sets this kernel's duration) and the 16 sums are added in lane order: the
-// result does not depend on timing.
+// result does not depend on timing. A block takes `cols` columns: 64, or, where a segment has about one tile (thousands of
+// experts), 1024: a segment of at most 16 blocks is then added by one thread per four columns, in the same order.
 __global__ void __launch_bounds__(256) colsum_blocks_final_kernel(const float *__restrict__ part, int32_t N,
                                                                   const int32_t *__restrict__ tile_prefix, int32_t G,
-                                                                  bf16 *__restrict__ out) {
+                                                                  int32_t cols, bf16 *__restrict__ out) {
     wait_previous_kernel();
     __shared__ float4 sh[16][16];
     const int32_t e = blockIdx.x, q = threadIdx.x >> 4, cl = threadIdx.x & 15;
-    const int32_t j = blockIdx.y * 64 + cl * 4;  // N is a multiple of 64
     const int32_t b0 = tile_prefix[e] * G, b1 = tile_prefix[e + 1] * G;
-    float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    int32_t b = b0 + q;
-    for (; b + 16 * 7 < b1; b += 16 * 8) {
-        float4 v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = *reinterpret_cast<const float4 *>(part + (int64_t)(b + 16 * u) * N + j);
-#pragma unroll
-        for (int u = 0; u < 8; ++u) { s.x += v[u].x; s.y += v[u].y; s.z += v[u].z; s.w += v[u].w; }
-    }
-    for (; b < b1; b += 16) {
-        const float4 v = *reinterpret_cast<const float4 *>(part + (int64_t)b * N + j);
-        s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
-    }
-    sh[q][cl] = s;
-    __syncthreads();
-    if (q == 0) {
-        float4 t = sh[0][cl];
-#pragma unroll
-        for (int u = 1; u < 16; ++u) { t.x += sh[u][cl].x; t.y += sh[u][cl].y; t.z += sh[u][cl].z; t.w += sh[u][cl].w; }
-        __nv_bfloat162 o0 = __floats2bfloat162_rn(t.x, t.y), o1 = __floats2bfloat162_rn(t.z, t.w);
+    auto store = [&](int32_t j, const float4 &t) {
+        const __nv_bfloat162 o0 = __floats2bfloat162_rn(t.x, t.y), o1 = __floats2bfloat162_rn(t.z, t.w);
         uint2 pk;
-        pk.x = *reinterpret_cast<uint32_t *>(&o0); pk.y = *reinterpret_cast<uint32_t *>(&o1);
+        pk.x = *reinterpret_cast<const uint32_t *>(&o0); pk.y = *reinterpret_cast<const uint32_t *>(&o1);
         *reinterpret_cast<uint2 *>(out + (int64_t)e * N + j) = pk;
+    };
+    if (cols > 64 && b1 - b0 <= 16) {
+        const int32_t j = blockIdx.y * cols + threadIdx.x * 4;
+        if (j >= N) return;
+        float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll 4
+        for (int32_t b = b0; b < b1; ++b) {
+            const float4 v = *reinterpret_cast<const float4 *>(part + (int64_t)b * N + j);
+            s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+        }
+        store(j, s);
+        return;
+    }
+    for (int32_t j0 = blockIdx.y * cols; j0 < N && j0 < (int32_t)(blockIdx.y + 1) * cols; j0 += 64) {  // N is a multiple of 64
+        const int32_t j = j0 + cl * 4;
+        float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        int32_t b = b0 + q;
+        for (; b + 16 * 7 < b1; b += 16 * 8) {
+            float4 v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = *reinterpret_cast<const float4 *>(part + (int64_t)(b + 16 * u) * N + j);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) { s.x += v[u].x; s.y += v[u].y; s.z += v[u].z; s.w += v[u].w; }
+        }
+        for (; b < b1; b += 16) {
+            const float4 v = *reinterpret_cast<const float4 *>(part + (int64_t)b * N + j);
+            s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+        }
+        __syncthreads();  // sh may still be read for the columns before
+        sh[q][cl] = s;
+        __syncthreads();
+        if (q == 0) {
+            float4 t = sh[0][cl];
+#pragma unroll
+            for (int u = 1; u < 16; ++u) { t.x += sh[u][cl].x; t.y += sh[u][cl].y; t.z += sh[u][cl].z; t.w += sh[u][cl].w; }
+            store(j, t);
+        }
     }
 }
 
@@ -1662,8 +1681,9 @@ int32_t tc_row_gemm(const void *A, const void *W, bool transposed, const int32_t
     }
     auto finish = [&](int32_t rc, int32_t G) -> int32_t {
         if (rc != MOE_OK || !colsum_out) return rc;
-        launch_kernel(colsum_blocks_final_kernel, dim3((unsigned)nseg, (unsigned)cdiv(N, 64)), 256, 0, st, colsum_part, N, plan.prefix[0], G,
-                                                                                                   (bf16 *)colsum_out);
+        const int32_t cols = nseg >= 128 && R <= 128 * (int64_t)nseg ? 1024 : 64;
+        launch_kernel(colsum_blocks_final_kernel, dim3((unsigned)nseg, (unsigned)cdiv(N, cols)), 256, 0, st, colsum_part, N,
+                      plan.prefix[0], G, cols, (bf16 *)colsum_out);
         MOE_LAUNCHED();
         return MOE_OK;
     };

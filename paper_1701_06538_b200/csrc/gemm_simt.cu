@@ -481,12 +481,12 @@ int64_t colsum_ws_floats(int64_t R, int32_t n, int32_t N) { return (cdiv(R, CS_R
 
 // One block per 128-row tile and per slab of 32 * V columns (V = elements of a 16-byte vector): lane l owns V adjacent
 // columns, warp w the tile's rows w, w + 8, ..., read with 16-byte loads, four rows in flight; the eight warps' sums are
-// added in warp order.
+// added in warp order. A segment of one tile is finished here.
 template <typename XT>
 __global__ void __launch_bounds__(256) colsum_partial_kernel(const XT *__restrict__ in,
                                                              const int32_t *__restrict__ offsets, int32_t nseg,
                                                              int32_t N, const int32_t *__restrict__ tile_prefix,
-                                                             float *__restrict__ part) {
+                                                             float *__restrict__ part, XT *__restrict__ out) {
     wait_previous_kernel();
     constexpr int V = 16 / sizeof(XT);
     __shared__ float sh[8][32 * V];
@@ -533,41 +533,47 @@ __global__ void __launch_bounds__(256) colsum_partial_kernel(const XT *__restric
             float t = sh[0][c];
 #pragma unroll
             for (int q = 1; q < 8; ++q) t += sh[q][c];
-            part[(int64_t)b * N + col] = t;
+            if (tile_prefix[lo + 1] - tile_prefix[lo] == 1) out[(int64_t)lo * N + col] = from_f32<XT>(t);
+            else part[(int64_t)b * N + col] = t;
         }
     }
 }
 
-// Sum of a segment's tile sums: a block takes 32 columns, its eight warps the tiles b0 + w, b0 + w + 8, ... (eight loads in
+// Sum of a segment's tile sums (a segment of one tile is complete already, which with thousands of experts most are: a
+// block then looks at 256 columns, 32 at a time): a block takes 32 columns, its eight warps the tiles b0 + w, b0 + w + 8, ... (eight loads in
 // flight: the largest expert of a skewed batch has hundreds of tiles), the eight sums are added in warp order.
 template <typename XT>
 __global__ void __launch_bounds__(256) colsum_final_kernel(const float *__restrict__ part, int32_t N,
                                                            const int32_t *__restrict__ tile_prefix,
-                                                           XT *__restrict__ out) {
+                                                           int32_t cols, XT *__restrict__ out) {
     wait_previous_kernel();
     __shared__ float sh[8][32];
     const int32_t e = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int32_t j = blockIdx.y * 32 + lane;
-    const int32_t b1 = tile_prefix[e + 1];
-    float s = 0.0f;
-    if (j < N) {
-        int32_t b = tile_prefix[e] + w;
-        for (; b + 8 * 7 < b1; b += 64) {
-            float v[8];
+    const int32_t b0 = tile_prefix[e], b1 = tile_prefix[e + 1];
+    if (b1 - b0 == 1) return;
+    for (int32_t j0 = blockIdx.y * cols; j0 < N && j0 < (int32_t)(blockIdx.y + 1) * cols; j0 += 32) {
+        const int32_t j = j0 + lane;
+        float s = 0.0f;
+        if (j < N) {
+            int32_t b = b0 + w;
+            for (; b + 8 * 7 < b1; b += 64) {
+                float v[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = part[(int64_t)(b + 8 * u) * N + j];
+                for (int u = 0; u < 8; ++u) v[u] = part[(int64_t)(b + 8 * u) * N + j];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) s += v[u];
+                for (int u = 0; u < 8; ++u) s += v[u];
+            }
+            for (; b < b1; b += 8) s += part[(int64_t)b * N + j];
         }
-        for (; b < b1; b += 8) s += part[(int64_t)b * N + j];
-    }
-    sh[w][lane] = s;
-    __syncthreads();
-    if (w == 0 && j < N) {
-        float t = sh[0][lane];
+        __syncthreads();  // sh may still be read for the columns before
+        sh[w][lane] = s;
+        __syncthreads();
+        if (w == 0 && j < N) {
+            float t = sh[0][lane];
 #pragma unroll
-        for (int u = 1; u < 8; ++u) t += sh[u][lane];
-        out[(int64_t)e * N + j] = from_f32<XT>(t);
+            for (int u = 1; u < 8; ++u) t += sh[u][lane];
+            out[(int64_t)e * N + j] = from_f32<XT>(t);
+        }
     }
 }
 
@@ -575,15 +581,16 @@ int32_t launch_segment_colsum(const void *in, int32_t act, const int32_t *offset
                               int32_t N, void *out, float *scratch, const int32_t *tile_prefix, cudaStream_t st) {
     const int vcols = act == MOE_BF16 ? 256 : 128;  // columns per block of the partial sums: 32 lanes x one 16-byte vector
     dim3 g1((unsigned)(cdiv(R, CS_ROWS) + nseg), (unsigned)cdiv(N, vcols));
-    dim3 g2((unsigned)nseg, (unsigned)cdiv(N, 32));
+    const int32_t cols = nseg >= 1024 ? 256 : 32;  // of a block of the final sums
+    dim3 g2((unsigned)nseg, (unsigned)cdiv(N, cols));
     if (act == MOE_BF16) {
-        launch_kernel(colsum_partial_kernel<bf16>, g1, 256, 0, st, (const bf16 *)in, offsets, nseg, N, tile_prefix, scratch);
+        launch_kernel(colsum_partial_kernel<bf16>, g1, 256, 0, st, (const bf16 *)in, offsets, nseg, N, tile_prefix, scratch, (bf16 *)out);
         MOE_LAUNCHED();
-        launch_kernel(colsum_final_kernel<bf16>, g2, 256, 0, st, scratch, N, tile_prefix, (bf16 *)out);
+        launch_kernel(colsum_final_kernel<bf16>, g2, 256, 0, st, scratch, N, tile_prefix, cols, (bf16 *)out);
     } else {
-        launch_kernel(colsum_partial_kernel<float>, g1, 256, 0, st, (const float *)in, offsets, nseg, N, tile_prefix, scratch);
+        launch_kernel(colsum_partial_kernel<float>, g1, 256, 0, st, (const float *)in, offsets, nseg, N, tile_prefix, scratch, (float *)out);
         MOE_LAUNCHED();
-        launch_kernel(colsum_final_kernel<float>, g2, 256, 0, st, scratch, N, tile_prefix, (float *)out);
+        launch_kernel(colsum_final_kernel<float>, g2, 256, 0, st, scratch, N, tile_prefix, cols, (float *)out);
     }
     MOE_LAUNCHED();
     return MOE_OK;

@@ -216,23 +216,26 @@ int32_t launch_level_sums(const int32_t *idx, const float *gates, const float *c
     return MOE_OK;
 }
 
-// the losses of vectors that are complete already, and the copies of everything
+// the losses of vectors that are complete already (block 0), and the copies of everything (the other blocks)
 __global__ void __launch_bounds__(256) cv2_kernel(const float *importance, int32_t n_imp, const float *load,
                                                   int32_t n_load, float w_imp, float w_load, float *losses, const LossOut copy) {
     wait_previous_kernel();
     __shared__ double sh[32];
-    cv2_block(importance, n_imp, load, n_load, w_imp, w_load, losses, copy.losses, sh);
-    if (copy.importance)
-        for (int32_t i = threadIdx.x; i < copy.n; i += 256) copy.importance[i] = importance[i];
-    if (copy.counts)
-        for (int32_t i = threadIdx.x; i < copy.n; i += 256) copy.counts[i] = copy.counts_src[i];
-    if (copy.load)
-        for (int32_t i = threadIdx.x; i < copy.n_load; i += 256) copy.load[i] = load[i];
+    if (blockIdx.x == 0) {
+        cv2_block(importance, n_imp, load, n_load, w_imp, w_load, losses, copy.losses, sh);
+        return;
+    }
+    const int32_t i = (blockIdx.x - 1) * 256 + threadIdx.x;
+    if (i < copy.n) {
+        if (copy.importance) copy.importance[i] = importance[i];
+        if (copy.counts) copy.counts[i] = copy.counts_src[i];
+    }
+    if (i < copy.n_load && copy.load) copy.load[i] = load[i];
 }
 
 int32_t launch_cv2(const float *importance, int32_t n_imp, const float *load, int32_t n_load, float w_imp,
                    float w_load, float *losses, cudaStream_t st, const LossOut &copy) {
-    launch_kernel(cv2_kernel, 1, 256, 0, st, importance, n_imp, load, n_load, w_imp, w_load, losses, copy);
+    launch_kernel(cv2_kernel, 1 + (unsigned)cdiv(copy.n > copy.n_load ? copy.n : copy.n_load, 256), 256, 0, st, importance, n_imp, load, n_load, w_imp, w_load, losses, copy);
     MOE_LAUNCHED();
     return MOE_OK;
 }
