@@ -436,17 +436,18 @@ SimtGemm base_gemm(const Dims &D) {
 
 // hid == nullptr (only with MOE_FLAG_RECOMPUTE_HID): the hidden activations stay in the workspace.
 // first_only: only hid = relu(xs.W1 + b1) is computed (ys is not touched). ready: a plan made already (with the row tiles
-// of the forward pass); else it is made here, which also clears the status word.
+// of the forward pass); else it is made here. clear: the status word if this is a call of its own, nullptr inside a fused
+// call: its first kernel has cleared the word, and what the gate's products reported since stays.
 int32_t do_expert_ffn(const moe_config *c, const Dims &D, const void *xs, const int32_t *offsets, const void *W1,
                       const void *b1, const void *W2, const void *b2, void *hid, void *ys, void *ws_base,
-                      Carver &cv, cudaStream_t st, bool first_only = false, void **hid_used = nullptr,
+                      Carver &cv, cudaStream_t st, int32_t *clear, bool first_only = false, void **hid_used = nullptr,
                       uint32_t *relu_bits = nullptr, const SegmentPlan *ready = nullptr) {
     FfnWs w(cv, D);
     if (!hid) hid = w.hid;
     if (!hid) return MOE_ERR_INVALID_ARG;
     if (hid_used) *hid_used = hid;
     const SegmentPlan plan = ready ? *ready : make_plan(c, D, w.plan, false);
-    if (!ready) MOE_TRY(launch_segment_plan(plan, offsets, (int32_t)D.n, D.R, status_word(ws_base), st));
+    if (!ready) MOE_TRY(launch_segment_plan(plan, offsets, (int32_t)D.n, D.R, clear, st));
     if (tc_ffn_supported(*c))
         return launch_tc_ffn(*c, xs, offsets, W1, b1, W2, b2, hid, ys, plan, status_word(ws_base), st, first_only, relu_bits);
     SimtGemm g = base_gemm(D);  // hid = relu(xs.W1 + b1)
@@ -771,7 +772,7 @@ int32_t moe_expert_ffn(const moe_config *cfg, const void *xs, const int32_t *off
     const Dims D = dims_of(cfg);
     Carver cv(ws);
     cv.take_bytes(kWsHeader);
-    return do_expert_ffn(cfg, D, xs, offsets, W1, b1, W2, b2, hid, ys, ws, cv, as_stream(stream));
+    return do_expert_ffn(cfg, D, xs, offsets, W1, b1, W2, b2, hid, ys, ws, cv, as_stream(stream), status_word(ws));
 }
 
 int32_t moe_expert_ffn_bits(const moe_config *cfg, const void *xs, const int32_t *offsets, const void *W1,
@@ -783,7 +784,8 @@ int32_t moe_expert_ffn_bits(const moe_config *cfg, const void *xs, const int32_t
     const Dims D = dims_of(cfg);
     Carver cv(ws);
     cv.take_bytes(kWsHeader);
-    return do_expert_ffn(cfg, D, xs, offsets, W1, b1, W2, b2, hid, ys, ws, cv, as_stream(stream), false, nullptr, relu_bits);
+    return do_expert_ffn(cfg, D, xs, offsets, W1, b1, W2, b2, hid, ys, ws, cv, as_stream(stream), status_word(ws), false, nullptr,
+                         relu_bits);
 }
 
 int32_t moe_expert_ffn_bwd_bits(const moe_config *cfg, const void *xs, const void *hid, const uint32_t *relu_bits,
@@ -887,7 +889,7 @@ static int32_t forward_impl(const moe_config *cfg, const void *x, const float *W
     { Carver cv = fresh();
       MOE_TRY(do_dispatch(D, x, C.topk_idx, C.xs, C.perm, C.inv_perm, C.counts, C.offsets, cv, st)); }
     { Carver cv = fresh();
-      MOE_TRY(do_expert_ffn(cfg, D, C.xs, C.offsets, W1, b1, W2, b2, C.hid, C.ys, ws, cv, st, false, nullptr,
+      MOE_TRY(do_expert_ffn(cfg, D, C.xs, C.offsets, W1, b1, W2, b2, C.hid, C.ys, ws, cv, st, nullptr, false, nullptr,
                             C.relu_bits)); }  // C.hid null: stays in ws
     MOE_TRY(launch_combine(C.ys, D.act, C.gates, C.inv_perm, D.T, (int32_t)D.k, (int32_t)D.d, y, st,
                            keep_bits ? x : nullptr, keep_bits, keep_bits ? 1.0f / (1.0f - drop_prob) : 1.0f));
@@ -946,7 +948,8 @@ static int32_t backward_impl(const moe_config *cfg, const void *dY, const void *
           FfnBwdWs own(cv, D);  // the expert backward's own scratch comes first, the recomputed tensor behind it
           void *again = nullptr;
           bits = own.bits;
-          MOE_TRY(do_expert_ffn(cfg, D, C.xs, C.offsets, W1, b1, W2, b2, nullptr, nullptr, ws, cv, st, true, &again, bits, &plan));
+          MOE_TRY(do_expert_ffn(cfg, D, C.xs, C.offsets, W1, b1, W2, b2, nullptr, nullptr, ws, cv, st, nullptr, true, &again, bits,
+                                &plan));
           hid = again;
           cv = fresh();
       }
