@@ -56,11 +56,11 @@ struct SimtRun {
     float *part;         // splits > 1: [splits][nseg][M][N] partial results instead of C
 };
 
-// AK: A(i, k) is contiguous along k (else along i); BJ: B(k, j) is contiguous along j (else along k). VEC: quads of A and B can
+// AK: A(i, k) is contiguous along k (else along i); BJ: B(k, j) is contiguous along j (else along k). QA4, QB4: quads of A / B can
 // be loaded at once (extents, strides, addresses and the border between two concatenated matrices are multiples of four
 // elements). Their loads are not guarded by branches: a quad outside the operand reads the operand's first elements
 // instead and counts as zero.
-template <typename TA, typename TB, typename TC, bool VEC, bool AK, bool BJ, int BM, int BN, int TM, int TN, int BK>
+template <typename TA, typename TB, typename TC, bool QA4, bool QB4, bool AK, bool BJ, int BM, int BN, int TM, int TN, int BK>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN), TM * TN >= 64 ? 3 : TM * TN >= 32 ? 4 : 8) simt_gemm_kernel(const __grid_constant__ SimtRun run) {
     wait_previous_kernel();
     constexpr int NTX = BN / TN, NTY = BM / TM, NT = NTX * NTY;
@@ -68,6 +68,11 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), TM * TN >= 64 ? 3 : TM 
     constexpr int QA = BM * BK / 4 / NT, QB = BN * BK / 4 / NT;  // quads a thread stages per K block
     constexpr int VA = TM < 4 ? TM : 4, VB = TN < 4 ? TN : 4;    // rows / columns per shared-memory read
     static_assert(QA * NT * 4 == BM * BK && QB * NT * 4 == BN * BK, "whole quads per thread");
+    // A projection onto weights of any width: a thread loads one column of B element by element, so that a warp's loads are
+    // adjacent and the choice between the two matrices is made once. (As guarded quads, four elements apart between the
+    // lanes, 32768 tokens x 512 features x 500 columns took 950 us, this way 400.)
+    constexpr bool COL_B = !QB4 && AK && BJ;
+    static_assert(!COL_B || NT % BN == 0, "a thread's column");
     static_assert(NT % (BK / 4) == 0 && NT % (BM / 4) == 0 && NT % (BN / 4) == 0, "a thread's quads are a fixed step apart");
     __shared__ __align__(16) float As[2][BK * LDA];
     __shared__ __align__(16) float Bs[2][BK * LDB];
@@ -149,7 +154,12 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), TM * TN >= 64 ? 3 : TM 
 
     Quad<TA> ra[QA];
     Quad<TB> rb[QB];
-    uint32_t live_a = 0u, live_b = 0u;  // VEC: which quads lie inside the operand
+    constexpr int COL_STEP = NT / BN, COL_N = COL_B ? 4 * QB : 1;  // COL_B: rows kcol, kcol + COL_STEP, ... of column jcol
+    const int jcol = tid % BN, kcol = tid / BN;
+    const TB *pcol = nullptr;
+    if (COL_B) pcol = (B2 && n0 + jcol >= g.b_split ? B2 + (n0 + jcol - g.b_split) : B + n0 + jcol) + (kbeg + kcol) * g.sb_k;
+    TB ecol[COL_N];
+    uint32_t live_a = 0u, live_b = 0u;  // QA4 / QB4: which quads lie inside the operand
     // rows gathered along the contraction index: the row numbers of the next K block, fetched one block ahead
     int32_t ga[QA], gb[QB];
     auto fetch_rows = [&](int k0) {
@@ -169,7 +179,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), TM * TN >= 64 ? 3 : TM 
             const int k = k0 + ka(q);
             const bool live = ia(q) < rows_valid && k < klen;
             const TA *src = gather_a ? pa[q] + (int64_t)(ga[q] / g.a_row_div) * g.sa_k : pa[q];
-            if constexpr (VEC) {
+            if constexpr (QA4) {
                 ra[q].load(live ? src : A);
                 live_a |= (uint32_t)live << q;
             } else {
@@ -182,12 +192,19 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), TM * TN >= 64 ? 3 : TM 
             if (AK) pa[q] += BK;
             else if (!gather_a) pa[q] += BK * g.sa_k;
         }
+        if constexpr (COL_B) {  // (mode 0: no rows to fetch)
+#pragma unroll
+            for (int q = 0; q < COL_N; ++q)
+                ecol[q] = jcol < cols_valid && k0 + kcol + q * COL_STEP < klen ? pcol[q * COL_STEP * g.sb_k] : from_f32<TB>(0.0f);
+            pcol += BK * g.sb_k;
+            return;
+        }
 #pragma unroll
         for (int q = 0; q < QB; ++q) {
             const int k = k0 + kb(q);
             const bool live = jb(q) < cols_valid && k < klen;
             const TB *src = gather_b ? pb[q] + (int64_t)gb[q] * g.sb_k : pb[q];
-            if constexpr (VEC) {
+            if constexpr (QB4) {
                 if (!BJ && k >= b_switch) src += to_b2;
                 rb[q].load(live ? src : B);
                 live_b |= (uint32_t)live << q;
@@ -214,14 +231,19 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), TM * TN >= 64 ? 3 : TM 
         const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
         for (int q = 0; q < QA; ++q) {
-            const float4 v = !VEC || ((live_a >> q) & 1u) ? ra[q].get() : zero;
+            const float4 v = !QA4 || ((live_a >> q) & 1u) ? ra[q].get() : zero;
             float *dst = &As[buf][ka(q) * LDA + ia(q)];
             if (AK) { dst[0] = v.x; dst[LDA] = v.y; dst[2 * LDA] = v.z; dst[3 * LDA] = v.w; }
             else *reinterpret_cast<float4 *>(dst) = v;
         }
+        if constexpr (COL_B) {
+#pragma unroll
+            for (int q = 0; q < COL_N; ++q) Bs[buf][(kcol + q * COL_STEP) * LDB + jcol] = to_f32(ecol[q]);
+            return;
+        }
 #pragma unroll
         for (int q = 0; q < QB; ++q) {
-            const float4 v = !VEC || ((live_b >> q) & 1u) ? rb[q].get() : zero;
+            const float4 v = !QB4 || ((live_b >> q) & 1u) ? rb[q].get() : zero;
             float *dst = &Bs[buf][kb(q) * LDB + jb(q)];
             if (!BJ) { dst[0] = v.x; dst[LDB] = v.y; dst[2 * LDB] = v.z; dst[3 * LDB] = v.w; }
             else *reinterpret_cast<float4 *>(dst) = v;
@@ -379,7 +401,7 @@ int32_t simt_wgrad_splits(int64_t M, int64_t N, int32_t nseg, int64_t K) {
 
 static bool quad_aligned(const void *p, int32_t t) { return (reinterpret_cast<uintptr_t>(p) & (t == G_F32 ? 15 : 7)) == 0; }
 
-template <typename TA, typename TB, typename TC, bool VEC, bool AK, bool BJ, int BM, int BN, int TM, int TN, int BK>
+template <typename TA, typename TB, typename TC, bool QA4, bool QB4, bool AK, bool BJ, int BM, int BN, int TM, int TN, int BK>
 static int32_t simt_launch(SimtRun &run, int32_t *tile_prefix, cudaStream_t st) {
     const SimtGemm &g = run.g;
     const int32_t *ready = g.mode == 0 && g.offsets && run.plan ? run.plan->prefix_of(BM) : nullptr;
@@ -399,7 +421,7 @@ static int32_t simt_launch(SimtRun &run, int32_t *tile_prefix, cudaStream_t st) 
     }
     if (grid.y > 65535 || grid.z > 65535) return MOE_ERR_UNSUPPORTED;
     run.tile_prefix = ready ? ready : tile_prefix;
-    launch_kernel((simt_gemm_kernel<TA, TB, TC, VEC, AK, BJ, BM, BN, TM, TN, BK>), grid, (BM / TM) * (BN / TN), 0, st, run);
+    launch_kernel((simt_gemm_kernel<TA, TB, TC, QA4, QB4, AK, BJ, BM, BN, TM, TN, BK>), grid, (BM / TM) * (BN / TN), 0, st, run);
     MOE_LAUNCHED();
     if (run.part) {
         launch_kernel(simt_reduce_kernel, (unsigned)cdiv(g.M * g.N * g.nseg, 256), 256, 0, st, run);
@@ -415,21 +437,35 @@ static int32_t simt_launch(SimtRun &run, int32_t *tile_prefix, cudaStream_t st) 
 // tiles 58); else 32 x 32 tiles (4 x 4), and where even those leave SMs idle 16 x 16 (2 x 2, K blocks of 64): there a
 // block's time is the latency of one chain and its loads (24 tokens x 512 features x 64 columns: 9 us; one 128 x 64
 // tile: 40).
+// Gate widths that are no multiple of four: the projection (AK, BJ) takes 128 x 64 tiles from one and a half per SM on (a whole
+// moe_gate, 4096 tokens x 512 features: 250 experts, 256 tiles, 77 us against 96 with 32 x 32 tiles; 130 experts, 160 tiles,
+// 71 against 59; 64 x 64 tiles in between: 82 and 63), else 32 x 32 ones; the gradients take 32 x 32 element-wise tiles.
 template <typename TA, typename TB, typename TC, bool AK, bool BJ>
-static int32_t simt_pick_tile(SimtRun &run, bool vec, int32_t *tile_prefix, cudaStream_t st) {
+static int32_t simt_pick_tile(SimtRun &run, bool vec_a, bool vec_b, int32_t *tile_prefix, cudaStream_t st) {
     const SimtGemm &g = run.g;
     const int64_t segs = g.offsets || g.mode == 1 ? g.nseg : 0;
     auto blocks = [&](int64_t bm, int64_t bn) {
         return (g.mode == 0 ? cdiv(g.M, bm) + segs : cdiv(g.M, bm) * segs * run.splits) * cdiv(g.N, bn);
     };
     const bool short_rows = g.mode == 0 && g.offsets && g.M <= 32 * (int64_t)g.nseg;  // segments of few rows: less padding
-    if (!vec) return simt_launch<TA, TB, TC, false, AK, BJ, 32, 32, 4, 4, 32>(run, tile_prefix, st);
+    if (!(vec_a && vec_b)) {
+        if constexpr (std::is_same<TC, bf16>::value) {  // expert products: widths are whole 16-byte vectors
+            return MOE_ERR_UNSUPPORTED;
+        } else if constexpr (AK && BJ) {
+            if (!vec_a) return MOE_ERR_UNSUPPORTED;  // activations have rows of whole 16-byte vectors
+            if (2 * blocks(128, 64) >= 3 * 148)
+                return simt_launch<TA, TB, TC, true, false, AK, BJ, 128, 64, 8, 8, 16>(run, tile_prefix, st);
+            return simt_launch<TA, TB, TC, true, false, AK, BJ, 32, 32, 4, 4, 32>(run, tile_prefix, st);
+        } else {
+            return simt_launch<TA, TB, TC, false, false, AK, BJ, 32, 32, 4, 4, 32>(run, tile_prefix, st);
+        }
+    }
     if (blocks(64, 128) >= 6 * 148 && !short_rows && g.N > 64)
-        return simt_launch<TA, TB, TC, true, AK, BJ, 64, 128, 8, 8, 16>(run, tile_prefix, st);
+        return simt_launch<TA, TB, TC, true, true, AK, BJ, 64, 128, 8, 8, 16>(run, tile_prefix, st);
     if (blocks(64, 64) >= 2 * 148 && !short_rows && !(run.part && g.N <= 32))
-        return simt_launch<TA, TB, TC, true, AK, BJ, 64, 64, 8, 4, 16>(run, tile_prefix, st);
-    if (blocks(32, 32) >= 148) return simt_launch<TA, TB, TC, true, AK, BJ, 32, 32, 4, 4, 32>(run, tile_prefix, st);
-    return simt_launch<TA, TB, TC, true, AK, BJ, 16, 16, 2, 2, 64>(run, tile_prefix, st);
+        return simt_launch<TA, TB, TC, true, true, AK, BJ, 64, 64, 8, 4, 16>(run, tile_prefix, st);
+    if (blocks(32, 32) >= 148) return simt_launch<TA, TB, TC, true, true, AK, BJ, 32, 32, 4, 4, 32>(run, tile_prefix, st);
+    return simt_launch<TA, TB, TC, true, true, AK, BJ, 16, 16, 2, 2, 64>(run, tile_prefix, st);
 }
 
 // part: simt_wgrad_splits(M, N, nseg, rows) * nseg * M * N floats (mode 1, float results), or nullptr: no slices
@@ -448,7 +484,6 @@ int32_t launch_simt_gemm(const SimtGemm &g_in, int32_t *tile_prefix, cudaStream_
                 (!g.B2 || (g.b_split % 4 == 0 && quad_aligned(g.B2, g.tb)));
     run.vec_c = g.N % 4 == 0 && g.sc_i % 4 == 0 && g.c_e % 4 == 0 && quad_aligned(g.C, g.tc) &&
                 (!g.C2 || (g.c_split % 4 == 0 && quad_aligned(g.C2, g.tc)));
-    const bool vec = vec_a && vec_b;
     run.splits = 1;
     run.part = nullptr;
     if (g.mode == 1 && part) {
@@ -458,16 +493,16 @@ int32_t launch_simt_gemm(const SimtGemm &g_in, int32_t *tile_prefix, cudaStream_
     const bool fff = g.ta == G_F32 && g.tb == G_F32 && g.tc == G_F32, bbb = g.ta == G_BF16 && g.tb == G_BF16 && g.tc == G_BF16;
     const bool bff = g.ta == G_BF16 && g.tb == G_F32 && g.tc == G_F32;
     if (ak && bj) {  // rows x weight [K, N]
-        if (fff) return simt_pick_tile<float, float, float, true, true>(run, vec, tile_prefix, st);
-        if (bbb) return simt_pick_tile<bf16, bf16, bf16, true, true>(run, vec, tile_prefix, st);
-        if (bff) return simt_pick_tile<bf16, float, float, true, true>(run, vec, tile_prefix, st);
+        if (fff) return simt_pick_tile<float, float, float, true, true>(run, vec_a, vec_b, tile_prefix, st);
+        if (bbb) return simt_pick_tile<bf16, bf16, bf16, true, true>(run, vec_a, vec_b, tile_prefix, st);
+        if (bff) return simt_pick_tile<bf16, float, float, true, true>(run, vec_a, vec_b, tile_prefix, st);
     } else if (ak) {  // rows x weight [N, K] read transposed
-        if (fff) return simt_pick_tile<float, float, float, true, false>(run, vec, tile_prefix, st);
-        if (bbb) return simt_pick_tile<bf16, bf16, bf16, true, false>(run, vec, tile_prefix, st);
+        if (fff) return simt_pick_tile<float, float, float, true, false>(run, vec_a, vec_b, tile_prefix, st);
+        if (bbb) return simt_pick_tile<bf16, bf16, bf16, true, false>(run, vec_a, vec_b, tile_prefix, st);
     } else if (bj) {  // contraction over rows
-        if (fff) return simt_pick_tile<float, float, float, false, true>(run, vec, tile_prefix, st);
-        if (bbb) return simt_pick_tile<bf16, bf16, bf16, false, true>(run, vec, tile_prefix, st);
-        if (bff) return simt_pick_tile<bf16, float, float, false, true>(run, vec, tile_prefix, st);
+        if (fff) return simt_pick_tile<float, float, float, false, true>(run, vec_a, vec_b, tile_prefix, st);
+        if (bbb) return simt_pick_tile<bf16, bf16, bf16, false, true>(run, vec_a, vec_b, tile_prefix, st);
+        if (bff) return simt_pick_tile<bf16, float, float, false, true>(run, vec_a, vec_b, tile_prefix, st);
     }
     return MOE_ERR_UNSUPPORTED;
 }
