@@ -33,14 +33,15 @@ __host__ __device__ __forceinline__ int select_rows_per_block(int32_t n) { retur
 
 // ------------------------------------------------------------------------------------------
 // Noisy logits H = clean + noise * softplus(raw) (Eq. 4), KeepTopK (Eq. 5) and the softmax over
-// the kept entries (Eq. 3). One warp per row. Each lane keeps the k+1 best of its columns in a
+// the kept entries (Eq. 3). A row is selected by one warp: each lane keeps the k+1 best of its columns in a
 // sorted register list (value descending, then index ascending); k+1 rounds of a warp arg-max
 // over the list heads then produce the global order. Lowest index wins ties everywhere.
 // softplus is evaluated in double and rounded once, H by one fused multiply-add.
 // ------------------------------------------------------------------------------------------
-// STAGED (n > 32, all rows): the noisy logits of the block's rows are formed first, one column per thread and step, and parked
+// STAGED (n > 32, few rows): the noisy logits of the block's rows are formed first, one column per thread and step, and parked
 // in shared memory for the row's warp. The softplus in double is a chain of 3000 cycles, and a warp that walks a wide row
-// alone goes through it n / 32 times (1019 rows of 256 columns: 14 us).
+// alone goes through it n / 32 times (1019 rows of 256 columns: 14 us). Where the rows alone fill the chip with warps, the
+// chains of different rows overlap and the unstaged form wins, which leaves no warp of a block idle (see launch_gate_select).
 template <int KL, bool STAGED>  // KL: length of the per-lane sorted lists, >= k + 1
 __global__ void __launch_bounds__(256) gate_select_kernel(const float *__restrict__ clean,
                                                           const float *__restrict__ raw,
@@ -145,7 +146,11 @@ int32_t launch_gate_select(const float *clean, const float *raw, const float *no
                            cudaStream_t st, const int32_t *row_list, const int32_t *row_count, const void *row_span,
                            const void *chain_list) {
     if (rows == 0) return MOE_OK;
-    const bool stage = n > 32 && !row_list;
+    // Staged up to eight rows per SM, wider rows up to n / 32 of them. A whole moe_gate with 16 features, staged / unstaged us:
+    // n = 129 (half of a step's threads idle): 1019 rows 12.3 / 11.8, 2048 rows 15.8 / 13.2, 65536 rows 239 / 170; n = 256: 12.1 / 13.6,
+    // 16.5 / 15.7, 290 / 236; n = 512: 1019 rows 16.6 / 21.0, 2048 rows 22.0 / 23.5, 3000 rows 31.5 / 30.8, 32768 rows 260 / 224; n = 4096:
+    // 2048 rows 129 / 156, 4096 rows 246 / 259.
+    const bool stage = n > 32 && !row_list && rows <= 148 * (int64_t)(n >= 256 ? n / 32 : 8);
     const int rpb = stage ? select_rows_per_block(n) : 8;
     const unsigned grid = (unsigned)cdiv(rows, rpb);
     const size_t sh = stage ? sizeof(float) * rpb * n : 0;  // at most 32 KiB
