@@ -138,7 +138,8 @@ __device__ __forceinline__ int32_t block_scan_1024(int32_t v, int32_t *sh /* [32
 //   RANK_FEW    from the chunks' histograms: every block adds the chunks before its own and scans the totals (n <= 1024)
 //   RANK_MANY   from the scanned chunk bases and offsets
 // Then 32 warps take 32 slots each: equal experts inside a warp are ranked with match_any, the warps advance the cursors one
-// after the other. (One warp walking the 32 groups with the loads on its critical path took 16 us per chunk, this takes 4.)
+// after the other. (One warp walking the 32 groups with the loads on its critical path took 16 us per chunk, this takes 4, but
+// two chunks fill an SM: see dispatch_rank_warp_kernel.)
 enum RankFrom { RANK_ONE, RANK_FEW, RANK_MANY };
 template <int FROM>
 __global__ void __launch_bounds__(1024) dispatch_rank_kernel(const int32_t *__restrict__ topk_idx, int64_t R, int32_t n,
@@ -224,6 +225,53 @@ __global__ void __launch_bounds__(1024) dispatch_rank_kernel(const int32_t *__re
     }
 }
 
+// RANK_MANY for more chunks than two per SM: one warp per chunk, up to 32 chunks in flight on an SM. It walks its slots in order,
+// 32 at a time, with the ids of eight such groups loaded together. (4 Mi slots, 16 experts, with the row copies: 371 us, a block
+// of 32 warps per chunk took 606; 512 Ki slots 51 against 54.)
+__global__ void __launch_bounds__(32) dispatch_rank_warp_kernel(const int32_t *__restrict__ topk_idx, int64_t R, int32_t n,
+                                                                const int32_t *__restrict__ chunk_base,
+                                                                const int32_t *__restrict__ offsets,
+                                                                int32_t *__restrict__ perm, int32_t *__restrict__ inv_perm) {
+    wait_previous_kernel();
+    extern __shared__ int32_t cursor[];  // next sorted row of each expert for this chunk
+    const int lane = threadIdx.x;
+    const int32_t *base = chunk_base + (int64_t)blockIdx.x * n;
+#pragma unroll 4
+    for (int32_t q = lane; q < n; q += 32) cursor[q] = offsets[q] + base[q];
+    __syncwarp();
+    const int64_t p0 = (int64_t)blockIdx.x * CH + lane;
+    for (int i0 = 0; i0 < CH; i0 += 256) {
+        int32_t id[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) id[u] = p0 + i0 + 32 * u < R ? topk_idx[p0 + i0 + 32 * u] : -1;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int64_t p = p0 + i0 + 32 * u;
+            const bool live = p < R;
+            int32_t e = id[u];
+            MOE_BOUNDS_NOTE(!live || (uint32_t)e < (uint32_t)n);
+            if ((uint32_t)e >= (uint32_t)n) e = -1;
+            const unsigned peers = __match_any_sync(0xffffffffu, e);
+            const int rank = __popc(peers & ((1u << lane) - 1u)), leader = __ffs(peers) - 1;
+            int32_t start = 0;
+            if (e >= 0 && lane == leader) {
+                start = cursor[e];
+                cursor[e] = start + __popc(peers);
+            }
+            start = __shfl_sync(0xffffffffu, start, leader);
+            if (e >= 0) {
+                const int32_t r = start + rank;
+                MOE_BOUNDS_NOTE((uint32_t)r < (uint32_t)R);
+                perm[r] = (int32_t)p;
+                inv_perm[p] = r;
+            } else if (live) {
+                inv_perm[p] = -1;  // dropped, as above
+            }
+            __syncwarp();
+        }
+    }
+}
+
 int32_t launch_dispatch_index(const int32_t *topk_idx, int64_t R, int32_t n, int32_t *perm, int32_t *inv_perm,
                               int32_t *counts, int32_t *offsets, int32_t *scratch, cudaStream_t st) {
     const int32_t nchunks = (int32_t)cdiv(R, CH);
@@ -234,7 +282,8 @@ int32_t launch_dispatch_index(const int32_t *topk_idx, int64_t R, int32_t n, int
     }
     const size_t sh = n * sizeof(int32_t);
     // one chunk: one launch. Up to 64 Ki histogram entries every block can afford to read them all (128 chunks x 256
-    // experts: 1.5 us), which saves the two scans' launches.
+    // experts: 1.5 us), which saves the two scans' launches, as long as all blocks run at once (two per SM: the entries
+    // read grow with the square of the chunks).
     if (nchunks == 1 && n <= 8192) {
         launch_kernel(dispatch_rank_kernel<RANK_ONE>, 1, 1024, sh, st, topk_idx, R, n, nullptr, 1, counts, offsets, perm, inv_perm);
         MOE_LAUNCHED();
@@ -242,7 +291,8 @@ int32_t launch_dispatch_index(const int32_t *topk_idx, int64_t R, int32_t n, int
     }
     launch_kernel(dispatch_hist_kernel, nchunks, 256, sh, st, topk_idx, R, n, scratch);
     MOE_LAUNCHED();
-    if (n <= 1024 && (int64_t)nchunks * n <= 65536) {
+    const bool one_wave = nchunks <= 2 * 148;
+    if (one_wave && n <= 1024 && (int64_t)nchunks * n <= 65536) {
         launch_kernel(dispatch_rank_kernel<RANK_FEW>, nchunks, 1024, sh, st, topk_idx, R, n, scratch, nchunks, counts, offsets, perm, inv_perm);
         MOE_LAUNCHED();
         return MOE_OK;
@@ -251,6 +301,12 @@ int32_t launch_dispatch_index(const int32_t *topk_idx, int64_t R, int32_t n, int
     MOE_LAUNCHED();
     launch_kernel(dispatch_scan_experts_kernel, 1, 1024, 0, st, counts, n, offsets);
     MOE_LAUNCHED();
+    // beyond 2048 experts the cursors leave room for few one-warp blocks (8192 experts, 1 Mi slots: 162 us, with 32 warps 134)
+    if (!one_wave && n <= 2048) {
+        launch_kernel(dispatch_rank_warp_kernel, nchunks, 32, sh, st, topk_idx, R, n, scratch, offsets, perm, inv_perm);
+        MOE_LAUNCHED();
+        return MOE_OK;
+    }
     launch_kernel(dispatch_rank_kernel<RANK_MANY>, nchunks, 1024, sh, st, topk_idx, R, n, scratch, nchunks, counts, offsets, perm, inv_perm);
     MOE_LAUNCHED();
     return MOE_OK;
