@@ -172,13 +172,20 @@ __global__ void __launch_bounds__(1024) bal_select_kernel(const float *__restric
 }
 
 // Per token (one warp): den = sum of p over the kept experts, cnt = how many keep it, the token's part of L_batchwise
-// (Eq. 20), and the per-expert counts of the threshold mask. Block partials of the loss go to loss_part. A warp takes eight
-// tokens, so that a block clears and adds up its n counts once per 64 tokens.
+// (Eq. 20), and the per-expert counts of the threshold mask. Block partials of the loss go to loss_part. A warp takes up to
+// eight tokens, so that a block clears and adds up its n counts once per 64 tokens, but no more than leave four blocks per SM:
+// the sweeps over a token's row are its time (whole gate, 4096 tokens x 2048 experts: 279 us, with eight tokens each 375;
+// 8192 x 8192: 1633, 2066; 32768 x 256 with eight: 184, with one: 234).
 constexpr int TOK_PER_WARP = 8;
+int32_t tokens_per_warp(int64_t T) {
+    const int64_t fit = T / (8 * 4 * 148);
+    return (int32_t)(fit < 1 ? 1 : imin(fit, TOK_PER_WARP));
+}
 __global__ void __launch_bounds__(256) bal_token_kernel(const float *__restrict__ p, const uint32_t *__restrict__ mask_bits,
                                                         const float *__restrict__ thr, int64_t T, int32_t n, int32_t words,
                                                         float *__restrict__ den, int32_t *__restrict__ cnt,
-                                                        int32_t *__restrict__ thr_counts, double *__restrict__ loss_part) {
+                                                        int32_t *__restrict__ thr_counts, double *__restrict__ loss_part,
+                                                        int32_t per_warp) {
     wait_previous_kernel();
     extern __shared__ int32_t s_cnt[];  // [n] threshold-mask counts of this block
     __shared__ double s_loss[8];
@@ -186,8 +193,8 @@ __global__ void __launch_bounds__(256) bal_token_kernel(const float *__restrict_
     for (int32_t j = threadIdx.x; j < n; j += blockDim.x) s_cnt[j] = 0;
     __syncthreads();
     double loss = 0.0;
-    for (int q = 0; q < TOK_PER_WARP; ++q) {
-        const int64_t t = ((int64_t)blockIdx.x * 8 + wp) * TOK_PER_WARP + q;
+    for (int q = 0; q < per_warp; ++q) {
+        const int64_t t = ((int64_t)blockIdx.x * 8 + wp) * per_warp + q;
         if (t >= T) break;
         double d = 0.0, l = 0.0;
         int32_t c = 0;
@@ -483,10 +490,12 @@ int32_t launch_balanced_gate(const void *x, int32_t act, int64_t T, int32_t d, i
     MOE_LAUNCHED();
     launch_kernel(bal_select_kernel, (unsigned)n, 1024, 0, st, pT, T, n, m, words, tok_of_row, mask_bits);
     MOE_LAUNCHED();
-    launch_kernel(bal_token_kernel, (unsigned)cdiv(T, 8 * TOK_PER_WARP), 256, n * sizeof(int32_t), st, probs, mask_bits, thr, T, n, words, den, cnt,
-                                                                             thr_counts, loss_part);
+    const int32_t per_warp = tokens_per_warp(T);
+    const int64_t tok_blocks = cdiv(T, 8 * per_warp);
+    launch_kernel(bal_token_kernel, (unsigned)tok_blocks, 256, n * sizeof(int32_t), st, probs, mask_bits, thr, T, n, words, den, cnt,
+                  thr_counts, loss_part, per_warp);
     MOE_LAUNCHED();
-    launch_kernel(bal_loss_final_kernel, 1, 256, 0, st, loss_part, cdiv(T, 8 * TOK_PER_WARP), loss);
+    launch_kernel(bal_loss_final_kernel, 1, 256, 0, st, loss_part, tok_blocks, loss);
     MOE_LAUNCHED();
     MOE_TRY(launch_exclusive_scan(cnt, (int32_t)T, tok_ptr, st, tile_sums));
     launch_kernel(bal_fill_kernel, (unsigned)cdiv(R > n ? R : n + 1, 256) + 1, 256, 0, st, tok_of_row, mask_bits, tok_ptr, R, n, m, words,
