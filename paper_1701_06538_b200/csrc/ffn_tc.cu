@@ -8,7 +8,8 @@
 //               in TMEM, double buffered (2 x 256 columns) so the epilogue of one tile overlaps
 //               the main loop of the next; tcgen05.commit releases the stage / publishes the tile
 //   warps 2-9   epilogue: tcgen05.ld (32 lanes x 32 columns per instruction), bias / ReLU / ReLU
-//               mask, round to bf16, 64-byte row stores with a row guard for ragged segments
+//               mask, round to bf16; whole [32][64] boxes leave as bulk tensor stores, boxes cut by a
+//               segment end as guarded row stores
 //
 // Three operand arrangements (KIND):
 //   ROW_BMN  rows x K activations (K-major A) times a per-expert [K, N] weight (N contiguous,
@@ -335,7 +336,7 @@ struct BoxArgs {
     int64_t colsum_row;
     const bf16 *next_bias;      // of the warp's next box, or nullptr
     uint2 keep;                 // mask bits
-    bool have_acc, wait_box;    // wait_box: an earlier store may still be reading the box
+    bool have_acc;
 };
 template <int EPI, bool MASKT, typename Release>
 __device__ __forceinline__ void epilogue_box(const GemmParams &p, int lane, const BoxArgs &b, uint4 (&bias)[2][4],
@@ -391,7 +392,7 @@ __device__ __forceinline__ void epilogue_box(const GemmParams &p, int lane, cons
         *reinterpret_cast<uint2 *>(p.bits_out + out_row * (p.N >> 5) + (b.col0 >> 5)) =
             make_uint2(positive_bits(packed[0]), positive_bits(packed[1]));
     if (staged) {
-        if (!MASKT && b.wait_box) {
+        if (!MASKT) {  // an earlier store may still be reading the box
             if (lane == 0) tma_store_wait_read();
             __syncwarp();
         }
@@ -463,7 +464,8 @@ struct Tile {
 // Tile ids are handed out round-robin. What a tile needs from global memory (its segment's bounds) is
 // fetched one tile ahead (tile_fetch) and only turned into a Tile (tile_decode) when the tile starts, so
 // the load latency never sits between two tiles. ROW_* with ragged segments read one 16-byte record per
-// M tile from a table built by tile_table_kernel; WGRAD reads the two segment bounds.
+// M tile (the experts' from the call's segment plan, the grouped gates' from tile_table_kernel); WGRAD reads the two
+// segment bounds.
 template <int KIND>
 __device__ __forceinline__ int4 tile_fetch(const GemmParams &p, int32_t id) {
     if (!p.offsets || id >= p.total_tiles) return make_int4(-1, 0, 0, 0);
@@ -552,8 +554,9 @@ template <int KIND, int TM> struct TileIter {
 // into sub-blocks of p.sub_kb0 / p.sub_kb K blocks (first term / other terms). Each sub-block is accumulated in TMEM on
 // its own (an fp32 tensor-core accumulator truncates, and a long run of same-sign terms loses low bits: 128 rows keep
 // that below 1e-5), handed to the epilogue like a tile, and added there, with rounding to nearest, to running sums in
-// registers (a lane's row of the warp's 128 columns); the sums go to global memory once per tile. (With the sums in shared
-// memory, which left room for two operand stages, a K block took 1850 cycles: the latency of its loads.)
+// registers (a lane's row of the warp's 128 columns; the cap of 168 registers makes the compiler spill 88 bytes of other
+// values); the sums go to global memory once per tile. (With the sums in shared memory, which left room for two operand
+// stages, a K block took 1850 cycles: the latency of its loads.)
 template <int KIND, int EPI, bool ACC = false>
 __global__ void __launch_bounds__(NTHREADS, 1)
 grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -776,7 +779,6 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             b.map_row = (int32_t)b.row0 + (KIND == WGRAD ? t.e * p.M : 0);
             b.colsum_row = t.mt * 4 + quarter;
             b.have_acc = have_acc;
-            b.wait_box = true;
             uint4 bias[2][4];
             const bf16 *bias_at = (EPI & EPI_BIAS) ? p.bias + (int64_t)t.e * p.N + first : nullptr;
             if ((EPI & EPI_BIAS) && boxes > 0) bias_load(bias_at, bias);
@@ -1254,7 +1256,6 @@ grouped_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
             b.map_row = (int32_t)b.row0 + (KIND == WGRAD ? t.e * p.M : 0);
             b.colsum_row = (t.mt * 2 + (int)rank) * 4 + quarter;
             b.have_acc = have_acc;
-            b.wait_box = true;
             uint4 bias[2][4];
             const bf16 *bias_at = (EPI & EPI_BIAS) ? p.bias + (int64_t)t.e * p.N + first : nullptr;
             if ((EPI & EPI_BIAS) && boxes > 0) bias_load(bias_at, bias);
@@ -1816,7 +1817,7 @@ bool tc_gate_bwd_supported(int32_t act, int32_t d, int32_t n) {
 // term, added in double afterwards), and inside a range the tensor-core accumulator is restarted every GB_ROWS_HI rows
 // for the leading (hi) term: an fp32 accumulator loses low bits when a long run of same-sign terms is added (e.g. the
 // gradient of a constant input feature); 128 rows keep that below 1e-5 of the result. The mid and lo terms are 2^-8
-// and 2^-16 of the hi term and restart every GB_ROWS_LO rows. The restarts' sums are added in shared memory (see the
+// and 2^-16 of the hi term and restart every GB_ROWS_LO rows. The restarts' sums are added in registers (see the
 // ACC kernel), so only one partial per range goes to global memory.
 constexpr int GB_ROWS_HI = 128, GB_ROWS_LO = 2048;
 static void gate_bwd_split(int64_t T, int32_t d, int32_t n, int32_t *nranges, int32_t *rows) {

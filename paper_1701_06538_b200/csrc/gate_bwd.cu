@@ -18,7 +18,8 @@ __global__ void __launch_bounds__(256) gate_logit_grads_kernel(
     const float *__restrict__ noise, const float *__restrict__ clean, const float *__restrict__ raw,
     const int32_t *__restrict__ idx, const float *__restrict__ gates, const float *__restrict__ kth_vals,
     const int32_t *__restrict__ kth_idx, const float *__restrict__ dgates, const float *__restrict__ dload,
-    const int32_t *__restrict__ dload_row_group, int64_t rows, int32_t n, int32_t k, float *__restrict__ dlogit, bf16 *__restrict__ dsplit, const int32_t *__restrict__ split_row_index) {
+    const int32_t *__restrict__ dload_row_group, int64_t rows, int32_t n, int32_t k, float *__restrict__ dlogit,
+    bf16 *__restrict__ dsplit, const int32_t *__restrict__ split_row_index) {
     wait_previous_kernel();
     const int lane = threadIdx.x & 31;
     const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
