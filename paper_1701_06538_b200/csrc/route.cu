@@ -607,8 +607,10 @@ int32_t launch_combine(const void *ys, int32_t act, const float *gates, const in
 
 // dgates[t,s] = <dy[t], ys[row]>,  dys[row] = gates[t,s] * dy[t], with dy = dY, or (LAYER: adjoint of the sigmoid and
 // the dropout of Appendix C) dy = dY * keep * keep_scale * s (1 - s), s = sigmoid(y), y recomputed from the ys rows
-// this kernel gathers anyway (same order of operations as the forward, so the same y bit for bit).
-template <typename XT, int KT, int VB, bool LAYER>
+// this kernel gathers anyway (same order of operations as the forward, so the same y bit for bit). IMP: dgates[t,s] gets the
+// Importance loss's gradient dimp of its expert added, fetched behind the rows' loop: a value that is alive beside the rows
+// costs the LAYER variants, at their cap of 80 registers, a third (131072 tokens x 1024, two slots: 303 us, this way 226).
+template <typename XT, int KT, int VB, bool LAYER, bool IMP>
 __global__ void __launch_bounds__(256, LAYER ? 3 : 1) combine_bwd_kernel(const XT *__restrict__ dY, const XT *__restrict__ ys,
                                                           const float *__restrict__ gates,
                                                           const int32_t *__restrict__ inv_perm, int64_t T,
@@ -623,11 +625,6 @@ __global__ void __launch_bounds__(256, LAYER ? 3 : 1) combine_bwd_kernel(const X
     const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
     const int nvec = d / VN;
     for (int64_t t = warp; t < T; t += nwarps) {
-        float imp = 0.0f;  // lane s: what the Importance loss adds to slot s (loaded beside the rows, used at the end)
-        if (dimp && lane < k) {
-            const int32_t e = topk_idx[t * k + lane];
-            if ((uint32_t)e < (uint32_t)n) imp = dimp[e];
-        }
         int64_t rowo[KT];
         float g[KT], dot[KT];
         bool valid[KT];
@@ -690,8 +687,14 @@ __global__ void __launch_bounds__(256, LAYER ? 3 : 1) combine_bwd_kernel(const X
                 float v = dot[s];
 #pragma unroll
                 for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-                const float imp_s = __shfl_sync(0xffffffffu, imp, s);
-                if (lane == 0) dgates[t * k + s] = (valid[s] ? v : 0.0f) + imp_s;
+                if (lane == 0) {
+                    v = valid[s] ? v : 0.0f;
+                    if (IMP) {
+                        const int32_t e = topk_idx[t * k + s];
+                        v += (uint32_t)e < (uint32_t)n ? dimp[e] : 0.0f;
+                    }
+                    dgates[t * k + s] = v;
+                }
             }
         }
     }
@@ -703,19 +706,23 @@ int32_t launch_combine_bwd(const void *dY, const void *ys, int32_t act, const fl
                            const float *dimp, int32_t n) {
     if (T == 0) return MOE_OK;
     const unsigned grid = (unsigned)imin(cdiv(T, 8), 148 * 16);
-#define MOE_CALL_L(KT, VB, L)                                                                                            \
+#define MOE_CALL_LI(KT, VB, L, I)                                                                                        \
     if (act == MOE_BF16)                                                                                                 \
-        launch_kernel((combine_bwd_kernel<bf16, KT, VB, L>), grid, 256, 0, st, (const bf16 *)dY, (const bf16 *)ys, gates, inv_perm, T, \
-                                                                   k, d, dgates, (bf16 *)dys, keep, keep_scale, topk_idx, dimp, n);          \
+        launch_kernel((combine_bwd_kernel<bf16, KT, VB, L, I>), grid, 256, 0, st, (const bf16 *)dY, (const bf16 *)ys, gates, \
+                      inv_perm, T, k, d, dgates, (bf16 *)dys, keep, keep_scale, topk_idx, dimp, n);                      \
     else                                                                                                                 \
-        launch_kernel((combine_bwd_kernel<float, KT, VB, L>), grid, 256, 0, st, (const float *)dY, (const float *)ys, gates, inv_perm, \
-                                                                    T, k, d, dgates, (float *)dys, keep, keep_scale, topk_idx, dimp, n)
+        launch_kernel((combine_bwd_kernel<float, KT, VB, L, I>), grid, 256, 0, st, (const float *)dY, (const float *)ys, gates, \
+                      inv_perm, T, k, d, dgates, (float *)dys, keep, keep_scale, topk_idx, dimp, n)
+#define MOE_CALL_L(KT, VB, L)                    \
+    if (dimp) { MOE_CALL_LI(KT, VB, L, true); }  \
+    else { MOE_CALL_LI(KT, VB, L, false); }
 #define MOE_CALL(KT, VB)                     \
-    if (keep) { MOE_CALL_L(KT, VB, true); }  \
-    else { MOE_CALL_L(KT, VB, false); }
+    if (keep) { MOE_CALL_L(KT, VB, true) }   \
+    else { MOE_CALL_L(KT, VB, false) }
     MOE_DISPATCH_KT(k, MOE_CALL);
 #undef MOE_CALL
 #undef MOE_CALL_L
+#undef MOE_CALL_LI
     MOE_LAUNCHED();
     return MOE_OK;
 }
