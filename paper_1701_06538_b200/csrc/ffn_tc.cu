@@ -1613,11 +1613,13 @@ static int32_t launch_tile_table(const int32_t *offsets, int32_t nseg, int32_t t
 // A thread block takes 64 columns of one segment: 16 column lanes (four adjacent columns each, 16-byte loads) by 16 row
 // lanes; row lane q takes the blocks b = b0 + q, b0 + q + 16, ... (eight loads in flight: the largest expert of a skewed
 // batch has over a thousand blocks and sets this kernel's duration) and the 16 sums are added in lane order: the
-// result does not depend on timing. A block takes `cols` columns: 64, or, where a segment has about one tile (thousands of
-// experts), 1024: a segment of at most 16 blocks is then added by one thread per four columns, in the same order.
+// result does not depend on timing. A block takes COLS columns: 64, or, where a segment has about one tile (thousands of
+// experts), 1024: a segment of at most 16 blocks is then added by one thread per four columns, in the same order. (Both
+// in one kernel cost the narrow form a loop and spills: 61 us instead of 41 at 128 experts x 4096 columns.)
+template <int COLS>
 __global__ void __launch_bounds__(256) colsum_blocks_final_kernel(const float *__restrict__ part, int32_t N,
                                                                   const int32_t *__restrict__ tile_prefix, int32_t G,
-                                                                  int32_t cols, bf16 *__restrict__ out) {
+                                                                  bf16 *__restrict__ out) {
     wait_previous_kernel();
     __shared__ float4 sh[16][16];
     const int32_t e = blockIdx.x, q = threadIdx.x >> 4, cl = threadIdx.x & 15;
@@ -1628,8 +1630,8 @@ __global__ void __launch_bounds__(256) colsum_blocks_final_kernel(const float *_
         pk.x = *reinterpret_cast<const uint32_t *>(&o0); pk.y = *reinterpret_cast<const uint32_t *>(&o1);
         *reinterpret_cast<uint2 *>(out + (int64_t)e * N + j) = pk;
     };
-    if (cols > 64 && b1 - b0 <= 16) {
-        const int32_t j = blockIdx.y * cols + threadIdx.x * 4;
+    if (COLS > 64 && b1 - b0 <= 16) {
+        const int32_t j = blockIdx.y * COLS + threadIdx.x * 4;
         if (j >= N) return;
         float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll 4
@@ -1640,8 +1642,9 @@ __global__ void __launch_bounds__(256) colsum_blocks_final_kernel(const float *_
         store(j, s);
         return;
     }
-    for (int32_t j0 = blockIdx.y * cols; j0 < N && j0 < (int32_t)(blockIdx.y + 1) * cols; j0 += 64) {  // N is a multiple of 64
-        const int32_t j = j0 + cl * 4;
+    for (int32_t c = 0; c < COLS; c += 64) {
+        const int32_t j = blockIdx.y * COLS + c + cl * 4;
+        if (COLS > 64 && j >= N) break;  // N is a multiple of 64: all threads alike
         float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         int32_t b = b0 + q;
         for (; b + 16 * 7 < b1; b += 16 * 8) {
@@ -1655,7 +1658,7 @@ __global__ void __launch_bounds__(256) colsum_blocks_final_kernel(const float *_
             const float4 v = *reinterpret_cast<const float4 *>(part + (int64_t)b * N + j);
             s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
         }
-        __syncthreads();  // sh may still be read for the columns before
+        if (COLS > 64) __syncthreads();  // sh may still be read for the columns before
         sh[q][cl] = s;
         __syncthreads();
         if (q == 0) {
@@ -1682,9 +1685,12 @@ int32_t tc_row_gemm(const void *A, const void *W, bool transposed, const int32_t
     }
     auto finish = [&](int32_t rc, int32_t G) -> int32_t {
         if (rc != MOE_OK || !colsum_out) return rc;
-        const int32_t cols = nseg >= 128 && R <= 128 * (int64_t)nseg ? 1024 : 64;
-        launch_kernel(colsum_blocks_final_kernel, dim3((unsigned)nseg, (unsigned)cdiv(N, cols)), 256, 0, st, colsum_part, N,
-                      plan.prefix[0], G, cols, (bf16 *)colsum_out);
+        if (nseg >= 128 && R <= 128 * (int64_t)nseg)
+            launch_kernel(colsum_blocks_final_kernel<1024>, dim3((unsigned)nseg, (unsigned)cdiv(N, 1024)), 256, 0, st, colsum_part, N,
+                          plan.prefix[0], G, (bf16 *)colsum_out);
+        else
+            launch_kernel(colsum_blocks_final_kernel<64>, dim3((unsigned)nseg, (unsigned)cdiv(N, 64)), 256, 0, st, colsum_part, N,
+                          plan.prefix[0], G, (bf16 *)colsum_out);
         MOE_LAUNCHED();
         return MOE_OK;
     };

@@ -575,19 +575,20 @@ __global__ void __launch_bounds__(256) colsum_partial_kernel(const XT *__restric
 }
 
 // Sum of a segment's tile sums (a segment of one tile is complete already, which with thousands of experts most are: a
-// block then looks at 256 columns, 32 at a time): a block takes 32 columns, its eight warps the tiles b0 + w, b0 + w + 8, ... (eight loads in
-// flight: the largest expert of a skewed batch has hundreds of tiles), the eight sums are added in warp order.
-template <typename XT>
+// block then looks at COLS = 256 columns, 32 at a time): a block takes 32 columns, its eight warps the tiles b0 + w, b0 + w + 8, ...
+// (eight loads in flight: the largest expert of a skewed batch has hundreds of tiles), the eight sums are added in warp order.
+template <typename XT, int COLS>
 __global__ void __launch_bounds__(256) colsum_final_kernel(const float *__restrict__ part, int32_t N,
                                                            const int32_t *__restrict__ tile_prefix,
-                                                           int32_t cols, XT *__restrict__ out) {
+                                                           XT *__restrict__ out) {
     wait_previous_kernel();
     __shared__ float sh[8][32];
     const int32_t e = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int32_t b0 = tile_prefix[e], b1 = tile_prefix[e + 1];
     if (b1 - b0 == 1) return;
-    for (int32_t j0 = blockIdx.y * cols; j0 < N && j0 < (int32_t)(blockIdx.y + 1) * cols; j0 += 32) {
-        const int32_t j = j0 + lane;
+    for (int32_t c = 0; c < COLS; c += 32) {
+        const int32_t j0 = blockIdx.y * COLS + c, j = j0 + lane;
+        if (COLS > 32 && j0 >= N) break;
         float s = 0.0f;
         if (j < N) {
             int32_t b = b0 + w;
@@ -600,7 +601,7 @@ __global__ void __launch_bounds__(256) colsum_final_kernel(const float *__restri
             }
             for (; b < b1; b += 8) s += part[(int64_t)b * N + j];
         }
-        __syncthreads();  // sh may still be read for the columns before
+        if (COLS > 32) __syncthreads();  // sh may still be read for the columns before
         sh[w][lane] = s;
         __syncthreads();
         if (w == 0 && j < N) {
@@ -616,19 +617,19 @@ int32_t launch_segment_colsum(const void *in, int32_t act, const int32_t *offset
                               int32_t N, void *out, float *scratch, const int32_t *tile_prefix, cudaStream_t st) {
     const int vcols = act == MOE_BF16 ? 256 : 128;  // columns per block of the partial sums: 32 lanes x one 16-byte vector
     dim3 g1((unsigned)(cdiv(R, CS_ROWS) + nseg), (unsigned)cdiv(N, vcols));
-    const int32_t cols = nseg >= 1024 ? 256 : 32;  // of a block of the final sums
-    dim3 g2((unsigned)nseg, (unsigned)cdiv(N, cols));
-    if (act == MOE_BF16) {
-        launch_kernel(colsum_partial_kernel<bf16>, g1, 256, 0, st, (const bf16 *)in, offsets, nseg, N, tile_prefix, scratch, (bf16 *)out);
+    const bool many = nseg >= 1024;
+    dim3 g2((unsigned)nseg, (unsigned)cdiv(N, many ? 256 : 32));
+    auto run = [&](auto *typed) -> int32_t {
+        using XT = typename std::remove_pointer<decltype(typed)>::type;
+        XT *o = static_cast<XT *>(out);
+        launch_kernel(colsum_partial_kernel<XT>, g1, 256, 0, st, static_cast<const XT *>(in), offsets, nseg, N, tile_prefix, scratch, o);
         MOE_LAUNCHED();
-        launch_kernel(colsum_final_kernel<bf16>, g2, 256, 0, st, scratch, N, tile_prefix, cols, (bf16 *)out);
-    } else {
-        launch_kernel(colsum_partial_kernel<float>, g1, 256, 0, st, (const float *)in, offsets, nseg, N, tile_prefix, scratch, (float *)out);
+        if (many) launch_kernel((colsum_final_kernel<XT, 256>), g2, 256, 0, st, scratch, N, tile_prefix, o);
+        else launch_kernel((colsum_final_kernel<XT, 32>), g2, 256, 0, st, scratch, N, tile_prefix, o);
         MOE_LAUNCHED();
-        launch_kernel(colsum_final_kernel<float>, g2, 256, 0, st, scratch, N, tile_prefix, cols, (float *)out);
-    }
-    MOE_LAUNCHED();
-    return MOE_OK;
+        return MOE_OK;
+    };
+    return act == MOE_BF16 ? run((bf16 *)nullptr) : run((float *)nullptr);
 }
 
 }  // namespace moe
