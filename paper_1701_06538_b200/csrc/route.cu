@@ -608,8 +608,9 @@ int32_t launch_combine(const void *ys, int32_t act, const float *gates, const in
 // dgates[t,s] = <dy[t], ys[row]>,  dys[row] = gates[t,s] * dy[t], with dy = dY, or (LAYER: adjoint of the sigmoid and
 // the dropout of Appendix C) dy = dY * keep * keep_scale * s (1 - s), s = sigmoid(y), y recomputed from the ys rows
 // this kernel gathers anyway (same order of operations as the forward, so the same y bit for bit). IMP: dgates[t,s] gets the
-// Importance loss's gradient dimp of its expert added, fetched behind the rows' loop: a value that is alive beside the rows
-// costs the LAYER variants, at their cap of 80 registers, a third (131072 tokens x 1024, two slots: 303 us, this way 226).
+// Importance loss's gradient dimp of its expert added, fetched beside the rows (lane s: slot s), but in the LAYER variants behind
+// their loop: at their cap of 80 registers a value that is alive beside the rows costs a third (131072 tokens x 1024, two
+// slots: 303 us, this way 226).
 template <typename XT, int KT, int VB, bool LAYER, bool IMP>
 __global__ void __launch_bounds__(256, LAYER ? 3 : 1) combine_bwd_kernel(const XT *__restrict__ dY, const XT *__restrict__ ys,
                                                           const float *__restrict__ gates,
@@ -625,6 +626,11 @@ __global__ void __launch_bounds__(256, LAYER ? 3 : 1) combine_bwd_kernel(const X
     const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
     const int nvec = d / VN;
     for (int64_t t = warp; t < T; t += nwarps) {
+        float imp = 0.0f;
+        if (IMP && !LAYER && lane < k) {
+            const int32_t e = topk_idx[t * k + lane];
+            if ((uint32_t)e < (uint32_t)n) imp = dimp[e];
+        }
         int64_t rowo[KT];
         float g[KT], dot[KT];
         bool valid[KT];
@@ -687,9 +693,10 @@ __global__ void __launch_bounds__(256, LAYER ? 3 : 1) combine_bwd_kernel(const X
                 float v = dot[s];
 #pragma unroll
                 for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+                const float imp_s = IMP && !LAYER ? __shfl_sync(0xffffffffu, imp, s) : 0.0f;
                 if (lane == 0) {
-                    v = valid[s] ? v : 0.0f;
-                    if (IMP) {
+                    v = (valid[s] ? v : 0.0f) + imp_s;
+                    if (IMP && LAYER) {
                         const int32_t e = topk_idx[t * k + s];
                         v += (uint32_t)e < (uint32_t)n ? dimp[e] : 0.0f;
                     }
