@@ -11,9 +11,11 @@ namespace moe {
 constexpr int LCHUNKS_MAX = 148 * 4;
 
 // a row per warp until the chip is full: the normal-CDF evaluations of a row are one long latency chain per lane. Up to 32
-// columns one block adds up all chunks, and half as many are enough (8192 rows: 6 columns 12.0 us for both launches, with all
-// chunks 15.2; 30 columns 13.4, 15.8)
-static inline int32_t level_chunks(int64_t rows, int32_t n) { return (int32_t)imin(cdiv(rows, 8), n <= 32 ? LCHUNKS_MAX / 2 : LCHUNKS_MAX); }
+// columns one block adds up all chunks, and up to 16384 rows half as many are enough (8192 rows: 6 columns 12.0 us for both
+// launches, with all chunks 15.2; 15000 rows of 30 columns 15.5, 17.9; but 60000 rows of 20 columns 28.4, 26.5)
+static inline int32_t level_chunks(int64_t rows, int32_t n) {
+    return (int32_t)imin(cdiv(rows, 8), n <= 32 && rows <= 16384 ? LCHUNKS_MAX / 2 : LCHUNKS_MAX);
+}
 int64_t losses_ws_floats(int64_t rows, int32_t n) { return 2 * (int64_t)level_chunks(rows, n) * n + 64; }
 
 __device__ __forceinline__ float softplus_f(float r) { return fmaxf(r, 0.0f) + log1pf(expf(-fabsf(r))); }

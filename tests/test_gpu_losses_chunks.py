@@ -12,8 +12,9 @@ from helpers import TOL_F32, assert_close, cfg_of, dev, f32, host, small_workloa
 pytestmark = pytest.mark.gpu
 
 
-# 296 chunks of eight rows up to 32 columns, 592 beyond
-@pytest.mark.parametrize("T,n,k", [(1, 3, 1), (2368, 32, 2), (2369, 6, 2), (2369, 33, 3), (4737, 32, 4), (4737, 40, 1), (9001, 5, 5)])
+# at most 296 chunks up to 32 columns and 16384 rows, 592 beyond
+@pytest.mark.parametrize("T,n,k", [(1, 3, 1), (2368, 32, 2), (2369, 6, 2), (2369, 33, 3), (4737, 32, 4), (4737, 40, 1), (9001, 5, 5), (16384, 8, 2),
+                                   (16385, 8, 2)])
 def test_losses_of_whole_batches(T, n, k):
     w = small_workload(f"losses-{T}-{n}", T=T, d=16, h=16, n=n, k=k, seed=30 + k)
     I = synth.make_all(w)
