@@ -120,7 +120,13 @@ __global__ void __launch_bounds__(256) adam_columns_kernel(const float *__restri
 // keeps one 16-byte column vector, with its column averages in registers, and walks down the block's rows, four of them
 // in flight. HBM bound: parameters read and written, gradients read (as one flat index space, the column averages came
 // from L1 with twice the loads of the parameters: 169 us for 134 M parameters, 4.8 TB/s).
+// The estimate is a product, so its root is the product of a row's and a column's root (each taken once per row and column and
+// correctly rounded): one multiply-add and one reciprocal per element.
+__device__ __forceinline__ float adam_step(float w, float g, float lr, float row_root, float col_root, float eps) {
+    return w - __fdividef(lr * g, fmaf(row_root, col_root, eps));
+}
 __device__ __forceinline__ float sqrt_fast(float x) { return x > 0.0f ? x * rsqrtf(x) : 0.0f; }  // ~2 ulp, no IEEE sqrt sequence
+__device__ __forceinline__ float root(float x) { return x > 0.0f ? sqrtf(x) : 0.0f; }
 
 template <typename XT>
 __global__ void __launch_bounds__(256) adam_update_kernel(XT *__restrict__ W, const XT *__restrict__ g, int32_t rows,
@@ -145,7 +151,7 @@ __global__ void __launch_bounds__(256) adam_update_kernel(XT *__restrict__ W, co
 #pragma unroll
         for (int q = 0; q < VN / 4; ++q) {
             const float4 f = reinterpret_cast<const float4 *>(ca + v * VN)[q];
-            c[4 * q] = f.x; c[4 * q + 1] = f.y; c[4 * q + 2] = f.z; c[4 * q + 3] = f.w;
+            c[4 * q] = root(f.x); c[4 * q + 1] = root(f.y); c[4 * q + 2] = root(f.z); c[4 * q + 3] = root(f.w);
         }
         for (int r = group; r < nr; r += 4 * groups) {
             Vec<XT> w[4], gr[4];
@@ -156,7 +162,7 @@ __global__ void __launch_bounds__(256) adam_update_kernel(XT *__restrict__ W, co
                 if (row < nr) {
                     w[u].raw = reinterpret_cast<const uint4 *>(W + base + (int64_t)row * cols)[v];
                     gr[u].raw = reinterpret_cast<const uint4 *>(g + base + (int64_t)row * cols)[v];
-                    rs[u] = row_avg[(int64_t)e * rows + r0 + row] * scale;
+                    rs[u] = sqrt_fast(row_avg[(int64_t)e * rows + r0 + row] * scale);
                 }
             }
 #pragma unroll
@@ -165,7 +171,7 @@ __global__ void __launch_bounds__(256) adam_update_kernel(XT *__restrict__ W, co
                 if (row >= nr) break;
 #pragma unroll
                 for (int i = 0; i < VN; ++i)
-                    w[u].set(i, w[u].get(i) - __fdividef(lr * gr[u].get(i), sqrt_fast(rs[u] * c[i]) + eps));
+                    w[u].set(i, adam_step(w[u].get(i), gr[u].get(i), lr, rs[u], c[i], eps));
                 reinterpret_cast<uint4 *>(W + base + (int64_t)row * cols)[v] = w[u].raw;
             }
         }
@@ -215,6 +221,241 @@ __global__ void __launch_bounds__(256) adam_update_flat_kernel(XT *__restrict__ 
     }
 }
 
+// ------------------------------------------------------------------------------------------
+// The whole step in one launch, for matrices that stay in L2 between the two looks at their gradient. A cluster of CTAs takes an
+// expert's matrix, each CTA a slab of its rows: squared row and column sums of the slab, the column sums of the cluster's
+// CTAs added through distributed shared memory, then the update of the slab, whose gradients are read from L2 the second time.
+// Two blocks per SM, of different clusters: one streams while the other one is at the cluster's barrier. HBM bound: gradients read
+// once, parameters read and written. The last clusters step the biases.
+// A warp takes a strip of 32 column vectors (a narrow matrix: several rows side by side) and walks down its share of the
+// slab's rows; strips and row shares are dealt to the 16 warps.
+// ------------------------------------------------------------------------------------------
+constexpr int FUSED_THREADS = 512, FUSED_WARPS = FUSED_THREADS / 32;
+constexpr int64_t FUSED_MATRIX_BYTES = 4 << 20, FUSED_SLAB_BYTES = 256 << 10;
+struct FusedMatrix {
+    void *W;
+    const void *g;
+    float *row_avg, *col_avg;
+    int32_t rows, cols, per;            // per: rows of a CTA's slab
+    int32_t lanes, strips, groups;      // lanes of a row, strips of `lanes` vectors, row shares (1 where strips exceed the warps)
+};
+struct FusedVector {
+    void *b;
+    const void *g;
+    float *v;
+    int64_t count;
+};
+struct FusedAdam {
+    FusedMatrix m[2];
+    FusedVector v[2];
+    int32_t n, cluster;
+    float lr, beta2, inv_correction, eps;
+};
+// floats of shared memory: column sums of the CTA, updated column and row averages, sums of the row shares / strips
+static int64_t fused_smem_floats(const FusedMatrix &m) {
+    return 2 * (int64_t)m.cols + m.per + (int64_t)m.groups * m.cols + (int64_t)m.strips * m.per + 4;
+}
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ uint32_t cluster_address(const void *p, uint32_t cta) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(cta));
+    return r;
+}
+__device__ __forceinline__ float ld_cluster(uint32_t at) {
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(at) : "memory");
+    return v;
+}
+__device__ __forceinline__ double ld_cluster_double(uint32_t at) {
+    double v;
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(at) : "memory");
+    return v;
+}
+
+template <typename XT>
+__device__ __forceinline__ void adam_vector_step(XT *b, const XT *g, float *v, int64_t i, float lr, float beta2, float inv_correction, float eps) {
+    const float gi = to_f32(g[i]);
+    const float vi = beta2 * v[i] + (1.0f - beta2) * gi * gi;
+    v[i] = vi;
+    b[i] = from_f32<XT>(to_f32(b[i]) - lr * gi / (sqrtf(vi * inv_correction) + eps));  // tiny tensor: exact operations
+}
+
+template <typename XT>
+__global__ void __launch_bounds__(FUSED_THREADS, 2) adam_fused_kernel(const __grid_constant__ FusedAdam a) {
+    wait_previous_kernel();
+    constexpr int VN = Vec<XT>::N, UR = 4;
+    extern __shared__ __align__(16) double fused_sh[];
+    double *row_total = fused_sh;  // this CTA's sum of updated row averages; [2..] its warps' shares
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int32_t C = a.cluster, item = blockIdx.x / C, rank = blockIdx.x % C;
+    if (item >= 2 * a.n) {
+        const int64_t first = ((int64_t)blockIdx.x - 2 * (int64_t)a.n * C) * FUSED_THREADS + tid;
+        const int64_t step = ((int64_t)gridDim.x - 2 * (int64_t)a.n * C) * FUSED_THREADS;
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+            for (int64_t i = first; i < a.v[q].count; i += step)
+                adam_vector_step((XT *)a.v[q].b, (const XT *)a.v[q].g, a.v[q].v, i, a.lr, a.beta2, a.inv_correction, a.eps);
+        return;
+    }
+    const FusedMatrix &m = a.m[item >= a.n];
+    const int32_t e = item >= a.n ? item - a.n : item;
+    const int32_t rows = m.rows, cols = m.cols, L = m.lanes, strips = m.strips, groups = m.groups, nvec = cols / VN;
+    const int32_t r0 = min(rank * m.per, rows), nr = min(m.per, rows - r0);
+    float *col_part = reinterpret_cast<float *>(fused_sh + 2 + FUSED_WARPS), *col_now = col_part + cols;
+    float *group_cols = col_now + cols, *row_now = group_cols + groups * cols, *strip_rows = row_now + m.per;
+    const int64_t base = ((int64_t)e * rows + r0) * nvec;  // in vectors
+    const uint4 *G = reinterpret_cast<const uint4 *>(m.g) + base;
+    uint4 *W = reinterpret_cast<uint4 *>(m.W) + base;
+    float *row_avg = m.row_avg + (int64_t)e * rows + r0, *col_avg = m.col_avg + (int64_t)e * cols;
+
+    // the old averages are fetched beside the first rows; every CTA reads them before its arrival at the barrier behind which they are written
+    for (int j = tid; j < cols; j += FUSED_THREADS) col_now[j] = a.beta2 * col_avg[j];
+    for (int r = tid; r < nr; r += FUSED_THREADS) row_now[r] = a.beta2 * row_avg[r];
+    const int side = 32 / L, sub = lane / L, vl = lane % L;             // rows side by side in a warp
+    const int grp = warp / min(strips, FUSED_WARPS), row_step = groups * side;
+    const bool warp_on = grp < groups;
+    if (warp_on) {
+        for (int strip = warp % min(strips, FUSED_WARPS); strip < strips; strip += FUSED_WARPS) {
+            const int v = strip * L + vl;
+            const bool live = v < nvec;
+            float colacc[VN];
+#pragma unroll
+            for (int i = 0; i < VN; ++i) colacc[i] = 0.0f;
+            for (int rb = grp * side; rb < nr; rb += UR * row_step) {
+                Vec<XT> in[UR];
+#pragma unroll
+                for (int u = 0; u < UR; ++u) {
+                    const int r = rb + sub + u * row_step;
+                    in[u].raw = live && r < nr ? G[(int64_t)r * nvec + v] : make_uint4(0, 0, 0, 0);
+                }
+                float c4[VN], s[UR];
+#pragma unroll
+                for (int u = 0; u < UR; ++u) {
+                    s[u] = 0.0f;
+#pragma unroll
+                    for (int i = 0; i < VN; ++i) {
+                        const float x = in[u].get(i), q = x * x;
+                        c4[i] = u ? c4[i] + q : q;
+                        s[u] += q;
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < VN; ++i) colacc[i] += c4[i];
+                if (L >= 4) {  // two halving steps over four rows, then one value per lane
+                    const bool up = vl & (L >> 1), up2 = vl & (L >> 2);
+                    const float k0 = up ? s[2] : s[0], k1 = up ? s[3] : s[1];
+                    float t0 = k0 + __shfl_xor_sync(0xffffffffu, up ? s[0] : s[2], L >> 1);
+                    float t1 = k1 + __shfl_xor_sync(0xffffffffu, up ? s[1] : s[3], L >> 1);
+                    float t = (up2 ? t1 : t0) + __shfl_xor_sync(0xffffffffu, up2 ? t0 : t1, L >> 2);
+                    for (int off = L >> 3; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+                    const int r = rb + sub + (2 * up + up2) * row_step;
+                    if ((vl & ((L >> 2) - 1)) == 0 && r < nr) strip_rows[strip * m.per + r] = t;
+                } else {
+#pragma unroll
+                    for (int u = 0; u < UR; ++u) {
+                        for (int off = L >> 1; off > 0; off >>= 1) s[u] += __shfl_xor_sync(0xffffffffu, s[u], off);
+                        const int r = rb + sub + u * row_step;
+                        if (vl == 0 && r < nr) strip_rows[strip * m.per + r] = s[u];
+                    }
+                }
+            }
+            for (int off = L; off < 32; off <<= 1) {
+#pragma unroll
+                for (int i = 0; i < VN; ++i) colacc[i] += __shfl_xor_sync(0xffffffffu, colacc[i], off);
+            }
+            if (live && sub == 0) {
+#pragma unroll
+                for (int i = 0; i < VN; ++i) group_cols[grp * cols + v * VN + i] = colacc[i];
+            }
+        }
+    }
+    __syncthreads();
+    double mine = 0.0;
+    for (int r = tid; r < nr; r += FUSED_THREADS) {
+        float s = 0.0f;
+        for (int q = 0; q < strips; ++q) s += strip_rows[q * m.per + r];
+        const float ra = row_now[r] + (1.0f - a.beta2) * (s / (float)cols);
+        row_avg[r] = ra;
+        row_now[r] = ra;
+        mine += (double)ra;
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, off);
+    if (lane == 0) row_total[2 + warp] = mine;
+    for (int j = tid; j < cols; j += FUSED_THREADS) {
+        double s = 0.0;
+        for (int q = 0; q < groups; ++q) s += (double)group_cols[q * cols + j];
+        col_part[j] = (float)s;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        double s = lane < FUSED_WARPS ? row_total[2 + lane] : 0.0;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        if (lane == 0) row_total[0] = s;
+    }
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();
+    double shares[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) shares[c] = c < C ? ld_cluster_double(cluster_address(row_total, c)) : 0.0;
+    const int32_t own = (cols + C - 1) / C;
+    for (int j = tid; j < cols; j += FUSED_THREADS) {
+        float v[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) v[c] = c < C ? ld_cluster(cluster_address(col_part + j, c)) : 0.0f;
+        double s = 0.0;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) s += (double)v[c];
+        const float ca = col_now[j] + (1.0f - a.beta2) * (float)(s / (double)rows);
+        col_now[j] = root(ca);
+        if (j / own == rank) col_avg[j] = ca;
+    }
+    double total = 0.0;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) total += shares[c];
+    const float rm = (float)(total / (double)rows);
+    const float scale = rm > 0.0f ? a.inv_correction / rm : 0.0f;  // v_hat = row_avg_i * col_avg_j * scale
+    for (int r = tid; r < nr; r += FUSED_THREADS) row_now[r] = root(row_now[r] * scale);
+    __syncthreads();
+    cluster_arrive();  // no more reads of the other CTAs' shared memory
+    if (warp_on) {
+        for (int strip = warp % min(strips, FUSED_WARPS); strip < strips; strip += FUSED_WARPS) {
+            const int v = strip * L + vl;
+            if (v >= nvec) continue;
+            float c[VN];
+#pragma unroll
+            for (int i = 0; i < VN; ++i) c[i] = col_now[v * VN + i];
+            constexpr int UW = 4;
+            for (int rb = grp * side + sub; rb < nr; rb += UW * row_step) {
+                Vec<XT> w[UW], gr[UW];
+#pragma unroll
+                for (int u = 0; u < UW; ++u) {
+                    const int r = rb + u * row_step;
+                    if (r < nr) {
+                        w[u].raw = __ldcs(W + (int64_t)r * nvec + v);
+                        gr[u].raw = __ldcs(G + (int64_t)r * nvec + v);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < UW; ++u) {
+                    const int r = rb + u * row_step;
+                    if (r >= nr) break;
+                    const float rs = row_now[r];
+#pragma unroll
+                    for (int i = 0; i < VN; ++i) w[u].set(i, adam_step(w[u].get(i), gr[u].get(i), a.lr, rs, c[i], a.eps));
+                    __stcs(W + (int64_t)r * nvec + v, w[u].raw);
+                }
+            }
+        }
+    }
+    __syncwarp();
+    cluster_wait();  // this CTA's shared memory is not read any more
+}
+
 // vectors (biases): full second-moment estimate
 template <typename XT>
 __global__ void __launch_bounds__(256) adam_vector_kernel(XT *__restrict__ b, const XT *__restrict__ g, int64_t count,
@@ -223,10 +464,7 @@ __global__ void __launch_bounds__(256) adam_vector_kernel(XT *__restrict__ b, co
     wait_previous_kernel();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= count) return;
-    const float gi = to_f32(g[i]);
-    const float vi = beta2 * v[i] + (1.0f - beta2) * gi * gi;
-    v[i] = vi;
-    b[i] = from_f32<XT>(to_f32(b[i]) - lr * gi / (sqrtf(vi * inv_correction) + eps));  // tiny tensor: exact operations
+    adam_vector_step(b, g, v, i, lr, beta2, inv_correction, eps);
 }
 
 template <typename XT>
@@ -261,6 +499,81 @@ int32_t adam_matrix(XT *W, const XT *g, int32_t n, int32_t rows, int32_t cols, f
     return MOE_OK;
 }
 
+// false: this step is not one for the fused kernel
+template <typename XT>
+bool plan_fused(FusedAdam &a, int32_t n, int32_t d, int32_t h, size_t *smem) {
+    constexpr int VN = 16 / sizeof(XT);
+    const int64_t bytes = (int64_t)d * h * sizeof(XT);
+    if (bytes > FUSED_MATRIX_BYTES) return false;
+    int32_t C = 1;  // slabs as large as that, smaller ones where there are few matrices
+    while (C < 8 && (bytes > C * FUSED_SLAB_BYTES || (2 * (int64_t)n * C < 2 * 148 && bytes > C * (int64_t)32768))) C <<= 1;
+    a.n = n; a.cluster = C;
+    const int32_t shape[2][2] = {{d, h}, {h, d}};
+    int64_t floats = 0;
+    for (int q = 0; q < 2; ++q) {
+        FusedMatrix &m = a.m[q];
+        m.rows = shape[q][0]; m.cols = shape[q][1];
+        const int32_t nvec = m.cols / VN;
+        m.lanes = 1;
+        while (m.lanes < 32 && m.lanes < nvec) m.lanes <<= 1;
+        m.strips = (int32_t)cdiv(nvec, m.lanes);
+        m.groups = m.strips < FUSED_WARPS ? FUSED_WARPS / m.strips : 1;
+        m.per = (int32_t)cdiv(m.rows, C);
+        if (fused_smem_floats(m) > floats) floats = fused_smem_floats(m);
+    }
+    *smem = (2 + FUSED_WARPS) * sizeof(double) + floats * sizeof(float);
+    return *smem <= 100 * 1024 && (2 * (int64_t)n + 64) * C < (int64_t)1 << 31;
+}
+
+template <typename XT>
+int32_t launch_fused(const FusedAdam &a, size_t smem, cudaStream_t st) {
+    static bool configured = false;
+    if (!configured) {
+        MOE_CUDA(cudaFuncSetAttribute(adam_fused_kernel<XT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));
+        configured = true;
+    }
+    const int64_t count = a.v[0].count > a.v[1].count ? a.v[0].count : a.v[1].count;
+    const int64_t vector_clusters = imin(cdiv(count, 2 * FUSED_THREADS * a.cluster), cdiv(2 * 148, a.cluster));
+    cudaLaunchAttribute attrs[2];
+    attrs[0].id = cudaLaunchAttributeClusterDimension;
+    attrs[0].val.clusterDim.x = (unsigned)a.cluster; attrs[0].val.clusterDim.y = 1; attrs[0].val.clusterDim.z = 1;
+    attrs[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // as launch_kernel
+    attrs[1].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((2 * (int64_t)a.n + vector_clusters) * a.cluster)); cfg.blockDim = dim3(FUSED_THREADS);
+    cfg.dynamicSmemBytes = smem; cfg.stream = st; cfg.attrs = attrs; cfg.numAttrs = 2;
+    MOE_CUDA(cudaLaunchKernelEx(&cfg, adam_fused_kernel<XT>, a));
+    MOE_LAUNCHED();
+    return MOE_OK;
+}
+
+template <typename XT>
+int32_t expert_adam(int32_t n, int32_t d, int32_t h, XT *W1, XT *b1, XT *W2, XT *b2, const XT *dW1, const XT *db1, const XT *dW2,
+                    const XT *db2, float *state, float lr, float beta2, float inv_correction, float eps, float *ws, cudaStream_t st) {
+    // state: r1 [n,d], c1 [n,h], r2 [n,h], c2 [n,d], vb1 [n,h], vb2 [n,d]
+    float *r1 = state, *c1 = r1 + (int64_t)n * d, *r2 = c1 + (int64_t)n * h, *c2 = r2 + (int64_t)n * h;
+    float *vb1 = c2 + (int64_t)n * d, *vb2 = vb1 + (int64_t)n * h;
+    FusedAdam a = {};
+    size_t smem = 0;
+    if (plan_fused<XT>(a, n, d, h, &smem)) {
+        a.m[0].W = W1; a.m[0].g = dW1; a.m[0].row_avg = r1; a.m[0].col_avg = c1;
+        a.m[1].W = W2; a.m[1].g = dW2; a.m[1].row_avg = r2; a.m[1].col_avg = c2;
+        a.v[0] = {b1, db1, vb1, (int64_t)n * h};
+        a.v[1] = {b2, db2, vb2, (int64_t)n * d};
+        a.lr = lr; a.beta2 = beta2; a.inv_correction = inv_correction; a.eps = eps;
+        return launch_fused<XT>(a, smem, st);
+    }
+    float *row_mean = ws, *colpart = ws + ((n + 63) & ~63);
+    const unsigned gb1 = (unsigned)cdiv((int64_t)n * h, 256), gb2 = (unsigned)cdiv((int64_t)n * d, 256);
+    MOE_TRY(adam_matrix<XT>(W1, dW1, n, d, h, r1, c1, lr, beta2, inv_correction, eps, colpart, row_mean, st));
+    MOE_TRY(adam_matrix<XT>(W2, dW2, n, h, d, r2, c2, lr, beta2, inv_correction, eps, colpart, row_mean, st));
+    launch_kernel(adam_vector_kernel<XT>, gb1, 256, 0, st, b1, db1, (int64_t)n * h, vb1, lr, beta2, inv_correction, eps);
+    MOE_LAUNCHED();
+    launch_kernel(adam_vector_kernel<XT>, gb2, 256, 0, st, b2, db2, (int64_t)n * d, vb2, lr, beta2, inv_correction, eps);
+    MOE_LAUNCHED();
+    return MOE_OK;
+}
+
 }  // namespace
 
 int64_t adam_ws_floats(int32_t n, int32_t d, int32_t h) {
@@ -271,28 +584,12 @@ int64_t adam_ws_floats(int32_t n, int32_t d, int32_t h) {
 int32_t launch_expert_adam(int32_t act, int32_t n, int32_t d, int32_t h, void *W1, void *b1, void *W2, void *b2,
                            const void *dW1, const void *db1, const void *dW2, const void *db2, float *state, float lr,
                            float beta2, float eps, int32_t step, float *ws, cudaStream_t st) {
-    // state: r1 [n,d], c1 [n,h], r2 [n,h], c2 [n,d], vb1 [n,h], vb2 [n,d]
-    float *r1 = state, *c1 = r1 + (int64_t)n * d, *r2 = c1 + (int64_t)n * h, *c2 = r2 + (int64_t)n * h;
-    float *vb1 = c2 + (int64_t)n * d, *vb2 = vb1 + (int64_t)n * h;
-    float *row_mean = ws, *colpart = ws + ((n + 63) & ~63);
     const float inv_correction = (float)(1.0 / (1.0 - pow((double)beta2, (double)step)));
-    const unsigned gb1 = (unsigned)cdiv((int64_t)n * h, 256), gb2 = (unsigned)cdiv((int64_t)n * d, 256);
-    if (act == MOE_BF16) {
-        MOE_TRY(adam_matrix<bf16>((bf16 *)W1, (const bf16 *)dW1, n, d, h, r1, c1, lr, beta2, inv_correction, eps, colpart, row_mean, st));
-        MOE_TRY(adam_matrix<bf16>((bf16 *)W2, (const bf16 *)dW2, n, h, d, r2, c2, lr, beta2, inv_correction, eps, colpart, row_mean, st));
-        launch_kernel(adam_vector_kernel<bf16>, gb1, 256, 0, st, (bf16 *)b1, (const bf16 *)db1, (int64_t)n * h, vb1, lr, beta2, inv_correction, eps);
-        MOE_LAUNCHED();
-        launch_kernel(adam_vector_kernel<bf16>, gb2, 256, 0, st, (bf16 *)b2, (const bf16 *)db2, (int64_t)n * d, vb2, lr, beta2, inv_correction, eps);
-        MOE_LAUNCHED();
-    } else {
-        MOE_TRY(adam_matrix<float>((float *)W1, (const float *)dW1, n, d, h, r1, c1, lr, beta2, inv_correction, eps, colpart, row_mean, st));
-        MOE_TRY(adam_matrix<float>((float *)W2, (const float *)dW2, n, h, d, r2, c2, lr, beta2, inv_correction, eps, colpart, row_mean, st));
-        launch_kernel(adam_vector_kernel<float>, gb1, 256, 0, st, (float *)b1, (const float *)db1, (int64_t)n * h, vb1, lr, beta2, inv_correction, eps);
-        MOE_LAUNCHED();
-        launch_kernel(adam_vector_kernel<float>, gb2, 256, 0, st, (float *)b2, (const float *)db2, (int64_t)n * d, vb2, lr, beta2, inv_correction, eps);
-        MOE_LAUNCHED();
-    }
-    return MOE_OK;
+    if (act == MOE_BF16)
+        return expert_adam<bf16>(n, d, h, (bf16 *)W1, (bf16 *)b1, (bf16 *)W2, (bf16 *)b2, (const bf16 *)dW1, (const bf16 *)db1,
+                                 (const bf16 *)dW2, (const bf16 *)db2, state, lr, beta2, inv_correction, eps, ws, st);
+    return expert_adam<float>(n, d, h, (float *)W1, (float *)b1, (float *)W2, (float *)b2, (const float *)dW1, (const float *)db1,
+                              (const float *)dW2, (const float *)db2, state, lr, beta2, inv_correction, eps, ws, st);
 }
 
 }  // namespace moe
