@@ -12,10 +12,8 @@ namespace moe {
 
 namespace {
 
-// p = softmax(c) per row: exponentials and their sum in double (largest logit subtracted), one rounding to float.
-// NV > 0: a row of at most 32 * NV columns stays in registers with its exponentials (the double exponential is what bounds this
-// kernel: 43 us when each was evaluated twice, 32768 x 256); NV = 0: any width, evaluated again.
-template <int NV>
+// p = softmax(c) per row: exponentials and their sum in double (largest logit subtracted), one rounding to float. The double
+// exponential is what bounds it: rows of up to 256 columns keep theirs in registers (below), this kernel evaluates each twice.
 __global__ void __launch_bounds__(256) bal_softmax_kernel(const float *__restrict__ c, int64_t T, int32_t n,
                                                           float *__restrict__ p) {
     wait_previous_kernel();
@@ -24,37 +22,14 @@ __global__ void __launch_bounds__(256) bal_softmax_kernel(const float *__restric
     if (t >= T) return;
     const float *row = c + t * n;
     float mx = -CUDART_INF_F;
-    float v[NV > 0 ? NV : 1];
-    if (NV > 0) {
-#pragma unroll
-        for (int u = 0; u < NV; ++u) v[u] = lane + 32 * u < n ? row[lane + 32 * u] : -CUDART_INF_F;
-#pragma unroll
-        for (int u = 0; u < NV; ++u) mx = fmaxf(mx, v[u]);
-    } else {
-        for (int32_t j = lane; j < n; j += 32) mx = fmaxf(mx, row[j]);
-    }
+    for (int32_t j = lane; j < n; j += 32) mx = fmaxf(mx, row[j]);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
     double s = 0.0;
-    double e[NV > 0 ? NV : 1];
-    if (NV > 0) {
-#pragma unroll
-        for (int u = 0; u < NV; ++u) {
-            e[u] = lane + 32 * u < n ? exp((double)v[u] - (double)mx) : 0.0;
-            s += e[u];
-        }
-    } else {
-        for (int32_t j = lane; j < n; j += 32) s += exp((double)row[j] - (double)mx);
-    }
+    for (int32_t j = lane; j < n; j += 32) s += exp((double)row[j] - (double)mx);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    if (NV > 0) {
-#pragma unroll
-        for (int u = 0; u < NV; ++u)
-            if (lane + 32 * u < n) p[t * n + lane + 32 * u] = (float)(e[u] / s);
-    } else {
-        for (int32_t j = lane; j < n; j += 32) p[t * n + j] = (float)(exp((double)row[j] - (double)mx) / s);
-    }
+    for (int32_t j = lane; j < n; j += 32) p[t * n + j] = (float)(exp((double)row[j] - (double)mx) / s);
 }
 
 // out [cols, rows] = in [rows, cols]^T, 32 x 32 tiles
@@ -72,103 +47,153 @@ __global__ void __launch_bounds__(256) bal_transpose_kernel(const float *__restr
         if (c0 + i < cols && r0 + tx < rows) out[(int64_t)(c0 + i) * rows + r0 + tx] = tile[tx][i];
 }
 
+// Softmax of rows of at most 32 * NV columns, and p^T [n, T] with it: a block takes 32 tokens, two per warp, and writes the
+// transposed values from shared memory, 128 bytes of a column at a time (a transposing pass of its own read and wrote p again:
+// 18 us of 48 for both, 32768 x 256).
+template <int NV>
+__global__ void __launch_bounds__(512) bal_softmax_both_kernel(const float *__restrict__ c, int64_t T, int32_t n,
+                                                               float *__restrict__ p, float *__restrict__ pT) {
+    wait_previous_kernel();
+    __shared__ float tile[32][32 * NV + 1];
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    const int64_t t0 = (int64_t)blockIdx.x * 32;
+    float v[2][NV];
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int u = 0; u < NV; ++u) {
+            const int64_t t = t0 + 2 * wp + q;
+            v[q][u] = t < T && lane + 32 * u < n ? c[t * n + lane + 32 * u] : -CUDART_INF_F;
+        }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int64_t t = t0 + 2 * wp + q;
+        if (t >= T) break;
+        float mx = -CUDART_INF_F;
+#pragma unroll
+        for (int u = 0; u < NV; ++u) mx = fmaxf(mx, v[q][u]);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+        double s = 0.0, e[NV];
+#pragma unroll
+        for (int u = 0; u < NV; ++u) {
+            e[u] = lane + 32 * u < n ? exp((double)v[q][u] - (double)mx) : 0.0;
+            s += e[u];
+        }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+#pragma unroll
+        for (int u = 0; u < NV; ++u)
+            if (lane + 32 * u < n) {
+                const float f = (float)(e[u] / s);
+                p[t * n + lane + 32 * u] = f;
+                tile[2 * wp + q][lane + 32 * u] = f;
+            }
+    }
+    __syncthreads();
+    if (t0 + lane < T)
+        for (int32_t j = wp; j < n; j += 16) pT[(int64_t)j * T + t0 + lane] = tile[lane][j];
+}
+
 // Batchwise mask of one expert (block = column i of p, given transposed: col [T]): the m largest values, equal values to
 // the lower token. Radix select of the m-th largest key (the bit patterns of non-negative floats order like the
 // values), then an order-preserving compaction: tok_of_row[i * m + q] = q-th kept token, and the expert's bit is set
-// in the token's mask words. What bounds it is the latency of six sweeps over the column, so every sweep keeps eight loads
-// per thread in flight; a warp owns a contiguous run of tokens in the compaction, so that its place in the list needs one
-// scan over the warps. (One load at a time, a serial digit search and four barriers per 1024 tokens: 90 us at 32768 x 256.)
-constexpr int SEL_BATCH = 8;
-__global__ void __launch_bounds__(1024) bal_select_kernel(const float *__restrict__ pT, int64_t T, int32_t n, int32_t m,
+// in the token's mask words. A warp owns a contiguous run of tokens, so that its place in the list needs one scan over the
+// warps. NK > 0: up to 1024 * NK keys stay in registers and the column is read once; NK = 0: any length, one sweep per digit
+// and two for the compaction, eight loads per thread in flight. Three digits of 11, 11 and 10 bits: the first one holds the exponent
+// and two bits of the mantissa, so that the lanes' additions to its few counters collide less (four digits of 8 bits and a sweep
+// each: 62 us at 32768 x 256).
+constexpr int SEL_BATCH = 8, SEL_BINS = 2048;
+template <int NK>
+__global__ void __launch_bounds__(1024, NK > 8 ? 1 : 2) bal_select_kernel(const float *__restrict__ pT, int64_t T, int32_t n, int32_t m,
                                                           int32_t words, int32_t *__restrict__ tok_of_row,
                                                           uint32_t *__restrict__ mask_bits) {
     wait_previous_kernel();
-    __shared__ int32_t hist[256];
+    __shared__ int32_t hist[SEL_BINS];
     __shared__ int32_t warp_gt[32], warp_eq[32];
     __shared__ uint32_t s_prefix;
     __shared__ int32_t s_need;
+    constexpr int NB = NK > 0 ? NK : SEL_BATCH;
     const int32_t i = blockIdx.x;
     const uint32_t *col = reinterpret_cast<const uint32_t *>(pT + (int64_t)i * T);
     const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
+    const int64_t run = ((T + 31) / 32 + 31) / 32 * 32, t_first = wp * run, t_last = min(T, t_first + run);
+    uint32_t key[NB];
+    // f(token of this lane, key, inside the run) for the warp's run in ascending order; all lanes take part
+    auto load = [&](int64_t t00) {
+#pragma unroll
+        for (int u = 0; u < NB; ++u) key[u] = t00 + 32 * u + lane < t_last ? col[t00 + 32 * u + lane] : 0u;
+    };
+    auto sweep = [&](auto f) {
+        for (int64_t t00 = t_first; t00 < t_last; t00 += 32 * NB) {
+            if (NK == 0) load(t00);
+#pragma unroll
+            for (int u = 0; u < NB; ++u) {
+                const int64_t t = t00 + 32 * u + lane;
+                f(t, key[u], t < t_last);
+            }
+        }
+    };
+    if (NK > 0) load(t_first);
     if (tid == 0) { s_prefix = 0u; s_need = m; }
     uint32_t known = 0u;  // mask of the key bits fixed so far
-    for (int shift = 24; shift >= 0; shift -= 8) {
-        if (tid < 256) hist[tid] = 0;
+#pragma unroll
+    for (int digit = 0; digit < 3; ++digit) {
+        const int shift = digit == 0 ? 21 : digit == 1 ? 10 : 0;
+        const uint32_t bins = digit == 2 ? 1024u : 2048u;
+        hist[tid] = 0; hist[tid + 1024] = 0;
         __syncthreads();
         const uint32_t prefix = s_prefix;
-        for (int64_t t0 = tid; t0 < T; t0 += 1024 * SEL_BATCH) {
-            uint32_t key[SEL_BATCH];
-#pragma unroll
-            for (int u = 0; u < SEL_BATCH; ++u) key[u] = t0 + 1024 * u < T ? col[t0 + 1024 * u] : 0u;
-#pragma unroll
-            for (int u = 0; u < SEL_BATCH; ++u)
-                if (t0 + 1024 * u < T && (key[u] & known) == prefix) atomicAdd(&hist[(key[u] >> shift) & 0xFFu], 1);
-        }
+        sweep([&](int64_t, uint32_t k, bool in) {
+            if (in && (k & known) == prefix) atomicAdd(&hist[(k >> shift) & (bins - 1u)], 1);
+        });
         __syncthreads();
-        if (wp == 0) {  // the digit that holds the need-th largest key: lane l holds the digits 255 - 8 l .. 248 - 8 l
-            const int32_t need = s_need;
-            int32_t h[8], sum = 0;
+        // the digit that holds the need-th largest key: thread tid holds the digits 2047 - 2 tid and the one below
+        const int32_t need = s_need, h0 = hist[SEL_BINS - 1 - 2 * tid], h1 = hist[SEL_BINS - 2 - 2 * tid];
+        int32_t inc = h0 + h1;
 #pragma unroll
-            for (int q = 0; q < 8; ++q) { h[q] = hist[255 - 8 * lane - q]; sum += h[q]; }
-            int32_t inc = sum;
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const int32_t o = __shfl_up_sync(0xffffffffu, inc, off);
-                if (lane >= off) inc += o;
-            }
-            int32_t before = inc - sum;  // keys with a larger digit than this lane's first
-            if (before < need && need <= inc) {
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    if (before < need && need <= before + h[q]) {
-                        s_need = need - before;
-                        s_prefix = prefix | ((uint32_t)(255 - 8 * lane - q) << shift);
-                    }
-                    before += h[q];
-                }
-            }
+        for (int off = 1; off < 32; off <<= 1) {
+            const int32_t o = __shfl_up_sync(0xffffffffu, inc, off);
+            if (lane >= off) inc += o;
         }
-        known |= 0xFFu << shift;
+        if (lane == 31) warp_gt[wp] = inc;
+        __syncthreads();
+        const int32_t before = __reduce_add_sync(0xffffffffu, lane < wp ? warp_gt[lane] : 0) + inc - h0 - h1;  // keys with a larger digit
+        if (before < need && need <= before + h0) {
+            s_need = need - before;
+            s_prefix = prefix | ((uint32_t)(SEL_BINS - 1 - 2 * tid) << shift);
+        } else if (before + h0 < need && need <= before + h0 + h1) {
+            s_need = need - before - h0;
+            s_prefix = prefix | ((uint32_t)(SEL_BINS - 2 - 2 * tid) << shift);
+        }
+        known |= (bins - 1u) << shift;
         __syncthreads();
     }
     const uint32_t kth = s_prefix;    // the m-th largest key
     const int32_t take_eq = s_need;   // how many of the keys equal to it are kept (the first ones in token order)
-    const int64_t run = ((T + 31) / 32 + 31) / 32 * 32, t_first = wp * run, t_last = min(T, t_first + run);
     int32_t gt = 0, eq = 0;
-    for (int64_t t0 = t_first + lane; t0 < t_last; t0 += 32 * SEL_BATCH) {
-        uint32_t key[SEL_BATCH];
-#pragma unroll
-        for (int u = 0; u < SEL_BATCH; ++u) key[u] = t0 + 32 * u < t_last ? col[t0 + 32 * u] : 0u;
-#pragma unroll
-        for (int u = 0; u < SEL_BATCH; ++u)
-            if (t0 + 32 * u < t_last) { gt += key[u] > kth; eq += key[u] == kth; }
-    }
+    sweep([&](int64_t, uint32_t k, bool in) {
+        if (in) { gt += k > kth; eq += k == kth; }
+    });
     gt = __reduce_add_sync(0xffffffffu, gt);
     eq = __reduce_add_sync(0xffffffffu, eq);
     if (lane == 0) { warp_gt[wp] = gt; warp_eq[wp] = eq; }
     __syncthreads();
     int32_t eq_base = __reduce_add_sync(0xffffffffu, lane < wp ? warp_eq[lane] : 0);  // in the warps before
     int32_t pos = __reduce_add_sync(0xffffffffu, lane < wp ? warp_gt[lane] : 0) + min(eq_base, take_eq);
-    for (int64_t t00 = t_first; t00 < t_last; t00 += 32 * SEL_BATCH) {
-        uint32_t key[SEL_BATCH];
-#pragma unroll
-        for (int u = 0; u < SEL_BATCH; ++u) key[u] = t00 + 32 * u + lane < t_last ? col[t00 + 32 * u + lane] : 0u;
-#pragma unroll
-        for (int u = 0; u < SEL_BATCH; ++u) {
-            const int64_t t = t00 + 32 * u + lane;
-            const bool is_eq = t < t_last && key[u] == kth;
-            const uint32_t below = (1u << lane) - 1u, b_eq = __ballot_sync(0xffffffffu, is_eq);
-            const bool keep = (t < t_last && key[u] > kth) || (is_eq && eq_base + __popc(b_eq & below) < take_eq);
-            const uint32_t b_keep = __ballot_sync(0xffffffffu, keep);
-            const int32_t at = pos + __popc(b_keep & below);
-            if (keep && at < m) {  // at < m always: exactly m keys are kept
-                tok_of_row[(int64_t)i * m + at] = (int32_t)t;
-                atomicOr(&mask_bits[t * words + (i >> 5)], 1u << (i & 31));
-            }
-            eq_base += __popc(b_eq);
-            pos += __popc(b_keep);
+    sweep([&](int64_t t, uint32_t k, bool in) {
+        const bool is_eq = in && k == kth;
+        const uint32_t below = (1u << lane) - 1u, b_eq = __ballot_sync(0xffffffffu, is_eq);
+        const bool keep = (in && k > kth) || (is_eq && eq_base + __popc(b_eq & below) < take_eq);
+        const uint32_t b_keep = __ballot_sync(0xffffffffu, keep);
+        const int32_t at = pos + __popc(b_keep & below);
+        if (keep && at < m) {  // at < m always: exactly m keys are kept
+            tok_of_row[(int64_t)i * m + at] = (int32_t)t;
+            atomicOr(&mask_bits[t * words + (i >> 5)], 1u << (i & 31));
         }
-    }
+        eq_base += __popc(b_eq);
+        pos += __popc(b_keep);
+    });
 }
 
 // Per token (one warp): den = sum of p over the kept experts, cnt = how many keep it, the token's part of L_batchwise
@@ -294,7 +319,42 @@ __global__ void __launch_bounds__(256) bal_gather_kernel(const XT *__restrict__ 
     }
 }
 
-// y[t] = sum over the rows of token t (ascending expert) of p[t, e] / den[t] * ys[row]   (Eq. 1 with the gates of Eq. 16)
+// Rows of token t that a lane holds for its warp: entry j of the list in lane j (the first 32 entries; `first` moves on). A row
+// outside [0, R) is -1 and contributes nothing.
+__device__ __forceinline__ int32_t token_row(const int32_t *tok_rows, int32_t first, int32_t j1, int64_t R, int lane) {
+    const int32_t r = first + lane < j1 ? tok_rows[first + lane] : -1;
+    return (uint32_t)r < (uint32_t)R ? r : -1;
+}
+
+// A warp's walk over tokens t, t + step, ...: the next token's list is fetched while the rows of this one move, and the bounds of the
+// list after it (the numbers of a token's rows, their gates and the rows are three loads one behind the other).
+struct TokenWalk {
+    const int32_t *tok_ptr, *tok_rows;
+    int64_t T, R, t, step;
+    int32_t j0, j1, n0, n1, row;  // this token's list, the next one's, this lane's entry of this one's
+    int lane;
+    __device__ __forceinline__ TokenWalk(const int32_t *tok_ptr_, const int32_t *tok_rows_, int64_t T_, int64_t R_, int lane_)
+        : tok_ptr(tok_ptr_), tok_rows(tok_rows_), T(T_), R(R_), t((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)),
+          step((int64_t)gridDim.x * 8), j0(0), j1(0), n0(0), n1(0), row(-1), lane(lane_) {
+        if (t < T) { j0 = tok_ptr[t]; j1 = tok_ptr[t + 1]; }
+        bounds();
+        row = token_row(tok_rows, j0, j1, R, lane);
+    }
+    __device__ __forceinline__ void bounds() {
+        n0 = n1 = 0;
+        if (t + step < T) { n0 = tok_ptr[t + step]; n1 = tok_ptr[t + step + 1]; }
+    }
+    __device__ __forceinline__ int32_t next_row() const { return token_row(tok_rows, n0, n1, R, lane); }
+    __device__ __forceinline__ void advance(int32_t row_) {
+        t += step;
+        j0 = n0; j1 = n1; row = row_;
+        bounds();
+    }
+};
+
+// y[t] = sum over the rows of token t (ascending expert) of p[t, e] / den[t] * ys[row]   (Eq. 1 with the gates of Eq. 16).
+// One warp per token, a vector of four rows in flight per lane (one row after the other, each behind the load of its number: 74 us
+// at 32768 tokens x 512 with four rows each, this way 58; the adjoints below, with the same walk, lost what it took in registers).
 template <typename XT>
 __global__ void __launch_bounds__(256) bal_combine_kernel(const XT *__restrict__ ys, const float *__restrict__ p,
                                                           const float *__restrict__ den, const int32_t *__restrict__ tok_ptr,
@@ -303,28 +363,50 @@ __global__ void __launch_bounds__(256) bal_combine_kernel(const XT *__restrict__
     wait_previous_kernel();
     constexpr int VN = V16<XT>::N;
     const int lane = threadIdx.x & 31;
-    const int64_t t = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (t >= T) return;
-    const int32_t j0 = tok_ptr[t], j1 = tok_ptr[t + 1];
-    const float dn = den[t];
     const int nvec = d / VN;
-    for (int v = lane; v < nvec; v += 32) {
-        float acc[VN];
+    for (TokenWalk w(tok_ptr, tok_rows, T, R, lane); w.t < T;) {
+        const int32_t next = w.next_row();
+        const float dn = den[w.t];
+        const float gate0 = w.row >= 0 ? p[w.t * n + w.row / m] / dn : 0.0f;
+        for (int v = lane; v - lane < nvec; v += 32) {
+            float acc[VN];
 #pragma unroll
-        for (int i = 0; i < VN; ++i) acc[i] = 0.0f;
-        for (int32_t j = j0; j < j1; ++j) {
-            const int32_t r = tok_rows[j];
-            if ((uint32_t)r >= (uint32_t)R) continue;
-            const float g = p[t * n + r / m] / dn;
-            V16<XT> in;
-            in.raw = reinterpret_cast<const uint4 *>(ys + (int64_t)r * d)[v];
+            for (int i = 0; i < VN; ++i) acc[i] = 0.0f;
+            int32_t row = w.row;
+            float gate = gate0;
+            for (int32_t first = w.j0; first < w.j1; first += 32) {
+                if (first > w.j0) {  // lists of more than 32 rows
+                    row = token_row(tok_rows, first, w.j1, R, lane);
+                    gate = row >= 0 ? p[w.t * n + row / m] / dn : 0.0f;
+                }
+                const int count = min(32, w.j1 - first);
+                for (int q0 = 0; q0 < count; q0 += 4) {
+                    V16<XT> in[4];
+                    int32_t r[4];
 #pragma unroll
-            for (int i = 0; i < VN; ++i) acc[i] = fmaf(g, in.get(i), acc[i]);
+                    for (int q = 0; q < 4; ++q) {
+                        r[q] = __shfl_sync(0xffffffffu, row, (q0 + q) & 31);
+                        if (q0 + q >= count) r[q] = -1;
+                        if (r[q] >= 0 && v < nvec) in[q].raw = reinterpret_cast<const uint4 *>(ys + (int64_t)r[q] * d)[v];
+                    }
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float g = __shfl_sync(0xffffffffu, gate, (q0 + q) & 31);
+                        if (r[q] >= 0) {
+#pragma unroll
+                            for (int i = 0; i < VN; ++i) acc[i] = fmaf(g, in[q].get(i), acc[i]);
+                        }
+                    }
+                }
+            }
+            if (v < nvec) {
+                V16<XT> out;
+#pragma unroll
+                for (int i = 0; i < VN; ++i) out.set(i, acc[i]);
+                reinterpret_cast<uint4 *>(y + w.t * d)[v] = out.raw;
+            }
         }
-        V16<XT> out;
-#pragma unroll
-        for (int i = 0; i < VN; ++i) out.set(i, acc[i]);
-        reinterpret_cast<uint4 *>(y + t * d)[v] = out.raw;
+        w.advance(next);
     }
 }
 
@@ -413,6 +495,79 @@ __global__ void __launch_bounds__(256) bal_gate_bwd_kernel(const float *__restri
     }
 }
 
+// The same for the tensor-core path and at most 64 * NP columns (n even): a lane owns pairs of adjacent columns, reads the row once
+// and keeps it, with the gradients of the kept ones, in registers, and the three bf16 terms of a pair leave as 4-byte stores
+// (three walks over the row, each behind its own loads: 85 us at 32768 x 256).
+template <int NP>
+__global__ void __launch_bounds__(256) bal_gate_bwd_pairs_kernel(const float *__restrict__ p, const uint32_t *__restrict__ mask_bits,
+                                                                 const float *__restrict__ den, const float *__restrict__ thr,
+                                                                 const int32_t *__restrict__ tok_ptr,
+                                                                 const int32_t *__restrict__ tok_rows,
+                                                                 const float *__restrict__ dG_row, float w, int64_t T, int32_t n,
+                                                                 int32_t words, bf16 *__restrict__ dsplit) {
+    wait_previous_kernel();
+    const int lane = threadIdx.x & 31;
+    const int64_t t = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (t >= T) return;
+    const int32_t j0 = tok_ptr[t];
+    const double dn = (double)den[t];
+    const uint32_t mine = lane < words ? mask_bits[t * words + lane] : 0u;  // word `lane` of the token's mask
+    float2 pv[NP], tv[NP];
+#pragma unroll
+    for (int u = 0; u < NP; ++u) {
+        const int32_t j = 2 * lane + 64 * u;
+        pv[u] = j < n ? *reinterpret_cast<const float2 *>(p + t * n + j) : make_float2(0.0f, 0.0f);
+        tv[u] = j < n ? *reinterpret_cast<const float2 *>(thr + j) : make_float2(0.0f, 0.0f);
+    }
+    float dg[2 * NP];
+    bool kept[2 * NP];
+    int32_t rank0 = 0;  // kept experts in the words before
+#pragma unroll
+    for (int u = 0; u < NP; ++u) {
+        const uint32_t w0 = __shfl_sync(0xffffffffu, mine, 2 * u), w1 = __shfl_sync(0xffffffffu, mine, 2 * u + 1);
+        const uint32_t word = lane < 16 ? w0 : w1;
+        const int bit = (2 * lane) & 31;
+        int32_t rank = rank0 + (lane < 16 ? 0 : __popc(w0)) + __popc(word & ((1u << bit) - 1u));
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            kept[2 * u + h] = (word >> (bit + h)) & 1u;
+            dg[2 * u + h] = kept[2 * u + h] ? dG_row[tok_rows[j0 + rank]] : 0.0f;
+            rank += kept[2 * u + h];
+        }
+        rank0 += __popc(w0) + __popc(w1);
+    }
+    auto value = [](const float2 &v, int h) { return h ? v.y : v.x; };
+    double inner = 0.0;  // sum over the kept experts of G * dG
+#pragma unroll
+    for (int q = 0; q < 2 * NP; ++q)
+        if (kept[q]) inner += (double)value(pv[q >> 1], q & 1) / dn * (double)dg[q];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) inner += __shfl_xor_sync(0xffffffffu, inner, off);
+    double dp[2 * NP], s2 = 0.0;
+#pragma unroll
+    for (int q = 0; q < 2 * NP; ++q) {
+        const float pj = value(pv[q >> 1], q & 1);
+        dp[q] = (double)w * ((pj > value(tv[q >> 1], q & 1) ? 1.0 : 0.0) - (kept[q] ? 1.0 : 0.0));
+        if (kept[q]) dp[q] += ((double)dg[q] - inner) / dn;
+        s2 += dp[q] * (double)pj;  // columns behind the row: p = 0
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, off);
+    bf16 *row = dsplit + t * 3 * n;  // three bf16 terms carry the 24 mantissa bits: [T, 3n] = (hi | mid | lo)
+#pragma unroll
+    for (int u = 0; u < NP; ++u) {
+        const int32_t j = 2 * lane + 64 * u;
+        if (j >= n) continue;
+        float v0 = (float)((double)pv[u].x * (dp[2 * u] - s2)), v1 = (float)((double)pv[u].y * (dp[2 * u + 1] - s2));
+#pragma unroll
+        for (int term = 0; term < 3; ++term) {
+            const __nv_bfloat162 h = __floats2bfloat162_rn(v0, v1);
+            *reinterpret_cast<__nv_bfloat162 *>(row + term * n + j) = h;
+            v0 -= __bfloat162float(h.x); v1 -= __bfloat162float(h.y);
+        }
+    }
+}
+
 __global__ void bal_dthr_kernel(const int32_t *__restrict__ thr_counts, int32_t n, int32_t m, float w,
                                 float *__restrict__ dthr) {
     wait_previous_kernel();
@@ -482,13 +637,19 @@ int32_t launch_balanced_gate(const void *x, int32_t act, int64_t T, int32_t d, i
     }
     // logits by the fixed fma chain (one matrix: the projection kernel's second one is absent)
     MOE_TRY(launch_projection(x, act, T, d, n, Wg, nullptr, logits, nullptr, nullptr, 0, nullptr, 1, nullptr, st));
-    if (n <= 128) launch_kernel(bal_softmax_kernel<4>, (unsigned)cdiv(T, 8), 256, 0, st, logits, T, n, probs);
-    else if (n <= 256) launch_kernel(bal_softmax_kernel<8>, (unsigned)cdiv(T, 8), 256, 0, st, logits, T, n, probs);
-    else launch_kernel(bal_softmax_kernel<0>, (unsigned)cdiv(T, 8), 256, 0, st, logits, T, n, probs);
+    const unsigned both = (unsigned)cdiv(T, 32);
+    if (n <= 64) launch_kernel(bal_softmax_both_kernel<2>, both, 512, 0, st, logits, T, n, probs, pT);
+    else if (n <= 128) launch_kernel(bal_softmax_both_kernel<4>, both, 512, 0, st, logits, T, n, probs, pT);
+    else if (n <= 256) launch_kernel(bal_softmax_both_kernel<8>, both, 512, 0, st, logits, T, n, probs, pT);
+    else {
+        launch_kernel(bal_softmax_kernel, (unsigned)cdiv(T, 8), 256, 0, st, logits, T, n, probs);
+        MOE_LAUNCHED();
+        launch_kernel(bal_transpose_kernel, dim3((unsigned)cdiv(T, 32), (unsigned)cdiv(n, 32)), 256, 0, st, probs, T, n, pT);
+    }
     MOE_LAUNCHED();
-    launch_kernel(bal_transpose_kernel, dim3((unsigned)cdiv(T, 32), (unsigned)cdiv(n, 32)), 256, 0, st, probs, T, n, pT);
-    MOE_LAUNCHED();
-    launch_kernel(bal_select_kernel, (unsigned)n, 1024, 0, st, pT, T, n, m, words, tok_of_row, mask_bits);
+    if (T <= 8 * 1024) launch_kernel(bal_select_kernel<8>, (unsigned)n, 1024, 0, st, pT, T, n, m, words, tok_of_row, mask_bits);
+    else if (T <= 32 * 1024) launch_kernel(bal_select_kernel<32>, (unsigned)n, 1024, 0, st, pT, T, n, m, words, tok_of_row, mask_bits);
+    else launch_kernel(bal_select_kernel<0>, (unsigned)n, 1024, 0, st, pT, T, n, m, words, tok_of_row, mask_bits);
     MOE_LAUNCHED();
     const int32_t per_warp = tokens_per_warp(T);
     const int64_t tok_blocks = cdiv(T, 8 * per_warp);
@@ -518,9 +679,9 @@ int32_t launch_balanced_combine(const void *ys, int32_t act, const float *p, con
                                 cudaStream_t st) {
     if (T == 0) return MOE_OK;
     if (act == MOE_BF16)
-        launch_kernel(bal_combine_kernel<bf16>, (unsigned)cdiv(T, 8), 256, 0, st, (const bf16 *)ys, p, den, tok_ptr, tok_rows, T, R, n, m, d, (bf16 *)y);
+        launch_kernel(bal_combine_kernel<bf16>, (unsigned)imin(cdiv(T, 8), 148 * 8), 256, 0, st, (const bf16 *)ys, p, den, tok_ptr, tok_rows, T, R, n, m, d, (bf16 *)y);
     else
-        launch_kernel(bal_combine_kernel<float>, (unsigned)cdiv(T, 8), 256, 0, st, (const float *)ys, p, den, tok_ptr, tok_rows, T, R, n, m, d, (float *)y);
+        launch_kernel(bal_combine_kernel<float>, (unsigned)imin(cdiv(T, 8), 148 * 8), 256, 0, st, (const float *)ys, p, den, tok_ptr, tok_rows, T, R, n, m, d, (float *)y);
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -542,7 +703,15 @@ int32_t launch_balanced_gate_bwd(const float *p, const uint32_t *mask_bits, cons
                                  const int32_t *thr_counts, float w, int64_t T, int32_t n, int32_t m, float *dc,
                                  void *dsplit, float *dthr, cudaStream_t st) {
     const int32_t words = (n + 31) / 32;
-    if (T > 0) {
+    if (T > 0 && dsplit && n % 2 == 0 && n <= 256) {
+        if (n <= 64)
+            launch_kernel(bal_gate_bwd_pairs_kernel<1>, (unsigned)cdiv(T, 8), 256, 0, st, p, mask_bits, den, thr, tok_ptr, tok_rows, dG_row, w, T, n,
+                          words, (bf16 *)dsplit);
+        else
+            launch_kernel(bal_gate_bwd_pairs_kernel<4>, (unsigned)cdiv(T, 8), 256, 0, st, p, mask_bits, den, thr, tok_ptr, tok_rows, dG_row, w, T, n,
+                          words, (bf16 *)dsplit);
+        MOE_LAUNCHED();
+    } else if (T > 0) {
         launch_kernel(bal_gate_bwd_kernel, (unsigned)cdiv(T, 8), 256, 0, st, p, mask_bits, den, thr, tok_ptr, tok_rows, dG_row, w, T, n, m, words, dc,
                                                                   (bf16 *)dsplit);
         MOE_LAUNCHED();
