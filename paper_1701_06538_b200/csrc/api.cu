@@ -180,6 +180,7 @@ SegmentPlan make_plan(const moe_config *c, const Dims &D, int32_t *ws, bool back
         p.bm[0] = 64; p.bm[1] = 32; p.bm[2] = 16;
         if (backward) p.bm[3] = COLSUM_ROWS;
         p.info = p.sched = nullptr;
+        p.maps = nullptr;
     }
     return p;
 }
@@ -447,7 +448,12 @@ int32_t do_expert_ffn(const moe_config *c, const Dims &D, const void *xs, const 
     if (!hid) return MOE_ERR_INVALID_ARG;
     if (hid_used) *hid_used = hid;
     const SegmentPlan plan = ready ? *ready : make_plan(c, D, w.plan, false);
-    if (!ready) MOE_TRY(launch_segment_plan(plan, offsets, (int32_t)D.n, D.R, clear, st));
+    if (!ready) {
+        SegmentMaps maps;
+        const bool tc = tc_ffn_supported(*c);
+        if (tc) MOE_TRY(tc_segment_maps(*c, &maps, xs, hid, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr));
+        MOE_TRY(launch_segment_plan(plan, offsets, (int32_t)D.n, D.R, clear, st, tc ? &maps : nullptr));
+    }
     if (tc_ffn_supported(*c))
         return launch_tc_ffn(*c, xs, offsets, W1, b1, W2, b2, hid, ys, plan, status_word(ws_base), st, first_only, relu_bits);
     SimtGemm g = base_gemm(D);  // hid = relu(xs.W1 + b1)
@@ -531,7 +537,14 @@ int32_t expert_ffn_bwd_stage(const moe_config *c, const Dims &D, const void *xs,
                              const int32_t *offsets, const void *W1, const void *W2, void *dxs, void *dW1, void *db1, void *dW2,
                              void *db2, void *ws, Carver &cv, cudaStream_t st, const uint32_t *relu_bits) {
     const SegmentPlan plan = make_plan(c, D, cv.take<int32_t>(plan_ints(D.R, D.n)), true);
-    MOE_TRY(launch_segment_plan(plan, offsets, (int32_t)D.n, D.R, status_word(ws), st));
+    SegmentMaps maps;
+    const bool tc = tc_ffn_supported(*c);
+    if (tc) {
+        Carver ahead = cv;  // where do_expert_ffn_bwd will have dz
+        const FfnBwdWs w(ahead, D);
+        MOE_TRY(tc_segment_maps(*c, &maps, nullptr, nullptr, dys, w.dz, hid, dys, xs, w.dz));
+    }
+    MOE_TRY(launch_segment_plan(plan, offsets, (int32_t)D.n, D.R, status_word(ws), st, tc ? &maps : nullptr));
     return do_expert_ffn_bwd(c, D, xs, hid, dys, offsets, W1, W2, dxs, dW1, db1, dW2, db2, ws, cv, st, plan, relu_bits);
 }
 
@@ -936,7 +949,16 @@ static int32_t backward_impl(const moe_config *cfg, const void *dY, const void *
     const SegmentPlan plan = make_plan(cfg, D, B.plan, true);
     const Cv2Job jobs[2] = {{C.importance, (int32_t)D.n, cfg->w_importance, B.dimp},
                             {C.load, (int32_t)D.n, cfg->w_load, D.hier ? B.dload_h : B.dload}};
-    MOE_TRY(launch_segment_plan(plan, C.offsets, (int32_t)D.n, D.R, status_word(ws), st, jobs));
+    SegmentMaps maps;
+    const bool tc = tc_ffn_supported(*cfg);
+    if (tc) {
+        Carver ahead = fresh();  // where the expert backward will have dz and hidden activations that are computed again
+        const FfnBwdWs w(ahead, D);
+        const FfnWs f(ahead, D);
+        const void *hid = C.hid ? C.hid : f.hid;
+        MOE_TRY(tc_segment_maps(*cfg, &maps, C.hid ? nullptr : C.xs, nullptr, B.dys, w.dz, hid, B.dys, C.xs, w.dz));
+    }
+    MOE_TRY(launch_segment_plan(plan, C.offsets, (int32_t)D.n, D.R, status_word(ws), st, tc ? &maps : nullptr, jobs));
     if (D.hier) MOE_TRY(launch_load_h_bwd(C.load, B.dload_h, (int32_t)D.a, (int32_t)D.b, B.dload, st));
     MOE_TRY(launch_combine_bwd(dY, C.ys, D.act, C.gates, C.inv_perm, D.T, (int32_t)D.k, (int32_t)D.d, B.dgates,
                                B.dys, st, keep_bits, keep_bits ? 1.0f / (1.0f - drop_prob) : 1.0f, C.topk_idx, B.dimp,

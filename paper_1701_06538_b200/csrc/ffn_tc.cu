@@ -17,8 +17,9 @@
 //   ROW_BK   same A, per-expert weight read transposed ([N, K], K contiguous, K-major B):
 //            dz = (dys.W2^T) * [hid > 0],  dxs = dz.W1^T
 //   WGRAD    contraction over the rows of a segment, both operands MN-major:
-//            dW2 = hid^T.dys,  dW1 = xs^T.dz. The last K block of a segment is ragged: the rows
-//            past the segment end are zeroed in shared memory in both operands.
+//            dW2 = hid^T.dys,  dW1 = xs^T.dz.
+// The last rows of a segment are loaded through a tensor map that ends with the segment: what lies behind them (the next
+// segment's rows) reads as zero, in both operands of a weight gradient.
 // Weights are addressed through one tensor map with the expert as a coordinate, segment bounds
 // are read on the device: no per-expert descriptors and no host synchronisation.
 //
@@ -42,7 +43,7 @@ constexpr int EPI_STAGE_BYTES = 8 * 4096;  // per epilogue warp: a 32 x 128 B sl
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /*alignment slack*/ + 1024 /*barriers; the boxes behind them are 1024-byte aligned*/ + EPI_STAGE_BYTES;
 constexpr int TMEM_COLS = 512;
 constexpr int NTHREADS = 320;   // TMA warp, MMA warp, 8 epilogue warps
-constexpr int NTHREADS2 = 384;  // two-CTA kernel: + one warp that fixes the ragged K tail of the wgrad ahead of the MMAs, + the tile scheduler warp
+constexpr int NTHREADS2 = 352;  // two-CTA kernel: + the tile scheduler warp
 constexpr unsigned long long WAIT_LIMIT_NS = 2000000000ull;
 
 enum Kind { ROW_BMN = 0, ROW_BK = 1, WGRAD = 2 };
@@ -85,6 +86,9 @@ struct GemmParams {
     int32_t interleave;                 // uniform WGRAD: number of terms whose tiles alternate in the id order (0: none)
     int32_t sub_kb0, sub_kb;            // ACC kernel: K blocks per separately accumulated sub-block, term 0 / other terms
     int32_t off_mod;                    // WGRAD with offsets: see tile_fetch
+    // one map per segment that ends with the segment: for the box of A (WGRAD: of A and of B) that reaches beyond it. Row
+    // products may do without (their rows behind the end are computed and dropped)
+    const CUtensorMap *seg_a, *seg_b;
     // ROW_*: the contraction is the concatenation of nterms pieces of length K; piece i reads A
     // columns a_term_col[i] + [0, K) and B columns b_term_col[i] + [0, K)
     int32_t nterms;
@@ -196,6 +200,12 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap *tm, uint32_t src
 __device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+
+// A map in global memory that an earlier kernel has written: made visible to the copies of this thread, and fetched ahead
+__device__ __forceinline__ void acquire_map(const CUtensorMap *tm) {
+    asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(tm) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(tm) : "memory");
+}
 
 // 256-bit store (sm_100): a whole 32-byte sector per instruction
 __device__ __forceinline__ void st_global_32B(uint4 *dst, const uint4 &a, const uint4 &b) {
@@ -550,6 +560,25 @@ template <int KIND, int TM> struct TileIter {
     }
 };
 
+// The maps of a tile whose last box of rows reaches beyond its segment (first row `row0` of a box of `height` rows; WGRAD: the
+// segment's last K block)
+template <int KIND> struct SegmentEnd {
+    const CUtensorMap *a, *b;
+    bool ragged;
+    __device__ __forceinline__ SegmentEnd(const GemmParams &p, const Tile &t, int32_t row0, int height) : a(nullptr), b(nullptr) {
+        if (KIND == WGRAD) ragged = p.seg_a && (t.row_end - t.row0) % BK != 0;
+        else ragged = p.seg_a && row0 + height > t.row_end;
+        if (!ragged) return;
+        const int32_t e = KIND == WGRAD && p.off_mod > 0 ? t.e % p.off_mod : t.e;
+        a = p.seg_a + e;
+        acquire_map(a);
+        if (KIND == WGRAD) {
+            b = p.seg_b + e;
+            acquire_map(b);
+        }
+    }
+};
+
 // ACC (WGRAD with float output over long uniform row ranges, the gate backward): the contraction of a tile is cut
 // into sub-blocks of p.sub_kb0 / p.sub_kb K blocks (first term / other terms). Each sub-block is accumulated in TMEM on
 // its own (an fp32 tensor-core accumulator truncates, and a long run of same-sign terms loses low bits: 128 rows keep
@@ -605,6 +634,8 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             Tile t;
             while (ok && it.next(t)) {
                 int term = 0, kk = 0;  // ROW_*: piece of the contraction and column inside it
+                const SegmentEnd<KIND> end(p, t, t.row0, BM);
+                const CUtensorMap *row_a = KIND != WGRAD && end.ragged ? end.a : &tmA;
                 for (int kb = 0; kb < t.kblocks && ok; ++kb) {
                     ok = mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, p.status);
                     if (!ok) break;
@@ -612,10 +643,11 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                     mbar_expect_tx(full_bar(s), STAGE_BYTES);
                     if (KIND == WGRAD) {
                         const int r = t.row0 + kb * BK;
-                        tma_load_3d(a_dst, &tmA, full_bar(s), 0, r, t.m0 / 64);
-                        tma_load_3d(b_dst, &tmB, full_bar(s), 0, r, t.b_chunk);
+                        const bool tail = end.ragged && kb == t.kblocks - 1;
+                        tma_load_3d(a_dst, tail ? end.a : &tmA, full_bar(s), 0, r, t.m0 / 64);
+                        tma_load_3d(b_dst, tail ? end.b : &tmB, full_bar(s), 0, r, t.b_chunk);
                     } else {
-                        tma_load_2d(a_dst, &tmA, full_bar(s), p.a_term_col[term] + kk, t.row0);
+                        tma_load_2d(a_dst, row_a, full_bar(s), p.a_term_col[term] + kk, t.row0);
                         if (KIND == ROW_BMN) tma_load_4d(b_dst, &tmB, full_bar(s), 0, p.b_term_col[term] + kk, t.n0 / 64, t.e);
                         else tma_load_3d(b_dst, &tmB, full_bar(s), p.b_term_col[term] + kk, t.n0, t.e);
                         kk += BK;
@@ -656,28 +688,8 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t a_src = base + s * STAGE_BYTES, b_src = a_src + A_BYTES;
-                int ksteps = BK / 16;  // K steps of 16 rows to issue for this block
-                if (KIND == WGRAD && kb == t.kblocks - 1) {
-                    const int valid = t.row_end - (t.row0 + kb * BK);  // rows of this block inside the segment
-                    if (valid < BK) {
-                        // The rows behind the segment's end belong to the next segment. Whole K steps behind it are not
-                        // issued at all; in the step that holds the end, K rows [valid, end of the step) are zeroed in A
-                        // AND in B (0 x finite = 0 would do for finite data; both keep a non-finite value of the next
-                        // segment out of this segment's sums): 128-B lines in all 64-column chunks, the A tile's two
-                        // chunks directly followed by the B tile's four.
-                        ksteps = (valid + 15) / 16;
-                        const int nz = ksteps * 16 - valid;
-                        const int lines = nz * ((BM + BN) / 64);
-                        for (int u = lane; u < lines * 8; u += 32) {
-                            const int line = u >> 3, part = u & 7;
-                            const int chunk = line / nz, krow = valid + line % nz;
-                            *reinterpret_cast<uint4 *>(smem + s * STAGE_BYTES + chunk * (BK * 128) + krow * 128 + part * 16) =
-                                make_uint4(0, 0, 0, 0);
-                        }
-                        if (nz > 0) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                        __syncwarp();
-                    }
-                }
+                int ksteps = BK / 16;  // K steps of 16 rows to issue for this block: those behind the segment's end hold zeros
+                if (KIND == WGRAD && kb == t.kblocks - 1) ksteps = min(BK, t.row_end - (t.row0 + kb * BK) + 15) / 16;
                 if (lane == 0) {
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k) {
@@ -989,10 +1001,6 @@ grouped_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     auto empty_bar = [&](int s) { return bars + 8u * (NST + s); };
     auto tfull_bar = [&](int a) { return bars + 8u * (2 * NST + a); };
     auto tempty_bar = [&](int a) { return bars + 8u * (2 * NST + 2 + a); };
-    // WGRAD only: afull = this CTA's own tiles of a ragged last K block have landed (the tail rows are zeroed before use);
-    // ready (even CTA) = both CTAs' tiles are landed and fixed
-    auto afull_bar = [&](int s) { return bars + 8u * (2 * NST + 4 + s); };
-    auto ready_bar = [&](int s) { return bars + 8u * (3 * NST + 4 + s); };
     const uint32_t mfull_bar = bars + 8u * 28, mempty_bar = bars + 8u * 29;  // mask tile landed / read by all 8 epilogue warps
     // dynamic tile scheduling (WGRAD): record published / record read by every role of both CTAs (barrier in the even CTA)
     const uint32_t sched_full0 = bars + 256, sched_empty0 = bars + 256 + 8u * SCHED_SLOTS, sched_ring = bars + 384;
@@ -1006,14 +1014,11 @@ grouped_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     const int64_t cluster_id = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < NST; ++s) {
-            mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1);
-            mbar_init(afull_bar(s), 1); mbar_init(ready_bar(s), 2);  // ready: both CTAs' tail-fixing warps
-        }
+        for (int s = 0; s < NST; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
         for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), 16); }
         mbar_init(mfull_bar, 1); mbar_init(mempty_bar, 8);
-        // readers of a scheduler record: producer, 8 epilogue warps (WGRAD: + tail warp) in each CTA, the MMA thread in the even one
-        for (int q = 0; q < SCHED_SLOTS; ++q) { mbar_init(sched_full0 + 8u * q, 1); mbar_init(sched_empty0 + 8u * q, KIND == WGRAD ? 21 : 19); }
+        // readers of a scheduler record: producer, 8 epilogue warps in each CTA, the MMA thread in the even one
+        for (int q = 0; q < SCHED_SLOTS; ++q) { mbar_init(sched_full0 + 8u * q, 1); mbar_init(sched_empty0 + 8u * q, 19); }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA) : "memory");
@@ -1034,22 +1039,6 @@ grouped_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     const uint32_t tmem_base = *tmem_slot;
     wait_previous_kernel();  // barriers and tensor memory are set up while the previous kernel drains
 
-    // K rows past the segment end in stage s's A and B tiles (two 64-column chunks each, the B tile directly behind the
-    // A tile) := 0. Zeroing A alone would do for finite data (0 x finite = 0); B as well keeps a non-finite value of the
-    // next segment out of this segment's sums.
-    auto zero_tail = [&](int s, int valid) {
-        const int nz = ((valid + 15) / 16) * 16 - valid;  // up to the end of the K step of 16 that holds the segment's end:
-                                                           // the K steps behind it are not issued at all
-        const int lines = nz * 4;
-        for (int u = lane; u < lines * 8; u += 32) {
-            const int line = u >> 3, part = u & 7;
-            const int chunk = line / nz, krow = valid + line % nz;
-            *reinterpret_cast<uint4 *>(smem + s * STAGE2_BYTES + chunk * (BK * 128) + krow * 128 + part * 16) =
-                make_uint4(0, 0, 0, 0);
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncwarp();
-    };
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer (both CTAs)
         if (lane == 0) {
@@ -1080,6 +1069,8 @@ grouped_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
             int trace_tile = -1;
             while (ok && it.next(t)) {
                 int term = 0, kk = 0;  // ROW_*: piece of the contraction and column inside it
+                const SegmentEnd<KIND> end(p, t, t.row0 + 128 * (int)rank, 128);
+                const CUtensorMap *row_a = KIND != WGRAD && end.ragged ? end.a : &tmA;
                 ++trace_tile;
                 long long tr_empty = 0;
                 for (int kb = 0; kb < t.kblocks && ok; ++kb) {
@@ -1093,20 +1084,13 @@ grouped_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                     const uint32_t a_dst = base + s * STAGE2_BYTES, b_dst = a_dst + A2_BYTES;
                     if (KIND == WGRAD) {
                         const int r = t.row0 + kb * BK;
-                        if (t.row_end - r < BK) {  // ragged last block: both tiles land on this CTA's own barrier first
-                            if (rank == 0) mbar_expect_tx(full_bar(s), 0);  // nothing counts on the pair's barrier: the
-                                                                            // "ready" barrier gates this stage
-                            mbar_expect_tx(afull_bar(s), STAGE2_BYTES);
-                            tma_load_3d(a_dst, &tmA, afull_bar(s), 0, r, t.m0 / 64 + 2 * (int)rank);
-                            tma_load_3d(b_dst, &tmB, afull_bar(s), 0, r, t.b_chunk + 2 * (int)rank);
-                        } else {
-                            if (rank == 0) mbar_expect_tx(full_bar(s), 2 * STAGE2_BYTES);
-                            tma2_load_3d(a_dst, &tmA, full_bar(s), 0, r, t.m0 / 64 + 2 * (int)rank);
-                            tma2_load_3d(b_dst, &tmB, full_bar(s), 0, r, t.b_chunk + 2 * (int)rank);
-                        }
+                        const bool tail = end.ragged && kb == t.kblocks - 1;
+                        if (rank == 0) mbar_expect_tx(full_bar(s), 2 * STAGE2_BYTES);
+                        tma2_load_3d(a_dst, tail ? end.a : &tmA, full_bar(s), 0, r, t.m0 / 64 + 2 * (int)rank);
+                        tma2_load_3d(b_dst, tail ? end.b : &tmB, full_bar(s), 0, r, t.b_chunk + 2 * (int)rank);
                     } else {
                         if (rank == 0) mbar_expect_tx(full_bar(s), 2 * STAGE2_BYTES);
-                        tma2_load_2d(a_dst, &tmA, full_bar(s), p.a_term_col[term] + kk, t.row0 + 128 * (int)rank);
+                        tma2_load_2d(a_dst, row_a, full_bar(s), p.a_term_col[term] + kk, t.row0 + 128 * (int)rank);
                         if (KIND == ROW_BMN)
                             tma2_load_4d(b_dst, &tmB, full_bar(s), 0, p.b_term_col[term] + kk, t.n0 / 64 + 2 * (int)rank, t.e);
                         else
@@ -1132,7 +1116,7 @@ grouped_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
         if (rank == 0 && lane == 0) {
             constexpr uint32_t idesc = make_idesc2(KIND == WGRAD ? 1 : 0, KIND == ROW_BK ? 0 : 1);
             int s = 0, acc = 0;
-            uint32_t ph = 0, acc_ph = 0, tail_ph = 0;  // tail_ph: one phase bit per stage for afull / ready
+            uint32_t ph = 0, acc_ph = 0;
             bool ok = true;
             PairTiles<KIND> it(p, dyn, (int32_t)cluster_id, (int32_t)n_clusters, sched_ring, sched_full0, sched_empty0, abort_flag, false, true);
             Tile t;
@@ -1149,12 +1133,6 @@ grouped_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                 const uint32_t d_tmem = tmem_base + acc * BN;
                 const int tail_valid = KIND == WGRAD ? (t.row_end - t.row0) - (t.kblocks - 1) * BK : BK;  // rows of the last block
                 for (int kb = 0; kb < t.kblocks; ++kb) {
-                    if (KIND == WGRAD && kb == t.kblocks - 1 && tail_valid < BK) {
-                        const uint32_t tp = (tail_ph >> s) & 1u;  // fixed by warp 10 of both CTAs, ahead of time
-                        ok = mbar_wait(ready_bar(s), tp, abort_flag, p.status) && mbar_try_wait_cluster(ready_bar(s), tp);
-                        if (!ok) break;
-                        tail_ph ^= 1u << s;
-                    }
                     const long long tw0 = TILE_CLOCK();
                     ok = mbar_wait(full_bar(s), ph, abort_flag, p.status);
                     if (!ok) break;
@@ -1182,7 +1160,7 @@ grouped_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                 if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
             }
         }
-    } else if (warp == 11) {
+    } else if (warp == 10) {
         // ------------------------------------------------------------------ tile scheduler (even CTA, one thread)
         if (dyn && rank == 0 && lane == 0) {
             const uint32_t peer_ring = peer_smem_addr(sched_ring, 1), peer_full0 = peer_smem_addr(sched_full0, 1);
@@ -1205,31 +1183,6 @@ grouped_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                 mbar_arrive(sched_full0 + 8u * slot);
                 mbar_arrive_cluster_addr(peer_full0 + 8u * slot);
                 if (rec.x < 0) break;
-            }
-        }
-    } else if (warp == 10) {
-        // ------------------------------------------------------------------ WGRAD: ragged K tail (both CTAs)
-        // The last K block of a segment holds rows of the next segment: they are zeroed in this CTA's A tile as soon as
-        // it has landed, several stages before the MMAs get there, and reported on the even CTA's "ready" barrier.
-        if (KIND == WGRAD) {
-            int s = 0;
-            uint32_t tail_ph = 0;
-            bool ok = true;
-            PairTiles<KIND> it(p, dyn, (int32_t)cluster_id, (int32_t)n_clusters, sched_ring, sched_full0, sched_empty0, abort_flag, true, lane == 0);
-            Tile t;
-            while (ok && it.next(t)) {
-                for (int kb = 0; kb < t.kblocks; ++kb) {
-                    const int valid = t.row_end - (t.row0 + kb * BK);
-                    if (valid < BK) {
-                        ok = mbar_wait(afull_bar(s), (tail_ph >> s) & 1u, abort_flag, p.status);
-                        if (!ok) break;
-                        zero_tail(s, valid);
-                        if (lane == 0) mbar_arrive_leader(ready_bar(s));
-                        __syncwarp();
-                        tail_ph ^= 1u << s;
-                    }
-                    if (++s == NST) s = 0;
-                }
             }
         }
     } else {
@@ -1540,15 +1493,48 @@ static bool use_two_cta(int64_t R, int32_t nseg, int32_t flags) {
     return R / (nseg > 0 ? nseg : 1) >= 384;
 }
 
+int32_t tc_segment_maps(const moe_config &c, SegmentMaps *maps, const void *xs_rows, const void *hid_rows, const void *dys_rows,
+                        const void *dz_rows, const void *hid_cols, const void *dys_cols, const void *xs_cols, const void *dz_cols) {
+    memset(maps, 0, sizeof(*maps));
+    const int64_t R = (int64_t)c.T * c.k, rows = R > 0 ? R : 1;
+    auto add = [&](SegmentMap which, const void *p, int64_t cols, int chunks) -> int32_t {
+        if (!p) return MOE_OK;
+        maps->made[which] = 1;
+        return chunks ? map_rows_mnmajor(&maps->base[which], p, rows, cols, chunks) : map_rows_kmajor(&maps->base[which], p, rows, cols);
+    };
+    // boxes as in tc_row_gemm and tc_wgrad_gemm
+    const bool two = use_two_cta(R, c.n, c.flags);
+    const int b2 = two && c.h >= 256 ? 2 : BN / 64, b1 = two && c.d >= 256 ? 2 : BN / 64;
+    MOE_TRY(add(MAP_XS_ROWS, xs_rows, c.d, 0));
+    MOE_TRY(add(MAP_HID_ROWS, hid_rows, c.h, 0));
+    MOE_TRY(add(MAP_DYS_ROWS, dys_rows, c.d, 0));
+    MOE_TRY(add(MAP_DZ_ROWS, dz_rows, c.h, 0));
+    MOE_TRY(add(MAP_HID_COLS, hid_cols, c.h, 2));
+    MOE_TRY(add(MAP_DYS_COLS, dys_cols, c.d, b2));
+    MOE_TRY(add(MAP_XS_COLS, xs_cols, c.d, 2));
+    return add(MAP_DZ_COLS, dz_cols, c.h, b1);
+}
+
 // C[rows, N] = epilogue(A[rows, K] . B_e) over the segments; B_e = W[e] as [K, N] (transposed = false)
 // or as [N, K] read transposed (transposed = true).
+// tensor maps of the two operands of a weight gradient over the groups, and where those that end with the groups go ([2][n])
+struct GroupMaps { CUtensorMap a, b; CUtensorMap *out; };
 // Tile table of a ragged row GEMM: tile_prefix[e] = number of tm-row tiles of the segments before e
 // (tile_prefix[nseg] = total), and one record per M tile {segment, first row, segment end, 0}; records past
-// the last tile carry segment -1. One block.
+// the last tile carry segment -1. One block; the others: the groups' tensor maps, where they are wanted.
 __global__ void __launch_bounds__(1024) tile_table_kernel(const int32_t *__restrict__ offsets, int32_t n, int32_t tm,
                                                           int32_t max_m, int32_t *__restrict__ tile_prefix,
-                                                          int4 *__restrict__ info) {
+                                                          int4 *__restrict__ info, const __grid_constant__ GroupMaps maps) {
     wait_previous_kernel();
+    __shared__ __align__(128) uint32_t map_sh[32][32];
+    if (blockIdx.x > 0) {  // the groups' tensor maps, one per warp
+        const int32_t i = (blockIdx.x - 1) * 32 + (threadIdx.x >> 5);
+        if (i < 2 * n) {
+            const int32_t e = i >= n ? i - n : i;
+            write_segment_map(i >= n ? maps.b : maps.a, maps.out + i, offsets[e + 1], map_sh[threadIdx.x >> 5]);
+        }
+        return;
+    }
     __shared__ int32_t warp_sum[32];
     __shared__ int32_t carry;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -1597,14 +1583,22 @@ __global__ void __launch_bounds__(1024) tile_table_kernel(const int32_t *__restr
 }
 
 // ints a tile table needs behind its [nseg + 1] prefix (records are 16 bytes, 16-byte aligned)
-int64_t tc_tile_ws_ints(int64_t R, int64_t nseg) { return ((nseg + 1 + 3) & ~(int64_t)3) + 4 * (cdiv(R, 128) + nseg + 1); }
+int64_t tc_tile_ws_ints(int64_t R, int64_t nseg) {
+    return ((nseg + 1 + 3) & ~(int64_t)3) + 4 * (cdiv(R, 128) + nseg + 1) + 32 /* alignment of the maps */ + 2 * 32 * nseg;
+}
 static int4 *tile_info_of(int32_t *tile_prefix, int32_t nseg) {
     return reinterpret_cast<int4 *>(tile_prefix + ((nseg + 1 + 3) & ~3));
 }
+static CUtensorMap *group_maps_of(int32_t *tile_prefix, int64_t R, int32_t nseg) {
+    return reinterpret_cast<CUtensorMap *>((reinterpret_cast<uintptr_t>(tile_info_of(tile_prefix, nseg) + cdiv(R, 128) + nseg + 1) + 127) & ~(uintptr_t)127);
+}
 static int32_t launch_tile_table(const int32_t *offsets, int32_t nseg, int32_t tm, int64_t R, int32_t *tile_prefix,
-                                 cudaStream_t st) {
-    launch_kernel(tile_table_kernel, 1, 1024, 0, st, offsets, nseg, tm, (int32_t)(cdiv(R, tm) + nseg), tile_prefix,
-                                          tile_info_of(tile_prefix, nseg));
+                                 cudaStream_t st, const GroupMaps *maps = nullptr) {
+    GroupMaps m;
+    if (maps) m = *maps;
+    else memset(&m, 0, sizeof(m));
+    launch_kernel(tile_table_kernel, maps ? 1 + (unsigned)cdiv(2 * nseg, 32) : 1u, 1024, 0, st, offsets, nseg, tm, (int32_t)(cdiv(R, tm) + nseg),
+                  tile_prefix, tile_info_of(tile_prefix, nseg), m);
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -1676,7 +1670,7 @@ int64_t tc_colsum_part_floats(int64_t R, int32_t nseg, int32_t N) { return (cdiv
 // and reduced into colsum_out [nseg, N]; colsum_part needs tc_colsum_part_floats(R, nseg, N) floats
 int32_t tc_row_gemm(const void *A, const void *W, bool transposed, const int32_t *offsets, int32_t nseg, int64_t R,
                     int32_t N, int32_t K, void *out, const void *bias, const void *mask, int relu,
-                    const SegmentPlan &plan, int counter, int32_t *status, cudaStream_t st, int32_t flags,
+                    const SegmentPlan &plan, int counter, SegmentMap seg, int32_t *status, cudaStream_t st, int32_t flags,
                     float *colsum_part = nullptr, void *colsum_out = nullptr, uint32_t *bits_out = nullptr,
                     const uint32_t *bits_in = nullptr) {
     if (R == 0) {
@@ -1699,6 +1693,7 @@ int32_t tc_row_gemm(const void *A, const void *W, bool transposed, const int32_t
     GemmParams p = default_params();
     p.offsets = offsets; p.tile_prefix = plan.prefix[0]; p.tile_info = plan.info;
     p.nseg = nseg; p.M = 0; p.N = N; p.K = K; p.R = R;
+    p.seg_a = plan.maps_of(seg);
     p.out = (bf16 *)out; p.bias = (const bf16 *)bias; p.mask = (const bf16 *)mask; p.relu = relu; p.status = status;
     p.bits_out = bits_out; p.bits_in = bits_in;
     if (bits_in) p.mask = nullptr;  // the bits replace the element-wise mask tensor
@@ -1731,10 +1726,12 @@ int32_t tc_row_gemm(const void *A, const void *W, bool transposed, const int32_t
 // dW[e] [M, N] = A_e^T . B_e, contraction over the rows of segment e; A [R, M], B [R, N].
 // plan.sched (if made): the two-CTA kernel hands its tiles out at run time, longest segments first.
 int32_t tc_wgrad_gemm(const void *A, const void *B, const int32_t *offsets, int32_t nseg, int64_t R, int32_t M,
-                      int32_t N, void *out, int32_t *status, cudaStream_t st, int32_t flags, const SegmentPlan &plan, int counter) {
+                      int32_t N, void *out, int32_t *status, cudaStream_t st, int32_t flags, const SegmentPlan &plan, int counter,
+                      SegmentMap seg_a, SegmentMap seg_b) {
     CUtensorMap tmA, tmB;
     GemmParams p = default_params();
     p.offsets = offsets; p.nseg = nseg; p.M = M; p.N = N; p.R = R;
+    p.seg_a = plan.maps_of(seg_a); p.seg_b = plan.maps_of(seg_b);
     p.out = (bf16 *)out; p.status = status;
     CUtensorMap tmO;  // the experts' matrices as one tall matrix (a 32-row box never straddles two: M is a multiple of 64)
     MOE_TRY(map_out_boxes(&tmO, out, (int64_t)nseg * M, N));
@@ -1763,9 +1760,9 @@ int32_t launch_tc_ffn(const moe_config &c, const void *xs, const int32_t *offset
                       cudaStream_t st, bool first_only, uint32_t *relu_bits) {
     const int64_t R = (int64_t)c.T * c.k;
     MOE_TRY(tc_row_gemm(xs, W1, false, offsets, c.n, R, c.h, c.d, hid, b1, nullptr, 1, plan, first_only ? PLAN_ROWS_AGAIN : PLAN_ROWS_A,
-                        status_word, st, c.flags, nullptr, nullptr, relu_bits));
+                        MAP_XS_ROWS, status_word, st, c.flags, nullptr, nullptr, relu_bits));
     if (first_only) return MOE_OK;
-    return tc_row_gemm(hid, W2, false, offsets, c.n, R, c.d, c.h, ys, b2, nullptr, 0, plan, PLAN_ROWS_B, status_word, st, c.flags);
+    return tc_row_gemm(hid, W2, false, offsets, c.n, R, c.d, c.h, ys, b2, nullptr, 0, plan, PLAN_ROWS_B, MAP_HID_ROWS, status_word, st, c.flags);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1959,7 +1956,10 @@ int32_t launch_tc_hier_secondary_bwd(const void *xs_p, const void *dsplit_s, voi
         CUtensorMap tmA, tmB;
         MOE_TRY(map_rows_mnmajor(&tmA, xs_p, P1 > 0 ? P1 : 1, d, BM / 64));
         MOE_TRY(map_rows_mnmajor(&tmB, dsplit_s, P1 > 0 ? P1 : 1, 3 * n2, BN / 64));
+        const GroupMaps maps = {tmA, tmB, group_maps_of(tile_prefix, P1, a)};
+        MOE_TRY(launch_tile_table(offsets_p, a, BM, P1, tile_prefix, st, &maps));  // the tiles of dX_sec below, too
         GemmParams p = default_params();
+        p.seg_a = maps.out; p.seg_b = maps.out + a;
         p.offsets = offsets_p; p.nseg = 3 * a; p.off_mod = a; p.b_term_chunks = n2 / 64;
         p.M = d; p.N = n2; p.R = P1; p.out_f32 = partials; p.status = status;
         MOE_TRY(launch<WGRAD>(tmA, tmB, p, (int64_t)p.nseg * cdiv(d, BM) * cdiv(n2, BN), st));
@@ -1971,7 +1971,6 @@ int32_t launch_tc_hier_secondary_bwd(const void *xs_p, const void *dsplit_s, voi
         CUtensorMap tmA, tmB;
         MOE_TRY(map_rows_kmajor(&tmA, dsplit_s, P1, 3 * n2));
         MOE_TRY(map_weight_kmajor(&tmB, wsplit_s, a, d, 3 * n2));
-        MOE_TRY(launch_tile_table(offsets_p, a, BM, P1, tile_prefix, st));
         GemmParams p = default_params();
         p.offsets = offsets_p; p.tile_prefix = tile_prefix; p.tile_info = tile_info_of(tile_prefix, a);
         p.nseg = a; p.N = d; p.K = n2; p.R = P1;
@@ -1990,12 +1989,14 @@ int32_t launch_tc_ffn_bwd(const moe_config &c, const void *xs, const void *hid, 
                           cudaStream_t st, const uint32_t *relu_bits) {
     const int64_t R = (int64_t)c.T * c.k;
     MOE_TRY(launch_segment_colsum(dys, c.act, offsets, c.n, R, c.d, db2, colsum, plan.prefix_of(COLSUM_ROWS), st));
-    MOE_TRY(tc_wgrad_gemm(hid, dys, offsets, c.n, R, c.h, c.d, dW2, status_word, st, c.flags, plan, PLAN_WGRAD_A));
+    MOE_TRY(tc_wgrad_gemm(hid, dys, offsets, c.n, R, c.h, c.d, dW2, status_word, st, c.flags, plan, PLAN_WGRAD_A,
+                          MAP_HID_COLS, MAP_DYS_COLS));
     // db1 = column sums of dz, formed in the epilogue of the GEMM that produces dz
-    MOE_TRY(tc_row_gemm(dys, W2, true, offsets, c.n, R, c.h, c.d, dz, nullptr, hid, 0, plan, PLAN_ROWS_A, status_word, st, c.flags,
+    MOE_TRY(tc_row_gemm(dys, W2, true, offsets, c.n, R, c.h, c.d, dz, nullptr, hid, 0, plan, PLAN_ROWS_A, MAP_DYS_ROWS, status_word, st, c.flags,
                         colsum, db1, nullptr, relu_bits));
-    MOE_TRY(tc_wgrad_gemm(xs, dz, offsets, c.n, R, c.d, c.h, dW1, status_word, st, c.flags, plan, PLAN_WGRAD_B));
-    return tc_row_gemm(dz, W1, true, offsets, c.n, R, c.d, c.h, dxs, nullptr, nullptr, 0, plan, PLAN_ROWS_B, status_word, st, c.flags);
+    MOE_TRY(tc_wgrad_gemm(xs, dz, offsets, c.n, R, c.d, c.h, dW1, status_word, st, c.flags, plan, PLAN_WGRAD_B,
+                          MAP_XS_COLS, MAP_DZ_COLS));
+    return tc_row_gemm(dz, W1, true, offsets, c.n, R, c.d, c.h, dxs, nullptr, nullptr, 0, plan, PLAN_ROWS_B, MAP_DZ_ROWS, status_word, st, c.flags);
 }
 
 // ------------------------------------------------------------------------------------------

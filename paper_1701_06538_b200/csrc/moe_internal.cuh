@@ -1,6 +1,7 @@
 // Internal declarations shared by the translation units of the library (not part of the ABI).
 #pragma once
 
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -171,7 +172,18 @@ int32_t launch_tile_prefix(const int32_t *offsets, int32_t n, int32_t bm, int32_
 constexpr int PLAN_HEIGHTS = 4, PLAN_COUNTERS = 8, PLAN_MAX_SORTED = 8192;
 // run-time tile counters of a plan, by the GEMM that uses them
 enum PlanCounter { PLAN_ROWS_A = 0, PLAN_ROWS_B = 1, PLAN_WGRAD_A = 2, PLAN_WGRAD_B = 3, PLAN_ROWS_AGAIN = 4 };
+// Tensor maps of a call's expert products whose rows end with a segment, one per segment: what lies behind a segment's last row reads
+// as zero, whatever follows it in memory. ROWS: K-major operand of a row product, COLS: operand of a weight gradient
+// (contraction over the rows).
+enum SegmentMap { MAP_XS_ROWS = 0, MAP_HID_ROWS, MAP_DYS_ROWS, MAP_DZ_ROWS, MAP_HID_COLS, MAP_DYS_COLS, MAP_XS_COLS, MAP_DZ_COLS, SEGMENT_MAPS };
+struct SegmentMaps {
+    CUtensorMap base[SEGMENT_MAPS];  // of the whole tensors
+    int32_t made[SEGMENT_MAPS];      // which of them are wanted
+};
 struct SegmentPlan {
+    CUtensorMap *maps;              // [SEGMENT_MAPS][n], or nullptr
+    int32_t n;
+    const CUtensorMap *maps_of(SegmentMap which) const { return maps ? maps + (int64_t)which * n : nullptr; }
     int32_t *prefix[PLAN_HEIGHTS];  // [n + 1] number of tiles of bm[i] rows in the segments before
     int32_t bm[PLAN_HEIGHTS];       // 0: prefix not made
     int4 *info;          // a record per tile of prefix[0], or nullptr: {segment or -1, first row, segment end, 0}
@@ -187,7 +199,19 @@ struct Cv2Job { const float *v; int32_t m; float scale; float *out; };  // out =
 int64_t plan_ints(int64_t R, int64_t n);
 SegmentPlan plan_at(int32_t *ws, int64_t R, int64_t n);
 int32_t launch_segment_plan(const SegmentPlan &plan, const int32_t *offsets, int32_t n, int64_t R, int32_t *status,
-                            cudaStream_t st, const Cv2Job *jobs = nullptr /* two */);
+                            cudaStream_t st, const SegmentMaps *maps = nullptr, const Cv2Job *jobs = nullptr /* two */);
+// One segment's map, by a warp: a copy of `base` whose rows (dimension 1) end at `rows`. sh: 128 bytes, 128-byte aligned
+__device__ __forceinline__ void write_segment_map(const CUtensorMap &base, CUtensorMap *out, int32_t rows, uint32_t *sh) {
+    const int lane = threadIdx.x & 31;
+    sh[lane] = reinterpret_cast<const uint32_t *>(&base)[lane];
+    __syncwarp();
+    const uint32_t at = (uint32_t)__cvta_generic_to_shared(sh);
+    if (lane == 0)
+        asm volatile("tensormap.replace.tile.global_dim.shared::cta.b1024.b32 [%0], 1, %1;" ::"r"(at), "r"(rows > 1 ? rows : 1) : "memory");
+    __syncwarp();
+    asm volatile("tensormap.cp_fenceproxy.global.shared::cta.tensormap::generic.release.gpu.sync.aligned [%0], [%1], 128;" ::"l"(out), "r"(at)
+                 : "memory");
+}
 
 // ----------------------------------------------------------------------------- losses (losses.cu)
 // where the fused forward wants second copies of the stage's results (nullptr: none), and of the expert counts
@@ -285,6 +309,9 @@ constexpr int COLSUM_ROWS = 128;  // height of the tiles of tile_prefix
 
 // ----------------------------------------------------------------------------- tensor-core experts (ffn_tc.cu)
 bool tc_ffn_supported(const moe_config &c);
+// base maps of the operands that are given (nullptr: not wanted)
+int32_t tc_segment_maps(const moe_config &c, SegmentMaps *maps, const void *xs_rows, const void *hid_rows, const void *dys_rows,
+                        const void *dz_rows, const void *hid_cols, const void *dys_cols, const void *xs_cols, const void *dz_cols);
 int32_t tc_row_tile(int64_t R, int32_t nseg, int32_t flags);  // tile height of the row GEMMs: what plan.bm[0] has to be
 bool tc_wgrad_sorted(const moe_config &c);                    // the weight gradients want plan.sched
 // first_only: only hid = relu(xs.W1 + b1) (the recomputation of the hidden activations in the backward pass)
