@@ -101,11 +101,45 @@ int32_t reset_status(void *ws, cudaStream_t st) {
 }
 
 // ---------------------------------------------------------------------------- stage workspaces
+// Index tensors of the hierarchical levels. A fused forward call keeps those of its gate in the context, for the losses and the
+// backward call; a stage call that needs them makes them again from topk_idx.
+struct HierIdx {
+    int32_t *idx_p, *idx_s, *perm_p, *inv_perm_p, *counts_p, *offsets_p;
+    HierIdx() { idx_p = idx_s = perm_p = inv_perm_p = counts_p = offsets_p = nullptr; }
+    HierIdx(Carver &cv, const Dims &D) : HierIdx() {
+        if (!D.hier) return;
+        idx_p = cv.take<int32_t>(D.T * D.k1);
+        idx_s = cv.take<int32_t>(D.T * D.k);
+        perm_p = cv.take<int32_t>(D.T * D.k1);
+        inv_perm_p = cv.take<int32_t>(D.T * D.k1);
+        counts_p = cv.take<int32_t>(D.a);
+        offsets_p = cv.take<int32_t>(D.a + 1);
+    }
+};
+
+struct HierIdxWs : HierIdx {
+    int32_t *scratch, *tile_prefix;
+    HierIdxWs(Carver &cv, const Dims &D) : HierIdx(cv, D) {
+        scratch = tile_prefix = nullptr;
+        if (!D.hier) return;
+        scratch = cv.take<int32_t>(dispatch_ws_elems(D.T * D.k1, (int32_t)D.a));
+        tile_prefix = cv.take<int32_t>(tc_tile_ws_ints(D.T * D.k1, D.a));  // prefix + tile table of the secondary-gate GEMMs
+    }
+    int32_t build(const Dims &D, const int32_t *topk_idx, const HierIdx *ready, cudaStream_t st) {
+        if (ready) {
+            static_cast<HierIdx &>(*this) = *ready;
+            return MOE_OK;
+        }
+        MOE_TRY(launch_hier_split_idx(topk_idx, D.T, (int32_t)D.k1, (int32_t)D.k2, (int32_t)D.a, (int32_t)D.b, idx_p, idx_s, st));
+        return launch_dispatch_index(idx_p, D.T * D.k1, (int32_t)D.a, perm_p, inv_perm_p, counts_p, offsets_p, scratch,
+                                     st);
+    }
+};
+
 struct GateWs {
-    int32_t *idx_p, *idx_s, *perm_p, *inv_perm_p, *counts_p, *offsets_p, *scratch, *tile_prefix;
     // tensor-core routing screen (flat layer, or the primary level of the hierarchical one)
     bool screen;
-    float *cr, *wnorm, *xnorm, *wt;
+    float *wnorm, *xnorm, *wt;
     void *wsplit;
     int32_t *unsafe_list, *unsafe_count, *full_list;
     float *unsafe_low, *unsafe_low_s;
@@ -114,17 +148,16 @@ struct GateWs {
     // the same for the secondary gates of the hierarchical layer (rows = slots sorted by primary group)
     bool screen2;
     void *xs_p, *wsplit_s, *chain_list_s;
-    float *cr_s, *wnorm_s, *wt_s;
+    float *wnorm_s, *wt_s;
     int32_t *unsafe_list_s, *unsafe_count_s;
-    GateWs(Carver &cv, const Dims &D) {
+    HierIdxWs H;
+    GateWs(Carver &cv, const Dims &D) : H(cv, D) {
         screen2 = false;
-        xs_p = wsplit_s = chain_list_s = nullptr; cr_s = wnorm_s = wt_s = nullptr; unsafe_list_s = unsafe_count_s = nullptr; unsafe_low = unsafe_low_s = nullptr; unsafe_span = unsafe_span_s = nullptr;
-        idx_p = idx_s = perm_p = inv_perm_p = counts_p = offsets_p = scratch = tile_prefix = nullptr;
-        cr = wnorm = xnorm = wt = nullptr; wsplit = nullptr; unsafe_list = unsafe_count = full_list = nullptr; chain_list = nullptr;
+        xs_p = wsplit_s = chain_list_s = nullptr; wnorm_s = wt_s = nullptr; unsafe_list_s = unsafe_count_s = nullptr; unsafe_low = unsafe_low_s = nullptr; unsafe_span = unsafe_span_s = nullptr;
+        wnorm = xnorm = wt = nullptr; wsplit = nullptr; unsafe_list = unsafe_count = full_list = nullptr; chain_list = nullptr;
         const int64_t n1 = D.hier ? D.a : D.n;  // width of the (first) gate
         screen = tc_gate_fwd_supported(D.act, D.T, (int32_t)D.d, (int32_t)n1, D.flags);
         if (screen) {
-            cr = cv.take<float>(D.T * 2 * n1);
             wsplit = cv.take<bf16>(3 * D.d * 2 * n1);
             wnorm = cv.take<float>(2 * n1);
             wt = cv.take<float>(2 * n1 * D.d);
@@ -137,20 +170,11 @@ struct GateWs {
             chain_list = cv.take_bytes(D.T * 2 * SCREEN_MAX_CAND * 8);
         }
         if (!D.hier) return;
-        idx_p = cv.take<int32_t>(D.T * D.k1);
-        idx_s = cv.take<int32_t>(D.T * D.k);
-        perm_p = cv.take<int32_t>(D.T * D.k1);
-        inv_perm_p = cv.take<int32_t>(D.T * D.k1);
-        counts_p = cv.take<int32_t>(D.a);
-        offsets_p = cv.take<int32_t>(D.a + 1);
-        scratch = cv.take<int32_t>(dispatch_ws_elems(D.T * D.k1, (int32_t)D.a));
-        tile_prefix = cv.take<int32_t>(tc_tile_ws_ints(D.T * D.k1, D.a));  // prefix + tile table of the grouped product
         const int64_t P1 = D.T * D.k1;
         screen2 = tc_gate_fwd_supported(D.act, P1, (int32_t)D.d, (int32_t)D.b, D.flags);
         if (screen2) {
             if (!xnorm) xnorm = cv.take<float>(D.T);
             xs_p = cv.take_bytes(P1 * D.d * (int64_t)D.esz);
-            cr_s = cv.take<float>(P1 * 2 * D.b);
             wsplit_s = cv.take<bf16>(3 * D.a * D.d * 2 * D.b);
             wnorm_s = cv.take<float>(D.a * 2 * D.b);
             wt_s = cv.take<float>(D.a * 2 * D.b * D.d);
@@ -191,28 +215,6 @@ struct FfnWs {
     FfnWs(Carver &cv, const Dims &D) {
         plan = cv.take<int32_t>(plan_ints(D.R, D.n));
         hid = (D.flags & MOE_FLAG_RECOMPUTE_HID) ? cv.take_bytes(D.R * D.h * (int64_t)D.esz) : nullptr;
-    }
-};
-
-// index tensors of the hierarchical levels, rebuilt from topk_idx where a stage needs them
-struct HierIdxWs {
-    int32_t *idx_p, *idx_s, *perm_p, *inv_perm_p, *counts_p, *offsets_p, *scratch, *tile_prefix;
-    HierIdxWs(Carver &cv, const Dims &D) {
-        idx_p = idx_s = perm_p = inv_perm_p = counts_p = offsets_p = scratch = tile_prefix = nullptr;
-        if (!D.hier) return;
-        idx_p = cv.take<int32_t>(D.T * D.k1);
-        idx_s = cv.take<int32_t>(D.T * D.k);
-        perm_p = cv.take<int32_t>(D.T * D.k1);
-        inv_perm_p = cv.take<int32_t>(D.T * D.k1);
-        counts_p = cv.take<int32_t>(D.a);
-        offsets_p = cv.take<int32_t>(D.a + 1);
-        scratch = cv.take<int32_t>(dispatch_ws_elems(D.T * D.k1, (int32_t)D.a));
-        tile_prefix = cv.take<int32_t>(tc_tile_ws_ints(D.T * D.k1, D.a));  // prefix + tile table of the secondary-gate GEMMs
-    }
-    int32_t build(const Dims &D, const int32_t *topk_idx, cudaStream_t st) {
-        MOE_TRY(launch_hier_split_idx(topk_idx, D.T, (int32_t)D.k1, (int32_t)D.k2, (int32_t)D.a, (int32_t)D.b, idx_p, idx_s, st));
-        return launch_dispatch_index(idx_p, D.T * D.k1, (int32_t)D.a, perm_p, inv_perm_p, counts_p, offsets_p, scratch,
-                                     st);
     }
 };
 
@@ -308,6 +310,7 @@ struct Ctx {
     float *gates, *clean, *raw_noise, *kth_vals, *importance, *load, *losses;
     void *xs, *hid, *ys;
     uint32_t *relu_bits;  // tensor-core layers that keep hid: one bit per hidden activation for the backward's ReLU mask
+    HierIdx hier;         // of the hierarchical layer's levels
     moe_ctx_layout off;
     Ctx(void *base, const Dims &D, bool has_bits) {
         Carver cv(base);
@@ -330,6 +333,7 @@ struct Ctx {
         off.losses = at(); losses = cv.take<float>(2);
         off.relu_bits = at();
         relu_bits = (has_bits && !(D.flags & MOE_FLAG_RECOMPUTE_HID)) ? cv.take<uint32_t>(D.R * (D.h / 32)) : nullptr;
+        hier = HierIdx(cv, D);
         bytes = (int64_t)cv.off;
     }
     int64_t bytes;
@@ -356,8 +360,9 @@ struct BwdWs {
 
 int32_t do_gate(const moe_config *c, const Dims &D, const void *x, const float *Wg, const float *Wnoise,
                 const float *noise, int32_t *topk_idx, float *gates, float *clean, float *raw_noise,
-                float *kth_vals, int32_t *kth_idx, void *ws_base, Carver &cv, cudaStream_t st) {
+                float *kth_vals, int32_t *kth_idx, void *ws_base, Carver &cv, cudaStream_t st, const HierIdx *keep = nullptr) {
     GateWs w(cv, D);
+    const HierIdx H = keep ? *keep : w.H;
     // the status word of the workspace is cleared by the first kernel
     int32_t *status = status_word(ws_base);
     if (D.T == 0) MOE_TRY(reset_status(ws_base, st));
@@ -366,15 +371,14 @@ int32_t do_gate(const moe_config *c, const Dims &D, const void *x, const float *
     // not provably that of the fixed fma chain are redone with the chain; otherwise the chain does all rows.
     auto first_gate = [&](int32_t n1, int32_t k1, int32_t *idx_out, float *gates_out) -> int32_t {
         if (w.screen) {
-            MOE_TRY(launch_gate_screen_prepare(x, D.act, D.T, (int32_t)D.d, n1, Wg, Wnoise, w.wsplit, w.wnorm, w.xnorm,
-                                               w.unsafe_count, w.wt, st, 1, true, status));
-            MOE_TRY(launch_tc_gate_fwd(x, D.T, (int32_t)D.d, n1, w.wsplit, w.cr, status_word(ws_base), st));
-            MOE_TRY(launch_gate_screen(w.cr, noise, w.xnorm, w.wnorm, (int32_t)D.d, D.T, n1, k1, idx_out, gates_out,
-                                       clean, raw_noise, kth_vals, kth_idx, w.unsafe_list, w.unsafe_low, w.unsafe_count,
-                                       w.chain_list, w.full_list, st, nullptr, 1, nullptr, w.unsafe_span));
+            MOE_TRY(launch_gate_screen_prepare(x, D.T, (int32_t)D.d, n1, Wg, Wnoise, w.wsplit, w.wnorm, w.xnorm, w.unsafe_count,
+                                               w.wt, st, 1, true, status));
+            MOE_TRY(launch_tc_gate_fwd(x, D.T, (int32_t)D.d, n1, w.wsplit, clean, raw_noise, status_word(ws_base), st));
+            MOE_TRY(launch_gate_screen(noise, w.xnorm, w.wnorm, (int32_t)D.d, D.T, n1, k1, idx_out, gates_out, clean, raw_noise, kth_vals,
+                                       kth_idx, w.unsafe_list, w.unsafe_low, w.unsafe_count, w.chain_list, w.full_list, w.unsafe_span, st,
+                                       nullptr, 1, nullptr));
             // exact chains for the few columns that decide an uncertain row; whole rows only where there are many
-            MOE_TRY(launch_gate_chains(x, D.act, (int32_t)D.d, n1, w.wt, w.chain_list, w.unsafe_count + 1, clean, raw_noise,
-                                       st));
+            MOE_TRY(launch_gate_chains(x, (int32_t)D.d, n1, w.wt, w.chain_list, w.unsafe_count + 1, clean, raw_noise, st));
             MOE_TRY(launch_projection(x, D.act, D.T, (int32_t)D.d, n1, Wg, Wnoise, clean, raw_noise, nullptr, 0,
                                       w.full_list, 1, nullptr, st, w.unsafe_count + 2));
             return launch_gate_select(clean, raw_noise, noise, D.T, n1, k1, idx_out, gates_out, kth_vals, kth_idx, st,
@@ -388,36 +392,36 @@ int32_t do_gate(const moe_config *c, const Dims &D, const void *x, const float *
     // primary gate over the a groups
     const int64_t P1 = D.T * D.k1;
     float *g_p = gates + D.T * D.k, *g_s = g_p + P1;
-    MOE_TRY(first_gate((int32_t)D.a, (int32_t)D.k1, w.idx_p, g_p));
+    MOE_TRY(first_gate((int32_t)D.a, (int32_t)D.k1, H.idx_p, g_p));
     // secondary gates: rows (t, s1) grouped by their group so each tile uses one group's matrices
-    MOE_TRY(launch_dispatch_index(w.idx_p, P1, (int32_t)D.a, w.perm_p, w.inv_perm_p, w.counts_p, w.offsets_p,
-                                  w.scratch, st));
+    MOE_TRY(launch_dispatch_index(H.idx_p, P1, (int32_t)D.a, H.perm_p, H.inv_perm_p, H.counts_p, H.offsets_p,
+                                  w.H.scratch, st));
     const int64_t lp = D.T * D.a;  // elements of the primary part of the logits tensors
     const float *Wg_s = Wg + D.d * D.a, *Wn_s = Wnoise + D.d * D.a;
+    const HierMerge merge = {topk_idx, gates, H.idx_p, g_p, (int32_t)D.b};
     if (w.screen2) {
         // the routing screen on the grouped product: token rows gathered by group, one weight pair per group
-        MOE_TRY(launch_dispatch_rows(x, D.act, D.T, (int32_t)D.k1, (int32_t)D.d, w.inv_perm_p, w.xs_p, st));
-        MOE_TRY(launch_gate_screen_prepare(x, D.act, D.T, (int32_t)D.d, (int32_t)D.b, Wg_s, Wn_s, w.wsplit_s, w.wnorm_s,
-                                           w.xnorm, w.unsafe_count_s, w.wt_s, st, (int32_t)D.a, !w.screen));
-        MOE_TRY(launch_tc_gate_fwd_grouped(w.xs_p, P1, (int32_t)D.d, (int32_t)D.a, (int32_t)D.b, w.wsplit_s, w.offsets_p,
-                                           w.tile_prefix, w.cr_s, status_word(ws_base), st, D.flags));
-        MOE_TRY(launch_gate_screen(w.cr_s, noise + lp, w.xnorm, w.wnorm_s, (int32_t)D.d, P1, (int32_t)D.b, (int32_t)D.k2,
-                                   w.idx_s, g_s, clean + lp, raw_noise + lp, kth_vals + 2 * D.T, kth_idx + 2 * D.T,
-                                   w.unsafe_list_s, w.unsafe_low_s, w.unsafe_count_s, w.chain_list_s, nullptr, st, w.perm_p,
-                                   (int32_t)D.k1, w.idx_p, w.unsafe_span_s));
-        MOE_TRY(launch_gate_chains(x, D.act, (int32_t)D.d, (int32_t)D.b, w.wt_s, w.chain_list_s, w.unsafe_count_s + 1,
+        MOE_TRY(launch_dispatch_rows(x, D.act, D.T, (int32_t)D.k1, (int32_t)D.d, H.inv_perm_p, w.xs_p, st));
+        MOE_TRY(launch_gate_screen_prepare(x, D.T, (int32_t)D.d, (int32_t)D.b, Wg_s, Wn_s, w.wsplit_s, w.wnorm_s, w.xnorm,
+                                           w.unsafe_count_s, w.wt_s, st, (int32_t)D.a, !w.screen));
+        MOE_TRY(launch_tc_gate_fwd_grouped(w.xs_p, P1, (int32_t)D.d, (int32_t)D.a, (int32_t)D.b, w.wsplit_s, H.offsets_p,
+                                           w.H.tile_prefix, H.perm_p, clean + lp, raw_noise + lp, status_word(ws_base), st, D.flags));
+        MOE_TRY(launch_gate_screen(noise + lp, w.xnorm, w.wnorm_s, (int32_t)D.d, P1, (int32_t)D.b, (int32_t)D.k2, H.idx_s, g_s,
+                                   clean + lp, raw_noise + lp, kth_vals + 2 * D.T, kth_idx + 2 * D.T, w.unsafe_list_s, w.unsafe_low_s,
+                                   w.unsafe_count_s, w.chain_list_s, nullptr, w.unsafe_span_s, st, H.perm_p, (int32_t)D.k1, H.idx_p,
+                                   merge));
+        MOE_TRY(launch_gate_chains(x, (int32_t)D.d, (int32_t)D.b, w.wt_s, w.chain_list_s, w.unsafe_count_s + 1,
                                    clean + lp, raw_noise + lp, st, (int32_t)D.k1));
-        MOE_TRY(launch_gate_select(clean + lp, raw_noise + lp, noise + lp, P1, (int32_t)D.b, (int32_t)D.k2, w.idx_s, g_s,
+        MOE_TRY(launch_gate_select(clean + lp, raw_noise + lp, noise + lp, P1, (int32_t)D.b, (int32_t)D.k2, H.idx_s, g_s,
                                    kth_vals + 2 * D.T, kth_idx + 2 * D.T, st, w.unsafe_list_s, w.unsafe_count_s, w.unsafe_span_s,
-                                   w.chain_list_s));
+                                   w.chain_list_s, merge));
     } else {
         MOE_TRY(launch_projection(x, D.act, P1, (int32_t)D.d, (int32_t)D.b, Wg_s, Wn_s, clean + lp, raw_noise + lp,
-                                  w.offsets_p, (int32_t)D.a, w.perm_p, (int32_t)D.k1, w.tile_prefix, st));
-        MOE_TRY(launch_gate_select(clean + lp, raw_noise + lp, noise + lp, P1, (int32_t)D.b, (int32_t)D.k2, w.idx_s,
-                                   g_s, kth_vals + 2 * D.T, kth_idx + 2 * D.T, st));
+                                  H.offsets_p, (int32_t)D.a, H.perm_p, (int32_t)D.k1, w.H.tile_prefix, st));
+        MOE_TRY(launch_gate_select(clean + lp, raw_noise + lp, noise + lp, P1, (int32_t)D.b, (int32_t)D.k2, H.idx_s,
+                                   g_s, kth_vals + 2 * D.T, kth_idx + 2 * D.T, st, nullptr, nullptr, nullptr, nullptr, merge));
     }
-    return launch_hier_merge(D.T, (int32_t)D.k1, (int32_t)D.k2, (int32_t)D.b, w.idx_p, g_p, w.idx_s, g_s, topk_idx,
-                             gates, st);
+    return MOE_OK;
 }
 
 int32_t do_dispatch(const Dims &D, const void *x, const int32_t *topk_idx, void *xs, int32_t *perm,
@@ -472,7 +476,7 @@ int32_t do_expert_ffn(const moe_config *c, const Dims &D, const void *xs, const 
 int32_t do_losses(const moe_config *c, const Dims &D, const int32_t *topk_idx, const float *gates,
                   const float *clean, const float *raw_noise, const float *kth_vals, float *importance, float *load,
                   float *losses, const int32_t *perm, const int32_t *offsets, Carver &cv, cudaStream_t st,
-                  const LossOut &copy = LossOut{}) {
+                  const LossOut &copy = LossOut{}, const HierIdx *ready = nullptr) {
     LossesWs w(cv, D);
     if (!D.hier) {
         const LossFinal fin = {c->w_importance, c->w_load, losses, copy};
@@ -488,16 +492,14 @@ int32_t do_losses(const moe_config *c, const Dims &D, const int32_t *topk_idx, c
     }
     MOE_TRY(launch_segment_sum(gates, perm, offsets, (int32_t)D.n, importance, st));
     // Eq. 14: Load_primary, the per-group Load_i over X^(i), |X^(i)|
-    MOE_TRY(w.H.build(D, topk_idx, st));
+    MOE_TRY(w.H.build(D, topk_idx, ready, st));
     const int64_t ab = D.a * D.b, lp = D.T * D.a;
-    float *load_p = load + ab, *load_s = load_p + D.a;
+    float *load_p = load + ab;
     MOE_TRY(launch_level_sums(w.H.idx_p, gates + D.T * D.k, clean, raw_noise, kth_vals, D.T, (int32_t)D.a,
                               (int32_t)D.k1, nullptr, load_p, w.scratch, st));
-    MOE_TRY(launch_grouped_load(w.H.idx_s, clean + lp, raw_noise + lp, kth_vals + 2 * D.T, w.H.perm_p, w.H.offsets_p,
-                                (int32_t)D.a, D.T * D.k1, (int32_t)D.b, (int32_t)D.k2, load_s, w.grouped,
-                                w.H.tile_prefix, st));
-    MOE_TRY(launch_load_h(load, w.H.counts_p, (int32_t)D.a, (int32_t)D.b, st));
-    return launch_cv2(importance, (int32_t)ab, load, (int32_t)ab, c->w_importance, c->w_load, losses, st, copy);
+    return launch_grouped_load(w.H.idx_s, clean + lp, raw_noise + lp, kth_vals + 2 * D.T, w.H.perm_p, w.H.offsets_p, w.H.counts_p,
+                               (int32_t)D.a, D.T * D.k1, (int32_t)D.b, (int32_t)D.k2, importance, load, w.grouped,
+                               LossFinal{c->w_importance, c->w_load, losses, copy}, st);
 }
 
 int32_t do_expert_ffn_bwd(const moe_config *c, const Dims &D, const void *xs, const void *hid, const void *dys,
@@ -585,13 +587,14 @@ int32_t do_gate_bwd(const moe_config *c, const Dims &D, const void *x, const flo
                     const float *noise, const float *clean, const float *raw_noise, const int32_t *topk_idx,
                     const float *gates, const float *kth_vals, const int32_t *kth_idx, float *dgates,
                     const float *dload, float *dWg, float *dWnoise, float *dX_gate, void *ws_base, Carver &cv,
-                    cudaStream_t st) {
+                    cudaStream_t st, const HierIdx *ready = nullptr, SecondaryRows *sec = nullptr) {
+    // sec: the caller adds the secondary gates' rows to dX_gate itself (they stay in the scratch)
     GateBwdWs w(cv, D);
     if (D.hier) {
         const int64_t P1 = D.T * D.k1, lp = D.T * D.a, wp = D.d * D.a;
         const float *g_p = gates + D.T * D.k, *g_s = g_p + P1;
         float *dg_p = dgates + D.T * D.k, *dg_s = dg_p + P1;
-        MOE_TRY(w.H.build(D, topk_idx, st));
+        MOE_TRY(w.H.build(D, topk_idx, ready, st));
         MOE_TRY(launch_hier_gate_product_bwd(gates, dgates, D.T, (int32_t)D.k1, (int32_t)D.k2, st));
         if (w.tc_hier) {
             // both levels on the tensor cores: split logit gradients (the secondary ones written in the
@@ -608,6 +611,10 @@ int32_t do_gate_bwd(const moe_config *c, const Dims &D, const void *x, const flo
                                                  w.H.tile_prefix, (int32_t)D.a, P1, (int32_t)D.d, (int32_t)D.b,
                                                  w.partials_s, dWg + wp, dWnoise + wp, w.dX_sec, status_word(ws_base),
                                                  st));
+            if (sec) {
+                *sec = {w.dX_sec, w.H.inv_perm_p, (int32_t)D.k1};
+                return MOE_OK;
+            }
             return launch_dispatch_bwd(w.dX_sec, MOE_F32, w.H.inv_perm_p, D.T, (int32_t)D.k1, (int32_t)D.d, dX_gate,
                                        dX_gate, nullptr, st);
         }
@@ -635,6 +642,10 @@ int32_t do_gate_bwd(const moe_config *c, const Dims &D, const void *x, const flo
         g.b_e = D.d * D.b;
         g.a_row_index = w.H.perm_p; g.a_row_div = 1; g.c_row_index = w.H.perm_p;
         MOE_TRY(launch_simt_gemm(g, w.H.tile_prefix, st));
+        if (sec) {
+            *sec = {w.dX_sec, nullptr, (int32_t)D.k1};
+            return MOE_OK;
+        }
         return launch_add_slot_rows(w.dX_sec, D.T, (int32_t)D.k1, (int32_t)D.d, dX_gate, st);
     }
     MOE_TRY(launch_gate_logit_grads(noise, clean, raw_noise, topk_idx, gates, kth_vals, kth_idx, dgates, dload,
@@ -898,7 +909,7 @@ static int32_t forward_impl(const moe_config *cfg, const void *x, const float *W
     auto fresh = [&]() { Carver cv(ws); cv.take_bytes(kWsHeader); return cv; };
     { Carver cv = fresh();
       MOE_TRY(do_gate(cfg, D, x, Wg, Wnoise, noise, C.topk_idx, C.gates, C.clean, C.raw_noise, C.kth_vals,
-                      C.kth_idx, ws, cv, st)); }
+                      C.kth_idx, ws, cv, st, &C.hier)); }
     { Carver cv = fresh();
       MOE_TRY(do_dispatch(D, x, C.topk_idx, C.xs, C.perm, C.inv_perm, C.counts, C.offsets, cv, st)); }
     { Carver cv = fresh();
@@ -909,7 +920,7 @@ static int32_t forward_impl(const moe_config *cfg, const void *x, const float *W
     { Carver cv = fresh();
       MOE_TRY(do_losses(cfg, D, C.topk_idx, C.gates, C.clean, C.raw_noise, C.kth_vals, C.importance, C.load,
                         C.losses, C.perm, C.offsets, cv, st,
-                        LossOut{losses, importance, load, counts, C.counts, (int32_t)D.n, (int32_t)D.load})); }
+                        LossOut{losses, importance, load, counts, C.counts, (int32_t)D.n, (int32_t)D.load}, &C.hier)); }
     return MOE_OK;
 }
 
@@ -977,12 +988,13 @@ static int32_t backward_impl(const moe_config *cfg, const void *dY, const void *
       }
       MOE_TRY(do_expert_ffn_bwd(cfg, D, C.xs, hid, B.dys, C.offsets, W1, W2, B.dxs, dW1, db1, dW2, db2, ws, cv,
                                 st, plan, bits)); }
+    SecondaryRows sec = {};
     { Carver cv = fresh();
       MOE_TRY(do_gate_bwd(cfg, D, x, Wg, Wnoise, noise, C.clean, C.raw_noise, C.topk_idx, C.gates, C.kth_vals,
-                          C.kth_idx, B.dgates, B.dload, dWg, dWnoise, B.dX_gate, ws, cv, st)); }
+                          C.kth_idx, B.dgates, B.dload, dWg, dWnoise, B.dX_gate, ws, cv, st, &C.hier, &sec)); }
     // dX = expert path + gating path (+ the upstream gradient itself through the residual connection)
     return launch_dispatch_bwd(B.dxs, D.act, C.inv_perm, D.T, (int32_t)D.k, (int32_t)D.d, B.dX_gate, nullptr, dX,
-                               st, keep_bits ? dY : nullptr);
+                               st, keep_bits ? dY : nullptr, sec);
 }
 
 int32_t moe_backward(const moe_config *cfg, const void *dY, const void *x, const float *Wg, const float *Wnoise,

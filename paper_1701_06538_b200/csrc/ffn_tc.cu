@@ -65,6 +65,11 @@ struct GemmParams {
     int32_t K;  // ROW_*: contraction length of one term; WGRAD: unused (segment rows)
     bf16 *out;  // ROW_*: [R, N]; WGRAD: [nseg, M, N]
     float *out_f32;    // if set, results are written here as float instead of `out`
+    // float results of two matrices side by side: columns from split_n on go to out2, both with rows of split_n (a multiple of 32);
+    // out_rows: where an output row goes (rows sorted by group); out_words: rows that do not start on 16 bytes
+    float *out2;
+    const int32_t *out_rows;
+    int32_t split_n, out_words;
     const bf16 *bias;  // [nseg, N] or nullptr
     const bf16 *mask;  // [R, N] or nullptr: result kept where mask > 0
     // the same mask as one bit per element, [R, N / 32] words (bit j of word c: column 32 c + j): bits_out is written by
@@ -370,12 +375,26 @@ __device__ __forceinline__ void epilogue_box(const GemmParams &p, int lane, cons
                 *reinterpret_cast<uint4 *>(b.box + lane * 128 + ((q ^ (lane & 7)) << 4)) =
                     make_uint4(v[u][4 * q], v[u][4 * q + 1], v[u][4 * q + 2], v[u][4 * q + 3]);
             __syncwarp();
+            const int32_t col = b.col0 + 32 * u;
+            float *dst = p.out_f32 + b.out_off + col + my_piece * 4;
+            int64_t pitch = p.N;
+            if (p.out2) {
+                dst = (col < p.split_n ? p.out_f32 + col : p.out2 + (col - p.split_n)) + my_piece * 4;
+                pitch = p.split_n;
+            }
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const int row = 4 * i + my_sub;
-                if (row < b.rows_valid)
-                    *reinterpret_cast<uint4 *>(p.out_f32 + b.out_off + (b.row0 + row) * p.N + b.col0 + 32 * u + my_piece * 4) =
-                        *reinterpret_cast<const uint4 *>(b.box + row * 128 + ((my_piece ^ (row & 7)) << 4));
+                if (row < b.rows_valid) {
+                    const uint4 v = *reinterpret_cast<const uint4 *>(b.box + row * 128 + ((my_piece ^ (row & 7)) << 4));
+                    float *at = dst + (p.out_rows ? (int64_t)p.out_rows[b.row0 + row] : b.row0 + row) * pitch;
+                    if (!p.out_words) {
+                        *reinterpret_cast<uint4 *>(at) = v;
+                    } else {
+                        at[0] = __uint_as_float(v.x); at[1] = __uint_as_float(v.y);
+                        at[2] = __uint_as_float(v.z); at[3] = __uint_as_float(v.w);
+                    }
+                }
             }
             __syncwarp();
         }
@@ -1888,7 +1907,11 @@ int32_t launch_tc_gate_bwd(const void *x, int64_t T, int32_t d, int32_t n, const
     return MOE_OK;
 }
 
-// Forward gate projection for the routing screen: cr = x . (W_lo + W_mid + W_hi), smallest term first.
+// Forward gate projection for the routing screen: clean | raw = x . (W_lo + W_mid + W_hi), smallest term first.
+static void two_outputs(GemmParams &p, float *clean, float *raw, int32_t n) {
+    p.out_f32 = clean; p.out2 = raw; p.split_n = n;
+    p.out_words = ((reinterpret_cast<uintptr_t>(clean) | reinterpret_cast<uintptr_t>(raw)) & 15) != 0;
+}
 bool tc_gate_fwd_supported(int32_t act, int64_t T, int32_t d, int32_t n, int32_t flags) {
     // MOE_FLAG_GATE_SCREEN_OFF: every token through the fma chain; _ON: screen whenever the shapes allow;
     // neither: screen when the projection is large enough to pay for the extra launches
@@ -1898,14 +1921,15 @@ bool tc_gate_fwd_supported(int32_t act, int64_t T, int32_t d, int32_t n, int32_t
     return (double)T * d * 2.0 * n >= 1.0e9;
 }
 
-int32_t launch_tc_gate_fwd(const void *x, int64_t T, int32_t d, int32_t n, const void *wsplit, float *cr,
+int32_t launch_tc_gate_fwd(const void *x, int64_t T, int32_t d, int32_t n, const void *wsplit, float *clean, float *raw,
                            int32_t *status, cudaStream_t st) {
     const int32_t n2 = 2 * n;
     CUtensorMap tmA, tmB;
     MOE_TRY(map_rows_kmajor(&tmA, x, T, d));
     MOE_TRY(map_weight_mnmajor_half(&tmB, wsplit, 1, 3 * (int64_t)d, n2));
     GemmParams p = default_params();
-    p.nseg = 1; p.N = n2; p.K = d; p.R = T; p.out_f32 = cr; p.status = status;
+    p.nseg = 1; p.N = n2; p.K = d; p.R = T; p.status = status;
+    two_outputs(p, clean, raw, n);
     p.nterms = 3;
     for (int i = 0; i < 3; ++i) { p.a_term_col[i] = 0; p.b_term_col[i] = (2 - i) * d; }
     return launch2<ROW_BMN>(tmA, tmB, p, cdiv(T, 256) * cdiv(n2, BN), st);
@@ -1913,10 +1937,10 @@ int32_t launch_tc_gate_fwd(const void *x, int64_t T, int32_t d, int32_t n, const
 
 // The same for the secondary gates of the hierarchical layer: rows = the slots (t, s1) sorted by primary group
 // (xs_p [P1, d], offsets_p [a + 1]), one [d, 2b] weight pair per group. wsplit_s [3][a * d][2b] (term, group, feature);
-// cr_s [P1, 2b] comes out in sorted order.
+// Sorted row r's logits go to row perm_p[r] of clean / raw [P1, b].
 int32_t launch_tc_gate_fwd_grouped(const void *xs_p, int64_t P1, int32_t d, int32_t a, int32_t b, const void *wsplit_s,
-                                   const int32_t *offsets_p, int32_t *tile_prefix, float *cr_s, int32_t *status,
-                                   cudaStream_t st, int32_t flags) {
+                                   const int32_t *offsets_p, int32_t *tile_prefix, const int32_t *perm_p, float *clean, float *raw,
+                                   int32_t *status, cudaStream_t st, int32_t flags) {
     if (P1 == 0) return MOE_OK;
     const int32_t n2 = 2 * b;
     const bool pairs = use_two_cta(P1, a, flags);
@@ -1930,7 +1954,9 @@ int32_t launch_tc_gate_fwd_grouped(const void *xs_p, int64_t P1, int32_t d, int3
     }
     GemmParams p = default_params();
     p.offsets = offsets_p; p.tile_prefix = tile_prefix; p.tile_info = tile_info_of(tile_prefix, a);
-    p.nseg = a; p.N = n2; p.K = d; p.R = P1; p.out_f32 = cr_s; p.status = status;
+    p.nseg = a; p.N = n2; p.K = d; p.R = P1; p.status = status;
+    two_outputs(p, clean, raw, b);
+    p.out_rows = perm_p;
     p.nterms = 3;
     for (int i = 0; i < 3; ++i) { p.a_term_col[i] = 0; p.b_term_col[i] = (2 - i) * a * d; }  // lo, mid, hi
     const int32_t tm = pairs ? 256 : BM;

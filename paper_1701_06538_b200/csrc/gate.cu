@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(256) gate_select_kernel(const float *__restric
                                                           const int32_t *__restrict__ row_list,
                                                           const int32_t *__restrict__ row_count,
                                                           const int2 *__restrict__ row_span,
-                                                          const int2 *__restrict__ chain_list) {
+                                                          const int2 *__restrict__ chain_list, const HierMerge merge) {
     wait_previous_kernel();
     extern __shared__ float staged[];  // [rows of the block][n]
     const int lane = threadIdx.x & 31, rpb = STAGED ? select_rows_per_block(n) : blockDim.x >> 5;
@@ -130,8 +130,10 @@ __global__ void __launch_bounds__(256) gate_select_kernel(const float *__restric
     float den = 0.0f;
     for (int s = 0; s < k; ++s) den += __shfl_sync(0xffffffffu, ex, s);
     if (lane < k) {
+        const float g = ex / den;
         idx[row * k + lane] = myi;
-        gates[row * k + lane] = ex / den;
+        gates[row * k + lane] = g;
+        if (merge.idx) merge.put(row, k, lane, myi, g);
     }
     if (lane == 0) {
         kth_vals[row * 2 + 0] = v_k;
@@ -144,7 +146,7 @@ __global__ void __launch_bounds__(256) gate_select_kernel(const float *__restric
 int32_t launch_gate_select(const float *clean, const float *raw, const float *noise, int64_t rows, int32_t n,
                            int32_t k, int32_t *idx, float *gates, float *kth_vals, int32_t *kth_idx,
                            cudaStream_t st, const int32_t *row_list, const int32_t *row_count, const void *row_span,
-                           const void *chain_list) {
+                           const void *chain_list, const HierMerge &merge) {
     if (rows == 0) return MOE_OK;
     // Staged up to eight rows per SM, wider rows up to n / 32 of them. A whole moe_gate with 16 features, staged / unstaged us:
     // n = 129 (half of a step's threads idle): 1019 rows 12.3 / 11.8, 2048 rows 15.8 / 13.2, 65536 rows 239 / 170; n = 256: 12.1 / 13.6,
@@ -156,7 +158,7 @@ int32_t launch_gate_select(const float *clean, const float *raw, const float *no
     const size_t sh = stage ? sizeof(float) * rpb * n : 0;  // at most 32 KiB
 #define MOE_SELECT_AS(KL, STAGED)                                                                                        \
     launch_kernel((gate_select_kernel<KL, STAGED>), grid, 256, sh, st, clean, raw, noise, rows, n, k, idx, gates, kth_vals, \
-                  kth_idx, row_list, row_count, (const int2 *)row_span, (const int2 *)chain_list)
+                  kth_idx, row_list, row_count, (const int2 *)row_span, (const int2 *)chain_list, merge)
 #define MOE_SELECT(KL)                        \
     do {                                      \
         if (stage) MOE_SELECT_AS(KL, true);   \
@@ -183,73 +185,93 @@ int32_t launch_gate_select(const float *clean, const float *raw, const float *no
 // same, so the routing taken from the approximate logits IS the bit-exact routing. The other tokens
 // (a few per cent) are listed and redone with the fma chain by the kernels above.
 // ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) split_gate_weights_kernel(const float *__restrict__ Wg,
-                                                                 const float *__restrict__ Wn, int32_t d, int32_t n,
-                                                                 bf16 *__restrict__ wsplit) {
+// What the screen needs beside its product, in one launch. The first blocks take 32 columns of [W_g | W_noise] each (of one group
+// where matrices are stacked [groups, d, n]) and walk down the features, four 32 x 32 tiles in flight: the three-term bf16 split
+// wsplit [3][groups * d][2n], the transposed weights wt [groups][2n][d] for single chains, and the columns' norms (slightly rounded
+// up) wnorm [groups][2n]. The other blocks: |x_t|_2 (slightly rounded up), one warp per row, 16 bytes per lane, four loads in flight.
+__global__ void __launch_bounds__(256) gate_prepare_kernel(const bf16 *__restrict__ x, int64_t T, int32_t d, int32_t n,
+                                                           const float *__restrict__ Wg, const float *__restrict__ Wn,
+                                                           int32_t groups, bf16 *__restrict__ wsplit, float *__restrict__ wt,
+                                                           float *__restrict__ wnorm, float *__restrict__ xnorm,
+                                                           int32_t *__restrict__ counters, int32_t *__restrict__ clear) {
     wait_previous_kernel();
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int32_t n2 = 2 * n;
-    if (i >= (int64_t)d * n2) return;
-    const int32_t q = (int32_t)(i / n2), j = (int32_t)(i % n2);
-    float v = j < n ? Wg[(int64_t)q * n + j] : Wn[(int64_t)q * n + (j - n)];
+    const int32_t n2 = 2 * n, column_blocks = groups * (n2 / 32);
+    if ((int32_t)blockIdx.x >= column_blocks) {
+        const int lane = threadIdx.x & 31;
+        const int64_t t = (int64_t)(blockIdx.x - column_blocks) * 8 + (threadIdx.x >> 5);
+        if (t >= T) return;
+        float s = 0.0f;
+        const uint4 *row = reinterpret_cast<const uint4 *>(x + t * d);
+        const int32_t pieces = d / 8;
+        for (int32_t q0 = lane; q0 < pieces; q0 += 128) {
+            uint4 v[4];
 #pragma unroll
-    for (int term = 0; term < 3; ++term) {  // wsplit[term][q][j]: hi, mid, lo
-        const bf16 b = __float2bfloat16_rn(v);
-        wsplit[((int64_t)term * d + q) * n2 + j] = b;
-        v -= __bfloat162float(b);
+            for (int i = 0; i < 4; ++i) v[i] = q0 + 32 * i < pieces ? row[q0 + 32 * i] : make_uint4(0, 0, 0, 0);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const bf16 *h = reinterpret_cast<const bf16 *>(&v[i]);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) { const float f = __bfloat162float(h[e]); s = fmaf(f, f, s); }
+            }
+        }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        if (lane == 0) xnorm[t] = sqrtf(s) * (1.0f + 1e-5f);
+        return;
     }
-}
-
-// one warp per column of [W_g | W_noise]; blockIdx.y = group (stacked [groups, d, n] matrices)
-__global__ void __launch_bounds__(256) gate_col_norms_kernel(const float *__restrict__ Wg, const float *__restrict__ Wn,
-                                                             int32_t d, int32_t n, float *__restrict__ wnorm) {
-    wait_previous_kernel();
-    const int lane = threadIdx.x & 31;
-    const int32_t j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (j >= 2 * n) return;
-    Wg += (int64_t)blockIdx.y * d * n; Wn += (int64_t)blockIdx.y * d * n; wnorm += (int64_t)blockIdx.y * 2 * n;
-    const float *W = j < n ? Wg + j : Wn + (j - n);
-    double s = 0.0;
-    for (int32_t q = lane; q < d; q += 32) { const double v = W[(int64_t)q * n]; s += v * v; }
+    if (blockIdx.x == 0) {  // rows to re-select, chains, full-chain rows; the status word
+        if (threadIdx.x < 4) counters[threadIdx.x] = 0;
+        if (threadIdx.x == 4 && clear) *clear = 0;
+    }
+    __shared__ float tile[4][32][33];
+    __shared__ double sums[8][32];
+    const int32_t group = blockIdx.x / (n2 / 32), c0 = (blockIdx.x % (n2 / 32)) * 32;  // 2n and d are multiples of 64 on this path
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int32_t c = c0 + tx;
+    const float *W = (c < n ? Wg + c : Wn + (c - n)) + (int64_t)group * d * n;
+    wt += ((int64_t)group * n2 + c0) * d;
+    double sum = 0.0;
+    for (int32_t q0 = 0; q0 < d; q0 += 128) {
+        const int tiles = min(4, (d - q0) / 32);
+        float v[4][4];
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    if (lane == 0) wnorm[j] = (float)(sqrt(s) * (1.0 + 1e-6));
-}
-
-// |x_t|_2 (slightly rounded up), one warp per row; bf16 rows are read 16 bytes per lane, four loads in flight
-template <typename XT>
-__global__ void __launch_bounds__(256) row_norms_kernel(const XT *__restrict__ x, int64_t T, int32_t d,
-                                                        float *__restrict__ xnorm) {
-    wait_previous_kernel();
-    const int lane = threadIdx.x & 31;
-    const int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (t >= T) return;
-    float s = 0.0f;
-    if constexpr (sizeof(XT) == 2) {
-        if (d % 8 == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0) {
-            const uint4 *row = reinterpret_cast<const uint4 *>(x + t * d);
-            const int32_t pieces = d / 8;
-            for (int32_t q0 = lane; q0 < pieces; q0 += 128) {
-                uint4 v[4];
+        for (int b = 0; b < 4; ++b)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) v[i] = q0 + 32 * i < pieces ? row[q0 + 32 * i] : make_uint4(0, 0, 0, 0);
+            for (int i = 0; i < 4; ++i) v[b][i] = b < tiles ? W[(int64_t)(q0 + 32 * b + ty + 8 * i) * n] : 0.0f;
+        __syncthreads();  // the tiles before have been read
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const bf16 *h = reinterpret_cast<const bf16 *>(&v[i]);
+        for (int b = 0; b < 4; ++b) {
+            if (b >= tiles) break;
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) { const float f = __bfloat162float(h[e]); s = fmaf(f, f, s); }
+            for (int i = 0; i < 4; ++i) {
+                float f = v[b][i];
+                sum += (double)f * (double)f;
+                tile[b][ty + 8 * i][tx] = f;
+                const int64_t q = (int64_t)group * d + q0 + 32 * b + ty + 8 * i;
+#pragma unroll
+                for (int term = 0; term < 3; ++term) {  // hi, mid, lo
+                    const bf16 h = __float2bfloat16_rn(f);
+                    wsplit[((int64_t)term * groups * d + q) * n2 + c] = h;
+                    f -= __bfloat162float(h);
                 }
             }
+        }
+        __syncthreads();
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-            if (lane == 0) xnorm[t] = sqrtf(s) * (1.0f + 1e-5f);
-            return;
+        for (int b = 0; b < 4; ++b) {
+            if (b >= tiles) break;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) wt[(int64_t)(ty + 8 * i) * d + q0 + 32 * b + tx] = tile[b][tx][ty + 8 * i];
         }
     }
-    for (int32_t q = lane; q < d; q += 32) { const float v = to_f32(x[t * d + q]); s = fmaf(v, v, s); }
+    sums[ty][tx] = sum;
+    __syncthreads();
+    if (ty == 0) {
+        double s = sums[0][tx];
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    if (lane == 0) xnorm[t] = sqrtf(s) * (1.0f + 1e-5f);
+        for (int q = 1; q < 8; ++q) s += sums[q][tx];
+        wnorm[group * n2 + c] = (float)(sqrt(s) * (1.0 + 1e-6));
+    }
 }
 
 // Approximate noisy logit v of one column and a bound u on its distance from the fma chain's value; c, r = the
@@ -268,16 +290,15 @@ __device__ __forceinline__ void screen_eval(float c, float r, float e, float xn,
     u = __fmaf_rn(2.0e-6f, ae, __fmaf_rn(xn, __fmaf_rn(ae, wn, wg), rounding));
 }
 
-// The screen, one thread per token (sorted row): a warp stages 16 columns of its 32 rows at a time through shared memory
-// (16-byte loads along the rows, 16-byte reads down the rows, both conflict free with a pitch of 20 words), copies
-// them to clean / raw on the way, and every thread then walks its own row: a sorted list of the KL >= k + 2 largest
-// approximate logits with their bounds, and the largest possible value of everything else. No shuffles, no arg-max
-// rounds: a few dozen instructions per column. Certified rows get their routing here; the others are listed
-// with `low`, the bound that decides which of their columns need an exact chain (gate_candidates_kernel).
-// Grouped use (secondary gates of the hierarchical layer): cr rows are sorted by group; perm maps a sorted row to its
-// output row (the slot t * k1 + s1), the token is output row / kdiv, group_of gives the slot's group, whose column
+// The screen. P adjacent lanes take a row (sorted row): each walks every P-th quad of its columns, one quad ahead in registers,
+// and keeps a sorted list of the KL >= k + 2 largest approximate logits with their
+// bounds and the largest possible value of everything else; the P lists are then merged by exchanging them. Bound by the
+// arithmetic of the list where the rows fill the chip, by the latency of one lane's walk where they do not, hence P by the
+// number of rows (see launch_gate_screen). Certified rows get their routing here; the others are listed with `low`, the
+// bound that decides which of their columns need an exact chain (gate_candidates_kernel).
+// Grouped use (secondary gates of the hierarchical layer): neighbours in a warp are of one group; perm maps a sorted row to its
+// row (the slot t * k1 + s1), the token is output row / kdiv, group_of gives the slot's group, whose column
 // norms are used. Flat use: perm = group_of = nullptr, kdiv = 1.
-constexpr int SCREEN_CH = 16, SCREEN_PITCH = 20;
 // four floats at p: one 16-byte access where the tensor allows it (V16), else four 4-byte ones (the secondary gates'
 // part of noise / clean / raw starts T * a floats into the tensor, not always a multiple of four)
 template <bool V16>
@@ -285,30 +306,24 @@ __device__ __forceinline__ float4 load4(const float *p) {
     if constexpr (V16) return *reinterpret_cast<const float4 *>(p);
     else return make_float4(p[0], p[1], p[2], p[3]);
 }
-template <bool V16>
-__device__ __forceinline__ void store4(float *p, float4 v) {
-    if constexpr (V16) *reinterpret_cast<float4 *>(p) = v;
-    else { p[0] = v.x; p[1] = v.y; p[2] = v.z; p[3] = v.w; }
-}
-template <int KL, bool V16>
-__global__ void __launch_bounds__(128) gate_screen_rows_kernel(const float *__restrict__ cr, const float *__restrict__ noise,
+template <int KL, int P, bool V16>
+__global__ void __launch_bounds__(128) gate_screen_rows_kernel(const float *__restrict__ noise,
                                                                const float *__restrict__ xnorm,
                                                                const float *__restrict__ wnorm, float theta, int64_t T,
                                                                int32_t n, int32_t k, int32_t *__restrict__ idx,
-                                                               float *__restrict__ gates, float *__restrict__ clean,
-                                                               float *__restrict__ raw, float *__restrict__ kth_vals,
+                                                               float *__restrict__ gates, const float *__restrict__ clean,
+                                                               const float *__restrict__ raw, float *__restrict__ kth_vals,
                                                                int32_t *__restrict__ kth_idx,
                                                                int32_t *__restrict__ unsafe_list,
                                                                float *__restrict__ unsafe_low,
                                                                int32_t *__restrict__ unsafe_count,
                                                                const int32_t *__restrict__ perm, int32_t kdiv,
-                                                               const int32_t *__restrict__ group_of) {
+                                                               const int32_t *__restrict__ group_of, const HierMerge merge) {
     wait_previous_kernel();
-    __shared__ __align__(16) float tile[4][3][32 * SCREEN_PITCH];
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    const int64_t s0 = ((int64_t)blockIdx.x * 4 + wp) * 32;  // first sorted row of this warp
+    const int lane = threadIdx.x & 31, sub = lane % P;
+    const int64_t s0 = ((int64_t)blockIdx.x * 4 + (threadIdx.x >> 5)) * (32 / P);  // first sorted row of this warp
     if (s0 >= T) return;
-    const int64_t srow = s0 + lane;
+    const int64_t srow = s0 + lane / P;
     const bool live = srow < T;
     const int64_t row = live ? (perm ? (int64_t)perm[srow] : srow) : 0;
     const float *wn = wnorm + (int64_t)(group_of && live ? group_of[row] : 0) * 2 * n;
@@ -320,8 +335,8 @@ __global__ void __launch_bounds__(128) gate_screen_rows_kernel(const float *__re
     float rest_hi = -CUDART_INF_F;  // largest possible chain value of anything that is not in the list
     auto insert = [&](int32_t j, float v, float u) {
         if (v > lv[KL - 1]) {
-            // enters the list behind every entry that is at least as large (those have lower indices), the last
-            // entry falls off
+            // enters the list behind every entry that is at least as large, the last entry falls off (equal values are
+            // never certified: their order does not matter here)
             rest_hi = fmaxf(rest_hi, lv[KL - 1] + lu[KL - 1]);
 #pragma unroll
             for (int s = KL - 1; s >= 1; --s) {
@@ -351,43 +366,28 @@ __global__ void __launch_bounds__(128) gate_screen_rows_kernel(const float *__re
         insert(j + 2, v2, u2);
         insert(j + 3, v3, u3);
     };
-    // loads: instruction i covers the rows 8 i + lane / 4 of the warp, four columns per lane
-    const int lr = lane >> 2, lq = (lane & 3) * 4;
-    float *tc = tile[wp][0], *tr = tile[wp][1], *te = tile[wp][2];
-    for (int32_t j0 = 0; j0 < n; j0 += SCREEN_CH) {
-        float4 c4[4], r4[4], e4[4];
-        int32_t orow[4];  // output rows fit 31 bits (they go into the int32 row lists)
+    const float *cp = clean + row * n + 4 * sub, *rp = raw + row * n + 4 * sub, *ep = noise + row * n + 4 * sub;  // a dead lane walks row 0
+    float4 c4 = load4<V16>(cp), r4 = load4<V16>(rp), e4 = load4<V16>(ep);  // n is a multiple of 4 P
+    for (int32_t j0 = 0; j0 < n; j0 += 4 * P) {
+        const int32_t next = j0 + 4 * P;
+        float4 cn = c4, rn = r4, en = e4;
+        if (next < n) { cn = load4<V16>(cp + next); rn = load4<V16>(rp + next); en = load4<V16>(ep + next); }
+        consider4(j0 + 4 * sub, c4, r4, e4);
+        c4 = cn; r4 = rn; e4 = en;
+    }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int64_t sr = s0 + 8 * i + lr;
-            orow[i] = __shfl_sync(0xffffffffu, (int32_t)row, 8 * i + lr);
-            c4[i] = r4[i] = e4[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            if (sr < T) {
-                c4[i] = load4<V16>(cr + sr * 2 * n + j0 + lq);
-                r4[i] = load4<V16>(cr + sr * 2 * n + n + j0 + lq);
-                e4[i] = load4<V16>(noise + (int64_t)orow[i] * n + j0 + lq);
-            }
-        }
+    for (int off = 1; off < P; off <<= 1) {  // afterwards every lane of the row holds the list of all columns
+        float ov[KL], ou[KL];
+        int32_t oi[KL];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int at = (8 * i + lr) * SCREEN_PITCH + lq;
-            *reinterpret_cast<float4 *>(tc + at) = c4[i];
-            *reinterpret_cast<float4 *>(tr + at) = r4[i];
-            *reinterpret_cast<float4 *>(te + at) = e4[i];
-            if (s0 + 8 * i + lr < T) {
-                store4<V16>(clean + (int64_t)orow[i] * n + j0 + lq, c4[i]);
-                store4<V16>(raw + (int64_t)orow[i] * n + j0 + lq, r4[i]);
-            }
+        for (int s = 0; s < KL; ++s) {
+            ov[s] = __shfl_xor_sync(0xffffffffu, lv[s], off);
+            ou[s] = __shfl_xor_sync(0xffffffffu, lu[s], off);
+            oi[s] = __shfl_xor_sync(0xffffffffu, li[s], off);
         }
-        __syncwarp();
+        rest_hi = fmaxf(rest_hi, __shfl_xor_sync(0xffffffffu, rest_hi, off));
 #pragma unroll
-        for (int q = 0; q < SCREEN_CH / 4; ++q) {
-            const float4 cq = *reinterpret_cast<const float4 *>(tc + lane * SCREEN_PITCH + 4 * q);
-            const float4 rq = *reinterpret_cast<const float4 *>(tr + lane * SCREEN_PITCH + 4 * q);
-            const float4 eq = *reinterpret_cast<const float4 *>(te + lane * SCREEN_PITCH + 4 * q);
-            consider4(j0 + 4 * q, cq, rq, eq);
-        }
-        __syncwarp();
+        for (int s = 0; s < KL; ++s) insert(oi[s], ov[s], ou[s]);
     }
     // the first `rounds` entries are the ranked ones, whatever else is in the list is "rest" as well
     const int rounds = min(k + 2, n);
@@ -425,7 +425,7 @@ __global__ void __launch_bounds__(128) gate_screen_rows_kernel(const float *__re
             }
         }
     }
-    const bool listed = live && !safe;
+    const bool listed = live && !safe && sub == 0;  // one lane of a row reports it
     const uint32_t lb = __ballot_sync(0xffffffffu, listed);
     if (lb) {
         int32_t base = 0;
@@ -437,7 +437,7 @@ __global__ void __launch_bounds__(128) gate_screen_rows_kernel(const float *__re
             unsafe_low[at] = low;
         }
     }
-    if (!live || !safe) return;
+    if (!live || !safe || sub != 0) return;
     float ex[KL], den = 0.0f;
 #pragma unroll
     for (int s = 0; s < KL; ++s) {
@@ -447,8 +447,10 @@ __global__ void __launch_bounds__(128) gate_screen_rows_kernel(const float *__re
 #pragma unroll
     for (int s = 0; s < KL; ++s)
         if (s < k) {
+            const float g = ex[s] / den;
             idx[row * k + s] = li[s];
-            gates[row * k + s] = ex[s] / den;
+            gates[row * k + s] = g;
+            if (merge.idx) merge.put(row, k, s, li[s], g);
         }
     float v_k = -CUDART_INF_F, v_k1 = -CUDART_INF_F;
     int32_t i_k = -1, i_k1 = -1;
@@ -549,8 +551,7 @@ __global__ void __launch_bounds__(256) gate_candidates_kernel(const float *__res
 // shared memory and every lane then reads its own row back. Loads for step s + 1 are in flight during the 32
 // dependent fused multiply-adds of step s.
 constexpr int CHAIN_PITCH = 144;  // bytes per staged row: 128 + 16, conflict-free both ways
-template <typename XT>
-__global__ void __launch_bounds__(128) gate_chain_kernel(const XT *__restrict__ x, int32_t d, int32_t n,
+__global__ void __launch_bounds__(128) gate_chain_kernel(const bf16 *__restrict__ x, int32_t d, int32_t n,
                                                          const float *__restrict__ Wt,
                                                          const int2 *__restrict__ chain_list,
                                                          const int32_t *__restrict__ chain_count,
@@ -566,7 +567,7 @@ __global__ void __launch_bounds__(128) gate_chain_kernel(const XT *__restrict__ 
     for (int32_t i0 = (blockIdx.x * 4 + wp) * 32; i0 < total; i0 += gridDim.x * 128) {  // warp-uniform
         const int32_t i = i0 + lane;
         const int2 en = chain_list[i < total ? i : total - 1];  // idle lanes shadow the last chain
-        const XT *xr = x + (int64_t)(en.x / kdiv) * d;
+        const bf16 *xr = x + (int64_t)(en.x / kdiv) * d;
         const float *wrow = Wt + (int64_t)en.y * d;
         // instruction u of a step loads 16 bytes of the row of lane 4 u + lane / 8, at byte (lane % 8) * 16
         const float *src[8];
@@ -580,10 +581,8 @@ __global__ void __launch_bounds__(128) gate_chain_kernel(const XT *__restrict__ 
         auto fetch = [&](int32_t st) {
 #pragma unroll
             for (int u = 0; u < 8; ++u) wreg[u] = *reinterpret_cast<const float4 *>(src[u] + st * 32);
-            if constexpr (sizeof(XT) == 2) {
 #pragma unroll
-                for (int g = 0; g < 4; ++g) xreg[g] = *reinterpret_cast<const uint4 *>(xr + st * 32 + 8 * g);
-            }
+            for (int g = 0; g < 4; ++g) xreg[g] = *reinterpret_cast<const uint4 *>(xr + st * 32 + 8 * g);
         };
         auto park = [&](int b) {
 #pragma unroll
@@ -604,17 +603,9 @@ __global__ void __launch_bounds__(128) gate_chain_kernel(const XT *__restrict__ 
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const float4 wv = *reinterpret_cast<const float4 *>(mine + 16 * u);
-                float x0, x1, x2, x3;
-                if constexpr (sizeof(XT) == 2) {
-                    const bf16 *hx = reinterpret_cast<const bf16 *>(&xcur[u >> 1]) + 4 * (u & 1);
-                    x0 = __bfloat162float(hx[0]); x1 = __bfloat162float(hx[1]);
-                    x2 = __bfloat162float(hx[2]); x3 = __bfloat162float(hx[3]);
-                } else {
-                    const int32_t q = st * 32 + 4 * u;
-                    x0 = to_f32(xr[q]); x1 = to_f32(xr[q + 1]); x2 = to_f32(xr[q + 2]); x3 = to_f32(xr[q + 3]);
-                }
-                acc = fmaf(x0, wv.x, acc); acc = fmaf(x1, wv.y, acc);
-                acc = fmaf(x2, wv.z, acc); acc = fmaf(x3, wv.w, acc);
+                const bf16 *hx = reinterpret_cast<const bf16 *>(&xcur[u >> 1]) + 4 * (u & 1);
+                acc = fmaf(__bfloat162float(hx[0]), wv.x, acc); acc = fmaf(__bfloat162float(hx[1]), wv.y, acc);
+                acc = fmaf(__bfloat162float(hx[2]), wv.z, acc); acc = fmaf(__bfloat162float(hx[3]), wv.w, acc);
             }
             if (st + 1 < steps) {
                 park((st + 1) & 1);  // the other buffer: its readers finished a step ago (syncwarp below)
@@ -631,66 +622,31 @@ __global__ void __launch_bounds__(128) gate_chain_kernel(const XT *__restrict__ 
     }
 }
 
-// Wt[c, q] = [W_g | W_noise][q, c]
-__global__ void __launch_bounds__(256) gate_transpose_weights_kernel(const float *__restrict__ Wg, const float *__restrict__ Wn,
-                                                                     int32_t d, int32_t n, float *__restrict__ Wt,
-                                                                     int32_t *__restrict__ counters, int32_t *__restrict__ clear) {
-    wait_previous_kernel();
-    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) {  // rows to re-select, chains, full-chain rows; the status word
-        if (threadIdx.x < 4) counters[threadIdx.x] = 0;
-        if (threadIdx.x == 4 && clear) *clear = 0;
-    }
-    __shared__ float tile[32][33];
-    Wg += (int64_t)blockIdx.z * d * n; Wn += (int64_t)blockIdx.z * d * n; Wt += (int64_t)blockIdx.z * 2 * n * d;  // group
-    const int q0 = blockIdx.x * 32, c0 = blockIdx.y * 32;  // 2n and d are multiples of 32 on this path
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    for (int i = ty; i < 32; i += 8) {
-        const int c = c0 + tx, q = q0 + i;
-        tile[i][tx] = c < n ? Wg[(int64_t)q * n + c] : Wn[(int64_t)q * n + (c - n)];
-    }
-    __syncthreads();
-    for (int i = ty; i < 32; i += 8) Wt[(int64_t)(c0 + i) * d + q0 + tx] = tile[tx][i];
-}
-
-int32_t launch_gate_chains(const void *x, int32_t act, int32_t d, int32_t n, const float *Wt, const void *chain_list,
+int32_t launch_gate_chains(const void *x, int32_t d, int32_t n, const float *Wt, const void *chain_list,
                            const int32_t *chain_count, float *clean, float *raw, cudaStream_t st, int32_t kdiv) {
-    const unsigned grid = 148 * 16;
-    if (act == MOE_BF16)
-        launch_kernel(gate_chain_kernel<bf16>, grid, 128, 0, st, (const bf16 *)x, d, n, Wt, (const int2 *)chain_list, chain_count, clean,
-                                                      raw, kdiv);
-    else
-        launch_kernel(gate_chain_kernel<float>, grid, 128, 0, st, (const float *)x, d, n, Wt, (const int2 *)chain_list, chain_count, clean,
-                                                       raw, kdiv);
+    launch_kernel(gate_chain_kernel, 148 * 16, 128, 0, st, (const bf16 *)x, d, n, Wt, (const int2 *)chain_list, chain_count, clean, raw, kdiv);
     MOE_LAUNCHED();
     return MOE_OK;
 }
 
-int32_t launch_gate_screen_prepare(const void *x, int32_t act, int64_t T, int32_t d, int32_t n, const float *Wg,
-                                   const float *Wn, void *wsplit, float *wnorm, float *xnorm,
-                                   int32_t *unsafe_count, float *wt, cudaStream_t st, int32_t groups, bool with_xnorm,
-                                   int32_t *clear) {
+static int screen_lanes(int64_t rows) { return rows >= 65536 ? 2 : rows >= 16384 ? 4 : 8; }
+
+int32_t launch_gate_screen_prepare(const void *x, int64_t T, int32_t d, int32_t n, const float *Wg, const float *Wn, void *wsplit,
+                                   float *wnorm, float *xnorm, int32_t *unsafe_count, float *wt, cudaStream_t st, int32_t groups,
+                                   bool with_xnorm, int32_t *clear) {
     // groups > 1: Wg, Wn are stacks [groups, d, n]; wsplit [3][groups * d][2n], wnorm [groups][2n], wt [groups][2n][d]
-    launch_kernel(gate_transpose_weights_kernel, dim3((unsigned)(d / 32), (unsigned)(2 * n / 32), (unsigned)groups), 256, 0, st, Wg, Wn, d, n,
-                                                                                                                      wt, unsafe_count, clear);
+    const int64_t blocks = (int64_t)groups * (2 * n / 32) + (with_xnorm ? cdiv(T, 8) : 0);
+    launch_kernel(gate_prepare_kernel, (unsigned)blocks, 256, 0, st, (const bf16 *)x, T, d, n, Wg, Wn, groups, (bf16 *)wsplit, wt, wnorm,
+                  xnorm, unsafe_count, clear);
     MOE_LAUNCHED();
-    launch_kernel(split_gate_weights_kernel, (unsigned)cdiv((int64_t)groups * d * 2 * n, 256), 256, 0, st, Wg, Wn, groups * d, n,
-                                                                                                  (bf16 *)wsplit);
-    MOE_LAUNCHED();
-    launch_kernel(gate_col_norms_kernel, dim3((unsigned)cdiv(2 * n, 8), (unsigned)groups), 256, 0, st, Wg, Wn, d, n, wnorm);
-    MOE_LAUNCHED();
-    if (with_xnorm) {
-        if (act == MOE_BF16) launch_kernel(row_norms_kernel<bf16>, (unsigned)cdiv(T, 8), 256, 0, st, (const bf16 *)x, T, d, xnorm);
-        else launch_kernel(row_norms_kernel<float>, (unsigned)cdiv(T, 8), 256, 0, st, (const float *)x, T, d, xnorm);
-        MOE_LAUNCHED();
-    }
     return MOE_OK;
 }
 
-int32_t launch_gate_screen(const float *cr, const float *noise, const float *xnorm, const float *wnorm, int32_t d,
-                           int64_t T, int32_t n, int32_t k, int32_t *idx, float *gates, float *clean, float *raw,
-                           float *kth_vals, int32_t *kth_idx, int32_t *unsafe_list, float *unsafe_low,
-                           int32_t *unsafe_count, void *chain_list, int32_t *full_list, cudaStream_t st,
-                           const int32_t *perm, int32_t kdiv, const int32_t *group_of, void *unsafe_span) {
+int32_t launch_gate_screen(const float *noise, const float *xnorm, const float *wnorm,
+                           int32_t d, int64_t T, int32_t n, int32_t k, int32_t *idx, float *gates, float *clean, float *raw,
+                           float *kth_vals, int32_t *kth_idx, int32_t *unsafe_list, float *unsafe_low, int32_t *unsafe_count,
+                           void *chain_list, int32_t *full_list, void *unsafe_span, cudaStream_t st, const int32_t *perm, int32_t kdiv,
+                           const int32_t *group_of, const HierMerge &merge) {
     // worst-case rounding of the fma chain, plus two truncations of an fp32 accumulator per MMA step of the
     // three-term tensor-core product (3d/16 steps and the additions inside a step), plus the split residual
     const double u = ldexp(1.0, -24);
@@ -698,53 +654,21 @@ int32_t launch_gate_screen(const float *cr, const float *noise, const float *xno
     const double tc = 2.0 * (3.0 * d / 16.0 + 8.0) * ldexp(1.0, -23) + ldexp(1.0, -22);
     const float theta = (float)((chain + tc) * 1.01);
     if (T == 0) return MOE_OK;
-    if (n % SCREEN_CH != 0) return MOE_ERR_INVALID_ARG;  // the screened path has 2n a multiple of 64
-    const unsigned grid = (unsigned)cdiv(T, 128);
-    const bool v16 = (((uintptr_t)noise | (uintptr_t)clean | (uintptr_t)raw | (uintptr_t)cr) & 15) == 0;
-#define MOE_SCREEN_KL(KL)                                                                                              \
-    do {                                                                                                               \
-        if (v16)                                                                                                       \
-            launch_kernel((gate_screen_rows_kernel<KL, true>), grid, 128, 0, st, cr, noise, xnorm, wnorm, theta, T, n,                   \
-                                                                    k, idx, gates, clean, raw, kth_vals, kth_idx,      \
-                                                                    unsafe_list, unsafe_low, unsafe_count, perm, kdiv, \
-                                                                    group_of);                                         \
-        else                                                                                                           \
-            launch_kernel((gate_screen_rows_kernel<KL, false>), grid, 128, 0, st, cr, noise, xnorm, wnorm, theta, T,                     \
-                                                                     n, k, idx, gates, clean, raw, kth_vals, kth_idx,  \
-                                                                     unsafe_list, unsafe_low, unsafe_count, perm,      \
-                                                                     kdiv, group_of);                                  \
-    } while (0)
+    if (n % 32 != 0) return MOE_ERR_INVALID_ARG;  // the screened path has 2n a multiple of 64
+    const bool v16 = (((uintptr_t)noise | (uintptr_t)clean | (uintptr_t)raw) & 15) == 0;
+    const int p = screen_lanes(T);
+#define MOE_SCREEN(KL, P, V16)                                                                                                 launch_kernel((gate_screen_rows_kernel<KL, P, V16>), (unsigned)cdiv(T, 4 * (32 / P)), 128, 0, st, noise, xnorm, wnorm, theta, T, n,                   k, idx, gates, clean, raw, kth_vals, kth_idx, unsafe_list, unsafe_low, unsafe_count, perm, kdiv, group_of, merge)
+#define MOE_SCREEN_P(KL, P)                        do {                                               if (v16) MOE_SCREEN(KL, P, true);              else MOE_SCREEN(KL, P, false);             } while (0)
+#define MOE_SCREEN_KL(KL)                          do {                                               if (p == 2) MOE_SCREEN_P(KL, 2);               else if (p == 4) MOE_SCREEN_P(KL, 4);          else MOE_SCREEN_P(KL, 8);                  } while (0)
     if (k <= 2) MOE_SCREEN_KL(4);
     else if (k <= 4) MOE_SCREEN_KL(6);
     else MOE_SCREEN_KL(MOE_MAX_K + 2);
 #undef MOE_SCREEN_KL
+#undef MOE_SCREEN_P
+#undef MOE_SCREEN
     MOE_LAUNCHED();
     launch_kernel(gate_candidates_kernel, 148 * 4, 256, 0, st, clean, raw, noise, xnorm, wnorm, theta, n, unsafe_list, unsafe_low,
-                                                    unsafe_count, (int2 *)chain_list, full_list, kdiv, group_of, k,
-                                                    (int2 *)unsafe_span);
-    MOE_LAUNCHED();
-    return MOE_OK;
-}
-
-// Hierarchical gate (Eq. 12): flat expert id i*b + j and product gate, slots primary-major.
-__global__ void hier_merge_kernel(int64_t total, int32_t k1, int32_t k2, int32_t b, const int32_t *idx_p,
-                                  const float *g_p, const int32_t *idx_s, const float *g_s, int32_t *topk_idx,
-                                  float *gates) {
-    wait_previous_kernel();
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // over T*k1*k2
-    if (i >= total) return;
-    const int64_t p1 = i / k2;  // t*k1 + s1
-    topk_idx[i] = idx_p[p1] * b + idx_s[i];
-    gates[i] = g_p[p1] * g_s[i];
-}
-
-int32_t launch_hier_merge(int64_t T, int32_t k1, int32_t k2, int32_t b, const int32_t *idx_p, const float *g_p,
-                          const int32_t *idx_s, const float *g_s, int32_t *topk_idx, float *gates,
-                          cudaStream_t st) {
-    const int64_t total = T * k1 * k2;
-    if (total == 0) return MOE_OK;
-    launch_kernel(hier_merge_kernel, (unsigned)cdiv(total, 256), 256, 0, st, total, k1, k2, b, idx_p, g_p, idx_s, g_s,
-                                                                    topk_idx, gates);
+                  unsafe_count, (int2 *)chain_list, full_list, kdiv, group_of, k, (int2 *)unsafe_span);
     MOE_LAUNCHED();
     return MOE_OK;
 }

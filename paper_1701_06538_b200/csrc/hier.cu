@@ -1,6 +1,7 @@
 // Two-level hierarchical mixture of experts (Appendix B, Eq. 12-14): the pieces that differ from
 // the flat layer. Rows of the secondary level are the slots p = t*k1 + s1 (token t, primary slot s1).
 #include "moe_internal.cuh"
+#include "moments.cuh"
 
 namespace moe {
 
@@ -57,21 +58,62 @@ int64_t grouped_sums_ws_floats(int64_t rows, int32_t nseg, int32_t n) { return (
 
 __device__ __forceinline__ float softplus_g(float r) { return fmaxf(r, 0.0f) + log1pf(expf(-fabsf(r))); }
 
+// first tile of group e = tiles of the groups before it: summed by the whole block (a launch of its own took longer)
+__device__ __forceinline__ int32_t tiles_before(const int32_t *offsets, int32_t e, int32_t *sh /* [8] */) {
+    int32_t s = 0;
+    for (int32_t q = threadIdx.x; q < e; q += 256) s += (offsets[q + 1] - offsets[q] + GS_ROWS - 1) / GS_ROWS;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+    __syncthreads();
+    s = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) s += sh[q];
+    return s;
+}
+
+// the group of a tile, and the group's first tile; group -1: past the last tile. By the whole block.
+__device__ __forceinline__ int2 group_of_tile(const int32_t *offsets, int32_t nseg, int32_t tile, int32_t *sh /* [8] */, int2 *found) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (threadIdx.x == 0) *found = make_int2(-1, 0);
+    int32_t carry = 0;
+    for (int32_t base = 0; base < nseg && carry <= tile; base += 256) {
+        const int32_t q = base + threadIdx.x;
+        const int32_t v = q < nseg ? (offsets[q + 1] - offsets[q] + GS_ROWS - 1) / GS_ROWS : 0;
+        int32_t inc = v;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int32_t o = __shfl_up_sync(0xffffffffu, inc, off);
+            if (lane >= off) inc += o;
+        }
+        __syncthreads();
+        if (lane == 31) sh[w] = inc;
+        __syncthreads();
+        int32_t total = 0, before = carry;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) { total += sh[u]; before += u < w ? sh[u] : 0; }
+        const int32_t excl = before + inc - v;
+        if (tile >= excl && tile < excl + v) *found = make_int2(q, excl);
+        carry += total;
+    }
+    __syncthreads();
+    return *found;
+}
+
 __global__ void __launch_bounds__(256) grouped_load_partial_kernel(
     const int32_t *__restrict__ idx_s, const float *__restrict__ clean, const float *__restrict__ raw,
-    const float *__restrict__ kth_vals, const int32_t *__restrict__ perm, const int32_t *__restrict__ offsets,
-    const int32_t *__restrict__ tile_prefix, int32_t nseg, int32_t n, int32_t k, int32_t CW, float *__restrict__ part) {
+    const float *__restrict__ kth_vals, const int32_t *__restrict__ perm, const int32_t *__restrict__ offsets, int32_t nseg, int32_t n,
+    int32_t k, int32_t CW, float *__restrict__ part, int32_t *__restrict__ ticket) {
     wait_previous_kernel();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *ticket = 0;  // of hier_load_kernel
     __shared__ float red[256];
-    const int32_t b = blockIdx.x;
-    if (b >= tile_prefix[nseg]) return;
-    int lo = 0, hi = nseg;
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (tile_prefix[mid] <= b) lo = mid; else hi = mid;
-    }
-    const int32_t r0 = offsets[lo] + (b - tile_prefix[lo]) * GS_ROWS;
-    const int32_t r1 = min(r0 + GS_ROWS, offsets[lo + 1]);
+    __shared__ int32_t sh[8];
+    __shared__ int2 found;
+    const int32_t tile = blockIdx.x;
+    const int2 at = group_of_tile(offsets, nseg, tile, sh, &found);
+    if (at.x < 0) return;
+    const int32_t r0 = offsets[at.x] + (tile - at.y) * GS_ROWS;
+    const int32_t r1 = min(r0 + GS_ROWS, offsets[at.x + 1]);
     const int cw = threadIdx.x % CW, tl = threadIdx.x / CW, TL = 256 / CW;
     for (int32_t jb = 0; jb < n; jb += CW) {
         const int32_t j = jb + cw;
@@ -90,53 +132,71 @@ __global__ void __launch_bounds__(256) grouped_load_partial_kernel(
         if (tl == 0 && j < n) {
             float a = 0.0f;
             for (int q = 0; q < TL; ++q) a += red[q * CW + cw];
-            part[(int64_t)b * n + j] = a;
+            part[(int64_t)tile * n + j] = a;
         }
         __syncthreads();
     }
 }
 
-__global__ void __launch_bounds__(256) grouped_reduce_kernel(const float *__restrict__ part,
-                                                             const int32_t *__restrict__ tile_prefix, int32_t n,
-                                                             float *__restrict__ out) {
+// Block i: the tiles of group i added up (Load_i), Load_H[i,j] = Load_primary[i] * Load_i[j] / |X^(i)| (Eq. 14; a group nobody
+// selected gets 0), and the second copies of everything that belongs to the group. The block that finishes last (counted by
+// `ticket`) forms the two losses.
+// load layout: [a*b] Load_H | [a] Load_primary | [a*b] Load_i | [a] |X^(i)|
+__global__ void __launch_bounds__(256) hier_load_kernel(const float *__restrict__ part, const int32_t *__restrict__ offsets,
+                                                        const int32_t *__restrict__ counts_p, int32_t a, int32_t b,
+                                                        const float *importance, float *load, const LossFinal fin, int32_t *ticket) {
     wait_previous_kernel();
-    const int32_t e = blockIdx.x;
-    const int32_t j = blockIdx.y * 256 + threadIdx.x;
-    if (j >= n) return;
-    double s = 0.0;
-    for (int32_t b = tile_prefix[e]; b < tile_prefix[e + 1]; ++b) s += (double)part[(int64_t)b * n + j];
-    out[(int64_t)e * n + j] = (float)s;
+    __shared__ double sh[32];
+    __shared__ int32_t shi[8];
+    __shared__ int last;
+    const int32_t i = blockIdx.x, c = counts_p[i];
+    const int64_t ab = (int64_t)a * b, at_p = ab + i, at_s = ab + a + (int64_t)i * b, at_c = 2 * ab + a + i;
+    const float load_p = load[at_p];
+    const int32_t t0 = tiles_before(offsets, i, shi), t1 = t0 + (offsets[i + 1] - offsets[i] + GS_ROWS - 1) / GS_ROWS;
+    auto put = [&](int64_t at, float v) {
+        load[at] = v;
+        if (fin.copy.load) fin.copy.load[at] = v;
+    };
+    for (int32_t j = threadIdx.x; j < b; j += 256) {
+        double s = 0.0;
+        int32_t t = t0;
+        for (; t + 8 <= t1; t += 8) {
+            float v[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) v[q] = part[(int64_t)(t + q) * b + j];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) s += (double)v[q];
+        }
+        for (; t < t1; ++t) s += (double)part[(int64_t)t * b + j];
+        const int64_t e = (int64_t)i * b + j;
+        put(at_s + j, (float)s);
+        put(e, c > 0 ? load_p * (float)s / (float)c : 0.0f);
+        if (fin.copy.importance) fin.copy.importance[e] = importance[e];
+        if (fin.copy.counts) fin.copy.counts[e] = fin.copy.counts_src[e];
+    }
+    if (threadIdx.x == 0) {
+        put(at_c, (float)c);
+        if (fin.copy.load) fin.copy.load[at_p] = load_p;
+    }
+    __threadfence();  // this block's part of Load_H, before its ticket
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(ticket, 1) == (int)gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    cv2_block(importance, (int32_t)ab, load, (int32_t)ab, fin.w_imp, fin.w_load, fin.losses, fin.copy.losses, sh);
 }
 
 int32_t launch_grouped_load(const int32_t *idx_s, const float *clean, const float *raw, const float *kth_vals,
-                            const int32_t *perm, const int32_t *offsets, int32_t nseg, int64_t rows, int32_t n,
-                            int32_t k, float *out, float *scratch, int32_t *tile_prefix, cudaStream_t st) {
-    MOE_TRY(launch_tile_prefix(offsets, nseg, GS_ROWS, tile_prefix, st));
+                            const int32_t *perm, const int32_t *offsets, const int32_t *counts_p, int32_t a, int64_t rows, int32_t b,
+                            int32_t k, const float *importance, float *load, float *scratch, const LossFinal &fin, cudaStream_t st) {
     int32_t CW = 1;
-    while (CW < n && CW < 256) CW <<= 1;
-    launch_kernel(grouped_load_partial_kernel, (unsigned)(cdiv(rows, GS_ROWS) + nseg), 256, 0, st, 
-        idx_s, clean, raw, kth_vals, perm, offsets, tile_prefix, nseg, n, k, CW, scratch);
+    while (CW < b && CW < 256) CW <<= 1;
+    int32_t *ticket = reinterpret_cast<int32_t *>(scratch + (cdiv(rows, GS_ROWS) + a) * (int64_t)b);
+    launch_kernel(grouped_load_partial_kernel, (unsigned)(cdiv(rows, GS_ROWS) + a), 256, 0, st, idx_s, clean, raw, kth_vals, perm, offsets, a,
+                  b, k, CW, scratch, ticket);
     MOE_LAUNCHED();
-    launch_kernel(grouped_reduce_kernel, dim3((unsigned)nseg, (unsigned)cdiv(n, 256)), 256, 0, st, scratch, tile_prefix, n, out);
-    MOE_LAUNCHED();
-    return MOE_OK;
-}
-
-// Load_H[i,j] = Load_primary[i] * Load_i[j] / |X^(i)|  (Eq. 14); a group nobody selected gets 0.
-// load layout: [a*b] Load_H | [a] Load_primary | [a*b] Load_i | [a] |X^(i)|
-__global__ void load_h_kernel(float *__restrict__ load, const int32_t *__restrict__ counts_p, int32_t a, int32_t b) {
-    wait_previous_kernel();
-    const int32_t i = blockIdx.x;
-    const float *load_p = load + (int64_t)a * b, *load_s = load_p + a;
-    float *cnt = load + 2 * (int64_t)a * b + a;
-    const int32_t c = counts_p[i];
-    for (int32_t j = threadIdx.x; j < b; j += blockDim.x)
-        load[(int64_t)i * b + j] = c > 0 ? load_p[i] * load_s[(int64_t)i * b + j] / (float)c : 0.0f;
-    if (threadIdx.x == 0) cnt[i] = (float)c;
-}
-
-int32_t launch_load_h(float *load, const int32_t *counts_p, int32_t a, int32_t b, cudaStream_t st) {
-    launch_kernel(load_h_kernel, a, 128, 0, st, load, counts_p, a, b);
+    launch_kernel(hier_load_kernel, (unsigned)a, 256, 0, st, scratch, offsets, counts_p, a, b, importance, load, fin, ticket);
     MOE_LAUNCHED();
     return MOE_OK;
 }

@@ -126,19 +126,8 @@ __global__ void __launch_bounds__(256) level_sums_rows_kernel(const int32_t *__r
     }
 }
 
-// the two losses (Eq. 7, 11), by one block of 256 threads; `losses` and, if given, a second copy
-__device__ __forceinline__ void cv2_block(const float *importance, int32_t n_imp, const float *load, int32_t n_load, float w_imp,
-                                          float w_load, float *losses, float *losses2, double *sh) {
-    const Moments a = block_moments(importance, n_imp, sh), b = block_moments(load, n_load, sh);
-    if (threadIdx.x == 0) {
-        const float l0 = (float)((double)w_imp * a.var / (a.mu * a.mu)), l1 = (float)((double)w_load * b.var / (b.mu * b.mu));
-        losses[0] = l0; losses[1] = l1;
-        if (losses2) { losses2[0] = l0; losses2[1] = l1; }
-    }
-}
-
 // Importance / Load = the blocks' partial sums added in double. A block takes 32 columns; its eight warps each add an
-// eighth of the chunks (in ascending order, eight loads in flight), the eight sums are then added in warp order. With
+// eighth of the chunks (in ascending order, ten loads in flight), the eight sums are then added in warp order. With
 // fin.losses set, the block that finishes last (counted by `ticket`) also forms the two losses from the complete vectors,
 // and the copies in fin.copy are written along the way.
 __global__ void __launch_bounds__(256) level_reduce_kernel(const float *__restrict__ part_imp,
@@ -154,42 +143,38 @@ __global__ void __launch_bounds__(256) level_reduce_kernel(const float *__restri
     const int32_t per = (chunks + 7) / 8, c0 = w * per, c1 = min(c0 + per, chunks);
     double a = 0.0, b = 0.0;
     if (j < n) {
-        int32_t c = c0;
-        for (; c + 8 <= c1; c += 8) {
-            float pa[8], pb[8];
+        for (int32_t c = c0; c < c1; c += 10) {
+            float pa[10], pb[10];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                pa[q] = part_imp[(int64_t)(c + q) * n + j];
-                pb[q] = part_load[(int64_t)(c + q) * n + j];
+            for (int q = 0; q < 10; ++q) {
+                pa[q] = c + q < c1 ? part_imp[(int64_t)(c + q) * n + j] : 0.0f;
+                pb[q] = c + q < c1 ? part_load[(int64_t)(c + q) * n + j] : 0.0f;
             }
 #pragma unroll
-            for (int q = 0; q < 8; ++q) { a += (double)pa[q]; b += (double)pb[q]; }
-        }
-        for (; c < c1; ++c) {
-            a += (double)part_imp[(int64_t)c * n + j];
-            b += (double)part_load[(int64_t)c * n + j];
+            for (int q = 0; q < 10; ++q) { a += (double)pa[q]; b += (double)pb[q]; }
         }
     }
     red[0][w][lane] = a;
     red[1][w][lane] = b;
     __syncthreads();
-    if (w == 0 && j < n) {
-        a = 0.0; b = 0.0;
+    if (w < 2 && j < n) {  // warp 0: Importance, warp 1: Load
+        double s = 0.0;
 #pragma unroll
-        for (int q = 0; q < 8; ++q) { a += red[0][q][lane]; b += red[1][q][lane]; }
-        if (importance) importance[j] = (float)a;
-        if (load) load[j] = (float)b;
-        if (fin.copy.importance) fin.copy.importance[j] = (float)a;
-        if (fin.copy.load) fin.copy.load[j] = (float)b;
-        if (fin.copy.counts) fin.copy.counts[j] = fin.copy.counts_src[j];
+        for (int q = 0; q < 8; ++q) s += red[w][q][lane];
+        float *out = w ? load : importance, *copy = w ? fin.copy.load : fin.copy.importance;
+        if (out) out[j] = (float)s;
+        if (copy) copy[j] = (float)s;
     }
+    if (w == 2 && j < n && fin.copy.counts) fin.copy.counts[j] = fin.copy.counts_src[j];
     if (!fin.losses) return;
     __threadfence();  // this block's sums, before its ticket
     __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(ticket, 1) == (int)gridDim.x - 1;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
+    if (gridDim.x > 1) {
+        if (threadIdx.x == 0) last = atomicAdd(ticket, 1) == (int)gridDim.x - 1;
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+    }
     cv2_block(importance, n, load, n, fin.w_imp, fin.w_load, fin.losses, fin.copy.losses, sh);
 }
 

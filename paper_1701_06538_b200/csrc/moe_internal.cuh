@@ -113,36 +113,44 @@ int32_t launch_projection(const void *x, int32_t act, int64_t M, int32_t d, int3
                           const float *W1, float *out0, float *out1, const int32_t *offsets, int32_t nseg,
                           const int32_t *perm, int32_t kdiv, int32_t *tile_prefix, cudaStream_t st,
                           const int32_t *row_count = nullptr, int32_t *clear = nullptr);
+// The hierarchical gate (Eq. 12), written where a secondary gate's row (the slot t * k1 + s1) gets its result: flat expert id i * b + j and
+// product gate, slots primary-major. idx == nullptr: not a secondary gate.
+struct HierMerge {
+    int32_t *idx;
+    float *gates;
+    const int32_t *idx_p;
+    const float *g_p;
+    int32_t b;
+    __device__ __forceinline__ void put(int64_t slot, int32_t k2, int s, int32_t j, float g) const {
+        idx[slot * k2 + s] = idx_p[slot] * b + j;
+        gates[slot * k2 + s] = g_p[slot] * g;
+    }
+};
 // Noisy logits, top-k, masked softmax for `rows` rows of n columns.
 int32_t launch_gate_select(const float *clean, const float *raw, const float *noise, int64_t rows, int32_t n,
                            int32_t k, int32_t *idx, float *gates, float *kth_vals, int32_t *kth_idx,
                            cudaStream_t st, const int32_t *row_list = nullptr, const int32_t *row_count = nullptr,
-                           const void *row_span = nullptr, const void *chain_list = nullptr);
+                           const void *row_span = nullptr, const void *chain_list = nullptr, const HierMerge &merge = HierMerge{});
 // Tensor-core screening of the routing (see gate.cu): weights split / norms, then the screening select.
-int32_t launch_gate_screen_prepare(const void *x, int32_t act, int64_t T, int32_t d, int32_t n, const float *Wg,
-                                   const float *Wn, void *wsplit, float *wnorm, float *xnorm,
-                                   int32_t *unsafe_count, float *wt /* [2n, d]: columns as rows */, cudaStream_t st,
-                                   int32_t groups = 1, bool with_xnorm = true, int32_t *clear = nullptr);
-int32_t launch_gate_screen(const float *cr, const float *noise, const float *xnorm, const float *wnorm, int32_t d,
-                           int64_t T, int32_t n, int32_t k, int32_t *idx, float *gates, float *clean, float *raw,
-                           float *kth_vals, int32_t *kth_idx, int32_t *unsafe_list, float *unsafe_low,
-                           int32_t *unsafe_count, void *chain_list, int32_t *full_list, cudaStream_t st,
-                           const int32_t *perm, int32_t kdiv, const int32_t *group_of, void *unsafe_span);
-// Rows the screen cannot certify: unsafe_list / unsafe_count[0] = rows whose selection is repeated (unsafe_low: the
-// bound that picks their candidate columns); chain_list
+int32_t launch_gate_screen_prepare(const void *x, int64_t T, int32_t d, int32_t n, const float *Wg, const float *Wn, void *wsplit,
+                                   float *wnorm, float *xnorm, int32_t *unsafe_count, float *wt /* [2n, d]: columns as rows */,
+                                   cudaStream_t st, int32_t groups = 1, bool with_xnorm = true, int32_t *clear = nullptr);
+// The screen of the products in clean / raw. Rows it cannot certify: unsafe_list / unsafe_count[0] = rows whose selection is
+// repeated (unsafe_low: the bound that picks their candidate columns; unsafe_span: where their candidates stand); chain_list
 // (int2 {row, column code}, unsafe_count[1] entries, at most 2 * SCREEN_MAX_CAND per row) = single fma chains to
 // recompute; full_list / unsafe_count[2] = rows with more candidates than that, which take the whole projection.
 constexpr int SCREEN_MAX_CAND = 16;
-int32_t launch_gate_chains(const void *x, int32_t act, int32_t d, int32_t n, const float *Wt, const void *chain_list,
-                           const int32_t *chain_count, float *clean, float *raw, cudaStream_t st,
-                           int32_t kdiv = 1);  // Wt [2n, d] (per group); token = output row / kdiv
+int32_t launch_gate_screen(const float *noise, const float *xnorm, const float *wnorm, int32_t d, int64_t T, int32_t n, int32_t k,
+                           int32_t *idx, float *gates, float *clean, float *raw, float *kth_vals, int32_t *kth_idx, int32_t *unsafe_list,
+                           float *unsafe_low, int32_t *unsafe_count, void *chain_list, int32_t *full_list, void *unsafe_span,
+                           cudaStream_t st, const int32_t *perm, int32_t kdiv, const int32_t *group_of,
+                           const HierMerge &merge = HierMerge{});
+int32_t launch_gate_chains(const void *x, int32_t d, int32_t n, const float *Wt, const void *chain_list, const int32_t *chain_count,
+                           float *clean, float *raw, cudaStream_t st, int32_t kdiv = 1);  // Wt [2n, d] (per group); token = output row / kdiv
 bool tc_gate_fwd_supported(int32_t act, int64_t T, int32_t d, int32_t n, int32_t flags);
-// cr [T, 2n] (float) = x . [W_g | W_noise] from the three-term split wsplit [3, d, 2n]
-int32_t launch_tc_gate_fwd(const void *x, int64_t T, int32_t d, int32_t n, const void *wsplit, float *cr,
+// clean | raw [T, n] (float) = x . [W_g | W_noise] from the three-term split wsplit [3, d, 2n]
+int32_t launch_tc_gate_fwd(const void *x, int64_t T, int32_t d, int32_t n, const void *wsplit, float *clean, float *raw,
                            int32_t *status, cudaStream_t st);
-int32_t launch_hier_merge(int64_t T, int32_t k1, int32_t k2, int32_t b, const int32_t *idx_p, const float *g_p,
-                          const int32_t *idx_s, const float *g_s, int32_t *topk_idx, float *gates,
-                          cudaStream_t st);
 
 // ----------------------------------------------------------------------------- routing (route.cu)
 int64_t dispatch_ws_elems(int64_t R, int32_t n);  // int32 elements of scratch
@@ -161,10 +169,26 @@ int32_t launch_combine_bwd(const void *dY, const void *ys, int32_t act, const fl
                            const int32_t *topk_idx = nullptr, const float *dimp = nullptr, int32_t n = 0);
 // (dimp [n]: the gradient of the Importance loss, added to the gate gradients of the experts in topk_idx)
 // out_f32 = sum_s dxs[inv_perm[t*k+s]] (+ add_f32 if given); written as float or, if out_act
-// is given instead, rounded to the act type.
+// is given instead, rounded to the act type. sec: float rows [T * k1, d] of the secondary gates, added to add_f32 (which is
+// given then); perm: row of a slot, or nullptr
+struct SecondaryRows { const float *rows; const int32_t *perm; int32_t k1; };
 int32_t launch_dispatch_bwd(const void *dxs, int32_t act, const int32_t *inv_perm, int64_t T, int32_t k,
                             int32_t d, const float *add_f32, float *out_f32, void *out_act, cudaStream_t st,
-                            const void *add_act = nullptr);
+                            const void *add_act = nullptr, const SecondaryRows &sec = SecondaryRows{});
+// The segment of tile `b` of a ragged product {segment, first row, segment end, tile inside the segment}, or segment -1 behind the last
+// tile, looked up by the whole block (barriers): every thread looks at its share of the segments, so that a block waits for
+// one round of loads (a binary search over the prefix waits for one per step, 2 of the 5 us of a block with little to do). sh: one int4
+__device__ __forceinline__ int4 segment_of_tile(const int32_t *__restrict__ tile_prefix, const int32_t *__restrict__ offsets, int32_t nseg,
+                                                int32_t b, int4 *sh) {
+    if (threadIdx.x == 0) *sh = make_int4(-1, 0, 0, 0);
+    __syncthreads();
+    for (int32_t q = threadIdx.x; q < nseg; q += blockDim.x) {
+        const int32_t p0 = tile_prefix[q], p1 = tile_prefix[q + 1], o0 = offsets[q], o1 = offsets[q + 1];
+        if (p0 <= b && b < p1) *sh = make_int4(q, o0, o1, b - p0);
+    }
+    __syncthreads();
+    return *sh;
+}
 // tile_prefix[e] = sum_{e' < e} ceil(count_e' / bm), e = 0..n
 int32_t launch_tile_prefix(const int32_t *offsets, int32_t n, int32_t bm, int32_t *tile_prefix, cudaStream_t st);
 
@@ -240,10 +264,11 @@ int32_t launch_hier_split_idx(const int32_t *topk_idx, int64_t T, int32_t k1, in
 int32_t launch_segment_sum(const float *vals, const int32_t *perm, const int32_t *offsets, int32_t nseg, float *out,
                            cudaStream_t st);
 int64_t grouped_sums_ws_floats(int64_t rows, int32_t nseg, int32_t n);
+// Load_i of every group, then Load_H, the two losses of the complete vectors and the copies (Eq. 14; `load` as laid out in load_h_bwd_kernel,
+// its Load_primary part is complete already)
 int32_t launch_grouped_load(const int32_t *idx_s, const float *clean, const float *raw, const float *kth_vals,
-                            const int32_t *perm, const int32_t *offsets, int32_t nseg, int64_t rows, int32_t n,
-                            int32_t k, float *out, float *scratch, int32_t *tile_prefix, cudaStream_t st);
-int32_t launch_load_h(float *load, const int32_t *counts_p, int32_t a, int32_t b, cudaStream_t st);
+                            const int32_t *perm, const int32_t *offsets, const int32_t *counts_p, int32_t a, int64_t rows, int32_t b,
+                            int32_t k, const float *importance, float *load, float *scratch, const LossFinal &fin, cudaStream_t st);
 int32_t launch_load_h_bwd(const float *load, const float *dload_h, int32_t a, int32_t b, float *dload,
                           cudaStream_t st);
 int32_t launch_hier_gate_product_bwd(const float *gates, float *dgates, int64_t T, int32_t k1, int32_t k2,
@@ -360,8 +385,8 @@ int32_t launch_tc_gate_bwd(const void *x, int64_t T, int32_t d, int32_t n, const
                            float *dX_gate, int32_t *status, cudaStream_t st, int32_t flags, int32_t ldw = 0);
 // (ldw > 0: Wg / Wn, dWg / dWn are the left and right column halves of one [d, 2n] matrix with row stride ldw)
 int32_t launch_tc_gate_fwd_grouped(const void *xs_p, int64_t P1, int32_t d, int32_t a, int32_t b, const void *wsplit_s,
-                                   const int32_t *offsets_p, int32_t *tile_prefix, float *cr_s, int32_t *status,
-                                   cudaStream_t st, int32_t flags);
+                                   const int32_t *offsets_p, int32_t *tile_prefix, const int32_t *perm_p, float *clean, float *raw,
+                                   int32_t *status, cudaStream_t st, int32_t flags);
 bool tc_hier_gate_bwd_supported(int32_t act, int32_t d, int32_t a, int32_t b);
 int32_t launch_tc_hier_secondary_bwd(const void *xs_p, const void *dsplit_s, void *wsplit_s, const float *Wg_s,
                                      const float *Wn_s, const int32_t *offsets_p, int32_t *tile_prefix, int32_t a,

@@ -137,19 +137,26 @@ __device__ __forceinline__ int32_t block_scan_1024(int32_t v, int32_t *sh /* [32
 //   RANK_ONE    the only chunk: counted here, no other kernel
 //   RANK_FEW    from the chunks' histograms: every block adds the chunks before its own and scans the totals (n <= 1024)
 //   RANK_MANY   from the scanned chunk bases and offsets
-// Then 32 warps take 32 slots each: equal experts inside a warp are ranked with match_any, the warps advance the cursors one
-// after the other. (One warp walking the 32 groups with the loads on its critical path took 16 us per chunk, this takes 4, but
-// two chunks fill an SM: see dispatch_rank_warp_kernel.)
+// Then 32 warps take 32 slots each: equal experts inside a warp are ranked with match_any. BYTES (n <= 1024): every warp leaves how many
+// slots of an expert it has in the expert's row of 32 bytes, and the slots' starts follow from the bytes of the warps before; else the
+// warps advance the cursors one after the other, 32 barriers. (One warp walking the 32 groups with the loads on its critical path
+// took 16 us per chunk, but two chunks of 32 warps fill an SM: see dispatch_rank_warp_kernel.)
 enum RankFrom { RANK_ONE, RANK_FEW, RANK_MANY };
-template <int FROM>
+constexpr int RANK_BYTES_MAX = 1024;
+template <int FROM, bool BYTES>
 __global__ void __launch_bounds__(1024) dispatch_rank_kernel(const int32_t *__restrict__ topk_idx, int64_t R, int32_t n,
                                                              const int32_t *__restrict__ chunk_table, int32_t nchunks,
                                                              int32_t *__restrict__ counts, int32_t *__restrict__ offsets,
                                                              int32_t *__restrict__ perm, int32_t *__restrict__ inv_perm) {
     wait_previous_kernel();
-    extern __shared__ int32_t cursor[];  // next sorted row of each expert for this chunk
+    extern __shared__ __align__(16) int32_t rank_sh[];
+    int32_t *cursor = rank_sh + (BYTES ? 8 * n : 0);  // next sorted row of each expert for this chunk; BYTES: behind the experts' rows of bytes
     __shared__ int32_t sh[32];
     __shared__ int32_t part_total[1024], part_before[1024];
+    uint4 *warp_counts = reinterpret_cast<uint4 *>(rank_sh);
+    if (BYTES) {
+        for (int32_t q = threadIdx.x; q < 2 * n; q += 1024) warp_counts[q] = make_uint4(0u, 0u, 0u, 0u);
+    }
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t p = (int64_t)blockIdx.x * CH + tid;
     const bool live = p < R;
@@ -192,28 +199,57 @@ __global__ void __launch_bounds__(1024) dispatch_rank_kernel(const int32_t *__re
     const unsigned peers = __match_any_sync(0xffffffffu, e);
     const int rank = __popc(peers & ((1u << lane) - 1u)), leader = __ffs(peers) - 1;
     int32_t start = 0;
-    const int busy_warps = (int)min((int64_t)32, (R - (int64_t)blockIdx.x * CH + 31) / 32);
-    for (int w = 0; w < busy_warps; ++w) {
+    if (BYTES) {
+        __syncthreads();  // the rows are cleared
+        if (e >= 0 && lane == leader) reinterpret_cast<uint8_t *>(warp_counts)[e * 32 + warp] = (uint8_t)__popc(peers);
         __syncthreads();
-        if (warp == w && e >= 0 && lane == leader) {
-            start = cursor[e];
-            cursor[e] = start + __popc(peers);
-        }
-    }
-    start = __shfl_sync(0xffffffffu, start, leader);
-    if (FROM == RANK_ONE) {  // the cursors hold the counts now: scan them, then shift the ranks by their expert's offset
-        __syncthreads();
-        int32_t carry = 0;
-        for (int32_t q0 = 0; q0 < n; q0 += 1024) {
-            const int32_t q = q0 + tid, v = q < n ? cursor[q] : 0;
+        // bytes of the first `warps` warps of an expert's row
+        auto sum_of = [&](int32_t q, int warps) {
+            const uint4 w[2] = {warp_counts[2 * q], warp_counts[2 * q + 1]};
+            const uint32_t *words = reinterpret_cast<const uint32_t *>(w);
+            uint32_t sum = 0u;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int bytes = min(4, max(0, warps - 4 * i));
+                sum = __dp4a(bytes == 4 ? words[i] : words[i] & ((1u << (8 * bytes)) - 1u), 0x01010101u, sum);
+            }
+            return (int32_t)sum;
+        };
+        if (e >= 0 && lane == leader) start = sum_of(e, warp) + (FROM == RANK_ONE ? 0 : cursor[e]);
+        start = __shfl_sync(0xffffffffu, start, leader);
+        if (FROM == RANK_ONE) {  // n <= 1024: a thread per expert
+            const int32_t v = tid < n ? sum_of(tid, 32) : 0;
             int32_t all;
-            const int32_t excl = carry + block_scan_1024(v, sh, &all);
-            if (q < n) { counts[q] = v; offsets[q] = excl; cursor[q] = excl; }
-            carry += all;
+            const int32_t excl = block_scan_1024(v, sh, &all);
+            if (tid < n) { counts[tid] = v; offsets[tid] = excl; cursor[tid] = excl; }
+            if (tid == 0) offsets[n] = all;
+            __syncthreads();
+            if (e >= 0) start += cursor[e];
         }
-        if (tid == 0) offsets[n] = carry;
-        __syncthreads();
-        if (e >= 0) start += cursor[e];
+    } else {
+        const int busy_warps = (int)min((int64_t)32, (R - (int64_t)blockIdx.x * CH + 31) / 32);
+        for (int w = 0; w < busy_warps; ++w) {
+            __syncthreads();
+            if (warp == w && e >= 0 && lane == leader) {
+                start = cursor[e];
+                cursor[e] = start + __popc(peers);
+            }
+        }
+        start = __shfl_sync(0xffffffffu, start, leader);
+        if (FROM == RANK_ONE) {  // the cursors hold the counts now: scan them, then shift the ranks by their expert's offset
+            __syncthreads();
+            int32_t carry = 0;
+            for (int32_t q0 = 0; q0 < n; q0 += 1024) {
+                const int32_t q = q0 + tid, v = q < n ? cursor[q] : 0;
+                int32_t all;
+                const int32_t excl = carry + block_scan_1024(v, sh, &all);
+                if (q < n) { counts[q] = v; offsets[q] = excl; cursor[q] = excl; }
+                carry += all;
+            }
+            if (tid == 0) offsets[n] = carry;
+            __syncthreads();
+            if (e >= 0) start += cursor[e];
+        }
     }
     if (e >= 0) {
         const int32_t r = start + rank;
@@ -284,16 +320,19 @@ int32_t launch_dispatch_index(const int32_t *topk_idx, int64_t R, int32_t n, int
     // one chunk: one launch. Up to 64 Ki histogram entries every block can afford to read them all (128 chunks x 256
     // experts: 1.5 us), which saves the two scans' launches, as long as all blocks run at once (two per SM: the entries
     // read grow with the square of the chunks).
+    const bool bytes = n <= RANK_BYTES_MAX;
+    const size_t sh_rank = bytes ? 9 * sh : sh;  // at most 36 KiB with the bytes
     if (nchunks == 1 && n <= 8192) {
-        launch_kernel(dispatch_rank_kernel<RANK_ONE>, 1, 1024, sh, st, topk_idx, R, n, nullptr, 1, counts, offsets, perm, inv_perm);
+        if (bytes) launch_kernel(dispatch_rank_kernel<RANK_ONE, true>, 1, 1024, sh_rank, st, topk_idx, R, n, nullptr, 1, counts, offsets, perm, inv_perm);
+        else launch_kernel(dispatch_rank_kernel<RANK_ONE, false>, 1, 1024, sh_rank, st, topk_idx, R, n, nullptr, 1, counts, offsets, perm, inv_perm);
         MOE_LAUNCHED();
         return MOE_OK;
     }
     launch_kernel(dispatch_hist_kernel, nchunks, 256, sh, st, topk_idx, R, n, scratch);
     MOE_LAUNCHED();
     const bool one_wave = nchunks <= 2 * 148;
-    if (one_wave && n <= 1024 && (int64_t)nchunks * n <= 65536) {
-        launch_kernel(dispatch_rank_kernel<RANK_FEW>, nchunks, 1024, sh, st, topk_idx, R, n, scratch, nchunks, counts, offsets, perm, inv_perm);
+    if (one_wave && bytes && (int64_t)nchunks * n <= 65536) {
+        launch_kernel(dispatch_rank_kernel<RANK_FEW, true>, nchunks, 1024, sh_rank, st, topk_idx, R, n, scratch, nchunks, counts, offsets, perm, inv_perm);
         MOE_LAUNCHED();
         return MOE_OK;
     }
@@ -307,7 +346,8 @@ int32_t launch_dispatch_index(const int32_t *topk_idx, int64_t R, int32_t n, int
         MOE_LAUNCHED();
         return MOE_OK;
     }
-    launch_kernel(dispatch_rank_kernel<RANK_MANY>, nchunks, 1024, sh, st, topk_idx, R, n, scratch, nchunks, counts, offsets, perm, inv_perm);
+    if (bytes) launch_kernel(dispatch_rank_kernel<RANK_MANY, true>, nchunks, 1024, sh_rank, st, topk_idx, R, n, scratch, nchunks, counts, offsets, perm, inv_perm);
+    else launch_kernel(dispatch_rank_kernel<RANK_MANY, false>, nchunks, 1024, sh_rank, st, topk_idx, R, n, scratch, nchunks, counts, offsets, perm, inv_perm);
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -735,13 +775,15 @@ int32_t launch_combine_bwd(const void *dY, const void *ys, int32_t act, const fl
 }
 
 // out[t] = sum_s dxs[inv_perm[t*k+s]] (+ add[t]) (+ add_act[t], a second addend in the act type: the gradient that
-// reaches the layer input through the residual connection); float output, or rounded to the act type
-template <typename XT, int KT, int VB>
+// reaches the layer input through the residual connection); float output, or rounded to the act type.
+// SEC: add[t] is the primary gate's part of the hierarchical layer, to which the rows of the token's sec.k1 secondary gates are added
+// (row sec.perm[t * k1 + s1], or t * k1 + s1 itself), instead of in a pass of their own over float rows as wide.
+template <typename XT, int KT, int VB, bool SEC>
 __global__ void __launch_bounds__(256) dispatch_bwd_kernel(const XT *__restrict__ dxs,
                                                            const int32_t *__restrict__ inv_perm, int64_t T,
                                                            int32_t k, int32_t d, const float *add,
                                                            float *out_f32, XT *__restrict__ out_act,
-                                                           const XT *__restrict__ add_act) {
+                                                           const XT *__restrict__ add_act, const SecondaryRows sec) {
     wait_previous_kernel();
     constexpr int VN = 16 / sizeof(XT);
     const int lane = threadIdx.x & 31;
@@ -773,6 +815,26 @@ __global__ void __launch_bounds__(256) dispatch_bwd_kernel(const XT *__restrict_
                         for (int q = 0; q < VN / 4; ++q)
                             addv[b][q] = reinterpret_cast<const float4 *>(add + t * d + (int64_t)(v0 + 32 * b) * VN)[q];
                     }
+                }
+            }
+            if (SEC) {
+                for (int s1 = 0; s1 < sec.k1; ++s1) {
+                    const int64_t slot = t * sec.k1 + s1, r = sec.perm ? (int64_t)sec.perm[slot] : slot;
+                    float4 more[VB][VN / 4];
+#pragma unroll
+                    for (int b = 0; b < VB; ++b)
+#pragma unroll
+                        for (int q = 0; q < VN / 4; ++q)
+                            if (v0 + 32 * b < nvec)
+                                more[b][q] = reinterpret_cast<const float4 *>(sec.rows + r * d + (int64_t)(v0 + 32 * b) * VN)[q];
+#pragma unroll
+                    for (int b = 0; b < VB; ++b)
+#pragma unroll
+                        for (int q = 0; q < VN / 4; ++q)
+                            if (v0 + 32 * b < nvec) {
+                                addv[b][q].x += more[b][q].x; addv[b][q].y += more[b][q].y;
+                                addv[b][q].z += more[b][q].z; addv[b][q].w += more[b][q].w;
+                            }
                 }
             }
 #pragma unroll
@@ -817,18 +879,22 @@ __global__ void __launch_bounds__(256) dispatch_bwd_kernel(const XT *__restrict_
 
 int32_t launch_dispatch_bwd(const void *dxs, int32_t act, const int32_t *inv_perm, int64_t T, int32_t k,
                             int32_t d, const float *add_f32, float *out_f32, void *out_act, cudaStream_t st,
-                            const void *add_act) {
+                            const void *add_act, const SecondaryRows &sec) {
     if (T == 0) return MOE_OK;
     const unsigned grid = (unsigned)imin(cdiv(T, 8), 148 * 16);
-#define MOE_CALL(KT, VB)                                                                                              \
+#define MOE_CALL_S(KT, VB, SEC)                                                                                       \
     if (act == MOE_BF16)                                                                                              \
-        launch_kernel((dispatch_bwd_kernel<bf16, KT, VB>), grid, 256, 0, st, (const bf16 *)dxs, inv_perm, T, k, d, add_f32, out_f32, \
-                                                                 (bf16 *)out_act, (const bf16 *)add_act);              \
+        launch_kernel((dispatch_bwd_kernel<bf16, KT, VB, SEC>), grid, 256, 0, st, (const bf16 *)dxs, inv_perm, T, k, d, add_f32, out_f32, \
+                                                                 (bf16 *)out_act, (const bf16 *)add_act, sec);         \
     else                                                                                                              \
-        launch_kernel((dispatch_bwd_kernel<float, KT, VB>), grid, 256, 0, st, (const float *)dxs, inv_perm, T, k, d, add_f32,       \
-                                                                  out_f32, (float *)out_act, (const float *)add_act)
+        launch_kernel((dispatch_bwd_kernel<float, KT, VB, SEC>), grid, 256, 0, st, (const float *)dxs, inv_perm, T, k, d, add_f32,  \
+                                                                  out_f32, (float *)out_act, (const float *)add_act, sec)
+#define MOE_CALL(KT, VB)                           \
+    if (sec.rows) { MOE_CALL_S(KT, VB, true); }    \
+    else { MOE_CALL_S(KT, VB, false); }
     MOE_DISPATCH_KT(k, MOE_CALL);
 #undef MOE_CALL
+#undef MOE_CALL_S
     MOE_LAUNCHED();
     return MOE_OK;
 }
