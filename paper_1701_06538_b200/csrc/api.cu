@@ -1,7 +1,7 @@
 // The C ABI (include/moe.h): argument checks, workspace carving and the order of the launches.
 #include <string.h>
 
-#include "moe_internal.cuh"
+#include "plan.cuh"
 
 #include <atomic>
 
@@ -238,18 +238,19 @@ struct LossesWs {
 
 struct FfnBwdWs {
     void *dz;
-    float *colsum;
+    float *colsum, *colsum2;  // of db1, of db2
     uint32_t *bits;  // MOE_FLAG_RECOMPUTE_HID on the tensor cores: the mask bits that the recomputation writes
     FfnBwdWs(Carver &cv, const Dims &D) {
         dz = cv.take_bytes(D.R * D.h * (int64_t)D.esz);
         const bool tc = D.act == MOE_BF16 && D.d % 64 == 0 && D.h % 64 == 0;
         bits = tc && (D.flags & MOE_FLAG_RECOMPUTE_HID) ? cv.take<uint32_t>(D.R * (D.h / 32)) : nullptr;
-        int64_t cs = colsum_ws_floats(D.R, (int32_t)D.n, (int32_t)(D.h > D.d ? D.h : D.d));
+        int64_t cs = colsum_ws_floats(D.R, (int32_t)D.n, (int32_t)D.h);
         if (D.act == MOE_BF16) {  // the tensor-core path sums dz's columns per 32-row block in the GEMM epilogue
             const int64_t cs_tc = tc_colsum_part_floats(D.R, (int32_t)D.n, (int32_t)D.h);
             if (cs_tc > cs) cs = cs_tc;
         }
         colsum = cv.take<float>(cs);
+        colsum2 = cv.take<float>(colsum_ws_floats(D.R, (int32_t)D.n, (int32_t)D.d));
     }
 };
 
@@ -424,11 +425,15 @@ int32_t do_gate(const moe_config *c, const Dims &D, const void *x, const float *
     return MOE_OK;
 }
 
+// plan, sums: what a fused call has done along with the dispatch, where it can be (the plan is made in any case)
 int32_t do_dispatch(const Dims &D, const void *x, const int32_t *topk_idx, void *xs, int32_t *perm,
-                    int32_t *inv_perm, int32_t *counts, int32_t *offsets, Carver &cv, cudaStream_t st) {
+                    int32_t *inv_perm, int32_t *counts, int32_t *offsets, Carver &cv, cudaStream_t st, const PlanArgs *plan = nullptr,
+                    const LevelSums *sums = nullptr) {
     DispatchWs w(cv, D);
-    MOE_TRY(launch_dispatch_index(topk_idx, D.R, (int32_t)D.n, perm, inv_perm, counts, offsets, w.scratch, st));
-    return launch_dispatch_rows(x, D.act, D.T, (int32_t)D.k, (int32_t)D.d, inv_perm, xs, st);
+    bool planned = false;
+    MOE_TRY(launch_dispatch_index(topk_idx, D.R, (int32_t)D.n, perm, inv_perm, counts, offsets, w.scratch, st, plan, &planned));
+    if (plan && !planned) MOE_TRY(launch_segment_plan(*plan, offsets, st));
+    return launch_dispatch_rows(x, D.act, D.T, (int32_t)D.k, (int32_t)D.d, inv_perm, xs, st, sums);
 }
 
 SimtGemm base_gemm(const Dims &D) {
@@ -456,7 +461,9 @@ int32_t do_expert_ffn(const moe_config *c, const Dims &D, const void *xs, const 
         SegmentMaps maps;
         const bool tc = tc_ffn_supported(*c);
         if (tc) MOE_TRY(tc_segment_maps(*c, &maps, xs, hid, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr));
-        MOE_TRY(launch_segment_plan(plan, offsets, (int32_t)D.n, D.R, clear, st, tc ? &maps : nullptr));
+        PlanArgs args;
+        fill_plan(&args, plan, (int32_t)D.n, D.R, clear, tc ? &maps : nullptr);
+        MOE_TRY(launch_segment_plan(args, offsets, st));
     }
     if (tc_ffn_supported(*c))
         return launch_tc_ffn(*c, xs, offsets, W1, b1, W2, b2, hid, ys, plan, status_word(ws_base), st, first_only, relu_bits);
@@ -473,16 +480,26 @@ int32_t do_expert_ffn(const moe_config *c, const Dims &D, const void *xs, const 
     return launch_simt_gemm(g, nullptr, st, nullptr, &plan);
 }
 
+// The batch sums over the columns of the flat gate, with the two losses, or of the primary gate (idx: its groups): Load_primary
+LevelSums first_level_sums(const moe_config *c, const Dims &D, const int32_t *idx, const float *gates, const float *clean,
+                           const float *raw_noise, const float *kth_vals, float *importance, float *load, float *losses, const LossOut &copy,
+                           float *scratch) {
+    if (D.hier)
+        return level_sums(idx, gates + D.T * D.k, clean, raw_noise, kth_vals, D.T, (int32_t)D.a, (int32_t)D.k1, nullptr, load + D.a * D.b, scratch);
+    const LossFinal fin = {c->w_importance, c->w_load, losses, copy};
+    return level_sums(idx, gates, clean, raw_noise, kth_vals, D.T, (int32_t)D.n, (int32_t)D.k, importance, load, scratch, &fin);
+}
+
 int32_t do_losses(const moe_config *c, const Dims &D, const int32_t *topk_idx, const float *gates,
                   const float *clean, const float *raw_noise, const float *kth_vals, float *importance, float *load,
                   float *losses, const int32_t *perm, const int32_t *offsets, Carver &cv, cudaStream_t st,
-                  const LossOut &copy = LossOut{}, const HierIdx *ready = nullptr) {
+                  const LossOut &copy = LossOut{}, const HierIdx *ready = nullptr, bool sums_done = false) {
+    // sums_done: the sums over the (first) gate's columns have been formed along with other launches (first_level_sums)
     LossesWs w(cv, D);
-    if (!D.hier) {
-        const LossFinal fin = {c->w_importance, c->w_load, losses, copy};
-        return launch_level_sums(topk_idx, gates, clean, raw_noise, kth_vals, D.T, (int32_t)D.n, (int32_t)D.k, importance, load,
-                                 w.scratch, st, &fin);
-    }
+    if (!D.hier)
+        return sums_done ? MOE_OK
+                         : launch_level_sums(first_level_sums(c, D, topk_idx, gates, clean, raw_noise, kth_vals, importance, load, losses, copy,
+                                                              w.scratch), st);
     // Eq. 13: Importance_H = batch sum of the product gates per expert (ordered sum over each expert's rows)
     if (!perm) {
         MOE_TRY(launch_dispatch_index(topk_idx, D.R, (int32_t)D.n, w.perm_e, w.inv_perm_e, w.counts_e, w.offsets_e,
@@ -493,25 +510,45 @@ int32_t do_losses(const moe_config *c, const Dims &D, const int32_t *topk_idx, c
     MOE_TRY(launch_segment_sum(gates, perm, offsets, (int32_t)D.n, importance, st));
     // Eq. 14: Load_primary, the per-group Load_i over X^(i), |X^(i)|
     MOE_TRY(w.H.build(D, topk_idx, ready, st));
-    const int64_t ab = D.a * D.b, lp = D.T * D.a;
-    float *load_p = load + ab;
-    MOE_TRY(launch_level_sums(w.H.idx_p, gates + D.T * D.k, clean, raw_noise, kth_vals, D.T, (int32_t)D.a,
-                              (int32_t)D.k1, nullptr, load_p, w.scratch, st));
+    const int64_t lp = D.T * D.a;
+    if (!sums_done)
+        MOE_TRY(launch_level_sums(first_level_sums(c, D, w.H.idx_p, gates, clean, raw_noise, kth_vals, nullptr, load, nullptr, LossOut{},
+                                                   w.scratch), st));
     return launch_grouped_load(w.H.idx_s, clean + lp, raw_noise + lp, kth_vals + 2 * D.T, w.H.perm_p, w.H.offsets_p, w.H.counts_p,
                                (int32_t)D.a, D.T * D.k1, (int32_t)D.b, (int32_t)D.k2, importance, load, w.grouped,
                                LossFinal{c->w_importance, c->w_load, losses, copy}, st);
 }
 
+ColumnSums db2_sums(const Dims &D, const void *dys, void *db2, const int32_t *offsets, const FfnBwdWs &w, const SegmentPlan &plan) {
+    return {dys, db2, D.act, (int32_t)D.n, (int32_t)D.d, D.R, offsets, plan.prefix_of(COLSUM_ROWS), w.colsum2};
+}
+// tail: the last passes over the bias gradients' sums may be left to the caller; db2_begun: the tile sums of db2 have been formed already
 int32_t do_expert_ffn_bwd(const moe_config *c, const Dims &D, const void *xs, const void *hid, const void *dys,
                           const int32_t *offsets, const void *W1, const void *W2, void *dxs, void *dW1, void *db1,
                           void *dW2, void *db2, void *ws_base, Carver &cv, cudaStream_t st, const SegmentPlan &plan,
-                          const uint32_t *relu_bits = nullptr) {
+                          const uint32_t *relu_bits = nullptr, BackwardTail *tail = nullptr, bool db2_begun = false) {
     FfnBwdWs w(cv, D);
     const int32_t n = (int32_t)D.n;
-    if (tc_ffn_supported(*c))
-        return launch_tc_ffn_bwd(*c, xs, hid, dys, offsets, W1, W2, dxs, dW1, db1, dW2, db2, w.dz, w.colsum, plan,
-                                 status_word(ws_base), st, relu_bits);
-    MOE_TRY(launch_segment_colsum(dys, D.act, offsets, n, D.R, (int32_t)D.d, db2, w.colsum, plan.prefix_of(COLSUM_ROWS), st));
+    BackwardTail *leave = n < COLSUM_MANY ? tail : nullptr;
+    auto finish = [&](const ColumnSums &sums, int which) -> int32_t {
+        if (!leave) return launch_segment_colsum_final(sums, st);
+        leave->columns[which] = sums;
+        leave->column_blocks[which] = (int32_t)(n * cdiv(sums.N, 32));
+        return MOE_OK;
+    };
+    const ColumnSums db2s = db2_sums(D, dys, db2, offsets, w, plan);
+    if (!db2_begun) MOE_TRY(launch_segment_colsum(db2s, false, st));
+    MOE_TRY(finish(db2s, 0));
+    if (tc_ffn_supported(*c)) {
+        BlockSums left = {};
+        MOE_TRY(launch_tc_ffn_bwd(*c, xs, hid, dys, offsets, W1, W2, dxs, dW1, db1, dW2, w.dz, w.colsum, plan,
+                                  status_word(ws_base), st, relu_bits, leave ? &left : nullptr));
+        if (left.part) {
+            leave->blocks = left;
+            leave->block_blocks = (int32_t)(n * cdiv(left.N, 64));
+        }
+        return MOE_OK;
+    }
     SimtGemm g = base_gemm(D);  // dW2[e] = hid_e^T . dys_e
     g.A = hid; g.B = dys; g.C = dW2;
     g.sa_i = 1; g.sa_k = D.h; g.sb_k = D.d; g.sb_j = 1; g.sc_i = D.d;
@@ -522,7 +559,9 @@ int32_t do_expert_ffn_bwd(const moe_config *c, const Dims &D, const void *xs, co
     g.sa_i = D.d; g.sa_k = 1; g.sb_k = 1; g.sb_j = D.d; g.sc_i = D.h;
     g.mode = 0; g.offsets = offsets; g.nseg = n; g.M = D.R; g.N = D.h; g.K = D.d; g.b_e = D.h * D.d;
     MOE_TRY(launch_simt_gemm(g, nullptr, st, nullptr, &plan));
-    MOE_TRY(launch_segment_colsum(w.dz, D.act, offsets, n, D.R, (int32_t)D.h, db1, w.colsum, plan.prefix_of(COLSUM_ROWS), st));
+    const ColumnSums db1s = {w.dz, db1, D.act, n, (int32_t)D.h, D.R, offsets, plan.prefix_of(COLSUM_ROWS), w.colsum};
+    MOE_TRY(launch_segment_colsum(db1s, false, st));
+    MOE_TRY(finish(db1s, 1));
     g = base_gemm(D);  // dW1[e] = xs_e^T . dz_e
     g.A = xs; g.B = w.dz; g.C = dW1;
     g.sa_i = 1; g.sa_k = D.d; g.sb_k = D.h; g.sb_j = 1; g.sc_i = D.h;
@@ -546,7 +585,9 @@ int32_t expert_ffn_bwd_stage(const moe_config *c, const Dims &D, const void *xs,
         const FfnBwdWs w(ahead, D);
         MOE_TRY(tc_segment_maps(*c, &maps, nullptr, nullptr, dys, w.dz, hid, dys, xs, w.dz));
     }
-    MOE_TRY(launch_segment_plan(plan, offsets, (int32_t)D.n, D.R, status_word(ws), st, tc ? &maps : nullptr));
+    PlanArgs args;
+    fill_plan(&args, plan, (int32_t)D.n, D.R, status_word(ws), tc ? &maps : nullptr);
+    MOE_TRY(launch_segment_plan(args, offsets, st));
     return do_expert_ffn_bwd(c, D, xs, hid, dys, offsets, W1, W2, dxs, dW1, db1, dW2, db2, ws, cv, st, plan, relu_bits);
 }
 
@@ -563,7 +604,7 @@ int32_t do_losses_bwd(const moe_config *c, const Dims &D, const float *importanc
 // dW = x^T . dlogit [d, n], dX = dlogit . W^T [T, d], with dlogit [T, cols] (cols = n, or 2n columns of [W_g | W_noise], whose
 // two halves then are W / W2 and dW / dW2)
 int32_t gate_weight_grads(const Dims &D, const void *x, const float *dlogit, const float *W, const float *W2, int64_t n,
-                          float *dW, float *dW2, float *dX, float *part, cudaStream_t st) {
+                          float *dW, float *dW2, float *dX, float *part, cudaStream_t st, GateParts *parts_left = nullptr) {
     const int64_t cols = W2 ? 2 * n : n;
     SimtGemm g;
     memset(&g, 0, sizeof(g));
@@ -572,7 +613,7 @@ int32_t gate_weight_grads(const Dims &D, const void *x, const float *dlogit, con
     g.A = x; g.B = dlogit; g.C = dW; g.C2 = dW2; g.c_split = n;
     g.sa_i = 1; g.sa_k = D.d; g.sb_k = cols; g.sb_j = 1; g.sc_i = n;
     g.mode = 1; g.offsets = nullptr; g.nseg = 1; g.M = D.d; g.N = cols; g.K = D.T;
-    MOE_TRY(launch_simt_gemm(g, nullptr, st, part));
+    MOE_TRY(launch_simt_gemm(g, nullptr, st, part, nullptr, parts_left));
     memset(&g, 0, sizeof(g));
     g.a_row_div = 1;
     g.ta = g.tb = g.tc = G_F32;
@@ -587,8 +628,17 @@ int32_t do_gate_bwd(const moe_config *c, const Dims &D, const void *x, const flo
                     const float *noise, const float *clean, const float *raw_noise, const int32_t *topk_idx,
                     const float *gates, const float *kth_vals, const int32_t *kth_idx, float *dgates,
                     const float *dload, float *dWg, float *dWnoise, float *dX_gate, void *ws_base, Carver &cv,
-                    cudaStream_t st, const HierIdx *ready = nullptr, SecondaryRows *sec = nullptr) {
-    // sec: the caller adds the secondary gates' rows to dX_gate itself (they stay in the scratch)
+                    cudaStream_t st, const HierIdx *ready = nullptr, SecondaryRows *sec = nullptr, const ColumnSums *beside = nullptr,
+                    BackwardTail *tail = nullptr) {
+    // sec: the caller adds the secondary gates' rows to dX_gate itself (they stay in the scratch); beside: tile sums to be formed along
+    // with the logit gradients; tail: the last pass over the (first) gate's weight gradient may be left to the caller
+    GateParts left = {};
+    GateParts *parts = tail ? &left : nullptr;
+    auto leave_parts = [&]() {
+        if (!left.part) return;
+        tail->parts = left;
+        tail->parts_blocks = (int32_t)cdiv((int64_t)left.d * left.cols, 256);
+    };
     GateBwdWs w(cv, D);
     if (D.hier) {
         const int64_t P1 = D.T * D.k1, lp = D.T * D.a, wp = D.d * D.a;
@@ -600,9 +650,10 @@ int32_t do_gate_bwd(const moe_config *c, const Dims &D, const void *x, const flo
             // both levels on the tensor cores: split logit gradients (the secondary ones written in the
             // order sorted by primary group), grouped products, then the slots' rows are added per token
             MOE_TRY(launch_gate_logit_grads(noise, clean, raw_noise, w.H.idx_p, g_p, kth_vals, kth_idx, dg_p, dload,
-                                            nullptr, D.T, (int32_t)D.a, (int32_t)D.k1, nullptr, w.dsplit, nullptr, st));
+                                            nullptr, D.T, (int32_t)D.a, (int32_t)D.k1, nullptr, w.dsplit, nullptr, st, beside));
             MOE_TRY(launch_tc_gate_bwd(x, D.T, (int32_t)D.d, (int32_t)D.a, Wg, Wnoise, w.dsplit, w.wsplit, w.partials,
-                                       dWg, dWnoise, dX_gate, status_word(ws_base), st, D.flags));
+                                       dWg, dWnoise, dX_gate, status_word(ws_base), st, D.flags, 0, parts));
+            leave_parts();
             MOE_TRY(launch_gate_logit_grads(noise + lp, clean + lp, raw_noise + lp, w.H.idx_s, g_s, kth_vals + 2 * D.T,
                                             kth_idx + 2 * D.T, dg_s, dload + D.a, w.H.idx_p, P1, (int32_t)D.b,
                                             (int32_t)D.k2, nullptr, w.dsplit_s, w.H.inv_perm_p, st));
@@ -620,8 +671,9 @@ int32_t do_gate_bwd(const moe_config *c, const Dims &D, const void *x, const flo
         }
         // primary gate (Eq. 12: G_primary), rows = tokens
         MOE_TRY(launch_gate_logit_grads(noise, clean, raw_noise, w.H.idx_p, g_p, kth_vals, kth_idx, dg_p, dload,
-                                        nullptr, D.T, (int32_t)D.a, (int32_t)D.k1, w.dlogit, nullptr, nullptr, st));
-        MOE_TRY(gate_weight_grads(D, x, w.dlogit, Wg, Wnoise, D.a, dWg, dWnoise, dX_gate, w.partials, st));
+                                        nullptr, D.T, (int32_t)D.a, (int32_t)D.k1, w.dlogit, nullptr, nullptr, st, beside));
+        MOE_TRY(gate_weight_grads(D, x, w.dlogit, Wg, Wnoise, D.a, dWg, dWnoise, dX_gate, w.partials, st, parts));
+        leave_parts();
         // secondary gates G_i, rows = slots (t, s1); dLoad_i of the row's group
         MOE_TRY(launch_gate_logit_grads(noise + lp, clean + lp, raw_noise + lp, w.H.idx_s, g_s, kth_vals + 2 * D.T,
                                         kth_idx + 2 * D.T, dg_s, dload + D.a, w.H.idx_p, P1, (int32_t)D.b,
@@ -649,11 +701,14 @@ int32_t do_gate_bwd(const moe_config *c, const Dims &D, const void *x, const flo
         return launch_add_slot_rows(w.dX_sec, D.T, (int32_t)D.k1, (int32_t)D.d, dX_gate, st);
     }
     MOE_TRY(launch_gate_logit_grads(noise, clean, raw_noise, topk_idx, gates, kth_vals, kth_idx, dgates, dload,
-                                    nullptr, D.T, (int32_t)D.n, (int32_t)D.k, w.dlogit, w.dsplit, nullptr, st));
+                                    nullptr, D.T, (int32_t)D.n, (int32_t)D.k, w.dlogit, w.dsplit, nullptr, st, beside));
     if (w.tc)
-        return launch_tc_gate_bwd(x, D.T, (int32_t)D.d, (int32_t)D.n, Wg, Wnoise, w.dsplit, w.wsplit, w.partials, dWg,
-                                  dWnoise, dX_gate, status_word(ws_base), st, D.flags);
-    return gate_weight_grads(D, x, w.dlogit, Wg, Wnoise, D.n, dWg, dWnoise, dX_gate, w.partials, st);
+        MOE_TRY(launch_tc_gate_bwd(x, D.T, (int32_t)D.d, (int32_t)D.n, Wg, Wnoise, w.dsplit, w.wsplit, w.partials, dWg,
+                                   dWnoise, dX_gate, status_word(ws_base), st, D.flags, 0, parts));
+    else
+        MOE_TRY(gate_weight_grads(D, x, w.dlogit, Wg, Wnoise, D.n, dWg, dWnoise, dX_gate, w.partials, st, parts));
+    leave_parts();
+    return MOE_OK;
 }
 
 }  // namespace
@@ -695,6 +750,7 @@ int32_t moe_query_sizes(const moe_config *cfg, moe_sizes *out) {
     const int64_t s_disp = measure([&](Carver &cv) { DispatchWs w(cv, D); (void)w; });
     const int64_t s_ffn = measure([&](Carver &cv) { FfnWs w(cv, D); (void)w; });
     const int64_t s_loss = measure([&](Carver &cv) { LossesWs w(cv, D); (void)w; });
+    const int64_t s_fused = measure([&](Carver &cv) { FfnWs f(cv, D); DispatchWs w(cv, D); LossesWs l(cv, D); (void)f; (void)w; (void)l; });
     const int64_t s_fbwd = measure([&](Carver &cv) { cv.take<int32_t>(plan_ints(D.R, D.n)); FfnBwdWs w(cv, D); (void)w; });
     const int64_t s_lbwd = measure([&](Carver &cv) { LossesBwdWs w(cv, D); (void)w; });
     const int64_t s_gbwd = measure([&](Carver &cv) { GateBwdWs w(cv, D); (void)w; });
@@ -702,16 +758,16 @@ int32_t moe_query_sizes(const moe_config *cfg, moe_sizes *out) {
     if (s_disp > fwd) fwd = s_disp;
     if (s_ffn > fwd) fwd = s_ffn;
     if (s_loss > fwd) fwd = s_loss;
+    const int64_t fused_fwd = s_fused > fwd ? s_fused : fwd;
     int64_t stage_bwd = s_fbwd;
     if (s_lbwd > stage_bwd) stage_bwd = s_lbwd;
     if (s_gbwd > stage_bwd) stage_bwd = s_gbwd;
-    const int64_t s_fbwd_recompute = measure([&](Carver &cv) { FfnBwdWs w(cv, D); FfnWs f(cv, D); (void)w; (void)f; });
-    if ((D.flags & MOE_FLAG_RECOMPUTE_HID) && s_fbwd_recompute > stage_bwd) stage_bwd = s_fbwd_recompute;
+    const int64_t s_fused_bwd = measure([&](Carver &cv) { BwdWs b(cv, D); FfnBwdWs w(cv, D); FfnWs f(cv, D); GateBwdWs g(cv, D); (void)b; (void)w; (void)f; (void)g; });
     out->adam_state_elems = D.n * (3 * D.d + 3 * D.h);
     out->ws_adam_bytes = kWsHeader + ((adam_ws_floats((int32_t)D.n, (int32_t)D.d, (int32_t)D.h) * 4 + 255) & ~(int64_t)255);
     out->ws_bytes = fwd > stage_bwd ? fwd : stage_bwd;
-    out->ws_fwd_bytes = fwd;
-    out->ws_bwd_bytes = measure([&](Carver &cv) { BwdWs w(cv, D); (void)w; }) + stage_bwd;
+    out->ws_fwd_bytes = fused_fwd;
+    out->ws_bwd_bytes = s_fused_bwd;
     Ctx ctx(nullptr, D, tc_ffn_supported(*cfg));
     out->ctx_bytes = ctx.bytes;
     return MOE_OK;
@@ -910,17 +966,36 @@ static int32_t forward_impl(const moe_config *cfg, const void *x, const float *W
     { Carver cv = fresh();
       MOE_TRY(do_gate(cfg, D, x, Wg, Wnoise, noise, C.topk_idx, C.gates, C.clean, C.raw_noise, C.kth_vals,
                       C.kth_idx, ws, cv, st, &C.hier)); }
-    { Carver cv = fresh();
-      MOE_TRY(do_dispatch(D, x, C.topk_idx, C.xs, C.perm, C.inv_perm, C.counts, C.offsets, cv, st)); }
-    { Carver cv = fresh();
-      MOE_TRY(do_expert_ffn(cfg, D, C.xs, C.offsets, W1, b1, W2, b2, C.hid, C.ys, ws, cv, st, nullptr, false, nullptr,
-                            C.relu_bits)); }  // C.hid null: stays in ws
+    // Behind the gate the workspace holds, one after the other, what the expert products need throughout, the dispatch's scratch and
+    // the losses': the segment plan is made along with the dispatch's index, the losses' sums with its rows, and they are
+    // completed with the combine.
+    Carver cv = fresh();
+    const FfnWs ffn(cv, D);
+    const SegmentPlan plan = make_plan(cfg, D, ffn.plan, false);
+    SegmentMaps maps;
+    const bool tc = tc_ffn_supported(*cfg);
+    if (tc)
+        MOE_TRY(tc_segment_maps(*cfg, &maps, C.xs, C.hid ? C.hid : ffn.hid, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr));
+    PlanArgs args;
+    fill_plan(&args, plan, (int32_t)D.n, D.R, nullptr, tc ? &maps : nullptr);
+    Carver dispatch_at = cv;
+    const DispatchWs dispatch(cv, D);
+    const Carver losses_at = cv;
+    const LossesWs losses_ws(cv, D);
+    const LossOut copy{losses, importance, load, counts, C.counts, (int32_t)D.n, (int32_t)D.load};
+    const LevelSums sums = first_level_sums(cfg, D, D.hier ? C.hier.idx_p : C.topk_idx, C.gates, C.clean, C.raw_noise, C.kth_vals,
+                                            D.hier ? nullptr : C.importance, C.load, D.hier ? nullptr : C.losses, D.hier ? LossOut{} : copy,
+                                            losses_ws.scratch);
+    const bool ride = D.T > 0 && sums.n <= LEVEL_RIDE_MAX;
+    MOE_TRY(do_dispatch(D, x, C.topk_idx, C.xs, C.perm, C.inv_perm, C.counts, C.offsets, dispatch_at, st, &args, ride ? &sums : nullptr));
+    { Carver at = fresh();
+      MOE_TRY(do_expert_ffn(cfg, D, C.xs, C.offsets, W1, b1, W2, b2, C.hid, C.ys, ws, at, st, nullptr, false, nullptr,
+                            C.relu_bits, &plan)); }  // C.hid null: stays in ws
     MOE_TRY(launch_combine(C.ys, D.act, C.gates, C.inv_perm, D.T, (int32_t)D.k, (int32_t)D.d, y, st,
-                           keep_bits ? x : nullptr, keep_bits, keep_bits ? 1.0f / (1.0f - drop_prob) : 1.0f));
-    { Carver cv = fresh();
+                           keep_bits ? x : nullptr, keep_bits, keep_bits ? 1.0f / (1.0f - drop_prob) : 1.0f, ride ? &sums : nullptr));
+    { Carver at = losses_at;
       MOE_TRY(do_losses(cfg, D, C.topk_idx, C.gates, C.clean, C.raw_noise, C.kth_vals, C.importance, C.load,
-                        C.losses, C.perm, C.offsets, cv, st,
-                        LossOut{losses, importance, load, counts, C.counts, (int32_t)D.n, (int32_t)D.load}, &C.hier)); }
+                        C.losses, C.perm, C.offsets, at, st, copy, &C.hier, ride)); }
     return MOE_OK;
 }
 
@@ -960,41 +1035,46 @@ static int32_t backward_impl(const moe_config *cfg, const void *dY, const void *
     const SegmentPlan plan = make_plan(cfg, D, B.plan, true);
     const Cv2Job jobs[2] = {{C.importance, (int32_t)D.n, cfg->w_importance, B.dimp},
                             {C.load, (int32_t)D.n, cfg->w_load, D.hier ? B.dload_h : B.dload}};
+    // Scratch: the expert backward's, hidden activations that are computed again, the gate's (all of it lives until the last launch)
+    Carver cv = fresh();
+    const FfnBwdWs ffn(cv, D);
+    const FfnWs again(cv, D);
     SegmentMaps maps;
     const bool tc = tc_ffn_supported(*cfg);
-    if (tc) {
-        Carver ahead = fresh();  // where the expert backward will have dz and hidden activations that are computed again
-        const FfnBwdWs w(ahead, D);
-        const FfnWs f(ahead, D);
-        const void *hid = C.hid ? C.hid : f.hid;
-        MOE_TRY(tc_segment_maps(*cfg, &maps, C.hid ? nullptr : C.xs, nullptr, B.dys, w.dz, hid, B.dys, C.xs, w.dz));
-    }
-    MOE_TRY(launch_segment_plan(plan, C.offsets, (int32_t)D.n, D.R, status_word(ws), st, tc ? &maps : nullptr, jobs));
+    if (tc)
+        MOE_TRY(tc_segment_maps(*cfg, &maps, C.hid ? nullptr : C.xs, nullptr, B.dys, ffn.dz, C.hid ? C.hid : again.hid, B.dys, C.xs, ffn.dz));
+    PlanArgs args;
+    fill_plan(&args, plan, (int32_t)D.n, D.R, status_word(ws), tc ? &maps : nullptr, jobs);
+    MOE_TRY(launch_segment_plan(args, C.offsets, st));
     if (D.hier) MOE_TRY(launch_load_h_bwd(C.load, B.dload_h, (int32_t)D.a, (int32_t)D.b, B.dload, st));
     MOE_TRY(launch_combine_bwd(dY, C.ys, D.act, C.gates, C.inv_perm, D.T, (int32_t)D.k, (int32_t)D.d, B.dgates,
                                B.dys, st, keep_bits, keep_bits ? 1.0f / (1.0f - drop_prob) : 1.0f, C.topk_idx, B.dimp,
                                (int32_t)D.n));
-    { Carver cv = fresh();
-      const void *hid = C.hid;
-      uint32_t *bits = C.relu_bits;
-      if (!hid) {  // MOE_FLAG_RECOMPUTE_HID: the forward kept no hidden activations; the first GEMM is run again
-          FfnBwdWs own(cv, D);  // the expert backward's own scratch comes first, the recomputed tensor behind it
-          void *again = nullptr;
-          bits = own.bits;
-          MOE_TRY(do_expert_ffn(cfg, D, C.xs, C.offsets, W1, b1, W2, b2, nullptr, nullptr, ws, cv, st, nullptr, true, &again, bits,
-                                &plan));
-          hid = again;
-          cv = fresh();
-      }
-      MOE_TRY(do_expert_ffn_bwd(cfg, D, C.xs, hid, B.dys, C.offsets, W1, W2, B.dxs, dW1, db1, dW2, db2, ws, cv,
-                                st, plan, bits)); }
+    // The gate's backward first: the tile sums of db2 go along with its logit gradients. What the bias and gate gradients have left to
+    // add goes along with the last launch.
+    BackwardTail tail = {};
+    BackwardTail *left = D.T > 0 ? &tail : nullptr;
     SecondaryRows sec = {};
-    { Carver cv = fresh();
-      MOE_TRY(do_gate_bwd(cfg, D, x, Wg, Wnoise, noise, C.clean, C.raw_noise, C.topk_idx, C.gates, C.kth_vals,
-                          C.kth_idx, B.dgates, B.dload, dWg, dWnoise, B.dX_gate, ws, cv, st, &C.hier, &sec)); }
+    const ColumnSums db2s = db2_sums(D, B.dys, db2, C.offsets, ffn, plan);
+    MOE_TRY(do_gate_bwd(cfg, D, x, Wg, Wnoise, noise, C.clean, C.raw_noise, C.topk_idx, C.gates, C.kth_vals,
+                        C.kth_idx, B.dgates, B.dload, dWg, dWnoise, B.dX_gate, ws, cv, st, &C.hier, &sec, left ? &db2s : nullptr, left));
+    const void *hid = C.hid;
+    uint32_t *bits = C.relu_bits;
+    if (!hid) {  // MOE_FLAG_RECOMPUTE_HID: the forward kept no hidden activations; the first GEMM is run again
+        Carver at = fresh();
+        FfnBwdWs own(at, D);
+        void *made = nullptr;
+        bits = own.bits;
+        MOE_TRY(do_expert_ffn(cfg, D, C.xs, C.offsets, W1, b1, W2, b2, nullptr, nullptr, ws, at, st, nullptr, true, &made, bits,
+                              &plan));
+        hid = made;
+    }
+    { Carver at = fresh();
+      MOE_TRY(do_expert_ffn_bwd(cfg, D, C.xs, hid, B.dys, C.offsets, W1, W2, B.dxs, dW1, db1, dW2, db2, ws, at,
+                                st, plan, bits, left, left != nullptr)); }
     // dX = expert path + gating path (+ the upstream gradient itself through the residual connection)
     return launch_dispatch_bwd(B.dxs, D.act, C.inv_perm, D.T, (int32_t)D.k, (int32_t)D.d, B.dX_gate, nullptr, dX,
-                               st, keep_bits ? dY : nullptr, sec);
+                               st, keep_bits ? dY : nullptr, sec, left);
 }
 
 int32_t moe_backward(const moe_config *cfg, const void *dY, const void *x, const float *Wg, const float *Wnoise,

@@ -19,7 +19,8 @@
 //   WGRAD    contraction over the rows of a segment, both operands MN-major:
 //            dW2 = hid^T.dys,  dW1 = xs^T.dz.
 // The last rows of a segment are loaded through a tensor map that ends with the segment: what lies behind them (the next
-// segment's rows) reads as zero, in both operands of a weight gradient.
+// segment's rows) reads as zero, in both operands of a weight gradient (short segments: see tc_wgrad_gemm). Zeros also cost the
+// tensor cores less power than the next segment's rows, which bounds the large products.
 // Weights are addressed through one tensor map with the expert as a coordinate, segment bounds
 // are read on the device: no per-expert descriptors and no host synchronisation.
 //
@@ -29,7 +30,9 @@
 #include <stdlib.h>
 #include <string.h>
 
-#include "moe_internal.cuh"
+#include <type_traits>
+
+#include "sums.cuh"
 
 namespace moe {
 
@@ -59,6 +62,7 @@ struct GemmParams {
     const int4 *tile_info;       // ROW_* with offsets: per M tile {segment or -1, first row, segment end, 0}
     // set by the launchers: N tiles per row of tiles, WGRAD tiles per segment, number of tile ids, K blocks of a ROW tile
     int32_t tiles_n, per_e, total_tiles, kblocks_row;
+    int32_t tile_n;  // columns of a tile: BN, or 128 in row products of the one-CTA kernel (see tc_row_gemm)
     int32_t nseg;
     int32_t M;  // WGRAD: rows of the per-segment output; ROW_*: unused
     int32_t N;  // output columns
@@ -259,9 +263,9 @@ __device__ __forceinline__ uint64_t desc_mnmajor(uint32_t addr) {
            ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
 }
 // Instruction descriptor: D fp32, A/B bf16, majors, N >> 3 at bit 17, M >> 4 at bit 24.
-__host__ __device__ constexpr uint32_t make_idesc(int a_mn, int b_mn) {
+__host__ __device__ constexpr uint32_t make_idesc(int a_mn, int b_mn, int n) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)a_mn << 15) | ((uint32_t)b_mn << 16) |
-           ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+           ((uint32_t)(n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
 }
 
 // Column sums over the 32 rows a warp holds (one row per lane, 32 columns per lane): returns in lane l
@@ -519,7 +523,7 @@ __device__ __forceinline__ bool tile_decode(const GemmParams &p, int32_t id, con
         t.e = e;
         t.mt = 0;
         t.m0 = tm * TM;
-        t.n0 = (rem - tm * p.tiles_n) * BN;
+        t.n0 = (rem - tm * p.tiles_n) * p.tile_n;
         t.b_chunk = t.n0 / 64;
         if (p.offsets) {
             t.row0 = raw.y;
@@ -548,7 +552,7 @@ __device__ __forceinline__ bool tile_decode(const GemmParams &p, int32_t id, con
         t.m0 = 0;
         t.b_chunk = 0;
         t.kblocks = p.kblocks_row;
-        t.n0 = (id - mt * p.tiles_n) * BN;
+        t.n0 = (id - mt * p.tiles_n) * p.tile_n;
         if (!p.offsets) {  // one segment of R rows; total_tiles is exact
             t.e = 0;
             t.row0 = mt * TM;
@@ -585,14 +589,13 @@ template <int KIND> struct SegmentEnd {
     const CUtensorMap *a, *b;
     bool ragged;
     __device__ __forceinline__ SegmentEnd(const GemmParams &p, const Tile &t, int32_t row0, int height) : a(nullptr), b(nullptr) {
-        if (KIND == WGRAD) ragged = p.seg_a && (t.row_end - t.row0) % BK != 0;
+        if (KIND == WGRAD) ragged = p.seg_a && (t.row_end - t.row0) % BK != 0;  // (never with off_mod)
         else ragged = p.seg_a && row0 + height > t.row_end;
         if (!ragged) return;
-        const int32_t e = KIND == WGRAD && p.off_mod > 0 ? t.e % p.off_mod : t.e;
-        a = p.seg_a + e;
+        a = p.seg_a + t.e;
         acquire_map(a);
         if (KIND == WGRAD) {
-            b = p.seg_b + e;
+            b = p.seg_b + t.e;
             acquire_map(b);
         }
     }
@@ -659,7 +662,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                     ok = mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, p.status);
                     if (!ok) break;
                     const uint32_t a_dst = base + s * STAGE_BYTES, b_dst = a_dst + A_BYTES;
-                    mbar_expect_tx(full_bar(s), STAGE_BYTES);
+                    mbar_expect_tx(full_bar(s), A_BYTES + p.tile_n * BK * 2);
                     if (KIND == WGRAD) {
                         const int r = t.row0 + kb * BK;
                         const bool tail = end.ragged && kb == t.kblocks - 1;
@@ -685,7 +688,6 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
-        constexpr uint32_t idesc = make_idesc(KIND == WGRAD ? 1 : 0, KIND == ROW_BK ? 0 : 1);
         int s = 0, acc = 0;
         uint32_t ph = 0, acc_ph = 0;
         bool ok = true;
@@ -693,6 +695,8 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         Tile t;
         while (ok && it.next(t)) {
             if (t.kblocks == 0) continue;  // empty segment (WGRAD): the epilogue writes zeros
+            // columns behind the output's are not computed (N is a multiple of 64)
+            const uint32_t idesc = make_idesc(KIND == WGRAD ? 1 : 0, KIND == ROW_BK ? 0 : 1, min(p.tile_n, p.N - t.n0));
             const int sub = ACC ? (t.e < p.segs_term0 ? p.sub_kb0 : p.sub_kb) : t.kblocks;  // K blocks per accumulator
             uint32_t d_tmem = tmem_base + acc * BN;
             for (int kb = 0; kb < t.kblocks; ++kb) {
@@ -707,8 +711,27 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t a_src = base + s * STAGE_BYTES, b_src = a_src + A_BYTES;
-                int ksteps = BK / 16;  // K steps of 16 rows to issue for this block: those behind the segment's end hold zeros
-                if (KIND == WGRAD && kb == t.kblocks - 1) ksteps = min(BK, t.row_end - (t.row0 + kb * BK) + 15) / 16;
+                int ksteps = BK / 16;  // K steps of 16 rows to issue for this block: none that lies behind the segment's end
+                if (KIND == WGRAD && kb == t.kblocks - 1) {
+                    const int valid = min(BK, t.row_end - (t.row0 + kb * BK));  // rows of this block inside the segment
+                    ksteps = (valid + 15) / 16;
+                    const int nz = ksteps * 16 - valid;
+                    // Without the segments' own maps (see tc_wgrad_gemm) the rows behind the end, up to the end of the step that holds
+                    // it, are the next segment's: zeroed in A AND in B (0 x finite = 0 would do for finite data; both keep a
+                    // non-finite value of the next segment out of this segment's sums): 128-B lines in all 64-column
+                    // chunks, the A tile's two chunks directly followed by the B tile's four.
+                    if (p.offsets && !p.seg_a && nz > 0) {
+                        const int lines = nz * ((BM + BN) / 64);
+                        for (int u = lane; u < lines * 8; u += 32) {
+                            const int line = u >> 3, part = u & 7;
+                            const int chunk = line / nz, krow = valid + line % nz;
+                            *reinterpret_cast<uint4 *>(smem + s * STAGE_BYTES + chunk * (BK * 128) + krow * 128 + part * 16) =
+                                make_uint4(0, 0, 0, 0);
+                        }
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        __syncwarp();
+                    }
+                }
                 if (lane == 0) {
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k) {
@@ -754,23 +777,33 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 for (int i = 0; i < 128; ++i) sums[i >> 5][i & 31] = 0.0f;
                 const int sub = t.e < p.segs_term0 ? p.sub_kb0 : p.sub_kb;
                 const int nsub = (t.kblocks + sub - 1) / sub;
+                const int columns = p.N - (t.n0 + half_a * 128);  // the warp's that exist (a multiple of 64); the others were not computed
+                auto release_acc = [&]() {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(tempty_bar(acc));
+                };
                 for (int sb = 0; sb < nsub; ++sb) {
                     ok = mbar_wait(tfull_bar(acc), acc_ph, abort_flag, p.status);
                     if (!ok) break;
                     tc_fence_after();
+                    // the accumulator goes back when it is read, before the last additions
+                    auto drain = [&](auto count_) {
+                        constexpr int COUNT = decltype(count_)::value;
+                        if (COUNT == 0) release_acc();
 #pragma unroll
-                    for (int cl = 0; cl < 4; ++cl) {
-                        uint32_t v[32];
-                        tc_ld_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + (half_a * 4 + cl) * 32, v);
-                        tc_ld_wait();
-                        if (cl == 3) {  // the accumulator is read: it goes back before the last additions
-                            tc_fence_before();
-                            __syncwarp();
-                            if (lane == 0) mbar_arrive(tempty_bar(acc));
+                        for (int cl = 0; cl < COUNT; ++cl) {
+                            uint32_t v[32];
+                            tc_ld_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + (half_a * 4 + cl) * 32, v);
+                            tc_ld_wait();
+                            if (cl == COUNT - 1) release_acc();
+#pragma unroll
+                            for (int j = 0; j < 32; ++j) sums[cl][j] += __uint_as_float(v[j]);
                         }
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) sums[cl][j] += __uint_as_float(v[j]);
-                    }
+                    };
+                    if (columns >= 128) drain(std::integral_constant<int, 4>());
+                    else if (columns > 0) drain(std::integral_constant<int, 2>());
+                    else drain(std::integral_constant<int, 0>());
                     if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
                 }
                 if (!ok) break;
@@ -797,10 +830,10 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 }
                 continue;
             }
-            // Two warps share each quarter of the accumulator's rows and take two boxes of 64 columns each.
+            // Two warps share each quarter of the accumulator's rows and take half of its columns each, in boxes of 64.
             const int half = (warp - 2) >> 2;
-            const int32_t first = t.n0 + half * (BN / 2);
-            const int boxes = min(2, max(0, (p.N - first) / 64));  // N is a multiple of 64
+            const int32_t first = t.n0 + half * (p.tile_n / 2);
+            const int boxes = min(p.tile_n / 128, max(0, (p.N - first) / 64));  // N is a multiple of 64
             BoxArgs b;
             b.tm_out = &tmO;
             b.box = smem + STAGES * STAGE_BYTES + 1024 + (warp - 2) * 4096;
@@ -827,7 +860,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             };
             for (int u = 0; u < boxes; ++u) {
                 b.col0 = first + 64 * u;
-                b.taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + half * (BN / 2) + 64 * u;
+                b.taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + half * (p.tile_n / 2) + 64 * u;
                 b.next_bias = (EPI & EPI_BIAS) && u + 1 < boxes ? bias_at + 64 : nullptr;
                 b.keep = u ? keep[1] : keep[0];
                 epilogue_box<EPI, false>(p, lane, b, bias, [&]() { if (u + 1 == boxes) release(); });
@@ -1331,17 +1364,17 @@ int32_t map_rows_mnmajor(CUtensorMap *tm, const void *p, int64_t rows, int64_t c
     return make_map(tm, p, 3, dims, str, box);
 }
 // per-expert weight [n, K, N] used as MN-major B: dims (64, K, N/64, n)
-int32_t map_weight_mnmajor(CUtensorMap *tm, const void *p, int64_t n, int64_t K, int64_t N) {
+int32_t map_weight_mnmajor(CUtensorMap *tm, const void *p, int64_t n, int64_t K, int64_t N, int tile_n = BN) {
     const uint64_t dims[4] = {64, (uint64_t)K, (uint64_t)(N / 64), (uint64_t)n};
     const uint64_t str[3] = {(uint64_t)N * 2, 128, (uint64_t)K * N * 2};
-    const uint32_t box[4] = {64, BK, BN / 64, 1};
+    const uint32_t box[4] = {64, BK, (uint32_t)tile_n / 64, 1};
     return make_map(tm, p, 4, dims, str, box);
 }
 // per-expert weight [n, N, K] used as K-major B: dims (K, N, n)
-int32_t map_weight_kmajor(CUtensorMap *tm, const void *p, int64_t n, int64_t N, int64_t K) {
+int32_t map_weight_kmajor(CUtensorMap *tm, const void *p, int64_t n, int64_t N, int64_t K, int tile_n = BN) {
     const uint64_t dims[3] = {(uint64_t)K, (uint64_t)N, (uint64_t)n};
     const uint64_t str[2] = {(uint64_t)K * 2, (uint64_t)N * K * 2};
-    const uint32_t box[3] = {64, BN, 1};
+    const uint32_t box[3] = {64, (uint32_t)tile_n, 1};
     return make_map(tm, p, 3, dims, str, box);
 }
 
@@ -1388,7 +1421,8 @@ int sm_count() {
 // Derived tile counts the device code divides by; ids are 32-bit.
 template <int KIND, int TM> int32_t complete_params(GemmParams &q, int64_t max_tiles) {
     if (max_tiles >= ((int64_t)1 << 31) - ((int64_t)1 << 22)) return MOE_ERR_UNSUPPORTED;
-    q.tiles_n = (int32_t)cdiv(q.N, BN);
+    if (!q.tile_n) q.tile_n = BN;
+    q.tiles_n = (int32_t)cdiv(q.N, q.tile_n);
     q.per_e = KIND == WGRAD ? (int32_t)cdiv(q.M, TM) * q.tiles_n : 1;
     q.total_tiles = (int32_t)max_tiles;
     q.kblocks_row = KIND == WGRAD ? 0 : q.nterms * (q.K / BK);
@@ -1536,24 +1570,13 @@ int32_t tc_segment_maps(const moe_config &c, SegmentMaps *maps, const void *xs_r
 
 // C[rows, N] = epilogue(A[rows, K] . B_e) over the segments; B_e = W[e] as [K, N] (transposed = false)
 // or as [N, K] read transposed (transposed = true).
-// tensor maps of the two operands of a weight gradient over the groups, and where those that end with the groups go ([2][n])
-struct GroupMaps { CUtensorMap a, b; CUtensorMap *out; };
 // Tile table of a ragged row GEMM: tile_prefix[e] = number of tm-row tiles of the segments before e
 // (tile_prefix[nseg] = total), and one record per M tile {segment, first row, segment end, 0}; records past
-// the last tile carry segment -1. One block; the others: the groups' tensor maps, where they are wanted.
+// the last tile carry segment -1. One block.
 __global__ void __launch_bounds__(1024) tile_table_kernel(const int32_t *__restrict__ offsets, int32_t n, int32_t tm,
                                                           int32_t max_m, int32_t *__restrict__ tile_prefix,
-                                                          int4 *__restrict__ info, const __grid_constant__ GroupMaps maps) {
+                                                          int4 *__restrict__ info) {
     wait_previous_kernel();
-    __shared__ __align__(128) uint32_t map_sh[32][32];
-    if (blockIdx.x > 0) {  // the groups' tensor maps, one per warp
-        const int32_t i = (blockIdx.x - 1) * 32 + (threadIdx.x >> 5);
-        if (i < 2 * n) {
-            const int32_t e = i >= n ? i - n : i;
-            write_segment_map(i >= n ? maps.b : maps.a, maps.out + i, offsets[e + 1], map_sh[threadIdx.x >> 5]);
-        }
-        return;
-    }
     __shared__ int32_t warp_sum[32];
     __shared__ int32_t carry;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -1602,108 +1625,48 @@ __global__ void __launch_bounds__(1024) tile_table_kernel(const int32_t *__restr
 }
 
 // ints a tile table needs behind its [nseg + 1] prefix (records are 16 bytes, 16-byte aligned)
-int64_t tc_tile_ws_ints(int64_t R, int64_t nseg) {
-    return ((nseg + 1 + 3) & ~(int64_t)3) + 4 * (cdiv(R, 128) + nseg + 1) + 32 /* alignment of the maps */ + 2 * 32 * nseg;
-}
+int64_t tc_tile_ws_ints(int64_t R, int64_t nseg) { return ((nseg + 1 + 3) & ~(int64_t)3) + 4 * (cdiv(R, 128) + nseg + 1); }
 static int4 *tile_info_of(int32_t *tile_prefix, int32_t nseg) {
     return reinterpret_cast<int4 *>(tile_prefix + ((nseg + 1 + 3) & ~3));
 }
-static CUtensorMap *group_maps_of(int32_t *tile_prefix, int64_t R, int32_t nseg) {
-    return reinterpret_cast<CUtensorMap *>((reinterpret_cast<uintptr_t>(tile_info_of(tile_prefix, nseg) + cdiv(R, 128) + nseg + 1) + 127) & ~(uintptr_t)127);
-}
 static int32_t launch_tile_table(const int32_t *offsets, int32_t nseg, int32_t tm, int64_t R, int32_t *tile_prefix,
-                                 cudaStream_t st, const GroupMaps *maps = nullptr) {
-    GroupMaps m;
-    if (maps) m = *maps;
-    else memset(&m, 0, sizeof(m));
-    launch_kernel(tile_table_kernel, maps ? 1 + (unsigned)cdiv(2 * nseg, 32) : 1u, 1024, 0, st, offsets, nseg, tm, (int32_t)(cdiv(R, tm) + nseg),
-                  tile_prefix, tile_info_of(tile_prefix, nseg), m);
+                                 cudaStream_t st) {
+    launch_kernel(tile_table_kernel, 1, 1024, 0, st, offsets, nseg, tm, (int32_t)(cdiv(R, tm) + nseg), tile_prefix,
+                                          tile_info_of(tile_prefix, nseg));
     MOE_LAUNCHED();
     return MOE_OK;
 }
 
-// Sum of the epilogue's 32-row column sums over each segment (bias gradient), G blocks per M tile.
-// A thread block takes 64 columns of one segment: 16 column lanes (four adjacent columns each, 16-byte loads) by 16 row
-// lanes; row lane q takes the blocks b = b0 + q, b0 + q + 16, ... (eight loads in flight: the largest expert of a skewed
-// batch has over a thousand blocks and sets this kernel's duration) and the 16 sums are added in lane order: the
-// result does not depend on timing. A block takes COLS columns: 64, or, where a segment has about one tile (thousands of
-// experts), 1024: a segment of at most 16 blocks is then added by one thread per four columns, in the same order. (Both
-// in one kernel cost the narrow form a loop and spills: 61 us instead of 41 at 128 experts x 4096 columns.)
-template <int COLS>
-__global__ void __launch_bounds__(256) colsum_blocks_final_kernel(const float *__restrict__ part, int32_t N,
-                                                                  const int32_t *__restrict__ tile_prefix, int32_t G,
-                                                                  bf16 *__restrict__ out) {
+template <int COLS> __global__ void __launch_bounds__(256) colsum_blocks_final_kernel(const BlockSums a) {
     wait_previous_kernel();
     __shared__ float4 sh[16][16];
-    const int32_t e = blockIdx.x, q = threadIdx.x >> 4, cl = threadIdx.x & 15;
-    const int32_t b0 = tile_prefix[e] * G, b1 = tile_prefix[e + 1] * G;
-    auto store = [&](int32_t j, const float4 &t) {
-        const __nv_bfloat162 o0 = __floats2bfloat162_rn(t.x, t.y), o1 = __floats2bfloat162_rn(t.z, t.w);
-        uint2 pk;
-        pk.x = *reinterpret_cast<const uint32_t *>(&o0); pk.y = *reinterpret_cast<const uint32_t *>(&o1);
-        *reinterpret_cast<uint2 *>(out + (int64_t)e * N + j) = pk;
-    };
-    if (COLS > 64 && b1 - b0 <= 16) {
-        const int32_t j = blockIdx.y * COLS + threadIdx.x * 4;
-        if (j >= N) return;
-        float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-#pragma unroll 4
-        for (int32_t b = b0; b < b1; ++b) {
-            const float4 v = *reinterpret_cast<const float4 *>(part + (int64_t)b * N + j);
-            s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
-        }
-        store(j, s);
-        return;
-    }
-    for (int32_t c = 0; c < COLS; c += 64) {
-        const int32_t j = blockIdx.y * COLS + c + cl * 4;
-        if (COLS > 64 && j >= N) break;  // N is a multiple of 64: all threads alike
-        float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        int32_t b = b0 + q;
-        for (; b + 16 * 7 < b1; b += 16 * 8) {
-            float4 v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = *reinterpret_cast<const float4 *>(part + (int64_t)(b + 16 * u) * N + j);
-#pragma unroll
-            for (int u = 0; u < 8; ++u) { s.x += v[u].x; s.y += v[u].y; s.z += v[u].z; s.w += v[u].w; }
-        }
-        for (; b < b1; b += 16) {
-            const float4 v = *reinterpret_cast<const float4 *>(part + (int64_t)b * N + j);
-            s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
-        }
-        if (COLS > 64) __syncthreads();  // sh may still be read for the columns before
-        sh[q][cl] = s;
-        __syncthreads();
-        if (q == 0) {
-            float4 t = sh[0][cl];
-#pragma unroll
-            for (int u = 1; u < 16; ++u) { t.x += sh[u][cl].x; t.y += sh[u][cl].y; t.z += sh[u][cl].z; t.w += sh[u][cl].w; }
-            store(j, t);
-        }
-    }
+    block_sums_final<COLS>(a, blockIdx.x, blockIdx.y, sh);
 }
 
 int64_t tc_colsum_part_floats(int64_t R, int32_t nseg, int32_t N) { return (cdiv(R, 128) * 4 + 8 * (int64_t)nseg + 8) * N; }
 
 // colsum_part / colsum_out: if set, out's column sums per segment (a bias gradient) are formed in the epilogue
-// and reduced into colsum_out [nseg, N]; colsum_part needs tc_colsum_part_floats(R, nseg, N) floats
+// and reduced into colsum_out [nseg, N] (sums_left given: that may be left to the caller); colsum_part needs tc_colsum_part_floats(R, nseg, N) floats
 int32_t tc_row_gemm(const void *A, const void *W, bool transposed, const int32_t *offsets, int32_t nseg, int64_t R,
                     int32_t N, int32_t K, void *out, const void *bias, const void *mask, int relu,
                     const SegmentPlan &plan, int counter, SegmentMap seg, int32_t *status, cudaStream_t st, int32_t flags,
                     float *colsum_part = nullptr, void *colsum_out = nullptr, uint32_t *bits_out = nullptr,
-                    const uint32_t *bits_in = nullptr) {
+                    const uint32_t *bits_in = nullptr, BlockSums *sums_left = nullptr) {
     if (R == 0) {
         if (colsum_out) MOE_CUDA(cudaMemsetAsync(colsum_out, 0, sizeof(bf16) * (size_t)nseg * N, st));
         return MOE_OK;
     }
     auto finish = [&](int32_t rc, int32_t G) -> int32_t {
         if (rc != MOE_OK || !colsum_out) return rc;
-        if (nseg >= 128 && R <= 128 * (int64_t)nseg)
-            launch_kernel(colsum_blocks_final_kernel<1024>, dim3((unsigned)nseg, (unsigned)cdiv(N, 1024)), 256, 0, st, colsum_part, N,
-                          plan.prefix[0], G, (bf16 *)colsum_out);
-        else
-            launch_kernel(colsum_blocks_final_kernel<64>, dim3((unsigned)nseg, (unsigned)cdiv(N, 64)), 256, 0, st, colsum_part, N,
-                          plan.prefix[0], G, (bf16 *)colsum_out);
+        const BlockSums sums = {colsum_part, plan.prefix[0], (bf16 *)colsum_out, nseg, N, G};
+        if (nseg >= 128 && R <= 128 * (int64_t)nseg) {
+            launch_kernel(colsum_blocks_final_kernel<1024>, dim3((unsigned)nseg, (unsigned)cdiv(N, 1024)), 256, 0, st, sums);
+        } else if (sums_left) {
+            *sums_left = sums;
+            return MOE_OK;
+        } else {
+            launch_kernel(colsum_blocks_final_kernel<64>, dim3((unsigned)nseg, (unsigned)cdiv(N, 64)), 256, 0, st, sums);
+        }
         MOE_LAUNCHED();
         return MOE_OK;
     };
@@ -1734,9 +1697,12 @@ int32_t tc_row_gemm(const void *A, const void *W, bool transposed, const int32_t
         return finish(transposed ? launch2<ROW_BK>(tmA, tmB, p, max_tiles2, st, nullptr, &tmO)
                                  : launch2<ROW_BMN>(tmA, tmB, p, max_tiles2, st, nullptr, &tmO), 8);
     }
-    if (transposed) MOE_TRY(map_weight_kmajor(&tmB, W, nseg, N, K));
-    else MOE_TRY(map_weight_mnmajor(&tmB, W, nseg, K, N));
-    const int64_t max_tiles = (cdiv(R, BM) + nseg) * cdiv(N, BN);
+    // Half as wide tiles where whole ones leave half of the SMs without: a handful of tokens, whose time is one tile's loads
+    const int64_t rows_of_tiles = cdiv(R, BM) + imin(nseg, R);
+    p.tile_n = N > 128 && 2 * rows_of_tiles * cdiv(N, BN) <= sm_count() ? 128 : BN;
+    if (transposed) MOE_TRY(map_weight_kmajor(&tmB, W, nseg, N, K, p.tile_n));
+    else MOE_TRY(map_weight_mnmajor(&tmB, W, nseg, K, N, p.tile_n));
+    const int64_t max_tiles = (cdiv(R, BM) + nseg) * cdiv(N, p.tile_n);
     CUtensorMap tmO;
     MOE_TRY(map_out_boxes(&tmO, out, R, N));
     return finish(transposed ? launch<ROW_BK>(tmA, tmB, p, max_tiles, st, &tmO) : launch<ROW_BMN>(tmA, tmB, p, max_tiles, st, &tmO), 4);
@@ -1750,7 +1716,11 @@ int32_t tc_wgrad_gemm(const void *A, const void *B, const int32_t *offsets, int3
     CUtensorMap tmA, tmB;
     GemmParams p = default_params();
     p.offsets = offsets; p.nseg = nseg; p.M = M; p.N = N; p.R = R;
-    p.seg_a = plan.maps_of(seg_a); p.seg_b = plan.maps_of(seg_b);
+    // The last K block of a segment through the segment's own maps: each costs the loading thread a fence, so that with one or two K
+    // blocks to a segment the one-CTA kernel clears the rows in shared memory instead (4096 experts x 64 rows: 1070 us, with maps 1187;
+    // 256 x 78: 67, 75; but 256 x 188: 93, 82; on SM pairs, where clearing held the tensor cores up for a third of a tile,
+    // 256 x 512: 192, 138)
+    if (R >= 128 * (int64_t)nseg) { p.seg_a = plan.maps_of(seg_a); p.seg_b = plan.maps_of(seg_b); }
     p.out = (bf16 *)out; p.status = status;
     CUtensorMap tmO;  // the experts' matrices as one tall matrix (a 32-row box never straddles two: M is a multiple of 64)
     MOE_TRY(map_out_boxes(&tmO, out, (int64_t)nseg * M, N));
@@ -1828,6 +1798,11 @@ __global__ void __launch_bounds__(256) reduce_partials_kernel(const float *__res
     else dWn[(g * d + q) * ldw + (j - n)] = (float)s;
 }
 
+__global__ void __launch_bounds__(256) gate_parts_kernel(const GateParts a) {
+    wait_previous_kernel();
+    gate_parts_sum(a, blockIdx.x);
+}
+
 bool tc_gate_bwd_supported(int32_t act, int32_t d, int32_t n) {
     // dX_gate contracts over the 2n logit columns (six split terms each) in one fp32 tensor-core accumulator, which
     // truncates: beyond 2n = 4096 the result drifts past 1e-5 (measured 2e-5 at n = 8192), so very wide flat gates take
@@ -1840,28 +1815,32 @@ bool tc_gate_bwd_supported(int32_t act, int32_t d, int32_t n) {
 // for the leading (hi) term: an fp32 accumulator loses low bits when a long run of same-sign terms is added (e.g. the
 // gradient of a constant input feature); 128 rows keep that below 1e-5 of the result. The mid and lo terms are 2^-8
 // and 2^-16 of the hi term and restart every GB_ROWS_LO rows. The restarts' sums are added in registers (see the
-// ACC kernel), so only one partial per range goes to global memory.
-constexpr int GB_ROWS_HI = 128, GB_ROWS_LO = 2048;
-static void gate_bwd_split(int64_t T, int32_t d, int32_t n, int32_t *nranges, int32_t *rows) {
+// ACC kernel), so only one partial per range goes to global memory. Ranges are whole lo sub-blocks, shorter ones where the batch
+// leaves fewer than two tiles per SM (8192 tokens, 512 features x 64 columns: 48 tiles, 24 us).
+constexpr int GB_ROWS_HI = 128, GB_ROWS_LO = 2048, GB_ROWS_LEAST = 256;
+static void gate_bwd_split(int64_t T, int32_t d, int32_t n, int32_t *nranges, int32_t *rows, int32_t *rows_lo) {
     const int64_t tiles_per_range = cdiv(d, BM) * cdiv(2 * n, BN);
+    int64_t lo = GB_ROWS_LO;
+    while (lo > GB_ROWS_LEAST && 3 * tiles_per_range * cdiv(T, lo) < 2 * (int64_t)sm_count()) lo /= 2;
     int64_t want = cdiv(3 * (int64_t)sm_count(), tiles_per_range);  // about three waves of hi-term tiles
-    const int64_t most = T > 0 ? cdiv(T, GB_ROWS_LO) : 1;
+    const int64_t most = T > 0 ? cdiv(T, lo) : 1;
     if (want > most) want = most;
     if (want < 1) want = 1;
-    const int64_t r = cdiv(cdiv(T > 0 ? T : 1, want), GB_ROWS_LO) * GB_ROWS_LO;  // whole lo sub-blocks per range
+    const int64_t r = cdiv(cdiv(T > 0 ? T : 1, want), lo) * lo;  // whole lo sub-blocks per range
+    *rows_lo = (int32_t)lo;
     *rows = (int32_t)r;
     *nranges = (int32_t)(T > 0 ? cdiv(T, r) : 1);
 }
 
 int64_t tc_gate_bwd_partials(int64_t T, int32_t d, int32_t n) {
-    int32_t nr, rows;
-    gate_bwd_split(T, d, n, &nr, &rows);
+    int32_t nr, rows, rows_lo;
+    gate_bwd_split(T, d, n, &nr, &rows, &rows_lo);
     return (int64_t)3 * nr * d * 2 * n;
 }
 
 int32_t launch_tc_gate_bwd(const void *x, int64_t T, int32_t d, int32_t n, const float *Wg, const float *Wn,
                            const void *dsplit, void *wsplit, float *partials, float *dWg, float *dWn,
-                           float *dX_gate, int32_t *status, cudaStream_t st, int32_t flags, int32_t ldw) {
+                           float *dX_gate, int32_t *status, cudaStream_t st, int32_t flags, int32_t ldw, GateParts *parts_left) {
     const int32_t n2 = 2 * n;
     if (T == 0 && ldw > 0) {
         for (int32_t q = 0; q < d; ++q) MOE_CUDA(cudaMemsetAsync(dWg + (int64_t)q * ldw, 0, sizeof(float) * n2, st));
@@ -1874,8 +1853,8 @@ int32_t launch_tc_gate_bwd(const void *x, int64_t T, int32_t d, int32_t n, const
     }
     launch_kernel(split_weights_kernel, (unsigned)cdiv((int64_t)d * n2, 256), 256, 0, st, Wg, Wn, d, n, (bf16 *)wsplit, ldw > 0 ? ldw : n);
     MOE_LAUNCHED();
-    int32_t nr, rows;
-    gate_bwd_split(T, d, n, &nr, &rows);
+    int32_t nr, rows, rows_lo;
+    gate_bwd_split(T, d, n, &nr, &rows, &rows_lo);
     {   // dW partials: contraction over the tokens, cut into row ranges, one set per precision term
         CUtensorMap tmA, tmB;
         MOE_TRY(map_rows_mnmajor(&tmA, x, T, d, BM / 64));
@@ -1884,11 +1863,15 @@ int32_t launch_tc_gate_bwd(const void *x, int64_t T, int32_t d, int32_t n, const
         p.nseg = 3 * nr; p.M = d; p.N = n2; p.R = T; p.out_f32 = partials; p.status = status;
         p.segs_term0 = nr; p.rows_per_seg0 = rows;
         p.rows_per_seg = rows; p.segs_per_term = nr; p.b_term_chunks = n2 / 64;
-        p.sub_kb0 = GB_ROWS_HI / BK; p.sub_kb = GB_ROWS_LO / BK; p.interleave = 3;
+        p.sub_kb0 = GB_ROWS_HI / BK; p.sub_kb = rows_lo / BK; p.interleave = 3;
         MOE_TRY(launch_acc_wgrad(tmA, tmB, p, (int64_t)p.nseg * cdiv(d, BM) * cdiv(n2, BN), st));
-        launch_kernel(reduce_partials_kernel, (unsigned)cdiv((int64_t)d * n2, 256), 256, 0, st, partials, 3 * nr, (int64_t)d * n2, d, n, dWg, dWn,
-                                                                                     ldw > 0 ? ldw : n);
-        MOE_LAUNCHED();
+        const GateParts parts = {partials, 3 * nr, d, n2, n, ldw > 0 ? ldw : n, dWg, dWn};
+        if (parts_left) {
+            *parts_left = parts;
+        } else {
+            launch_kernel(gate_parts_kernel, (unsigned)cdiv((int64_t)d * n2, 256), 256, 0, st, parts);
+            MOE_LAUNCHED();
+        }
     }
     {   // dX_gate: six cross terms of the two split operands, concatenated along the contraction
         CUtensorMap tmA, tmB;
@@ -1982,10 +1965,7 @@ int32_t launch_tc_hier_secondary_bwd(const void *xs_p, const void *dsplit_s, voi
         CUtensorMap tmA, tmB;
         MOE_TRY(map_rows_mnmajor(&tmA, xs_p, P1 > 0 ? P1 : 1, d, BM / 64));
         MOE_TRY(map_rows_mnmajor(&tmB, dsplit_s, P1 > 0 ? P1 : 1, 3 * n2, BN / 64));
-        const GroupMaps maps = {tmA, tmB, group_maps_of(tile_prefix, P1, a)};
-        MOE_TRY(launch_tile_table(offsets_p, a, BM, P1, tile_prefix, st, &maps));  // the tiles of dX_sec below, too
         GemmParams p = default_params();
-        p.seg_a = maps.out; p.seg_b = maps.out + a;
         p.offsets = offsets_p; p.nseg = 3 * a; p.off_mod = a; p.b_term_chunks = n2 / 64;
         p.M = d; p.N = n2; p.R = P1; p.out_f32 = partials; p.status = status;
         MOE_TRY(launch<WGRAD>(tmA, tmB, p, (int64_t)p.nseg * cdiv(d, BM) * cdiv(n2, BN), st));
@@ -1997,6 +1977,7 @@ int32_t launch_tc_hier_secondary_bwd(const void *xs_p, const void *dsplit_s, voi
         CUtensorMap tmA, tmB;
         MOE_TRY(map_rows_kmajor(&tmA, dsplit_s, P1, 3 * n2));
         MOE_TRY(map_weight_kmajor(&tmB, wsplit_s, a, d, 3 * n2));
+        MOE_TRY(launch_tile_table(offsets_p, a, BM, P1, tile_prefix, st));
         GemmParams p = default_params();
         p.offsets = offsets_p; p.tile_prefix = tile_prefix; p.tile_info = tile_info_of(tile_prefix, a);
         p.nseg = a; p.N = d; p.K = n2; p.R = P1;
@@ -2011,15 +1992,14 @@ int32_t launch_tc_hier_secondary_bwd(const void *xs_p, const void *dsplit_s, voi
 
 int32_t launch_tc_ffn_bwd(const moe_config &c, const void *xs, const void *hid, const void *dys,
                           const int32_t *offsets, const void *W1, const void *W2, void *dxs, void *dW1, void *db1,
-                          void *dW2, void *db2, void *dz, float *colsum, const SegmentPlan &plan, int32_t *status_word,
-                          cudaStream_t st, const uint32_t *relu_bits) {
+                          void *dW2, void *dz, float *colsum, const SegmentPlan &plan, int32_t *status_word,
+                          cudaStream_t st, const uint32_t *relu_bits, BlockSums *db1_left) {
     const int64_t R = (int64_t)c.T * c.k;
-    MOE_TRY(launch_segment_colsum(dys, c.act, offsets, c.n, R, c.d, db2, colsum, plan.prefix_of(COLSUM_ROWS), st));
     MOE_TRY(tc_wgrad_gemm(hid, dys, offsets, c.n, R, c.h, c.d, dW2, status_word, st, c.flags, plan, PLAN_WGRAD_A,
                           MAP_HID_COLS, MAP_DYS_COLS));
     // db1 = column sums of dz, formed in the epilogue of the GEMM that produces dz
     MOE_TRY(tc_row_gemm(dys, W2, true, offsets, c.n, R, c.h, c.d, dz, nullptr, hid, 0, plan, PLAN_ROWS_A, MAP_DYS_ROWS, status_word, st, c.flags,
-                        colsum, db1, nullptr, relu_bits));
+                        colsum, db1, nullptr, relu_bits, db1_left));
     MOE_TRY(tc_wgrad_gemm(xs, dz, offsets, c.n, R, c.d, c.h, dW1, status_word, st, c.flags, plan, PLAN_WGRAD_B,
                           MAP_XS_COLS, MAP_DZ_COLS));
     return tc_row_gemm(dz, W1, true, offsets, c.n, R, c.d, c.h, dxs, nullptr, nullptr, 0, plan, PLAN_ROWS_B, MAP_DZ_ROWS, status_word, st, c.flags);

@@ -3,9 +3,19 @@
 // c = x.W_g and the raw noise logits r = x.W_noise.
 #include <math_constants.h>
 
-#include "moe_internal.cuh"
+#include "sums.cuh"
 
 namespace moe {
+
+// Tile sums of a bias gradient by the first blocks of a launch (memory beside the arithmetic of the others); their number
+struct Beside {
+    ColumnSums sums;
+    int32_t blocks, slabs;
+    __device__ __forceinline__ void run(int32_t block) const {
+        if (sums.act == MOE_BF16) column_sums_partial<bf16>(sums, block / slabs, block % slabs);
+        else column_sums_partial<float>(sums, block / slabs, block % slabs);
+    }
+};
 
 // One warp per row. With sigma = softplus(r), z = (c - thr)/sigma, q_j = dLoad_j * phi(z_j)/sigma_j:
 //   softmax over the kept slots:  dH[idx_s] += g_s (dg_s - sum_s' g_s' dg_s')
@@ -19,10 +29,11 @@ __global__ void __launch_bounds__(256) gate_logit_grads_kernel(
     const int32_t *__restrict__ idx, const float *__restrict__ gates, const float *__restrict__ kth_vals,
     const int32_t *__restrict__ kth_idx, const float *__restrict__ dgates, const float *__restrict__ dload,
     const int32_t *__restrict__ dload_row_group, int64_t rows, int32_t n, int32_t k, float *__restrict__ dlogit,
-    bf16 *__restrict__ dsplit, const int32_t *__restrict__ split_row_index) {
+    bf16 *__restrict__ dsplit, const int32_t *__restrict__ split_row_index, const __grid_constant__ Beside beside) {
     wait_previous_kernel();
+    if ((int32_t)blockIdx.x < beside.blocks) return beside.run(blockIdx.x);
     const int lane = threadIdx.x & 31;
-    const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int64_t row = (int64_t)(blockIdx.x - beside.blocks) * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (row >= rows) return;
     int32_t sel_idx[MOE_MAX_K];
     float sel_dh[MOE_MAX_K];
@@ -144,10 +155,11 @@ __global__ void __launch_bounds__(256) gate_logit_grads_pairs_kernel(
     const int32_t *__restrict__ idx, const float *__restrict__ gates, const float *__restrict__ kth_vals,
     const int32_t *__restrict__ kth_idx, const float *__restrict__ dgates, const float *__restrict__ dload,
     const int32_t *__restrict__ dload_row_group, int64_t rows, int32_t n, int32_t k, bf16 *__restrict__ dsplit,
-    const int32_t *__restrict__ split_row_index) {
+    const int32_t *__restrict__ split_row_index, const __grid_constant__ Beside beside) {
     wait_previous_kernel();
+    if ((int32_t)blockIdx.x < beside.blocks) return beside.run(blockIdx.x);
     const int lane = threadIdx.x & 31;
-    const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int64_t row = (int64_t)(blockIdx.x - beside.blocks) * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (row >= rows) return;
     int32_t sel_idx[KS];
     float sel_dh[KS];
@@ -238,14 +250,16 @@ int32_t launch_gate_logit_grads(const float *noise, const float *clean, const fl
                                 const float *gates, const float *kth_vals, const int32_t *kth_idx,
                                 const float *dgates, const float *dload, const int32_t *dload_row_group,
                                 int64_t rows, int32_t n, int32_t k, float *dlogit, void *dsplit,
-                                const int32_t *split_row_index, cudaStream_t st) {
-    if (rows == 0) return MOE_OK;
-    const unsigned grid = (unsigned)cdiv(rows, 8);
+                                const int32_t *split_row_index, cudaStream_t st, const ColumnSums *sums) {
+    if (rows == 0) return sums ? launch_segment_colsum(*sums, false, st) : MOE_OK;
+    Beside beside = {};
+    if (sums) beside = {*sums, (int32_t)(column_tiles(*sums) * column_slabs(*sums)), (int32_t)column_slabs(*sums)};
+    const unsigned grid = (unsigned)(cdiv(rows, 8) + beside.blocks);
     if (dsplit && n % 32 == 0 && n <= 256) {  // the tensor-core path: paired columns
 #define MOE_LOGIT_PAIRS_KS(NVP, KS)                                                                                      \
     launch_kernel((gate_logit_grads_pairs_kernel<NVP, KS>), grid, 256, 0, st, noise, clean, raw, idx, gates, kth_vals, kth_idx, dgates, \
                                                                  dload, dload_row_group, rows, n, k, (bf16 *)dsplit,      \
-                                                                 split_row_index)
+                                                                 split_row_index, beside)
 #define MOE_LOGIT_PAIRS(NVP)                                \
     do {                                                    \
         if (k <= 2) MOE_LOGIT_PAIRS_KS(NVP, 2);             \
@@ -263,7 +277,7 @@ int32_t launch_gate_logit_grads(const float *noise, const float *clean, const fl
 #define MOE_LOGIT_GRADS(NV)                                                                                          \
     launch_kernel(gate_logit_grads_kernel<NV>, grid, 256, 0, st, noise, clean, raw, idx, gates, kth_vals, kth_idx, dgates, dload, \
                                                       dload_row_group, rows, n, k, dlogit, (bf16 *)dsplit,      \
-                                                      split_row_index)
+                                                      split_row_index, beside)
     if (n <= 32) MOE_LOGIT_GRADS(1);
     else if (n <= 64) MOE_LOGIT_GRADS(2);
     else if (n <= 128) MOE_LOGIT_GRADS(4);

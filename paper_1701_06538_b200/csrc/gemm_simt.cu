@@ -11,7 +11,7 @@
 #include <algorithm>
 #include <type_traits>
 
-#include "moe_internal.cuh"
+#include "sums.cuh"
 
 namespace moe {
 
@@ -54,6 +54,7 @@ struct SimtRun {
     int32_t splits;      // mode 1: the contraction range of a segment is cut into this many slices
     const SegmentPlan *plan;  // host side: tile prefixes made already, or nullptr
     float *part;         // splits > 1: [splits][nseg][M][N] partial results instead of C
+    GateParts *parts_left;  // host side: where a product over one segment leaves its partial results to be added later, or nullptr
 };
 
 // AK: A(i, k) is contiguous along k (else along i); BJ: B(k, j) is contiguous along j (else along k). QA4, QB4: quads of A / B can
@@ -64,7 +65,15 @@ template <typename TA, typename TB, typename TC, bool QA4, bool QB4, bool AK, bo
 __global__ void __launch_bounds__((BM / TM) * (BN / TN), TM * TN >= 64 ? 3 : TM * TN >= 32 ? 4 : 8) simt_gemm_kernel(const __grid_constant__ SimtRun run) {
     wait_previous_kernel();
     constexpr int NTX = BN / TN, NTY = BM / TM, NT = NTX * NTY;
+    // An operand whose contraction index is the contiguous one is stored transposed, four elements of a quad in four rows of the
+    // tile: the lanes of a warp hold BK / 4 quads of 128 / BK tile rows, and without a swizzle those stores met in a few banks (four
+    // to a bank at 32 x 32 x 32). Tile row i of step k stands at i ^ swizzle(k). (Not in the larger tiles: two to a bank there, and
+    // the reads of every step would pay for it, 38 -> 41 us at 4170 x 512 x 256.)
     constexpr int LDA = BM + 4, LDB = BN + 4;
+    constexpr bool SWZ = BM * BN <= 32 * 32;
+    constexpr int SWZ_UNIT = BK <= 32 ? 128 / BK : 4, SWZ_K = BK <= 32 ? 4 : 8;
+    auto swizzle_a = [](int k) { return SWZ && AK ? (k / SWZ_K % ((BM < 32 ? BM : 32) / SWZ_UNIT)) * SWZ_UNIT : 0; };
+    auto swizzle_b = [](int k) { return SWZ && !BJ ? (k / SWZ_K % ((BN < 32 ? BN : 32) / SWZ_UNIT)) * SWZ_UNIT : 0; };
     constexpr int QA = BM * BK / 4 / NT, QB = BN * BK / 4 / NT;  // quads a thread stages per K block
     constexpr int VA = TM < 4 ? TM : 4, VB = TN < 4 ? TN : 4;    // rows / columns per shared-memory read
     static_assert(QA * NT * 4 == BM * BK && QB * NT * 4 == BN * BK, "whole quads per thread");
@@ -76,6 +85,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), TM * TN >= 64 ? 3 : TM 
     static_assert(NT % (BK / 4) == 0 && NT % (BM / 4) == 0 && NT % (BN / 4) == 0, "a thread's quads are a fixed step apart");
     __shared__ __align__(16) float As[2][BK * LDA];
     __shared__ __align__(16) float Bs[2][BK * LDB];
+    __shared__ int4 tile_at;
     const SimtGemm &g = run.g;
     if (g.clear && threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0) *g.clear = 0;
     const int tid = threadIdx.x, tx = tid % NTX, ty = tid / NTX;
@@ -84,16 +94,11 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), TM * TN >= 64 ? 3 : TM 
     int32_t e = 0, slice = 0;
     if (g.mode == 0) {
         if (g.offsets) {
-            const int32_t b = blockIdx.x;
-            if (b >= run.tile_prefix[g.nseg]) return;
-            int lo = 0, hi = g.nseg;
-            while (hi - lo > 1) {
-                const int mid = (lo + hi) >> 1;
-                if (run.tile_prefix[mid] <= b) lo = mid; else hi = mid;
-            }
-            e = lo;
-            m0 = g.offsets[e] + (int64_t)(b - run.tile_prefix[e]) * BM;
-            m_end = g.offsets[e + 1];
+            const int4 at = segment_of_tile(run.tile_prefix, g.offsets, g.nseg, blockIdx.x, &tile_at);
+            if (at.x < 0) return;
+            e = at.x;
+            m0 = at.y + (int64_t)at.w * BM;
+            m_end = at.z;
         } else {
             m0 = (int64_t)blockIdx.x * BM;
             m_end = g.row_count ? (int64_t)*g.row_count : g.M;
@@ -232,7 +237,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), TM * TN >= 64 ? 3 : TM 
 #pragma unroll
         for (int q = 0; q < QA; ++q) {
             const float4 v = !QA4 || ((live_a >> q) & 1u) ? ra[q].get() : zero;
-            float *dst = &As[buf][ka(q) * LDA + ia(q)];
+            float *dst = &As[buf][ka(q) * LDA + (ia(q) ^ swizzle_a(ka(q)))];
             if (AK) { dst[0] = v.x; dst[LDA] = v.y; dst[2 * LDA] = v.z; dst[3 * LDA] = v.w; }
             else *reinterpret_cast<float4 *>(dst) = v;
         }
@@ -244,7 +249,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), TM * TN >= 64 ? 3 : TM 
 #pragma unroll
         for (int q = 0; q < QB; ++q) {
             const float4 v = !QB4 || ((live_b >> q) & 1u) ? rb[q].get() : zero;
-            float *dst = &Bs[buf][kb(q) * LDB + jb(q)];
+            float *dst = &Bs[buf][kb(q) * LDB + (jb(q) ^ swizzle_b(kb(q)))];
             if (!BJ) { dst[0] = v.x; dst[LDB] = v.y; dst[2 * LDB] = v.z; dst[3 * LDB] = v.w; }
             else *reinterpret_cast<float4 *>(dst) = v;
         }
@@ -262,7 +267,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), TM * TN >= 64 ? 3 : TM 
     auto load_frag = [&](int buf, int k, int f) {
 #pragma unroll
         for (int i = 0; i < TM; i += VA) {
-            const float *src = &As[buf][k * LDA + row_at(i)];
+            const float *src = &As[buf][k * LDA + (row_at(i) ^ swizzle_a(k))];
             if constexpr (VA == 4) {
                 const float4 w = *reinterpret_cast<const float4 *>(src);
                 fa[f][i] = w.x; fa[f][i + 1] = w.y; fa[f][i + 2] = w.z; fa[f][i + 3] = w.w;
@@ -273,7 +278,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), TM * TN >= 64 ? 3 : TM 
         }
 #pragma unroll
         for (int j = 0; j < TN; j += VB) {
-            const float *src = &Bs[buf][k * LDB + col_at(j)];
+            const float *src = &Bs[buf][k * LDB + (col_at(j) ^ swizzle_b(k))];
             if constexpr (VB == 4) {
                 const float4 w = *reinterpret_cast<const float4 *>(src);
                 fb[f][j] = w.x; fb[f][j + 1] = w.y; fb[f][j + 2] = w.z; fb[f][j + 3] = w.w;
@@ -423,7 +428,9 @@ static int32_t simt_launch(SimtRun &run, int32_t *tile_prefix, cudaStream_t st) 
     run.tile_prefix = ready ? ready : tile_prefix;
     launch_kernel((simt_gemm_kernel<TA, TB, TC, QA4, QB4, AK, BJ, BM, BN, TM, TN, BK>), grid, (BM / TM) * (BN / TN), 0, st, run);
     MOE_LAUNCHED();
-    if (run.part) {
+    if (run.part && run.parts_left) {  // left for a later launch
+        *run.parts_left = {run.part, run.splits, (int32_t)g.M, (int32_t)g.N, (int32_t)(g.C2 ? g.c_split : g.N), (int32_t)g.sc_i, (float *)g.C, (float *)g.C2};
+    } else if (run.part) {
         launch_kernel(simt_reduce_kernel, (unsigned)cdiv(g.M * g.N * g.nseg, 256), 256, 0, st, run);
         MOE_LAUNCHED();
     }
@@ -469,9 +476,11 @@ static int32_t simt_pick_tile(SimtRun &run, bool vec_a, bool vec_b, int32_t *til
 }
 
 // part: simt_wgrad_splits(M, N, nseg, rows) * nseg * M * N floats (mode 1, float results), or nullptr: no slices
-int32_t launch_simt_gemm(const SimtGemm &g_in, int32_t *tile_prefix, cudaStream_t st, float *part, const SegmentPlan *plan) {
+int32_t launch_simt_gemm(const SimtGemm &g_in, int32_t *tile_prefix, cudaStream_t st, float *part, const SegmentPlan *plan,
+                         GateParts *parts_left) {
     SimtRun run;
     run.plan = plan;
+    run.parts_left = parts_left;
     run.g = g_in;
     SimtGemm &g = run.g;
     if (!g.offsets) g.nseg = 1;
@@ -511,125 +520,30 @@ int32_t launch_simt_gemm(const SimtGemm &g_in, int32_t *tile_prefix, cudaStream_
 // Column sums per segment (bias gradients): partial sums over tiles of 128 rows, then an ordered
 // pass over each segment's tiles. Deterministic.
 // ------------------------------------------------------------------------------------------
-constexpr int CS_ROWS = COLSUM_ROWS;
-int64_t colsum_ws_floats(int64_t R, int32_t n, int32_t N) { return (cdiv(R, CS_ROWS) + n) * (int64_t)N + 64; }
+int64_t colsum_ws_floats(int64_t R, int32_t n, int32_t N) { return (cdiv(R, COLSUM_ROWS) + n) * (int64_t)N + 64; }
 
-// One block per 128-row tile and per slab of 32 * V columns (V = elements of a 16-byte vector): lane l owns V adjacent
-// columns, warp w the tile's rows w, w + 8, ..., read with 16-byte loads, four rows in flight; the eight warps' sums are
-// added in warp order. A segment of one tile is finished here.
-template <typename XT>
-__global__ void __launch_bounds__(256) colsum_partial_kernel(const XT *__restrict__ in,
-                                                             const int32_t *__restrict__ offsets, int32_t nseg,
-                                                             int32_t N, const int32_t *__restrict__ tile_prefix,
-                                                             float *__restrict__ part, XT *__restrict__ out) {
+template <typename XT> __global__ void __launch_bounds__(256) colsum_partial_kernel(const ColumnSums a) {
     wait_previous_kernel();
-    constexpr int V = 16 / sizeof(XT);
-    __shared__ float sh[8][32 * V];
-    const int32_t b = blockIdx.x;
-    if (b >= tile_prefix[nseg]) return;
-    int lo = 0, hi = nseg;
-    while (hi - lo > 1) {
-        int mid = (lo + hi) >> 1;
-        if (tile_prefix[mid] <= b) lo = mid; else hi = mid;
-    }
-    const int64_t r0 = offsets[lo] + (int64_t)(b - tile_prefix[lo]) * CS_ROWS;
-    const int64_t r1 = min(r0 + (int64_t)CS_ROWS, (int64_t)offsets[lo + 1]);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int32_t j = (blockIdx.y * 32 + lane) * V;
-    float s[V];
-#pragma unroll
-    for (int u = 0; u < V; ++u) s[u] = 0.0f;
-    if (j + V <= N) {  // N is a multiple of V wherever rows are 16-byte aligned
-        int64_t r = r0 + w;
-        for (; r + 24 < r1; r += 32) {
-            uint4 v[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) v[q] = *reinterpret_cast<const uint4 *>(in + (r + 8 * q) * N + j);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const XT *e = reinterpret_cast<const XT *>(&v[q]);
-#pragma unroll
-                for (int u = 0; u < V; ++u) s[u] += to_f32(e[u]);
-            }
-        }
-        for (; r < r1; r += 8) {
-            const uint4 v = *reinterpret_cast<const uint4 *>(in + r * N + j);
-            const XT *e = reinterpret_cast<const XT *>(&v);
-#pragma unroll
-            for (int u = 0; u < V; ++u) s[u] += to_f32(e[u]);
-        }
-    }
-#pragma unroll
-    for (int u = 0; u < V; ++u) sh[w][lane * V + u] = s[u];
-    __syncthreads();
-    for (int c = threadIdx.x; c < 32 * V; c += 256) {
-        const int32_t col = blockIdx.y * 32 * V + c;
-        if (col < N) {
-            float t = sh[0][c];
-#pragma unroll
-            for (int q = 1; q < 8; ++q) t += sh[q][c];
-            if (tile_prefix[lo + 1] - tile_prefix[lo] == 1) out[(int64_t)lo * N + col] = from_f32<XT>(t);
-            else part[(int64_t)b * N + col] = t;
-        }
-    }
+    column_sums_partial<XT>(a, blockIdx.x, blockIdx.y);
 }
-
-// Sum of a segment's tile sums (a segment of one tile is complete already, which with thousands of experts most are: a
-// block then looks at COLS = 256 columns, 32 at a time): a block takes 32 columns, its eight warps the tiles b0 + w, b0 + w + 8, ...
-// (eight loads in flight: the largest expert of a skewed batch has hundreds of tiles), the eight sums are added in warp order.
-template <typename XT, int COLS>
-__global__ void __launch_bounds__(256) colsum_final_kernel(const float *__restrict__ part, int32_t N,
-                                                           const int32_t *__restrict__ tile_prefix,
-                                                           XT *__restrict__ out) {
+template <int COLS> __global__ void __launch_bounds__(256) colsum_final_kernel(const ColumnSums a) {
     wait_previous_kernel();
     __shared__ float sh[8][32];
-    const int32_t e = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int32_t b0 = tile_prefix[e], b1 = tile_prefix[e + 1];
-    if (b1 - b0 == 1) return;
-    for (int32_t c = 0; c < COLS; c += 32) {
-        const int32_t j0 = blockIdx.y * COLS + c, j = j0 + lane;
-        if (COLS > 32 && j0 >= N) break;
-        float s = 0.0f;
-        if (j < N) {
-            int32_t b = b0 + w;
-            for (; b + 8 * 7 < b1; b += 64) {
-                float v[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) v[u] = part[(int64_t)(b + 8 * u) * N + j];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) s += v[u];
-            }
-            for (; b < b1; b += 8) s += part[(int64_t)b * N + j];
-        }
-        if (COLS > 32) __syncthreads();  // sh may still be read for the columns before
-        sh[w][lane] = s;
-        __syncthreads();
-        if (w == 0 && j < N) {
-            float t = sh[0][lane];
-#pragma unroll
-            for (int u = 1; u < 8; ++u) t += sh[u][lane];
-            out[(int64_t)e * N + j] = from_f32<XT>(t);
-        }
-    }
+    column_sums_final<COLS>(a, blockIdx.x, blockIdx.y, sh);
 }
 
-int32_t launch_segment_colsum(const void *in, int32_t act, const int32_t *offsets, int32_t nseg, int64_t R,
-                              int32_t N, void *out, float *scratch, const int32_t *tile_prefix, cudaStream_t st) {
-    const int vcols = act == MOE_BF16 ? 256 : 128;  // columns per block of the partial sums: 32 lanes x one 16-byte vector
-    dim3 g1((unsigned)(cdiv(R, CS_ROWS) + nseg), (unsigned)cdiv(N, vcols));
-    const bool many = nseg >= 1024;
-    dim3 g2((unsigned)nseg, (unsigned)cdiv(N, many ? 256 : 32));
-    auto run = [&](auto *typed) -> int32_t {
-        using XT = typename std::remove_pointer<decltype(typed)>::type;
-        XT *o = static_cast<XT *>(out);
-        launch_kernel(colsum_partial_kernel<XT>, g1, 256, 0, st, static_cast<const XT *>(in), offsets, nseg, N, tile_prefix, scratch, o);
-        MOE_LAUNCHED();
-        if (many) launch_kernel((colsum_final_kernel<XT, 256>), g2, 256, 0, st, scratch, N, tile_prefix, o);
-        else launch_kernel((colsum_final_kernel<XT, 32>), g2, 256, 0, st, scratch, N, tile_prefix, o);
-        MOE_LAUNCHED();
-        return MOE_OK;
-    };
-    return act == MOE_BF16 ? run((bf16 *)nullptr) : run((float *)nullptr);
+int32_t launch_segment_colsum(const ColumnSums &a, bool finish, cudaStream_t st) {
+    const dim3 tiles((unsigned)column_tiles(a), (unsigned)column_slabs(a));
+    if (a.act == MOE_BF16) launch_kernel(colsum_partial_kernel<bf16>, tiles, 256, 0, st, a);
+    else launch_kernel(colsum_partial_kernel<float>, tiles, 256, 0, st, a);
+    MOE_LAUNCHED();
+    return finish ? launch_segment_colsum_final(a, st) : MOE_OK;
+}
+int32_t launch_segment_colsum_final(const ColumnSums &a, cudaStream_t st) {
+    if (a.nseg >= COLSUM_MANY) launch_kernel(colsum_final_kernel<256>, dim3((unsigned)a.nseg, (unsigned)cdiv(a.N, 256)), 256, 0, st, a);
+    else launch_kernel(colsum_final_kernel<32>, dim3((unsigned)a.nseg, (unsigned)cdiv(a.N, 32)), 256, 0, st, a);
+    MOE_LAUNCHED();
+    return MOE_OK;
 }
 
 }  // namespace moe

@@ -154,15 +154,19 @@ int32_t launch_tc_gate_fwd(const void *x, int64_t T, int32_t d, int32_t n, const
 
 // ----------------------------------------------------------------------------- routing (route.cu)
 int64_t dispatch_ws_elems(int64_t R, int32_t n);  // int32 elements of scratch
+// plan: the segment plan, in the same launches if they can (*planned says so)
 int32_t launch_dispatch_index(const int32_t *topk_idx, int64_t R, int32_t n, int32_t *perm, int32_t *inv_perm,
-                              int32_t *counts, int32_t *offsets, int32_t *scratch, cudaStream_t st);
+                              int32_t *counts, int32_t *offsets, int32_t *scratch, cudaStream_t st,
+                              const struct PlanArgs *plan = nullptr, bool *planned = nullptr);
+// sums: the loss sums over the batch, by blocks of their own in the same launch (one launch after it completes them:
+// level_reduce, by combine or by itself)
 int32_t launch_dispatch_rows(const void *x, int32_t act, int64_t T, int32_t k, int32_t d, const int32_t *inv_perm,
-                             void *xs, cudaStream_t st);
+                             void *xs, cudaStream_t st, const struct LevelSums *sums = nullptr);
 // keep != nullptr: the layer epilogue of Appendix C (sigmoid, dropout through the packed keep bits [T, d/8] with the
 // kept activations scaled by keep_scale = 1 / (1 - DropProb), residual xres added); see route.cu
 int32_t launch_combine(const void *ys, int32_t act, const float *gates, const int32_t *inv_perm, int64_t T,
                        int32_t k, int32_t d, void *y, cudaStream_t st, const void *xres = nullptr,
-                       const uint8_t *keep = nullptr, float keep_scale = 1.0f);
+                       const uint8_t *keep = nullptr, float keep_scale = 1.0f, const struct LevelSums *sums = nullptr);
 int32_t launch_combine_bwd(const void *dY, const void *ys, int32_t act, const float *gates,
                            const int32_t *inv_perm, int64_t T, int32_t k, int32_t d, float *dgates, void *dys,
                            cudaStream_t st, const uint8_t *keep = nullptr, float keep_scale = 1.0f,
@@ -172,16 +176,31 @@ int32_t launch_combine_bwd(const void *dY, const void *ys, int32_t act, const fl
 // is given instead, rounded to the act type. sec: float rows [T * k1, d] of the secondary gates, added to add_f32 (which is
 // given then); perm: row of a slot, or nullptr
 struct SecondaryRows { const float *rows; const int32_t *perm; int32_t k1; };
+// tail: sums that earlier launches have left, by blocks of their own
 int32_t launch_dispatch_bwd(const void *dxs, int32_t act, const int32_t *inv_perm, int64_t T, int32_t k,
                             int32_t d, const float *add_f32, float *out_f32, void *out_act, cudaStream_t st,
-                            const void *add_act = nullptr, const SecondaryRows &sec = SecondaryRows{});
+                            const void *add_act = nullptr, const SecondaryRows &sec = SecondaryRows{},
+                            const struct BackwardTail *tail = nullptr);
 // The segment of tile `b` of a ragged product {segment, first row, segment end, tile inside the segment}, or segment -1 behind the last
 // tile, looked up by the whole block (barriers): every thread looks at its share of the segments, so that a block waits for
-// one round of loads (a binary search over the prefix waits for one per step, 2 of the 5 us of a block with little to do). sh: one int4
+// one round of loads (a binary search over the prefix waits for one per step, 2 of the 5 us of a block with little to do). With
+// thousands of segments the search is less work (12288 blocks, 4096 segments: 80 us, this way 96). sh: one int4
 __device__ __forceinline__ int4 segment_of_tile(const int32_t *__restrict__ tile_prefix, const int32_t *__restrict__ offsets, int32_t nseg,
                                                 int32_t b, int4 *sh) {
     if (threadIdx.x == 0) *sh = make_int4(-1, 0, 0, 0);
     __syncthreads();
+    if (nseg > 1024) {
+        if (threadIdx.x == 0 && b < tile_prefix[nseg]) {
+            int32_t lo = 0, hi = nseg;
+            while (hi - lo > 1) {
+                const int32_t mid = (lo + hi) >> 1;
+                if (tile_prefix[mid] <= b) lo = mid; else hi = mid;
+            }
+            *sh = make_int4(lo, offsets[lo], offsets[lo + 1], b - tile_prefix[lo]);
+        }
+        __syncthreads();
+        return *sh;
+    }
     for (int32_t q = threadIdx.x; q < nseg; q += blockDim.x) {
         const int32_t p0 = tile_prefix[q], p1 = tile_prefix[q + 1], o0 = offsets[q], o1 = offsets[q + 1];
         if (p0 <= b && b < p1) *sh = make_int4(q, o0, o1, b - p0);
@@ -222,8 +241,11 @@ struct SegmentPlan {
 struct Cv2Job { const float *v; int32_t m; float scale; float *out; };  // out = scale * dCV^2(v)/dv
 int64_t plan_ints(int64_t R, int64_t n);
 SegmentPlan plan_at(int32_t *ws, int64_t R, int64_t n);
-int32_t launch_segment_plan(const SegmentPlan &plan, const int32_t *offsets, int32_t n, int64_t R, int32_t *status,
-                            cudaStream_t st, const SegmentMaps *maps = nullptr, const Cv2Job *jobs = nullptr /* two */);
+struct PlanArgs;  // plan.cuh
+// status: cleared if given; maps: base maps of the operands, or nullptr; jobs: two, or nullptr
+void fill_plan(PlanArgs *a, const SegmentPlan &plan, int32_t n, int64_t R, int32_t *status, const SegmentMaps *maps = nullptr,
+               const Cv2Job *jobs = nullptr);
+int32_t launch_segment_plan(const PlanArgs &a, const int32_t *offsets, cudaStream_t st);
 // One segment's map, by a warp: a copy of `base` whose rows (dimension 1) end at `rows`. sh: 128 bytes, 128-byte aligned
 __device__ __forceinline__ void write_segment_map(const CUtensorMap &base, CUtensorMap *out, int32_t rows, uint32_t *sh) {
     const int lane = threadIdx.x & 31;
@@ -247,13 +269,22 @@ struct LossOut {
 };
 struct LossFinal { float w_imp, w_load; float *losses; LossOut copy; };
 int64_t losses_ws_floats(int64_t rows, int32_t n);
-// Partial column sums over rows of the gate mass (importance) and of P(x, i) (load).
-// flat / primary level: seg == nullptr. Secondary level: rows are slots p, grouped through
-// perm/offsets (sorted row r -> slot perm[r]); sums are per segment: load_out [nseg, n].
-int32_t launch_level_sums(const int32_t *idx, const float *gates, const float *clean, const float *raw,
-                          const float *kth_vals, int64_t rows, int32_t n, int32_t k, float *importance_out,
-                          float *load_out, float *scratch, cudaStream_t st, const LossFinal *fin = nullptr);
-// (fin: the two losses as well, in the same launches; importance_out and load_out are both wanted then)
+// Column sums over rows of the gate mass (importance) and of P(x, i) (load), and with fin.losses set the two losses: per-chunk sums
+// by one launch, an ordered pass over the chunks by the next.
+struct LevelSums {
+    const int32_t *idx;
+    const float *gates, *clean, *raw, *kth_vals;
+    int64_t rows;
+    int32_t n, k, chunks;
+    float *part_imp, *part_load;
+    int32_t *ticket;
+    float *importance, *load;  // nullptr: not wanted (with fin.losses both are)
+    LossFinal fin;
+};
+LevelSums level_sums(const int32_t *idx, const float *gates, const float *clean, const float *raw, const float *kth_vals, int64_t rows,
+                     int32_t n, int32_t k, float *importance, float *load, float *scratch, const LossFinal *fin = nullptr);
+int32_t launch_level_sums(const LevelSums &sums, cudaStream_t st);   // both launches
+constexpr int LEVEL_RIDE_MAX = 256;  // columns up to which the sums go along with other launches
 int32_t launch_cv2(const float *importance, int32_t n_imp, const float *load, int32_t n_load, float w_imp,
                    float w_load, float *losses, cudaStream_t st, const LossOut &copy);
 int32_t launch_cv2_grads(const Cv2Job *jobs /* two */, cudaStream_t st);
@@ -283,7 +314,8 @@ int32_t launch_gate_logit_grads(const float *noise, const float *clean, const fl
                                 const float *gates, const float *kth_vals, const int32_t *kth_idx,
                                 const float *dgates, const float *dload, const int32_t *dload_row_group,
                                 int64_t rows, int32_t n, int32_t k, float *dlogit, void *dsplit,
-                                const int32_t *split_row_index, cudaStream_t st);
+                                const int32_t *split_row_index, cudaStream_t st, const struct ColumnSums *beside = nullptr);
+// beside: tile sums of a bias gradient, by blocks of their own in the same launch
 
 // ----------------------------------------------------------------------------- SIMT grouped GEMM (gemm_simt.cu)
 enum GemmType { G_F32 = 0, G_BF16 = 1 };
@@ -321,16 +353,56 @@ struct SimtGemm {
     const int32_t *b_row_index;
     const int32_t *c_row_index;
 };
+// partial sums of a gate's weight gradient [nparts][d][cols], to be added into dW (columns before split) and dW2 (the others), rows ld apart
+struct GateParts {
+    const float *part;
+    int32_t nparts, d, cols, split, ld;
+    float *dW, *dW2;
+};
 // Mode 1 over segments: K is the number of rows of all segments. part: simt_wgrad_splits(M, N, nseg, K) * nseg * M * N
 // floats let a product with few tiles be cut along its contraction (float results only)
 int32_t simt_wgrad_splits(int64_t M, int64_t N, int32_t nseg, int64_t K);
 int32_t launch_simt_gemm(const SimtGemm &g, int32_t *tile_prefix, cudaStream_t st, float *part = nullptr,
-                         const SegmentPlan *plan = nullptr);  // plan: tile prefixes made already (heights 16 / 32 / 64)
-// out[e, j] = sum over the rows of segment e of in[r, j]   (out, in of the act type)
+                         const SegmentPlan *plan = nullptr,   // plan: tile prefixes made already (heights 16 / 32 / 64)
+                         GateParts *parts_left = nullptr);    // given: slices' results of a product over one segment are left to be added
+constexpr int COLSUM_ROWS = 128;   // height of the tiles of ColumnSums::tile_prefix
+constexpr int COLSUM_MANY = 1024;  // segments from which the pass over the tiles looks at 256 columns a block
+// out[e, j] = sum over the rows of segment e of in[r, j]   (out, in of the act type): sums of tiles, then an ordered pass over them
+struct ColumnSums {
+    const void *in;
+    void *out;
+    int32_t act, nseg, N;
+    int64_t R;
+    const int32_t *offsets, *tile_prefix;
+    float *part;  // colsum_ws_floats
+    __device__ __forceinline__ void put(int32_t e, int32_t j, float v) const {
+        if (act == MOE_BF16) static_cast<bf16 *>(out)[(int64_t)e * N + j] = from_f32<bf16>(v);
+        else static_cast<float *>(out)[(int64_t)e * N + j] = v;
+    }
+};
 int64_t colsum_ws_floats(int64_t R, int32_t n, int32_t N);
-int32_t launch_segment_colsum(const void *in, int32_t act, const int32_t *offsets, int32_t nseg, int64_t R,
-                              int32_t N, void *out, float *scratch, const int32_t *tile_prefix, cudaStream_t st);
-constexpr int COLSUM_ROWS = 128;  // height of the tiles of tile_prefix
+static inline int64_t column_tiles(const ColumnSums &a) { return cdiv(a.R, COLSUM_ROWS) + a.nseg; }
+static inline int64_t column_slabs(const ColumnSums &a) { return cdiv(a.N, a.act == MOE_BF16 ? 256 : 128); }  // of 32 lanes x one 16-byte vector
+int32_t launch_segment_colsum(const ColumnSums &a, bool finish, cudaStream_t st);
+int32_t launch_segment_colsum_final(const ColumnSums &a, cudaStream_t st);
+// out[e, j] = sum of segment e's blocks of 32-row column sums, G blocks a tile
+struct BlockSums {
+    const float *part;
+    const int32_t *tile_prefix;
+    bf16 *out;
+    int32_t nseg, N, G;
+};
+// What the fused backward leaves for its last launch (0 blocks: nothing)
+struct BackwardTail {
+    GateParts parts;
+    BlockSums blocks;
+    ColumnSums columns[2];
+    int32_t parts_blocks, block_blocks, column_blocks[2];
+    int64_t total() const { return (int64_t)parts_blocks + block_blocks + column_blocks[0] + column_blocks[1]; }
+};
+// blocks up to which they go along with the rows' (whose registers leave three on an SM); more take one launch of their own
+// (32768 rows x 512, 256 experts, 9216 blocks: 111 us together, 83 apart; 3001 rows x 320, 20 experts, 510 blocks: 10 us, apart 16)
+constexpr int64_t TAIL_RIDE_MAX = 8 * 148;
 
 // ----------------------------------------------------------------------------- tensor-core experts (ffn_tc.cu)
 bool tc_ffn_supported(const moe_config &c);
@@ -382,7 +454,8 @@ bool tc_gate_bwd_supported(int32_t act, int32_t d, int32_t n);
 int64_t tc_gate_bwd_partials(int64_t T, int32_t d, int32_t n);  // floats of partial-sum scratch
 int32_t launch_tc_gate_bwd(const void *x, int64_t T, int32_t d, int32_t n, const float *Wg, const float *Wn,
                            const void *dsplit, void *wsplit, float *partials, float *dWg, float *dWn,
-                           float *dX_gate, int32_t *status, cudaStream_t st, int32_t flags, int32_t ldw = 0);
+                           float *dX_gate, int32_t *status, cudaStream_t st, int32_t flags, int32_t ldw = 0,
+                           GateParts *parts_left = nullptr);
 // (ldw > 0: Wg / Wn, dWg / dWn are the left and right column halves of one [d, 2n] matrix with row stride ldw)
 int32_t launch_tc_gate_fwd_grouped(const void *xs_p, int64_t P1, int32_t d, int32_t a, int32_t b, const void *wsplit_s,
                                    const int32_t *offsets_p, int32_t *tile_prefix, const int32_t *perm_p, float *clean, float *raw,
@@ -394,9 +467,10 @@ int32_t launch_tc_hier_secondary_bwd(const void *xs_p, const void *dsplit_s, voi
                                      float *dX_sec, int32_t *status, cudaStream_t st);
 int64_t tc_tile_ws_ints(int64_t R, int64_t nseg);  // int32s of a [nseg + 1] tile prefix followed by its tile table
 int64_t tc_colsum_part_floats(int64_t R, int32_t nseg, int32_t N);  // scratch of the fused bias-gradient sums
+// db2 (column sums of dys) is the caller's; db1_left given: the last pass over db1's block sums may be, too
 int32_t launch_tc_ffn_bwd(const moe_config &c, const void *xs, const void *hid, const void *dys,
                           const int32_t *offsets, const void *W1, const void *W2, void *dxs, void *dW1, void *db1,
-                          void *dW2, void *db2, void *dz, float *colsum, const SegmentPlan &plan, int32_t *status_word,
-                          cudaStream_t st, const uint32_t *relu_bits = nullptr);
+                          void *dW2, void *dz, float *colsum, const SegmentPlan &plan, int32_t *status_word,
+                          cudaStream_t st, const uint32_t *relu_bits = nullptr, BlockSums *db1_left = nullptr);
 
 }  // namespace moe

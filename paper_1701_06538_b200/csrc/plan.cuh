@@ -1,0 +1,118 @@
+// The segment plan of a call (see plan.cu) as device code: one piece of it per block, by plan_kernel or by blocks of their own in the
+// launch that finds the segments (route.cu).
+#pragma once
+
+#include "moe_internal.cuh"
+#include "moments.cuh"
+
+namespace moe {
+
+struct PlanArgs {
+    SegmentPlan plan;
+    int32_t n, max_m;  // max_m: tile records of plan.info
+    int32_t *status;   // cleared if given
+    Cv2Job cv2[2];
+    int32_t map_block0;  // first block of the tensor maps
+    SegmentMaps maps;
+};
+constexpr int MAPS_PER_BLOCK = 64;  // two per warp
+inline int64_t plan_blocks(const PlanArgs &a) {
+    int64_t maps = 0;
+    for (int i = 0; i < SEGMENT_MAPS; ++i) maps += a.maps.made[i] ? a.n : 0;
+    return a.map_block0 + cdiv(maps, MAPS_PER_BLOCK);
+}
+// ints of shared memory a piece of the plan needs: the segments' lengths, or the maps under construction
+inline int64_t plan_shared_ints(int32_t n) { return n > MAPS_PER_BLOCK * 32 ? n : MAPS_PER_BLOCK * 32; }
+
+__device__ __forceinline__ int32_t *on_128_bytes(int32_t *shared) {
+    return shared + ((128u - ((uint32_t)__cvta_generic_to_shared(shared) & 127u)) & 127u) / 4u;
+}
+
+// exclusive prefix of the segments' tiles of bm rows; returns the total to every thread (1024 threads)
+static __device__ int32_t tile_prefix_block(const int32_t *offsets, int32_t n, int32_t bm, int32_t *prefix, int32_t *sh /* [32] */) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    int32_t carry = 0;
+    for (int32_t base = 0; base < n; base += 1024) {
+        const int32_t e = base + threadIdx.x;
+        const int32_t v = e < n ? (offsets[e + 1] - offsets[e] + bm - 1) / bm : 0;
+        int32_t inc = v;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int32_t o = __shfl_up_sync(0xffffffffu, inc, off);
+            if (lane >= off) inc += o;
+        }
+        __syncthreads();
+        if (lane == 31) sh[w] = inc;
+        __syncthreads();
+        const int32_t sw = sh[lane];
+        int32_t si = sw;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int32_t o = __shfl_up_sync(0xffffffffu, si, off);
+            if (lane >= off) si += o;
+        }
+        const int32_t before = __shfl_sync(0xffffffffu, si - sw, w);
+        if (e < n) prefix[e] = carry + before + inc - v;
+        carry += __shfl_sync(0xffffffffu, si, 31);
+    }
+    if (threadIdx.x == 0) prefix[n] = carry;
+    return carry;
+}
+
+// Piece `block` of the plan, by 1024 threads; offsets: global or shared memory; cnt: plan_shared_ints(n), on 128 bytes.
+// Pieces 0..3: tile prefixes (0: the records, the counters and the status word as well); 4, 5: loss gradients; from 6 on:
+// 1024 segments each of the order by size; from map_block0 on: the segments' tensor maps
+__device__ __forceinline__ void plan_piece(const PlanArgs &a, int32_t block, const int32_t *offsets, int32_t *cnt, int32_t *sh /* [32] */,
+                                           double *moments /* [32] */) {
+    const int32_t n = a.n;
+    if (block >= a.map_block0) {
+        const int w = threadIdx.x >> 5;
+        for (int q = 0; q < MAPS_PER_BLOCK / 32; ++q) {
+            int64_t i = (int64_t)(block - a.map_block0) * MAPS_PER_BLOCK + 32 * q + w;
+            int which = 0;  // the (i / n)-th map that is wanted
+            for (; which < SEGMENT_MAPS; ++which) {
+                if (!a.maps.made[which]) continue;
+                if (i < n) break;
+                i -= n;
+            }
+            if (which < SEGMENT_MAPS)
+                write_segment_map(a.maps.base[which], a.plan.maps + (int64_t)which * n + i, offsets[i + 1], (uint32_t *)cnt + 64 * w + 32 * q);
+        }
+        return;
+    }
+    if (block < PLAN_HEIGHTS) {
+        const int which = block;
+        if (which == 0) {
+            if (threadIdx.x < PLAN_COUNTERS && a.plan.counters) a.plan.counters[threadIdx.x] = 0;
+            if (threadIdx.x == 0 && a.status) *a.status = 0;
+        }
+        if (a.plan.bm[which] == 0) return;
+        int32_t *prefix = a.plan.prefix[which];
+        const int32_t bm = a.plan.bm[which], total = tile_prefix_block(offsets, n, bm, prefix, sh);
+        if (which != 0 || !a.plan.info) return;
+        __syncthreads();  // the prefix (global memory, this block's own writes) is complete
+        for (int32_t mt = threadIdx.x; mt < a.max_m; mt += 1024) {
+            if (mt >= total) { a.plan.info[mt] = make_int4(-1, 0, 0, 0); continue; }
+            int lo = 0, hi = n;  // last e with prefix[e] <= mt (empty segments share a prefix: take the last)
+            while (hi - lo > 1) {
+                const int mid = (lo + hi) >> 1;
+                if (prefix[mid] <= mt) lo = mid; else hi = mid;
+            }
+            a.plan.info[mt] = make_int4(lo, offsets[lo] + (mt - prefix[lo]) * bm, offsets[lo + 1], 0);
+        }
+    } else if (block < PLAN_HEIGHTS + 2) {
+        const Cv2Job &job = a.cv2[block - PLAN_HEIGHTS];
+        if (job.v) cv2_grad_block(job, moments);
+    } else if (a.plan.sched) {  // rank by descending size, equal sizes by index
+        for (int32_t e = threadIdx.x; e < n; e += 1024) cnt[e] = offsets[e + 1] - offsets[e];
+        __syncthreads();
+        const int32_t e = (block - PLAN_HEIGHTS - 2) * 1024 + threadIdx.x;
+        if (e >= n) return;
+        const int32_t mine = cnt[e];
+        int32_t rank = 0;
+        for (int32_t o = 0; o < n; ++o) rank += (cnt[o] > mine || (cnt[o] == mine && o < e)) ? 1 : 0;
+        a.plan.sched[rank] = make_int4(e, offsets[e], offsets[e + 1], 0);
+    }
+}
+
+}  // namespace moe

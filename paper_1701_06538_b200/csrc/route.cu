@@ -2,7 +2,11 @@
 // gate-weighted combine (Eq. 1) and their adjoints. All of it is HBM streaming: rows are moved
 // with 16-byte vector accesses, every token row is read once and written k times (dispatch) or
 // gathered k times and written once (combine).
-#include "moe_internal.cuh"
+#include <string.h>
+
+#include "losses.cuh"
+#include "plan.cuh"
+#include "sums.cuh"
 
 namespace moe {
 
@@ -14,7 +18,7 @@ namespace moe {
 //   3. exclusive scan of counts -> offsets                                (dispatch_scan_experts)
 //   4. per chunk the slots are ranked, 32 per warp with match_any, across the warps with a
 //      shared-memory cursor per expert                                     (dispatch_rank)
-// A single chunk needs only step 4, a moderate number of histogram entries only 1 and 4 (see launch_dispatch_index).
+// A few chunks need one launch, a moderate number of histogram entries only 1 and 4 (see launch_dispatch_index).
 // Integer atomics only (order-independent results); the permutation is unique and bit-exact.
 // ------------------------------------------------------------------------------------------
 constexpr int CH = 1024;  // slots per chunk
@@ -133,45 +137,93 @@ __device__ __forceinline__ int32_t block_scan_1024(int32_t v, int32_t *sh /* [32
     return __shfl_sync(0xffffffffu, si - sw, w) + inc - v;
 }
 
-// Where the sorted rows of a chunk's slots start, per expert (cursor[e], shared memory), found by one of
-//   RANK_ONE    the only chunk: counted here, no other kernel
-//   RANK_FEW    from the chunks' histograms: every block adds the chunks before its own and scans the totals (n <= 1024)
-//   RANK_MANY   from the scanned chunk bases and offsets
-// Then 32 warps take 32 slots each: equal experts inside a warp are ranked with match_any. BYTES (n <= 1024): every warp leaves how many
-// slots of an expert it has in the expert's row of 32 bytes, and the slots' starts follow from the bytes of the warps before; else the
-// warps advance the cursors one after the other, 32 barriers. (One warp walking the 32 groups with the loads on its critical path
-// took 16 us per chunk, but two chunks of 32 warps fill an SM: see dispatch_rank_warp_kernel.)
-enum RankFrom { RANK_ONE, RANK_FEW, RANK_MANY };
-constexpr int RANK_BYTES_MAX = 1024;
-template <int FROM, bool BYTES>
-__global__ void __launch_bounds__(1024) dispatch_rank_kernel(const int32_t *__restrict__ topk_idx, int64_t R, int32_t n,
-                                                             const int32_t *__restrict__ chunk_table, int32_t nchunks,
-                                                             int32_t *__restrict__ counts, int32_t *__restrict__ offsets,
-                                                             int32_t *__restrict__ perm, int32_t *__restrict__ inv_perm) {
+// Places of a chunk's 1024 slots (32 warps of 32): equal experts inside a warp are ranked with match_any; every warp leaves how many
+// slots of an expert it has in the expert's row of 32 bytes (warp_counts, cleared, 16 bytes each), and the slots' starts follow from
+// the bytes of the warps before: two barriers (the warps advancing a cursor one after the other: 32). Returns the slot's place
+// behind its expert's cursor.
+__device__ __forceinline__ int32_t bytes_before(const uint4 *row, int warps) {  // sum of the first `warps` bytes of an expert's row
+    const uint4 w[2] = {row[0], row[1]};
+    const uint32_t *words = reinterpret_cast<const uint32_t *>(w);
+    uint32_t sum = 0u;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int bytes = min(4, max(0, warps - 4 * i));
+        sum = __dp4a(bytes == 4 ? words[i] : words[i] & ((1u << (8 * bytes)) - 1u), 0x01010101u, sum);
+    }
+    return (int32_t)sum;
+}
+__device__ __forceinline__ int32_t rank_in_chunk(int32_t e, uint4 *warp_counts) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned peers = __match_any_sync(0xffffffffu, e);
+    const int leader = __ffs(peers) - 1;
+    __syncthreads();  // the rows are cleared
+    if (e >= 0 && lane == leader) reinterpret_cast<uint8_t *>(warp_counts)[e * 32 + warp] = (uint8_t)__popc(peers);
+    __syncthreads();
+    int32_t before = 0;
+    if (e >= 0 && lane == leader) before = bytes_before(warp_counts + 2 * e, warp);
+    return __shfl_sync(0xffffffffu, before, leader) + __popc(peers & ((1u << lane) - 1u));
+}
+__device__ __forceinline__ void place_slot(int32_t e, int32_t r, int64_t p, int64_t R, int32_t *perm, int32_t *inv_perm) {
+    if (e >= 0) {
+        MOE_BOUNDS_NOTE((uint32_t)r < (uint32_t)R);
+        perm[r] = (int32_t)p;
+        inv_perm[p] = r;
+    } else if (p < R) {
+        inv_perm[p] = -1;  // expert id outside [0, n): the slot is dropped; the row movers skip negative rows
+    }
+}
+__device__ __forceinline__ int32_t slot_expert(const int32_t *topk_idx, int64_t p, int64_t R, int32_t n) {
+    const int32_t e = p < R ? topk_idx[p] : -1;
+    return (uint32_t)e < (uint32_t)n ? e : -1;
+}
+
+// Up to 1024 experts: the blocks find the segments themselves, from all slots (SCAN: up to eight chunks, whose ids are read
+// together; no other launch) or from the chunks' histograms. Blocks behind the chunks' do the pieces of the
+// segment plan on the offsets they have found, which is then no launch of its own either.
+constexpr int INDEX_EXPERTS_MAX = 1024, INDEX_SCAN_MAX = 8;
+inline int64_t index_front_ints(int32_t n) { return 8 * n > plan_shared_ints(0) ? 8 * n : plan_shared_ints(0); }
+template <bool SCAN>
+__global__ void __launch_bounds__(1024) dispatch_index_kernel(const int32_t *__restrict__ topk_idx, int64_t R, int32_t n,
+                                                              const int32_t *__restrict__ chunk_table, int32_t nchunks, int32_t front_ints,
+                                                              int32_t *__restrict__ counts, int32_t *__restrict__ offsets,
+                                                              int32_t *__restrict__ perm, int32_t *__restrict__ inv_perm,
+                                                              const __grid_constant__ PlanArgs plan) {
     wait_previous_kernel();
-    extern __shared__ __align__(16) int32_t rank_sh[];
-    int32_t *cursor = rank_sh + (BYTES ? 8 * n : 0);  // next sorted row of each expert for this chunk; BYTES: behind the experts' rows of bytes
+    extern __shared__ __align__(128) int32_t index_sh[];
     __shared__ int32_t sh[32];
     __shared__ int32_t part_total[1024], part_before[1024];
-    uint4 *warp_counts = reinterpret_cast<uint4 *>(rank_sh);
-    if (BYTES) {
-        for (int32_t q = threadIdx.x; q < 2 * n; q += 1024) warp_counts[q] = make_uint4(0u, 0u, 0u, 0u);
-    }
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __shared__ double moments[32];
+    int32_t *front = on_128_bytes(index_sh);  // the experts' rows of bytes, or the scratch of the plan
+    int32_t *cursor = front + front_ints;     // next sorted row of each expert for this chunk; plan: the offsets, n + 1
+    uint4 *warp_counts = reinterpret_cast<uint4 *>(front);
+    const int tid = threadIdx.x, lane = tid & 31;
+    const bool ranks = (int32_t)blockIdx.x < nchunks;
     const int64_t p = (int64_t)blockIdx.x * CH + tid;
-    const bool live = p < R;
-    int32_t e = live ? topk_idx[p] : -1;
-    MOE_BOUNDS_NOTE(!live || (uint32_t)e < (uint32_t)n);
-    if ((uint32_t)e >= (uint32_t)n) e = -1;
-    if (FROM == RANK_MANY) {
-        const int32_t *base = chunk_table + (int64_t)blockIdx.x * n;
-        for (int32_t q = tid; q < n; q += 1024) cursor[q] = offsets[q] + base[q];
-    } else if (FROM == RANK_FEW) {
+    int32_t e = -1;
+    if (ranks) {
+        e = slot_expert(topk_idx, p, R, n);
+        MOE_BOUNDS_NOTE(p >= R || e >= 0);
+        for (int32_t q = tid; q < 2 * n; q += 1024) warp_counts[q] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    int32_t total = 0, before = 0;
+    if (SCAN) {
+        part_total[tid] = 0;
+        part_before[tid] = 0;
+        __syncthreads();
+        int32_t id[INDEX_SCAN_MAX];
+#pragma unroll
+        for (int c = 0; c < INDEX_SCAN_MAX; ++c) id[c] = c < nchunks ? slot_expert(topk_idx, (int64_t)c * CH + tid, R, n) : -1;
+#pragma unroll
+        for (int c = 0; c < INDEX_SCAN_MAX; ++c)
+            if (id[c] >= 0) atomicAdd(c < (int32_t)blockIdx.x ? &part_before[id[c]] : &part_total[id[c]], 1);
+        __syncthreads();
+        before = part_before[tid];
+        total = part_total[tid] + before;
+    } else {
         // thread (group, expert) adds its group's share of the chunks, the groups are then added per expert
         int32_t width = 32;
         while (width < n) width <<= 1;
         const int32_t q = tid & (width - 1), group = tid / width, groups = 1024 / width;
-        int32_t total = 0, before = 0;
         if (q < n) {
 #pragma unroll 8
             for (int32_t c = group; c < nchunks; c += groups) {
@@ -186,79 +238,77 @@ __global__ void __launch_bounds__(1024) dispatch_rank_kernel(const int32_t *__re
         total = before = 0;
         if (tid < n)
             for (int32_t g = 0; g < groups; ++g) { total += part_total[g * width + tid]; before += part_before[g * width + tid]; }
-        int32_t all;
-        const int32_t excl = block_scan_1024(total, sh, &all);
-        if (tid < n) {
-            cursor[tid] = excl + before;
-            if (blockIdx.x == 0) { counts[tid] = total; offsets[tid] = excl; }
-        }
-        if (tid == 0 && blockIdx.x == 0) offsets[n] = all;
-    } else {
-        for (int32_t q = tid; q < n; q += 1024) cursor[q] = 0;
+    }
+    int32_t all;
+    const int32_t excl = block_scan_1024(total, sh, &all);
+    if (!ranks) {
+        if (tid < n) cursor[tid] = excl;
+        if (tid == 0) cursor[n] = all;
+        __syncthreads();
+        plan_piece(plan, blockIdx.x - nchunks, cursor, front, sh, moments);
+        return;
+    }
+    if (tid < n) {
+        cursor[tid] = excl + before;
+        if (blockIdx.x == 0) { counts[tid] = total; offsets[tid] = excl; }
+    }
+    if (tid == 0 && blockIdx.x == 0) offsets[n] = all;
+    const int32_t place = rank_in_chunk(e, warp_counts);  // (its barriers: the cursors are written)
+    place_slot(e, e >= 0 ? cursor[e] + place : 0, p, R, perm, inv_perm);
+}
+
+// The same from the scanned chunk bases and offsets. BYTES: up to 1024 experts; else the warps advance the cursors one after the other.
+// (One warp walking the 32 groups with the loads on its critical path took 16 us per chunk, but two chunks of 32 warps fill an SM:
+// see dispatch_rank_warp_kernel.) ONE: the only chunk, counted here, no other kernel (more than 1024 experts).
+template <bool ONE, bool BYTES>
+__global__ void __launch_bounds__(1024) dispatch_rank_kernel(const int32_t *__restrict__ topk_idx, int64_t R, int32_t n,
+                                                             const int32_t *__restrict__ chunk_base,
+                                                             int32_t *__restrict__ counts, int32_t *__restrict__ offsets,
+                                                             int32_t *__restrict__ perm, int32_t *__restrict__ inv_perm) {
+    wait_previous_kernel();
+    extern __shared__ __align__(16) int32_t rank_sh[];
+    int32_t *cursor = rank_sh + (BYTES ? 8 * n : 0);  // next sorted row of each expert for this chunk
+    __shared__ int32_t sh[32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t p = (int64_t)blockIdx.x * CH + tid;
+    const int32_t e = slot_expert(topk_idx, p, R, n);
+    MOE_BOUNDS_NOTE(p >= R || e >= 0);
+    if (BYTES)
+        for (int32_t q = tid; q < 2 * n; q += 1024) reinterpret_cast<uint4 *>(rank_sh)[q] = make_uint4(0u, 0u, 0u, 0u);
+    const int32_t *base = chunk_base + (int64_t)blockIdx.x * n;
+    for (int32_t q = tid; q < n; q += 1024) cursor[q] = ONE ? 0 : offsets[q] + base[q];
+    if (BYTES) {
+        const int32_t place = rank_in_chunk(e, reinterpret_cast<uint4 *>(rank_sh));
+        place_slot(e, e >= 0 ? cursor[e] + place : 0, p, R, perm, inv_perm);
+        return;
     }
     const unsigned peers = __match_any_sync(0xffffffffu, e);
     const int rank = __popc(peers & ((1u << lane) - 1u)), leader = __ffs(peers) - 1;
     int32_t start = 0;
-    if (BYTES) {
-        __syncthreads();  // the rows are cleared
-        if (e >= 0 && lane == leader) reinterpret_cast<uint8_t *>(warp_counts)[e * 32 + warp] = (uint8_t)__popc(peers);
+    const int busy_warps = (int)min((int64_t)32, (R - (int64_t)blockIdx.x * CH + 31) / 32);
+    for (int w = 0; w < busy_warps; ++w) {
         __syncthreads();
-        // bytes of the first `warps` warps of an expert's row
-        auto sum_of = [&](int32_t q, int warps) {
-            const uint4 w[2] = {warp_counts[2 * q], warp_counts[2 * q + 1]};
-            const uint32_t *words = reinterpret_cast<const uint32_t *>(w);
-            uint32_t sum = 0u;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int bytes = min(4, max(0, warps - 4 * i));
-                sum = __dp4a(bytes == 4 ? words[i] : words[i] & ((1u << (8 * bytes)) - 1u), 0x01010101u, sum);
-            }
-            return (int32_t)sum;
-        };
-        if (e >= 0 && lane == leader) start = sum_of(e, warp) + (FROM == RANK_ONE ? 0 : cursor[e]);
-        start = __shfl_sync(0xffffffffu, start, leader);
-        if (FROM == RANK_ONE) {  // n <= 1024: a thread per expert
-            const int32_t v = tid < n ? sum_of(tid, 32) : 0;
+        if (warp == w && e >= 0 && lane == leader) {
+            start = cursor[e];
+            cursor[e] = start + __popc(peers);
+        }
+    }
+    start = __shfl_sync(0xffffffffu, start, leader);
+    if (ONE) {  // the cursors hold the counts now: scan them, then shift the ranks by their expert's offset
+        __syncthreads();
+        int32_t carry = 0;
+        for (int32_t q0 = 0; q0 < n; q0 += 1024) {
+            const int32_t q = q0 + tid, v = q < n ? cursor[q] : 0;
             int32_t all;
-            const int32_t excl = block_scan_1024(v, sh, &all);
-            if (tid < n) { counts[tid] = v; offsets[tid] = excl; cursor[tid] = excl; }
-            if (tid == 0) offsets[n] = all;
-            __syncthreads();
-            if (e >= 0) start += cursor[e];
+            const int32_t excl = carry + block_scan_1024(v, sh, &all);
+            if (q < n) { counts[q] = v; offsets[q] = excl; cursor[q] = excl; }
+            carry += all;
         }
-    } else {
-        const int busy_warps = (int)min((int64_t)32, (R - (int64_t)blockIdx.x * CH + 31) / 32);
-        for (int w = 0; w < busy_warps; ++w) {
-            __syncthreads();
-            if (warp == w && e >= 0 && lane == leader) {
-                start = cursor[e];
-                cursor[e] = start + __popc(peers);
-            }
-        }
-        start = __shfl_sync(0xffffffffu, start, leader);
-        if (FROM == RANK_ONE) {  // the cursors hold the counts now: scan them, then shift the ranks by their expert's offset
-            __syncthreads();
-            int32_t carry = 0;
-            for (int32_t q0 = 0; q0 < n; q0 += 1024) {
-                const int32_t q = q0 + tid, v = q < n ? cursor[q] : 0;
-                int32_t all;
-                const int32_t excl = carry + block_scan_1024(v, sh, &all);
-                if (q < n) { counts[q] = v; offsets[q] = excl; cursor[q] = excl; }
-                carry += all;
-            }
-            if (tid == 0) offsets[n] = carry;
-            __syncthreads();
-            if (e >= 0) start += cursor[e];
-        }
+        if (tid == 0) offsets[n] = carry;
+        __syncthreads();
+        if (e >= 0) start += cursor[e];
     }
-    if (e >= 0) {
-        const int32_t r = start + rank;
-        MOE_BOUNDS_NOTE((uint32_t)r < (uint32_t)R);
-        perm[r] = (int32_t)p;
-        inv_perm[p] = r;
-    } else if (live) {
-        inv_perm[p] = -1;  // expert id outside [0, n): the slot is dropped; the row movers skip negative rows
-    }
+    place_slot(e, start + rank, p, R, perm, inv_perm);
 }
 
 // RANK_MANY for more chunks than two per SM: one warp per chunk, up to 32 chunks in flight on an SM. It walks its slots in order,
@@ -309,31 +359,43 @@ __global__ void __launch_bounds__(32) dispatch_rank_warp_kernel(const int32_t *_
 }
 
 int32_t launch_dispatch_index(const int32_t *topk_idx, int64_t R, int32_t n, int32_t *perm, int32_t *inv_perm,
-                              int32_t *counts, int32_t *offsets, int32_t *scratch, cudaStream_t st) {
+                              int32_t *counts, int32_t *offsets, int32_t *scratch, cudaStream_t st, const PlanArgs *plan, bool *planned) {
     const int32_t nchunks = (int32_t)cdiv(R, CH);
+    if (planned) *planned = false;
     if (nchunks == 0) {
         MOE_CUDA(cudaMemsetAsync(counts, 0, sizeof(int32_t) * n, st));
         MOE_CUDA(cudaMemsetAsync(offsets, 0, sizeof(int32_t) * (n + 1), st));
         return MOE_OK;
     }
     const size_t sh = n * sizeof(int32_t);
-    // one chunk: one launch. Up to 64 Ki histogram entries every block can afford to read them all (128 chunks x 256
-    // experts: 1.5 us), which saves the two scans' launches, as long as all blocks run at once (two per SM: the entries
-    // read grow with the square of the chunks).
-    const bool bytes = n <= RANK_BYTES_MAX;
-    const size_t sh_rank = bytes ? 9 * sh : sh;  // at most 36 KiB with the bytes
-    if (nchunks == 1 && n <= 8192) {
-        if (bytes) launch_kernel(dispatch_rank_kernel<RANK_ONE, true>, 1, 1024, sh_rank, st, topk_idx, R, n, nullptr, 1, counts, offsets, perm, inv_perm);
-        else launch_kernel(dispatch_rank_kernel<RANK_ONE, false>, 1, 1024, sh_rank, st, topk_idx, R, n, nullptr, 1, counts, offsets, perm, inv_perm);
+    // Up to eight chunks every block counts all of them (the histograms' launch takes 3 us). Up to 64 Ki histogram entries
+    // every block can afford to read them all (128 chunks x 256 experts: 1.5 us), which saves the two scans' launches, as long as
+    // all blocks run at once (two per SM: the entries read grow with the square of the chunks).
+    const bool few_experts = n <= INDEX_EXPERTS_MAX, one_wave = nchunks <= 2 * 148;
+    const bool scan = few_experts && nchunks <= INDEX_SCAN_MAX, few = few_experts && one_wave && (int64_t)nchunks * n <= 65536;
+    if (!few_experts && nchunks == 1 && n <= 8192) {
+        launch_kernel(dispatch_rank_kernel<true, false>, 1, 1024, sh, st, topk_idx, R, n, nullptr, counts, offsets, perm, inv_perm);
         MOE_LAUNCHED();
         return MOE_OK;
     }
-    launch_kernel(dispatch_hist_kernel, nchunks, 256, sh, st, topk_idx, R, n, scratch);
-    MOE_LAUNCHED();
-    const bool one_wave = nchunks <= 2 * 148;
-    if (one_wave && bytes && (int64_t)nchunks * n <= 65536) {
-        launch_kernel(dispatch_rank_kernel<RANK_FEW, true>, nchunks, 1024, sh_rank, st, topk_idx, R, n, scratch, nchunks, counts, offsets, perm, inv_perm);
+    if (!scan) {
+        launch_kernel(dispatch_hist_kernel, nchunks, 256, sh, st, topk_idx, R, n, scratch);
         MOE_LAUNCHED();
+    }
+    if (scan || few) {
+        PlanArgs none;
+        if (!plan) memset(&none, 0, sizeof(none));
+        const int32_t front = (int32_t)index_front_ints(n);
+        const unsigned grid = (unsigned)(nchunks + (plan ? plan_blocks(*plan) : 0));
+        const size_t shared = 128 + sizeof(int32_t) * (front + n + 1);  // at most 36 KiB
+        if (scan)
+            launch_kernel(dispatch_index_kernel<true>, grid, 1024, shared, st, topk_idx, R, n, nullptr, nchunks, front, counts, offsets, perm,
+                          inv_perm, plan ? *plan : none);
+        else
+            launch_kernel(dispatch_index_kernel<false>, grid, 1024, shared, st, topk_idx, R, n, scratch, nchunks, front, counts, offsets, perm,
+                          inv_perm, plan ? *plan : none);
+        MOE_LAUNCHED();
+        if (planned) *planned = plan != nullptr;
         return MOE_OK;
     }
     launch_kernel(dispatch_scan_chunks_kernel, (unsigned)cdiv(n, 32), 1024, 0, st, scratch, nchunks, n, counts);
@@ -346,8 +408,10 @@ int32_t launch_dispatch_index(const int32_t *topk_idx, int64_t R, int32_t n, int
         MOE_LAUNCHED();
         return MOE_OK;
     }
-    if (bytes) launch_kernel(dispatch_rank_kernel<RANK_MANY, true>, nchunks, 1024, sh_rank, st, topk_idx, R, n, scratch, nchunks, counts, offsets, perm, inv_perm);
-    else launch_kernel(dispatch_rank_kernel<RANK_MANY, false>, nchunks, 1024, sh_rank, st, topk_idx, R, n, scratch, nchunks, counts, offsets, perm, inv_perm);
+    if (few_experts)
+        launch_kernel(dispatch_rank_kernel<false, true>, nchunks, 1024, 9 * sh, st, topk_idx, R, n, scratch, counts, offsets, perm, inv_perm);
+    else
+        launch_kernel(dispatch_rank_kernel<false, false>, nchunks, 1024, sh, st, topk_idx, R, n, scratch, counts, offsets, perm, inv_perm);
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -498,16 +562,26 @@ template <typename XT> struct Vec16 {
     __device__ __forceinline__ void set(int i, float v) { reinterpret_cast<XT *>(&raw)[i] = from_f32<XT>(v); }
 };
 
-// xs[inv_perm[t*k+s]] = x[t] for every slot s: x is read once, written k times
-template <typename XT>
+// xs[inv_perm[t*k+s]] = x[t] for every slot s: x is read once, written k times. NV > 0: the first blocks form the loss sums
+// of up to 32 * NV columns (arithmetic) while the others move rows (memory).
+template <typename XT, int NV>
 __global__ void __launch_bounds__(256) dispatch_rows_kernel(const XT *__restrict__ x, int64_t T, int32_t k,
                                                             int32_t d, const int32_t *__restrict__ inv_perm,
-                                                            XT *__restrict__ xs) {
+                                                            XT *__restrict__ xs, const __grid_constant__ LevelSums sums) {
     wait_previous_kernel();
     constexpr int VN = 16 / sizeof(XT);
+    int32_t block = blockIdx.x, blocks = gridDim.x;
+    if constexpr (NV > 0) {
+        if (block < sums.chunks) {
+            level_sums_rows<NV>(sums, block);
+            return;
+        }
+        block -= sums.chunks;
+        blocks -= sums.chunks;
+    }
     const int lane = threadIdx.x & 31;
-    const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    const int64_t warp = (int64_t)block * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int64_t nwarps = (int64_t)blocks * (blockDim.x >> 5);
     const int nvec = d / VN;
     const int64_t R = T * k;  // a row index outside [0, R) (dropped slot, or a caller's bad inv_perm) is skipped, never followed
     for (int64_t t = warp; t < T; t += nwarps) {
@@ -528,13 +602,24 @@ __global__ void __launch_bounds__(256) dispatch_rows_kernel(const XT *__restrict
 }
 
 int32_t launch_dispatch_rows(const void *x, int32_t act, int64_t T, int32_t k, int32_t d, const int32_t *inv_perm,
-                             void *xs, cudaStream_t st) {
+                             void *xs, cudaStream_t st, const LevelSums *sums) {
     if (T == 0) return MOE_OK;
-    const unsigned grid = (unsigned)imin(cdiv(T, 8), 148 * 16);
-    if (act == MOE_BF16)
-        launch_kernel(dispatch_rows_kernel<bf16>, grid, 256, 0, st, (const bf16 *)x, T, k, d, inv_perm, (bf16 *)xs);
-    else
-        launch_kernel(dispatch_rows_kernel<float>, grid, 256, 0, st, (const float *)x, T, k, d, inv_perm, (float *)xs);
+    const LevelSums job = sums ? *sums : LevelSums{};
+    const unsigned grid = (unsigned)(imin(cdiv(T, 8), 148 * 16) + (sums ? sums->chunks : 0));
+#define MOE_ROWS(NV)                                                                                                          \
+    do {                                                                                                                      \
+        if (act == MOE_BF16)                                                                                                  \
+            launch_kernel((dispatch_rows_kernel<bf16, NV>), grid, 256, 0, st, (const bf16 *)x, T, k, d, inv_perm, (bf16 *)xs, job); \
+        else                                                                                                                  \
+            launch_kernel((dispatch_rows_kernel<float, NV>), grid, 256, 0, st, (const float *)x, T, k, d, inv_perm, (float *)xs, job); \
+    } while (0)
+    if (!sums) MOE_ROWS(0);
+    else if (sums->n <= 32) MOE_ROWS(1);
+    else if (sums->n <= 64) MOE_ROWS(2);
+    else if (sums->n <= 128) MOE_ROWS(4);
+    else if (sums->n <= LEVEL_RIDE_MAX) MOE_ROWS(8);
+    else return MOE_ERR_INVALID_ARG;
+#undef MOE_ROWS
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -561,16 +646,23 @@ __device__ __forceinline__ float logistic(float y) { return __fdividef(1.0f, 1.0
 
 // y[t] = sum_s gates[t,s] * ys[inv_perm[t*k+s]]   (Eq. 1), float sum in slot order.
 // LAYER (Appendix C): out[t] = x[t] + keep[t] * sigmoid(y[t]) * keep_scale, y itself is not stored.
+// sums.chunks > 0: the first blocks complete the loss sums, 32 columns each.
 template <typename XT, int KT, int VB, bool LAYER>
 __global__ void __launch_bounds__(256, LAYER ? 3 : 1) combine_kernel(const XT *__restrict__ ys, const float *__restrict__ gates,
                                                       const int32_t *__restrict__ inv_perm, int64_t T, int32_t k,
                                                       int32_t d, XT *__restrict__ y, const XT *__restrict__ xres,
-                                                      const uint8_t *__restrict__ keep, float keep_scale) {
+                                                      const uint8_t *__restrict__ keep, float keep_scale,
+                                                      const __grid_constant__ LevelSums sums) {
     wait_previous_kernel();
+    const int32_t reduces = sums.chunks > 0 ? (sums.n + 31) / 32 : 0;
+    if ((int32_t)blockIdx.x < reduces) {
+        level_reduce(sums, blockIdx.x);
+        return;
+    }
     constexpr int VN = 16 / sizeof(XT);
     const int lane = threadIdx.x & 31;
-    const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    const int64_t warp = (int64_t)(blockIdx.x - reduces) * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int64_t nwarps = (int64_t)(gridDim.x - reduces) * (blockDim.x >> 5);
     const int nvec = d / VN;
     for (int64_t t = warp; t < T; t += nwarps) {
         const uint4 *rowp[KT];
@@ -625,16 +717,17 @@ __global__ void __launch_bounds__(256, LAYER ? 3 : 1) combine_kernel(const XT *_
 
 int32_t launch_combine(const void *ys, int32_t act, const float *gates, const int32_t *inv_perm, int64_t T,
                        int32_t k, int32_t d, void *y, cudaStream_t st, const void *xres, const uint8_t *keep,
-                       float keep_scale) {
+                       float keep_scale, const LevelSums *sums) {
     if (T == 0) return MOE_OK;
-    const unsigned grid = (unsigned)imin(cdiv(T, 8), 148 * 16);
+    const LevelSums job = sums ? *sums : LevelSums{};
+    const unsigned grid = (unsigned)(imin(cdiv(T, 8), 148 * 16) + (sums ? cdiv(sums->n, 32) : 0));
 #define MOE_CALL_L(KT, VB, L)                                                                                         \
     if (act == MOE_BF16)                                                                                              \
         launch_kernel((combine_kernel<bf16, KT, VB, L>), grid, 256, 0, st, (const bf16 *)ys, gates, inv_perm, T, k, d, (bf16 *)y,  \
-                                                              (const bf16 *)xres, keep, keep_scale);                  \
+                                                              (const bf16 *)xres, keep, keep_scale, job);                  \
     else                                                                                                              \
         launch_kernel((combine_kernel<float, KT, VB, L>), grid, 256, 0, st, (const float *)ys, gates, inv_perm, T, k, d, (float *)y, \
-                                                               (const float *)xres, keep, keep_scale)
+                                                               (const float *)xres, keep, keep_scale, job)
 #define MOE_CALL(KT, VB)                     \
     if (keep) { MOE_CALL_L(KT, VB, true); }  \
     else { MOE_CALL_L(KT, VB, false); }
@@ -783,12 +876,14 @@ __global__ void __launch_bounds__(256) dispatch_bwd_kernel(const XT *__restrict_
                                                            const int32_t *__restrict__ inv_perm, int64_t T,
                                                            int32_t k, int32_t d, const float *add,
                                                            float *out_f32, XT *__restrict__ out_act,
-                                                           const XT *__restrict__ add_act, const SecondaryRows sec) {
+                                                           const XT *__restrict__ add_act, const SecondaryRows sec,
+                                                           const int32_t row_blocks, const __grid_constant__ BackwardTail tail) {
     wait_previous_kernel();
+    if ((int32_t)blockIdx.x >= row_blocks) return run_backward_tail(tail, blockIdx.x - row_blocks);
     constexpr int VN = 16 / sizeof(XT);
     const int lane = threadIdx.x & 31;
     const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    const int64_t nwarps = (int64_t)row_blocks * (blockDim.x >> 5);
     const int nvec = d / VN;
     for (int64_t t = warp; t < T; t += nwarps) {
         const uint4 *rowp[KT];
@@ -877,18 +972,30 @@ __global__ void __launch_bounds__(256) dispatch_bwd_kernel(const XT *__restrict_
     }
 }
 
+__global__ void __launch_bounds__(256) backward_tail_kernel(const __grid_constant__ BackwardTail tail) {
+    wait_previous_kernel();
+    run_backward_tail(tail, blockIdx.x);
+}
+
 int32_t launch_dispatch_bwd(const void *dxs, int32_t act, const int32_t *inv_perm, int64_t T, int32_t k,
                             int32_t d, const float *add_f32, float *out_f32, void *out_act, cudaStream_t st,
-                            const void *add_act, const SecondaryRows &sec) {
-    if (T == 0) return MOE_OK;
-    const unsigned grid = (unsigned)imin(cdiv(T, 8), 148 * 16);
+                            const void *add_act, const SecondaryRows &sec, const BackwardTail *tail_in) {
+    if (T == 0) return MOE_OK;  // (without rows nothing has been left)
+    BackwardTail tail = tail_in ? *tail_in : BackwardTail{};
+    if (tail.total() > TAIL_RIDE_MAX) {
+        launch_kernel(backward_tail_kernel, (unsigned)tail.total(), 256, 0, st, tail);
+        MOE_LAUNCHED();
+        tail = BackwardTail{};
+    }
+    const int32_t row_blocks = (int32_t)imin(cdiv(T, 8), 148 * 16);
+    const unsigned grid = (unsigned)(row_blocks + tail.total());
 #define MOE_CALL_S(KT, VB, SEC)                                                                                       \
     if (act == MOE_BF16)                                                                                              \
         launch_kernel((dispatch_bwd_kernel<bf16, KT, VB, SEC>), grid, 256, 0, st, (const bf16 *)dxs, inv_perm, T, k, d, add_f32, out_f32, \
-                                                                 (bf16 *)out_act, (const bf16 *)add_act, sec);         \
+                                                                 (bf16 *)out_act, (const bf16 *)add_act, sec, row_blocks, tail);         \
     else                                                                                                              \
         launch_kernel((dispatch_bwd_kernel<float, KT, VB, SEC>), grid, 256, 0, st, (const float *)dxs, inv_perm, T, k, d, add_f32,  \
-                                                                  out_f32, (float *)out_act, (const float *)add_act, sec)
+                                                                  out_f32, (float *)out_act, (const float *)add_act, sec, row_blocks, tail)
 #define MOE_CALL(KT, VB)                           \
     if (sec.rows) { MOE_CALL_S(KT, VB, true); }    \
     else { MOE_CALL_S(KT, VB, false); }
