@@ -601,6 +601,62 @@ template <int KIND> struct SegmentEnd {
     }
 };
 
+// The epilogue of an ACC tile (see grouped_gemm_kernel) by one warp: a lane's row of the warp's 128 columns, the running sums in registers.
+// row0: the warp's first output row; tfull0: the barriers of the two accumulators; release() hands the current one back.
+template <typename Release>
+__device__ __forceinline__ bool acc_tile(const GemmParams &p, const Tile &t, int lane, int quarter, int half, int64_t row0, uint8_t *slab,
+                                         uint32_t tmem_base, uint32_t tfull0, volatile int *abort_flag, int &acc, uint32_t &acc_ph,
+                                         Release release) {
+    float sums[4][32];
+#pragma unroll
+    for (int i = 0; i < 128; ++i) sums[i >> 5][i & 31] = 0.0f;
+    const int sub = t.e < p.segs_term0 ? p.sub_kb0 : p.sub_kb;
+    const int nsub = (t.kblocks + sub - 1) / sub;
+    const int columns = p.N - (t.n0 + half * 128);  // the warp's that exist (a multiple of 64); the others were not computed
+    for (int sb = 0; sb < nsub; ++sb) {
+        if (!mbar_wait(tfull0 + 8u * acc, acc_ph, abort_flag, p.status)) return false;
+        tc_fence_after();
+        // the accumulator goes back when it is read, before the last additions
+        auto drain = [&](auto count_) {
+            constexpr int COUNT = decltype(count_)::value;
+            if (COUNT == 0) release();
+#pragma unroll
+            for (int cl = 0; cl < COUNT; ++cl) {
+                uint32_t v[32];
+                tc_ld_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + (half * 4 + cl) * 32, v);
+                tc_ld_wait();
+                if (cl == COUNT - 1) release();
+#pragma unroll
+                for (int j = 0; j < 32; ++j) sums[cl][j] += __uint_as_float(v[j]);
+            }
+        };
+        if (columns >= 128) drain(std::integral_constant<int, 4>());
+        else if (columns > 0) drain(std::integral_constant<int, 2>());
+        else drain(std::integral_constant<int, 0>());
+        if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
+    }
+    // to global memory by way of the warp's 4 KiB: lane l moves piece l % 8 of row 4 * i + l / 8
+    float *dst = p.out_f32 + (int64_t)t.e * p.M * p.N + row0 * p.N + t.n0 + half * 128 + (lane & 7) * 4;
+#pragma unroll
+    for (int cl = 0; cl < 4; ++cl) {
+        if (t.n0 + half * 128 + cl * 32 >= p.N) break;
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            *reinterpret_cast<float4 *>(slab + lane * 128 + ((q ^ (lane & 7)) << 4)) =
+                make_float4(sums[cl][4 * q], sums[cl][4 * q + 1], sums[cl][4 * q + 2], sums[cl][4 * q + 3]);
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int row = 4 * i + (lane >> 3);
+            if (row0 + row < p.M)
+                *reinterpret_cast<float4 *>(dst + (int64_t)row * p.N + cl * 32) =
+                    *reinterpret_cast<const float4 *>(slab + row * 128 + (((lane & 7) ^ (row & 7)) << 4));
+        }
+        __syncwarp();
+    }
+    return true;
+}
+
 // ACC (WGRAD with float output over long uniform row ranges, the gate backward): the contraction of a tile is cut
 // into sub-blocks of p.sub_kb0 / p.sub_kb K blocks (first term / other terms). Each sub-block is accumulated in TMEM on
 // its own (an fp32 tensor-core accumulator truncates, and a long run of same-sign terms loses low bits: 128 rows keep
@@ -770,64 +826,14 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         while (ok && it.next(t)) {
             const bool have_acc = t.kblocks > 0;
             if constexpr (ACC) {
-                // a lane's row of the warp's 128 columns: the running sums stay in registers
-                const int half_a = (warp - 2) >> 2;
-                float sums[4][32];
-#pragma unroll
-                for (int i = 0; i < 128; ++i) sums[i >> 5][i & 31] = 0.0f;
-                const int sub = t.e < p.segs_term0 ? p.sub_kb0 : p.sub_kb;
-                const int nsub = (t.kblocks + sub - 1) / sub;
-                const int columns = p.N - (t.n0 + half_a * 128);  // the warp's that exist (a multiple of 64); the others were not computed
-                auto release_acc = [&]() {
+                auto release = [&]() {
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(tempty_bar(acc));
                 };
-                for (int sb = 0; sb < nsub; ++sb) {
-                    ok = mbar_wait(tfull_bar(acc), acc_ph, abort_flag, p.status);
-                    if (!ok) break;
-                    tc_fence_after();
-                    // the accumulator goes back when it is read, before the last additions
-                    auto drain = [&](auto count_) {
-                        constexpr int COUNT = decltype(count_)::value;
-                        if (COUNT == 0) release_acc();
-#pragma unroll
-                        for (int cl = 0; cl < COUNT; ++cl) {
-                            uint32_t v[32];
-                            tc_ld_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + (half_a * 4 + cl) * 32, v);
-                            tc_ld_wait();
-                            if (cl == COUNT - 1) release_acc();
-#pragma unroll
-                            for (int j = 0; j < 32; ++j) sums[cl][j] += __uint_as_float(v[j]);
-                        }
-                    };
-                    if (columns >= 128) drain(std::integral_constant<int, 4>());
-                    else if (columns > 0) drain(std::integral_constant<int, 2>());
-                    else drain(std::integral_constant<int, 0>());
-                    if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
-                }
+                ok = acc_tile(p, t, lane, quarter, (warp - 2) >> 2, (int64_t)t.m0 + quarter * 32, smem + NST * STAGE_BYTES + 1024 + (warp - 2) * 4096,
+                              tmem_base, bars + 8u * 2 * NST, abort_flag, acc, acc_ph, release);
                 if (!ok) break;
-                // to global memory by way of the warp's 4 KiB: lane l moves piece l % 8 of row 4 * i + l / 8
-                uint8_t *slab = smem + NST * STAGE_BYTES + 1024 + (warp - 2) * 4096;
-                const int64_t row0 = (int64_t)t.m0 + quarter * 32;
-                float *dst = p.out_f32 + (int64_t)t.e * p.M * p.N + row0 * p.N + t.n0 + half_a * 128 + (lane & 7) * 4;
-#pragma unroll
-                for (int cl = 0; cl < 4; ++cl) {
-                    if (t.n0 + half_a * 128 + cl * 32 >= p.N) break;
-#pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        *reinterpret_cast<float4 *>(slab + lane * 128 + ((q ^ (lane & 7)) << 4)) =
-                            make_float4(sums[cl][4 * q], sums[cl][4 * q + 1], sums[cl][4 * q + 2], sums[cl][4 * q + 3]);
-                    __syncwarp();
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const int row = 4 * i + (lane >> 3);
-                        if (row0 + row < p.M)
-                            *reinterpret_cast<float4 *>(dst + (int64_t)row * p.N + cl * 32) =
-                                *reinterpret_cast<const float4 *>(slab + row * 128 + (((lane & 7) ^ (row & 7)) << 4));
-                    }
-                    __syncwarp();
-                }
                 continue;
             }
             // Two warps share each quarter of the accumulator's rows and take half of its columns each, in boxes of 64.
@@ -1035,7 +1041,7 @@ template <int KIND> struct PairTiles {
 
 // MASKT: the ReLU mask of the dgrad GEMM is not read row by row from global memory by the epilogue but
 // fetched as a 128 x 256 tile by TMA (one stage fewer in exchange for the 64 KiB it occupies).
-template <int KIND, int EPI, bool MASKT>
+template <int KIND, int EPI, bool MASKT, bool ACC>
 __global__ void __launch_bounds__(NTHREADS2, 1)
 grouped_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                      const __grid_constant__ CUtensorMap tmM, const __grid_constant__ CUtensorMap tmO,
@@ -1177,12 +1183,14 @@ grouped_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                 ++trace_tile;
                 if (t.kblocks == 0) continue;  // empty segment (WGRAD): the epilogue writes zeros
                 TILE_TRACE_SET(1, trace_tile, 0, TILE_CLOCK());
+                const int sub = !ACC ? t.kblocks : t.e < p.segs_term0 ? p.sub_kb0 : p.sub_kb;  // K blocks per accumulator
+                int kin = 0;                                                                  // the block's place among them
                 ok = mbar_wait(tempty_bar(acc), acc_ph ^ 1u, abort_flag, p.status);
                 if (!ok) break;
                 tc_fence_after();
                 TILE_TRACE_SET(1, trace_tile, 1, TILE_CLOCK());
                 long long tr_wait = 0, tr_issue = 0;
-                const uint32_t d_tmem = tmem_base + acc * BN;
+                uint32_t d_tmem = tmem_base + acc * BN;
                 const int tail_valid = KIND == WGRAD ? (t.row_end - t.row0) - (t.kblocks - 1) * BK : BK;  // rows of the last block
                 for (int kb = 0; kb < t.kblocks; ++kb) {
                     const long long tw0 = TILE_CLOCK();
@@ -1201,8 +1209,18 @@ grouped_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                     const int ksteps = (KIND == WGRAD && kb == t.kblocks - 1) ? (tail_valid + 15) / 16 : BK / 16;
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k)
-                        if (k < ksteps) tc_mma2_bf16(d_tmem, ad0 + k * a_step, bd0 + k * b_step, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+                        if (k < ksteps) tc_mma2_bf16(d_tmem, ad0 + k * a_step, bd0 + k * b_step, idesc, (kin > 0 || k > 0) ? 1u : 0u);
                     tc_commit2(empty_bar(s));
+                    ++kin;
+                    if (ACC && kin == sub && kb + 1 < t.kblocks) {  // sub-block complete: the next one has the other accumulator
+                        tc_commit2(tfull_bar(acc));
+                        if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
+                        kin = 0;
+                        ok = mbar_wait(tempty_bar(acc), acc_ph ^ 1u, abort_flag, p.status);
+                        if (!ok) break;
+                        tc_fence_after();
+                        d_tmem = tmem_base + acc * BN;
+                    }
                     tr_issue += TILE_CLOCK() - ti0;
                     if (++s == NST) { s = 0; ph ^= 1u; }
                 }
@@ -1251,6 +1269,17 @@ grouped_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
             const bool have_acc = t.kblocks > 0;
             ++trace_tile;
             if (warp == 2 && lane == 0) TILE_TRACE_SET(2, trace_tile, 0, TILE_CLOCK());
+            if constexpr (ACC) {
+                auto release = [&]() {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_leader_relaxed(tempty_bar(acc));
+                };
+                ok = acc_tile(p, t, lane, quarter, half, (int64_t)t.m0 + 128 * (int)rank + quarter * 32, smem + NST * STAGE2_BYTES + (warp - 2) * 4096,
+                              tmem_base, bars + 8u * 2 * NST, abort_flag, acc, acc_ph, release);
+                if (!ok) break;
+                continue;
+            }
             const int32_t first = t.n0 + half * (BN / 2);
             const int boxes = min(2, max(0, (p.N - first) / 64));  // N is a multiple of 64
             BoxArgs b;
@@ -1478,7 +1507,7 @@ int32_t launch_acc_wgrad(const CUtensorMap &tmA, const CUtensorMap &tmB, const G
     return MOE_OK;
 }
 
-template <int KIND, int EPI, bool MASKT = false>
+template <int KIND, int EPI, bool MASKT = false, bool ACC = false>
 int32_t launch2_as(const CUtensorMap &tmA, const CUtensorMap &tmB, const GemmParams &p_in, int64_t max_tiles,
                    cudaStream_t st, const CUtensorMap *tmM, const CUtensorMap *tmO) {
     GemmParams p = p_in;
@@ -1495,10 +1524,10 @@ int32_t launch2_as(const CUtensorMap &tmA, const CUtensorMap &tmB, const GemmPar
     cfg.blockDim = dim3(NTHREADS2); cfg.dynamicSmemBytes = SMEM2_BYTES; cfg.stream = st;
     cfg.attrs = attrs; cfg.numAttrs = 2;
     if (!max_clusters) {
-        MOE_CUDA(cudaFuncSetAttribute((grouped_gemm2_kernel<KIND, EPI, MASKT>), cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM2_BYTES));
+        MOE_CUDA(cudaFuncSetAttribute((grouped_gemm2_kernel<KIND, EPI, MASKT, ACC>), cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM2_BYTES));
         cfg.gridDim = dim3(2 * (sm_count() / 2));
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, (grouped_gemm2_kernel<KIND, EPI, MASKT>), &cfg) != cudaSuccess || n <= 0) return MOE_ERR_CUDA;
+        if (cudaOccupancyMaxActiveClusters(&n, (grouped_gemm2_kernel<KIND, EPI, MASKT, ACC>), &cfg) != cudaSuccess || n <= 0) return MOE_ERR_CUDA;
         max_clusters = n;
     }
     if (max_tiles <= 0) return MOE_OK;
@@ -1510,7 +1539,7 @@ int32_t launch2_as(const CUtensorMap &tmA, const CUtensorMap &tmB, const GemmPar
     }
 #endif
     cfg.gridDim = dim3(2 * (unsigned)imin(max_tiles, max_clusters));
-    MOE_CUDA(cudaLaunchKernelEx(&cfg, (grouped_gemm2_kernel<KIND, EPI, MASKT>), tmA, tmB, tmM ? *tmM : tmA, tmO ? *tmO : tmA, p));
+    MOE_CUDA(cudaLaunchKernelEx(&cfg, (grouped_gemm2_kernel<KIND, EPI, MASKT, ACC>), tmA, tmB, tmM ? *tmM : tmA, tmO ? *tmO : tmA, p));
     MOE_LAUNCHED();
     return MOE_OK;
 }
@@ -1814,22 +1843,32 @@ bool tc_gate_bwd_supported(int32_t act, int32_t d, int32_t n) {
 // term, added in double afterwards), and inside a range the tensor-core accumulator is restarted every GB_ROWS_HI rows
 // for the leading (hi) term: an fp32 accumulator loses low bits when a long run of same-sign terms is added (e.g. the
 // gradient of a constant input feature); 128 rows keep that below 1e-5 of the result. The mid and lo terms are 2^-8
-// and 2^-16 of the hi term and restart every GB_ROWS_LO rows. The restarts' sums are added in registers (see the
-// ACC kernel), so only one partial per range goes to global memory. Ranges are whole lo sub-blocks, shorter ones where the batch
-// leaves fewer than two tiles per SM (8192 tokens, 512 features x 64 columns: 48 tiles, 24 us).
-constexpr int GB_ROWS_HI = 128, GB_ROWS_LO = 2048, GB_ROWS_LEAST = 256;
+// and 2^-16 of the hi term and restart every GB_ROWS_LO rows. The restarts' sums are added in registers (see acc_tile), so only one
+// partial per range goes to global memory.
+// SM pairs where a tile of theirs is full: on one CTA a 64-row K block brings 48 KiB to an SM for 512 cycles of tensor work, which the L2
+// does not deliver (32768 tokens, 512 x 512: 91 us, on pairs 73; 131072, 1024 x 256: 383, 271).
+// Ranges: whole waves of tiles. A tile costs its K blocks and about eight more for its 128 KiB of sums, read again later at the copy
+// rate; no longer than GB_ROWS_MOST rows unless there are more than three waves of the leading term's tiles.
+constexpr int GB_ROWS_HI = 128, GB_ROWS_LO = 2048, GB_ROWS_LEAST = 256, GB_ROWS_MOST = 4096;
+static bool gate_bwd_pairs(int32_t d, int32_t n) { return d >= 256 && 2 * n >= 256; }
 static void gate_bwd_split(int64_t T, int32_t d, int32_t n, int32_t *nranges, int32_t *rows, int32_t *rows_lo) {
-    const int64_t tiles_per_range = cdiv(d, BM) * cdiv(2 * n, BN);
-    int64_t lo = GB_ROWS_LO;
-    while (lo > GB_ROWS_LEAST && 3 * tiles_per_range * cdiv(T, lo) < 2 * (int64_t)sm_count()) lo /= 2;
-    int64_t want = cdiv(3 * (int64_t)sm_count(), tiles_per_range);  // about three waves of hi-term tiles
-    const int64_t most = T > 0 ? cdiv(T, lo) : 1;
-    if (want > most) want = most;
-    if (want < 1) want = 1;
-    const int64_t r = cdiv(cdiv(T > 0 ? T : 1, want), lo) * lo;  // whole lo sub-blocks per range
-    *rows_lo = (int32_t)lo;
-    *rows = (int32_t)r;
-    *nranges = (int32_t)(T > 0 ? cdiv(T, r) : 1);
+    const bool pairs = gate_bwd_pairs(d, n);
+    const int64_t tiles = 3 * cdiv(d, pairs ? 256 : BM) * cdiv(2 * n, BN), workers = pairs ? sm_count() / 2 : sm_count();
+    const int64_t most = cdiv(9 * workers, tiles);
+    const int64_t rows_most = imax(GB_ROWS_MOST, cdiv(cdiv(T, most), GB_ROWS_HI) * GB_ROWS_HI);
+    double least = 0.0;
+    for (int64_t w = 1; w <= 9; ++w) {
+        const int64_t ranges = imax(1, w * workers / tiles);
+        const int64_t r = imin(rows_most, imax(GB_ROWS_LEAST, cdiv(cdiv(T, ranges), GB_ROWS_HI) * GB_ROWS_HI));
+        const int64_t made = T > 0 ? cdiv(T, r) : 1, waves = cdiv(made * tiles, workers);
+        const double cost = (double)waves * (r / BK + 8) + 12.0 * made * d * 2 * n / 2.2e6;  // K blocks; 2.2 MB are read in the time of one
+        if (w == 1 || cost < least) {
+            least = cost;
+            *rows = (int32_t)r;
+            *rows_lo = (int32_t)imin(r, GB_ROWS_LO);
+            *nranges = (int32_t)made;
+        }
+    }
 }
 
 int64_t tc_gate_bwd_partials(int64_t T, int32_t d, int32_t n) {
@@ -1857,14 +1896,16 @@ int32_t launch_tc_gate_bwd(const void *x, int64_t T, int32_t d, int32_t n, const
     gate_bwd_split(T, d, n, &nr, &rows, &rows_lo);
     {   // dW partials: contraction over the tokens, cut into row ranges, one set per precision term
         CUtensorMap tmA, tmB;
+        const bool pairs = gate_bwd_pairs(d, n) && !(flags & MOE_FLAG_TC_ONE_CTA);
         MOE_TRY(map_rows_mnmajor(&tmA, x, T, d, BM / 64));
-        MOE_TRY(map_rows_mnmajor(&tmB, dsplit, T, 3 * n2, BN / 64));
+        MOE_TRY(map_rows_mnmajor(&tmB, dsplit, T, 3 * n2, (pairs ? 128 : BN) / 64));
         GemmParams p = default_params();
         p.nseg = 3 * nr; p.M = d; p.N = n2; p.R = T; p.out_f32 = partials; p.status = status;
         p.segs_term0 = nr; p.rows_per_seg0 = rows;
         p.rows_per_seg = rows; p.segs_per_term = nr; p.b_term_chunks = n2 / 64;
         p.sub_kb0 = GB_ROWS_HI / BK; p.sub_kb = rows_lo / BK; p.interleave = 3;
-        MOE_TRY(launch_acc_wgrad(tmA, tmB, p, (int64_t)p.nseg * cdiv(d, BM) * cdiv(n2, BN), st));
+        if (pairs) MOE_TRY((launch2_as<WGRAD, EPI_F32, false, true>(tmA, tmB, p, (int64_t)p.nseg * cdiv(d, 256) * cdiv(n2, BN), st, nullptr, nullptr)));
+        else MOE_TRY(launch_acc_wgrad(tmA, tmB, p, (int64_t)p.nseg * cdiv(d, BM) * cdiv(n2, BN), st));
         const GateParts parts = {partials, 3 * nr, d, n2, n, ldw > 0 ? ldw : n, dWg, dWn};
         if (parts_left) {
             *parts_left = parts;
