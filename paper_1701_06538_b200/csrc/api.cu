@@ -197,7 +197,7 @@ struct DispatchWs {
 SegmentPlan make_plan(const moe_config *c, const Dims &D, int32_t *ws, bool backward) {
     SegmentPlan p = plan_at(ws, D.R, D.n);
     if (tc_ffn_supported(*c)) {
-        p.bm[0] = tc_row_tile(D.R, (int32_t)D.n, D.flags);
+        p.bm[0] = tc_row_tile(D.R, (int32_t)D.n, D.flags, (int32_t)(D.d > D.h ? D.d : D.h));
         if (backward && p.bm[0] != COLSUM_ROWS) p.bm[1] = COLSUM_ROWS;
         if (!backward || !tc_wgrad_sorted(*c)) p.sched = nullptr;
     } else {

@@ -1569,9 +1569,12 @@ bool tc_ffn_supported(const moe_config &c) {
 }
 
 
-// The 256-row tiles of the two-CTA kernel pay off when the average segment fills them.
-static bool use_two_cta(int64_t R, int32_t nseg, int32_t flags) {
-    if (flags & MOE_FLAG_TC_ONE_CTA) return false;
+// The two-CTA kernel's 256 x 256 tiles pay off when the average segment fills them and there are more of them than SMs (cols: the wider
+// side of an expert's matrices). A step with all its products on pairs / on one CTA each, us: 4000 rows x 1024 columns
+// (64 tiles) 131 / 119, 8000 x 1024 (128) 155 / 152, 9000 x 832 (144) 171 / 166, but 6000 x 2048 (192) 244 / 255, 16384 x 1024 (256)
+// 242 / 244, 32000 x 1024 399 / 421.
+static bool use_two_cta(int64_t R, int32_t nseg, int32_t flags, int32_t cols) {
+    if ((flags & MOE_FLAG_TC_ONE_CTA) || cdiv(R, 256) * cdiv(cols, 256) <= sm_count()) return false;
     return R / (nseg > 0 ? nseg : 1) >= 384;
 }
 
@@ -1585,7 +1588,7 @@ int32_t tc_segment_maps(const moe_config &c, SegmentMaps *maps, const void *xs_r
         return chunks ? map_rows_mnmajor(&maps->base[which], p, rows, cols, chunks) : map_rows_kmajor(&maps->base[which], p, rows, cols);
     };
     // boxes as in tc_row_gemm and tc_wgrad_gemm
-    const bool two = use_two_cta(R, c.n, c.flags);
+    const bool two = use_two_cta(R, c.n, c.flags, c.d > c.h ? c.d : c.h);
     const int b2 = two && c.h >= 256 ? 2 : BN / 64, b1 = two && c.d >= 256 ? 2 : BN / 64;
     MOE_TRY(add(MAP_XS_ROWS, xs_rows, c.d, 0));
     MOE_TRY(add(MAP_HID_ROWS, hid_rows, c.h, 0));
@@ -1709,7 +1712,7 @@ int32_t tc_row_gemm(const void *A, const void *W, bool transposed, const int32_t
     p.bits_out = bits_out; p.bits_in = bits_in;
     if (bits_in) p.mask = nullptr;  // the bits replace the element-wise mask tensor
     p.colsum_part = colsum_out ? colsum_part : nullptr;
-    if (use_two_cta(R, nseg, flags)) {  // segments long enough to fill 256-row tiles: SM pairs
+    if (use_two_cta(R, nseg, flags, N > K ? N : K)) {  // segments long enough to fill 256-row tiles: SM pairs
         if (transposed) MOE_TRY(map_weight_kmajor_half(&tmB, W, nseg, N, K));
         else MOE_TRY(map_weight_mnmajor_half(&tmB, W, nseg, K, N));
         p.sched_counter = plan.counters + counter;  // tiles handed out at run time
@@ -1753,7 +1756,7 @@ int32_t tc_wgrad_gemm(const void *A, const void *B, const int32_t *offsets, int3
     p.out = (bf16 *)out; p.status = status;
     CUtensorMap tmO;  // the experts' matrices as one tall matrix (a 32-row box never straddles two: M is a multiple of 64)
     MOE_TRY(map_out_boxes(&tmO, out, (int64_t)nseg * M, N));
-    if (use_two_cta(R, nseg, flags) && M >= 256) {  // SM pairs: 256 x 256 tiles, each CTA stages half of A and half of B
+    if (use_two_cta(R, nseg, flags, M > N ? M : N) && M >= 256) {  // SM pairs: 256 x 256 tiles, each CTA stages half of A and half of B
         MOE_TRY(map_rows_mnmajor(&tmA, A, R > 0 ? R : 1, M, 2));
         MOE_TRY(map_rows_mnmajor(&tmB, B, R > 0 ? R : 1, N, 2));
         if (plan.sched) {
@@ -1768,9 +1771,9 @@ int32_t tc_wgrad_gemm(const void *A, const void *B, const int32_t *offsets, int3
     return launch<WGRAD>(tmA, tmB, p, (int64_t)nseg * cdiv(M, BM) * cdiv(N, BN), st, &tmO);
 }
 
-int32_t tc_row_tile(int64_t R, int32_t nseg, int32_t flags) { return use_two_cta(R, nseg, flags) ? 256 : BM; }
+int32_t tc_row_tile(int64_t R, int32_t nseg, int32_t flags, int32_t cols) { return use_two_cta(R, nseg, flags, cols) ? 256 : BM; }
 bool tc_wgrad_sorted(const moe_config &c) {
-    return use_two_cta((int64_t)c.T * c.k, c.n, c.flags) && c.n > 1 && c.n <= PLAN_MAX_SORTED;
+    return use_two_cta((int64_t)c.T * c.k, c.n, c.flags, c.d > c.h ? c.d : c.h) && c.n > 1 && c.n <= PLAN_MAX_SORTED;
 }
 
 int32_t launch_tc_ffn(const moe_config &c, const void *xs, const int32_t *offsets, const void *W1, const void *b1,
@@ -1967,7 +1970,7 @@ int32_t launch_tc_gate_fwd_grouped(const void *xs_p, int64_t P1, int32_t d, int3
                                    int32_t *status, cudaStream_t st, int32_t flags) {
     if (P1 == 0) return MOE_OK;
     const int32_t n2 = 2 * b;
-    const bool pairs = use_two_cta(P1, a, flags);
+    const bool pairs = use_two_cta(P1, a, flags, n2 > d ? n2 : d);
     CUtensorMap tmA, tmB;
     MOE_TRY(map_rows_kmajor(&tmA, xs_p, P1, d));
     {   // the group is the map's last coordinate (stride d rows), the precision term an offset of a * d rows along K

@@ -410,7 +410,7 @@ bool tc_ffn_supported(const moe_config &c);
 // base maps of the operands that are given (nullptr: not wanted)
 int32_t tc_segment_maps(const moe_config &c, SegmentMaps *maps, const void *xs_rows, const void *hid_rows, const void *dys_rows,
                         const void *dz_rows, const void *hid_cols, const void *dys_cols, const void *xs_cols, const void *dz_cols);
-int32_t tc_row_tile(int64_t R, int32_t nseg, int32_t flags);  // tile height of the row GEMMs: what plan.bm[0] has to be
+int32_t tc_row_tile(int64_t R, int32_t nseg, int32_t flags, int32_t cols);  // tile height of the row GEMMs: what plan.bm[0] has to be
 bool tc_wgrad_sorted(const moe_config &c);                    // the weight gradients want plan.sched
 // first_only: only hid = relu(xs.W1 + b1) (the recomputation of the hidden activations in the backward pass)
 int32_t launch_tc_ffn(const moe_config &c, const void *xs, const int32_t *offsets, const void *W1, const void *b1,
