@@ -148,8 +148,9 @@ __global__ void __launch_bounds__(256) gate_logit_grads_kernel(
 
 // The same for the tensor-core path (split output, n a multiple of 32): a lane owns PAIRS of adjacent columns, so the
 // row is read with 8-byte loads and the six bf16 terms of a pair leave as 4-byte stores (half the memory instructions),
-// and only the first KS slots are compared (KS >= k).
-template <int NVP, int KS>  // column pairs per lane (n <= 64 * NVP)
+// and only the first KS slots are compared (KS >= k). LANES lanes take a row, NVP pairs each: what a row costs besides its columns
+// (its slots' gates, two sums over its lanes) is most of a row of 64 when a warp has one row.
+template <int LANES, int NVP, int KS>  // n <= 2 * LANES * NVP
 __global__ void __launch_bounds__(256) gate_logit_grads_pairs_kernel(
     const float *__restrict__ noise, const float *__restrict__ clean, const float *__restrict__ raw,
     const int32_t *__restrict__ idx, const float *__restrict__ gates, const float *__restrict__ kth_vals,
@@ -158,9 +159,10 @@ __global__ void __launch_bounds__(256) gate_logit_grads_pairs_kernel(
     const int32_t *__restrict__ split_row_index, const __grid_constant__ Beside beside) {
     wait_previous_kernel();
     if ((int32_t)blockIdx.x < beside.blocks) return beside.run(blockIdx.x);
-    const int lane = threadIdx.x & 31;
-    const int64_t row = (int64_t)(blockIdx.x - beside.blocks) * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (row >= rows) return;
+    const int lane = threadIdx.x & (LANES - 1);
+    const int64_t place = (int64_t)(blockIdx.x - beside.blocks) * (256 / LANES) + threadIdx.x / LANES;
+    const bool live = place < rows;
+    const int64_t row = live ? place : rows - 1;  // (the lanes behind the last row stay for the sums over a warp's lanes)
     int32_t sel_idx[KS];
     float sel_dh[KS];
     float inner = 0.0f;
@@ -180,7 +182,7 @@ __global__ void __launch_bounds__(256) gate_logit_grads_pairs_kernel(
     float dhv[2 * NVP], qv[2 * NVP], zqv[2 * NVP];
 #pragma unroll
     for (int u = 0; u < NVP; ++u) {  // all loads of the row first
-        const int32_t j = 2 * lane + 64 * u;
+        const int32_t j = 2 * lane + 2 * LANES * u;
         const bool in = j < n;
         const float2 z2 = make_float2(0.0f, 0.0f);
         cv[u] = in ? *reinterpret_cast<const float2 *>(c + j) : z2;
@@ -191,7 +193,7 @@ __global__ void __launch_bounds__(256) gate_logit_grads_pairs_kernel(
     float q_sel = 0.0f, q_uns = 0.0f;
 #pragma unroll
     for (int u = 0; u < 2 * NVP; ++u) {
-        const int32_t j = 2 * lane + 64 * (u >> 1) + (u & 1);
+        const int32_t j = 2 * lane + 2 * LANES * (u >> 1) + (u & 1);
         const float cj = (u & 1) ? cv[u >> 1].y : cv[u >> 1].x, rj = (u & 1) ? rv[u >> 1].y : rv[u >> 1].x;
         const float dlj = (u & 1) ? dv[u >> 1].y : dv[u >> 1].x;
         dhv[u] = qv[u] = zqv[u] = 0.0f;
@@ -213,15 +215,16 @@ __global__ void __launch_bounds__(256) gate_logit_grads_pairs_kernel(
         }
     }
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
+    for (int off = LANES / 2; off > 0; off >>= 1) {
         q_sel += __shfl_xor_sync(0xffffffffu, q_sel, off);
         q_uns += __shfl_xor_sync(0xffffffffu, q_uns, off);
     }
+    if (!live) return;
     const int64_t orow = split_row_index ? split_row_index[row] : row;  // e.g. sorted by primary group
     bf16 *o = dsplit + orow * (6 * (int64_t)n);
 #pragma unroll
     for (int u = 0; u < NVP; ++u) {
-        const int32_t j = 2 * lane + 64 * u;
+        const int32_t j = 2 * lane + 2 * LANES * u;
         if (j >= n) continue;
         float dc[2], dr[2];
 #pragma unroll
@@ -256,19 +259,27 @@ int32_t launch_gate_logit_grads(const float *noise, const float *clean, const fl
     if (sums) beside = {*sums, (int32_t)(column_tiles(*sums) * column_slabs(*sums)), (int32_t)column_slabs(*sums)};
     const unsigned grid = (unsigned)(cdiv(rows, 8) + beside.blocks);
     if (dsplit && n % 32 == 0 && n <= 256) {  // the tensor-core path: paired columns
-#define MOE_LOGIT_PAIRS_KS(NVP, KS)                                                                                      \
-    launch_kernel((gate_logit_grads_pairs_kernel<NVP, KS>), grid, 256, 0, st, noise, clean, raw, idx, gates, kth_vals, kth_idx, dgates, \
-                                                                 dload, dload_row_group, rows, n, k, (bf16 *)dsplit,      \
-                                                                 split_row_index, beside)
-#define MOE_LOGIT_PAIRS(NVP)                                \
+#define MOE_LOGIT_PAIRS_KS(LANES, NVP, KS)                                                                               \
+    launch_kernel((gate_logit_grads_pairs_kernel<LANES, NVP, KS>), (unsigned)(cdiv(rows, 256 / LANES) + beside.blocks), 256, 0, st, \
+                  noise, clean, raw, idx, gates, kth_vals, kth_idx, dgates, dload, dload_row_group, rows, n, k, (bf16 *)dsplit,      \
+                  split_row_index, beside)
+#define MOE_LOGIT_PAIRS(LANES, NVP)                         \
     do {                                                    \
-        if (k <= 2) MOE_LOGIT_PAIRS_KS(NVP, 2);             \
-        else if (k <= 4) MOE_LOGIT_PAIRS_KS(NVP, 4);        \
-        else MOE_LOGIT_PAIRS_KS(NVP, MOE_MAX_K);            \
+        if (k <= 2) MOE_LOGIT_PAIRS_KS(LANES, NVP, 2);      \
+        else if (k <= 4) MOE_LOGIT_PAIRS_KS(LANES, NVP, 4); \
+        else MOE_LOGIT_PAIRS_KS(LANES, NVP, MOE_MAX_K);     \
     } while (0)
-        if (n <= 64) MOE_LOGIT_PAIRS(1);
-        else if (n <= 128) MOE_LOGIT_PAIRS(2);
-        else MOE_LOGIT_PAIRS(4);
+        // four pairs a lane where that still leaves every SM four blocks of 32 or 16 rows
+        const bool many = rows >= (n <= 64 ? 32 : 16) * 4 * (int64_t)148;
+        if (n <= 64) {
+            if (many) MOE_LOGIT_PAIRS(8, 4);
+            else MOE_LOGIT_PAIRS(32, 1);
+        } else if (n <= 128) {
+            if (many) MOE_LOGIT_PAIRS(16, 4);
+            else MOE_LOGIT_PAIRS(32, 2);
+        } else {
+            MOE_LOGIT_PAIRS(32, 4);
+        }
 #undef MOE_LOGIT_PAIRS
 #undef MOE_LOGIT_PAIRS_KS
         MOE_LAUNCHED();
