@@ -56,12 +56,30 @@ enum Epilogue { EPI_PLAIN = 0, EPI_BIAS = 1, EPI_RELU = 2, EPI_MASK = 4, EPI_BIT
 
 constexpr int MAX_TERMS = 8;
 
+// Division by a launch's constant as a multiplication (Granlund and Montgomery, 1994): q = (high word of x * m + x) >> s for
+// 0 <= x < 2^31. A tile's place is three divisions, which every warp role makes between two tiles: as integer divisions they and the
+// look-up behind them were 700 of a 3700-cycle tile of 64 rows.
+struct Divisor {
+    uint32_t d, m, s;
+    static Divisor of(int64_t by) {
+        Divisor v = {(uint32_t)(by > 0 ? by : 1), 0, 0};
+        while ((1ull << v.s) < v.d) ++v.s;
+        v.m = (uint32_t)((((1ull << v.s) - v.d) << 32) / v.d + 1);
+        return v;
+    }
+    __device__ __forceinline__ int32_t operator()(int32_t x, int32_t &rest) const {
+        const int32_t q = (int32_t)((__umulhi((uint32_t)x, m) + (uint32_t)x) >> s);
+        rest = x - q * (int32_t)d;
+        return q;
+    }
+};
 struct GemmParams {
     const int32_t *offsets;      // [nseg + 1] segment bounds (rows); nullptr = uniform segments
     const int32_t *tile_prefix;  // ROW_* with offsets: [nseg + 1] prefix of the M tiles
     const int4 *tile_info;       // ROW_* with offsets: per M tile {segment or -1, first row, segment end, 0}
     // set by the launchers: N tiles per row of tiles, WGRAD tiles per segment, number of tile ids, K blocks of a ROW tile
     int32_t tiles_n, per_e, total_tiles, kblocks_row;
+    Divisor by_tiles_n, by_per_e, by_mod, by_terms, by_interleave, by_group;  // tiles_n, per_e, off_mod, segs_per_term, interleave, sched_group
     int32_t tile_n;  // columns of a tile: BN, or 128 in row products of the one-CTA kernel (see tc_row_gemm)
     int32_t nseg;
     int32_t M;  // WGRAD: rows of the per-segment output; ROW_*: unused
@@ -503,41 +521,50 @@ template <int KIND>
 __device__ __forceinline__ int4 tile_fetch(const GemmParams &p, int32_t id) {
     if (!p.offsets || id >= p.total_tiles) return make_int4(-1, 0, 0, 0);
     if (KIND == WGRAD) {
-        const int32_t e = id / p.per_e;
-        const int32_t seg = p.off_mod > 0 ? e % p.off_mod : e;  // with off_mod: segment s reads the rows of group s % off_mod
+        int32_t rest, seg;
+        const int32_t e = p.by_per_e(id, rest);
+        if (p.off_mod > 0) p.by_mod(e, seg);  // segment s reads the rows of group s % off_mod
+        else seg = e;
         return make_int4(e, p.offsets[seg], p.offsets[seg + 1], 0);
     }
-    return p.tile_info[id / p.tiles_n];
+    int32_t rest;
+    return p.tile_info[p.by_tiles_n(id, rest)];
 }
 
 template <int KIND, int TM>
 __device__ __forceinline__ bool tile_decode(const GemmParams &p, int32_t id, const int4 &raw, Tile &t) {
     if (id >= p.total_tiles) return false;
     if (KIND == WGRAD) {
-        int32_t e = id / p.per_e;
-        const int32_t rem = id - e * p.per_e;
+        int32_t rem, tn;
+        int32_t e = p.by_per_e(id, rem);
         // uniform ranges, interleaved terms: consecutive ids walk the terms of one row range (its rows stay in L2 for all
         // of them) while the segment index stays term-major
-        if (p.interleave > 1) e = (e % p.interleave) * p.segs_per_term + e / p.interleave;
-        const int32_t tm = rem / p.tiles_n;
+        if (p.interleave > 1) {
+            int32_t term;
+            const int32_t range = p.by_interleave(e, term);
+            e = term * p.segs_per_term + range;
+        }
+        const int32_t tm = p.by_tiles_n(rem, tn);
         t.e = e;
         t.mt = 0;
         t.m0 = tm * TM;
-        t.n0 = (rem - tm * p.tiles_n) * p.tile_n;
+        t.n0 = tn * p.tile_n;
         t.b_chunk = t.n0 / 64;
         if (p.offsets) {
             t.row0 = raw.y;
             t.row_end = raw.z;
-            if (p.off_mod > 0) t.b_chunk += (e / p.off_mod) * p.b_term_chunks;  // B term s / off_mod
+            if (p.off_mod > 0) {
+                int32_t group;
+                t.b_chunk += p.by_mod(e, group) * p.b_term_chunks;  // B term s / off_mod
+            }
         } else {
-            int64_t c, rps;
-            int32_t term;
+            int64_t rps;
+            int32_t c, term;
             if (e < p.segs_term0) {  // term 0 may use its own (shorter) row ranges
                 c = e; rps = p.rows_per_seg0; term = 0;
             } else {
-                const int32_t e2 = e - p.segs_term0;
-                c = e2 % p.segs_per_term; rps = p.rows_per_seg;
-                term = e2 / p.segs_per_term + (p.segs_term0 > 0 ? 1 : 0);
+                term = p.by_terms(e - p.segs_term0, c) + (p.segs_term0 > 0 ? 1 : 0);
+                rps = p.rows_per_seg;
             }
             t.row0 = (int32_t)(c * rps);
             t.row_end = (int32_t)(((c + 1) * rps < p.R) ? (c + 1) * rps : p.R);
@@ -547,12 +574,13 @@ __device__ __forceinline__ bool tile_decode(const GemmParams &p, int32_t id, con
         t.kblocks = (t.row_end - t.row0 + BK - 1) / BK;
         return true;
     } else {
-        const int32_t mt = id / p.tiles_n;
+        int32_t tn;
+        const int32_t mt = p.by_tiles_n(id, tn);
         t.mt = mt;
         t.m0 = 0;
         t.b_chunk = 0;
         t.kblocks = p.kblocks_row;
-        t.n0 = (id - mt * p.tiles_n) * p.tile_n;
+        t.n0 = tn * p.tile_n;
         if (!p.offsets) {  // one segment of R rows; total_tiles is exact
             t.e = 0;
             t.row0 = mt * TM;
@@ -755,8 +783,9 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             const uint32_t idesc = make_idesc(KIND == WGRAD ? 1 : 0, KIND == ROW_BK ? 0 : 1, min(p.tile_n, p.N - t.n0));
             const int sub = ACC ? (t.e < p.segs_term0 ? p.sub_kb0 : p.sub_kb) : t.kblocks;  // K blocks per accumulator
             uint32_t d_tmem = tmem_base + acc * BN;
-            for (int kb = 0; kb < t.kblocks; ++kb) {
-                const int kin = ACC ? kb % sub : kb;  // K block inside the accumulator's sub-block
+            int kin = 0;  // K block inside the accumulator's sub-block
+            for (int kb = 0; kb < t.kblocks; ++kb, ++kin) {
+                if (ACC && kin == sub) kin = 0;
                 if (kin == 0) {
                     ok = mbar_wait(tempty_bar(acc), acc_ph ^ 1u, abort_flag, p.status);
                     if (!ok) break;
@@ -777,13 +806,13 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                     // non-finite value of the next segment out of this segment's sums): 128-B lines in all 64-column
                     // chunks, the A tile's two chunks directly followed by the B tile's four.
                     if (p.offsets && !p.seg_a && nz > 0) {
-                        const int lines = nz * ((BM + BN) / 64);
-                        for (int u = lane; u < lines * 8; u += 32) {
-                            const int line = u >> 3, part = u & 7;
-                            const int chunk = line / nz, krow = valid + line % nz;
-                            *reinterpret_cast<uint4 *>(smem + s * STAGE_BYTES + chunk * (BK * 128) + krow * 128 + part * 16) =
-                                make_uint4(0, 0, 0, 0);
-                        }
+                        // eight lanes a line of one chunk, four lines at a time (as one loop over all lines, with a division for
+                        // each, this was 1450 cycles a tile of 64 rows)
+                        uint8_t *z = smem + s * STAGE_BYTES + (valid + (lane >> 3)) * 128 + (lane & 7) * 16;
+                        for (int r = lane >> 3; r < nz; r += 4, z += 4 * 128)
+#pragma unroll
+                            for (int chunk = 0; chunk < (BM + BN) / 64; ++chunk)
+                                *reinterpret_cast<uint4 *>(z + chunk * (BK * 128)) = make_uint4(0, 0, 0, 0);
                         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                         __syncwarp();
                     }
@@ -1020,12 +1049,13 @@ template <int KIND> struct PairTiles {
         if (rec.x < 0) return false;
         MOE_BOUNDS_NOTE(rec.x < p.nseg && rec.y >= 0 && rec.y <= rec.z && (int64_t)rec.z <= p.R);
         t.e = rec.x; t.row0 = rec.y; t.row_end = rec.z;
-        const int32_t grp = rec.w / p.sched_group, rem = rec.w - grp * p.sched_group;  // rec.w: the tile id
+        int32_t rem, tn;
+        const int32_t grp = p.by_group(rec.w, rem);  // rec.w: the tile id
         if (KIND == WGRAD) {
-            const int32_t tm = rem / p.tiles_n;
+            const int32_t tm = p.by_tiles_n(rem, tn);
             t.mt = 0;
             t.m0 = tm * 256;
-            t.n0 = (rem - tm * p.tiles_n) * BN;
+            t.n0 = tn * BN;
             t.b_chunk = t.n0 / 64;
             t.kblocks = (t.row_end - t.row0 + BK - 1) / BK;
         } else {
@@ -1245,7 +1275,8 @@ grouped_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                 const int32_t id = atomicAdd(p.sched_counter, 1);
                 int4 rec = make_int4(-1, 0, 0, 0);
                 if (id < p.total_tiles) {
-                    rec = p.sched_table[id / p.sched_group];
+                    int32_t rest;
+                    rec = p.sched_table[p.by_group(id, rest)];
                     rec.w = id;
                 }
                 asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(sched_ring + 16u * slot), "r"(rec.x), "r"(rec.y), "r"(rec.z), "r"(rec.w) : "memory");
@@ -1454,6 +1485,8 @@ template <int KIND, int TM> int32_t complete_params(GemmParams &q, int64_t max_t
     q.tiles_n = (int32_t)cdiv(q.N, q.tile_n);
     q.per_e = KIND == WGRAD ? (int32_t)cdiv(q.M, TM) * q.tiles_n : 1;
     q.total_tiles = (int32_t)max_tiles;
+    q.by_tiles_n = Divisor::of(q.tiles_n); q.by_per_e = Divisor::of(q.per_e); q.by_mod = Divisor::of(q.off_mod);
+    q.by_terms = Divisor::of(q.segs_per_term); q.by_interleave = Divisor::of(q.interleave); q.by_group = Divisor::of(q.sched_group);
     q.kblocks_row = KIND == WGRAD ? 0 : q.nterms * (q.K / BK);
     return MOE_OK;
 }
