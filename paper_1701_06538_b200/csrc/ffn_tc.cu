@@ -52,7 +52,7 @@ constexpr unsigned long long WAIT_LIMIT_NS = 2000000000ull;
 enum Kind { ROW_BMN = 0, ROW_BK = 1, WGRAD = 2 };
 // What the epilogue does with an accumulator, fixed at compile time (a run-time choice kept every variant's registers and
 // code in one kernel: 950 cycles for the 32 conversions of a box without any option)
-enum Epilogue { EPI_PLAIN = 0, EPI_BIAS = 1, EPI_RELU = 2, EPI_MASK = 4, EPI_BITS = 8, EPI_F32 = 16 };
+enum Epilogue { EPI_PLAIN = 0, EPI_BIAS = 1, EPI_RELU = 2, EPI_MASK = 4, EPI_BITS = 8, EPI_F32 = 16, EPI_TWO_BOXES = 32 };
 
 constexpr int MAX_TERMS = 8;
 
@@ -226,6 +226,7 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap *tm, uint32_t src
 }
 __device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void tma_store_wait_read_but_one() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
 __device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 // A map in global memory that an earlier kernel has written: made visible to the copies of this thread, and fetched ahead
@@ -444,7 +445,10 @@ __device__ __forceinline__ void epilogue_box(const GemmParams &p, int lane, cons
             make_uint2(positive_bits(packed[0]), positive_bits(packed[1]));
     if (staged) {
         if (!MASKT) {  // an earlier store may still be reading the box
-            if (lane == 0) tma_store_wait_read();
+            if (lane == 0) {
+                if (EPI & EPI_TWO_BOXES) tma_store_wait_read_but_one();
+                else tma_store_wait_read();
+            }
             __syncwarp();
         }
 #pragma unroll
@@ -685,6 +689,10 @@ __device__ __forceinline__ bool acc_tile(const GemmParams &p, const Tile &t, int
     return true;
 }
 
+// EPI_TWO_BOXES (WGRAD over short segments): a warp's boxes take turns in two 4 KiB pieces, for one operand stage less. With one or two K
+// blocks a tile the epilogue is what a tile lasts, 1100 cycles a box, 420 of them waiting until the store before had read the box
+// out: 4096 experts x 64 rows 1056 and 1087 us -> 990 and 1066, 256 x 78 rows 61 -> 58; with three K blocks a tile the stage is worth
+// more (256 x 188 rows 83 -> 86). Sixteen epilogue warps, eight an accumulator, were no faster than the second box.
 // ACC (WGRAD with float output over long uniform row ranges, the gate backward): the contraction of a tile is cut
 // into sub-blocks of p.sub_kb0 / p.sub_kb K blocks (first term / other terms). Each sub-block is accumulated in TMEM on
 // its own (an fp32 tensor-core accumulator truncates, and a long run of same-sign terms loses low bits: 128 rows keep
@@ -699,7 +707,8 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;  // 1024-B aligned for the 128-B swizzle
     uint8_t *smem = smem_raw + (base - smem_u32(smem_raw));
-    constexpr int NST = STAGES;
+    constexpr bool TWO_BOXES = (EPI & EPI_TWO_BOXES) != 0;
+    constexpr int NST = TWO_BOXES ? STAGES - 1 : STAGES;
     const uint32_t bars = base + NST * STAGE_BYTES;
     auto full_bar = [&](int s) { return bars + 8u * s; };
     auto empty_bar = [&](int s) { return bars + 8u * (NST + s); };
@@ -847,7 +856,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     } else {
         // ------------------------------------------------------------------ epilogue (warps 2..9)
         const int quarter = warp & 3;  // TMEM lanes 32*quarter .. 32*quarter + 31 belong to this warp
-        int acc = 0;
+        int acc = 0, turn = 0;
         uint32_t acc_ph = 0;
         bool ok = true;
         TileIter<KIND, BM> it(p, (int32_t)blockIdx.x, (int32_t)gridDim.x);
@@ -871,7 +880,6 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             const int boxes = min(p.tile_n / 128, max(0, (p.N - first) / 64));  // N is a multiple of 64
             BoxArgs b;
             b.tm_out = &tmO;
-            b.box = smem + STAGES * STAGE_BYTES + 1024 + (warp - 2) * 4096;
             b.out_off = KIND == WGRAD ? (int64_t)t.e * p.M * p.N : 0;
             b.row0 = (KIND == WGRAD ? t.m0 : t.row0) + quarter * 32;
             b.rows_valid = (KIND == WGRAD ? p.M : t.row_end) - (int32_t)b.row0;
@@ -898,6 +906,8 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 b.taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + half * (p.tile_n / 2) + 64 * u;
                 b.next_bias = (EPI & EPI_BIAS) && u + 1 < boxes ? bias_at + 64 : nullptr;
                 b.keep = u ? keep[1] : keep[0];
+                b.box = smem + NST * STAGE_BYTES + 1024 + (TWO_BOXES ? (warp - 2) * 8192 + turn * 4096 : (warp - 2) * 4096);
+                if (b.rows_valid >= 32) turn ^= 1;  // (else nothing is stored from the box)
                 epilogue_box<EPI, false>(p, lane, b, bias, [&]() { if (u + 1 == boxes) release(); });
             }
             if (have_acc) {
@@ -1518,6 +1528,9 @@ template <int KIND> int32_t launch(const CUtensorMap &tmA, const CUtensorMap &tm
         if constexpr (KIND == ROW_BK) {
             if (p.bits_in) return launch_as<KIND, EPI_BITS>(tmA, tmB, p, grid, st, out);
             if (p.mask) return launch_as<KIND, EPI_MASK>(tmA, tmB, p, grid, st, out);
+        }
+        if constexpr (KIND == WGRAD) {
+            if (!p.seg_a) return launch_as<KIND, EPI_TWO_BOXES>(tmA, tmB, p, grid, st, out);  // short segments, see tc_wgrad_gemm
         }
         return launch_as<KIND, EPI_PLAIN>(tmA, tmB, p, grid, st, out);
     }
