@@ -691,7 +691,7 @@ __device__ __forceinline__ bool acc_tile(const GemmParams &p, const Tile &t, int
 
 // EPI_TWO_BOXES (WGRAD over short segments): a warp's boxes take turns in two 4 KiB pieces, for one operand stage less. With one or two K
 // blocks a tile the epilogue is what a tile lasts, 1100 cycles a box, 420 of them waiting until the store before had read the box
-// out: 4096 experts x 64 rows 1056 and 1087 us -> 990 and 1066, 256 x 78 rows 61 -> 58; with three K blocks a tile the stage is worth
+// out: 4096 experts x 64 rows 1056 and 1087 us -> 981 to 1012 and 1056 to 1076, 256 x 78 rows 61 -> 58; with three K blocks a tile the stage is worth
 // more (256 x 188 rows 83 -> 86). Sixteen epilogue warps, eight an accumulator, were no faster than the second box.
 // ACC (WGRAD with float output over long uniform row ranges, the gate backward): the contraction of a tile is cut
 // into sub-blocks of p.sub_kb0 / p.sub_kb K blocks (first term / other terms). Each sub-block is accumulated in TMEM on

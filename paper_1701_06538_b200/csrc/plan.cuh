@@ -1,4 +1,4 @@
-// The segment plan of a call (see plan.cu) as device code: one piece of it per block, by plan_kernel or by blocks of their own in the
+// The segment plan of a call (see plan.cu) as device code: one piece of it per block, by segment_plan_kernel or by blocks of their own in the
 // launch that finds the segments (route.cu).
 #pragma once
 
