@@ -4,6 +4,8 @@
 // estimators is taken to be their outer product divided by the mean of the row vector. Biases (vectors) keep a full
 // second-moment estimate. All of it is HBM streaming: the gradient is read twice (averages, update), the parameters
 // are read and written once. Sums are taken in fixed orders (no floating-point atomics): two runs agree bit for bit.
+#include <math_constants.h>
+
 #include "moe_internal.cuh"
 
 namespace moe {
@@ -120,13 +122,26 @@ __global__ void __launch_bounds__(256) adam_columns_kernel(const float *__restri
 // keeps one 16-byte column vector, with its column averages in registers, and walks down the block's rows, four of them
 // in flight. HBM bound: parameters read and written, gradients read (as one flat index space, the column averages came
 // from L1 with twice the loads of the parameters: 169 us for 134 M parameters, 4.8 TB/s).
-// The estimate is a product, so its root is the product of a row's and a column's root (each taken once per row and column and
-// correctly rounded): one multiply-add and one reciprocal per element.
+// The estimate is a product, so its root is the product of a row's and a column's root, each taken once per row and column: one
+// multiply-add and one reciprocal per element.
 __device__ __forceinline__ float adam_step(float w, float g, float lr, float row_root, float col_root, float eps) {
     return w - __fdividef(lr * g, fmaf(row_root, col_root, eps));
 }
 __device__ __forceinline__ float sqrt_fast(float x) { return x > 0.0f ? x * rsqrtf(x) : 0.0f; }  // ~2 ulp, no IEEE sqrt sequence
-__device__ __forceinline__ float root(float x) { return x > 0.0f ? sqrtf(x) : 0.0f; }
+// 0 for what is no number as well: an infinite gradient makes its column's average infinite and every row's factor 0
+__device__ __forceinline__ float root(float x) { return x > 0.0f && x < CUDART_INF_F ? sqrtf(x) : 0.0f; }
+// v_hat = row_avg_i * lift * factor * col_avg_j. The averages of an expert that gets no rows decay to the smallest floats, where
+// the quotient by their mean alone overflows; a row's average over that mean is at most the number of rows. 2^100 is exact and 1
+// elsewhere.
+struct RowFactor {
+    float lift, factor;
+    __device__ __forceinline__ RowFactor(float mean, float inv_correction) {
+        lift = mean < 1e-30f ? 0x1p100f : 1.0f;
+        mean *= lift;
+        factor = mean > 0.0f ? inv_correction / mean : 0.0f;
+    }
+    __device__ __forceinline__ float operator()(float row_avg) const { return row_avg * lift * factor; }
+};
 
 template <typename XT>
 __global__ void __launch_bounds__(256) adam_update_kernel(XT *__restrict__ W, const XT *__restrict__ g, int32_t rows,
@@ -137,8 +152,7 @@ __global__ void __launch_bounds__(256) adam_update_kernel(XT *__restrict__ W, co
     wait_previous_kernel();
     constexpr int VN = Vec<XT>::N;
     const int32_t e = blockIdx.y;
-    const float rm = row_mean[e];
-    const float scale = rm > 0.0f ? inv_correction / rm : 0.0f;  // v_hat = row_avg_i * col_avg_j * scale
+    const RowFactor scaled(row_mean[e], inv_correction);
     const int nvec = cols / VN;
     const float *ca = col_avg + (int64_t)e * cols;
     const int32_t r0 = blockIdx.x * ur, nr = min(ur, rows - r0);
@@ -162,7 +176,7 @@ __global__ void __launch_bounds__(256) adam_update_kernel(XT *__restrict__ W, co
                 if (row < nr) {
                     w[u].raw = reinterpret_cast<const uint4 *>(W + base + (int64_t)row * cols)[v];
                     gr[u].raw = reinterpret_cast<const uint4 *>(g + base + (int64_t)row * cols)[v];
-                    rs[u] = sqrt_fast(row_avg[(int64_t)e * rows + r0 + row] * scale);
+                    rs[u] = sqrt_fast(scaled(row_avg[(int64_t)e * rows + r0 + row]));
                 }
             }
 #pragma unroll
@@ -190,8 +204,7 @@ __global__ void __launch_bounds__(256) adam_update_flat_kernel(XT *__restrict__ 
     wait_previous_kernel();
     constexpr int VN = Vec<XT>::N;
     const int32_t e = blockIdx.y;
-    const float rm = row_mean[e];
-    const float scale = rm > 0.0f ? inv_correction / rm : 0.0f;  // v_hat = row_avg_i * col_avg_j * scale
+    const RowFactor scaled(row_mean[e], inv_correction);
     const int nvec = cols / VN;
     const float *ca = col_avg + (int64_t)e * cols;
     const int32_t r0 = blockIdx.x * FLAT_ROWS, nr = min(FLAT_ROWS, rows - r0);
@@ -212,7 +225,7 @@ __global__ void __launch_bounds__(256) adam_update_flat_kernel(XT *__restrict__ 
             const int idx = i0 + u * 256;
             if (idx >= total) break;
             const int r = idx / nvec, v = idx - r * nvec;
-            const float rs = row_avg[(int64_t)e * rows + r0 + r] * scale;
+            const float rs = scaled(row_avg[(int64_t)e * rows + r0 + r]);
 #pragma unroll
             for (int i = 0; i < VN; ++i)
                 w[u].set(i, w[u].get(i) - __fdividef(lr * gr[u].get(i), sqrt_fast(rs * ca[v * VN + i]) + eps));
@@ -417,9 +430,8 @@ __global__ void __launch_bounds__(FUSED_THREADS, 2) adam_fused_kernel(const __gr
     double total = 0.0;
 #pragma unroll
     for (int c = 0; c < 8; ++c) total += shares[c];
-    const float rm = (float)(total / (double)rows);
-    const float scale = rm > 0.0f ? a.inv_correction / rm : 0.0f;  // v_hat = row_avg_i * col_avg_j * scale
-    for (int r = tid; r < nr; r += FUSED_THREADS) row_now[r] = root(row_now[r] * scale);
+    const RowFactor scaled((float)(total / (double)rows), a.inv_correction);
+    for (int r = tid; r < nr; r += FUSED_THREADS) row_now[r] = root(scaled(row_now[r]));
     __syncthreads();
     cluster_arrive();  // no more reads of the other CTAs' shared memory
     if (warp_on) {
