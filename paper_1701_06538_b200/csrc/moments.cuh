@@ -60,7 +60,9 @@ __device__ __forceinline__ void cv2_block(const float *importance, int32_t n_imp
         const int t = threadIdx.x;
         double s1 = 0.0, s2 = 0.0;
         for (int q = 0; q < warps; ++q) { s1 += sh[4 * q + 2 * t]; s2 += sh[4 * q + 2 * t + 1]; }
-        const double m = t ? n_load : n_imp, mean = s1 / m, mu = (t ? c1 : c0) + mean, var = fmax(s2 / m - mean * mean, 0.0);
+        const double m = t ? n_load : n_imp, mean = s1 / m, mu = (t ? c1 : c0) + mean;
+        double var = s2 / m - mean * mean;
+        if (var < 0.0) var = 0.0;  // rounding; a NaN (of an infinite element) stays one, as in the gradient
         const float l = (float)((double)(t ? w_load : w_imp) * var / (mu * mu));
         losses[t] = l;
         if (losses2) losses2[t] = l;
