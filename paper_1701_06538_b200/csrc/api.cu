@@ -783,7 +783,7 @@ int32_t moe_query_ctx_layout(const moe_config *cfg, moe_ctx_layout *out) {
 
 int64_t moe_debug_bounds_violations(void) {
     const unsigned long long parts[] = {bounds_violations_route(), bounds_violations_losses(), bounds_violations_hier(),
-                                        bounds_violations_gate(), bounds_violations_ffn()};
+                                        bounds_violations_gate(), bounds_violations_gate_bwd(), bounds_violations_ffn()};
     unsigned long long sum = 0;
     for (unsigned long long v : parts) {
         if (v == ~0ull) return -1;

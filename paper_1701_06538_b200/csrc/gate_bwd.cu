@@ -76,6 +76,8 @@ __global__ void __launch_bounds__(256) gate_logit_grads_kernel(
         if (dsplit) {
             // three-term bf16 split (hi | mid | lo), row layout [3][clean n | raw n], for the tensor-core products
             const int64_t orow = split_row_index ? split_row_index[row] : row;  // e.g. sorted by primary group
+            MOE_BOUNDS_NOTE((uint64_t)orow < (uint64_t)rows);
+            if ((uint64_t)orow >= (uint64_t)rows) return;  // a slot without a row
             bf16 *o = dsplit + orow * (6 * (int64_t)n);
             float v = dc;
 #pragma unroll
@@ -221,6 +223,8 @@ __global__ void __launch_bounds__(256) gate_logit_grads_pairs_kernel(
     }
     if (!live) return;
     const int64_t orow = split_row_index ? split_row_index[row] : row;  // e.g. sorted by primary group
+    MOE_BOUNDS_NOTE((uint64_t)orow < (uint64_t)rows);
+    if ((uint64_t)orow >= (uint64_t)rows) return;  // a slot without a row
     bf16 *o = dsplit + orow * (6 * (int64_t)n);
 #pragma unroll
     for (int u = 0; u < NVP; ++u) {
@@ -298,5 +302,7 @@ int32_t launch_gate_logit_grads(const float *noise, const float *clean, const fl
     MOE_LAUNCHED();
     return MOE_OK;
 }
+
+MOE_BOUNDS_READER(bounds_violations_gate_bwd)
 
 }  // namespace moe

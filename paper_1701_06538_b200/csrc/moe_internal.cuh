@@ -71,6 +71,7 @@ unsigned long long bounds_violations_route();
 unsigned long long bounds_violations_losses();
 unsigned long long bounds_violations_hier();
 unsigned long long bounds_violations_gate();
+unsigned long long bounds_violations_gate_bwd();
 unsigned long long bounds_violations_ffn();
 
 typedef __nv_bfloat16 bf16;

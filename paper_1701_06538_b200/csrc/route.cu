@@ -915,6 +915,9 @@ __global__ void __launch_bounds__(256) dispatch_bwd_kernel(const XT *__restrict_
             if (SEC) {
                 for (int s1 = 0; s1 < sec.k1; ++s1) {
                     const int64_t slot = t * sec.k1 + s1, r = sec.perm ? (int64_t)sec.perm[slot] : slot;
+                    const bool has_row = (uint64_t)r < (uint64_t)(T * sec.k1);  // like a dropped slot of the experts
+                    MOE_BOUNDS_NOTE(has_row);
+                    if (!has_row) continue;
                     float4 more[VB][VN / 4];
 #pragma unroll
                     for (int b = 0; b < VB; ++b)
