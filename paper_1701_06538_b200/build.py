@@ -45,7 +45,7 @@ def build(force: bool = False, verbose: bool = False, defines=(), obj_dir=None, 
     OBJ, LIB = obj_dir or globals()["OBJ"], lib or globals()["LIB"]
     os.makedirs(OBJ, exist_ok=True)
     sources = sorted(glob.glob(os.path.join(CSRC, "*.cu")))
-    headers = sorted(glob.glob(os.path.join(CSRC, "*.cuh"))) + sorted(glob.glob(os.path.join(ROOT, "include", "*.h")))
+    headers = sorted(glob.glob(os.path.join(CSRC, "*.cuh"))) + sorted(glob.glob(os.path.join(CSRC, "*.h"))) + sorted(glob.glob(os.path.join(ROOT, "include", "*.h")))
     nvcc = _nvcc()
     jobs = []
     for src in sources:

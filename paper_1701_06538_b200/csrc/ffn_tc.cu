@@ -1478,14 +1478,12 @@ int32_t map_weight_kmajor_half(CUtensorMap *tm, const void *p, int64_t n, int64_
 }
 
 int sm_count() {
-    static int n = 0;
-    if (!n) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        if (n <= 0) n = 148;
-    }
-    return n;
+    static PerDevice count;
+    const int n = count.get([]() {
+        int dev = 0, v = 0;
+        return cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? v : 0;
+    });
+    return n > 0 ? n : 148;
 }
 
 // Derived tile counts the device code divides by; ids are 32-bit.
@@ -1503,11 +1501,8 @@ template <int KIND, int TM> int32_t complete_params(GemmParams &q, int64_t max_t
 
 template <int KIND, int EPI> int32_t launch_as(const CUtensorMap &tmA, const CUtensorMap &tmB, const GemmParams &p, unsigned grid,
                                                cudaStream_t st, const CUtensorMap &tmO) {
-    static bool configured = false;
-    if (!configured) {
-        MOE_CUDA(cudaFuncSetAttribute(grouped_gemm_kernel<KIND, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
-        configured = true;
-    }
+    static PerDevice configured;
+    if (!allow_shared(configured, grouped_gemm_kernel<KIND, EPI>, SMEM_BYTES)) return MOE_ERR_CUDA;
     if (grid == 0) return MOE_OK;
     launch_kernel(grouped_gemm_kernel<KIND, EPI>, grid, NTHREADS, SMEM_BYTES, st, tmA, tmB, tmO, p);
     MOE_LAUNCHED();
@@ -1541,11 +1536,8 @@ int32_t launch_acc_wgrad(const CUtensorMap &tmA, const CUtensorMap &tmB, const G
                          cudaStream_t st) {
     GemmParams p = p_in;
     MOE_TRY((complete_params<WGRAD, BM>(p, max_tiles)));
-    static bool configured = false;
-    if (!configured) {
-        MOE_CUDA(cudaFuncSetAttribute(grouped_gemm_kernel<WGRAD, EPI_F32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
-        configured = true;
-    }
+    static PerDevice configured;
+    if (!allow_shared(configured, grouped_gemm_kernel<WGRAD, EPI_F32, true>, SMEM_BYTES)) return MOE_ERR_CUDA;
     if (max_tiles <= 0) return MOE_OK;
     const unsigned grid = (unsigned)imin(max_tiles, sm_count());
     launch_kernel((grouped_gemm_kernel<WGRAD, EPI_F32, true>), grid, NTHREADS, SMEM_BYTES, st, tmA, tmB, tmA, p);
@@ -1559,7 +1551,7 @@ int32_t launch2_as(const CUtensorMap &tmA, const CUtensorMap &tmB, const GemmPar
     GemmParams p = p_in;
     p.tma_out = tmO != nullptr;
     MOE_TRY((complete_params<KIND, 256>(p, max_tiles)));
-    static int max_clusters = 0;
+    static PerDevice clusters;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cudaLaunchAttribute attrs[2];
@@ -1569,13 +1561,14 @@ int32_t launch2_as(const CUtensorMap &tmA, const CUtensorMap &tmB, const GemmPar
     attrs[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.blockDim = dim3(NTHREADS2); cfg.dynamicSmemBytes = SMEM2_BYTES; cfg.stream = st;
     cfg.attrs = attrs; cfg.numAttrs = 2;
-    if (!max_clusters) {
-        MOE_CUDA(cudaFuncSetAttribute((grouped_gemm2_kernel<KIND, EPI, MASKT, ACC>), cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM2_BYTES));
+    const int max_clusters = clusters.get([&]() {
         cfg.gridDim = dim3(2 * (sm_count() / 2));
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, (grouped_gemm2_kernel<KIND, EPI, MASKT, ACC>), &cfg) != cudaSuccess || n <= 0) return MOE_ERR_CUDA;
-        max_clusters = n;
-    }
+        const auto kernel = grouped_gemm2_kernel<KIND, EPI, MASKT, ACC>;
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM2_BYTES) != cudaSuccess) return 0;
+        return cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess ? n : 0;
+    });
+    if (max_clusters <= 0) return MOE_ERR_CUDA;
     if (max_tiles <= 0) return MOE_OK;
 #ifdef MOE_TILE_TRACE
     {   // the launch whose index (counted over the two-CTA launches of the process) equals MOE_TRACE_LAUNCH records

@@ -9,6 +9,7 @@
 #include <utility>
 
 #include "moe.h"
+#include "per_device.h"
 
 #define MOE_TRY(expr)                                \
     do {                                             \

@@ -539,11 +539,8 @@ bool plan_fused(FusedAdam &a, int32_t n, int32_t d, int32_t h, size_t *smem) {
 
 template <typename XT>
 int32_t launch_fused(const FusedAdam &a, size_t smem, cudaStream_t st) {
-    static bool configured = false;
-    if (!configured) {
-        MOE_CUDA(cudaFuncSetAttribute(adam_fused_kernel<XT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));
-        configured = true;
-    }
+    static PerDevice configured;
+    if (!allow_shared(configured, adam_fused_kernel<XT>, 100 * 1024)) return MOE_ERR_CUDA;
     const int64_t count = a.v[0].count > a.v[1].count ? a.v[0].count : a.v[1].count;
     const int64_t vector_clusters = imin(cdiv(count, 2 * FUSED_THREADS * a.cluster), cdiv(2 * 148, a.cluster));
     cudaLaunchAttribute attrs[2];
