@@ -236,11 +236,18 @@ struct LossesWs {
     }
 };
 
-struct FfnBwdWs {
+// Scratch of the expert backward. The tile sums of db2 stand by themselves: a fused call has them formed while the gate's backward has the
+// place of everything else (FusedBwdWs).
+struct Db2Sums {
+    float *colsum2;
+    Db2Sums(Carver &cv, const Dims &D) : colsum2(cv.take<float>(colsum_ws_floats(D.R, (int32_t)D.n, (int32_t)D.d))) {}
+};
+
+struct FfnBwdWs : Db2Sums {
     void *dz;
-    float *colsum, *colsum2;  // of db1, of db2
+    float *colsum;   // of db1
     uint32_t *bits;  // MOE_FLAG_RECOMPUTE_HID on the tensor cores: the mask bits that the recomputation writes
-    FfnBwdWs(Carver &cv, const Dims &D) {
+    FfnBwdWs(const Db2Sums &sums, Carver &cv, const Dims &D) : Db2Sums(sums) {
         dz = cv.take_bytes(D.R * D.h * (int64_t)D.esz);
         const bool tc = D.act == MOE_BF16 && D.d % 64 == 0 && D.h % 64 == 0;
         bits = tc && (D.flags & MOE_FLAG_RECOMPUTE_HID) ? cv.take<uint32_t>(D.R * (D.h / 32)) : nullptr;
@@ -250,8 +257,8 @@ struct FfnBwdWs {
             if (cs_tc > cs) cs = cs_tc;
         }
         colsum = cv.take<float>(cs);
-        colsum2 = cv.take<float>(colsum_ws_floats(D.R, (int32_t)D.n, (int32_t)D.d));
     }
+    FfnBwdWs(Carver &cv, const Dims &D) : FfnBwdWs(Db2Sums(cv, D), cv, D) {}
 };
 
 struct LossesBwdWs {
@@ -264,21 +271,33 @@ struct LossesBwdWs {
 
 int64_t gate_weight_grads_part(const Dims &D, int64_t cols);  // floats of scratch of gate_weight_grads
 
-struct GateBwdWs {
-    float *dlogit, *dlogit_s, *partials, *dX_sec, *partials_s;  // dlogit rows: (clean | raw noise) columns
-    void *dsplit, *wsplit, *dsplit_s, *wsplit_s, *xs_p;
+// Scratch of the gate backward: what the last launch of a fused call still reads (GateBwdSums), and what is free again behind the gate.
+// MOE_FLAG_RECOMPUTE_HID saves memory: the float rows of the secondary gates are not kept for the last launch then.
+bool keeps_secondary_rows(const Dims &D) { return !(D.flags & MOE_FLAG_RECOMPUTE_HID); }
+struct GateBwdSums {
+    float *partials, *dX_sec;
     bool tc, tc_hier;
-    HierIdxWs H;
-    GateBwdWs(Carver &cv, const Dims &D) : H(cv, D) {
-        dlogit = dlogit_s = partials = dX_sec = partials_s = nullptr;
-        dsplit = wsplit = dsplit_s = wsplit_s = xs_p = nullptr;
-        if (D.hier) dX_sec = cv.take<float>(D.T * D.k1 * D.d);
+    GateBwdSums(Carver &cv, const Dims &D) {
         tc = !D.hier && tc_gate_bwd_supported(D.act, (int32_t)D.d, (int32_t)D.n);
         tc_hier = D.hier && tc_hier_gate_bwd_supported(D.act, (int32_t)D.d, (int32_t)D.a, (int32_t)D.b);
+        const int32_t n1 = (int32_t)(D.hier ? D.a : D.n);
+        partials = cv.take<float>(tc || tc_hier ? tc_gate_bwd_partials(D.T, (int32_t)D.d, n1) : gate_weight_grads_part(D, 2 * n1));
+        dX_sec = D.hier && keeps_secondary_rows(D) ? cv.take<float>(D.T * D.k1 * D.d) : nullptr;
+    }
+};
+
+struct GateBwdWs : GateBwdSums {
+    float *dlogit, *dlogit_s, *partials_s;  // dlogit rows: (clean | raw noise) columns
+    void *dsplit, *wsplit, *dsplit_s, *wsplit_s, *xs_p;
+    HierIdxWs H;
+    GateBwdWs(Carver &cv, const Dims &D) : GateBwdWs(GateBwdSums(cv, D), cv, D) {}
+    GateBwdWs(const GateBwdSums &sums, Carver &cv, const Dims &D) : GateBwdSums(sums), H(cv, D) {
+        if (D.hier && !keeps_secondary_rows(D)) dX_sec = cv.take<float>(D.T * D.k1 * D.d);
+        dlogit = dlogit_s = partials_s = nullptr;
+        dsplit = wsplit = dsplit_s = wsplit_s = xs_p = nullptr;
         if (tc_hier) {
             dsplit = cv.take<bf16>(D.T * 6 * D.a);
             wsplit = cv.take<bf16>(D.d * 6 * D.a);
-            partials = cv.take<float>(tc_gate_bwd_partials(D.T, (int32_t)D.d, (int32_t)D.a));
             dsplit_s = cv.take<bf16>(D.T * D.k1 * 6 * D.b);
             wsplit_s = cv.take<bf16>(D.a * D.d * 6 * D.b);
             partials_s = cv.take<float>(3 * D.a * D.d * 2 * D.b);
@@ -286,11 +305,9 @@ struct GateBwdWs {
         } else if (tc) {
             dsplit = cv.take<bf16>(D.T * 6 * D.n);
             wsplit = cv.take<bf16>(D.d * 6 * D.n);
-            partials = cv.take<float>(tc_gate_bwd_partials(D.T, (int32_t)D.d, (int32_t)D.n));
         } else {
             const int64_t n1 = D.hier ? D.a : D.n, P1 = D.T * D.k1;
             dlogit = cv.take<float>(D.T * 2 * n1);
-            partials = cv.take<float>(gate_weight_grads_part(D, 2 * n1));
             if (D.hier) {
                 dlogit_s = cv.take<float>(P1 * 2 * D.b);
                 partials_s = cv.take<float>(simt_wgrad_splits(D.d, 2 * D.b, (int32_t)D.a, P1) * D.a * D.d * 2 * D.b);
@@ -342,7 +359,7 @@ struct Ctx {
 
 struct BwdWs {
     float *dgates, *dload, *dX_gate, *dimp, *dload_h;
-    void *dys, *dxs;
+    void *dys;
     int32_t *plan;
     BwdWs(Carver &cv, const Dims &D) {
         plan = cv.take<int32_t>(plan_ints(D.R, D.n));
@@ -352,7 +369,27 @@ struct BwdWs {
         dload = cv.take<float>(D.dload);
         dX_gate = cv.take<float>(D.T * D.d);
         dys = cv.take_bytes(D.R * D.d * (int64_t)D.esz);
-        dxs = cv.take_bytes(D.R * D.d * (int64_t)D.esz);
+    }
+};
+
+// Workspace of a fused backward call: what lives throughout, then one piece that the gate's scratch has first and the experts' (dxs, dz,
+// hidden activations that are computed again) afterwards.
+struct FusedBwdWs : BwdWs {
+  private:
+    Db2Sums db2;
+    GateBwdSums gate_sums;
+    Carver experts_at, gate_at;
+
+  public:
+    void *dxs;
+    FfnBwdWs ffn;
+    FfnWs again;
+    GateBwdWs gate;
+    FusedBwdWs(Carver &cv, const Dims &D)
+        : BwdWs(cv, D), db2(cv, D), gate_sums(cv, D), experts_at(cv), gate_at(cv),
+          dxs(experts_at.take_bytes(D.R * D.d * (int64_t)D.esz)), ffn(db2, experts_at, D), again(experts_at, D),
+          gate(gate_sums, gate_at, D) {
+        cv = experts_at.off > gate_at.off ? experts_at : gate_at;
     }
 };
 
@@ -450,12 +487,11 @@ SimtGemm base_gemm(const Dims &D) {
 // call: its first kernel has cleared the word, and what the gate's products reported since stays.
 int32_t do_expert_ffn(const moe_config *c, const Dims &D, const void *xs, const int32_t *offsets, const void *W1,
                       const void *b1, const void *W2, const void *b2, void *hid, void *ys, void *ws_base,
-                      Carver &cv, cudaStream_t st, int32_t *clear, bool first_only = false, void **hid_used = nullptr,
+                      Carver &cv, cudaStream_t st, int32_t *clear, bool first_only = false,
                       uint32_t *relu_bits = nullptr, const SegmentPlan *ready = nullptr) {
     FfnWs w(cv, D);
     if (!hid) hid = w.hid;
     if (!hid) return MOE_ERR_INVALID_ARG;
-    if (hid_used) *hid_used = hid;
     const SegmentPlan plan = ready ? *ready : make_plan(c, D, w.plan, false);
     if (!ready) {
         SegmentMaps maps;
@@ -525,9 +561,8 @@ ColumnSums db2_sums(const Dims &D, const void *dys, void *db2, const int32_t *of
 // tail: the last passes over the bias gradients' sums may be left to the caller; db2_begun: the tile sums of db2 have been formed already
 int32_t do_expert_ffn_bwd(const moe_config *c, const Dims &D, const void *xs, const void *hid, const void *dys,
                           const int32_t *offsets, const void *W1, const void *W2, void *dxs, void *dW1, void *db1,
-                          void *dW2, void *db2, void *ws_base, Carver &cv, cudaStream_t st, const SegmentPlan &plan,
+                          void *dW2, void *db2, void *ws_base, const FfnBwdWs &w, cudaStream_t st, const SegmentPlan &plan,
                           const uint32_t *relu_bits = nullptr, BackwardTail *tail = nullptr, bool db2_begun = false) {
-    FfnBwdWs w(cv, D);
     const int32_t n = (int32_t)D.n;
     BackwardTail *leave = n < COLSUM_MANY ? tail : nullptr;
     auto finish = [&](const ColumnSums &sums, int which) -> int32_t {
@@ -578,17 +613,14 @@ int32_t expert_ffn_bwd_stage(const moe_config *c, const Dims &D, const void *xs,
                              const int32_t *offsets, const void *W1, const void *W2, void *dxs, void *dW1, void *db1, void *dW2,
                              void *db2, void *ws, Carver &cv, cudaStream_t st, const uint32_t *relu_bits) {
     const SegmentPlan plan = make_plan(c, D, cv.take<int32_t>(plan_ints(D.R, D.n)), true);
+    const FfnBwdWs w(cv, D);
     SegmentMaps maps;
     const bool tc = tc_ffn_supported(*c);
-    if (tc) {
-        Carver ahead = cv;  // where do_expert_ffn_bwd will have dz
-        const FfnBwdWs w(ahead, D);
-        MOE_TRY(tc_segment_maps(*c, &maps, nullptr, nullptr, dys, w.dz, hid, dys, xs, w.dz));
-    }
+    if (tc) MOE_TRY(tc_segment_maps(*c, &maps, nullptr, nullptr, dys, w.dz, hid, dys, xs, w.dz));
     PlanArgs args;
     fill_plan(&args, plan, (int32_t)D.n, D.R, status_word(ws), tc ? &maps : nullptr);
     MOE_TRY(launch_segment_plan(args, offsets, st));
-    return do_expert_ffn_bwd(c, D, xs, hid, dys, offsets, W1, W2, dxs, dW1, db1, dW2, db2, ws, cv, st, plan, relu_bits);
+    return do_expert_ffn_bwd(c, D, xs, hid, dys, offsets, W1, W2, dxs, dW1, db1, dW2, db2, ws, w, st, plan, relu_bits);
 }
 
 int32_t do_losses_bwd(const moe_config *c, const Dims &D, const float *importance, const float *load,
@@ -627,7 +659,7 @@ int64_t gate_weight_grads_part(const Dims &D, int64_t cols) { return simt_wgrad_
 int32_t do_gate_bwd(const moe_config *c, const Dims &D, const void *x, const float *Wg, const float *Wnoise,
                     const float *noise, const float *clean, const float *raw_noise, const int32_t *topk_idx,
                     const float *gates, const float *kth_vals, const int32_t *kth_idx, float *dgates,
-                    const float *dload, float *dWg, float *dWnoise, float *dX_gate, void *ws_base, Carver &cv,
+                    const float *dload, float *dWg, float *dWnoise, float *dX_gate, void *ws_base, GateBwdWs &w,
                     cudaStream_t st, const HierIdx *ready = nullptr, SecondaryRows *sec = nullptr, const ColumnSums *beside = nullptr,
                     BackwardTail *tail = nullptr) {
     // sec: the caller adds the secondary gates' rows to dX_gate itself (they stay in the scratch); beside: tile sums to be formed along
@@ -639,7 +671,6 @@ int32_t do_gate_bwd(const moe_config *c, const Dims &D, const void *x, const flo
         tail->parts = left;
         tail->parts_blocks = (int32_t)cdiv((int64_t)left.d * left.cols, 256);
     };
-    GateBwdWs w(cv, D);
     if (D.hier) {
         const int64_t P1 = D.T * D.k1, lp = D.T * D.a, wp = D.d * D.a;
         const float *g_p = gates + D.T * D.k, *g_s = g_p + P1;
@@ -762,7 +793,7 @@ int32_t moe_query_sizes(const moe_config *cfg, moe_sizes *out) {
     int64_t stage_bwd = s_fbwd;
     if (s_lbwd > stage_bwd) stage_bwd = s_lbwd;
     if (s_gbwd > stage_bwd) stage_bwd = s_gbwd;
-    const int64_t s_fused_bwd = measure([&](Carver &cv) { BwdWs b(cv, D); FfnBwdWs w(cv, D); FfnWs f(cv, D); GateBwdWs g(cv, D); (void)b; (void)w; (void)f; (void)g; });
+    const int64_t s_fused_bwd = measure([&](Carver &cv) { FusedBwdWs w(cv, D); (void)w; });
     out->adam_state_elems = D.n * (3 * D.d + 3 * D.h);
     out->ws_adam_bytes = kWsHeader + ((adam_ws_floats((int32_t)D.n, (int32_t)D.d, (int32_t)D.h) * 4 + 255) & ~(int64_t)255);
     out->ws_bytes = fwd > stage_bwd ? fwd : stage_bwd;
@@ -864,7 +895,7 @@ int32_t moe_expert_ffn_bits(const moe_config *cfg, const void *xs, const int32_t
     const Dims D = dims_of(cfg);
     Carver cv(ws);
     cv.take_bytes(kWsHeader);
-    return do_expert_ffn(cfg, D, xs, offsets, W1, b1, W2, b2, hid, ys, ws, cv, as_stream(stream), status_word(ws), false, nullptr,
+    return do_expert_ffn(cfg, D, xs, offsets, W1, b1, W2, b2, hid, ys, ws, cv, as_stream(stream), status_word(ws), false,
                          relu_bits);
 }
 
@@ -947,8 +978,9 @@ int32_t moe_gate_bwd(const moe_config *cfg, const void *x, const float *Wg, cons
     Carver cv(ws);
     cv.take_bytes(kWsHeader);
     MOE_TRY(reset_status(ws, as_stream(stream)));
+    GateBwdWs w(cv, D);
     return do_gate_bwd(cfg, D, x, Wg, Wnoise, noise, clean, raw_noise, topk_idx, gates, kth_vals, kth_idx, dgates,
-                       dload, dWg, dWnoise, dX_gate, ws, cv, as_stream(stream));
+                       dload, dWg, dWnoise, dX_gate, ws, w, as_stream(stream));
 }
 
 // keep_bits != nullptr: the output is that of the layer epilogue (sigmoid, dropout, residual) instead of Eq. 1 alone
@@ -989,7 +1021,7 @@ static int32_t forward_impl(const moe_config *cfg, const void *x, const float *W
     const bool ride = D.T > 0 && sums.n <= LEVEL_RIDE_MAX;
     MOE_TRY(do_dispatch(D, x, C.topk_idx, C.xs, C.perm, C.inv_perm, C.counts, C.offsets, dispatch_at, st, &args, ride ? &sums : nullptr));
     { Carver at = fresh();
-      MOE_TRY(do_expert_ffn(cfg, D, C.xs, C.offsets, W1, b1, W2, b2, C.hid, C.ys, ws, at, st, nullptr, false, nullptr,
+      MOE_TRY(do_expert_ffn(cfg, D, C.xs, C.offsets, W1, b1, W2, b2, C.hid, C.ys, ws, at, st, nullptr, false,
                             C.relu_bits, &plan)); }  // C.hid null: stays in ws
     MOE_TRY(launch_combine(C.ys, D.act, C.gates, C.inv_perm, D.T, (int32_t)D.k, (int32_t)D.d, y, st,
                            keep_bits ? x : nullptr, keep_bits, keep_bits ? 1.0f / (1.0f - drop_prob) : 1.0f, ride ? &sums : nullptr));
@@ -1026,23 +1058,18 @@ static int32_t backward_impl(const moe_config *cfg, const void *dY, const void *
     const Dims D = dims_of(cfg);
     cudaStream_t st = as_stream(stream);
     Ctx C(const_cast<void *>(ctx), D, tc_ffn_supported(*cfg));
-    Carver base(ws);
-    base.take_bytes(kWsHeader);
-    BwdWs B(base, D);
-    auto fresh = [&]() { return base; };  // stage scratch starts after the tensors that live across stages
+    Carver cv(ws);
+    cv.take_bytes(kWsHeader);
+    FusedBwdWs B(cv, D);
     // everything that depends on the routing alone in one launch: the segment plan, the gradients of the balancing losses
     // (load[0 : n] is Load_H in the hierarchical layer), the status word
     const SegmentPlan plan = make_plan(cfg, D, B.plan, true);
     const Cv2Job jobs[2] = {{C.importance, (int32_t)D.n, cfg->w_importance, B.dimp},
                             {C.load, (int32_t)D.n, cfg->w_load, D.hier ? B.dload_h : B.dload}};
-    // Scratch: the expert backward's, hidden activations that are computed again, the gate's (all of it lives until the last launch)
-    Carver cv = fresh();
-    const FfnBwdWs ffn(cv, D);
-    const FfnWs again(cv, D);
     SegmentMaps maps;
     const bool tc = tc_ffn_supported(*cfg);
     if (tc)
-        MOE_TRY(tc_segment_maps(*cfg, &maps, C.hid ? nullptr : C.xs, nullptr, B.dys, ffn.dz, C.hid ? C.hid : again.hid, B.dys, C.xs, ffn.dz));
+        MOE_TRY(tc_segment_maps(*cfg, &maps, C.hid ? nullptr : C.xs, nullptr, B.dys, B.ffn.dz, C.hid ? C.hid : B.again.hid, B.dys, C.xs, B.ffn.dz));
     PlanArgs args;
     fill_plan(&args, plan, (int32_t)D.n, D.R, status_word(ws), tc ? &maps : nullptr, jobs);
     MOE_TRY(launch_segment_plan(args, C.offsets, st));
@@ -1055,23 +1082,19 @@ static int32_t backward_impl(const moe_config *cfg, const void *dY, const void *
     BackwardTail tail = {};
     BackwardTail *left = D.T > 0 ? &tail : nullptr;
     SecondaryRows sec = {};
-    const ColumnSums db2s = db2_sums(D, B.dys, db2, C.offsets, ffn, plan);
+    const ColumnSums db2s = db2_sums(D, B.dys, db2, C.offsets, B.ffn, plan);
     MOE_TRY(do_gate_bwd(cfg, D, x, Wg, Wnoise, noise, C.clean, C.raw_noise, C.topk_idx, C.gates, C.kth_vals,
-                        C.kth_idx, B.dgates, B.dload, dWg, dWnoise, B.dX_gate, ws, cv, st, &C.hier, &sec, left ? &db2s : nullptr, left));
+                        C.kth_idx, B.dgates, B.dload, dWg, dWnoise, B.dX_gate, ws, B.gate, st, &C.hier, keeps_secondary_rows(D) ? &sec : nullptr, left ? &db2s : nullptr, left));
     const void *hid = C.hid;
     uint32_t *bits = C.relu_bits;
     if (!hid) {  // MOE_FLAG_RECOMPUTE_HID: the forward kept no hidden activations; the first GEMM is run again
-        Carver at = fresh();
-        FfnBwdWs own(at, D);
-        void *made = nullptr;
-        bits = own.bits;
-        MOE_TRY(do_expert_ffn(cfg, D, C.xs, C.offsets, W1, b1, W2, b2, nullptr, nullptr, ws, at, st, nullptr, true, &made, bits,
-                              &plan));
-        hid = made;
+        bits = B.ffn.bits;
+        Carver none(nullptr);  // (both buffers are given)
+        MOE_TRY(do_expert_ffn(cfg, D, C.xs, C.offsets, W1, b1, W2, b2, B.again.hid, nullptr, ws, none, st, nullptr, true, bits, &plan));
+        hid = B.again.hid;
     }
-    { Carver at = fresh();
-      MOE_TRY(do_expert_ffn_bwd(cfg, D, C.xs, hid, B.dys, C.offsets, W1, W2, B.dxs, dW1, db1, dW2, db2, ws, at,
-                                st, plan, bits, left, left != nullptr)); }
+    MOE_TRY(do_expert_ffn_bwd(cfg, D, C.xs, hid, B.dys, C.offsets, W1, W2, B.dxs, dW1, db1, dW2, db2, ws, B.ffn, st, plan, bits, left,
+                              left != nullptr));
     // dX = expert path + gating path (+ the upstream gradient itself through the residual connection)
     return launch_dispatch_bwd(B.dxs, D.act, C.inv_perm, D.T, (int32_t)D.k, (int32_t)D.d, B.dX_gate, nullptr, dX,
                                st, keep_bits ? dY : nullptr, sec, left);
