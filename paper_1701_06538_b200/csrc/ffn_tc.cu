@@ -1617,6 +1617,12 @@ static bool use_two_cta(int64_t R, int32_t nseg, int32_t flags, int32_t cols) {
     return R / (nseg > 0 ? nseg : 1) >= 384;
 }
 
+// The last K block of a segment through the segment's own maps: each costs the loading thread a fence, so that with one or two K
+// blocks to a segment the one-CTA kernel clears the rows in shared memory instead (4096 experts x 64 rows: 1070 us, with maps 1187;
+// 256 x 78: 67, 75; but 256 x 188: 93, 82; on SM pairs, where clearing held the tensor cores up for a third of a tile,
+// 256 x 512: 192, 138)
+static bool wgrad_uses_maps(int64_t R, int32_t nseg) { return R >= 128 * (int64_t)nseg; }
+
 int32_t tc_segment_maps(const moe_config &c, SegmentMaps *maps, const void *xs_rows, const void *hid_rows, const void *dys_rows,
                         const void *dz_rows, const void *hid_cols, const void *dys_cols, const void *xs_cols, const void *dz_cols) {
     memset(maps, 0, sizeof(*maps));
@@ -1633,6 +1639,7 @@ int32_t tc_segment_maps(const moe_config &c, SegmentMaps *maps, const void *xs_r
     MOE_TRY(add(MAP_HID_ROWS, hid_rows, c.h, 0));
     MOE_TRY(add(MAP_DYS_ROWS, dys_rows, c.d, 0));
     MOE_TRY(add(MAP_DZ_ROWS, dz_rows, c.h, 0));
+    if (!wgrad_uses_maps(R, c.n)) return MOE_OK;
     MOE_TRY(add(MAP_HID_COLS, hid_cols, c.h, 2));
     MOE_TRY(add(MAP_DYS_COLS, dys_cols, c.d, b2));
     MOE_TRY(add(MAP_XS_COLS, xs_cols, c.d, 2));
@@ -1787,11 +1794,7 @@ int32_t tc_wgrad_gemm(const void *A, const void *B, const int32_t *offsets, int3
     CUtensorMap tmA, tmB;
     GemmParams p = default_params();
     p.offsets = offsets; p.nseg = nseg; p.M = M; p.N = N; p.R = R;
-    // The last K block of a segment through the segment's own maps: each costs the loading thread a fence, so that with one or two K
-    // blocks to a segment the one-CTA kernel clears the rows in shared memory instead (4096 experts x 64 rows: 1070 us, with maps 1187;
-    // 256 x 78: 67, 75; but 256 x 188: 93, 82; on SM pairs, where clearing held the tensor cores up for a third of a tile,
-    // 256 x 512: 192, 138)
-    if (R >= 128 * (int64_t)nseg) { p.seg_a = plan.maps_of(seg_a); p.seg_b = plan.maps_of(seg_b); }
+    if (wgrad_uses_maps(R, nseg)) { p.seg_a = plan.maps_of(seg_a); p.seg_b = plan.maps_of(seg_b); }
     p.out = (bf16 *)out; p.status = status;
     CUtensorMap tmO;  // the experts' matrices as one tall matrix (a 32-row box never straddles two: M is a multiple of 64)
     MOE_TRY(map_out_boxes(&tmO, out, (int64_t)nseg * M, N));
