@@ -38,6 +38,7 @@ void fill_plan(PlanArgs *a, const SegmentPlan &plan, int32_t n, int64_t R, int32
     a->max_m = plan.info && plan.bm[0] ? (int32_t)(cdiv(R, plan.bm[0]) + n) : 0;
     if (jobs) { a->cv2[0] = jobs[0]; a->cv2[1] = jobs[1]; }
     a->map_block0 = PLAN_HEIGHTS + (plan.sched ? 2 + (int32_t)cdiv(n, 1024) : jobs ? 2 : 0);
+    a->rows = (int32_t)R;
     if (maps && plan.maps) a->maps = *maps;
 }
 

@@ -13,6 +13,7 @@ struct PlanArgs {
     int32_t *status;   // cleared if given
     Cv2Job cv2[2];
     int32_t map_block0;  // first block of the tensor maps
+    int32_t rows;        // of the mapped tensors: no map ends behind them, whatever the offsets say
     SegmentMaps maps;
 };
 constexpr int MAPS_PER_BLOCK = 64;  // two per warp
@@ -76,7 +77,7 @@ __device__ __forceinline__ void plan_piece(const PlanArgs &a, int32_t block, con
                 i -= n;
             }
             if (which < SEGMENT_MAPS)
-                write_segment_map(a.maps.base[which], a.plan.maps + (int64_t)which * n + i, offsets[i + 1], (uint32_t *)cnt + 64 * w + 32 * q);
+                write_segment_map(a.maps.base[which], a.plan.maps + (int64_t)which * n + i, min(offsets[i + 1], a.rows), (uint32_t *)cnt + 64 * w + 32 * q);
         }
         return;
     }
