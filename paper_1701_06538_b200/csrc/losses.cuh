@@ -72,7 +72,8 @@ template <int NV> __device__ __forceinline__ void level_sums_rows(const LevelSum
 }
 
 // Importance / Load = the blocks' partial sums added in double. A block takes 32 columns; its eight warps each add an
-// eighth of the chunks (in ascending order, ten loads in flight), the eight sums are then added in warp order. With
+// eighth of the chunks (in ascending order, eight loads in flight: with a condition on each of ten they wait for one another, both
+// launches of 32768 x 64 36 us, this way 24), the eight sums are then added in warp order. With
 // fin.losses set, the block that finishes last (counted by `ticket`) also forms the two losses from the complete vectors,
 // and the copies in fin.copy are written along the way.
 __device__ __forceinline__ void level_reduce(const LevelSums &s, int32_t block) {
@@ -85,15 +86,20 @@ __device__ __forceinline__ void level_reduce(const LevelSums &s, int32_t block) 
     const int32_t per = (chunks + 7) / 8, c0 = w * per, c1 = min(c0 + per, chunks);
     double a = 0.0, b = 0.0;
     if (j < n) {
-        for (int32_t c = c0; c < c1; c += 10) {
-            float pa[10], pb[10];
+        int32_t c = c0;
+        for (; c + 8 <= c1; c += 8) {
+            float pa[8], pb[8];
 #pragma unroll
-            for (int q = 0; q < 10; ++q) {
-                pa[q] = c + q < c1 ? s.part_imp[(int64_t)(c + q) * n + j] : 0.0f;
-                pb[q] = c + q < c1 ? s.part_load[(int64_t)(c + q) * n + j] : 0.0f;
+            for (int q = 0; q < 8; ++q) {
+                pa[q] = s.part_imp[(int64_t)(c + q) * n + j];
+                pb[q] = s.part_load[(int64_t)(c + q) * n + j];
             }
 #pragma unroll
-            for (int q = 0; q < 10; ++q) { a += (double)pa[q]; b += (double)pb[q]; }
+            for (int q = 0; q < 8; ++q) { a += (double)pa[q]; b += (double)pb[q]; }
+        }
+        for (; c < c1; ++c) {
+            a += (double)s.part_imp[(int64_t)c * n + j];
+            b += (double)s.part_load[(int64_t)c * n + j];
         }
     }
     red[0][w][lane] = a;
