@@ -405,12 +405,25 @@ __device__ __forceinline__ void epilogue_box(const GemmParams &p, int lane, cons
                 dst = (col < p.split_n ? p.out_f32 + col : p.out2 + (col - p.split_n)) + my_piece * 4;
                 pitch = p.split_n;
             }
+            auto piece = [&](int row) { return *reinterpret_cast<const uint4 *>(b.box + row * 128 + ((my_piece ^ (row & 7)) << 4)); };
+            if (!p.out_rows && !p.out_words) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int row = 4 * i + my_sub;
-                if (row < b.rows_valid) {
-                    const uint4 v = *reinterpret_cast<const uint4 *>(b.box + row * 128 + ((my_piece ^ (row & 7)) << 4));
-                    float *at = dst + (p.out_rows ? (int64_t)p.out_rows[b.row0 + row] : b.row0 + row) * pitch;
+                for (int i = 0; i < 8; ++i) {
+                    const int row = 4 * i + my_sub;
+                    if (row < b.rows_valid) *reinterpret_cast<uint4 *>(dst + (b.row0 + row) * pitch) = piece(row);
+                }
+            } else {
+                int32_t to[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int64_t row = b.row0 + 4 * i + my_sub;
+                    to[i] = 4 * i + my_sub >= b.rows_valid ? -1 : p.out_rows ? p.out_rows[row] : (int32_t)row;
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    if (to[i] < 0) continue;
+                    const uint4 v = piece(4 * i + my_sub);
+                    float *at = dst + (int64_t)to[i] * pitch;
                     if (!p.out_words) {
                         *reinterpret_cast<uint4 *>(at) = v;
                     } else {
