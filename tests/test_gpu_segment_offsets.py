@@ -10,9 +10,11 @@ from paper_1701_06538_b200 import binding as B
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("T,n", [(600, 4), (4096, 2)])  # one CTA a tile, SM pairs
-def test_rows_behind_the_batch_read_as_zeros(T, n):
-    d, h, over = 1024, 1024, 5
+@pytest.mark.parametrize("T,n,d,h", [(600, 4, 1024, 1024),    # one CTA a tile
+                                     (4096, 2, 1024, 1024),   # SM pairs
+                                     (1000, 300, 64, 4096)])  # one CTA a tile, segments with maps of their own
+def test_rows_behind_the_batch_read_as_zeros(T, n, d, h):
+    over = 5
     cfg = B.make_config(T, d, h, n, 1, "bf16", 0.1, 0.1)
     g = torch.Generator(device="cuda")
     g.manual_seed(3)
