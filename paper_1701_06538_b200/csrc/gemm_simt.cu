@@ -67,10 +67,12 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), TM * TN >= 64 ? 3 : TM 
     constexpr int NTX = BN / TN, NTY = BM / TM, NT = NTX * NTY;
     // An operand whose contraction index is the contiguous one is stored transposed, four elements of a quad in four rows of the
     // tile: the lanes of a warp hold BK / 4 quads of 128 / BK tile rows, and without a swizzle those stores met in a few banks (four
-    // to a bank at 32 x 32 x 32). Tile row i of step k stands at i ^ swizzle(k). (Not in the larger tiles: two to a bank there, and
-    // the reads of every step would pay for it, 38 -> 41 us at 4170 x 512 x 256.)
+    // to a bank at 32 x 32 x 32). Tile row i of step k stands at i ^ swizzle(k). The reads of every step pay for it, so only where both
+    // operands are stored that way, and not in the larger tiles, where two stores meet (the backward products of 256 experts x 16 rows
+    // of 256 x 256 floats 229 us, without 240; but with one such operand a gate of 24 x 512 x 64 12.1, without 11.3, and
+    // 4170 x 512 x 256 in larger tiles 41, 38).
     constexpr int LDA = BM + 4, LDB = BN + 4;
-    constexpr bool SWZ = BM * BN <= 32 * 32;
+    constexpr bool SWZ = BM * BN <= 32 * 32 && AK && !BJ;
     constexpr int SWZ_UNIT = BK <= 32 ? 128 / BK : 4, SWZ_K = BK <= 32 ? 4 : 8;
     auto swizzle_a = [](int k) { return SWZ && AK ? (k / SWZ_K % ((BM < 32 ? BM : 32) / SWZ_UNIT)) * SWZ_UNIT : 0; };
     auto swizzle_b = [](int k) { return SWZ && !BJ ? (k / SWZ_K % ((BN < 32 ? BN : 32) / SWZ_UNIT)) * SWZ_UNIT : 0; };

@@ -186,13 +186,14 @@ int32_t launch_dispatch_bwd(const void *dxs, int32_t act, const int32_t *inv_per
                             const struct BackwardTail *tail = nullptr);
 // The segment of tile `b` of a ragged product {segment, first row, segment end, tile inside the segment}, or segment -1 behind the last
 // tile, looked up by the whole block (barriers): every thread looks at its share of the segments, so that a block waits for
-// one round of loads (a binary search over the prefix waits for one per step, 2 of the 5 us of a block with little to do). With
-// thousands of segments the search is less work (12288 blocks, 4096 segments: 80 us, this way 96). sh: one int4
+// one round of loads (a binary search over the prefix waits for one per step, 2 of the 5 us of a block with little to do). With more
+// than four segments a thread the search is less work (12288 blocks of 256 threads, 4096 segments: 80 us, this way 96; the float
+// products of 24 rows of 64 in 480 segments, 64 threads a block: 101, 122; with 256 segments of 500 rows 77, this way 74). sh: one int4
 __device__ __forceinline__ int4 segment_of_tile(const int32_t *__restrict__ tile_prefix, const int32_t *__restrict__ offsets, int32_t nseg,
                                                 int32_t b, int4 *sh) {
     if (threadIdx.x == 0) *sh = make_int4(-1, 0, 0, 0);
     __syncthreads();
-    if (nseg > 1024) {
+    if (nseg > 4 * (int32_t)blockDim.x) {
         if (threadIdx.x == 0 && b < tile_prefix[nseg]) {
             int32_t lo = 0, hi = nseg;
             while (hi - lo > 1) {
