@@ -23,17 +23,21 @@ struct Beside {
 //                                 the threshold is another entry's noisy logit:
 //                                 dH[j_(k+1)] -= sum_{kept j} q_j ; dH[j_k] -= sum_{other j} q_j
 //   H = c + eps * sigma:          dc += dH ; dsigma += eps * dH ; dr = dsigma * sigmoid(r)
-template <int NV>  // columns per lane kept in registers (n <= 32 * NV); 0: any n, recompute in a second pass
+template <int NV, typename Ride>  // NV: columns per lane kept in registers (n <= 32 * NV); 0: any n, recompute in a second pass
 __global__ void __launch_bounds__(256) gate_logit_grads_kernel(
     const float *__restrict__ noise, const float *__restrict__ clean, const float *__restrict__ raw,
     const int32_t *__restrict__ idx, const float *__restrict__ gates, const float *__restrict__ kth_vals,
     const int32_t *__restrict__ kth_idx, const float *__restrict__ dgates, const float *__restrict__ dload,
     const int32_t *__restrict__ dload_row_group, int64_t rows, int32_t n, int32_t k, float *__restrict__ dlogit,
-    bf16 *__restrict__ dsplit, const int32_t *__restrict__ split_row_index, const __grid_constant__ Beside beside) {
+    bf16 *__restrict__ dsplit, const int32_t *__restrict__ split_row_index, const __grid_constant__ Ride beside) {
     wait_previous_kernel();
-    if ((int32_t)blockIdx.x < beside.blocks) return beside.run(blockIdx.x);
+    int32_t block = blockIdx.x;
+    if constexpr (rides<Ride>()) {
+        if (block < beside.blocks) return beside.run(block);
+        block -= beside.blocks;
+    }
     const int lane = threadIdx.x & 31;
-    const int64_t row = (int64_t)(blockIdx.x - beside.blocks) * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int64_t row = (int64_t)block * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (row >= rows) return;
     int32_t sel_idx[MOE_MAX_K];
     float sel_dh[MOE_MAX_K];
@@ -152,17 +156,21 @@ __global__ void __launch_bounds__(256) gate_logit_grads_kernel(
 // row is read with 8-byte loads and the six bf16 terms of a pair leave as 4-byte stores (half the memory instructions),
 // and only the first KS slots are compared (KS >= k). LANES lanes take a row, NVP pairs each: what a row costs besides its columns
 // (its slots' gates, two sums over its lanes) is most of a row of 64 when a warp has one row.
-template <int LANES, int NVP, int KS>  // n <= 2 * LANES * NVP
+template <int LANES, int NVP, int KS, typename Ride>  // n <= 2 * LANES * NVP
 __global__ void __launch_bounds__(256) gate_logit_grads_pairs_kernel(
     const float *__restrict__ noise, const float *__restrict__ clean, const float *__restrict__ raw,
     const int32_t *__restrict__ idx, const float *__restrict__ gates, const float *__restrict__ kth_vals,
     const int32_t *__restrict__ kth_idx, const float *__restrict__ dgates, const float *__restrict__ dload,
     const int32_t *__restrict__ dload_row_group, int64_t rows, int32_t n, int32_t k, bf16 *__restrict__ dsplit,
-    const int32_t *__restrict__ split_row_index, const __grid_constant__ Beside beside) {
+    const int32_t *__restrict__ split_row_index, const __grid_constant__ Ride beside) {
     wait_previous_kernel();
-    if ((int32_t)blockIdx.x < beside.blocks) return beside.run(blockIdx.x);
+    int32_t block = blockIdx.x;
+    if constexpr (rides<Ride>()) {
+        if (block < beside.blocks) return beside.run(block);
+        block -= beside.blocks;
+    }
     const int lane = threadIdx.x & (LANES - 1);
-    const int64_t place = (int64_t)(blockIdx.x - beside.blocks) * (256 / LANES) + threadIdx.x / LANES;
+    const int64_t place = (int64_t)block * (256 / LANES) + threadIdx.x / LANES;
     const bool live = place < rows;
     const int64_t row = live ? place : rows - 1;  // (the lanes behind the last row stay for the sums over a warp's lanes)
     int32_t sel_idx[KS];
@@ -259,12 +267,13 @@ int32_t launch_gate_logit_grads(const float *noise, const float *clean, const fl
                                 int64_t rows, int32_t n, int32_t k, float *dlogit, void *dsplit,
                                 const int32_t *split_row_index, cudaStream_t st, const ColumnSums *sums) {
     if (rows == 0) return sums ? launch_segment_colsum(*sums, false, st) : MOE_OK;
-    Beside beside = {};
-    if (sums) beside = {*sums, (int32_t)(column_tiles(*sums) * column_slabs(*sums)), (int32_t)column_slabs(*sums)};
-    const unsigned grid = (unsigned)(cdiv(rows, 8) + beside.blocks);
-    if (dsplit && n % 32 == 0 && n <= 256) {  // the tensor-core path: paired columns
+    const int64_t more = sums ? column_tiles(*sums) * column_slabs(*sums) : 0;
+    const unsigned grid = (unsigned)(cdiv(rows, 8) + more);
+    auto run = [&](const auto &beside) -> int32_t {
+        using Ride = std::decay_t<decltype(beside)>;
+        if (dsplit && n % 32 == 0 && n <= 256) {  // the tensor-core path: paired columns
 #define MOE_LOGIT_PAIRS_KS(LANES, NVP, KS)                                                                               \
-    launch_kernel((gate_logit_grads_pairs_kernel<LANES, NVP, KS>), (unsigned)(cdiv(rows, 256 / LANES) + beside.blocks), 256, 0, st, \
+    launch_kernel((gate_logit_grads_pairs_kernel<LANES, NVP, KS, Ride>), (unsigned)(cdiv(rows, 256 / LANES) + more), 256, 0, st, \
                   noise, clean, raw, idx, gates, kth_vals, kth_idx, dgates, dload, dload_row_group, rows, n, k, (bf16 *)dsplit,      \
                   split_row_index, beside)
 #define MOE_LOGIT_PAIRS(LANES, NVP)                         \
@@ -273,34 +282,36 @@ int32_t launch_gate_logit_grads(const float *noise, const float *clean, const fl
         else if (k <= 4) MOE_LOGIT_PAIRS_KS(LANES, NVP, 4); \
         else MOE_LOGIT_PAIRS_KS(LANES, NVP, MOE_MAX_K);     \
     } while (0)
-        // four pairs a lane where that still leaves every SM four blocks of 32 or 16 rows
-        const bool many = rows >= (n <= 64 ? 32 : 16) * 4 * (int64_t)148;
-        if (n <= 64) {
-            if (many) MOE_LOGIT_PAIRS(8, 4);
-            else MOE_LOGIT_PAIRS(32, 1);
-        } else if (n <= 128) {
-            if (many) MOE_LOGIT_PAIRS(16, 4);
-            else MOE_LOGIT_PAIRS(32, 2);
-        } else {
-            MOE_LOGIT_PAIRS(32, 4);
-        }
+            // four pairs a lane where that still leaves every SM four blocks of 32 or 16 rows
+            const bool many = rows >= (n <= 64 ? 32 : 16) * 4 * (int64_t)148;
+            if (n <= 64) {
+                if (many) MOE_LOGIT_PAIRS(8, 4);
+                else MOE_LOGIT_PAIRS(32, 1);
+            } else if (n <= 128) {
+                if (many) MOE_LOGIT_PAIRS(16, 4);
+                else MOE_LOGIT_PAIRS(32, 2);
+            } else {
+                MOE_LOGIT_PAIRS(32, 4);
+            }
 #undef MOE_LOGIT_PAIRS
 #undef MOE_LOGIT_PAIRS_KS
-        MOE_LAUNCHED();
-        return MOE_OK;
-    }
+            MOE_LAUNCHED();
+            return MOE_OK;
+        }
 #define MOE_LOGIT_GRADS(NV)                                                                                          \
-    launch_kernel(gate_logit_grads_kernel<NV>, grid, 256, 0, st, noise, clean, raw, idx, gates, kth_vals, kth_idx, dgates, dload, \
+    launch_kernel((gate_logit_grads_kernel<NV, Ride>), grid, 256, 0, st, noise, clean, raw, idx, gates, kth_vals, kth_idx, dgates, dload, \
                                                       dload_row_group, rows, n, k, dlogit, (bf16 *)dsplit,      \
                                                       split_row_index, beside)
-    if (n <= 32) MOE_LOGIT_GRADS(1);
-    else if (n <= 64) MOE_LOGIT_GRADS(2);
-    else if (n <= 128) MOE_LOGIT_GRADS(4);
-    else if (n <= 256) MOE_LOGIT_GRADS(8);
-    else MOE_LOGIT_GRADS(0);
+        if (n <= 32) MOE_LOGIT_GRADS(1);
+        else if (n <= 64) MOE_LOGIT_GRADS(2);
+        else if (n <= 128) MOE_LOGIT_GRADS(4);
+        else if (n <= 256) MOE_LOGIT_GRADS(8);
+        else MOE_LOGIT_GRADS(0);
 #undef MOE_LOGIT_GRADS
-    MOE_LAUNCHED();
-    return MOE_OK;
+        MOE_LAUNCHED();
+        return MOE_OK;
+    };
+    return sums ? run(Beside{*sums, (int32_t)more, (int32_t)column_slabs(*sums)}) : run(Nothing{});
 }
 
 MOE_BOUNDS_READER(bounds_violations_gate_bwd)

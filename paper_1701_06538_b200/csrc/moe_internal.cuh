@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
 #include <utility>
 
 #include "moe.h"
@@ -88,6 +89,11 @@ static inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 static inline int64_t imin(int64_t a, int64_t b) { return a < b ? a : b; }
 static inline int64_t imax(int64_t a, int64_t b) { return a > b ? a : b; }
 static inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 31) == 0; }  // 32 bytes: the epilogues use 256-bit stores
+
+// In the place of work that rides along with a launch, where none does: the parameters and registers of the work cost the launch's own
+// (moe_combine of 32768 x 512, one slot: 14.1 us with them, 9.3 without; 1000 x 512: 1.67, 1.55)
+struct Nothing {};
+template <typename Ride> constexpr bool rides() { return !std::is_same<Ride, Nothing>::value; }
 
 // Carves 256-byte aligned pieces out of a workspace. With base == nullptr it only measures,
 // so the size queries and the calls that use the workspace run the same code.

@@ -2,8 +2,6 @@
 // gate-weighted combine (Eq. 1) and their adjoints. All of it is HBM streaming: rows are moved
 // with 16-byte vector accesses, every token row is read once and written k times (dispatch) or
 // gathered k times and written once (combine).
-#include <string.h>
-
 #include "losses.cuh"
 #include "plan.cuh"
 #include "sums.cuh"
@@ -181,18 +179,17 @@ __device__ __forceinline__ int32_t slot_expert(const int32_t *topk_idx, int64_t 
 // together; no other launch) or from the chunks' histograms. Blocks behind the chunks' do the pieces of the
 // segment plan on the offsets they have found, which is then no launch of its own either.
 constexpr int INDEX_EXPERTS_MAX = 1024, INDEX_SCAN_MAX = 8;
-inline int64_t index_front_ints(int32_t n) { return 8 * n > plan_shared_ints(0) ? 8 * n : plan_shared_ints(0); }
-template <bool SCAN>
+inline int64_t index_front_ints(int32_t n, bool plan) { return plan && plan_shared_ints(0) > 8 * n ? plan_shared_ints(0) : 8 * n; }
+template <bool SCAN, typename Plan>
 __global__ void __launch_bounds__(1024) dispatch_index_kernel(const int32_t *__restrict__ topk_idx, int64_t R, int32_t n,
                                                               const int32_t *__restrict__ chunk_table, int32_t nchunks, int32_t front_ints,
                                                               int32_t *__restrict__ counts, int32_t *__restrict__ offsets,
                                                               int32_t *__restrict__ perm, int32_t *__restrict__ inv_perm,
-                                                              const __grid_constant__ PlanArgs plan) {
+                                                              const __grid_constant__ Plan plan) {
     wait_previous_kernel();
     extern __shared__ __align__(128) int32_t index_sh[];
     __shared__ int32_t sh[32];
     __shared__ int32_t part_total[1024], part_before[1024];
-    __shared__ double moments[32];
     int32_t *front = on_128_bytes(index_sh);  // the experts' rows of bytes, or the scratch of the plan
     int32_t *cursor = front + front_ints;     // next sorted row of each expert for this chunk; plan: the offsets, n + 1
     uint4 *warp_counts = reinterpret_cast<uint4 *>(front);
@@ -241,12 +238,15 @@ __global__ void __launch_bounds__(1024) dispatch_index_kernel(const int32_t *__r
     }
     int32_t all;
     const int32_t excl = block_scan_1024(total, sh, &all);
-    if (!ranks) {
-        if (tid < n) cursor[tid] = excl;
-        if (tid == 0) cursor[n] = all;
-        __syncthreads();
-        plan_piece(plan, blockIdx.x - nchunks, cursor, front, sh, moments);
-        return;
+    if constexpr (rides<Plan>()) {
+        __shared__ double moments[32];
+        if (!ranks) {
+            if (tid < n) cursor[tid] = excl;
+            if (tid == 0) cursor[n] = all;
+            __syncthreads();
+            plan_piece(plan, blockIdx.x - nchunks, cursor, front, sh, moments);
+            return;
+        }
     }
     if (tid < n) {
         cursor[tid] = excl + before;
@@ -383,17 +383,20 @@ int32_t launch_dispatch_index(const int32_t *topk_idx, int64_t R, int32_t n, int
         MOE_LAUNCHED();
     }
     if (scan || few) {
-        PlanArgs none;
-        if (!plan) memset(&none, 0, sizeof(none));
-        const int32_t front = (int32_t)index_front_ints(n);
+        const int32_t front = (int32_t)index_front_ints(n, plan != nullptr);
         const unsigned grid = (unsigned)(nchunks + (plan ? plan_blocks(*plan) : 0));
         const size_t shared = 128 + sizeof(int32_t) * (front + n + 1);  // at most 36 KiB
-        if (scan)
-            launch_kernel(dispatch_index_kernel<true>, grid, 1024, shared, st, topk_idx, R, n, nullptr, nchunks, front, counts, offsets, perm,
-                          inv_perm, plan ? *plan : none);
-        else
-            launch_kernel(dispatch_index_kernel<false>, grid, 1024, shared, st, topk_idx, R, n, scratch, nchunks, front, counts, offsets, perm,
-                          inv_perm, plan ? *plan : none);
+        auto run = [&](const auto &ride) {
+            using Plan = std::decay_t<decltype(ride)>;
+            if (scan)
+                launch_kernel((dispatch_index_kernel<true, Plan>), grid, 1024, shared, st, topk_idx, R, n, nullptr, nchunks, front, counts,
+                              offsets, perm, inv_perm, ride);
+            else
+                launch_kernel((dispatch_index_kernel<false, Plan>), grid, 1024, shared, st, topk_idx, R, n, scratch, nchunks, front, counts,
+                              offsets, perm, inv_perm, ride);
+        };
+        if (plan) run(*plan);
+        else run(Nothing{});
         MOE_LAUNCHED();
         if (planned) *planned = plan != nullptr;
         return MOE_OK;
@@ -567,7 +570,8 @@ template <typename XT> struct Vec16 {
 template <typename XT, int NV>
 __global__ void __launch_bounds__(256) dispatch_rows_kernel(const XT *__restrict__ x, int64_t T, int32_t k,
                                                             int32_t d, const int32_t *__restrict__ inv_perm,
-                                                            XT *__restrict__ xs, const __grid_constant__ LevelSums sums) {
+                                                            XT *__restrict__ xs,
+                                                            const __grid_constant__ std::conditional_t<(NV > 0), LevelSums, Nothing> sums) {
     wait_previous_kernel();
     constexpr int VN = 16 / sizeof(XT);
     int32_t block = blockIdx.x, blocks = gridDim.x;
@@ -604,20 +608,19 @@ __global__ void __launch_bounds__(256) dispatch_rows_kernel(const XT *__restrict
 int32_t launch_dispatch_rows(const void *x, int32_t act, int64_t T, int32_t k, int32_t d, const int32_t *inv_perm,
                              void *xs, cudaStream_t st, const LevelSums *sums) {
     if (T == 0) return MOE_OK;
-    const LevelSums job = sums ? *sums : LevelSums{};
     const unsigned grid = (unsigned)(imin(cdiv(T, 8), 148 * 16) + (sums ? sums->chunks : 0));
-#define MOE_ROWS(NV)                                                                                                          \
+#define MOE_ROWS(NV, JOB)                                                                                                      \
     do {                                                                                                                      \
         if (act == MOE_BF16)                                                                                                  \
-            launch_kernel((dispatch_rows_kernel<bf16, NV>), grid, 256, 0, st, (const bf16 *)x, T, k, d, inv_perm, (bf16 *)xs, job); \
+            launch_kernel((dispatch_rows_kernel<bf16, NV>), grid, 256, 0, st, (const bf16 *)x, T, k, d, inv_perm, (bf16 *)xs, JOB); \
         else                                                                                                                  \
-            launch_kernel((dispatch_rows_kernel<float, NV>), grid, 256, 0, st, (const float *)x, T, k, d, inv_perm, (float *)xs, job); \
+            launch_kernel((dispatch_rows_kernel<float, NV>), grid, 256, 0, st, (const float *)x, T, k, d, inv_perm, (float *)xs, JOB); \
     } while (0)
-    if (!sums) MOE_ROWS(0);
-    else if (sums->n <= 32) MOE_ROWS(1);
-    else if (sums->n <= 64) MOE_ROWS(2);
-    else if (sums->n <= 128) MOE_ROWS(4);
-    else if (sums->n <= LEVEL_RIDE_MAX) MOE_ROWS(8);
+    if (!sums) MOE_ROWS(0, Nothing{});
+    else if (sums->n <= 32) MOE_ROWS(1, *sums);
+    else if (sums->n <= 64) MOE_ROWS(2, *sums);
+    else if (sums->n <= 128) MOE_ROWS(4, *sums);
+    else if (sums->n <= LEVEL_RIDE_MAX) MOE_ROWS(8, *sums);
     else return MOE_ERR_INVALID_ARG;
 #undef MOE_ROWS
     MOE_LAUNCHED();
@@ -646,18 +649,21 @@ __device__ __forceinline__ float logistic(float y) { return __fdividef(1.0f, 1.0
 
 // y[t] = sum_s gates[t,s] * ys[inv_perm[t*k+s]]   (Eq. 1), float sum in slot order.
 // LAYER (Appendix C): out[t] = x[t] + keep[t] * sigmoid(y[t]) * keep_scale, y itself is not stored.
-// sums.chunks > 0: the first blocks complete the loss sums, 32 columns each.
-template <typename XT, int KT, int VB, bool LAYER>
+// Sums = LevelSums: the first blocks complete the loss sums, 32 columns each.
+template <typename XT, int KT, int VB, bool LAYER, typename Sums>
 __global__ void __launch_bounds__(256, LAYER ? 3 : 1) combine_kernel(const XT *__restrict__ ys, const float *__restrict__ gates,
                                                       const int32_t *__restrict__ inv_perm, int64_t T, int32_t k,
                                                       int32_t d, XT *__restrict__ y, const XT *__restrict__ xres,
                                                       const uint8_t *__restrict__ keep, float keep_scale,
-                                                      const __grid_constant__ LevelSums sums) {
+                                                      const __grid_constant__ Sums sums) {
     wait_previous_kernel();
-    const int32_t reduces = sums.chunks > 0 ? (sums.n + 31) / 32 : 0;
-    if ((int32_t)blockIdx.x < reduces) {
-        level_reduce(sums, blockIdx.x);
-        return;
+    int32_t reduces = 0;
+    if constexpr (rides<Sums>()) {
+        reduces = (sums.n + 31) / 32;
+        if ((int32_t)blockIdx.x < reduces) {
+            level_reduce(sums, blockIdx.x);
+            return;
+        }
     }
     constexpr int VN = 16 / sizeof(XT);
     const int lane = threadIdx.x & 31;
@@ -719,23 +725,26 @@ int32_t launch_combine(const void *ys, int32_t act, const float *gates, const in
                        int32_t k, int32_t d, void *y, cudaStream_t st, const void *xres, const uint8_t *keep,
                        float keep_scale, const LevelSums *sums) {
     if (T == 0) return MOE_OK;
-    const LevelSums job = sums ? *sums : LevelSums{};
     const unsigned grid = (unsigned)(imin(cdiv(T, 8), 148 * 16) + (sums ? cdiv(sums->n, 32) : 0));
+    auto run = [&](const auto &job) -> int32_t {
+        using Sums = std::decay_t<decltype(job)>;
 #define MOE_CALL_L(KT, VB, L)                                                                                         \
     if (act == MOE_BF16)                                                                                              \
-        launch_kernel((combine_kernel<bf16, KT, VB, L>), grid, 256, 0, st, (const bf16 *)ys, gates, inv_perm, T, k, d, (bf16 *)y,  \
+        launch_kernel((combine_kernel<bf16, KT, VB, L, Sums>), grid, 256, 0, st, (const bf16 *)ys, gates, inv_perm, T, k, d, (bf16 *)y,  \
                                                               (const bf16 *)xres, keep, keep_scale, job);                  \
     else                                                                                                              \
-        launch_kernel((combine_kernel<float, KT, VB, L>), grid, 256, 0, st, (const float *)ys, gates, inv_perm, T, k, d, (float *)y, \
+        launch_kernel((combine_kernel<float, KT, VB, L, Sums>), grid, 256, 0, st, (const float *)ys, gates, inv_perm, T, k, d, (float *)y, \
                                                                (const float *)xres, keep, keep_scale, job)
 #define MOE_CALL(KT, VB)                     \
     if (keep) { MOE_CALL_L(KT, VB, true); }  \
     else { MOE_CALL_L(KT, VB, false); }
-    MOE_DISPATCH_KT(k, MOE_CALL);
+        MOE_DISPATCH_KT(k, MOE_CALL);
 #undef MOE_CALL
 #undef MOE_CALL_L
-    MOE_LAUNCHED();
-    return MOE_OK;
+        MOE_LAUNCHED();
+        return MOE_OK;
+    };
+    return sums ? run(*sums) : run(Nothing{});
 }
 
 // dgates[t,s] = <dy[t], ys[row]>,  dys[row] = gates[t,s] * dy[t], with dy = dY, or (LAYER: adjoint of the sigmoid and
@@ -871,15 +880,18 @@ int32_t launch_combine_bwd(const void *dY, const void *ys, int32_t act, const fl
 // reaches the layer input through the residual connection); float output, or rounded to the act type.
 // SEC: add[t] is the primary gate's part of the hierarchical layer, to which the rows of the token's sec.k1 secondary gates are added
 // (row sec.perm[t * k1 + s1], or t * k1 + s1 itself), instead of in a pass of their own over float rows as wide.
-template <typename XT, int KT, int VB, bool SEC>
+// Tail = BackwardTail: sums that earlier launches have left, by the blocks behind the rows'.
+template <typename XT, int KT, int VB, bool SEC, typename Tail>
 __global__ void __launch_bounds__(256) dispatch_bwd_kernel(const XT *__restrict__ dxs,
                                                            const int32_t *__restrict__ inv_perm, int64_t T,
                                                            int32_t k, int32_t d, const float *add,
                                                            float *out_f32, XT *__restrict__ out_act,
                                                            const XT *__restrict__ add_act, const SecondaryRows sec,
-                                                           const int32_t row_blocks, const __grid_constant__ BackwardTail tail) {
+                                                           const int32_t row_blocks, const __grid_constant__ Tail tail) {
     wait_previous_kernel();
-    if ((int32_t)blockIdx.x >= row_blocks) return run_backward_tail(tail, blockIdx.x - row_blocks);
+    if constexpr (rides<Tail>()) {
+        if ((int32_t)blockIdx.x >= row_blocks) return run_backward_tail(tail, blockIdx.x - row_blocks);
+    }
     constexpr int VN = 16 / sizeof(XT);
     const int lane = threadIdx.x & 31;
     const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -992,21 +1004,25 @@ int32_t launch_dispatch_bwd(const void *dxs, int32_t act, const int32_t *inv_per
     }
     const int32_t row_blocks = (int32_t)imin(cdiv(T, 8), 148 * 16);
     const unsigned grid = (unsigned)(row_blocks + tail.total());
+    auto run = [&](const auto &job) -> int32_t {
+        using Tail = std::decay_t<decltype(job)>;
 #define MOE_CALL_S(KT, VB, SEC)                                                                                       \
     if (act == MOE_BF16)                                                                                              \
-        launch_kernel((dispatch_bwd_kernel<bf16, KT, VB, SEC>), grid, 256, 0, st, (const bf16 *)dxs, inv_perm, T, k, d, add_f32, out_f32, \
-                                                                 (bf16 *)out_act, (const bf16 *)add_act, sec, row_blocks, tail);         \
+        launch_kernel((dispatch_bwd_kernel<bf16, KT, VB, SEC, Tail>), grid, 256, 0, st, (const bf16 *)dxs, inv_perm, T, k, d, add_f32, out_f32, \
+                                                                 (bf16 *)out_act, (const bf16 *)add_act, sec, row_blocks, job);         \
     else                                                                                                              \
-        launch_kernel((dispatch_bwd_kernel<float, KT, VB, SEC>), grid, 256, 0, st, (const float *)dxs, inv_perm, T, k, d, add_f32,  \
-                                                                  out_f32, (float *)out_act, (const float *)add_act, sec, row_blocks, tail)
+        launch_kernel((dispatch_bwd_kernel<float, KT, VB, SEC, Tail>), grid, 256, 0, st, (const float *)dxs, inv_perm, T, k, d, add_f32,  \
+                                                                  out_f32, (float *)out_act, (const float *)add_act, sec, row_blocks, job)
 #define MOE_CALL(KT, VB)                           \
     if (sec.rows) { MOE_CALL_S(KT, VB, true); }    \
     else { MOE_CALL_S(KT, VB, false); }
-    MOE_DISPATCH_KT(k, MOE_CALL);
+        MOE_DISPATCH_KT(k, MOE_CALL);
 #undef MOE_CALL
 #undef MOE_CALL_S
-    MOE_LAUNCHED();
-    return MOE_OK;
+        MOE_LAUNCHED();
+        return MOE_OK;
+    };
+    return tail.total() > 0 ? run(tail) : run(Nothing{});
 }
 
 MOE_BOUNDS_READER(bounds_violations_route)
