@@ -3,7 +3,7 @@
 // weight matrix only the running row-wise and column-wise averages of the squared gradient are kept, and the matrix of
 // estimators is taken to be their outer product divided by the mean of the row vector. Biases (vectors) keep a full
 // second-moment estimate. All of it is HBM streaming: the gradient is read twice (averages, update), the parameters
-// are read and written once. Sums are taken in fixed orders (no floating-point atomics): two runs agree bit for bit.
+// are read and written once (small matrices: the second look finds the gradient in L2). Sums are taken in fixed orders (no floating-point atomics): two runs agree bit for bit.
 #include <math_constants.h>
 
 #include "moe_internal.cuh"
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(256) adam_update_flat_kernel(XT *__restrict__ 
 // slab's rows; strips and row shares are dealt to the 16 warps.
 // ------------------------------------------------------------------------------------------
 constexpr int FUSED_THREADS = 512, FUSED_WARPS = FUSED_THREADS / 32;
-constexpr int64_t FUSED_MATRIX_BYTES = 4 << 20, FUSED_SLAB_BYTES = 256 << 10;
+constexpr int64_t FUSED_MATRIX_BYTES = 4 << 20, FUSED_SLAB_BYTES = 256 << 10, FUSED_EXPERT_BYTES = 112 << 10;
 struct FusedMatrix {
     void *W;
     const void *g;
@@ -519,6 +519,9 @@ bool plan_fused(FusedAdam &a, int32_t n, int32_t d, int32_t h, size_t *smem) {
     if (bytes > FUSED_MATRIX_BYTES) return false;
     int32_t C = 1;  // slabs as large as that, smaller ones where there are few matrices
     while (C < 8 && (bytes > C * FUSED_SLAB_BYTES || (2 * (int64_t)n * C < 2 * 148 && bytes > C * (int64_t)32768))) C <<= 1;
+    // Few large matrices: a slab's time is its CTA's, and the kernels of their own spread over more of the chip. A step, us, in one launch /
+    // apart (bf16): 4 MiB matrices of 1 expert 46 / 34, 2 47 / 37, 4 50 / 48; 2.25 MiB 1 33 / 29, 2 34 / 32, 3 and more faster in one
+    if (bytes > C * FUSED_SLAB_BYTES && bytes > C * n * FUSED_EXPERT_BYTES) return false;
     a.n = n; a.cluster = C;
     const int32_t shape[2][2] = {{d, h}, {h, d}};
     int64_t floats = 0;
