@@ -196,14 +196,18 @@ __global__ void __launch_bounds__(1024) dispatch_index_kernel(const int32_t *__r
     const int tid = threadIdx.x, lane = tid & 31;
     const bool ranks = (int32_t)blockIdx.x < nchunks;
     const int64_t p = (int64_t)blockIdx.x * CH + tid;
-    int32_t e = -1;
-    if (ranks) {
-        e = slot_expert(topk_idx, p, R, n);
-        MOE_BOUNDS_NOTE(p >= R || e >= 0);
+    const bool one = SCAN && nchunks == 1;  // the places in the chunk give the counts as well, to the plan's blocks too
+    int32_t e = -1, place = 0;
+    if (ranks || one) {
+        e = slot_expert(topk_idx, one ? tid : p, R, n);
+        MOE_BOUNDS_NOTE((one ? tid : p) >= R || e >= 0);
         for (int32_t q = tid; q < 2 * n; q += 1024) warp_counts[q] = make_uint4(0u, 0u, 0u, 0u);
     }
     int32_t total = 0, before = 0;
-    if (SCAN) {
+    if (one) {
+        place = rank_in_chunk(e, warp_counts);
+        if (tid < n) total = bytes_before(warp_counts + 2 * tid, 32);
+    } else if (SCAN) {
         part_total[tid] = 0;
         part_before[tid] = 0;
         __syncthreads();
@@ -253,7 +257,8 @@ __global__ void __launch_bounds__(1024) dispatch_index_kernel(const int32_t *__r
         if (blockIdx.x == 0) { counts[tid] = total; offsets[tid] = excl; }
     }
     if (tid == 0 && blockIdx.x == 0) offsets[n] = all;
-    const int32_t place = rank_in_chunk(e, warp_counts);  // (its barriers: the cursors are written)
+    if (one) __syncthreads();  // the cursors are written
+    else place = rank_in_chunk(e, warp_counts);  // (by its barriers)
     place_slot(e, e >= 0 ? cursor[e] + place : 0, p, R, perm, inv_perm);
 }
 
