@@ -1521,6 +1521,8 @@ template <int KIND, int EPI> int32_t launch_as(const CUtensorMap &tmA, const CUt
     MOE_LAUNCHED();
     return MOE_OK;
 }
+// one or two K blocks in the average segment of a weight gradient
+static bool short_segments(int64_t R, int32_t nseg) { return R < 128 * (int64_t)nseg; }
 template <int KIND> int32_t launch(const CUtensorMap &tmA, const CUtensorMap &tmB, const GemmParams &p_in,
                                    int64_t max_tiles, cudaStream_t st, const CUtensorMap *tmO = nullptr) {
     GemmParams p = p_in;
@@ -1538,7 +1540,7 @@ template <int KIND> int32_t launch(const CUtensorMap &tmA, const CUtensorMap &tm
             if (p.mask) return launch_as<KIND, EPI_MASK>(tmA, tmB, p, grid, st, out);
         }
         if constexpr (KIND == WGRAD) {
-            if (!p.seg_a) return launch_as<KIND, EPI_TWO_BOXES>(tmA, tmB, p, grid, st, out);  // short segments, see tc_wgrad_gemm
+            if (short_segments(p.R, p.nseg)) return launch_as<KIND, EPI_TWO_BOXES>(tmA, tmB, p, grid, st, out);
         }
         return launch_as<KIND, EPI_PLAIN>(tmA, tmB, p, grid, st, out);
     }
@@ -1630,11 +1632,16 @@ static bool use_two_cta(int64_t R, int32_t nseg, int32_t flags, int32_t cols) {
     return R / (nseg > 0 ? nseg : 1) >= 384;
 }
 
-// The last K block of a segment through the segment's own maps: each costs the loading thread a fence, so that with one or two K
-// blocks to a segment the one-CTA kernel clears the rows in shared memory instead (4096 experts x 64 rows: 1070 us, with maps 1187;
-// 256 x 78: 67, 75; but 256 x 188: 93, 82; on SM pairs, where clearing held the tensor cores up for a third of a tile,
-// 256 x 512: 192, 138)
-static bool wgrad_uses_maps(int64_t R, int32_t nseg) { return R >= 128 * (int64_t)nseg; }
+// The last K block of a segment through the segment's own maps: each costs the loading thread a fence, and the call a pass that writes
+// them, so that with one or two K blocks to a segment, or few tiles to a CTA, the one-CTA kernel clears the rows in shared memory
+// instead (4096 experts x 64 rows: 1070 us, with maps 1187; 256 x 78: 67, 75; but 256 x 188: 93, 82; a step with 20 experts
+// x 450 rows of 320 x 832, two tiles a CTA: 165, 170; on SM pairs, where clearing held the tensor cores up for a third of a
+// tile, 256 x 512: 192, 138)
+static bool wgrad_uses_maps(int64_t R, int32_t nseg, int32_t M, int32_t N, int32_t flags) {
+    const int32_t wide = M > N ? M : N, narrow = M > N ? N : M;
+    if (short_segments(R, nseg)) return false;
+    return use_two_cta(R, nseg, flags, wide) || nseg * cdiv(narrow, BM) * cdiv(wide, BN) >= 4 * (int64_t)sm_count();
+}
 // The rows of a row product behind a segment's end are read and dropped, or, through the segment's own map, not read. That saves half of
 // A's bytes where segments are half a tile, but the fence delays the tile: worth it only where a CTA has so many tiles that the
 // loads of the ones before cover it (a step with 4096 experts x 64 rows, 110 tiles a CTA: 6440 us, without 6490; but 480 x 24 rows, ten
@@ -1661,7 +1668,7 @@ int32_t tc_segment_maps(const moe_config &c, SegmentMaps *maps, const void *xs_r
         MOE_TRY(add(MAP_DYS_ROWS, dys_rows, c.d, 0));
         MOE_TRY(add(MAP_DZ_ROWS, dz_rows, c.h, 0));
     }
-    if (!wgrad_uses_maps(R, c.n)) return MOE_OK;
+    if (!wgrad_uses_maps(R, c.n, c.d, c.h, c.flags)) return MOE_OK;
     MOE_TRY(add(MAP_HID_COLS, hid_cols, c.h, 2));
     MOE_TRY(add(MAP_DYS_COLS, dys_cols, c.d, b2));
     MOE_TRY(add(MAP_XS_COLS, xs_cols, c.d, 2));
@@ -1816,7 +1823,7 @@ int32_t tc_wgrad_gemm(const void *A, const void *B, const int32_t *offsets, int3
     CUtensorMap tmA, tmB;
     GemmParams p = default_params();
     p.offsets = offsets; p.nseg = nseg; p.M = M; p.N = N; p.R = R;
-    if (wgrad_uses_maps(R, nseg)) { p.seg_a = plan.maps_of(seg_a); p.seg_b = plan.maps_of(seg_b); }
+    if (wgrad_uses_maps(R, nseg, M, N, flags)) { p.seg_a = plan.maps_of(seg_a); p.seg_b = plan.maps_of(seg_b); }
     p.out = (bf16 *)out; p.status = status;
     CUtensorMap tmO;  // the experts' matrices as one tall matrix (a 32-row box never straddles two: M is a multiple of 64)
     MOE_TRY(map_out_boxes(&tmO, out, (int64_t)nseg * M, N));
