@@ -10,7 +10,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("T,n,k", [(1, 1, 1), (31, 5, 1), (256, 8192, 4), (512, 40, 2), (1024, 33, 1), (1025, 33, 1), (5000, 1, 1),
-                                   (16384, 1024, 4), (16640, 1024, 4), (3000, 1025, 4), (40000, 256, 6), (2100, 8192, 4)])
+                                   (16384, 1024, 4), (16640, 1024, 4), (3000, 1025, 4), (40000, 256, 6), (2100, 8192, 4),
+                                   (1024, 1024, 1), (200, 1024, 5), (1000, 1025, 1), (8192, 1024, 1), (8193, 1024, 1), (2048, 7, 4)])
 def test_dispatch_index_is_a_stable_sort(T, n, k):
     g = np.random.default_rng(T + n)
     idx = (n * g.random((T, k)) ** 3).astype(np.int32)  # skewed, repeats inside a token allowed

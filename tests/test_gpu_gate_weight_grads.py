@@ -11,7 +11,8 @@ from helpers import TOL_F32, assert_close, cfg_of, dev, device_inputs, f32, host
 
 pytestmark = pytest.mark.gpu
 
-SHAPES = [(1, 256, 128), (127, 256, 128), (257, 320, 160), (1500, 512, 256), (6017, 576, 224), (9000, 256, 128), (3333, 192, 256), (3333, 512, 96)]
+# the first two: logit gradients by 8 and by 16 lanes a row, the last block of rows not full
+SHAPES = [(18949, 64, 64), (9475, 64, 96), (1, 256, 128), (127, 256, 128), (257, 320, 160), (1500, 512, 256), (6017, 576, 224), (9000, 256, 128), (3333, 192, 256), (3333, 512, 96)]
 
 
 @pytest.mark.parametrize("flags", [0, B.MOE_FLAG_TC_ONE_CTA])

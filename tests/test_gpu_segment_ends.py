@@ -10,11 +10,15 @@ pytestmark = pytest.mark.gpu
 ENDS = [0, 1, 15, 16, 17, 31, 33, 48, 63, 64, 65, 127, 128, 129, 191, 255, 256, 257, 300, 0]
 
 
-@pytest.mark.parametrize("d,h,scale,flags", [(64, 128, 1, 0), (192, 320, 1, 0), (256, 512, 5, 0), (320, 256, 5, B.MOE_FLAG_TC_ONE_CTA),
-                                             (320, 256, 5, 0)])
-def test_rows_behind_a_segment_do_not_count(d, h, scale, flags):
+@pytest.mark.parametrize("d,h,scale,flags,times", [(64, 128, 1, 0, 1), (192, 320, 1, 0, 1), (256, 512, 5, 0, 1),
+                                                   (320, 256, 5, B.MOE_FLAG_TC_ONE_CTA, 1), (320, 256, 5, 0, 1),
+                                                   # from four tiles a CTA on: weight gradients through maps of the segments
+                                                   (640, 1024, 2, B.MOE_FLAG_TC_ONE_CTA, 1),
+                                                   # from 32 tiles a CTA on, short segments: row products through them as well
+                                                   (64, 4096, 1, 0, 8)])
+def test_rows_behind_a_segment_do_not_count(d, h, scale, flags, times):
     counts = []
-    for c in ENDS:  # every segment is followed by one whose rows are infinite
+    for c in ENDS * times:  # every segment is followed by one whose rows are infinite
         counts += [c + 256 * (scale - 1) if c else 0, 3]
     n, R = len(counts), sum(counts)
     cfg = B.make_config(R, d, h, n, 1, "bf16", flags=flags)
