@@ -68,11 +68,12 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), TM * TN >= 64 ? 3 : TM 
     // An operand whose contraction index is the contiguous one is stored transposed, four elements of a quad in four rows of the
     // tile: the lanes of a warp hold BK / 4 quads of 128 / BK tile rows, and without a swizzle those stores met in a few banks (four
     // to a bank at 32 x 32 x 32). Tile row i of step k stands at i ^ swizzle(k). The reads of every step pay for it, so only where both
-    // operands are stored that way, and not in the larger tiles, where two stores meet (the backward products of 256 experts x 16 rows
-    // of 256 x 256 floats 229 us, without 240; but with one such operand a gate of 24 x 512 x 64 12.1, without 11.3, and
-    // 4170 x 512 x 256 in larger tiles 41, 38).
+    // operands are stored that way, or one of two bytes an element in 32 x 32 tiles, and not in the larger tiles, where two stores meet
+    // (the backward products of 256 experts x 16 rows of 256 x 256 floats 229 us, without 240; a whole forward call with a gate of
+    // 1019 x 512 x 512 145.0, without 146.9; but a gate of 24 x 512 x 64 12.1, without 11.3, of 4000 x 256 x 64 floats
+    // 14.1, 13.4, and 4170 x 512 x 256 in larger tiles 41, 38).
     constexpr int LDA = BM + 4, LDB = BN + 4;
-    constexpr bool SWZ = BM * BN <= 32 * 32 && AK && !BJ;
+    constexpr bool SWZ = AK && (BJ ? BM * BN == 32 * 32 && sizeof(TA) == 2 : BM * BN <= 32 * 32);
     constexpr int SWZ_UNIT = BK <= 32 ? 128 / BK : 4, SWZ_K = BK <= 32 ? 4 : 8;
     auto swizzle_a = [](int k) { return SWZ && AK ? (k / SWZ_K % ((BM < 32 ? BM : 32) / SWZ_UNIT)) * SWZ_UNIT : 0; };
     auto swizzle_b = [](int k) { return SWZ && !BJ ? (k / SWZ_K % ((BN < 32 ? BN : 32) / SWZ_UNIT)) * SWZ_UNIT : 0; };
