@@ -572,7 +572,7 @@ int32_t do_expert_ffn_bwd(const moe_config *c, const Dims &D, const void *xs, co
         return MOE_OK;
     };
     const ColumnSums db2s = db2_sums(D, dys, db2, offsets, w, plan);
-    if (!db2_begun) MOE_TRY(launch_segment_colsum(db2s, false, st));
+    if (!db2_begun) MOE_TRY(launch_segment_colsum(db2s, st));
     MOE_TRY(finish(db2s, 0));
     if (tc_ffn_supported(*c)) {
         BlockSums left = {};
@@ -595,7 +595,7 @@ int32_t do_expert_ffn_bwd(const moe_config *c, const Dims &D, const void *xs, co
     g.mode = 0; g.offsets = offsets; g.nseg = n; g.M = D.R; g.N = D.h; g.K = D.d; g.b_e = D.h * D.d;
     MOE_TRY(launch_simt_gemm(g, nullptr, st, nullptr, &plan));
     const ColumnSums db1s = {w.dz, db1, D.act, n, (int32_t)D.h, D.R, offsets, plan.prefix_of(COLSUM_ROWS), w.colsum};
-    MOE_TRY(launch_segment_colsum(db1s, false, st));
+    MOE_TRY(launch_segment_colsum(db1s, st));
     MOE_TRY(finish(db1s, 1));
     g = base_gemm(D);  // dW1[e] = xs_e^T . dz_e
     g.A = xs; g.B = w.dz; g.C = dW1;

@@ -710,8 +710,8 @@ __device__ __forceinline__ bool acc_tile(const GemmParams &p, const Tile &t, int
 // into sub-blocks of p.sub_kb0 / p.sub_kb K blocks (first term / other terms). Each sub-block is accumulated in TMEM on
 // its own (an fp32 tensor-core accumulator truncates, and a long run of same-sign terms loses low bits: 128 rows keep
 // that below 1e-5), handed to the epilogue like a tile, and added there, with rounding to nearest, to running sums in
-// registers (a lane's row of the warp's 128 columns; the cap of 168 registers makes the compiler spill 88 bytes of other
-// values); the sums go to global memory once per tile. (With the sums in shared memory, which left room for two operand
+// registers (a lane's row of the warp's 128 columns; the cap of 168 registers makes the compiler spill 96 bytes of other
+// values, 132 on SM pairs); the sums go to global memory once per tile. (With the sums in shared memory, which left room for two operand
 // stages, a K block took 1850 cycles: the latency of its loads.)
 template <int KIND, int EPI, bool ACC = false>
 __global__ void __launch_bounds__(NTHREADS, 1)

@@ -266,7 +266,7 @@ int32_t launch_gate_logit_grads(const float *noise, const float *clean, const fl
                                 const float *dgates, const float *dload, const int32_t *dload_row_group,
                                 int64_t rows, int32_t n, int32_t k, float *dlogit, void *dsplit,
                                 const int32_t *split_row_index, cudaStream_t st, const ColumnSums *sums) {
-    if (rows == 0) return sums ? launch_segment_colsum(*sums, false, st) : MOE_OK;
+    if (rows == 0) return sums ? launch_segment_colsum(*sums, st) : MOE_OK;
     const int64_t more = sums ? column_tiles(*sums) * column_slabs(*sums) : 0;
     const unsigned grid = (unsigned)(cdiv(rows, 8) + more);
     auto run = [&](const auto &beside) -> int32_t {

@@ -535,12 +535,12 @@ template <int COLS> __global__ void __launch_bounds__(256) colsum_final_kernel(c
     column_sums_final<COLS>(a, blockIdx.x, blockIdx.y, sh);
 }
 
-int32_t launch_segment_colsum(const ColumnSums &a, bool finish, cudaStream_t st) {
+int32_t launch_segment_colsum(const ColumnSums &a, cudaStream_t st) {
     const dim3 tiles((unsigned)column_tiles(a), (unsigned)column_slabs(a));
     if (a.act == MOE_BF16) launch_kernel(colsum_partial_kernel<bf16>, tiles, 256, 0, st, a);
     else launch_kernel(colsum_partial_kernel<float>, tiles, 256, 0, st, a);
     MOE_LAUNCHED();
-    return finish ? launch_segment_colsum_final(a, st) : MOE_OK;
+    return MOE_OK;
 }
 int32_t launch_segment_colsum_final(const ColumnSums &a, cudaStream_t st) {
     if (a.nseg >= COLSUM_MANY) launch_kernel(colsum_final_kernel<256>, dim3((unsigned)a.nseg, (unsigned)cdiv(a.N, 256)), 256, 0, st, a);

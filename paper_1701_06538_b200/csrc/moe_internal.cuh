@@ -393,7 +393,7 @@ struct ColumnSums {
 int64_t colsum_ws_floats(int64_t R, int32_t n, int32_t N);
 static inline int64_t column_tiles(const ColumnSums &a) { return cdiv(a.R, COLSUM_ROWS) + a.nseg; }
 static inline int64_t column_slabs(const ColumnSums &a) { return cdiv(a.N, a.act == MOE_BF16 ? 256 : 128); }  // of 32 lanes x one 16-byte vector
-int32_t launch_segment_colsum(const ColumnSums &a, bool finish, cudaStream_t st);
+int32_t launch_segment_colsum(const ColumnSums &a, cudaStream_t st);  // the tiles
 int32_t launch_segment_colsum_final(const ColumnSums &a, cudaStream_t st);
 // out[e, j] = sum of segment e's blocks of 32-row column sums, G blocks a tile
 struct BlockSums {
@@ -410,7 +410,7 @@ struct BackwardTail {
     int32_t parts_blocks, block_blocks, column_blocks[2];
     int64_t total() const { return (int64_t)parts_blocks + block_blocks + column_blocks[0] + column_blocks[1]; }
 };
-// blocks up to which they go along with the rows' (whose registers leave three on an SM); more take one launch of their own
+// blocks up to which they go along with the rows' (whose registers leave two on an SM in bf16, one of one slot); more take one launch of their own
 // (32768 rows x 512, 256 experts, 9216 blocks: 111 us together, 83 apart; 3001 rows x 320, 20 experts, 510 blocks: 10 us, apart 16)
 constexpr int64_t TAIL_RIDE_MAX = 8 * 148;
 
