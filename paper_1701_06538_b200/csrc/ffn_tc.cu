@@ -1642,12 +1642,16 @@ static bool wgrad_uses_maps(int64_t R, int32_t nseg, int32_t M, int32_t N, int32
     if (short_segments(R, nseg)) return false;
     return use_two_cta(R, nseg, flags, wide) || nseg * cdiv(narrow, BM) * cdiv(wide, BN) >= 4 * (int64_t)sm_count();
 }
-// The rows of a row product behind a segment's end are read and dropped, or, through the segment's own map, not read. That saves half of
-// A's bytes where segments are half a tile, but the fence delays the tile: worth it only where a CTA has so many tiles that the
-// loads of the ones before cover it (a step with 4096 experts x 64 rows, 110 tiles a CTA: 6440 us, without 6490; but 480 x 24 rows, ten
-// tiles: 386, 374; 32 x 1024: 353, 345; the two products alone at 64 x 62 rows: 22.7, 16.9). cols: the wider side, as in use_two_cta
-static bool rows_use_maps(int64_t R, int32_t nseg, int32_t cols) {
-    return R < 128 * (int64_t)nseg && (cdiv(R, 128) + nseg) * cdiv(cols, BN) >= 32 * (int64_t)sm_count();
+// The rows of a row product behind a segment's end are read and dropped, or, through the segment's own map, not read. That saves bytes
+// of A (half of them where segments are half a tile), but the fence delays the tile: worth it only where a CTA or pair has so many tiles
+// that the loads of the ones before cover it. Steps, us: 4096 experts x 64 rows, 110 tiles a CTA, 6440, without 6490; on pairs 256 x 512
+// rows, 41 tiles a pair, 1420, without 1430; but 480 x 24 rows, ten tiles a CTA, 386, 374; 32 x 1024 rows, nine a pair, 353, 345; the
+// two products alone at 64 x 62 rows 22.7, 16.9. On one CTA a tile longer segments gain too little. cols: the wider side, as in
+// use_two_cta
+static bool rows_use_maps(int64_t R, int32_t nseg, int32_t flags, int32_t cols) {
+    const bool two = use_two_cta(R, nseg, flags, cols);
+    if (!two && !short_segments(R, nseg)) return false;
+    return (cdiv(R, two ? 256 : BM) + nseg) * cdiv(cols, BN) >= 32 * (int64_t)(two ? sm_count() / 2 : sm_count());
 }
 
 int32_t tc_segment_maps(const moe_config &c, SegmentMaps *maps, const void *xs_rows, const void *hid_rows, const void *dys_rows,
@@ -1662,7 +1666,7 @@ int32_t tc_segment_maps(const moe_config &c, SegmentMaps *maps, const void *xs_r
     // boxes as in tc_row_gemm and tc_wgrad_gemm
     const bool two = use_two_cta(R, c.n, c.flags, c.d > c.h ? c.d : c.h);
     const int b2 = two && c.h >= 256 ? 2 : BN / 64, b1 = two && c.d >= 256 ? 2 : BN / 64;
-    if (rows_use_maps(R, c.n, c.d > c.h ? c.d : c.h)) {
+    if (rows_use_maps(R, c.n, c.flags, c.d > c.h ? c.d : c.h)) {
         MOE_TRY(add(MAP_XS_ROWS, xs_rows, c.d, 0));
         MOE_TRY(add(MAP_HID_ROWS, hid_rows, c.h, 0));
         MOE_TRY(add(MAP_DYS_ROWS, dys_rows, c.d, 0));
@@ -1782,7 +1786,7 @@ int32_t tc_row_gemm(const void *A, const void *W, bool transposed, const int32_t
     GemmParams p = default_params();
     p.offsets = offsets; p.tile_prefix = plan.prefix[0]; p.tile_info = plan.info;
     p.nseg = nseg; p.M = 0; p.N = N; p.K = K; p.R = R;
-    if (rows_use_maps(R, nseg, N > K ? N : K)) p.seg_a = plan.maps_of(seg);
+    if (rows_use_maps(R, nseg, flags, N > K ? N : K)) p.seg_a = plan.maps_of(seg);
     p.out = (bf16 *)out; p.bias = (const bf16 *)bias; p.mask = (const bf16 *)mask; p.relu = relu; p.status = status;
     p.bits_out = bits_out; p.bits_in = bits_in;
     if (bits_in) p.mask = nullptr;  // the bits replace the element-wise mask tensor

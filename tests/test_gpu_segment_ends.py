@@ -15,7 +15,9 @@ ENDS = [0, 1, 15, 16, 17, 31, 33, 48, 63, 64, 65, 127, 128, 129, 191, 255, 256, 
                                                    # from four tiles a CTA on: weight gradients through maps of the segments
                                                    (640, 1024, 2, B.MOE_FLAG_TC_ONE_CTA, 1),
                                                    # from 32 tiles a CTA on, short segments: row products through them as well
-                                                   (64, 4096, 1, 0, 8)])
+                                                   (64, 4096, 1, 0, 8),
+                                                   # the same on SM pairs
+                                                   (256, 3072, 5, 0, 4)])
 def test_rows_behind_a_segment_do_not_count(d, h, scale, flags, times):
     counts = []
     for c in ENDS * times:  # every segment is followed by one whose rows are infinite

@@ -12,7 +12,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("T,n,d,h", [(600, 4, 1024, 1024),    # one CTA a tile
                                      (4096, 2, 1024, 1024),   # SM pairs
-                                     (1000, 300, 64, 4096)])  # one CTA a tile, segments with maps of their own
+                                     (1000, 300, 64, 4096),   # one CTA a tile, segments with maps of their own
+                                     (36000, 70, 256, 3072)])  # SM pairs, segments with maps of their own
 def test_rows_behind_the_batch_read_as_zeros(T, n, d, h):
     over = 5
     cfg = B.make_config(T, d, h, n, 1, "bf16", 0.1, 0.1)
