@@ -11,7 +11,7 @@
  *    allocates or frees device memory and never synchronises the host with the device (except
  *    moe_check_status and moe_debug_bounds_violations, which say so). It keeps no state between
  *    calls, with three small exceptions: a host-side launch counter (diagnostics), function
- *    attributes set on a kernel's first launch, and moe_dispatch_noalloc (see there: a fixed
+ *    attributes and SM counts, set and looked up at a kernel's first launch on each device, and moe_dispatch_noalloc (see there: a fixed
  *    scratch array inside the library's device image and its cached address). All work is enqueued
  *    on `stream` (a cudaStream_t passed as void*; NULL is the default stream).
  *  - `ws` and `ctx` are bare pointers: a buffer that is too small cannot be detected by the call it
