@@ -197,9 +197,12 @@ struct DispatchWs {
 SegmentPlan make_plan(const moe_config *c, const Dims &D, int32_t *ws, bool backward) {
     SegmentPlan p = plan_at(ws, D.R, D.n);
     if (tc_ffn_supported(*c)) {
-        p.bm[0] = tc_row_tile(D.R, (int32_t)D.n, D.flags, (int32_t)(D.d > D.h ? D.d : D.h));
+        p.bm[0] = tc_row_tile(*c);
         if (backward && p.bm[0] != COLSUM_ROWS) p.bm[1] = COLSUM_ROWS;
-        if (!backward || !tc_wgrad_sorted(*c)) p.sched = nullptr;
+        if (!backward || !tc_wgrad_sorted(*c)) {
+            p.sched = nullptr;
+            p.by_rank = p.prefix[0];
+        }
     } else {
         p.bm[0] = 64; p.bm[1] = 32; p.bm[2] = 16;
         if (backward) p.bm[3] = COLSUM_ROWS;
@@ -814,7 +817,7 @@ int32_t moe_query_ctx_layout(const moe_config *cfg, moe_ctx_layout *out) {
 
 int64_t moe_debug_bounds_violations(void) {
     const unsigned long long parts[] = {bounds_violations_route(), bounds_violations_losses(), bounds_violations_hier(),
-                                        bounds_violations_gate(), bounds_violations_gate_bwd(), bounds_violations_ffn()};
+                                        bounds_violations_gate(), bounds_violations_gate_bwd(), bounds_violations_ffn(), bounds_violations_products()};
     unsigned long long sum = 0;
     for (unsigned long long v : parts) {
         if (v == ~0ull) return -1;

@@ -75,6 +75,7 @@ unsigned long long bounds_violations_hier();
 unsigned long long bounds_violations_gate();
 unsigned long long bounds_violations_gate_bwd();
 unsigned long long bounds_violations_ffn();
+unsigned long long bounds_violations_products();
 
 typedef __nv_bfloat16 bf16;
 
@@ -222,9 +223,8 @@ __device__ __forceinline__ int4 segment_of_tile(const int32_t *__restrict__ tile
 int32_t launch_tile_prefix(const int32_t *offsets, int32_t n, int32_t bm, int32_t *tile_prefix, cudaStream_t st);
 
 // ----------------------------------------------------------------------------- per-call segment plan (plan.cu)
-constexpr int PLAN_HEIGHTS = 4, PLAN_COUNTERS = 8, PLAN_MAX_SORTED = 8192;
-// run-time tile counters of a plan, by the GEMM that uses them
-enum PlanCounter { PLAN_ROWS_A = 0, PLAN_ROWS_B = 1, PLAN_WGRAD_A = 2, PLAN_WGRAD_B = 3, PLAN_ROWS_AGAIN = 4 };
+constexpr int PLAN_HEIGHTS = 4, PLAN_COUNTERS = 8, PLAN_MAX_SORTED = 2048;
+enum PlanCounter { PLAN_HID = 0, PLAN_YS, PLAN_DZ_DW2, PLAN_DW1_DXS };  // the tiles drawn so far, by launch of expert products
 // Tensor maps of a call's expert products whose rows end with a segment, one per segment: what lies behind a segment's last row reads
 // as zero, whatever follows it in memory. ROWS: K-major operand of a row product, COLS: operand of a weight gradient
 // (contraction over the rows).
@@ -239,8 +239,11 @@ struct SegmentPlan {
     const CUtensorMap *maps_of(SegmentMap which) const { return maps ? maps + (int64_t)which * n : nullptr; }
     int32_t *prefix[PLAN_HEIGHTS];  // [n + 1] number of tiles of bm[i] rows in the segments before
     int32_t bm[PLAN_HEIGHTS];       // 0: prefix not made
-    int4 *info;          // a record per tile of prefix[0], or nullptr: {segment or -1, first row, segment end, 0}
-    int4 *sched;         // {segment, first row, end row, 0} in descending size, or nullptr
+    // Tensor-core products take the segments by rank: by descending size (sched), or as they lie
+    int4 *sched;         // {segment, first row, end row, 0} by rank, or nullptr
+    int32_t *by_rank;    // [n + 1] tiles of bm[0] rows in the segments before, by rank (prefix[0] if sched is not made); prefix[0] is its copy by
+                         // segment, without an end
+    int4 *info;          // a record per tile of by_rank, or nullptr: {segment, first row, segment end, number of the tile}
     int32_t *counters;   // [PLAN_COUNTERS], zeroed
     const int32_t *prefix_of(int32_t height) const {
         for (int i = 0; i < PLAN_HEIGHTS; ++i)
@@ -398,9 +401,9 @@ int32_t launch_segment_colsum_final(const ColumnSums &a, cudaStream_t st);
 // out[e, j] = sum of segment e's blocks of 32-row column sums, G blocks a tile
 struct BlockSums {
     const float *part;
-    const int32_t *tile_prefix;
+    const int32_t *first_tile, *offsets;
     bf16 *out;
-    int32_t nseg, N, G;
+    int32_t nseg, N, G, tile_rows;
 };
 // What the fused backward leaves for its last launch (0 blocks: nothing)
 struct BackwardTail {
@@ -419,8 +422,8 @@ bool tc_ffn_supported(const moe_config &c);
 // base maps of the operands that are given (nullptr: not wanted)
 int32_t tc_segment_maps(const moe_config &c, SegmentMaps *maps, const void *xs_rows, const void *hid_rows, const void *dys_rows,
                         const void *dz_rows, const void *hid_cols, const void *dys_cols, const void *xs_cols, const void *dz_cols);
-int32_t tc_row_tile(int64_t R, int32_t nseg, int32_t flags, int32_t cols);  // tile height of the row GEMMs: what plan.bm[0] has to be
-bool tc_wgrad_sorted(const moe_config &c);                    // the weight gradients want plan.sched
+int32_t tc_row_tile(const moe_config &c);    // tile height of the row products: what plan.bm[0] has to be
+bool tc_wgrad_sorted(const moe_config &c);   // the backward products want plan.sched
 // first_only: only hid = relu(xs.W1 + b1) (the recomputation of the hidden activations in the backward pass)
 int32_t launch_tc_ffn(const moe_config &c, const void *xs, const int32_t *offsets, const void *W1, const void *b1,
                       const void *W2, const void *b2, void *hid, void *ys, const SegmentPlan &plan, int32_t *status_word,

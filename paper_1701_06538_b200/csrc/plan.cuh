@@ -9,7 +9,7 @@ namespace moe {
 
 struct PlanArgs {
     SegmentPlan plan;
-    int32_t n, max_m;  // max_m: tile records of plan.info
+    int32_t n;
     int32_t *status;   // cleared if given
     Cv2Job cv2[2];
     int32_t map_block0;  // first block of the tensor maps
@@ -22,20 +22,21 @@ inline int64_t plan_blocks(const PlanArgs &a) {
     for (int i = 0; i < SEGMENT_MAPS; ++i) maps += a.maps.made[i] ? a.n : 0;
     return a.map_block0 + cdiv(maps, MAPS_PER_BLOCK);
 }
-// ints of shared memory a piece of the plan needs: the segments' lengths, or the maps under construction
-inline int64_t plan_shared_ints(int32_t n) { return n > MAPS_PER_BLOCK * 32 ? n : MAPS_PER_BLOCK * 32; }
+// ints of shared memory a piece of the plan needs: the lengths of n sorted segments and their order, or the maps under construction
+inline int64_t plan_shared_ints(int32_t n) { return 2 * n > MAPS_PER_BLOCK * 32 ? 2 * n : MAPS_PER_BLOCK * 32; }
 
 __device__ __forceinline__ int32_t *on_128_bytes(int32_t *shared) {
     return shared + ((128u - ((uint32_t)__cvta_generic_to_shared(shared) & 127u)) & 127u) / 4u;
 }
 
-// exclusive prefix of the segments' tiles of bm rows; returns the total to every thread (1024 threads)
-static __device__ int32_t tile_prefix_block(const int32_t *offsets, int32_t n, int32_t bm, int32_t *prefix, int32_t *sh /* [32] */) {
+// exclusive prefix of the tiles of bm rows of segments of rows(i) rows; returns the total to every thread (1024 threads)
+template <typename Rows>
+static __device__ __forceinline__ int32_t tile_prefix_block(Rows rows, int32_t n, int32_t bm, int32_t *prefix, int32_t *sh /* [32] */) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     int32_t carry = 0;
     for (int32_t base = 0; base < n; base += 1024) {
         const int32_t e = base + threadIdx.x;
-        const int32_t v = e < n ? (offsets[e + 1] - offsets[e] + bm - 1) / bm : 0;
+        const int32_t v = e < n ? (rows(e) + bm - 1) / bm : 0;
         int32_t inc = v;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
@@ -61,8 +62,8 @@ static __device__ int32_t tile_prefix_block(const int32_t *offsets, int32_t n, i
 }
 
 // Piece `block` of the plan, by 1024 threads; offsets: global or shared memory; cnt: plan_shared_ints(n), on 128 bytes.
-// Pieces 0..3: tile prefixes (0: the records, the counters and the status word as well); 4, 5: loss gradients; from 6 on:
-// 1024 segments each of the order by size; from map_block0 on: the segments' tensor maps
+// Pieces 0..3: tile prefixes (0: the order by size, the records, the counters and the status word as well); 4, 5: loss gradients; from
+// map_block0 on: the segments' tensor maps
 __device__ __forceinline__ void plan_piece(const PlanArgs &a, int32_t block, const int32_t *offsets, int32_t *cnt, int32_t *sh /* [32] */,
                                            double *moments /* [32] */) {
     const int32_t n = a.n;
@@ -88,31 +89,52 @@ __device__ __forceinline__ void plan_piece(const PlanArgs &a, int32_t block, con
             if (threadIdx.x == 0 && a.status) *a.status = 0;
         }
         if (a.plan.bm[which] == 0) return;
-        int32_t *prefix = a.plan.prefix[which];
-        const int32_t bm = a.plan.bm[which], total = tile_prefix_block(offsets, n, bm, prefix, sh);
-        if (which != 0 || !a.plan.info) return;
+        const int32_t bm = a.plan.bm[which];
+        auto rows_of = [&](int32_t e) { return offsets[e + 1] - offsets[e]; };
+        if (which != 0 || !a.plan.info) {
+            tile_prefix_block(rows_of, n, bm, a.plan.prefix[which], sh);
+            return;
+        }
+        int32_t *by_rank = a.plan.by_rank, *order = cnt + n;
+        const bool sorted = a.plan.sched != nullptr;
+        int32_t total;
+        if (sorted) {  // rank by descending size, equal sizes by index: `lanes` lanes a segment, each compares with its share of the others
+            int32_t lanes = 1;
+            while (lanes < 32 && 2 * lanes * n <= 1024) lanes *= 2;
+            for (int32_t e = threadIdx.x; e < n; e += 1024) cnt[e] = rows_of(e);
+            __syncthreads();
+            const int32_t share = threadIdx.x & (lanes - 1);
+            for (int32_t e0 = 0; e0 < n; e0 += 1024 / lanes) {
+                const int32_t e = e0 + threadIdx.x / lanes, mine = e < n ? cnt[e] : 0;
+                int32_t rank = 0;
+                for (int32_t o = share; o < n; o += lanes) rank += (cnt[o] > mine || (cnt[o] == mine && o < e)) ? 1 : 0;
+                for (int32_t s = 1; s < lanes; s <<= 1) rank += __shfl_xor_sync(0xffffffffu, rank, s);
+                if (e < n && share == 0) {
+                    order[rank] = e;
+                    a.plan.sched[rank] = make_int4(e, offsets[e], offsets[e + 1], 0);
+                }
+            }
+            __syncthreads();
+            total = tile_prefix_block([&](int32_t r) { return cnt[order[r]]; }, n, bm, by_rank, sh);
+        } else {
+            by_rank = a.plan.prefix[0];
+            total = tile_prefix_block(rows_of, n, bm, by_rank, sh);
+        }
         __syncthreads();  // the prefix (global memory, this block's own writes) is complete
-        for (int32_t mt = threadIdx.x; mt < a.max_m; mt += 1024) {
-            if (mt >= total) { a.plan.info[mt] = make_int4(-1, 0, 0, 0); continue; }
-            int lo = 0, hi = n;  // last e with prefix[e] <= mt (empty segments share a prefix: take the last)
+        if (sorted)
+            for (int32_t r = threadIdx.x; r < n; r += 1024) a.plan.prefix[0][order[r]] = by_rank[r];
+        for (int32_t mt = threadIdx.x; mt < total; mt += 1024) {
+            int lo = 0, hi = n;  // last rank with by_rank <= mt (empty segments share a prefix: take the last)
             while (hi - lo > 1) {
                 const int mid = (lo + hi) >> 1;
-                if (prefix[mid] <= mt) lo = mid; else hi = mid;
+                if (by_rank[mid] <= mt) lo = mid; else hi = mid;
             }
-            a.plan.info[mt] = make_int4(lo, offsets[lo] + (mt - prefix[lo]) * bm, offsets[lo + 1], 0);
+            const int32_t e = sorted ? order[lo] : lo;
+            a.plan.info[mt] = make_int4(e, offsets[e] + (mt - by_rank[lo]) * bm, offsets[e + 1], mt);
         }
     } else if (block < PLAN_HEIGHTS + 2) {
         const Cv2Job &job = a.cv2[block - PLAN_HEIGHTS];
         if (job.v) cv2_grad_block(job, moments);
-    } else if (a.plan.sched) {  // rank by descending size, equal sizes by index
-        for (int32_t e = threadIdx.x; e < n; e += 1024) cnt[e] = offsets[e + 1] - offsets[e];
-        __syncthreads();
-        const int32_t e = (block - PLAN_HEIGHTS - 2) * 1024 + threadIdx.x;
-        if (e >= n) return;
-        const int32_t mine = cnt[e];
-        int32_t rank = 0;
-        for (int32_t o = 0; o < n; ++o) rank += (cnt[o] > mine || (cnt[o] == mine && o < e)) ? 1 : 0;
-        a.plan.sched[rank] = make_int4(e, offsets[e], offsets[e + 1], 0);
     }
 }
 

@@ -106,10 +106,9 @@ template <int COLS> __device__ __forceinline__ void column_sums_final(const Colu
 // in one kernel cost the narrow form a loop and spills: 61 us instead of 41 at 128 experts x 4096 columns.)
 template <int COLS> __device__ __forceinline__ void block_sums_final(const BlockSums &a, int32_t e, int32_t slab, float4 (&sh)[16][16]) {
     const float *__restrict__ part = a.part;
-    const int32_t *__restrict__ tile_prefix = a.tile_prefix;
     bf16 *__restrict__ out = a.out;
     const int32_t N = a.N, G = a.G, q = threadIdx.x >> 4, cl = threadIdx.x & 15;
-    const int32_t b0 = tile_prefix[e] * G, b1 = tile_prefix[e + 1] * G;
+    const int32_t b0 = a.first_tile[e] * G, b1 = b0 + (a.offsets[e + 1] - a.offsets[e] + a.tile_rows - 1) / a.tile_rows * G;
     auto store = [&](int32_t j, const float4 &t) {
         const __nv_bfloat162 o0 = __floats2bfloat162_rn(t.x, t.y), o1 = __floats2bfloat162_rn(t.z, t.w);
         uint2 pk;
