@@ -19,6 +19,7 @@ struct Dims {
     int64_t gate_cols, logits, gates, kth, wg, load, dload;
     int32_t act, flags;
     size_t esz;
+    bool float_terms[2];  // float experts on the tensor cores: forward, backward
 };
 
 int32_t check_config(const moe_config *c) {
@@ -57,6 +58,7 @@ Dims dims_of(const moe_config *c) {
     D.act = c->act;
     D.flags = c->flags;
     D.esz = act_bytes(c->act);
+    for (int backward = 0; backward < 2; ++backward) D.float_terms[backward] = tc_float_supported(*c, backward);
     if (D.hier) {
         D.gate_cols = D.a + D.k1 * D.b;
         D.gates = D.T * (2 * D.k + D.k1);
@@ -203,6 +205,11 @@ SegmentPlan make_plan(const moe_config *c, const Dims &D, int32_t *ws, bool back
             p.sched = nullptr;
             p.by_rank = p.prefix[0];
         }
+    } else if (D.float_terms[backward]) {
+        p.bm[0] = COLSUM_ROWS;
+        p.sched = nullptr;
+        p.by_rank = p.prefix[0];
+        p.maps = nullptr;
     } else {
         p.bm[0] = 64; p.bm[1] = 32; p.bm[2] = 16;
         if (backward) p.bm[3] = COLSUM_ROWS;
@@ -212,11 +219,26 @@ SegmentPlan make_plan(const moe_config *c, const Dims &D, int32_t *ws, bool back
     return p;
 }
 
+FloatTerms float_terms(Carver &cv, const Dims &D, bool backward) {
+    FloatTerms t = {};
+    if (!D.float_terms[backward]) return t;
+    t.xs = cv.take<bf16>(3 * D.R * D.d);
+    t.hid = cv.take<bf16>(3 * D.R * D.h);
+    t.W1 = cv.take<bf16>(3 * D.n * D.d * D.h);
+    t.W2 = cv.take<bf16>(3 * D.n * D.d * D.h);
+    if (!backward) return t;
+    t.dys = cv.take<bf16>(3 * D.R * D.d);
+    t.dz = cv.take<bf16>(3 * D.R * D.h);
+    return t;
+}
+
 struct FfnWs {
     int32_t *plan;
+    FloatTerms terms;
     void *hid;  // MOE_FLAG_RECOMPUTE_HID: the hidden activations live here instead of in a buffer that is kept
-    FfnWs(Carver &cv, const Dims &D) {
+    FfnWs(Carver &cv, const Dims &D, bool forward = true) {  // the backward pass has terms of its own
         plan = cv.take<int32_t>(plan_ints(D.R, D.n));
+        terms = forward ? float_terms(cv, D, false) : FloatTerms{};
         hid = (D.flags & MOE_FLAG_RECOMPUTE_HID) ? cv.take_bytes(D.R * D.h * (int64_t)D.esz) : nullptr;
     }
 };
@@ -250,6 +272,7 @@ struct FfnBwdWs : Db2Sums {
     void *dz;
     float *colsum;   // of db1
     uint32_t *bits;  // MOE_FLAG_RECOMPUTE_HID on the tensor cores: the mask bits that the recomputation writes
+    FloatTerms terms;
     FfnBwdWs(const Db2Sums &sums, Carver &cv, const Dims &D) : Db2Sums(sums) {
         dz = cv.take_bytes(D.R * D.h * (int64_t)D.esz);
         const bool tc = D.act == MOE_BF16 && D.d % 64 == 0 && D.h % 64 == 0;
@@ -259,6 +282,7 @@ struct FfnBwdWs : Db2Sums {
             const int64_t cs_tc = tc_colsum_part_floats(D.R, (int32_t)D.n, (int32_t)D.h);
             if (cs_tc > cs) cs = cs_tc;
         }
+        terms = float_terms(cv, D, true);
         colsum = cv.take<float>(cs);
     }
     FfnBwdWs(Carver &cv, const Dims &D) : FfnBwdWs(Db2Sums(cv, D), cv, D) {}
@@ -390,7 +414,7 @@ struct FusedBwdWs : BwdWs {
     GateBwdWs gate;
     FusedBwdWs(Carver &cv, const Dims &D)
         : BwdWs(cv, D), db2(cv, D), gate_sums(cv, D), experts_at(cv), gate_at(cv),
-          dxs(experts_at.take_bytes(D.R * D.d * (int64_t)D.esz)), ffn(db2, experts_at, D), again(experts_at, D),
+          dxs(experts_at.take_bytes(D.R * D.d * (int64_t)D.esz)), ffn(db2, experts_at, D), again(experts_at, D, false),
           gate(gate_sums, gate_at, D) {
         cv = experts_at.off > gate_at.off ? experts_at : gate_at;
     }
@@ -506,6 +530,7 @@ int32_t do_expert_ffn(const moe_config *c, const Dims &D, const void *xs, const 
     }
     if (tc_ffn_supported(*c))
         return launch_tc_ffn(*c, xs, offsets, W1, b1, W2, b2, hid, ys, plan, status_word(ws_base), st, first_only, relu_bits);
+    if (D.float_terms[0] && !first_only) return launch_float_ffn(*c, xs, offsets, W1, b1, W2, b2, hid, ys, plan, w.terms, status_word(ws_base), st);
     SimtGemm g = base_gemm(D);  // hid = relu(xs.W1 + b1)
     g.A = xs; g.B = W1; g.C = hid; g.bias = b1; g.relu = 1;
     g.sa_i = D.d; g.sa_k = 1; g.sb_k = D.h; g.sb_j = 1; g.sc_i = D.h;
@@ -565,7 +590,9 @@ ColumnSums db2_sums(const Dims &D, const void *dys, void *db2, const int32_t *of
 int32_t do_expert_ffn_bwd(const moe_config *c, const Dims &D, const void *xs, const void *hid, const void *dys,
                           const int32_t *offsets, const void *W1, const void *W2, void *dxs, void *dW1, void *db1,
                           void *dW2, void *db2, void *ws_base, const FfnBwdWs &w, cudaStream_t st, const SegmentPlan &plan,
-                          const uint32_t *relu_bits = nullptr, BackwardTail *tail = nullptr, bool db2_begun = false) {
+                          const uint32_t *relu_bits = nullptr, BackwardTail *tail = nullptr, bool db2_begun = false,
+                          const void *b1_again = nullptr) {
+    // b1_again (float experts on the tensor cores): hid is computed first
     const int32_t n = (int32_t)D.n;
     BackwardTail *leave = n < COLSUM_MANY ? tail : nullptr;
     auto finish = [&](const ColumnSums &sums, int which) -> int32_t {
@@ -587,6 +614,13 @@ int32_t do_expert_ffn_bwd(const moe_config *c, const Dims &D, const void *xs, co
         }
         return MOE_OK;
     }
+    const ColumnSums db1s = {w.dz, db1, D.act, n, (int32_t)D.h, D.R, offsets, plan.prefix_of(COLSUM_ROWS), w.colsum};
+    if (D.float_terms[1]) {
+        MOE_TRY(launch_float_ffn_bwd(*c, xs, const_cast<void *>(hid), b1_again != nullptr, dys, offsets, W1, b1_again, W2, dxs, dW1, dW2, w.dz, plan,
+                                     w.terms, status_word(ws_base), st));
+        MOE_TRY(launch_segment_colsum(db1s, st));
+        return finish(db1s, 1);
+    }
     SimtGemm g = base_gemm(D);  // dW2[e] = hid_e^T . dys_e
     g.A = hid; g.B = dys; g.C = dW2;
     g.sa_i = 1; g.sa_k = D.h; g.sb_k = D.d; g.sb_j = 1; g.sc_i = D.d;
@@ -597,7 +631,6 @@ int32_t do_expert_ffn_bwd(const moe_config *c, const Dims &D, const void *xs, co
     g.sa_i = D.d; g.sa_k = 1; g.sb_k = 1; g.sb_j = D.d; g.sc_i = D.h;
     g.mode = 0; g.offsets = offsets; g.nseg = n; g.M = D.R; g.N = D.h; g.K = D.d; g.b_e = D.h * D.d;
     MOE_TRY(launch_simt_gemm(g, nullptr, st, nullptr, &plan));
-    const ColumnSums db1s = {w.dz, db1, D.act, n, (int32_t)D.h, D.R, offsets, plan.prefix_of(COLSUM_ROWS), w.colsum};
     MOE_TRY(launch_segment_colsum(db1s, st));
     MOE_TRY(finish(db1s, 1));
     g = base_gemm(D);  // dW1[e] = xs_e^T . dz_e
@@ -1093,11 +1126,11 @@ static int32_t backward_impl(const moe_config *cfg, const void *dY, const void *
     if (!hid) {  // MOE_FLAG_RECOMPUTE_HID: the forward kept no hidden activations; the first GEMM is run again
         bits = B.ffn.bits;
         Carver none(nullptr);  // (both buffers are given)
-        MOE_TRY(do_expert_ffn(cfg, D, C.xs, C.offsets, W1, b1, W2, b2, B.again.hid, nullptr, ws, none, st, nullptr, true, bits, &plan));
+        if (!D.float_terms[1]) MOE_TRY(do_expert_ffn(cfg, D, C.xs, C.offsets, W1, b1, W2, b2, B.again.hid, nullptr, ws, none, st, nullptr, true, bits, &plan));
         hid = B.again.hid;
     }
     MOE_TRY(do_expert_ffn_bwd(cfg, D, C.xs, hid, B.dys, C.offsets, W1, W2, B.dxs, dW1, db1, dW2, db2, ws, B.ffn, st, plan, bits, left,
-                              left != nullptr));
+                              left != nullptr, C.hid ? nullptr : b1));
     // dX = expert path + gating path (+ the upstream gradient itself through the residual connection)
     return launch_dispatch_bwd(B.dxs, D.act, C.inv_perm, D.T, (int32_t)D.k, (int32_t)D.d, B.dX_gate, nullptr, dX,
                                st, keep_bits ? dY : nullptr, sec, left);

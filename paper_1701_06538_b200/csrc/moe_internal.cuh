@@ -431,6 +431,17 @@ int32_t launch_tc_ffn(const moe_config &c, const void *xs, const int32_t *offset
 // relu_bits [R, h / 32]: one bit per hidden activation (set where hid > 0), written by the first expert GEMM if given;
 // the backward then masks dz with these bits instead of reading hid again as a mask (16 times less traffic)
 
+// ----------------------------------------------------------------------------- float experts on the tensor cores (products_f32.cu)
+bool tc_float_supported(const moe_config &c, bool backward);
+// three bf16 terms of a call's operands, [rows][3 columns]: rows of xs, hid, dys, dz; matrices W1 [n d][3 h], W2 [n h][3 d]
+struct FloatTerms { void *xs, *hid, *dys, *dz, *W1, *W2; };
+int32_t launch_float_ffn(const moe_config &c, const void *xs, const int32_t *offsets, const void *W1, const void *b1, const void *W2, const void *b2,
+                         void *hid, void *ys, const SegmentPlan &plan, const FloatTerms &t, int32_t *status, cudaStream_t st);
+// again: hid is computed first. The column sums of dys and dz are the caller's
+int32_t launch_float_ffn_bwd(const moe_config &c, const void *xs, void *hid, bool again, const void *dys, const int32_t *offsets, const void *W1,
+                             const void *b1, const void *W2, void *dxs, void *dW1, void *dW2, void *dz, const SegmentPlan &plan, const FloatTerms &t,
+                             int32_t *status, cudaStream_t st);
+
 // ----------------------------------------------------------------------------- strictly balanced gating (balanced.cu)
 int32_t launch_exclusive_scan(const int32_t *counts, int32_t n, int32_t *out, cudaStream_t st,
                               int32_t *tile_sums = nullptr /* cdiv(n + 1, 4096) ints: long inputs in parallel */);  // route.cu

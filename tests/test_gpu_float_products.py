@@ -1,0 +1,73 @@
+"""The float experts' products on the tensor cores (three bf16 terms an operand): segments around the 16-row steps, 64-row blocks and 128-row
+tiles, widths of one and a half tiles, against 64 bits; infinities, NaN and sums beyond float's range come out as the chain of
+fused multiply-adds gives them."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import moe_oracle as O
+from paper_1701_06538_b200 import binding as B
+
+pytestmark = pytest.mark.gpu
+
+ENDS = [0, 1, 15, 16, 17, 63, 64, 65, 127, 128, 129, 200, 0]
+
+
+def layer(counts, d, h, seed):
+    n, R = len(counts), sum(counts)
+    cfg = B.make_config(R, d, h, n, 1, "f32")
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    f = lambda *s: torch.randn(*s, device="cuda", generator=g)
+    offsets = torch.tensor([0] + counts, device="cuda").cumsum(0).to(torch.int32)
+    W1, W2 = f(n, d, h) * d ** -0.5, f(n, h, d) * h ** -0.5
+    return cfg, offsets, f(R, d), f(R, d), W1, f(n, h), W2, f(n, d), B.empty_bytes(B.moe_query_sizes(cfg).ws_bytes)
+
+
+@pytest.mark.parametrize("d,h,pad", [(192, 320, 1300), (64, 1024, 900), (448, 64, 3000)])
+def test_against_64_bits(d, h, pad):
+    counts = ENDS + [pad]  # enough rows for the path (asserted: its scratch is asked for)
+    cfg, offsets, xs, dys, W1, b1, W2, b2, ws = layer(counts, d, h, d + h)
+    n, R = len(counts), sum(counts)
+    assert B.moe_query_sizes(cfg).ws_fwd_bytes > 12 * n * d * h and B.moe_query_sizes(cfg).ws_bwd_bytes > 12 * n * d * h
+    hid, ys = torch.full((R, h), float("nan"), device="cuda"), torch.full_like(xs, float("nan"))
+    B.moe_expert_ffn(cfg, xs, offsets, W1, b1, W2, b2, hid, ys, ws)
+    out = [torch.full_like(t, float("nan")) for t in (xs, W1, b1, W2, b2)]
+    B.moe_expert_ffn_bwd(cfg, xs, hid, dys, offsets, W1, W2, *out, ws)
+    assert B.moe_check_status(ws) == 0
+    for e in range(n):
+        r = slice(int(offsets[e]), int(offsets[e + 1]))
+        x, dy, hd, w1, w2 = (t.double() for t in (xs[r], dys[r], hid[r], W1[e], W2[e]))
+        dz = (dy @ w2.t()) * (hd > 0)
+        want = [(hid[r], torch.relu(x @ w1 + b1[e].double())), (ys[r], hd @ w2 + b2[e].double()), (out[0][r], dz @ w1.t()),
+                (out[1][e], x.t() @ dz), (out[2][e], dz.sum(0)), (out[3][e], hd.t() @ dy), (out[4][e], dy.sum(0))]
+        for i, (got, exp) in enumerate(want):
+            if exp.numel():
+                err = ((got.double() - exp).abs() / (exp.abs() + exp.square().mean().sqrt() + 1e-30)).max()
+                assert err <= 1e-5, (e, counts[e], i, float(err))  # the tolerance of the float layer
+
+
+def test_values_that_are_no_numbers():
+    d, h, rows = 128, 256, 1600
+    cfg, offsets, xs, dys, W1, b1, W2, b2, ws = layer([rows, rows], d, h, 5)
+    xs[3, 7], xs[40, 9], xs[70], xs[200, 1:3] = float("inf"), float("nan"), 3.3e38, torch.tensor([float("inf"), -float("inf")], device="cuda")
+    xs[300, 0], xs[301] = 3.4e38, 1e-41  # would round beyond bf16's range; denormal
+    W1[0, 5, 6] = -float("inf")
+    hid, ys = torch.empty(2 * rows, h, device="cuda"), torch.empty_like(xs)
+    B.moe_expert_ffn(cfg, xs, offsets, W1, b1, W2, b2, hid, ys, ws)
+    assert B.moe_check_status(ws) == 0
+    chain = lambda a, w: O.project(np.ascontiguousarray(a.cpu().numpy()), np.ascontiguousarray(w.cpu().numpy()), "f32")
+    for got, a, w, b, relu in ((hid, xs, W1, b1, True), (ys, hid, W2, b2, False)):
+        for e in range(2):
+            r = slice(e * rows, e * rows + rows)
+            want = chain(a[r], w[e]) + b[e].cpu().numpy()
+            if relu:
+                want = np.where(want > 0, want, np.float32(0))  # NaN counts as 0, as before
+            have = got[r].cpu().numpy()
+            finite = np.isfinite(want)
+            # sums of values near float's range may or may not leave it on the way, by the order of their parts
+            wide = (np.abs(a[r].cpu().numpy()) > 1e30).any(1, keepdims=True) & np.isfinite(a[r].cpu().numpy()).all(1, keepdims=True)
+            assert ((np.isnan(have) == np.isnan(want)) | wide).all()
+            assert ((have == want) | finite | np.isnan(want) | wide).all() and ((have == want) | np.isfinite(have) | np.isnan(have)).all()
+            sound = finite & ~wide
+            scale = np.abs(want) + np.sqrt(np.mean(np.square(want[sound].astype(np.float64))))
+            assert (np.abs(have - want)[sound] <= 1e-5 * scale[sound]).all()
