@@ -6,28 +6,6 @@
 
 namespace moe {
 
-// ------------------------------------------------------------------------------------------
-// Projection  clean = x.W_g,  raw = x.W_noise   (the two products of Eq. 4)
-//
-// The routing must be reproducible bit for bit, so every output is ONE chain of fused
-// multiply-adds over the input features in ascending order, starting from +0. The register-tiled
-// SIMT product keeps that order by construction (each accumulator sees k = 0, 1, 2, ...); a
-// tensor-core MMA would not. It is therefore bound by the FP32 pipes, not by HBM.
-// ------------------------------------------------------------------------------------------
-int32_t launch_projection(const void *x, int32_t act, int64_t M, int32_t d, int32_t n0, const float *W0,
-                          const float *W1, float *out0, float *out1, const int32_t *offsets, int32_t nseg,
-                          const int32_t *perm, int32_t kdiv, int32_t *tile_prefix, cudaStream_t st,
-                          const int32_t *row_count, int32_t *clear) {
-    SimtGemm g;  // rows x [W0 | W1] (W1 == nullptr: one matrix only)
-    memset(&g, 0, sizeof(g));
-    g.ta = act == MOE_BF16 ? G_BF16 : G_F32; g.tb = g.tc = G_F32;
-    g.A = x; g.B = W0; g.B2 = W1; g.C = out0; g.C2 = W1 ? out1 : nullptr; g.b_split = g.c_split = n0;
-    g.sa_i = d; g.sa_k = 1; g.sb_k = n0; g.sb_j = 1; g.sc_i = n0;
-    g.mode = 0; g.offsets = offsets; g.nseg = nseg; g.M = M; g.N = W1 ? 2 * n0 : n0; g.K = d; g.b_e = (int64_t)d * n0;
-    g.a_row_index = perm; g.a_row_div = kdiv; g.c_row_index = perm; g.row_count = row_count; g.clear = clear;
-    return launch_simt_gemm(g, tile_prefix, st);
-}
-
 // rows that a block of 256 threads takes: a thread per column as far as that goes
 __host__ __device__ __forceinline__ int select_rows_per_block(int32_t n) { return n <= 64 ? 4 : n <= 128 ? 2 : 1; }
 

@@ -1,6 +1,6 @@
-// Strided SIMT grouped GEMM in float accumulation. It serves the gate projection (whose fixed order of fused
-// multiply-adds decides the routing), the all-float32 layer (where the 1e-5 tolerance rules out tensor-core formats),
-// shapes the tensor-core kernels do not take, and the two dense contractions of their gate backward.
+// Strided SIMT grouped GEMM in float accumulation. It serves gate projections whose widths are no whole quads (the others: projection.cu), float
+// layers of few rows or little work (the others: products_f32.cu), shapes the tensor-core kernels do not take, and the two dense
+// contractions of their gate backward.
 //
 // Every output is one chain of fused multiply-adds over the contraction index in ascending order, starting from +0
 // (contractions cut into slices: one such chain per slice, the slices added in double). That is bound by the FP32
@@ -470,12 +470,16 @@ static int32_t simt_pick_tile(SimtRun &run, bool vec_a, bool vec_b, int32_t *til
             return simt_launch<TA, TB, TC, false, false, AK, BJ, 32, 32, 4, 4, 32>(run, tile_prefix, st);
         }
     }
-    if (blocks(64, 128) >= 6 * 148 && !short_rows && g.N > 64)
-        return simt_launch<TA, TB, TC, true, true, AK, BJ, 64, 128, 8, 8, 16>(run, tile_prefix, st);
-    if (blocks(64, 64) >= 2 * 148 && !short_rows && !(run.part && g.N <= 32))
-        return simt_launch<TA, TB, TC, true, true, AK, BJ, 64, 64, 8, 4, 16>(run, tile_prefix, st);
-    if (blocks(32, 32) >= 148) return simt_launch<TA, TB, TC, true, true, AK, BJ, 32, 32, 4, 4, 32>(run, tile_prefix, st);
-    return simt_launch<TA, TB, TC, true, true, AK, BJ, 16, 16, 2, 2, 64>(run, tile_prefix, st);
+    if constexpr (AK && BJ && std::is_same<TA, bf16>::value && std::is_same<TB, float>::value) {
+        return MOE_ERR_UNSUPPORTED;  // projections of whole quads: projection.cu
+    } else {
+        if (blocks(64, 128) >= 6 * 148 && !short_rows && g.N > 64)
+            return simt_launch<TA, TB, TC, true, true, AK, BJ, 64, 128, 8, 8, 16>(run, tile_prefix, st);
+        if (blocks(64, 64) >= 2 * 148 && !short_rows && !(run.part && g.N <= 32))
+            return simt_launch<TA, TB, TC, true, true, AK, BJ, 64, 64, 8, 4, 16>(run, tile_prefix, st);
+        if (blocks(32, 32) >= 148) return simt_launch<TA, TB, TC, true, true, AK, BJ, 32, 32, 4, 4, 32>(run, tile_prefix, st);
+        return simt_launch<TA, TB, TC, true, true, AK, BJ, 16, 16, 2, 2, 64>(run, tile_prefix, st);
+    }
 }
 
 // part: simt_wgrad_splits(M, N, nseg, rows) * nseg * M * N floats (mode 1, float results), or nullptr: no slices
