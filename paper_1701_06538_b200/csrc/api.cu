@@ -674,14 +674,20 @@ int32_t do_losses_bwd(const moe_config *c, const Dims &D, const float *importanc
 int32_t gate_weight_grads(const Dims &D, const void *x, const float *dlogit, const float *W, const float *W2, int64_t n,
                           float *dW, float *dW2, float *dX, float *part, cudaStream_t st, GateParts *parts_left = nullptr) {
     const int64_t cols = W2 ? 2 * n : n;
+    const GateProduct p = {x, D.act, (int32_t)D.d, (int32_t)n, 1, 1, dlogit, W, W2, dW, dW2, dX, D.T, nullptr, nullptr};
     SimtGemm g;
-    memset(&g, 0, sizeof(g));
-    g.a_row_div = 1;
-    g.ta = D.act == MOE_BF16 ? G_BF16 : G_F32; g.tb = G_F32; g.tc = G_F32;
-    g.A = x; g.B = dlogit; g.C = dW; g.C2 = dW2; g.c_split = n;
-    g.sa_i = 1; g.sa_k = D.d; g.sb_k = cols; g.sb_j = 1; g.sc_i = n;
-    g.mode = 1; g.offsets = nullptr; g.nseg = 1; g.M = D.d; g.N = cols; g.K = D.T;
-    MOE_TRY(launch_simt_gemm(g, nullptr, st, part, nullptr, parts_left));
+    if (gate_wgrad_supported(p)) {
+        MOE_TRY(launch_gate_wgrad(p, part, st, parts_left));
+    } else {
+        memset(&g, 0, sizeof(g));
+        g.a_row_div = 1;
+        g.ta = D.act == MOE_BF16 ? G_BF16 : G_F32; g.tb = G_F32; g.tc = G_F32;
+        g.A = x; g.B = dlogit; g.C = dW; g.C2 = dW2; g.c_split = n;
+        g.sa_i = 1; g.sa_k = D.d; g.sb_k = cols; g.sb_j = 1; g.sc_i = n;
+        g.mode = 1; g.offsets = nullptr; g.nseg = 1; g.M = D.d; g.N = cols; g.K = D.T;
+        MOE_TRY(launch_simt_gemm(g, nullptr, st, part, nullptr, parts_left));
+    }
+    if (gate_rows_supported(p)) return launch_gate_rows(p, nullptr, st);
     memset(&g, 0, sizeof(g));
     g.a_row_div = 1;
     g.ta = g.tb = g.tc = G_F32;
@@ -745,22 +751,32 @@ int32_t do_gate_bwd(const moe_config *c, const Dims &D, const void *x, const flo
         MOE_TRY(launch_gate_logit_grads(noise + lp, clean + lp, raw_noise + lp, w.H.idx_s, g_s, kth_vals + 2 * D.T,
                                         kth_idx + 2 * D.T, dg_s, dload + D.a, w.H.idx_p, P1, (int32_t)D.b,
                                         (int32_t)D.k2, w.dlogit_s, nullptr, nullptr, st));
+        const GateProduct p = {x, D.act, (int32_t)D.d, (int32_t)D.b, (int32_t)D.a, (int32_t)D.k1, w.dlogit_s, Wg + wp, Wnoise + wp, dWg + wp, dWnoise + wp,
+                               w.dX_sec, P1, w.H.offsets_p, w.H.perm_p};
         SimtGemm g;  // dW_s[i] = sum over the slots of group i of x[token]^T . dlogit[slot]
-        memset(&g, 0, sizeof(g));
-        g.ta = D.act == MOE_BF16 ? G_BF16 : G_F32; g.tb = G_F32; g.tc = G_F32;
-        g.A = x; g.B = w.dlogit_s; g.C = dWg + wp; g.C2 = dWnoise + wp; g.c_split = D.b;
-        g.sa_i = 1; g.sa_k = D.d; g.sb_k = 2 * D.b; g.sb_j = 1; g.sc_i = D.b;
-        g.mode = 1; g.offsets = w.H.offsets_p; g.nseg = (int32_t)D.a; g.M = D.d; g.N = 2 * D.b; g.K = P1; g.c_e = D.d * D.b;
-        g.a_row_index = w.H.perm_p; g.a_row_div = (int32_t)D.k1; g.b_row_index = w.H.perm_p;
-        MOE_TRY(launch_simt_gemm(g, w.H.tile_prefix, st, w.partials_s));
-        memset(&g, 0, sizeof(g));  // dX_sec[slot] = dlogit[slot] . [W_g | W_noise]_s[group]^T
-        g.ta = g.tb = g.tc = G_F32;
-        g.A = w.dlogit_s; g.B = Wg + wp; g.B2 = Wnoise + wp; g.b_split = D.b; g.b_k_contiguous = 1; g.C = w.dX_sec;
-        g.sa_i = 2 * D.b; g.sa_k = 1; g.sb_k = 1; g.sb_j = D.b; g.sc_i = D.d;
-        g.mode = 0; g.offsets = w.H.offsets_p; g.nseg = (int32_t)D.a; g.M = P1; g.N = D.d; g.K = 2 * D.b;
-        g.b_e = D.d * D.b;
-        g.a_row_index = w.H.perm_p; g.a_row_div = 1; g.c_row_index = w.H.perm_p;
-        MOE_TRY(launch_simt_gemm(g, w.H.tile_prefix, st));
+        if (gate_wgrad_supported(p)) {
+            MOE_TRY(launch_gate_wgrad(p, w.partials_s, st));
+        } else {
+            memset(&g, 0, sizeof(g));
+            g.ta = D.act == MOE_BF16 ? G_BF16 : G_F32; g.tb = G_F32; g.tc = G_F32;
+            g.A = x; g.B = w.dlogit_s; g.C = dWg + wp; g.C2 = dWnoise + wp; g.c_split = D.b;
+            g.sa_i = 1; g.sa_k = D.d; g.sb_k = 2 * D.b; g.sb_j = 1; g.sc_i = D.b;
+            g.mode = 1; g.offsets = w.H.offsets_p; g.nseg = (int32_t)D.a; g.M = D.d; g.N = 2 * D.b; g.K = P1; g.c_e = D.d * D.b;
+            g.a_row_index = w.H.perm_p; g.a_row_div = (int32_t)D.k1; g.b_row_index = w.H.perm_p;
+            MOE_TRY(launch_simt_gemm(g, w.H.tile_prefix, st, w.partials_s));
+        }
+        if (gate_rows_supported(p)) {
+            MOE_TRY(launch_gate_rows(p, w.H.tile_prefix, st));
+        } else {
+            memset(&g, 0, sizeof(g));  // dX_sec[slot] = dlogit[slot] . [W_g | W_noise]_s[group]^T
+            g.ta = g.tb = g.tc = G_F32;
+            g.A = w.dlogit_s; g.B = Wg + wp; g.B2 = Wnoise + wp; g.b_split = D.b; g.b_k_contiguous = 1; g.C = w.dX_sec;
+            g.sa_i = 2 * D.b; g.sa_k = 1; g.sb_k = 1; g.sb_j = D.b; g.sc_i = D.d;
+            g.mode = 0; g.offsets = w.H.offsets_p; g.nseg = (int32_t)D.a; g.M = P1; g.N = D.d; g.K = 2 * D.b;
+            g.b_e = D.d * D.b;
+            g.a_row_index = w.H.perm_p; g.a_row_div = 1; g.c_row_index = w.H.perm_p;
+            MOE_TRY(launch_simt_gemm(g, w.H.tile_prefix, st));
+        }
         if (sec) {
             *sec = {w.dX_sec, nullptr, (int32_t)D.k1};
             return MOE_OK;

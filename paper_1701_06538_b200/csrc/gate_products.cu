@@ -1,0 +1,298 @@
+// The two products of a gate's backward pass by FP32 multiply-adds (gates that the tensor-core contractions do not take: float tokens, widths that
+// are no multiple of 32, most levels of a hierarchy):
+//   dX[r] = dlogit[r] . [W_g | W_noise]^T      contraction over the logits, a few dozen
+//   dW    = x^T . dlogit                       contraction over the tokens, cut into slices
+// Narrow gates are small next to the latency of their loads: 5000 tokens x 512 features x 32 logits are 2 us of multiply-adds each. So the K blocks come
+// in by asynchronous copies, all in flight together or several ahead, sixteen bytes of a row at a time and as the rows lie in memory. Wider ones stay
+// with the float product of gemm_simt.cu (see gate_rows_supported). Every output of dX is one chain of multiply-adds in ascending order,
+// every slice of dW likewise.
+#include <string.h>
+
+#include <type_traits>
+
+#include "async_copy.cuh"
+#include "moe_internal.cuh"
+
+namespace moe {
+
+namespace {
+
+// lanes of a warp: 4 (rows) x 8 (columns)
+template <int BM, int BN, int TM, int TN, int BK, int S> struct RowsTile {
+    static constexpr int WARPS_M = BM / (4 * TM), WARPS_N = BN / (8 * TN), NT = 32 * WARPS_M * WARPS_N;
+    static constexpr int ROW_BYTES = BK * 4 + 16;  // the rows that a warp reads together stand in different banks
+    static constexpr int A_STAGE = BM * ROW_BYTES, STAGE = A_STAGE + BN * ROW_BYTES, SHARED = S * STAGE;
+};
+template <int BM, int BN, int TM, int TN, int BK, int S, int BLOCKS>
+__global__ void __launch_bounds__(RowsTile<BM, BN, TM, TN, BK, S>::NT, BLOCKS) gate_rows_kernel(const __grid_constant__ GateProduct p, const int32_t *__restrict__ tile_prefix) {
+    using Tile = RowsTile<BM, BN, TM, TN, BK, S>;
+    constexpr int NT = Tile::NT, ROW = BK / 4, QA = BM * ROW / NT, QB = BN * ROW / NT;
+    static_assert(QA * NT == BM * ROW && QB * NT == BN * ROW && TN % 2 == 0, "whole copies a thread, pairs of columns");
+    wait_previous_kernel();
+    extern __shared__ __align__(16) uint8_t stages[];
+    __shared__ int4 tile_at;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int64_t m0 = (int64_t)blockIdx.x * BM, m_end = p.rows;
+    int32_t group = 0;
+    if (p.offsets) {
+        const int4 at = segment_of_tile(tile_prefix, p.offsets, p.groups, blockIdx.x, &tile_at);
+        if (at.x < 0) return;
+        group = at.x;
+        m0 = at.y + (int64_t)at.w * BM;
+        m_end = at.z;
+    }
+    if (m0 >= m_end) return;
+    const int32_t n_at = blockIdx.y * BN, cols = p.W2 ? 2 * p.n : p.n;
+    const int64_t matrix = (int64_t)group * p.d * p.n;
+    const float *from_a[QA];
+    int64_t from_b[QB];
+#pragma unroll
+    for (int q = 0; q < QA; ++q) {
+        int64_t r = m0 + (tid + q * NT) / ROW;
+        if (r >= m_end) r = m0;  // (a row that is computed and dropped)
+        if (p.perm) r = p.perm[r];
+        from_a[q] = p.dlogit + r * cols;
+    }
+#pragma unroll
+    for (int q = 0; q < QB; ++q) {
+        const int32_t j = n_at + (tid + q * NT) / ROW;
+        from_b[q] = matrix + (int64_t)(j < p.d ? j : 0) * p.n;  // (a column that is computed and dropped)
+    }
+    const int blocks = (cols + BK - 1) / BK;
+    auto load = [&](int kb) {  // logits behind the last one are zero in both operands
+        uint8_t *to = stages + kb % S * Tile::STAGE;
+#pragma unroll
+        for (int q = 0; q < QA; ++q) {
+            const int id = tid + q * NT, k = kb * BK + id % ROW * 4;
+            copy16(to + id / ROW * Tile::ROW_BYTES + id % ROW * 16, k < cols ? from_a[q] + k : p.dlogit, k < cols);
+        }
+#pragma unroll
+        for (int q = 0; q < QB; ++q) {
+            const int id = tid + q * NT, k = kb * BK + id % ROW * 4;
+            copy16(to + Tile::A_STAGE + id / ROW * Tile::ROW_BYTES + id % ROW * 16,
+                   k >= cols ? p.W : k < p.n ? p.W + from_b[q] + k : p.W2 + from_b[q] + (k - p.n), k < cols);
+        }
+    };
+#pragma unroll
+    for (int s = 0; s < S - 1; ++s) {
+        if (s < blocks) load(s);
+        copies_commit();
+    }
+    const int tx = lane & 7, ty = lane >> 3;
+    const int row0 = warp % Tile::WARPS_M * 4 * TM + ty, col0 = warp / Tile::WARPS_M * 8 * TN + tx;  // rows row0 + 4 i, columns col0 + 8 j
+    float acc[TM][TN];
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) acc[i][j] = 0.0f;
+    for (int kb = 0; kb < blocks; ++kb) {
+        copies_wait<S - 2>();
+        __syncthreads();  // block kb is there for all, block kb - 1 is read by all
+        if (kb + S - 1 < blocks) load(kb + S - 1);
+        copies_commit();
+        const uint8_t *a = stages + kb % S * Tile::STAGE + row0 * Tile::ROW_BYTES, *b = stages + kb % S * Tile::STAGE + Tile::A_STAGE + col0 * Tile::ROW_BYTES;
+        const int steps = min(BK, cols - kb * BK);  // a multiple of four
+        for (int kk = 0; kk < steps; kk += 4) {
+            float4 av[TM], bv[TN];
+#pragma unroll
+            for (int i = 0; i < TM; ++i) av[i] = *reinterpret_cast<const float4 *>(a + 4 * i * Tile::ROW_BYTES + kk * 4);
+#pragma unroll
+            for (int j = 0; j < TN; ++j) bv[j] = *reinterpret_cast<const float4 *>(b + 8 * j * Tile::ROW_BYTES + kk * 4);
+#pragma unroll
+            for (int v = 0; v < 4; ++v)
+#pragma unroll
+                for (int i = 0; i < TM; ++i)
+#pragma unroll
+                    for (int j = 0; j < TN; j += 2)
+                        fma_two(acc[i][j], acc[i][j + 1], reinterpret_cast<const float *>(&av[i])[v], reinterpret_cast<const float *>(&bv[j])[v],
+                                reinterpret_cast<const float *>(&bv[j + 1])[v]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < TM; ++i) {
+        int64_t r = m0 + row0 + 4 * i;
+        if (r >= m_end) continue;
+        if (p.perm) r = p.perm[r];
+        float *to = p.dX + r * p.d + n_at + col0;
+#pragma unroll
+        for (int j = 0; j < TN; ++j)
+            if (n_at + col0 + 8 * j < p.d) to[8 * j] = acc[i][j];
+    }
+}
+
+// dW: a thread has four features, or eight (two quads 16 apart), and TN logits
+template <typename T, int BM, int BN, int TM, int TN, int BK, int S> struct WgradTile {
+    static constexpr int WARPS_M = BM / (4 * TM), WARPS_N = BN / (8 * TN), NT = 32 * WARPS_M * WARPS_N;
+    static constexpr int A_STAGE = BK * BM * (int)sizeof(T), STAGE = A_STAGE + BK * BN * 4, SHARED = S * STAGE;
+};
+template <typename T, int BM, int BN, int TM, int TN, int BK, int S, int BLOCKS>
+__global__ void __launch_bounds__(WgradTile<T, BM, BN, TM, TN, BK, S>::NT, BLOCKS) gate_wgrad_kernel(const __grid_constant__ GateProduct p, int32_t splits, float *__restrict__ part) {
+    using Tile = WgradTile<T, BM, BN, TM, TN, BK, S>;
+    constexpr int NT = Tile::NT, VK = 16 / sizeof(T), A_ROW = BM / VK, B_ROW = BN / 4, QA = BK * A_ROW / NT, QB = BK * B_ROW / NT;
+    static_assert(QA * NT == BK * A_ROW && QB * NT == BK * B_ROW, "whole copies a thread");
+    wait_previous_kernel();
+    extern __shared__ __align__(16) uint8_t stages[];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int32_t group = blockIdx.z / splits, slice = blockIdx.z % splits, cols = p.W2 ? 2 * p.n : p.n, m_at = blockIdx.x * BM, n_at = blockIdx.y * BN;
+    int64_t begin = p.offsets ? p.offsets[group] : 0, end = p.offsets ? p.offsets[group + 1] : p.rows;
+    const int64_t len = ((end - begin + splits - 1) / splits + BK - 1) / BK * BK;
+    begin += slice * len;
+    if (begin + len < end) end = begin + len;
+    const int count = (int)(end > begin ? end - begin : 0), blocks = (count + BK - 1) / BK;
+    // rows of a K block that this thread copies, fetched one block ahead where they are gathered
+    int32_t ra[QA], rb[QB];
+    auto fetch = [&](int kb) {
+#pragma unroll
+        for (int q = 0; q < QA; ++q) {
+            const int k = kb * BK + (tid + q * NT) / A_ROW;
+            ra[q] = k < count ? (p.perm ? p.perm[begin + k] : (int32_t)(begin + k)) : -1;
+        }
+#pragma unroll
+        for (int q = 0; q < QB; ++q) {
+            const int k = kb * BK + (tid + q * NT) / B_ROW;
+            rb[q] = k < count ? (p.perm ? p.perm[begin + k] : (int32_t)(begin + k)) : -1;
+        }
+    };
+    auto load = [&](int kb) {  // rows behind the last one are zero in both operands
+        uint8_t *to = stages + kb % S * Tile::STAGE;
+#pragma unroll
+        for (int q = 0; q < QA; ++q) {
+            const int id = tid + q * NT, m = m_at + id % A_ROW * VK;
+            const bool live = ra[q] >= 0 && m < p.d;
+            copy16(to + id * 16, live ? static_cast<const T *>(p.x) + (int64_t)(ra[q] / p.row_div) * p.d + m : static_cast<const T *>(p.x), live);
+        }
+#pragma unroll
+        for (int q = 0; q < QB; ++q) {
+            const int id = tid + q * NT, c = n_at + id % B_ROW * 4;
+            const bool live = rb[q] >= 0 && c < cols;
+            copy16(to + Tile::A_STAGE + id * 16, live ? p.dlogit + (int64_t)rb[q] * cols + c : p.dlogit, live);
+        }
+        fetch(kb + 1);
+    };
+    fetch(0);
+#pragma unroll
+    for (int s = 0; s < S - 1; ++s) {
+        if (s < blocks) load(s);
+        copies_commit();
+    }
+    const int tx = lane & 7, ty = lane >> 3, m0 = warp % Tile::WARPS_M * 4 * TM + ty * 4, c0 = warp / Tile::WARPS_M * 8 * TN + tx * TN;  // features m0 + i % 4 + 16 (i / 4)
+    float acc[TM][TN];
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) acc[i][j] = 0.0f;
+    for (int kb = 0; kb < blocks; ++kb) {
+        copies_wait<S - 2>();
+        __syncthreads();
+        if (kb + S - 1 < blocks) load(kb + S - 1);
+        copies_commit();
+        const T *a = reinterpret_cast<const T *>(stages + kb % S * Tile::STAGE) + m0;
+        const float *b = reinterpret_cast<const float *>(stages + kb % S * Tile::STAGE + Tile::A_STAGE) + c0;
+#pragma unroll 4
+        for (int k = 0; k < BK; ++k) {
+            float av[TM], bv[TN];
+#pragma unroll
+            for (int h = 0; h < TM / 4; ++h) {
+                if constexpr (sizeof(T) == 4) {
+                    *reinterpret_cast<float4 *>(av + 4 * h) = *reinterpret_cast<const float4 *>(a + k * BM + 16 * h);
+                } else {
+                    const uint2 w = *reinterpret_cast<const uint2 *>(a + k * BM + 16 * h);
+                    av[4 * h] = __uint_as_float(w.x << 16); av[4 * h + 1] = __uint_as_float(w.x & 0xffff0000u);
+                    av[4 * h + 2] = __uint_as_float(w.y << 16); av[4 * h + 3] = __uint_as_float(w.y & 0xffff0000u);
+                }
+            }
+            if constexpr (TN == 4) *reinterpret_cast<float4 *>(bv) = *reinterpret_cast<const float4 *>(b + k * BN);
+            else *reinterpret_cast<float2 *>(bv) = *reinterpret_cast<const float2 *>(b + k * BN);
+#pragma unroll
+            for (int i = 0; i < TM; ++i)
+#pragma unroll
+                for (int j = 0; j < TN; j += 2) fma_two(acc[i][j], acc[i][j + 1], av[i], bv[j], bv[j + 1]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < TM; ++i) {
+        const int32_t m = m_at + m0 + i % 4 + 16 * (i / 4), c = n_at + c0;
+        if (m >= p.d || c >= cols) continue;  // (cols is a multiple of four, TN of two)
+        float *to;
+        if (splits > 1) to = part + (((int64_t)slice * p.groups + group) * p.d + m) * cols + c;
+        else to = (c < p.n ? p.dW + c : p.dW2 + (c - p.n)) + ((int64_t)group * p.d + m) * p.n;
+#pragma unroll
+        for (int j = 0; j < TN; ++j) to[j] = acc[i][j];
+    }
+}
+
+template <int BM, int BN, int TM, int TN, int BK, int S, int BLOCKS> int32_t launch_rows(const GateProduct &p, int32_t *tile_prefix, cudaStream_t st) {
+    using Tile = RowsTile<BM, BN, TM, TN, BK, S>;
+    int64_t tiles = cdiv(p.rows, BM);
+    if (p.offsets) {
+        MOE_TRY(launch_tile_prefix(p.offsets, p.groups, BM, tile_prefix, st));
+        tiles += p.groups;
+    }
+    static PerDevice configured;
+    const auto kernel = gate_rows_kernel<BM, BN, TM, TN, BK, S, BLOCKS>;
+    if (!allow_shared(configured, kernel, Tile::SHARED)) return MOE_ERR_CUDA;
+    if (cdiv(p.d, BN) > 65535) return MOE_ERR_UNSUPPORTED;
+    launch_kernel(kernel, dim3((unsigned)tiles, (unsigned)cdiv(p.d, BN)), Tile::NT, Tile::SHARED, st, p, (const int32_t *)tile_prefix);
+    MOE_LAUNCHED();
+    return MOE_OK;
+}
+template <typename T, int BM, int BN, int TM, int TN, int BK, int S, int BLOCKS> int32_t launch_wgrad(const GateProduct &p, int32_t splits, float *part, cudaStream_t st) {
+    using Tile = WgradTile<T, BM, BN, TM, TN, BK, S>;
+    static PerDevice configured;
+    const auto kernel = gate_wgrad_kernel<T, BM, BN, TM, TN, BK, S, BLOCKS>;
+    if (!allow_shared(configured, kernel, Tile::SHARED)) return MOE_ERR_CUDA;
+    const int64_t cols = p.W2 ? 2 * (int64_t)p.n : p.n;
+    if (cdiv(cols, BN) > 65535 || (int64_t)p.groups * splits > 65535) return MOE_ERR_UNSUPPORTED;
+    launch_kernel(kernel, dim3((unsigned)cdiv(p.d, BM), (unsigned)cdiv(cols, BN), (unsigned)(p.groups * splits)), Tile::NT, Tile::SHARED, st, p, splits, part);
+    MOE_LAUNCHED();
+    return MOE_OK;
+}
+}  // namespace
+
+static bool whole_quads(const GateProduct &p) {
+    return p.n % 4 == 0 && aligned16(p.W) && (!p.W2 || aligned16(p.W2)) && aligned16(p.dlogit) && aligned16(p.x);
+}
+
+// Where the products below are faster than the float product of gemm_simt.cu; us, that way and this way, tokens x features x logits:
+//   dX: 256 x 64 x 16 4.1 2.4; 81 x 128 x 128 5.4 4.1 (16 x 16 tiles); 2085 x 256 x 32 5.7 5.0; 3001 x 320 x 40 9.7 7.9; 5000 x 512 x 32 14.8 12.1;
+//       15000 x 512 x 16 34.8 19.1; but 15000 x 128 x 72 16.3 20.8, 12000 x 256 x 128 30 44: with a wider contraction the multiply-adds count, of which
+//       eight rows and columns a thread from transposed tiles need fewer moves
+//   dW: 256 x 64 x 16 4.4 4.1, 15000 x 512 x 16 22.9 15.8 (64 x 16 tiles); 1000 x 512 x 24 6.2 4.4, 2085 x 256 x 32 6.3 4.6 (32 x 32, two warps);
+//       3001 x 320 x 40 9.2 7.3, 5000 x 512 x 32 11.5 9.2, 15000 x 128 x 72 17.7 15.5 (64 x 32); but 12000 x 256 x 128 26.8 28.6, 20000 x 1024 x 40 70 75
+bool gate_rows_supported(const GateProduct &p) {
+    const int32_t cols = p.W2 ? 2 * p.n : p.n;
+    if (!whole_quads(p) || cdiv(p.d, 16) > 65535) return false;
+    return p.rows < 512 ? cols <= 256 : cols <= 40 && 4 * cdiv(p.d, 64) * 64 <= 5 * (int64_t)p.d;
+}
+int32_t launch_gate_rows(const GateProduct &p, int32_t *tile_prefix, cudaStream_t st) {
+    if (p.rows == 0) return MOE_OK;
+    if (p.rows < 512) return launch_rows<16, 16, 2, 2, 32, 4, 8>(p, tile_prefix, st);
+    if (2 * (cdiv(p.rows, 64) + p.groups / 2) * cdiv(p.d, 64) >= 148) return launch_rows<64, 64, 8, 4, 32, 2, 4>(p, tile_prefix, st);
+    return launch_rows<32, 32, 4, 4, 32, 2, 8>(p, tile_prefix, st);
+}
+
+static bool few_blocks(const GateProduct &p, int32_t cols, int32_t splits) { return cdiv(p.d, 32) * cdiv(cols, 32) * p.groups * splits <= 2 * 148; }
+bool gate_wgrad_supported(const GateProduct &p) {
+    const int32_t cols = p.W2 ? 2 * p.n : p.n, splits = simt_wgrad_splits(p.d, cols, p.groups, p.rows);
+    if (!whole_quads(p) || cdiv(cols, 16) > 65535 || (int64_t)p.groups * splits > 65535) return false;
+    return cols <= 16 || few_blocks(p, cols, splits) || (cols <= 72 && p.d <= 512);
+}
+// part: simt_wgrad_splits(d, logits, groups, rows) * groups * d * logits floats
+int32_t launch_gate_wgrad(const GateProduct &p, float *part, cudaStream_t st, GateParts *parts_left) {
+    const int32_t cols = p.W2 ? 2 * p.n : p.n, splits = simt_wgrad_splits(p.d, cols, p.groups, p.rows);
+    auto run = [&](auto x) {
+        using T = decltype(x);
+        if (cols <= 16) return launch_wgrad<T, 64, 16, 4, 2, 32, 4, 4>(p, splits, part, st);
+        if (few_blocks(p, cols, splits)) return launch_wgrad<T, 32, 32, 4, 2, 32, 4, 4>(p, splits, part, st);
+        return launch_wgrad<T, 64, 32, 4, 4, 32, 4, 4>(p, splits, part, st);
+    };
+    MOE_TRY(p.act == MOE_BF16 ? run(bf16()) : run(float()));
+    if (splits == 1) return MOE_OK;
+    if (parts_left) {
+        *parts_left = {part, splits, p.d, cols, p.n, p.n, p.dW, p.dW2};
+        return MOE_OK;
+    }
+    return launch_slices_sum(part, splits, p.groups, p.d, cols, p.n, p.dW, p.dW2, st);
+}
+
+}  // namespace moe

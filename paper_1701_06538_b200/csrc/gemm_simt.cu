@@ -8,6 +8,8 @@
 // number of blocks it leaves (see pick_tile). Operand tiles go through registers into one of two shared-memory buffers
 // while the other one is used: one barrier per K block, the loads of a block are in flight during the arithmetic of
 // the one before, and the shared-memory reads of step k + 1 during the arithmetic of step k.
+#include <string.h>
+
 #include <algorithm>
 #include <type_traits>
 
@@ -480,6 +482,16 @@ static int32_t simt_pick_tile(SimtRun &run, bool vec_a, bool vec_b, int32_t *til
         if (blocks(32, 32) >= 148) return simt_launch<TA, TB, TC, true, true, AK, BJ, 32, 32, 4, 4, 32>(run, tile_prefix, st);
         return simt_launch<TA, TB, TC, true, true, AK, BJ, 16, 16, 2, 2, 64>(run, tile_prefix, st);
     }
+}
+
+int32_t launch_slices_sum(float *part, int32_t splits, int32_t groups, int32_t d, int32_t cols, int32_t n, float *dW, float *dW2, cudaStream_t st) {
+    SimtRun run;
+    memset(&run, 0, sizeof(run));
+    run.g.M = d; run.g.N = cols; run.g.nseg = groups; run.g.C = dW; run.g.C2 = dW2; run.g.c_split = n; run.g.sc_i = n; run.g.c_e = (int64_t)d * n;
+    run.splits = splits; run.part = part;
+    launch_kernel(simt_reduce_kernel, (unsigned)cdiv((int64_t)d * cols * groups, 256), 256, 0, st, run);
+    MOE_LAUNCHED();
+    return MOE_OK;
 }
 
 // part: simt_wgrad_splits(M, N, nseg, rows) * nseg * M * N floats (mode 1, float results), or nullptr: no slices

@@ -372,6 +372,23 @@ struct GateParts {
     int32_t nparts, d, cols, split, ld;
     float *dW, *dW2;
 };
+// The two products of a gate's backward pass (gate_products.cu). Rows [rows] are tokens, or slots (token = slot / row_div) in an order `perm` sorted by
+// group; the groups' matrices stand one behind the other
+struct GateProduct {
+    const void *x;
+    int32_t act, d, n, groups, row_div;
+    const float *dlogit;          // [rows, n or 2 n], not sorted
+    const float *W, *W2;          // [d, n] per group; W2: of the logits from n on, or nullptr
+    float *dW, *dW2, *dX;         // dX [rows, d], not sorted
+    int64_t rows;
+    const int32_t *offsets, *perm;  // nullptr: one group
+};
+bool gate_rows_supported(const GateProduct &p);  // whether to
+bool gate_wgrad_supported(const GateProduct &p);
+int32_t launch_gate_rows(const GateProduct &p, int32_t *tile_prefix, cudaStream_t st);
+int32_t launch_gate_wgrad(const GateProduct &p, float *part, cudaStream_t st, GateParts *parts_left = nullptr);
+// dW (and dW2) of every group = the slices' results [splits][groups][d][cols] added in double, in slice order (gemm_simt.cu)
+int32_t launch_slices_sum(float *part, int32_t splits, int32_t groups, int32_t d, int32_t cols, int32_t n, float *dW, float *dW2, cudaStream_t st);
 // Mode 1 over segments: K is the number of rows of all segments. part: simt_wgrad_splits(M, N, nseg, K) * nseg * M * N
 // floats let a product with few tiles be cut along its contraction (float results only)
 int32_t simt_wgrad_splits(int64_t M, int64_t N, int32_t nseg, int64_t K);

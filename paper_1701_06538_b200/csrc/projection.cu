@@ -10,6 +10,7 @@
 
 #include <type_traits>
 
+#include "async_copy.cuh"
 #include "moe_internal.cuh"
 
 namespace moe {
@@ -30,15 +31,6 @@ struct ProjectionArgs {
     int32_t *clear;              // status word, cleared if given
 };
 
-__device__ __forceinline__ void copy16(void *to, const void *from, bool live) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(to)), "l"(from), "r"(live ? 16 : 0) : "memory");
-}
-// two fused multiply-adds with one instruction (each rounded as fmaf rounds it): c += a * b
-__device__ __forceinline__ void fma_two(float &c0, float &c1, float a, float b0, float b1) {
-    asm("{\n .reg .b64 a, b, c;\n mov.b64 a, {%2, %2};\n mov.b64 b, {%3, %4};\n mov.b64 c, {%0, %1};\n"
-        " fma.rn.f32x2 c, a, b, c;\n mov.b64 {%0, %1}, c;\n}"
-        : "+f"(c0), "+f"(c1) : "f"(a), "f"(b0), "f"(b1));
-}
 // element v of sixteen bytes
 template <typename T> __device__ __forceinline__ float element(const uint4 &q, int v) {
     const uint32_t *w = reinterpret_cast<const uint32_t *>(&q);
@@ -112,7 +104,7 @@ __global__ void __launch_bounds__(ProjectionTile<T, BM, BN, TM, TN, BK, S>::NT, 
 #pragma unroll
     for (int s = 0; s < S - 1; ++s) {
         if (s < blocks) load(s);
-        asm volatile("cp.async.commit_group;" ::: "memory");
+        copies_commit();
     }
     const int tx = lane & 7, ty = lane >> 3;
     const int row0 = warp % Tile::WARPS_M * 4 * TM + ty, col0 = warp / Tile::WARPS_M * 8 * TN + tx * VN;  // rows row0 + 4 i, columns col0 + 32 (j / 4) + j % 4
@@ -122,10 +114,10 @@ __global__ void __launch_bounds__(ProjectionTile<T, BM, BN, TM, TN, BK, S>::NT, 
 #pragma unroll
         for (int j = 0; j < TN; ++j) acc[i][j] = 0.0f;
     for (int kb = 0; kb < blocks; ++kb) {
-        asm volatile("cp.async.wait_group %0;" ::"n"(S - 2) : "memory");
+        copies_wait<S - 2>();
         __syncthreads();  // block kb is there for all, block kb - 1 is read by all
         if (kb + S - 1 < blocks) load(kb + S - 1);
-        asm volatile("cp.async.commit_group;" ::: "memory");
+        copies_commit();
         const uint8_t *a = stages + kb % S * Tile::STAGE + row0 * Tile::ROW_BYTES;
         const float *b = reinterpret_cast<const float *>(stages + kb % S * Tile::STAGE + Tile::A_STAGE) + col0;
 #pragma unroll 2
