@@ -198,7 +198,7 @@ struct DispatchWs {
 // it may pick). Backward: those of the bias gradients' column sums, the order of the weight gradients' tiles.
 SegmentPlan make_plan(const moe_config *c, const Dims &D, int32_t *ws, bool backward) {
     SegmentPlan p = plan_at(ws, D.R, D.n);
-    if (tc_ffn_supported(*c)) {
+    if (tc_ffn_takes(*c)) {
         p.bm[0] = tc_row_tile(*c);
         if (backward && p.bm[0] != COLSUM_ROWS) p.bm[1] = COLSUM_ROWS;
         if (!backward || !tc_wgrad_sorted(*c)) {
@@ -500,10 +500,10 @@ int32_t do_dispatch(const Dims &D, const void *x, const int32_t *topk_idx, void 
     return launch_dispatch_rows(x, D.act, D.T, (int32_t)D.k, (int32_t)D.d, inv_perm, xs, st, sums);
 }
 
-SimtGemm base_gemm(const Dims &D) {
+SimtGemm base_gemm() {  // of float experts
     SimtGemm g;
     memset(&g, 0, sizeof(g));
-    g.ta = g.tb = g.tc = D.act == MOE_BF16 ? G_BF16 : G_F32;
+    g.ta = g.tb = g.tc = G_F32;
     g.a_row_div = 1;
     return g;
 }
@@ -522,22 +522,22 @@ int32_t do_expert_ffn(const moe_config *c, const Dims &D, const void *xs, const 
     const SegmentPlan plan = ready ? *ready : make_plan(c, D, w.plan, false);
     if (!ready) {
         SegmentMaps maps;
-        const bool tc = tc_ffn_supported(*c);
+        const bool tc = tc_ffn_takes(*c);
         if (tc) MOE_TRY(tc_segment_maps(*c, &maps, xs, hid, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr));
         PlanArgs args;
         fill_plan(&args, plan, (int32_t)D.n, D.R, clear, tc ? &maps : nullptr);
         MOE_TRY(launch_segment_plan(args, offsets, st));
     }
-    if (tc_ffn_supported(*c))
+    if (tc_ffn_takes(*c))
         return launch_tc_ffn(*c, xs, offsets, W1, b1, W2, b2, hid, ys, plan, status_word(ws_base), st, first_only, relu_bits);
     if (D.float_terms[0] && !first_only) return launch_float_ffn(*c, xs, offsets, W1, b1, W2, b2, hid, ys, plan, w.terms, status_word(ws_base), st);
-    SimtGemm g = base_gemm(D);  // hid = relu(xs.W1 + b1)
+    SimtGemm g = base_gemm();  // hid = relu(xs.W1 + b1)
     g.A = xs; g.B = W1; g.C = hid; g.bias = b1; g.relu = 1;
     g.sa_i = D.d; g.sa_k = 1; g.sb_k = D.h; g.sb_j = 1; g.sc_i = D.h;
     g.mode = 0; g.offsets = offsets; g.nseg = (int32_t)D.n; g.M = D.R; g.N = D.h; g.K = D.d; g.b_e = D.d * D.h;
     MOE_TRY(launch_simt_gemm(g, nullptr, st, nullptr, &plan));
     if (first_only) return MOE_OK;
-    g = base_gemm(D);  // ys = hid.W2 + b2
+    g = base_gemm();  // ys = hid.W2 + b2
     g.A = hid; g.B = W2; g.C = ys; g.bias = b2;
     g.sa_i = D.h; g.sa_k = 1; g.sb_k = D.d; g.sb_j = 1; g.sc_i = D.d;
     g.mode = 0; g.offsets = offsets; g.nseg = (int32_t)D.n; g.M = D.R; g.N = D.d; g.K = D.h; g.b_e = D.h * D.d;
@@ -604,7 +604,7 @@ int32_t do_expert_ffn_bwd(const moe_config *c, const Dims &D, const void *xs, co
     const ColumnSums db2s = db2_sums(D, dys, db2, offsets, w, plan);
     if (!db2_begun) MOE_TRY(launch_segment_colsum(db2s, st));
     MOE_TRY(finish(db2s, 0));
-    if (tc_ffn_supported(*c)) {
+    if (tc_ffn_takes(*c)) {
         BlockSums left = {};
         MOE_TRY(launch_tc_ffn_bwd(*c, xs, hid, dys, offsets, W1, W2, dxs, dW1, db1, dW2, w.dz, w.colsum, plan,
                                   status_word(ws_base), st, relu_bits, leave ? &left : nullptr));
@@ -621,24 +621,24 @@ int32_t do_expert_ffn_bwd(const moe_config *c, const Dims &D, const void *xs, co
         MOE_TRY(launch_segment_colsum(db1s, st));
         return finish(db1s, 1);
     }
-    SimtGemm g = base_gemm(D);  // dW2[e] = hid_e^T . dys_e
+    SimtGemm g = base_gemm();  // dW2[e] = hid_e^T . dys_e
     g.A = hid; g.B = dys; g.C = dW2;
     g.sa_i = 1; g.sa_k = D.h; g.sb_k = D.d; g.sb_j = 1; g.sc_i = D.d;
     g.mode = 1; g.offsets = offsets; g.nseg = n; g.M = D.h; g.N = D.d; g.c_e = D.h * D.d;
     MOE_TRY(launch_simt_gemm(g, nullptr, st, nullptr, &plan));
-    g = base_gemm(D);  // dz = (dys . W2[e]^T) * [hid > 0]
+    g = base_gemm();  // dz = (dys . W2[e]^T) * [hid > 0]
     g.A = dys; g.B = W2; g.C = w.dz; g.mask = hid;
     g.sa_i = D.d; g.sa_k = 1; g.sb_k = 1; g.sb_j = D.d; g.sc_i = D.h;
     g.mode = 0; g.offsets = offsets; g.nseg = n; g.M = D.R; g.N = D.h; g.K = D.d; g.b_e = D.h * D.d;
     MOE_TRY(launch_simt_gemm(g, nullptr, st, nullptr, &plan));
     MOE_TRY(launch_segment_colsum(db1s, st));
     MOE_TRY(finish(db1s, 1));
-    g = base_gemm(D);  // dW1[e] = xs_e^T . dz_e
+    g = base_gemm();  // dW1[e] = xs_e^T . dz_e
     g.A = xs; g.B = w.dz; g.C = dW1;
     g.sa_i = 1; g.sa_k = D.d; g.sb_k = D.h; g.sb_j = 1; g.sc_i = D.h;
     g.mode = 1; g.offsets = offsets; g.nseg = n; g.M = D.d; g.N = D.h; g.c_e = D.d * D.h;
     MOE_TRY(launch_simt_gemm(g, nullptr, st, nullptr, &plan));
-    g = base_gemm(D);  // dxs = dz . W1[e]^T
+    g = base_gemm();  // dxs = dz . W1[e]^T
     g.A = w.dz; g.B = W1; g.C = dxs;
     g.sa_i = D.h; g.sa_k = 1; g.sb_k = 1; g.sb_j = D.h; g.sc_i = D.d;
     g.mode = 0; g.offsets = offsets; g.nseg = n; g.M = D.R; g.N = D.d; g.K = D.h; g.b_e = D.d * D.h;
@@ -651,7 +651,7 @@ int32_t expert_ffn_bwd_stage(const moe_config *c, const Dims &D, const void *xs,
     const SegmentPlan plan = make_plan(c, D, cv.take<int32_t>(plan_ints(D.R, D.n)), true);
     const FfnBwdWs w(cv, D);
     SegmentMaps maps;
-    const bool tc = tc_ffn_supported(*c);
+    const bool tc = tc_ffn_takes(*c);
     if (tc) MOE_TRY(tc_segment_maps(*c, &maps, nullptr, nullptr, dys, w.dz, hid, dys, xs, w.dz));
     PlanArgs args;
     fill_plan(&args, plan, (int32_t)D.n, D.R, status_word(ws), tc ? &maps : nullptr);
@@ -1057,7 +1057,7 @@ static int32_t forward_impl(const moe_config *cfg, const void *x, const float *W
     const FfnWs ffn(cv, D);
     const SegmentPlan plan = make_plan(cfg, D, ffn.plan, false);
     SegmentMaps maps;
-    const bool tc = tc_ffn_supported(*cfg);
+    const bool tc = tc_ffn_takes(*cfg);
     if (tc)
         MOE_TRY(tc_segment_maps(*cfg, &maps, C.xs, C.hid ? C.hid : ffn.hid, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr));
     PlanArgs args;
@@ -1119,7 +1119,7 @@ static int32_t backward_impl(const moe_config *cfg, const void *dY, const void *
     const Cv2Job jobs[2] = {{C.importance, (int32_t)D.n, cfg->w_importance, B.dimp},
                             {C.load, (int32_t)D.n, cfg->w_load, D.hier ? B.dload_h : B.dload}};
     SegmentMaps maps;
-    const bool tc = tc_ffn_supported(*cfg);
+    const bool tc = tc_ffn_takes(*cfg);
     if (tc)
         MOE_TRY(tc_segment_maps(*cfg, &maps, C.hid ? nullptr : C.xs, nullptr, B.dys, B.ffn.dz, C.hid ? C.hid : B.again.hid, B.dys, C.xs, B.ffn.dz));
     PlanArgs args;

@@ -805,10 +805,10 @@ int32_t tc_make_map(CUtensorMap *tm, const void *base, int rank, const uint64_t 
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? MOE_OK : MOE_ERR_CUDA;
 }
-// rows x cols activations, K-major operand: box 64 (cols) x 128 (rows)
-int32_t tc_map_rows_kmajor(CUtensorMap *tm, const void *p, int64_t rows, int64_t cols) {
+// rows x cols activations, K-major operand: box 64 (cols) x box_rows
+int32_t tc_map_rows_kmajor(CUtensorMap *tm, const void *p, int64_t rows, int64_t cols, int box_rows) {
     const uint64_t dims[2] = {(uint64_t)cols, (uint64_t)rows}, str[1] = {(uint64_t)cols * 2};
-    const uint32_t box[2] = {64, BM};
+    const uint32_t box[2] = {64, (uint32_t)box_rows};
     return tc_make_map(tm, p, 2, dims, str, box);
 }
 // rows x cols activations, MN-major operand (contraction over rows): dims (64, rows, cols/64)
@@ -1042,7 +1042,7 @@ int32_t launch_tc_gate_bwd(const void *x, int64_t T, int32_t d, int32_t n, const
     {   // dX_gate: six cross terms of the two split operands, concatenated along the contraction
         CUtensorMap tmA, tmB;
         const bool pairs = T >= 256 * 74 && !(flags & MOE_FLAG_TC_ONE_CTA);  // enough 256-row tiles for every SM pair
-        MOE_TRY(tc_map_rows_kmajor(&tmA, dsplit, T, 3 * n2));
+        MOE_TRY(tc_map_rows_kmajor(&tmA, dsplit, T, 3 * n2, BM));
         if (pairs) MOE_TRY(tc_map_weight_kmajor(&tmB, wsplit, 1, d, 3 * n2, 128));
         else MOE_TRY(tc_map_weight_kmajor(&tmB, wsplit, 1, d, 3 * n2, BN));
         GemmParams p = default_params();
@@ -1074,7 +1074,7 @@ int32_t launch_tc_gate_fwd(const void *x, int64_t T, int32_t d, int32_t n, const
                            int32_t *status, cudaStream_t st) {
     const int32_t n2 = 2 * n;
     CUtensorMap tmA, tmB;
-    MOE_TRY(tc_map_rows_kmajor(&tmA, x, T, d));
+    MOE_TRY(tc_map_rows_kmajor(&tmA, x, T, d, BM));
     MOE_TRY(tc_map_weight_mnmajor(&tmB, wsplit, 1, 3 * (int64_t)d, n2, 128));
     GemmParams p = default_params();
     p.nseg = 1; p.N = n2; p.K = d; p.R = T; p.status = status;
@@ -1094,7 +1094,7 @@ int32_t launch_tc_gate_fwd_grouped(const void *xs_p, int64_t P1, int32_t d, int3
     const int32_t n2 = 2 * b;
     const bool pairs = tc_use_pairs(P1, a, flags, n2 > d ? n2 : d);
     CUtensorMap tmA, tmB;
-    MOE_TRY(tc_map_rows_kmajor(&tmA, xs_p, P1, d));
+    MOE_TRY(tc_map_rows_kmajor(&tmA, xs_p, P1, d, BM));
     {   // the group is the map's last coordinate (stride d rows), the precision term an offset of a * d rows along K
         const uint64_t dims[4] = {64, (uint64_t)3 * a * d, (uint64_t)(n2 / 64), (uint64_t)a};
         const uint64_t str[3] = {(uint64_t)n2 * 2, 128, (uint64_t)d * n2 * 2};
@@ -1141,7 +1141,7 @@ int32_t launch_tc_hier_secondary_bwd(const void *xs_p, const void *dsplit_s, voi
     }
     if (P1 > 0) {   // dX_sec[row] = dlogit[row] . [W_g | W_noise][group]^T, six cross terms
         CUtensorMap tmA, tmB;
-        MOE_TRY(tc_map_rows_kmajor(&tmA, dsplit_s, P1, 3 * n2));
+        MOE_TRY(tc_map_rows_kmajor(&tmA, dsplit_s, P1, 3 * n2, BM));
         MOE_TRY(tc_map_weight_kmajor(&tmB, wsplit_s, a, d, 3 * n2, BN));
         MOE_TRY(launch_tile_table(offsets_p, a, BM, P1, tile_prefix, st));
         GemmParams p = default_params();

@@ -1,6 +1,6 @@
 // Strided SIMT grouped GEMM in float accumulation. It serves gate projections whose widths are no whole quads (the others: projection.cu), float
-// layers of few rows or little work (the others: products_f32.cu), shapes the tensor-core kernels do not take, and the two dense
-// contractions of their gate backward.
+// layers of few rows or little work (the others: products_f32.cu), and the two dense contractions of the gate backward where neither the tensor
+// cores (ffn_tc.cu) nor gate_products.cu take them.
 //
 // Every output is one chain of fused multiply-adds over the contraction index in ascending order, starting from +0
 // (contractions cut into slices: one such chain per slice, the slices added in double). That is bound by the FP32
@@ -461,9 +461,7 @@ static int32_t simt_pick_tile(SimtRun &run, bool vec_a, bool vec_b, int32_t *til
     };
     const bool short_rows = g.mode == 0 && g.offsets && g.M <= 32 * (int64_t)g.nseg;  // segments of few rows: less padding
     if (!(vec_a && vec_b)) {
-        if constexpr (std::is_same<TC, bf16>::value) {  // expert products: widths are whole 16-byte vectors
-            return MOE_ERR_UNSUPPORTED;
-        } else if constexpr (AK && BJ) {
+        if constexpr (AK && BJ) {
             if (!vec_a) return MOE_ERR_UNSUPPORTED;  // activations have rows of whole 16-byte vectors
             if (2 * blocks(128, 64) >= 3 * 148)
                 return simt_launch<TA, TB, TC, true, false, AK, BJ, 128, 64, 8, 8, 16>(run, tile_prefix, st);
@@ -518,18 +516,15 @@ int32_t launch_simt_gemm(const SimtGemm &g_in, int32_t *tile_prefix, cudaStream_
         run.splits = simt_wgrad_splits(g.M, g.N, g.nseg, g.K);
         if (run.splits > 1) run.part = part;
     }
-    const bool fff = g.ta == G_F32 && g.tb == G_F32 && g.tc == G_F32, bbb = g.ta == G_BF16 && g.tb == G_BF16 && g.tc == G_BF16;
+    const bool fff = g.ta == G_F32 && g.tb == G_F32 && g.tc == G_F32;
     const bool bff = g.ta == G_BF16 && g.tb == G_F32 && g.tc == G_F32;
     if (ak && bj) {  // rows x weight [K, N]
         if (fff) return simt_pick_tile<float, float, float, true, true>(run, vec_a, vec_b, tile_prefix, st);
-        if (bbb) return simt_pick_tile<bf16, bf16, bf16, true, true>(run, vec_a, vec_b, tile_prefix, st);
         if (bff) return simt_pick_tile<bf16, float, float, true, true>(run, vec_a, vec_b, tile_prefix, st);
     } else if (ak) {  // rows x weight [N, K] read transposed
         if (fff) return simt_pick_tile<float, float, float, true, false>(run, vec_a, vec_b, tile_prefix, st);
-        if (bbb) return simt_pick_tile<bf16, bf16, bf16, true, false>(run, vec_a, vec_b, tile_prefix, st);
     } else if (bj) {  // contraction over rows
         if (fff) return simt_pick_tile<float, float, float, false, true>(run, vec_a, vec_b, tile_prefix, st);
-        if (bbb) return simt_pick_tile<bf16, bf16, bf16, false, true>(run, vec_a, vec_b, tile_prefix, st);
         if (bff) return simt_pick_tile<bf16, float, float, false, true>(run, vec_a, vec_b, tile_prefix, st);
     }
     return MOE_ERR_UNSUPPORTED;

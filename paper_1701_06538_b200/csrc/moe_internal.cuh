@@ -435,7 +435,8 @@ struct BackwardTail {
 constexpr int64_t TAIL_RIDE_MAX = 8 * 148;
 
 // ----------------------------------------------------------------------------- tensor-core experts (ffn_tc.cu)
-bool tc_ffn_supported(const moe_config &c);
+bool tc_ffn_supported(const moe_config &c);  // with mask bits
+bool tc_ffn_takes(const moe_config &c);
 // base maps of the operands that are given (nullptr: not wanted)
 int32_t tc_segment_maps(const moe_config &c, SegmentMaps *maps, const void *xs_rows, const void *hid_rows, const void *dys_rows,
                         const void *dz_rows, const void *hid_cols, const void *dys_cols, const void *xs_cols, const void *dz_cols);

@@ -68,6 +68,7 @@ constexpr int MAX_PRODUCTS = 2;
 struct Product {
     int32_t N, M;  // output columns; WGRAD: rows of the per-segment output
     int32_t tile_n, tiles_n, per_e, kblocks;  // columns of a tile (256 or 128), tiles beside each other, WGRAD: tiles of a segment, ROW_*: K blocks
+    int32_t last_steps;                       // ROW_*: K steps of 16 in the last K block
     Divisor by_tiles_n, by_per_e;
     bf16 *out;                 // ROW_*: [R, N]; WGRAD: [nseg, M, N]
     const bf16 *bias;          // [nseg, N]
@@ -146,9 +147,9 @@ __device__ __forceinline__ uint32_t positive_bits(const uint4 (&packed)[4]) {
 }
 // The bias values of a 64-column box, the same for every lane (broadcast loads). They are fetched one box ahead: the
 // first box's before the warp waits for its accumulator.
-__device__ __forceinline__ void bias_load(const bf16 *bias, uint4 (&out)[2][4]) {
+template <bool WHOLE> __device__ __forceinline__ void bias_load(const bf16 *bias, int32_t columns, uint4 (&out)[2][4]) {  // columns: that exist
 #pragma unroll
-    for (int q = 0; q < 8; ++q) out[q >> 2][q & 3] = reinterpret_cast<const uint4 *>(bias)[q];
+    for (int q = 0; q < 8; ++q) out[q >> 2][q & 3] = WHOLE || 8 * q < columns ? reinterpret_cast<const uint4 *>(bias)[q] : make_uint4(0u, 0u, 0u, 0u);
 }
 // mask bits of a lane's row, 128 columns from col0 on (two boxes), as far as the row has them
 __device__ __forceinline__ void keep_load(const Product &p, int64_t row, int32_t col0, uint2 (&keep)[2]) {
@@ -160,7 +161,7 @@ __device__ __forceinline__ void keep_load(const Product &p, int64_t row, int32_t
 // eight values of a load into a byte, and passes the bytes through `box` to the lanes that own the rows.
 __device__ __forceinline__ void keep_from_mask(const Product &p, int64_t row0, int32_t rows_valid, int32_t col0, int lane, uint8_t *box, uint2 (&keep)[2]) {
     const int32_t col = col0 + (lane & 15) * 8;
-    const bool in_row = col < p.N;  // N is a multiple of 64
+    const bool in_row = col < p.N;  // N is a multiple of eight
     const bf16 *src = p.mask + row0 * p.N + col;
     const __nv_bfloat162 zero = __float2bfloat162_rn(0.0f);
     uint4 v[16];  // all in flight together: the accumulator's registers are free yet
@@ -205,7 +206,7 @@ struct BoxArgs {
     uint2 keep;                 // mask bits
     bool have_acc;
 };
-template <int EPI, int BOXES, typename Release>
+template <int EPI, int BOXES, bool WHOLE, typename Release>
 __device__ __forceinline__ void epilogue_box(const Product &p, int lane, const BoxArgs &b, uint4 (&bias)[2][4], Release release) {
     uint32_t v[2][32];
     if (b.have_acc) {
@@ -223,7 +224,7 @@ __device__ __forceinline__ void epilogue_box(const Product &p, int lane, const B
     uint4 packed[2][4];
 #pragma unroll
     for (int u = 0; u < 2; ++u) pack32<EPI>(v[u], bias[u], packed[u], u ? b.keep.y : b.keep.x);
-    if (epi_bias(EPI) && b.next_bias) bias_load(b.next_bias, bias);
+    if (epi_bias(EPI) && b.next_bias) bias_load<WHOLE>(b.next_bias, p.N - b.col0 - 64, bias);
     if (EPI == EPI_BIAS_RELU && p.bits_out && row_ok)
         *reinterpret_cast<uint2 *>(p.bits_out + out_row * (p.N >> 5) + (b.col0 >> 5)) =
             make_uint2(positive_bits(packed[0]), positive_bits(packed[1]));
@@ -253,15 +254,22 @@ __device__ __forceinline__ void epilogue_box(const Product &p, int lane, const B
                 s0 += __uint_as_float(w0 << 16); s1 += __uint_as_float(w0 & 0xffff0000u);
                 u0 += __uint_as_float(w1 << 16); u1 += __uint_as_float(w1 & 0xffff0000u);
             }
-            *reinterpret_cast<float2 *>(p.colsum_part + b.colsum_row * p.N + b.col0 + 2 * lane) = make_float2(s0 + u0, s1 + u1);
+            if (WHOLE || b.col0 + 2 * lane < p.N)
+                *reinterpret_cast<float2 *>(p.colsum_part + b.colsum_row * p.N + b.col0 + 2 * lane) = make_float2(s0 + u0, s1 + u1);
             __syncwarp();  // read before the next box overwrites this one
         }
         return;
     }
     if (row_ok) {
         uint4 *dst = reinterpret_cast<uint4 *>(p.out + b.out_off + out_row * p.N + b.col0);
+        if (WHOLE) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) st_global_32B(dst + 2 * q, packed[q >> 1][2 * (q & 1)], packed[q >> 1][2 * (q & 1) + 1]);
+            for (int q = 0; q < 4; ++q) st_global_32B(dst + 2 * q, packed[q >> 1][2 * (q & 1)], packed[q >> 1][2 * (q & 1) + 1]);
+        } else {
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if (b.col0 + 8 * q < p.N) dst[q] = packed[q >> 2][q & 3];
+        }
     }
     if (epi_keep(EPI)) {  // sums of the rounded values, rows past the segment end count as 0; the whole warp: shuffles
 #pragma unroll
@@ -273,7 +281,8 @@ __device__ __forceinline__ void epilogue_box(const Product &p, int lane, const B
                 a[2 * j] = row_ok ? __uint_as_float(pw[j] << 16) : 0.0f;
                 a[2 * j + 1] = row_ok ? __uint_as_float(pw[j] & 0xffff0000u) : 0.0f;
             }
-            p.colsum_part[b.colsum_row * p.N + b.col0 + 32 * u + lane] = warp_column_sums(a, lane);
+            const float s = warp_column_sums(a, lane);
+            if (WHOLE || b.col0 + 32 * u + lane < p.N) p.colsum_part[b.colsum_row * p.N + b.col0 + 32 * u + lane] = s;
         }
     }
 }
@@ -381,7 +390,9 @@ template <bool PAIR, int NST> constexpr int box_count() { return NST == (PAIR ? 
 template <bool PAIR, int NST> constexpr int data_bytes() { return NST * stage_bytes<PAIR>() + 8 * 4096 * box_count<PAIR, NST>(); }
 template <bool PAIR, int NST> constexpr int shared_bytes() { return data_bytes<PAIR, NST>() + 1024 /*alignment*/ + 384 /*barriers, ring*/; }
 
-template <bool PAIR, int NST, int SET>
+// WHOLE: all widths are multiples of 64. Otherwise of eight, and one CTA: MN-major operands come in chunk by chunk through maps of the whole width, what lies
+// behind it reads as zero and is not stored.
+template <bool PAIR, int NST, int SET, bool WHOLE>
 __global__ void __maxnreg__(most_registers(SET)) expert_products_kernel(const __grid_constant__ ProductMaps maps, const __grid_constant__ Products P) {
     constexpr bool SHORT = !PAIR && NST == 3;
     constexpr int RING = ring_slots<SHORT>(), BOXES = box_count<PAIR, NST>(), STAGE = stage_bytes<PAIR>(), TM = tile_rows<PAIR>();
@@ -472,8 +483,13 @@ __global__ void __maxnreg__(most_registers(SET)) expert_products_kernel(const __
                         const bool tail = ragged && kb == kblocks - 1;
                         const int r = t.row0 + kb * BK;
                         stage([&](uint32_t a, uint32_t b, uint32_t bar) {
-                            load_3d(a, tail ? p.seg_a + t.e : tm_a, bar, 0, r, ca);
-                            load_3d(b, tail ? p.seg_b + t.e : tm_b, bar, 0, r, cb);
+                            if (WHOLE) {
+                                load_3d(a, tail ? p.seg_a + t.e : tm_a, bar, 0, r, ca);
+                                load_3d(b, tail ? p.seg_b + t.e : tm_b, bar, 0, r, cb);
+                            } else {
+                                for (int c = 0; c < BM / 64; ++c) tma_load_2d(a + c * (BK * 128), tm_a, bar, t.m0 + 64 * c, r);
+                                for (int c = 0; c < p.tile_n / 64; ++c) tma_load_2d(b + c * (BK * 128), tm_b, bar, t.n0 + 64 * c, r);
+                            }
                         });
                     }
                 } else {
@@ -487,7 +503,8 @@ __global__ void __maxnreg__(most_registers(SET)) expert_products_kernel(const __
                         for (int kb = 0; kb < kblocks && ok; ++kb)
                             stage([&](uint32_t a, uint32_t b, uint32_t bar) {
                                 load_2d(a, tm_a, bar, kb * BK, row);
-                                load_4d(b, tm_b, bar, 0, kb * BK, cb, t.e);
+                                if (WHOLE) load_4d(b, tm_b, bar, 0, kb * BK, cb, t.e);
+                                else for (int c = 0; c < p.tile_n / 64; ++c) tma_load_3d(b + c * (BK * 128), tm_b, bar, t.n0 + 64 * c, kb * BK, t.e);
                             });
                     } else {
                         const int cb = t.n0 + 128 * (int)rank;
@@ -524,8 +541,8 @@ __global__ void __maxnreg__(most_registers(SET)) expert_products_kernel(const __
                 const int kblocks = wgrad ? (t.row_end - t.row0 + BK - 1) / BK : p.kblocks;
                 if (kblocks == 0) return;  // empty segment (WGRAD): the epilogue writes zeros
                 constexpr int a_mn = wgrad ? 1 : 0, b_mn = KIND == ROW_BK ? 0 : 1;
-                // one CTA: columns behind the output's are not computed (N is a multiple of 64)
-                const uint32_t idesc = PAIR ? make_idesc2(a_mn, b_mn) : make_idesc(a_mn, b_mn, min(p.tile_n, p.N - t.n0));
+                // one CTA: columns behind the output's are not computed
+                const uint32_t idesc = PAIR ? make_idesc2(a_mn, b_mn) : make_idesc(a_mn, b_mn, min(p.tile_n, WHOLE ? p.N - t.n0 : (p.N - t.n0 + 15) & ~15));
                 // a K step of 16 advances the start address (low descriptor bits, in 16-byte units) by 32 bytes in a
                 // K-major tile and by 16 rows of 128 bytes in an MN-major one; the sum never leaves the address field
                 constexpr uint64_t a_step = a_mn ? (16 * 128) >> 4 : 32 >> 4, b_step = b_mn ? (16 * 128) >> 4 : 32 >> 4;
@@ -540,7 +557,7 @@ __global__ void __maxnreg__(most_registers(SET)) expert_products_kernel(const __
                     tc_fence_after();
                     const uint32_t a_src = base + s * STAGE, b_src = a_src + A_BYTES;
                     // K steps of 16 rows to issue for this block: none that lies behind the segment's end
-                    const int ksteps = wgrad && kb == kblocks - 1 ? (tail + 15) / 16 : BK / 16;
+                    const int ksteps = kb < kblocks - 1 || (WHOLE && !wgrad) ? BK / 16 : wgrad ? (tail + 15) / 16 : p.last_steps;
                     if (!PAIR && wgrad && kb == kblocks - 1 && !p.seg_a && ksteps * 16 > tail) {
                         // Without the segments' own maps (see wgrad_uses_maps) the rows behind the end, up to the end of the step that holds
                         // it, are the next segment's: zeroed in A AND in B (0 x finite = 0 would do for finite data; both keep a
@@ -631,7 +648,7 @@ __global__ void __maxnreg__(most_registers(SET)) expert_products_kernel(const __
                 const Product &p = P.p[I];
                 const bool have_acc = !wgrad || t.row_end > t.row0;
                 const int32_t first = t.n0 + half * (p.tile_n / 2);
-                const int boxes = min(p.tile_n / 128, max(0, (p.N - first) / 64));  // N is a multiple of 64
+                const int boxes = min(p.tile_n / 128, max(0, (WHOLE ? p.N - first : p.N - first + 63) / 64));
                 BoxArgs b;
                 b.tm_out = &maps.out[I];
                 b.out_off = wgrad ? (int64_t)t.e * p.M * p.N : 0;
@@ -644,7 +661,7 @@ __global__ void __maxnreg__(most_registers(SET)) expert_products_kernel(const __
                 const bf16 *bias_at = nullptr;
                 if (epi_bias(EPI)) {
                     bias_at = p.bias + (int64_t)t.e * p.N + first;
-                    if (boxes > 0) bias_load(bias_at, bias);
+                    if (boxes > 0) bias_load<WHOLE>(bias_at, p.N - first, bias);
                 }
                 uint2 keep[2] = {make_uint2(0u, 0u), make_uint2(0u, 0u)};
                 if (EPI == EPI_KEEP_BITS && lane < b.rows_valid) keep_load(p, b.row0 + lane, first, keep);
@@ -669,7 +686,7 @@ __global__ void __maxnreg__(most_registers(SET)) expert_products_kernel(const __
                     b.keep = u ? keep[1] : keep[0];
                     b.box = boxes_at + (BOXES > 1 ? turn * 4096 : 0);
                     if (b.rows_valid >= 32) turn ^= 1;  // (else nothing is stored from the box)
-                    epilogue_box<EPI, BOXES>(p, lane, b, bias, [&]() { if (u + 1 == boxes) release(); });
+                    epilogue_box<EPI, BOXES, WHOLE>(p, lane, b, bias, [&]() { if (u + 1 == boxes) release(); });
                 }
                 if (have_acc) {
                     if (boxes == 0) release();
@@ -708,7 +725,8 @@ bool use_pairs(int64_t R, int32_t nseg, int32_t flags, int32_t cols) {
     if ((flags & MOE_FLAG_TC_ONE_CTA) || cdiv(R, 256) * cdiv(cols, 256) <= tc_sm_count()) return false;
     return R / (nseg > 0 ? nseg : 1) >= 384;
 }
-bool use_pairs(const moe_config &c) { return use_pairs((int64_t)c.T * c.k, c.n, c.flags, c.d > c.h ? c.d : c.h); }
+bool whole(const moe_config &c) { return c.d % 64 == 0 && c.h % 64 == 0; }
+bool use_pairs(const moe_config &c) { return whole(c) && use_pairs((int64_t)c.T * c.k, c.n, c.flags, c.d > c.h ? c.d : c.h); }
 // one or two K blocks in the average segment of a weight gradient
 bool short_segments(int64_t R, int32_t nseg) { return R < 128 * (int64_t)nseg; }
 
@@ -721,7 +739,7 @@ bool wgrad_uses_maps(const moe_config &c) {
     const int64_t R = (int64_t)c.T * c.k;
     const int32_t wide = c.d > c.h ? c.d : c.h, narrow = c.d > c.h ? c.h : c.d;
     if (use_pairs(c)) return true;
-    if (short_segments(R, c.n)) return false;
+    if (!whole(c) || short_segments(R, c.n)) return false;
     return c.n * cdiv(narrow, BM) * cdiv(wide, BN) >= 4 * (int64_t)tc_sm_count();
 }
 // The rows of a row product behind a segment's end are read and dropped, or, through the segment's own map, not read. That saves bytes
@@ -732,13 +750,13 @@ bool wgrad_uses_maps(const moe_config &c) {
 bool rows_use_maps(const moe_config &c) {
     const int64_t R = (int64_t)c.T * c.k;
     const bool pairs = use_pairs(c);
-    if (!pairs && !short_segments(R, c.n)) return false;
+    if (!whole(c) || (!pairs && !short_segments(R, c.n))) return false;
     return (cdiv(R, pairs ? 256 : BM) + c.n) * cdiv(c.d > c.h ? c.d : c.h, BN) >= 32 * (int64_t)(pairs ? tc_sm_count() / 2 : tc_sm_count());
 }
 
-template <bool PAIR, int NST, int SET> int32_t launch_products_as(const ProductMaps &maps, const Products &P, int64_t tiles, cudaStream_t st) {
+template <bool PAIR, int NST, int SET, bool WHOLE> int32_t launch_products_as(const ProductMaps &maps, const Products &P, int64_t tiles, cudaStream_t st) {
     static PerDevice slots;  // CTAs or pairs that run at once
-    const auto kernel = expert_products_kernel<PAIR, NST, SET>;
+    const auto kernel = expert_products_kernel<PAIR, NST, SET, WHOLE>;
     constexpr int SHARED = shared_bytes<PAIR, NST>();
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
@@ -789,7 +807,7 @@ class ProductList {
     // out [R, N] = epilogue(A [R, K] . W[e]), W[e] as [K, N], or [N, K] read transposed
     int32_t row(Product **made, const void *A, const void *W, bool transposed, int32_t N, int32_t K, void *out, SegmentMap seg) {
         Product &p = P.p[count];
-        p.N = N; p.kblocks = K / BK;
+        p.N = N; p.kblocks = (int32_t)cdiv(K, BK); p.last_steps = (int32_t)cdiv(K - (p.kblocks - 1) * BK, 16);
         // Half as wide tiles where whole ones leave half of the SMs without: a handful of tokens, whose time is one tile's loads
         const int64_t row_tiles = cdiv(R, tm) + imin(c.n, R);
         p.tile_n = !pairs && N > 128 && 2 * row_tiles * cdiv(N, BN) <= tc_sm_count() ? 128 : BN;
@@ -798,8 +816,9 @@ class ProductList {
         p.out = (bf16 *)out;
         if (row_maps) p.seg_a = plan.maps_of(seg);
         const int box_n = pairs ? 128 : p.tile_n;
-        MOE_TRY(tc_map_rows_kmajor(&maps.a[count], A, R, K));
+        MOE_TRY(tc_map_rows_kmajor(&maps.a[count], A, R, K, BM));
         if (transposed) MOE_TRY(tc_map_weight_kmajor(&maps.b[count], W, c.n, N, K, box_n));
+        else if (!whole(c)) MOE_TRY(tc_map_weight_kmajor(&maps.b[count], W, c.n, K, N, BK));  // (64 columns of 64 rows)
         else MOE_TRY(tc_map_weight_mnmajor(&maps.b[count], W, c.n, K, N, box_n));
         MOE_TRY(map_out_boxes(&maps.out[count], out, R, N));
         add((cdiv(R, tm) + c.n) * p.tiles_n);
@@ -815,9 +834,14 @@ class ProductList {
         p.by_tiles_n = Divisor::of(p.tiles_n); p.by_per_e = Divisor::of(p.per_e);
         p.out = (bf16 *)out;
         if (wgrad_maps) { p.seg_a = plan.maps_of(seg_a); p.seg_b = plan.maps_of(seg_b); }
-        MOE_TRY(tc_map_rows_mnmajor(&maps.a[count], A, R, M, 2));
-        MOE_TRY(tc_map_rows_mnmajor(&maps.b[count], B, R, N, pairs ? 2 : BN / 64));
-        // the experts' matrices as one tall matrix (a 32-row box never straddles two: M is a multiple of 64)
+        if (whole(c)) {
+            MOE_TRY(tc_map_rows_mnmajor(&maps.a[count], A, R, M, 2));
+            MOE_TRY(tc_map_rows_mnmajor(&maps.b[count], B, R, N, pairs ? 2 : BN / 64));
+        } else {
+            MOE_TRY(tc_map_rows_kmajor(&maps.a[count], A, R, M, BK));
+            MOE_TRY(tc_map_rows_kmajor(&maps.b[count], B, R, N, BK));
+        }
+        // the experts' matrices as one tall matrix (a box that is stored whole has 32 rows of its expert)
         MOE_TRY(map_out_boxes(&maps.out[count], out, (int64_t)c.n * M, N));
         add((int64_t)c.n * p.per_e);
         return MOE_OK;
@@ -828,15 +852,19 @@ class ProductList {
         // 6680); with few the thread that draws is ahead by a good part of them (256 x 78 rows, 10 and 28 a CTA: 576, dealt 570; a step of
         // 256 x 188 rows 1289, dealt 1273)
         P.counter = pairs || tiles > 64 * (int64_t)tc_sm_count() ? drawn : nullptr;
-        if (pairs) return launch_products_as<true, 6, SET>(maps, P, tiles, st);
+        if (!whole(c)) {
+            if constexpr (SET != SET_DZ_DW2) return launch_products_as<false, 4, SET, false>(maps, P, tiles, st);
+            return MOE_ERR_UNSUPPORTED;  // (no bits without whole words)
+        }
+        if (pairs) return launch_products_as<true, 6, SET, true>(maps, P, tiles, st);
         // Weight gradients of one or two K blocks a tile last as long as their epilogue, 1100 cycles a box, 420 of them waiting until the
         // store before had read the box out: a warp's boxes take turns in two 4 KiB pieces, for one operand stage less (4096 experts x
         // 64 rows, a product: 1056 and 1087 us -> 981 to 1012 and 1056 to 1076, 256 x 78 rows 61 -> 58). With three K blocks a tile the stage is
         // worth more (256 x 188 rows 83 -> 86). Sixteen epilogue warps, eight an accumulator, were no faster than the second box.
         if constexpr (set_size(SET) > 1) {
-            if (short_segments(R, c.n)) return launch_products_as<false, 3, SET>(maps, P, tiles, st);
+            if (short_segments(R, c.n)) return launch_products_as<false, 3, SET, true>(maps, P, tiles, st);
         }
-        return launch_products_as<false, 4, SET>(maps, P, tiles, st);
+        return launch_products_as<false, 4, SET, true>(maps, P, tiles, st);
     }
 
   private:
@@ -852,6 +880,11 @@ bool tc_ffn_supported(const moe_config &c) {
     return c.act == MOE_BF16 && c.d % 64 == 0 && c.h % 64 == 0 && c.d >= 64 && c.h >= 64;
 }
 
+// All bf16 layers: their widths are multiples of eight (a configuration's rows are whole 16-byte vectors). us a step by FP32 multiply-adds, which widths that
+// are no multiples of 64 had, and this way: 64 experts x 200 rows of 72 x 2056 1257, 238; 20 x 300 of 120 x 1000 396, 98; 32 x 500 of 200 x 200 452, 135;
+// 200 x 2 of 136 x 264 245, 118; 16 x 40 of 8 x 16 73, 67; forward calls of a few tokens, bound by their launches: 32 x 72 x 136 30.7, 31.8.
+bool tc_ffn_takes(const moe_config &c) { return c.act == MOE_BF16; }
+
 int32_t tc_segment_maps(const moe_config &c, SegmentMaps *maps, const void *xs_rows, const void *hid_rows, const void *dys_rows,
                         const void *dz_rows, const void *hid_cols, const void *dys_cols, const void *xs_cols, const void *dz_cols) {
     memset(maps, 0, sizeof(*maps));
@@ -859,7 +892,7 @@ int32_t tc_segment_maps(const moe_config &c, SegmentMaps *maps, const void *xs_r
     auto add = [&](SegmentMap which, const void *p, int64_t cols, int chunks) -> int32_t {
         if (!p) return MOE_OK;
         maps->made[which] = 1;
-        return chunks ? tc_map_rows_mnmajor(&maps->base[which], p, rows, cols, chunks) : tc_map_rows_kmajor(&maps->base[which], p, rows, cols);
+        return chunks ? tc_map_rows_mnmajor(&maps->base[which], p, rows, cols, chunks) : tc_map_rows_kmajor(&maps->base[which], p, rows, cols, BM);
     };
     if (rows_use_maps(c)) {
         MOE_TRY(add(MAP_XS_ROWS, xs_rows, c.d, 0));

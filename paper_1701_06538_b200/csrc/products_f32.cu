@@ -434,7 +434,7 @@ struct FloatCall {
         const int64_t tiles = (cdiv(R, F_TILE) + c.n) * p.tiles_n;
         if (tiles >= (int64_t)1 << 30) return MOE_ERR_UNSUPPORTED;
         p.total = (int32_t)tiles;
-        MOE_TRY(tc_map_rows_kmajor(&L->row_a, a, R, 3 * (int64_t)K));
+        MOE_TRY(tc_map_rows_kmajor(&L->row_a, a, R, 3 * (int64_t)K, F_TILE));
         if (ROW == ROW_BMN) return tc_map_weight_mnmajor(&L->row_b, b, c.n, K, 3 * (int64_t)N, F_TILE);
         return tc_map_weight_kmajor(&L->row_b, b, c.n, N, 3 * (int64_t)K, F_TILE);
     }

@@ -129,9 +129,10 @@ template <int COLS> __device__ __forceinline__ void block_sums_final(const Block
     }
     for (int32_t c = 0; c < COLS; c += 64) {
         const int32_t j = slab * COLS + c + cl * 4;
-        if (COLS > 64 && j >= N) break;  // N is a multiple of 64: all threads alike
+        if (COLS > 64 && slab * COLS + c >= N) break;
+        const bool in_row = j < N;  // (N is a multiple of four)
         float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        int32_t b = b0 + q;
+        int32_t b = in_row ? b0 + q : b1;
         for (; b + 16 * 7 < b1; b += 16 * 8) {
             float4 v[8];
 #pragma unroll
@@ -146,7 +147,7 @@ template <int COLS> __device__ __forceinline__ void block_sums_final(const Block
         if (COLS > 64) __syncthreads();  // sh may still be read for the columns before
         sh[q][cl] = s;
         __syncthreads();
-        if (q == 0) {
+        if (q == 0 && in_row) {
             float4 t = sh[0][cl];
 #pragma unroll
             for (int u = 1; u < 16; ++u) { t.x += sh[u][cl].x; t.y += sh[u][cl].y; t.z += sh[u][cl].z; t.w += sh[u][cl].w; }

@@ -265,7 +265,7 @@ __device__ __forceinline__ void mbar_arrive_cluster_addr(uint32_t cluster_addr) 
 
 // host (ffn_tc.cu): bf16 tensor maps with 128-byte swizzle; dims innermost first, strides (bytes) for dims 1.., box per dim
 int32_t tc_make_map(CUtensorMap *tm, const void *base, int rank, const uint64_t *dims, const uint64_t *strides, const uint32_t *box);
-int32_t tc_map_rows_kmajor(CUtensorMap *tm, const void *p, int64_t rows, int64_t cols);
+int32_t tc_map_rows_kmajor(CUtensorMap *tm, const void *p, int64_t rows, int64_t cols, int box_rows);
 int32_t tc_map_rows_mnmajor(CUtensorMap *tm, const void *p, int64_t rows, int64_t cols, int chunks);
 int32_t tc_map_weight_mnmajor(CUtensorMap *tm, const void *p, int64_t n, int64_t K, int64_t N, int tile_n);
 int32_t tc_map_weight_kmajor(CUtensorMap *tm, const void *p, int64_t n, int64_t N, int64_t K, int tile_n);

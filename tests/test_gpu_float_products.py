@@ -70,4 +70,4 @@ def test_values_that_are_no_numbers():
             assert ((have == want) | finite | np.isnan(want) | wide).all() and ((have == want) | np.isfinite(have) | np.isnan(have)).all()
             sound = finite & ~wide
             scale = np.abs(want) + np.sqrt(np.mean(np.square(want[sound].astype(np.float64))))
-            assert (np.abs(have - want)[sound] <= 1e-5 * scale[sound]).all()
+            assert (np.abs(have[sound] - want[sound]) <= 1e-5 * scale[sound]).all()
