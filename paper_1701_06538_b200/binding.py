@@ -89,22 +89,46 @@ def act_dtype(cfg: moe_config):
 
 def _p(t):
     if t is None:
-        return ctypes.c_void_p(0)
+        return None
     assert t.is_cuda and t.is_contiguous(), "device tensors must be contiguous CUDA tensors"
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
+
+
+# The current stream's handle without an object for the stream, 0.3 us instead of 4 to 5 (half of what a call's marshalling took)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
+
+
+_prototypes = {}  # (name, kinds of the arguments) -> function with these argument types, so that pointers are passed as plain integers
+_KINDS = {float: ctypes.c_float, int: ctypes.c_int32}
+
+
+def _function(name, kinds):
+    fn = getattr(lib(), name)
+    types = [ctypes.POINTER(moe_config)] + [_KINDS.get(k, ctypes.c_void_p) for k in kinds]
+    return ctypes.CFUNCTYPE(ctypes.c_int32, *types)(ctypes.cast(fn, ctypes.c_void_p).value)
 
 
 def _call(name, cfg, *tensors, stream=True):
     # device tensors become pointers; a Python float is a `float` argument passed by value
-    args = [ctypes.byref(cfg)] + [ctypes.c_float(t) if isinstance(t, float) else
-                                  ctypes.c_int32(t) if isinstance(t, int) else _p(t) for t in tensors]
+    kinds, args = [], [cfg]
+    for t in tensors:
+        kind = None if isinstance(t, torch.Tensor) else float if isinstance(t, float) else int if isinstance(t, int) else None
+        kinds.append(kind)
+        args.append(t if kind else _p(t))
     if stream:
+        kinds.append(None)
         args.append(_stream())
-    status = getattr(lib(), name)(*args)
+    key = (name, *kinds)
+    fn = _prototypes.get(key)
+    if fn is None:
+        fn = _prototypes[key] = _function(name, kinds)
+    status = fn(*args)
     if status != 0:
         raise MoeError(name, status)
 
@@ -147,7 +171,7 @@ def moe_check_buffer_sizes(cfg, which, nbytes) -> int:
 
 
 def moe_debug_wait_timeout(ws, limit_ns):
-    status = lib().moe_debug_wait_timeout(_p(ws), ctypes.c_int64(limit_ns), _stream())
+    status = lib().moe_debug_wait_timeout(ctypes.c_void_p(_p(ws)), ctypes.c_int64(limit_ns), ctypes.c_void_p(_stream()))
     if status:
         raise MoeError("moe_debug_wait_timeout", status)
 
@@ -157,7 +181,7 @@ def moe_debug_bounds_violations() -> int:
 
 
 def moe_check_status(ws) -> int:
-    return lib().moe_check_status(_p(ws), _stream())
+    return lib().moe_check_status(ctypes.c_void_p(_p(ws)), ctypes.c_void_p(_stream()))
 
 
 def moe_gate(cfg, x, Wg, Wnoise, noise, topk_idx, gates, clean, raw_noise, kth_vals, kth_idx, ws):
