@@ -23,10 +23,11 @@ template <int BM, int BN, int TM, int TN, int BK, int S> struct RowsTile {
     static constexpr int ROW_BYTES = BK * 4 + 16;  // the rows that a warp reads together stand in different banks
     static constexpr int A_STAGE = BM * ROW_BYTES, STAGE = A_STAGE + BN * ROW_BYTES, SHARED = S * STAGE;
 };
-template <int BM, int BN, int TM, int TN, int BK, int S, int BLOCKS>
+// QUADS: rows of logits come in sixteen bytes at a time; otherwise (widths that are no multiple of four) four
+template <int BM, int BN, int TM, int TN, int BK, int S, int BLOCKS, bool QUADS>
 __global__ void __launch_bounds__(RowsTile<BM, BN, TM, TN, BK, S>::NT, BLOCKS) gate_rows_kernel(const __grid_constant__ GateProduct p, const int32_t *__restrict__ tile_prefix) {
     using Tile = RowsTile<BM, BN, TM, TN, BK, S>;
-    constexpr int NT = Tile::NT, ROW = BK / 4, QA = BM * ROW / NT, QB = BN * ROW / NT;
+    constexpr int NT = Tile::NT, V = QUADS ? 4 : 1, ROW = BK / V, QA = BM * ROW / NT, QB = BN * ROW / NT;
     static_assert(QA * NT == BM * ROW && QB * NT == BN * ROW && TN % 2 == 0, "whole copies a thread, pairs of columns");
     wait_previous_kernel();
     extern __shared__ __align__(16) uint8_t stages[];
@@ -44,33 +45,36 @@ __global__ void __launch_bounds__(RowsTile<BM, BN, TM, TN, BK, S>::NT, BLOCKS) g
     if (m0 >= m_end) return;
     const int32_t n_at = blockIdx.y * BN, cols = p.W2 ? 2 * p.n : p.n;
     const int64_t matrix = (int64_t)group * p.d * p.n;
-    const float *from_a[QA];
-    int64_t from_b[QB];
+    int32_t from_a[QA], from_b[QB];  // rows of dlogit and W that this thread copies from
 #pragma unroll
     for (int q = 0; q < QA; ++q) {
         int64_t r = m0 + (tid + q * NT) / ROW;
         if (r >= m_end) r = m0;  // (a row that is computed and dropped)
-        if (p.perm) r = p.perm[r];
-        from_a[q] = p.dlogit + r * cols;
+        from_a[q] = p.perm ? p.perm[r] : (int32_t)r;
     }
 #pragma unroll
     for (int q = 0; q < QB; ++q) {
         const int32_t j = n_at + (tid + q * NT) / ROW;
-        from_b[q] = matrix + (int64_t)(j < p.d ? j : 0) * p.n;  // (a column that is computed and dropped)
+        from_b[q] = j < p.d ? j : 0;  // (a column that is computed and dropped)
     }
     const int blocks = (cols + BK - 1) / BK;
     auto load = [&](int kb) {  // logits behind the last one are zero in both operands
         uint8_t *to = stages + kb % S * Tile::STAGE;
 #pragma unroll
         for (int q = 0; q < QA; ++q) {
-            const int id = tid + q * NT, k = kb * BK + id % ROW * 4;
-            copy16(to + id / ROW * Tile::ROW_BYTES + id % ROW * 16, k < cols ? from_a[q] + k : p.dlogit, k < cols);
+            const int id = tid + q * NT, k = kb * BK + id % ROW * V;
+            uint8_t *at = to + id / ROW * Tile::ROW_BYTES + id % ROW * (4 * V);
+            const float *from = k < cols ? p.dlogit + (int64_t)from_a[q] * cols + k : p.dlogit;
+            if (QUADS) copy16(at, from, k < cols);
+            else copy4(at, from, k < cols);
         }
 #pragma unroll
         for (int q = 0; q < QB; ++q) {
-            const int id = tid + q * NT, k = kb * BK + id % ROW * 4;
-            copy16(to + Tile::A_STAGE + id / ROW * Tile::ROW_BYTES + id % ROW * 16,
-                   k >= cols ? p.W : k < p.n ? p.W + from_b[q] + k : p.W2 + from_b[q] + (k - p.n), k < cols);
+            const int id = tid + q * NT, k = kb * BK + id % ROW * V;
+            uint8_t *at = to + Tile::A_STAGE + id / ROW * Tile::ROW_BYTES + id % ROW * (4 * V);
+            const float *from = k >= cols ? p.W : (k < p.n ? p.W + k : p.W2 + (k - p.n)) + matrix + (int64_t)from_b[q] * p.n;
+            if (QUADS) copy16(at, from, k < cols);
+            else copy4(at, from, k < cols);
         }
     };
 #pragma unroll
@@ -91,7 +95,7 @@ __global__ void __launch_bounds__(RowsTile<BM, BN, TM, TN, BK, S>::NT, BLOCKS) g
         if (kb + S - 1 < blocks) load(kb + S - 1);
         copies_commit();
         const uint8_t *a = stages + kb % S * Tile::STAGE + row0 * Tile::ROW_BYTES, *b = stages + kb % S * Tile::STAGE + Tile::A_STAGE + col0 * Tile::ROW_BYTES;
-        const int steps = min(BK, cols - kb * BK);  // a multiple of four
+        const int steps = min(BK, (cols - kb * BK + 3) & ~3);
         for (int kk = 0; kk < steps; kk += 4) {
             float4 av[TM], bv[TN];
 #pragma unroll
@@ -125,10 +129,10 @@ template <typename T, int BM, int BN, int TM, int TN, int BK, int S> struct Wgra
     static constexpr int WARPS_M = BM / (4 * TM), WARPS_N = BN / (8 * TN), NT = 32 * WARPS_M * WARPS_N;
     static constexpr int A_STAGE = BK * BM * (int)sizeof(T), STAGE = A_STAGE + BK * BN * 4, SHARED = S * STAGE;
 };
-template <typename T, int BM, int BN, int TM, int TN, int BK, int S, int BLOCKS>
+template <typename T, int BM, int BN, int TM, int TN, int BK, int S, int BLOCKS, bool QUADS>
 __global__ void __launch_bounds__(WgradTile<T, BM, BN, TM, TN, BK, S>::NT, BLOCKS) gate_wgrad_kernel(const __grid_constant__ GateProduct p, int32_t splits, float *__restrict__ part) {
     using Tile = WgradTile<T, BM, BN, TM, TN, BK, S>;
-    constexpr int NT = Tile::NT, VK = 16 / sizeof(T), A_ROW = BM / VK, B_ROW = BN / 4, QA = BK * A_ROW / NT, QB = BK * B_ROW / NT;
+    constexpr int NT = Tile::NT, VK = 16 / sizeof(T), A_ROW = BM / VK, VB = QUADS ? 4 : 1, B_ROW = BN / VB, QA = BK * A_ROW / NT, QB = BK * B_ROW / NT;
     static_assert(QA * NT == BK * A_ROW && QB * NT == BK * B_ROW, "whole copies a thread");
     wait_previous_kernel();
     extern __shared__ __align__(16) uint8_t stages[];
@@ -163,9 +167,11 @@ __global__ void __launch_bounds__(WgradTile<T, BM, BN, TM, TN, BK, S>::NT, BLOCK
         }
 #pragma unroll
         for (int q = 0; q < QB; ++q) {
-            const int id = tid + q * NT, c = n_at + id % B_ROW * 4;
+            const int id = tid + q * NT, c = n_at + id % B_ROW * VB;
             const bool live = rb[q] >= 0 && c < cols;
-            copy16(to + Tile::A_STAGE + id * 16, live ? p.dlogit + (int64_t)rb[q] * cols + c : p.dlogit, live);
+            const float *from = live ? p.dlogit + (int64_t)rb[q] * cols + c : p.dlogit;
+            if (QUADS) copy16(to + Tile::A_STAGE + id * 16, from, live);
+            else copy4(to + Tile::A_STAGE + id * 4, from, live);
         }
         fetch(kb + 1);
     };
@@ -212,14 +218,19 @@ __global__ void __launch_bounds__(WgradTile<T, BM, BN, TM, TN, BK, S>::NT, BLOCK
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
         const int32_t m = m_at + m0 + i % 4 + 16 * (i / 4), c = n_at + c0;
-        if (m >= p.d || c >= cols) continue;  // (cols is a multiple of four, TN of two)
-        float *to;
-        if (splits > 1) to = part + (((int64_t)slice * p.groups + group) * p.d + m) * cols + c;
-        else to = (c < p.n ? p.dW + c : p.dW2 + (c - p.n)) + ((int64_t)group * p.d + m) * p.n;
+        if (m >= p.d) continue;
 #pragma unroll
-        for (int j = 0; j < TN; ++j) to[j] = acc[i][j];
+        for (int j = 0; j < TN; ++j) {
+            if (c + j >= cols) break;
+            if (splits > 1) part[(((int64_t)slice * p.groups + group) * p.d + m) * cols + c + j] = acc[i][j];
+            else ((c + j < p.n ? p.dW + c : p.dW2 + (c - p.n)) + ((int64_t)group * p.d + m) * p.n)[j] = acc[i][j];
+        }
     }
 }
+
+// whether rows come in sixteen bytes at a time: of logits, and of the weights as well
+bool quads_of_logits(const GateProduct &p) { return (p.W2 ? 2 * (int64_t)p.n : p.n) % 4 == 0 && aligned16(p.dlogit); }
+bool quads_of_rows(const GateProduct &p) { return p.n % 4 == 0 && aligned16(p.W) && (!p.W2 || aligned16(p.W2)) && quads_of_logits(p); }
 
 template <int BM, int BN, int TM, int TN, int BK, int S, int BLOCKS> int32_t launch_rows(const GateProduct &p, int32_t *tile_prefix, cudaStream_t st) {
     using Tile = RowsTile<BM, BN, TM, TN, BK, S>;
@@ -228,40 +239,46 @@ template <int BM, int BN, int TM, int TN, int BK, int S, int BLOCKS> int32_t lau
         MOE_TRY(launch_tile_prefix(p.offsets, p.groups, BM, tile_prefix, st));
         tiles += p.groups;
     }
-    static PerDevice configured;
-    const auto kernel = gate_rows_kernel<BM, BN, TM, TN, BK, S, BLOCKS>;
-    if (!allow_shared(configured, kernel, Tile::SHARED)) return MOE_ERR_CUDA;
     if (cdiv(p.d, BN) > 65535) return MOE_ERR_UNSUPPORTED;
-    launch_kernel(kernel, dim3((unsigned)tiles, (unsigned)cdiv(p.d, BN)), Tile::NT, Tile::SHARED, st, p, (const int32_t *)tile_prefix);
-    MOE_LAUNCHED();
-    return MOE_OK;
+    auto run = [&](auto quads) -> int32_t {
+        static PerDevice configured;
+        const auto kernel = gate_rows_kernel<BM, BN, TM, TN, BK, S, BLOCKS, decltype(quads)::value>;
+        if (!allow_shared(configured, kernel, Tile::SHARED)) return MOE_ERR_CUDA;
+        launch_kernel(kernel, dim3((unsigned)tiles, (unsigned)cdiv(p.d, BN)), Tile::NT, Tile::SHARED, st, p, (const int32_t *)tile_prefix);
+        MOE_LAUNCHED();
+        return MOE_OK;
+    };
+    return quads_of_rows(p) ? run(std::true_type()) : run(std::false_type());
 }
 template <typename T, int BM, int BN, int TM, int TN, int BK, int S, int BLOCKS> int32_t launch_wgrad(const GateProduct &p, int32_t splits, float *part, cudaStream_t st) {
     using Tile = WgradTile<T, BM, BN, TM, TN, BK, S>;
-    static PerDevice configured;
-    const auto kernel = gate_wgrad_kernel<T, BM, BN, TM, TN, BK, S, BLOCKS>;
-    if (!allow_shared(configured, kernel, Tile::SHARED)) return MOE_ERR_CUDA;
     const int64_t cols = p.W2 ? 2 * (int64_t)p.n : p.n;
     if (cdiv(cols, BN) > 65535 || (int64_t)p.groups * splits > 65535) return MOE_ERR_UNSUPPORTED;
-    launch_kernel(kernel, dim3((unsigned)cdiv(p.d, BM), (unsigned)cdiv(cols, BN), (unsigned)(p.groups * splits)), Tile::NT, Tile::SHARED, st, p, splits, part);
-    MOE_LAUNCHED();
-    return MOE_OK;
+    auto run = [&](auto quads) -> int32_t {
+        static PerDevice configured;
+        const auto kernel = gate_wgrad_kernel<T, BM, BN, TM, TN, BK, S, BLOCKS, decltype(quads)::value>;
+        if (!allow_shared(configured, kernel, Tile::SHARED)) return MOE_ERR_CUDA;
+        launch_kernel(kernel, dim3((unsigned)cdiv(p.d, BM), (unsigned)cdiv(cols, BN), (unsigned)(p.groups * splits)), Tile::NT, Tile::SHARED, st, p, splits, part);
+        MOE_LAUNCHED();
+        return MOE_OK;
+    };
+    return quads_of_logits(p) ? run(std::true_type()) : run(std::false_type());
 }
 }  // namespace
-
-static bool whole_quads(const GateProduct &p) {
-    return p.n % 4 == 0 && aligned16(p.W) && (!p.W2 || aligned16(p.W2)) && aligned16(p.dlogit) && aligned16(p.x);
-}
 
 // Where the products below are faster than the float product of gemm_simt.cu; us, that way and this way, tokens x features x logits:
 //   dX: 256 x 64 x 16 4.1 2.4; 81 x 128 x 128 5.4 4.1 (16 x 16 tiles); 2085 x 256 x 32 5.7 5.0; 3001 x 320 x 40 9.7 7.9; 5000 x 512 x 32 14.8 12.1;
 //       15000 x 512 x 16 34.8 19.1; but 15000 x 128 x 72 16.3 20.8, 12000 x 256 x 128 30 44: with a wider contraction the multiply-adds count, of which
 //       eight rows and columns a thread from transposed tiles need fewer moves
+//       single floats (n no multiple of four): 24 x 512 x 66 7.0 4.4; 3000 x 128 x 14 5.3 5.0; 5000 x 320 x 26 11.5 9.0; 60000 x 256 x 10 63 40;
+//       20000 x 1024 x 44 131 120; but 2000 x 1024 x 78 22 26, 8192 x 512 x 94 41 48, 1019 x 512 x 222 15 25: the same line
 //   dW: 256 x 64 x 16 4.4 4.1, 15000 x 512 x 16 22.9 15.8 (64 x 16 tiles); 1000 x 512 x 24 6.2 4.4, 2085 x 256 x 32 6.3 4.6 (32 x 32, two warps);
 //       3001 x 320 x 40 9.2 7.3, 5000 x 512 x 32 11.5 9.2, 15000 x 128 x 72 17.7 15.5 (64 x 32); but 12000 x 256 x 128 26.8 28.6, 20000 x 1024 x 40 70 75
+//       single floats (rows of logits that are no multiple of sixteen bytes): that way twice at all sizes, 3000 x 128 x 14 11.1 4.2, 8192 x 512 x 94
+//       64 29, 60000 x 256 x 10 69 35, 15000 x 256 x 650 280 161, 32768 x 512 x 510 1119 529
 bool gate_rows_supported(const GateProduct &p) {
     const int32_t cols = p.W2 ? 2 * p.n : p.n;
-    if (!whole_quads(p) || cdiv(p.d, 16) > 65535) return false;
+    if (cdiv(p.d, 16) > 65535) return false;
     return p.rows < 512 ? cols <= 256 : cols <= 40 && 4 * cdiv(p.d, 64) * 64 <= 5 * (int64_t)p.d;
 }
 int32_t launch_gate_rows(const GateProduct &p, int32_t *tile_prefix, cudaStream_t st) {
@@ -274,8 +291,8 @@ int32_t launch_gate_rows(const GateProduct &p, int32_t *tile_prefix, cudaStream_
 static bool few_blocks(const GateProduct &p, int32_t cols, int32_t splits) { return cdiv(p.d, 32) * cdiv(cols, 32) * p.groups * splits <= 2 * 148; }
 bool gate_wgrad_supported(const GateProduct &p) {
     const int32_t cols = p.W2 ? 2 * p.n : p.n, splits = simt_wgrad_splits(p.d, cols, p.groups, p.rows);
-    if (!whole_quads(p) || cdiv(cols, 16) > 65535 || (int64_t)p.groups * splits > 65535) return false;
-    return cols <= 16 || few_blocks(p, cols, splits) || (cols <= 72 && p.d <= 512);
+    if (cdiv(cols, 16) > 65535 || (int64_t)p.groups * splits > 65535) return false;
+    return !quads_of_logits(p) || cols <= 16 || few_blocks(p, cols, splits) || (cols <= 72 && p.d <= 512);
 }
 // part: simt_wgrad_splits(d, logits, groups, rows) * groups * d * logits floats
 int32_t launch_gate_wgrad(const GateProduct &p, float *part, cudaStream_t st, GateParts *parts_left) {

@@ -26,7 +26,7 @@ struct ProjectionArgs {
     const int32_t *offsets, *tile_prefix;  // rows sorted by group, or nullptr: one group
     int32_t groups;
     const int32_t *row_index;    // row r: x row row_index[r] / row_div, output row row_index[r]; or nullptr
-    int32_t row_div, vec_out;
+    int32_t row_div, vec_out, quads;
     const int32_t *row_count;    // number of rows, read on the device (at most `rows`), or nullptr
     int32_t *clear;              // status word, cleared if given
 };
@@ -44,11 +44,13 @@ template <typename T, int BM, int BN, int TM, int TN, int BK, int S> struct Proj
     static constexpr int ROW_BYTES = BK * (int)sizeof(T) + 16;  // 16 more: the four rows that a warp reads together stand in different banks
     static constexpr int A_STAGE = BM * ROW_BYTES, B_STAGE = BK * BN * 4, STAGE = A_STAGE + B_STAGE, SHARED = S * STAGE;
 };
-template <typename T, int BM, int BN, int TM, int TN, int BK, int S, int BLOCKS>
+// QUADS: rows of the weights come in sixteen bytes at a time; otherwise (widths that are no multiple of four) four
+template <typename T, int BM, int BN, int TM, int TN, int BK, int S, int BLOCKS, bool QUADS>
 __global__ void __launch_bounds__(ProjectionTile<T, BM, BN, TM, TN, BK, S>::NT, BLOCKS) projection_kernel(const __grid_constant__ ProjectionArgs p) {
     using Tile = ProjectionTile<T, BM, BN, TM, TN, BK, S>;
-    constexpr int NT = Tile::NT, VK = 16 / sizeof(T), A_ROW = BK / VK, A_COPIES = BM * A_ROW, B_ROW = BN / 4, B_COPIES = BK * B_ROW;
-    constexpr int QA = A_COPIES / NT, QB = B_COPIES / NT, VN = TN < 4 ? TN : 4;
+    constexpr int NT = Tile::NT, VK = 16 / sizeof(T), A_ROW = BK / VK, A_COPIES = BM * A_ROW, VB = QUADS ? 4 : 1, B_ROW = BN / VB, B_COPIES = BK * B_ROW;
+    constexpr int QA = A_COPIES / NT, QB = B_COPIES / NT, COLS = QUADS ? QB : (BN > NT ? BN / NT : 1), VN = TN < 4 ? TN : 4;
+    static_assert(QUADS || NT % BN == 0 || BN % NT == 0, "a thread's single floats are of COLS columns");
     static_assert(QA * NT == A_COPIES && QB * NT == B_COPIES, "whole copies a thread");
     wait_previous_kernel();
     extern __shared__ __align__(16) uint8_t stages[];
@@ -70,7 +72,7 @@ __global__ void __launch_bounds__(ProjectionTile<T, BM, BN, TM, TN, BK, S>::NT, 
 
     // the copies of this thread: the same rows of x and columns of W in every K block
     const T *from_a[QA];
-    const float *from_b[QB];
+    const float *from_b[COLS];
 #pragma unroll
     for (int q = 0; q < QA; ++q) {
         const int id = tid + q * NT;
@@ -80,12 +82,15 @@ __global__ void __launch_bounds__(ProjectionTile<T, BM, BN, TM, TN, BK, S>::NT, 
         from_a[q] = static_cast<const T *>(p.x) + r * p.d + id % A_ROW * VK;
     }
 #pragma unroll
-    for (int q = 0; q < QB; ++q) {
+    for (int q = 0; q < COLS; ++q) {
         const int id = tid + q * NT;
-        int32_t col = n_at + id % B_ROW * 4;
-        if (col >= p.N) col = 0;  // (columns that are computed and dropped)
+        int32_t col = n_at + id % B_ROW * VB;
+        // columns behind the last one are computed and dropped; not all from one column: copies from one address go one by one (6000 x 512 x 174 in
+        // 64 x 128 tiles 92 us, 58; 20000 x 1024 x 40 100, 79)
+        if (col >= p.N) col = min(col - p.N, p.N - VB);
         from_b[q] = (col < p.n0 ? W0 + col : W1 + (col - p.n0)) + (int64_t)(id / B_ROW) * p.n0;
     }
+    const int64_t step = (int64_t)(NT > BN ? NT / BN : 1) * p.n0;  // single floats: a thread's copies of a column stand this far apart
     const int blocks = (p.d + BK - 1) / BK;
     auto load = [&](int kb) {  // features behind the last one are zero in both operands
         uint8_t *to = stages + kb % S * Tile::STAGE;
@@ -95,10 +100,27 @@ __global__ void __launch_bounds__(ProjectionTile<T, BM, BN, TM, TN, BK, S>::NT, 
             const int id = tid + q * NT, k = k0 + id % A_ROW * VK;
             copy16(to + id / A_ROW * Tile::ROW_BYTES + id % A_ROW * 16, k < p.d ? from_a[q] + k0 : static_cast<const T *>(p.x), k < p.d);
         }
+        if constexpr (QUADS) {
 #pragma unroll
-        for (int q = 0; q < QB; ++q) {
-            const int id = tid + q * NT, k = k0 + id / B_ROW;
-            copy16(to + Tile::A_STAGE + id * 16, k < p.d ? from_b[q] + (int64_t)k0 * p.n0 : W0, k < p.d);
+            for (int q = 0; q < QB; ++q) {
+                const int id = tid + q * NT, k = k0 + id / B_ROW;
+                copy16(to + Tile::A_STAGE + id * 16, k < p.d ? from_b[q] + (int64_t)k0 * p.n0 : W0, k < p.d);
+            }
+        } else {
+            auto column = [&](auto whole) {
+#pragma unroll
+                for (int c = 0; c < COLS; ++c) {
+                    const float *from = from_b[c] + (int64_t)k0 * p.n0;
+#pragma unroll
+                    for (int q = c; q < QB; q += COLS, from += step) {
+                        const int id = tid + q * NT;
+                        if constexpr (decltype(whole)::value) copy4(to + Tile::A_STAGE + id * 4, from, true);
+                        else copy4(to + Tile::A_STAGE + id * 4, k0 + id / B_ROW < p.d ? from : W0, k0 + id / B_ROW < p.d);
+                    }
+                }
+            };
+            if (k0 + BK <= p.d) column(std::true_type());
+            else column(std::false_type());
         }
     };
 #pragma unroll
@@ -150,20 +172,26 @@ __global__ void __launch_bounds__(ProjectionTile<T, BM, BN, TM, TN, BK, S>::NT, 
 #pragma unroll
         for (int j = 0; j < TN; j += VN) {
             const int32_t col = n_at + col0 + 8 * j;
-            if (col >= p.N) continue;  // N and n0 are multiples of four
-            float *to = (col < p.n0 ? p.out0 + col : p.out1 + (col - p.n0)) + r * p.n0;
-            if (VN == 4 && p.vec_out) {
-                *reinterpret_cast<float4 *>(to) = make_float4(acc[i][j], acc[i][j + 1], acc[i][j + VN - 2], acc[i][j + VN - 1]);
+            if constexpr (QUADS) {
+                if (col >= p.N) continue;  // N and n0 are multiples of four
+                float *to = (col < p.n0 ? p.out0 + col : p.out1 + (col - p.n0)) + r * p.n0;
+                if (VN == 4 && p.vec_out) {
+                    *reinterpret_cast<float4 *>(to) = make_float4(acc[i][j], acc[i][j + 1], acc[i][j + VN - 2], acc[i][j + VN - 1]);
+                } else {
+#pragma unroll
+                    for (int z = 0; z < VN; ++z) to[z] = acc[i][j + z];
+                }
             } else {
 #pragma unroll
-                for (int z = 0; z < VN; ++z) to[z] = acc[i][j + z];
+                for (int z = 0; z < VN; ++z)
+                    if (col + z < p.N) (col + z < p.n0 ? p.out0 + (col + z) : p.out1 + (col + z - p.n0))[r * p.n0] = acc[i][j + z];
             }
         }
     }
 }
 
-template <typename T, int BM, int BN, int TM, int TN, int BK, int S, int BLOCKS>
-int32_t launch_tile(ProjectionArgs p, int32_t *tile_prefix, cudaStream_t st) {
+template <typename T, int BM, int BN, int TM, int TN, int BK, int S, int BLOCKS, bool QUADS>
+int32_t launch_tile_as(ProjectionArgs p, int32_t *tile_prefix, cudaStream_t st) {
     using Tile = ProjectionTile<T, BM, BN, TM, TN, BK, S>;
     int64_t tiles = cdiv(p.rows, BM);
     if (p.offsets) {
@@ -174,37 +202,44 @@ int32_t launch_tile(ProjectionArgs p, int32_t *tile_prefix, cudaStream_t st) {
     }
     if (cdiv(p.N, BN) > 65535) return MOE_ERR_UNSUPPORTED;
     static PerDevice configured;
-    const auto kernel = projection_kernel<T, BM, BN, TM, TN, BK, S, BLOCKS>;
+    const auto kernel = projection_kernel<T, BM, BN, TM, TN, BK, S, BLOCKS, QUADS>;
     if (!allow_shared(configured, kernel, Tile::SHARED)) return MOE_ERR_CUDA;
     launch_kernel(kernel, dim3((unsigned)tiles, (unsigned)cdiv(p.N, BN)), Tile::NT, Tile::SHARED, st, p);
     MOE_LAUNCHED();
     return MOE_OK;
 }
 
-// The tile that takes the least time by an estimate: a block's chain cannot be faster than `chain` ns a feature, and an SM's share of the blocks takes
-// `share` ns a feature each and `more` us. Read off kernels of all sizes; us, by the 64 x 128 tile and the others in order:
-//   32768 x 512 x 256 179 198 222 591;  6000 x 512 x 192 60 35 39 89;  1019 x 512 x 512 32 21 21 43;  2000 x 1024 x 128 59 37 24 44;
-//   24 x 512 x 64 33 20 12 5.9;  15000 x 512 x 16 (bf16) - 60 43 34 16 19;  3001 x 320 x 40 25 15 11 12 10 7.8;  60000 x 256 x 8 (float) - 234 205 100 33 45.
-// Against one chain per output of float tiles in shared memory (gemm_simt.cu, which widths that are no multiple of four still take):
-// 24 x 512 x 64 10.5 5.9, 1019 x 512 x 512 25 21, 3001 x 320 x 40 13 7.8, 8192 x 512 x 64 25 21, 15000 x 128 x 72 21 16, 32768 x 512 x 256 185 179.
+template <typename T, int BM, int BN, int TM, int TN, int BK, int S, int BLOCKS>
+int32_t launch_tile(const ProjectionArgs &p, int32_t *tile_prefix, cudaStream_t st) {
+    return p.quads ? launch_tile_as<T, BM, BN, TM, TN, BK, S, BLOCKS, true>(p, tile_prefix, st)
+                   : launch_tile_as<T, BM, BN, TM, TN, BK, S, BLOCKS, false>(p, tile_prefix, st);
+}
+
+// The tile that takes the least time by an estimate: an SM's first block takes `chain` ns a feature, each further one `share`, and each `more` us besides.
+// Read off kernels of all sizes; us, by the 64 x 128 tile and the others in order:
+//   32768 x 512 x 510 363 406 460 - 507 550;  6000 x 512 x 168 54 35 38 81 42 39;  1019 x 512 x 222 33 22 14 25 15 14;  24 x 512 x 64 30 21 12 6.4 15 10;
+//   20000 x 1024 x 44 157 95 89 159 80 75;  15000 x 256 x 648 125 132 138 - 159 164;  60000 x 256 x 10 (float) 90 53 38 50 26 25.
+// Against one chain per output of float tiles in shared memory (gemm_simt.cu): 24 x 512 x 64 10.5 6.1, 1019 x 512 x 512 25 21, 3001 x 320 x 40 13 7.8,
+// 8192 x 512 x 64 25 21, 15000 x 128 x 72 21 16, 32768 x 512 x 256 185 179. Widths that are no multiple of four cost next to nothing more (single floats
+// of the weights are a tenth of a thread's instructions), and that way twice: 24 x 512 x 66 18.4 7.0, 300 x 256 x 50 11.2 4.3, 60000 x 256 x 10 61 26.
 constexpr int32_t PROJECTION_ELSEWHERE = -1;  // (no status)
-struct ProjectionCost { int32_t bm, bn; double chain, share[2], more[2]; };  // [bf16, float]
+struct ProjectionCost { int32_t bm, bn; double chain, share[2], more; };  // [bf16, float]
 template <typename T> int32_t pick_tile(const ProjectionArgs &p, int32_t *tile_prefix, cudaStream_t st) {
     constexpr int F = sizeof(T) == 4 ? 1 : 0;
-    static const ProjectionCost costs[6] = {{64, 128, 53, {44, 45}, {2.5, 2.5}}, {64, 64, 33, {24, 24}, {2.3, 4.0}},
-                                            {32, 32, 19.5, {7.5, 10}, {0.75, 0.75}}, {16, 16, 10, {5.2, 6.5}, {0.5, 0.5}},
-                                            {128, 16, 27, {20, 28}, {0.9, 0.9}}, {64, 16, 18, {14, 20}, {0.4, 0.4}}};
+    static const ProjectionCost costs[6] = {{64, 128, 53, {44, 45}, 2.5}, {64, 64, 33, {24, 24}, 2.3}, {32, 32, 19.5, {6.5, 8}, 0.75},
+                                            {16, 16, 10, {5.2, 6.5}, 0.5}, {128, 16, 27, {16, 22}, 0.9}, {64, 16, 18, {9, 14}, 0.6}};
     int best = 0;
     double least = 0.0;
     for (int i = 0; i < 6; ++i) {
         const ProjectionCost &c = costs[i];
         const int64_t blocks = (cdiv(p.rows, c.bm) + (p.offsets ? p.groups / 2 : 0)) * cdiv(p.N, c.bn);
-        const double chain = 1e-3 * c.chain * p.d, share = (double)cdiv(blocks, 148) * (1e-3 * c.share[F] * p.d + c.more[F]);
-        const double cost = chain > share ? chain : share;
+        const double cost = 1e-3 * c.chain * p.d + c.more + (double)(cdiv(blocks, 148) - 1) * (1e-3 * c.share[F] * p.d + c.more);
         if (i == 0 || cost < least) { best = i; least = cost; }
     }
     // float rows have as many shared-memory reads in the largest tiles as the float product has (32768 x 512 x 512: 362, that way 349)
     if (F && best == 0 && p.d >= 256 && !p.offsets && cdiv(p.rows, 64) * cdiv(p.N, 128) >= 6 * 148) return PROJECTION_ELSEWHERE;
+    // and short chains of single floats fill the pipeline of the copies too often (15000 x 256 x 650: 136, that way 130; 32768 x 512 x 510: 363, 367)
+    if (!p.quads && best == 0 && p.d < 512 && !p.offsets && cdiv(p.rows, 64) * cdiv(p.N, 128) >= 6 * 148) return PROJECTION_ELSEWHERE;
     switch (best) {
         case 0: return launch_tile<T, 64, 128, 8, 8, 32, 3, 3>(p, tile_prefix, st);
         case 1: return launch_tile<T, 64, 64, 8, 4, 32, 4, 3>(p, tile_prefix, st);
@@ -222,11 +257,12 @@ int32_t launch_projection(const void *x, int32_t act, int64_t M, int32_t d, int3
                           const int32_t *perm, int32_t kdiv, int32_t *tile_prefix, cudaStream_t st,
                           const int32_t *row_count, int32_t *clear) {
     if (M == 0) return MOE_OK;
-    if (n0 % 4 == 0 && aligned16(W0) && (!W1 || aligned16(W1))) {
+    {
         ProjectionArgs p;
         memset(&p, 0, sizeof(p));
         p.x = x; p.W0 = W0; p.W1 = W1 ? W1 : W0; p.out0 = out0; p.out1 = out1; p.rows = M; p.group_stride = (int64_t)d * n0;
         p.d = d; p.n0 = n0; p.N = W1 ? 2 * n0 : n0; p.offsets = offsets; p.groups = nseg; p.row_index = perm; p.row_div = kdiv > 0 ? kdiv : 1;
+        p.quads = n0 % 4 == 0 && aligned16(W0) && (!W1 || aligned16(W1));
         p.vec_out = aligned16(out0) && (!W1 || aligned16(out1));
         p.row_count = row_count; p.clear = clear;
         const int32_t rc = act == MOE_BF16 ? pick_tile<bf16>(p, tile_prefix, st) : pick_tile<float>(p, tile_prefix, st);

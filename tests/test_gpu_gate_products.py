@@ -19,11 +19,23 @@ FLAT = [
     small_workload("gp-slices", T=3001, d=320, h=64, n=20, k=3, act="bf16", seed=107),
     small_workload("gp-72-logits", T=2200, d=136, h=64, n=36, k=2, act="bf16", seed=108),
     small_workload("gp-few-rows-wide", T=40, d=260, h=64, n=100, k=2, seed=109),
+    # rows of logits and weights that are no whole quads: both, the weights only
+    small_workload("gp-one-expert", T=1, d=64, h=64, n=1, k=1, seed=121),
+    small_workload("gp-511-single", T=511, d=72, h=64, n=21, k=2, act="bf16", seed=122),
+    small_workload("gp-512-even", T=512, d=68, h=64, n=18, k=2, seed=123),
+    small_workload("gp-513-wide-single", T=513, d=128, h=64, n=23, k=3, act="bf16", seed=124),
+    small_workload("gp-narrow-single", T=2100, d=328, h=64, n=7, k=2, act="bf16", seed=125),
+    small_workload("gp-slices-single", T=3001, d=320, h=64, n=19, k=3, act="bf16", seed=126),
+    small_workload("gp-even", T=2200, d=136, h=64, n=34, k=2, act="bf16", seed=127),
+    small_workload("gp-many-single", T=2500, d=200, h=64, n=111, k=2, act="bf16", seed=128),
+    small_workload("gp-few-rows-single", T=40, d=260, h=64, n=101, k=2, seed=129),
 ]
 HIER = [
     small_workload("gp-hier", T=1500, d=128, h=64, n=64, k=4, act="bf16", a=16, k1=2, b=4, k2=2, seed=111),
     small_workload("gp-hier-odd-groups", T=700, d=64, h=64, n=60, k=4, act="bf16", a=5, k1=2, b=12, k2=2, seed=112),
     small_workload("gp-hier-few", T=100, d=64, h=64, n=160, k=2, a=8, k1=1, b=20, k2=2, seed=113),
+    small_workload("gp-hier-single", T=1500, d=128, h=64, n=63, k=4, act="bf16", a=9, k1=2, b=7, k2=2, seed=114),
+    small_workload("gp-hier-even", T=900, d=64, h=64, n=60, k=4, a=10, k1=2, b=6, k2=2, seed=115),
 ]
 
 
