@@ -535,13 +535,13 @@ int32_t do_expert_ffn(const moe_config *c, const Dims &D, const void *xs, const 
     g.A = xs; g.B = W1; g.C = hid; g.bias = b1; g.relu = 1;
     g.sa_i = D.d; g.sa_k = 1; g.sb_k = D.h; g.sb_j = 1; g.sc_i = D.h;
     g.mode = 0; g.offsets = offsets; g.nseg = (int32_t)D.n; g.M = D.R; g.N = D.h; g.K = D.d; g.b_e = D.d * D.h;
-    MOE_TRY(launch_simt_gemm(g, nullptr, st, nullptr, &plan));
+    MOE_TRY(launch_float_expert_product(g, plan, D.R, st));
     if (first_only) return MOE_OK;
     g = base_gemm();  // ys = hid.W2 + b2
     g.A = hid; g.B = W2; g.C = ys; g.bias = b2;
     g.sa_i = D.h; g.sa_k = 1; g.sb_k = D.d; g.sb_j = 1; g.sc_i = D.d;
     g.mode = 0; g.offsets = offsets; g.nseg = (int32_t)D.n; g.M = D.R; g.N = D.d; g.K = D.h; g.b_e = D.h * D.d;
-    return launch_simt_gemm(g, nullptr, st, nullptr, &plan);
+    return launch_float_expert_product(g, plan, D.R, st);
 }
 
 // The batch sums over the columns of the flat gate, with the two losses, or of the primary gate (idx: its groups): Load_primary
@@ -625,24 +625,24 @@ int32_t do_expert_ffn_bwd(const moe_config *c, const Dims &D, const void *xs, co
     g.A = hid; g.B = dys; g.C = dW2;
     g.sa_i = 1; g.sa_k = D.h; g.sb_k = D.d; g.sb_j = 1; g.sc_i = D.d;
     g.mode = 1; g.offsets = offsets; g.nseg = n; g.M = D.h; g.N = D.d; g.c_e = D.h * D.d;
-    MOE_TRY(launch_simt_gemm(g, nullptr, st, nullptr, &plan));
+    MOE_TRY(launch_float_expert_product(g, plan, D.R, st));
     g = base_gemm();  // dz = (dys . W2[e]^T) * [hid > 0]
     g.A = dys; g.B = W2; g.C = w.dz; g.mask = hid;
     g.sa_i = D.d; g.sa_k = 1; g.sb_k = 1; g.sb_j = D.d; g.sc_i = D.h;
     g.mode = 0; g.offsets = offsets; g.nseg = n; g.M = D.R; g.N = D.h; g.K = D.d; g.b_e = D.h * D.d;
-    MOE_TRY(launch_simt_gemm(g, nullptr, st, nullptr, &plan));
+    MOE_TRY(launch_float_expert_product(g, plan, D.R, st));
     MOE_TRY(launch_segment_colsum(db1s, st));
     MOE_TRY(finish(db1s, 1));
     g = base_gemm();  // dW1[e] = xs_e^T . dz_e
     g.A = xs; g.B = w.dz; g.C = dW1;
     g.sa_i = 1; g.sa_k = D.d; g.sb_k = D.h; g.sb_j = 1; g.sc_i = D.h;
     g.mode = 1; g.offsets = offsets; g.nseg = n; g.M = D.d; g.N = D.h; g.c_e = D.d * D.h;
-    MOE_TRY(launch_simt_gemm(g, nullptr, st, nullptr, &plan));
+    MOE_TRY(launch_float_expert_product(g, plan, D.R, st));
     g = base_gemm();  // dxs = dz . W1[e]^T
     g.A = w.dz; g.B = W1; g.C = dxs;
     g.sa_i = D.h; g.sa_k = 1; g.sb_k = 1; g.sb_j = D.h; g.sc_i = D.d;
     g.mode = 0; g.offsets = offsets; g.nseg = n; g.M = D.R; g.N = D.d; g.K = D.h; g.b_e = D.d * D.h;
-    return launch_simt_gemm(g, nullptr, st, nullptr, &plan);
+    return launch_float_expert_product(g, plan, D.R, st);
 }
 
 int32_t expert_ffn_bwd_stage(const moe_config *c, const Dims &D, const void *xs, const void *hid, const void *dys,

@@ -366,6 +366,8 @@ struct SimtGemm {
     const int32_t *b_row_index;
     const int32_t *c_row_index;
 };
+// A product of float experts (few_rows.cu) over R rows; plan: with tile prefixes of heights 16 / 32 / 64
+int32_t launch_float_expert_product(const SimtGemm &g, const struct SegmentPlan &plan, int64_t R, cudaStream_t st);
 // partial sums of a gate's weight gradient [nparts][d][cols], to be added into dW (columns before split) and dW2 (the others), rows ld apart
 struct GateParts {
     const float *part;
