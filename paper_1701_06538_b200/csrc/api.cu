@@ -207,6 +207,7 @@ SegmentPlan make_plan(const moe_config *c, const Dims &D, int32_t *ws, bool back
         }
     } else if (D.float_terms[backward]) {
         p.bm[0] = COLSUM_ROWS;
+        p.bm[1] = 64; p.bm[2] = 32; p.bm[3] = 16;  // of the product that makes hid
         p.sched = nullptr;
         p.by_rank = p.prefix[0];
         p.maps = nullptr;
@@ -222,11 +223,11 @@ SegmentPlan make_plan(const moe_config *c, const Dims &D, int32_t *ws, bool back
 FloatTerms float_terms(Carver &cv, const Dims &D, bool backward) {
     FloatTerms t = {};
     if (!D.float_terms[backward]) return t;
-    t.xs = cv.take<bf16>(3 * D.R * D.d);
     t.hid = cv.take<bf16>(3 * D.R * D.h);
-    t.W1 = cv.take<bf16>(3 * D.n * D.d * D.h);
     t.W2 = cv.take<bf16>(3 * D.n * D.d * D.h);
     if (!backward) return t;
+    t.xs = cv.take<bf16>(3 * D.R * D.d);
+    t.W1 = cv.take<bf16>(3 * D.n * D.d * D.h);
     t.dys = cv.take<bf16>(3 * D.R * D.d);
     t.dz = cv.take<bf16>(3 * D.R * D.h);
     return t;
@@ -530,13 +531,15 @@ int32_t do_expert_ffn(const moe_config *c, const Dims &D, const void *xs, const 
     }
     if (tc_ffn_takes(*c))
         return launch_tc_ffn(*c, xs, offsets, W1, b1, W2, b2, hid, ys, plan, status_word(ws_base), st, first_only, relu_bits);
-    if (D.float_terms[0] && !first_only) return launch_float_ffn(*c, xs, offsets, W1, b1, W2, b2, hid, ys, plan, w.terms, status_word(ws_base), st);
-    SimtGemm g = base_gemm();  // hid = relu(xs.W1 + b1)
+    // hid = relu(xs.W1 + b1): one chain of multiply-adds per output, whatever computes the other products, since its zeros decide the mask of the backward
+    // pass: a value next to 0 that rounds to the other side with another order of its sum is a whole term of dW1 and dX
+    SimtGemm g = base_gemm();
     g.A = xs; g.B = W1; g.C = hid; g.bias = b1; g.relu = 1;
     g.sa_i = D.d; g.sa_k = 1; g.sb_k = D.h; g.sb_j = 1; g.sc_i = D.h;
     g.mode = 0; g.offsets = offsets; g.nseg = (int32_t)D.n; g.M = D.R; g.N = D.h; g.K = D.d; g.b_e = D.d * D.h;
-    MOE_TRY(launch_float_expert_product(g, plan, D.R, st));
+    MOE_TRY(launch_simt_gemm(g, nullptr, st, nullptr, &plan));
     if (first_only) return MOE_OK;
+    if (D.float_terms[0]) return launch_float_ys(*c, offsets, hid, W2, b2, ys, plan, w.terms, status_word(ws_base), st);
     g = base_gemm();  // ys = hid.W2 + b2
     g.A = hid; g.B = W2; g.C = ys; g.bias = b2;
     g.sa_i = D.h; g.sa_k = 1; g.sb_k = D.d; g.sb_j = 1; g.sc_i = D.d;
@@ -590,9 +593,7 @@ ColumnSums db2_sums(const Dims &D, const void *dys, void *db2, const int32_t *of
 int32_t do_expert_ffn_bwd(const moe_config *c, const Dims &D, const void *xs, const void *hid, const void *dys,
                           const int32_t *offsets, const void *W1, const void *W2, void *dxs, void *dW1, void *db1,
                           void *dW2, void *db2, void *ws_base, const FfnBwdWs &w, cudaStream_t st, const SegmentPlan &plan,
-                          const uint32_t *relu_bits = nullptr, BackwardTail *tail = nullptr, bool db2_begun = false,
-                          const void *b1_again = nullptr) {
-    // b1_again (float experts on the tensor cores): hid is computed first
+                          const uint32_t *relu_bits = nullptr, BackwardTail *tail = nullptr, bool db2_begun = false) {
     const int32_t n = (int32_t)D.n;
     BackwardTail *leave = n < COLSUM_MANY ? tail : nullptr;
     auto finish = [&](const ColumnSums &sums, int which) -> int32_t {
@@ -616,8 +617,7 @@ int32_t do_expert_ffn_bwd(const moe_config *c, const Dims &D, const void *xs, co
     }
     const ColumnSums db1s = {w.dz, db1, D.act, n, (int32_t)D.h, D.R, offsets, plan.prefix_of(COLSUM_ROWS), w.colsum};
     if (D.float_terms[1]) {
-        MOE_TRY(launch_float_ffn_bwd(*c, xs, const_cast<void *>(hid), b1_again != nullptr, dys, offsets, W1, b1_again, W2, dxs, dW1, dW2, w.dz, plan,
-                                     w.terms, status_word(ws_base), st));
+        MOE_TRY(launch_float_ffn_bwd(*c, xs, hid, dys, offsets, W1, W2, dxs, dW1, dW2, w.dz, plan, w.terms, status_word(ws_base), st));
         MOE_TRY(launch_segment_colsum(db1s, st));
         return finish(db1s, 1);
     }
@@ -1142,11 +1142,11 @@ static int32_t backward_impl(const moe_config *cfg, const void *dY, const void *
     if (!hid) {  // MOE_FLAG_RECOMPUTE_HID: the forward kept no hidden activations; the first GEMM is run again
         bits = B.ffn.bits;
         Carver none(nullptr);  // (both buffers are given)
-        if (!D.float_terms[1]) MOE_TRY(do_expert_ffn(cfg, D, C.xs, C.offsets, W1, b1, W2, b2, B.again.hid, nullptr, ws, none, st, nullptr, true, bits, &plan));
+        MOE_TRY(do_expert_ffn(cfg, D, C.xs, C.offsets, W1, b1, W2, b2, B.again.hid, nullptr, ws, none, st, nullptr, true, bits, &plan));
         hid = B.again.hid;
     }
     MOE_TRY(do_expert_ffn_bwd(cfg, D, C.xs, hid, B.dys, C.offsets, W1, W2, B.dxs, dW1, db1, dW2, db2, ws, B.ffn, st, plan, bits, left,
-                              left != nullptr, C.hid ? nullptr : b1));
+                              left != nullptr));
     // dX = expert path + gating path (+ the upstream gradient itself through the residual connection)
     return launch_dispatch_bwd(B.dxs, D.act, C.inv_perm, D.T, (int32_t)D.k, (int32_t)D.d, B.dX_gate, nullptr, dX,
                                st, keep_bits ? dY : nullptr, sec, left);

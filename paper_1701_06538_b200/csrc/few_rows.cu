@@ -23,16 +23,12 @@ struct FewRows {
     const float *A, *W;
     float *C;
     const float *bias, *mask;
-    int32_t relu, N, K, nseg;
+    int32_t N, K, nseg;
     int64_t w_e;
     const int32_t *offsets, *prefix;
 };
 
-__device__ __forceinline__ float few_epilogue(const FewRows &p, float v, float bias, float mask) {
-    v += bias;
-    if (p.relu) v = fmaxf(v, 0.0f);
-    return mask > 0.0f ? v : 0.0f;
-}
+__device__ __forceinline__ float few_epilogue(float v, float bias, float mask) { return mask > 0.0f ? v + bias : 0.0f; }
 
 // A tile: the rows of a segment from row0 on, by the least of 4, 8 and 16 that holds them
 struct FewTile { int32_t e, row0, rows; };
@@ -123,7 +119,7 @@ template <int LC, int WARPS> __global__ void __launch_bounds__(32 * WARPS, WARPS
             const float4 b = p.bias ? *reinterpret_cast<const float4 *>(p.bias + (int64_t)t.e * p.N + c) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             const float4 m = p.mask ? *reinterpret_cast<const float4 *>(p.mask + at) : make_float4(1.0f, 1.0f, 1.0f, 1.0f);
             *reinterpret_cast<float4 *>(p.C + at) =
-                make_float4(few_epilogue(p, s.x, b.x, m.x), few_epilogue(p, s.y, b.y, m.y), few_epilogue(p, s.z, b.z, m.z), few_epilogue(p, s.w, b.w, m.w));
+                make_float4(few_epilogue(s.x, b.x, m.x), few_epilogue(s.y, b.y, m.y), few_epilogue(s.z, b.z, m.z), few_epilogue(s.w, b.w, m.w));
         }
     });
 }
@@ -176,7 +172,7 @@ template <int LK, int KS> __global__ void __launch_bounds__(FEW_THREADS, 4) few_
                 const int r = f / NB, n = first + f % NB;
                 if (r >= t.rows || n >= p.N) return;
                 const int64_t at = (int64_t)(t.row0 + r) * p.N + n;
-                p.C[at] = few_epilogue(p, v, p.bias ? p.bias[(int64_t)t.e * p.N + n] : 0.0f, p.mask ? p.mask[at] : 1.0f);
+                p.C[at] = few_epilogue(v, p.bias ? p.bias[(int64_t)t.e * p.N + n] : 0.0f, p.mask ? p.mask[at] : 1.0f);
             };
             if constexpr (KS == 1) {
 #pragma unroll
@@ -264,7 +260,7 @@ bool few_rows_take(const SimtGemm &g, const SegmentPlan &plan, int64_t R) {
     const bool grad = g.mode == 1;
     if (g.N % 4 != 0 || g.K % 4 != 0 || g.M % (grad ? 4 : 1) != 0 || !aligned16(g.A) || !aligned16(g.B) || !aligned16(g.C)) return false;
     if ((g.bias && !aligned16(g.bias)) || (g.mask && !aligned16(g.mask)) || g.nseg > 65535 || cdiv(g.N, 8) > 65535) return false;
-    if (!grad && !plan.prefix_of(FEW_ROWS)) return false;
+    if (g.relu || (!grad && !plan.prefix_of(FEW_ROWS))) return false;
     const int64_t n = g.nseg;
     if (grad) return R <= 16 * n || (R <= 128 * n && n * cdiv(g.M, 64) * cdiv(g.N, 128) >= 64);
     return R <= (g.sb_j == 1 ? 64 : 32) * n;
@@ -296,7 +292,7 @@ int32_t launch_float_expert_product(const SimtGemm &g, const SegmentPlan &plan, 
         FewGradients p = {(const float *)g.A, (const float *)g.B, (float *)g.C, (int32_t)g.M, (int32_t)g.N, g.nseg, 0, g.offsets};
         return g.N <= 64 ? launch_gradients<16>(p, st) : launch_gradients<32>(p, st);
     }
-    const FewRows p = {(const float *)g.A, (const float *)g.B, (float *)g.C, (const float *)g.bias, (const float *)g.mask, g.relu, (int32_t)g.N, (int32_t)g.K, g.nseg, g.b_e,
+    const FewRows p = {(const float *)g.A, (const float *)g.B, (float *)g.C, (const float *)g.bias, (const float *)g.mask, (int32_t)g.N, (int32_t)g.K, g.nseg, g.b_e,
                        g.offsets, plan.prefix_of(FEW_ROWS)};
     const int64_t tiles = imin(cdiv(R, FEW_ROWS) + g.nseg, R), live = imin(R, cdiv(R, FEW_ROWS) + g.nseg / 2);  // launched, and about how many have rows
     // Blocks enough for every SM first, then the widest rows; warps that share a long contraction where there are few blocks. us:

@@ -455,11 +455,11 @@ int32_t launch_tc_ffn(const moe_config &c, const void *xs, const int32_t *offset
 bool tc_float_supported(const moe_config &c, bool backward);
 // three bf16 terms of a call's operands, [rows][3 columns]: rows of xs, hid, dys, dz; matrices W1 [n d][3 h], W2 [n h][3 d]
 struct FloatTerms { void *xs, *hid, *dys, *dz, *W1, *W2; };
-int32_t launch_float_ffn(const moe_config &c, const void *xs, const int32_t *offsets, const void *W1, const void *b1, const void *W2, const void *b2,
-                         void *hid, void *ys, const SegmentPlan &plan, const FloatTerms &t, int32_t *status, cudaStream_t st);
-// again: hid is computed first. The column sums of dys and dz are the caller's
-int32_t launch_float_ffn_bwd(const moe_config &c, const void *xs, void *hid, bool again, const void *dys, const int32_t *offsets, const void *W1,
-                             const void *b1, const void *W2, void *dxs, void *dW1, void *dW2, void *dz, const SegmentPlan &plan, const FloatTerms &t,
+int32_t launch_float_ys(const moe_config &c, const int32_t *offsets, const void *hid, const void *W2, const void *b2, void *ys, const SegmentPlan &plan,
+                        const FloatTerms &t, int32_t *status, cudaStream_t st);
+// The column sums of dys and dz are the caller's
+int32_t launch_float_ffn_bwd(const moe_config &c, const void *xs, const void *hid, const void *dys, const int32_t *offsets, const void *W1,
+                             const void *W2, void *dxs, void *dW1, void *dW2, void *dz, const SegmentPlan &plan, const FloatTerms &t,
                              int32_t *status, cudaStream_t st);
 
 // ----------------------------------------------------------------------------- strictly balanced gating (balanced.cu)

@@ -1,7 +1,8 @@
 // The float experts' products on the tensor cores: every operand as three bf16 terms (hi + mid + lo hold a float's 24 bits), a product as the
 // six terms of at most 2^-16 of the leading one and more: hi.hi, and hi.mid, mid.hi, mid.mid, hi.lo, lo.hi. Float products by FP32
-// multiply-adds (gemm_simt.cu) run at 20 to 29 of the chip's 74 TFLOP/s; this way the six products of that step take 16 to 19 us each instead of
-// 38 to 52, most of it the way of the operands from L2 (a step with 8 experts x 500 rows of 1024 x 512: 797 us, this way 295).
+// multiply-adds (gemm_simt.cu) run at 20 to 29 of the chip's 74 TFLOP/s; this way five of the six products of a step with 16 experts x 260 rows
+// of 256 x 512 take 14 to 16 us each instead of 38 to 52, most of it the way of the operands from L2. (The first, whose signs are the ReLU mask, stays
+// with one chain of multiply-adds per output.)
 //
 // Precision. A tensor core's accumulator drops low bits at every step of 16: over a long contraction more than the one rounding per term of a
 // chain of multiply-adds. So the leading products are summed in tensor memory over 128 terms of the contraction only and these sums added,
@@ -41,7 +42,7 @@ struct FloatProduct {
     const float *bias, *mask, *A, *B;    // [nseg, N]; [R, N]; the operands themselves
     int32_t *status;
 };
-enum FloatEpilogue { FE_PLAIN = 0, FE_BIAS = 1, FE_BIAS_RELU = 2, FE_MASK = 3 };
+enum FloatEpilogue { FE_PLAIN = 0, FE_BIAS, FE_MASK };
 
 // Three bf16 terms of a float: hi + mid + lo == v exactly, but for bits below 2^-133. (Rounding to nearest; values that would round to infinity
 // are cut instead. Infinities and NaN are their own leading term.)
@@ -317,16 +318,12 @@ __global__ void __launch_bounds__(NTHREADS, 1) float_products_kernel(const __gri
                         if (!isfinite(sums[u][j])) sums[u][j] = float_chain<KIND>(p, t.e, t.row0, t.row_end, row0 + lane, col + j);
                 }
                 __syncwarp();
-                if (EPI == FE_BIAS || EPI == FE_BIAS_RELU) {
+                if (EPI == FE_BIAS) {
 #pragma unroll
                     for (int q = 0; q < 8; ++q) {
                         const float4 b = reinterpret_cast<const float4 *>(p.bias + (int64_t)t.e * p.N + col)[q];
                         sums[u][4 * q] += b.x; sums[u][4 * q + 1] += b.y; sums[u][4 * q + 2] += b.z; sums[u][4 * q + 3] += b.w;
                     }
-                }
-                if (EPI == FE_BIAS_RELU) {
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) sums[u][j] = fmaxf(sums[u][j], 0.0f);
                 }
                 if (EPI == FE_MASK && lane < rows_valid) {
 #pragma unroll
@@ -352,7 +349,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) float_products_kernel(const __gri
                     const int64_t r = out0 + row0 + row;
                     const int32_t c = col + (lane & 7) * 4;
                     *reinterpret_cast<float4 *>(p.out + r * p.N + c) = v;
-                    if ((EPI == FE_BIAS_RELU || EPI == FE_MASK) && p.terms) store_terms(v, p.terms + r * 3 * p.N + c, p.N);
+                    if (EPI == FE_MASK && p.terms) store_terms(v, p.terms + r * 3 * p.N + c, p.N);
                 }
                 __syncwarp();
             }
@@ -470,42 +467,32 @@ bool tc_float_supported(const moe_config &c, bool backward) {
     const int64_t R = (int64_t)c.T * c.k;
     if (c.act != MOE_F32 || c.d % 64 != 0 || c.h % 64 != 0) return false;
     if ((int64_t)c.n * c.d * c.h >= (int64_t)1 << 32 || R * (c.d > c.h ? c.d : c.h) >= (int64_t)1 << 32) return false;  // quads are numbered with 31 bits
-    if (c.flags & MOE_FLAG_RECOMPUTE_HID) backward = false;  // the activations have to come out again as the forward call computed them
     return R >= (backward ? 24 : 32) * (int64_t)c.n && (double)R * c.d * c.h >= (backward ? 4.0e6 : 1.0e8);
 }
 
-int32_t launch_float_ffn(const moe_config &c, const void *xs, const int32_t *offsets, const void *W1, const void *b1, const void *W2, const void *b2,
-                         void *hid, void *ys, const SegmentPlan &plan, const FloatTerms &t, int32_t *status, cudaStream_t st) {
+int32_t launch_float_ys(const moe_config &c, const int32_t *offsets, const void *hid, const void *W2, const void *b2, void *ys, const SegmentPlan &plan,
+                        const FloatTerms &t, int32_t *status, cudaStream_t st) {
     const FloatCall call = {c, plan, offsets, status, st, (int64_t)c.T * c.k};
     TermsList list;
-    list.add(xs, t.xs, call.R, c.d);
-    list.add(W1, t.W1, (int64_t)c.n * c.d, c.h);
+    list.add(hid, t.hid, call.R, c.h);
     list.add(W2, t.W2, (int64_t)c.n * c.h, c.d);
     MOE_TRY(list.launch(st));
-    FloatLaunch<ROW_BMN, FE_BIAS_RELU, false> first;
-    MOE_TRY(call.row(&first, xs, t.xs, W1, t.W1, c.h, c.d, hid, b1, nullptr, t.hid));
-    MOE_TRY(call.launch(first));
-    FloatLaunch<ROW_BMN, FE_BIAS, false> second;
-    MOE_TRY(call.row(&second, hid, t.hid, W2, t.W2, c.d, c.h, ys, b2, nullptr, nullptr));
-    return call.launch(second);
+    FloatLaunch<ROW_BMN, FE_BIAS, false> L;
+    MOE_TRY(call.row(&L, hid, t.hid, W2, t.W2, c.d, c.h, ys, b2, nullptr, nullptr));
+    return call.launch(L);
 }
 
-int32_t launch_float_ffn_bwd(const moe_config &c, const void *xs, void *hid, bool again, const void *dys, const int32_t *offsets, const void *W1,
-                             const void *b1, const void *W2, void *dxs, void *dW1, void *dW2, void *dz, const SegmentPlan &plan, const FloatTerms &t,
+int32_t launch_float_ffn_bwd(const moe_config &c, const void *xs, const void *hid, const void *dys, const int32_t *offsets, const void *W1,
+                             const void *W2, void *dxs, void *dW1, void *dW2, void *dz, const SegmentPlan &plan, const FloatTerms &t,
                              int32_t *status, cudaStream_t st) {
     const FloatCall call = {c, plan, offsets, status, st, (int64_t)c.T * c.k};
     TermsList list;
     list.add(xs, t.xs, call.R, c.d);
     list.add(dys, t.dys, call.R, c.d);
+    list.add(hid, t.hid, call.R, c.h);
     list.add(W1, t.W1, (int64_t)c.n * c.d, c.h);
     list.add(W2, t.W2, (int64_t)c.n * c.h, c.d);
-    if (!again) list.add(hid, t.hid, call.R, c.h);
     MOE_TRY(list.launch(st));
-    if (again) {
-        FloatLaunch<ROW_BMN, FE_BIAS_RELU, false> first;
-        MOE_TRY(call.row(&first, xs, t.xs, W1, t.W1, c.h, c.d, hid, b1, nullptr, t.hid));
-        MOE_TRY(call.launch(first));
-    }
     FloatLaunch<ROW_BK, FE_MASK, true> by_w2;
     MOE_TRY(call.wgrad(&by_w2, hid, t.hid, dys, t.dys, c.h, c.d, dW2));
     MOE_TRY(call.row(&by_w2, dys, t.dys, W2, t.W2, c.h, c.d, dz, nullptr, hid, t.dz));
