@@ -1,6 +1,6 @@
-// Strided SIMT grouped GEMM in float accumulation. It serves gate projections whose widths are no whole quads (the others: projection.cu), float
-// layers of few rows or little work (the others: products_f32.cu), and the two dense contractions of the gate backward where neither the tensor
-// cores (ffn_tc.cu) nor gate_products.cu take them.
+// Strided SIMT grouped GEMM in float accumulation. It serves the largest float projections and those of short single-float rows (the others:
+// projection.cu), float layers with many rows an expert whose widths are no multiples of 64 or whose work is little (the others: products_f32.cu, few_rows.cu),
+// and the two dense contractions of the gate backward where neither the tensor cores (ffn_tc.cu) nor gate_products.cu take them.
 //
 // Every output is one chain of fused multiply-adds over the contraction index in ascending order, starting from +0
 // (contractions cut into slices: one such chain per slice, the slices added in double). That is bound by the FP32
@@ -449,9 +449,8 @@ static int32_t simt_launch(SimtRun &run, int32_t *tile_prefix, cudaStream_t st) 
 // tiles 58); else 32 x 32 tiles (4 x 4), and where even those leave SMs idle 16 x 16 (2 x 2, K blocks of 64): there a
 // block's time is the latency of one chain and its loads (24 tokens x 512 features x 64 columns: 9 us; one 128 x 64
 // tile: 40).
-// Gate widths that are no multiple of four: the projection (AK, BJ) takes 128 x 64 tiles from one and a half per SM on (a whole
-// moe_gate, 4096 tokens x 512 features: 250 experts, 256 tiles, 77 us against 96 with 32 x 32 tiles; 130 experts, 160 tiles,
-// 71 against 59; 64 x 64 tiles in between: 82 and 63), else 32 x 32 ones; the gradients take 32 x 32 element-wise tiles.
+// Gate widths that are no multiple of four: the projections that come here (projection.cu keeps the smaller ones) have six 128 x 64 tiles and more
+// per SM; the gradient of x takes 32 x 32 element-wise tiles.
 template <typename TA, typename TB, typename TC, bool AK, bool BJ>
 static int32_t simt_pick_tile(SimtRun &run, bool vec_a, bool vec_b, int32_t *tile_prefix, cudaStream_t st) {
     const SimtGemm &g = run.g;
@@ -463,11 +462,11 @@ static int32_t simt_pick_tile(SimtRun &run, bool vec_a, bool vec_b, int32_t *til
     if (!(vec_a && vec_b)) {
         if constexpr (AK && BJ) {
             if (!vec_a) return MOE_ERR_UNSUPPORTED;  // activations have rows of whole 16-byte vectors
-            if (2 * blocks(128, 64) >= 3 * 148)
-                return simt_launch<TA, TB, TC, true, false, AK, BJ, 128, 64, 8, 8, 16>(run, tile_prefix, st);
-            return simt_launch<TA, TB, TC, true, false, AK, BJ, 32, 32, 4, 4, 32>(run, tile_prefix, st);
-        } else {
+            return simt_launch<TA, TB, TC, true, false, AK, BJ, 128, 64, 8, 8, 16>(run, tile_prefix, st);
+        } else if constexpr (AK) {
             return simt_launch<TA, TB, TC, false, false, AK, BJ, 32, 32, 4, 4, 32>(run, tile_prefix, st);
+        } else {
+            return MOE_ERR_UNSUPPORTED;  // gate_products.cu
         }
     }
     if constexpr (AK && BJ && std::is_same<TA, bf16>::value && std::is_same<TB, float>::value) {
