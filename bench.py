@@ -38,7 +38,7 @@ FP32_PEAK_TFLOPS = 148 * 128 * 2 * 1.965e9 / 1e12
 # under profiles/ records the figure per workload together with the hash of the GEMM source it was taken with: a figure
 # taken with another version of the kernels is not reported (null) rather than carried along
 TRAFFIC_SUMMARY = os.path.join(ROOT, "profiles", "grouped_gemm_dram_traffic.txt")
-GEMM_SOURCE = os.path.join(ROOT, "paper_1701_06538_b200", "csrc", "ffn_tc.cu")
+GEMM_SOURCE = os.path.join(ROOT, "paper_1701_06538_b200", "csrc", "products.cu")
 
 
 def ncu_traffic_bytes_per_step(workload_name):
@@ -51,7 +51,7 @@ def ncu_traffic_bytes_per_step(workload_name):
         sha = hashlib.sha256(open(GEMM_SOURCE, "rb").read()).hexdigest()
     except OSError:
         return None
-    m = re.search(r"^ffn_tc_sha256:\s*([0-9a-f]{64})", text, re.M)
+    m = re.search(r"^products_sha256:\s*([0-9a-f]{64})", text, re.M)
     if not m or m.group(1) != sha:
         return None
     m = re.search(r"^traffic_bytes_per_step\[%s\]:\s*([0-9.eE+]+)" % re.escape(workload_name), text, re.M)

@@ -6,8 +6,9 @@
 // load sixteen bytes a lane along their rows and many in flight; the rows of A wait in shared memory or the first-level cache. Sixteen rows a tile; a tile
 // with fewer runs with eight or four, so that the arithmetic follows the rows that are there. The float product of gemm_simt.cu, whose tiles of 32
 // rows and more stage both operands in shared memory, and this way, us:
-//   416 experts x 1 row of 832 x 512 (709 MB of weights): rows 312, 312 -> 130, 138; transposed 334, 333 -> 133, 128; gradients 402, 374 -> 122, 119
-//   (5.5 TB/s in, 5.9 TB/s out); 32 x 9 of 512 x 3712 (243 MB): rows 125, 190 -> 74, 100; transposed 139, 208 -> 89, 88; gradients 142, 138 -> 53, 53
+//   416 experts x 1 row of 832 x 512 (709 MB of weights): rows 312 -> 138; transposed 334, 333 -> 133, 128; gradients 402, 374 -> 122, 119
+//   (5.5 TB/s in, 5.9 TB/s out); 32 x 9 of 512 x 3712 (243 MB): rows 190 -> 100; transposed 139, 208 -> 89, 88; gradients 142, 138 -> 53, 53
+// The product that makes hid is not among them: its signs are the ReLU mask, and it keeps one chain of multiply-adds per output (api.cu).
 #include "async_copy.cuh"
 #include "moe_internal.cuh"
 
@@ -252,7 +253,7 @@ template <int LC> __global__ void __launch_bounds__(FEW_THREADS, 4) few_gradient
 }
 
 // Up to as many rows an expert as this way is the faster one. us, products of 64 experts of 200 x 520, by the float product and this way, rows an expert:
-//   rows         16 29.5 + 34.6, 23.9 + 24.4;  32 42.0 + 36.8, 32.6 + 36.0;  48 36.4 + 54.4, 42.6 + 38.0;  64 50.5 + 68.7, 51.3 + 54.1;  128 75 + 89, 86 + 83
+//   rows         16 34.6, 24.4;  32 36.8, 36.0;  48 54.4, 38.0;  64 68.7, 54.1;  128 89, 83, and 50.5, 51.3 at 64 and 75, 86 at 128 into the wider side
 //   transposed   16 31.3 + 35.5, 22.5 + 22.5;  32 37.7 + 37.0, 36.0 + 31.4;  48 37.0 + 53.0, 49.4 + 43.1;  64 52.9 + 68.5, 63.0 + 54.0
 //   gradients    16 39.0 + 35.6, 13.5 + 14.4;  64 55.9 + 57.6, 36.7 + 40.6;  128 72.8 + 76.7, 66.1 + 72.3;  256 122 + 125, 128 + 141
 // Gradients of many rows need blocks besides: 8 experts of 64 x 128 with 32 rows, 16 blocks, 4.6 + 4.4, this way 5.7 + 5.8.

@@ -1,6 +1,7 @@
 // Strided SIMT grouped GEMM in float accumulation. It serves the largest float projections and those of short single-float rows (the others:
-// projection.cu), float layers with many rows an expert whose widths are no multiples of 64 or whose work is little (the others: products_f32.cu, few_rows.cu),
-// and the two dense contractions of the gate backward where neither the tensor cores (ffn_tc.cu) nor gate_products.cu take them.
+// projection.cu), the first product of float layers and, with many rows an expert, the other ones of widths that are no multiples of 64 or of little
+// work (else: products_f32.cu, few_rows.cu), and the contractions of the gate backward where neither the tensor cores (ffn_tc.cu) nor
+// gate_products.cu take them.
 //
 // Every output is one chain of fused multiply-adds over the contraction index in ascending order, starting from +0
 // (contractions cut into slices: one such chain per slice, the slices added in double). That is bound by the FP32
