@@ -458,16 +458,16 @@ struct FloatCall {
 
 }  // namespace
 
-// A call has to make the terms of all weights (16 bytes of traffic a float): forward from 32 rows an expert and 1e8 multiply-adds a product on,
-// backward, with twice the products for the same terms, from 24 and 4e6. us, by FP32 multiply-adds (few_rows.cu up to 64 rows) and this way. A forward
-// call: 32 experts x 64 rows of 1024 x 1024 332, 244; 32 x 32 230, 237; 16 x 64 of 256 x 512 (1.3e8) 48.5, 52.7; 8 x 128 of 128 x 128 (1.7e7) 31.1, 35.3.
-// A step: 64 experts x 16 rows of 256 x 512 162, 176; x 24 199, 201; x 32 222, 212; x 48 279, 226; 300 x 24 901, 902; 8 x 25 of 512 x 4096 314, 365;
-// 32 x 31 of 1024 x 1024 578, 555; 64 x 32 of 64 x 128 85.6, 77.9. The backward call of 8 x 64 of 64 x 128 (4.2e6) 41.0, 39.4.
+// A call has to make the terms of the weights (10 bytes of traffic a float): forward, one product, from 32 rows an expert and 1e8 multiply-adds a product
+// on, backward, four products, from 28 and 4e6. us, by FP32 multiply-adds (few_rows.cu up to 64 rows) and this way. A forward call: 32 experts x 64
+// rows of 1024 x 1024 365, 318; 32 x 32 277, 278; 16 x 64 of 256 x 512 (1.3e8) 54.2, 56.0; 16 x 100 75.0, 68.8; 64 x 40 of 512 x 512 167, 163.
+// A step: 64 experts x 24 rows of 256 x 512 198, 203; x 32 237, 223; x 48 283, 231; 300 x 24 931, 934; 8 x 25 of 512 x 4096 339, 393;
+// 32 x 31 of 1024 x 1024 625, 603; 64 x 32 of 64 x 128 86.2, 79.0. The backward call of 8 x 64 of 64 x 128 (4.2e6) 41.0, 39.4.
 bool tc_float_supported(const moe_config &c, bool backward) {
     const int64_t R = (int64_t)c.T * c.k;
     if (c.act != MOE_F32 || c.d % 64 != 0 || c.h % 64 != 0) return false;
     if ((int64_t)c.n * c.d * c.h >= (int64_t)1 << 32 || R * (c.d > c.h ? c.d : c.h) >= (int64_t)1 << 32) return false;  // quads are numbered with 31 bits
-    return R >= (backward ? 24 : 32) * (int64_t)c.n && (double)R * c.d * c.h >= (backward ? 4.0e6 : 1.0e8);
+    return R >= (backward ? 28 : 32) * (int64_t)c.n && (double)R * c.d * c.h >= (backward ? 4.0e6 : 1.0e8);
 }
 
 int32_t launch_float_ys(const moe_config &c, const int32_t *offsets, const void *hid, const void *W2, const void *b2, void *ys, const SegmentPlan &plan,
