@@ -409,7 +409,7 @@ def run_ours(args, w):
     achieved = gemm_flop / (gemm_ms / 1e3) / 1e12
     achieved_gbs = gemm_bytes / (gemm_ms / 1e3) / 1e9
     traffic = ncu_traffic_bytes_per_step(workload_config(w)["workload"])
-    kernel = "expert grouped GEMMs (moe_expert_ffn + moe_expert_ffn_bwd, 6 launches; achieved = per-step flop or bytes / per-step time)"
+    kernel = "expert grouped GEMMs (moe_expert_ffn + moe_expert_ffn_bwd, 6 products; achieved = per-step flop or bytes / per-step time)"
     if w.act != "bf16":
         roof = {"bound": "alu", "kernel": "expert grouped GEMMs, fp32 SIMT", "achieved": achieved,
                 "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": achieved / FP32_PEAK_TFLOPS, "traffic": None,
