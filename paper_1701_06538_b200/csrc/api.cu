@@ -201,6 +201,7 @@ SegmentPlan make_plan(const moe_config *c, const Dims &D, int32_t *ws, bool back
     if (tc_ffn_takes(*c)) {
         p.bm[0] = tc_row_tile(*c);
         if (backward && p.bm[0] != COLSUM_ROWS) p.bm[1] = COLSUM_ROWS;
+        if (!tc_ffn_supported(*c)) { p.bm[1] = 64; p.bm[2] = 32; p.bm[3] = 16; }  // of the product that makes hid
         if (!backward || !tc_wgrad_sorted(*c)) {
             p.sched = nullptr;
             p.by_rank = p.prefix[0];
@@ -501,10 +502,10 @@ int32_t do_dispatch(const Dims &D, const void *x, const int32_t *topk_idx, void 
     return launch_dispatch_rows(x, D.act, D.T, (int32_t)D.k, (int32_t)D.d, inv_perm, xs, st, sums);
 }
 
-SimtGemm base_gemm() {  // of float experts
+SimtGemm base_gemm(GemmType type = G_F32) {  // of experts
     SimtGemm g;
     memset(&g, 0, sizeof(g));
-    g.ta = g.tb = g.tc = G_F32;
+    g.ta = g.tb = g.tc = type;
     g.a_row_div = 1;
     return g;
 }
@@ -529,16 +530,17 @@ int32_t do_expert_ffn(const moe_config *c, const Dims &D, const void *xs, const 
         fill_plan(&args, plan, (int32_t)D.n, D.R, clear, tc ? &maps : nullptr);
         MOE_TRY(launch_segment_plan(args, offsets, st));
     }
-    if (tc_ffn_takes(*c))
+    if (tc_ffn_supported(*c))
         return launch_tc_ffn(*c, xs, offsets, W1, b1, W2, b2, hid, ys, plan, status_word(ws_base), st, first_only, relu_bits);
-    // hid = relu(xs.W1 + b1): one chain of multiply-adds per output, whatever computes the other products, since its zeros decide the mask of the backward
-    // pass: a value next to 0 that rounds to the other side with another order of its sum is a whole term of dW1 and dX
-    SimtGemm g = base_gemm();
+    // hid = relu(xs.W1 + b1) of float layers and odd widths: one chain of multiply-adds per output, whatever computes the other products, since its zeros
+    // decide the mask of the backward pass: a value next to 0 that rounds to the other side with another order of its sum is a whole term of dW1 and dX
+    SimtGemm g = base_gemm(D.act == MOE_BF16 ? G_BF16 : G_F32);
     g.A = xs; g.B = W1; g.C = hid; g.bias = b1; g.relu = 1;
     g.sa_i = D.d; g.sa_k = 1; g.sb_k = D.h; g.sb_j = 1; g.sc_i = D.h;
     g.mode = 0; g.offsets = offsets; g.nseg = (int32_t)D.n; g.M = D.R; g.N = D.h; g.K = D.d; g.b_e = D.d * D.h;
     MOE_TRY(launch_simt_gemm(g, nullptr, st, nullptr, &plan));
     if (first_only) return MOE_OK;
+    if (tc_ffn_takes(*c)) return launch_tc_ys(*c, offsets, W2, b2, hid, ys, plan, status_word(ws_base), st);
     if (D.float_terms[0]) return launch_float_ys(*c, offsets, hid, W2, b2, ys, plan, w.terms, status_word(ws_base), st);
     g = base_gemm();  // ys = hid.W2 + b2
     g.A = hid; g.B = W2; g.C = ys; g.bias = b2;

@@ -1,5 +1,5 @@
 // Strided SIMT grouped GEMM in float accumulation. It serves the largest float projections and those of short single-float rows (the others:
-// projection.cu), the first product of float layers and, with many rows an expert, the other ones of widths that are no multiples of 64 or of little
+// projection.cu), the first product of float layers and of bf16 layers of odd widths and, with many rows an expert, the other ones of widths that are no multiples of 64 or of little
 // work (else: products_f32.cu, few_rows.cu), and the contractions of the gate backward where neither the tensor cores (ffn_tc.cu) nor
 // gate_products.cu take them.
 //
@@ -461,7 +461,9 @@ static int32_t simt_pick_tile(SimtRun &run, bool vec_a, bool vec_b, int32_t *til
     };
     const bool short_rows = g.mode == 0 && g.offsets && g.M <= 32 * (int64_t)g.nseg;  // segments of few rows: less padding
     if (!(vec_a && vec_b)) {
-        if constexpr (AK && BJ) {
+        if constexpr (std::is_same<TC, bf16>::value) {  // an expert product: widths are whole 16-byte vectors
+            return MOE_ERR_UNSUPPORTED;
+        } else if constexpr (AK && BJ) {
             if (!vec_a) return MOE_ERR_UNSUPPORTED;  // activations have rows of whole 16-byte vectors
             return simt_launch<TA, TB, TC, true, false, AK, BJ, 128, 64, 8, 8, 16>(run, tile_prefix, st);
         } else if constexpr (AK) {
@@ -521,6 +523,7 @@ int32_t launch_simt_gemm(const SimtGemm &g_in, int32_t *tile_prefix, cudaStream_
     if (ak && bj) {  // rows x weight [K, N]
         if (fff) return simt_pick_tile<float, float, float, true, true>(run, vec_a, vec_b, tile_prefix, st);
         if (bff) return simt_pick_tile<bf16, float, float, true, true>(run, vec_a, vec_b, tile_prefix, st);
+        if (g.ta == G_BF16 && g.tb == G_BF16 && g.tc == G_BF16) return simt_pick_tile<bf16, bf16, bf16, true, true>(run, vec_a, vec_b, tile_prefix, st);
     } else if (ak) {  // rows x weight [N, K] read transposed
         if (fff) return simt_pick_tile<float, float, float, true, false>(run, vec_a, vec_b, tile_prefix, st);
     } else if (bj) {  // contraction over rows

@@ -445,6 +445,8 @@ int32_t tc_segment_maps(const moe_config &c, SegmentMaps *maps, const void *xs_r
 int32_t tc_row_tile(const moe_config &c);    // tile height of the row products: what plan.bm[0] has to be
 bool tc_wgrad_sorted(const moe_config &c);   // the backward products want plan.sched
 // first_only: only hid = relu(xs.W1 + b1) (the recomputation of the hidden activations in the backward pass)
+int32_t launch_tc_ys(const moe_config &c, const int32_t *offsets, const void *W2, const void *b2, const void *hid, void *ys, const SegmentPlan &plan,
+                     int32_t *status_word, cudaStream_t st);  // the second product alone
 int32_t launch_tc_ffn(const moe_config &c, const void *xs, const int32_t *offsets, const void *W1, const void *b1,
                       const void *W2, const void *b2, void *hid, void *ys, const SegmentPlan &plan, int32_t *status_word,
                       cudaStream_t st, bool first_only = false, uint32_t *relu_bits = nullptr);

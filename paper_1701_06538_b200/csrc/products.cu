@@ -853,8 +853,8 @@ class ProductList {
         // 256 x 188 rows 1289, dealt 1273)
         P.counter = pairs || tiles > 64 * (int64_t)tc_sm_count() ? drawn : nullptr;
         if (!whole(c)) {
-            if constexpr (SET != SET_DZ_DW2) return launch_products_as<false, 4, SET, false>(maps, P, tiles, st);
-            return MOE_ERR_UNSUPPORTED;  // (no bits without whole words)
+            if constexpr (SET != SET_DZ_DW2 && SET != SET_HID) return launch_products_as<false, 4, SET, false>(maps, P, tiles, st);
+            return MOE_ERR_UNSUPPORTED;  // (no bits without whole words; hid: api.cu)
         }
         if (pairs) return launch_products_as<true, 6, SET, true>(maps, P, tiles, st);
         // Weight gradients of one or two K blocks a tile last as long as their epilogue, 1100 cycles a box, 420 of them waiting until the
@@ -880,9 +880,9 @@ bool tc_ffn_supported(const moe_config &c) {
     return c.act == MOE_BF16 && c.d % 64 == 0 && c.h % 64 == 0 && c.d >= 64 && c.h >= 64;
 }
 
-// All bf16 layers: their widths are multiples of eight (a configuration's rows are whole 16-byte vectors). us a step by FP32 multiply-adds, which widths that
-// are no multiples of 64 had, and this way: 64 experts x 200 rows of 72 x 2056 1257, 238; 20 x 300 of 120 x 1000 396, 98; 32 x 500 of 200 x 200 452, 135;
-// 200 x 2 of 136 x 264 245, 118; 16 x 40 of 8 x 16 73, 67; forward calls of a few tokens, bound by their launches: 32 x 72 x 136 30.7, 31.8.
+// All bf16 layers: their widths are multiples of eight (a configuration's rows are whole 16-byte vectors). us a step of widths that are no multiples of 64 by
+// FP32 multiply-adds and this way (hid stays with them, see api.cu): 64 experts x 200 rows of 72 x 2056 1257, 368; 20 x 300 of 120 x 1000 396, 165;
+// 32 x 500 of 200 x 200 452, 181.
 bool tc_ffn_takes(const moe_config &c) { return c.act == MOE_BF16; }
 
 int32_t tc_segment_maps(const moe_config &c, SegmentMaps *maps, const void *xs_rows, const void *hid_rows, const void *dys_rows,
@@ -916,12 +916,18 @@ int32_t launch_tc_ffn(const moe_config &c, const void *xs, const int32_t *offset
                       const void *W2, const void *b2, void *hid, void *ys, const SegmentPlan &plan, int32_t *status_word,
                       cudaStream_t st, bool first_only, uint32_t *relu_bits) {
     if ((int64_t)c.T * c.k == 0) return MOE_OK;
-    ProductList hidden(c, plan, offsets, PLAN_HID, status_word), out(c, plan, offsets, PLAN_YS, status_word);
+    ProductList hidden(c, plan, offsets, PLAN_HID, status_word);
     Product *p;
     MOE_TRY(hidden.row(&p, xs, W1, false, c.h, c.d, hid, MAP_XS_ROWS));
     p->bias = (const bf16 *)b1; p->bits_out = relu_bits;
     MOE_TRY(hidden.launch<SET_HID>(st));
-    if (first_only) return MOE_OK;
+    return first_only ? MOE_OK : launch_tc_ys(c, offsets, W2, b2, hid, ys, plan, status_word, st);
+}
+int32_t launch_tc_ys(const moe_config &c, const int32_t *offsets, const void *W2, const void *b2, const void *hid, void *ys, const SegmentPlan &plan,
+                     int32_t *status_word, cudaStream_t st) {
+    if ((int64_t)c.T * c.k == 0) return MOE_OK;
+    ProductList out(c, plan, offsets, PLAN_YS, status_word);
+    Product *p;
     MOE_TRY(out.row(&p, hid, W2, false, c.d, c.h, ys, MAP_HID_ROWS));
     p->bias = (const bf16 *)b2;
     return out.launch<SET_YS>(st);
