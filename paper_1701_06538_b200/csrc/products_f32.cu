@@ -11,7 +11,8 @@
 // and 3.1e-7, 3.2e-7, 3.2e-7; 12 experts, 3000 rows, 128 x 4096: 8.5e-7, 8.5e-7, 3.3e-7 and 2.7e-7, 2.8e-7, 2.5e-7.
 //
 // Values that are no numbers. An infinite operand meets terms of either sign and zeros, and becomes NaN where the float chain has an infinity. Every
-// element that does not come out finite is therefore computed again as the float chain that gemm_simt.cu computes, with its result. (Sums whose
+// element that does not come out finite is therefore computed again as the float chain that gemm_simt.cu computes, with its result: by the CTA that has
+// the tile, when its tensor-core work is done and nothing waits for it any more, as a tile of multiply-adds. (Sums whose
 // parts leave float's range on the way depend on the order of the parts, as ever.)
 //
 // One CTA, 128 x 128 tiles, K blocks of 64: a stage holds the three terms of both operands (96 KiB, two stages), of which the six products
@@ -21,6 +22,7 @@
 
 #include <type_traits>
 
+#include "async_copy.cuh"
 #include "tc.cuh"
 
 namespace moe {
@@ -34,7 +36,7 @@ constexpr int F_SHARED = F_STAGES * F_STAGE + 1024 /*alignment*/ + 8 * 4096 /*a 
 struct FloatProduct {
     const int32_t *offsets, *row_tiles;  // [nseg + 1] bounds of the segments (rows); &number of row tiles
     const int4 *info;                    // per row tile {segment, first row, segment end, number}
-    int32_t nseg, N, M, K;               // ROW_*: K is the contraction, M unused; WGRAD: [M, N] per segment
+    int32_t N, M, K;                     // ROW_*: K is the contraction, M unused; WGRAD: [M, N] per segment
     int32_t tiles_n, per_e, total;       // tiles beside each other; WGRAD: of a segment, of all segments; ROW_*: at most
     Divisor by_tiles_n, by_per_e;
     float *out;
@@ -101,16 +103,127 @@ template <int ROW, int EPI, bool WITH_WGRAD, typename F> __device__ __forceinlin
     f(L.row, std::integral_constant<int, ROW>(), std::integral_constant<int, EPI>());
 }
 
-// One element as the chain of multiply-adds in ascending order
-template <int KIND> __device__ __noinline__ float float_chain(const FloatProduct &p, int32_t e, int32_t row0, int32_t row_end, int64_t row, int32_t col) {
-    float s = 0.0f;
-    if (KIND == WGRAD) {
-        for (int64_t r = row0; r < row_end; ++r) s = fmaf(p.A[r * p.M + row], p.B[r * p.N + col], s);
-    } else {
-        const float *a = p.A + row * p.K;
-        for (int32_t k = 0; k < p.K; ++k) s = fmaf(a[k], KIND == ROW_BMN ? p.B[((int64_t)e * p.K + k) * p.N + col] : p.B[((int64_t)e * p.N + col) * p.K + k], s);
+// The elements of a stored tile that are not finite once more, each as one chain of multiply-adds in ascending order, through shared memory: 8 x 8 outputs a
+// thread of the first 256, bound by the reads of shared memory (16 cycles a warp and row of 180 in all). A backward call, and with a NaN in dys, which makes whole
+// matrices of gradients NaN: 4 experts x 2000 rows of 128 x 256 105 us, 535; 20000 rows of 64 x 128, one tile, 0.80 ms, 4.6. Every element by itself,
+// straight from memory and while the MMA warp waited with its limit of 2 s, 3.8 ms and 37.
+constexpr int R_BK = 32, R_PITCH = F_TILE + 4;
+template <int KIND, int EPI> __device__ __forceinline__ void repair_tile(const FloatProduct &p, const FloatTile &t) {
+    const int tid = threadIdx.x;
+    const int64_t row0 = KIND == WGRAD ? t.m0 : t.row0;
+    float *out = p.out + ((KIND == WGRAD ? (int64_t)t.e * p.M : 0) + row0) * p.N + t.n0;
+    const int rows = (int)min((int64_t)F_TILE, (KIND == WGRAD ? p.M : t.row_end) - row0), cols = min(F_TILE, p.N - t.n0);
+    bool odd = false;
+    for (int i = tid; i < rows * (cols / 4); i += NTHREADS) {
+        const float4 v = *reinterpret_cast<const float4 *>(out + (int64_t)(i / (cols / 4)) * p.N + i % (cols / 4) * 4);
+        odd = odd || !isfinite(v.x) || !isfinite(v.y) || !isfinite(v.z) || !isfinite(v.w);
     }
-    return s;
+    if (!__syncthreads_or(odd)) return;
+    extern __shared__ uint8_t smem_raw[];  // the stages are free
+    constexpr int OPERAND = R_BK * R_PITCH, LOADS = R_BK * F_TILE / 4 / 256;  // [R_BK][R_PITCH] floats: the contraction's index first
+    float *stage = reinterpret_cast<float *>(smem_raw);
+    const int depth = KIND == WGRAD ? t.row_end - t.row0 : p.K, tx = tid & 15, ty = tid >> 4;
+    float acc[8][8];  // rows 4 ty + i % 4 + 64 (i / 4), columns 4 tx + j % 4 + 64 (j / 4)
+#pragma unroll
+    for (int i = 0; i < 64; ++i) acc[i >> 3][i & 7] = 0.0f;
+    // Four neighbours at a time, into one stage while the other one is used: as they lie, by asynchronous copies; or, where they are neighbours along the
+    // contraction, through registers, turned on the way
+    constexpr bool TURN_A = KIND != WGRAD, TURN_B = KIND == ROW_BK;
+    auto place = [&](bool turn, int q, int &across, int &along) {
+        const int i = tid + 256 * q;
+        across = turn ? i / (R_BK / 4) : i % (F_TILE / 4) * 4;
+        along = turn ? i % (R_BK / 4) * 4 : i / (F_TILE / 4);
+    };
+    float4 turned[TURN_A + TURN_B + 1][LOADS];
+    auto fetch = [&](int k0, float *as) {
+        float *bs = as + OPERAND;
+#pragma unroll
+        for (int q = 0; q < LOADS; ++q) {
+            int c, k;
+            place(TURN_A, q, c, k);
+            const bool live_a = c < rows && k0 + k < depth;
+            const float *a = !live_a ? p.A : TURN_A ? p.A + (t.row0 + c) * (int64_t)p.K + k0 + k : p.A + (int64_t)(t.row0 + k0 + k) * p.M + t.m0 + c;
+            if (TURN_A) turned[0][q] = live_a ? *reinterpret_cast<const float4 *>(a) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            else copy16(as + k * R_PITCH + c, a, live_a);
+            place(TURN_B, q, c, k);
+            const bool live_b = c < cols && k0 + k < depth;
+            const float *b = !live_b         ? p.B
+                             : KIND == WGRAD ? p.B + (int64_t)(t.row0 + k0 + k) * p.N + t.n0 + c
+                             : TURN_B        ? p.B + ((int64_t)t.e * p.N + t.n0 + c) * p.K + k0 + k
+                                             : p.B + ((int64_t)t.e * p.K + k0 + k) * p.N + t.n0 + c;
+            if (TURN_B) turned[1][q] = live_b ? *reinterpret_cast<const float4 *>(b) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            else copy16(bs + k * R_PITCH + c, b, live_b);
+        }
+        copies_commit();
+    };
+    auto put = [&](float *to, bool turn, const float4 (&v)[LOADS]) {
+        if (!turn) return;
+#pragma unroll
+        for (int q = 0; q < LOADS; ++q) {
+            int c, k;
+            place(true, q, c, k);
+            float *at = to + k * R_PITCH + c;
+            at[0] = v[q].x; at[R_PITCH] = v[q].y; at[2 * R_PITCH] = v[q].z; at[3 * R_PITCH] = v[q].w;
+        }
+    };
+    const int last_row = rows > 64, last_col = cols > 64;  // whether the tile's second halves have elements
+    __syncthreads();
+    if (tid < 256) fetch(0, stage);
+    int at = 0;
+    for (int k0 = 0; k0 < depth; k0 += R_BK, at ^= 1) {
+        float *as = stage + at * 2 * OPERAND, *bs = as + OPERAND;
+        if (tid < 256) {
+            put(as, TURN_A, turned[0]);
+            put(bs, TURN_B, turned[TURN_B]);
+            copies_wait<0>();
+        }
+        __syncthreads();  // this stage is there for all, the other one is read by all
+        if (tid >= 256) continue;
+        if (k0 + R_BK < depth) fetch(k0 + R_BK, stage + (at ^ 1) * 2 * OPERAND);
+#pragma unroll 4
+        for (int k = 0; k < R_BK; ++k) {  // (zeros behind the end: a sum that began with +0 is never -0, so they do not change it)
+            float a[8], b[8];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                *reinterpret_cast<float4 *>(a + 4 * u) = *reinterpret_cast<const float4 *>(as + k * R_PITCH + 4 * ty + 64 * u);
+                *reinterpret_cast<float4 *>(b + 4 * u) = *reinterpret_cast<const float4 *>(bs + k * R_PITCH + 4 * tx + 64 * u);
+            }
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                if ((h >> 1) > last_row || (h & 1) > last_col) continue;
+#pragma unroll
+                for (int i = 4 * (h >> 1); i < 4 * (h >> 1) + 4; ++i)
+#pragma unroll
+                    for (int j = 4 * (h & 1); j < 4 * (h & 1) + 4; j += 2) fma_two(acc[i][j], acc[i][j + 1], a[i], b[j], b[j + 1]);
+            }
+        }
+    }
+    if (tid < 256) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int r = 4 * ty + i % 4 + 64 * (i / 4);
+            if (r >= rows) break;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int c = 4 * tx + j % 4 + 64 * (j / 4);
+                if (c >= cols) continue;
+                float *to = out + (int64_t)r * p.N + c;
+                if (isfinite(*to)) continue;  // (zeros of the mask among them)
+                float v = acc[i][j];
+                if (EPI == FE_BIAS) v += p.bias[(int64_t)t.e * p.N + t.n0 + c];
+                *to = v;
+                if (EPI == FE_MASK && p.terms) {
+                    bf16 *terms = p.terms + (row0 + r) * 3 * p.N + t.n0 + c;
+                    three_terms(v, terms[0], terms[p.N], terms[2 * (int64_t)p.N]);
+                }
+            }
+        }
+    }
+}
+template <int ROW, int EPI_ROW, bool WITH_WGRAD> __device__ __noinline__ void repair_tiles(const FloatLaunch<ROW, EPI_ROW, WITH_WGRAD> &L) {
+    FloatTile t;
+    for (int32_t id = blockIdx.x; float_tile(L, id, t); id += gridDim.x)
+        with_product(L, t, [&](const FloatProduct &p, auto KIND_, auto EPI_) { repair_tile<decltype(KIND_)::value, decltype(EPI_)::value>(p, t); });
 }
 
 template <int ROW, int EPI_ROW, bool WITH_WGRAD>
@@ -127,6 +240,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) float_products_kernel(const __gri
     auto sempty_bar = [&](int a) { return bars + 80u + 8u * a; };
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(smem + F_STAGES * F_STAGE + 8 * 4096 + 96);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + F_STAGES * F_STAGE + 8 * 4096 + 104);
+    volatile int *odd_tiles = reinterpret_cast<volatile int *>(smem + F_STAGES * F_STAGE + 8 * 4096 + 108);  // a stored element is not finite
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < 2; ++s) {
@@ -135,6 +249,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) float_products_kernel(const __gri
             mbar_init(sfull_bar(s), 1); mbar_init(sempty_bar(s), 8);
         }
         *abort_flag = 0;
+        *odd_tiles = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(WITH_WGRAD ? &L.wgrad_a : &L.row_a) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(WITH_WGRAD ? &L.wgrad_b : &L.row_b) : "memory");
@@ -309,15 +424,6 @@ __global__ void __launch_bounds__(NTHREADS, 1) float_products_kernel(const __gri
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
                 const int32_t col = col0 + 32 * u;
-                float odd = 0.0f;  // x - x is 0, or NaN where x is not finite
-#pragma unroll
-                for (int j = 0; j < 32; ++j) odd += sums[u][j] - sums[u][j];
-                if (odd != 0.0f && lane < rows_valid) {
-#pragma unroll
-                    for (int j = 0; j < 32; ++j)
-                        if (!isfinite(sums[u][j])) sums[u][j] = float_chain<KIND>(p, t.e, t.row0, t.row_end, row0 + lane, col + j);
-                }
-                __syncwarp();
                 if (EPI == FE_BIAS) {
 #pragma unroll
                     for (int q = 0; q < 8; ++q) {
@@ -335,6 +441,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) float_products_kernel(const __gri
                         if (!(m.w > 0.0f)) sums[u][4 * q + 3] = 0.0f;
                     }
                 }
+                float odd = 0.0f;  // x - x is 0, or NaN where x is not finite
+#pragma unroll
+                for (int j = 0; j < 32; ++j) odd += sums[u][j] - sums[u][j];
+                if (odd != 0.0f && lane < rows_valid) *odd_tiles = 1;
                 // through the warp's slab: lane l moves piece l % 8 of row 4 * i + l / 8
 #pragma unroll
                 for (int q = 0; q < 8; ++q)
@@ -363,6 +473,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) float_products_kernel(const __gri
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)TMEM_COLS) : "memory");
     }
+    if (*odd_tiles && !*abort_flag) repair_tiles(L);
 }
 
 // The three terms of several tensors [rows, cols] in one launch, to [rows][3 cols]: four neighbours a thread, four times
@@ -417,7 +528,7 @@ struct FloatCall {
     FloatProduct product(const void *A, const void *B, int32_t N, void *out) const {
         FloatProduct p;
         memset(&p, 0, sizeof(p));
-        p.offsets = offsets; p.row_tiles = plan.by_rank + c.n; p.info = plan.info; p.nseg = c.n; p.N = N;
+        p.offsets = offsets; p.row_tiles = plan.by_rank + c.n; p.info = plan.info; p.N = N;
         p.tiles_n = (int32_t)cdiv(N, F_TILE); p.by_tiles_n = Divisor::of(p.tiles_n);
         p.out = (float *)out; p.A = (const float *)A; p.B = (const float *)B; p.status = status;
         return p;
