@@ -1,4 +1,4 @@
-// The float experts' products on the tensor cores: every operand as three bf16 terms (hi + mid + lo hold a float's 24 bits), a product as the
+// The float experts' products on the tensor cores: every operand as three bf16 terms (hi + mid + lo hold a float's 24 bits, see three_terms), a product as the
 // six terms of at most 2^-16 of the leading one and more: hi.hi, and hi.mid, mid.hi, mid.mid, hi.lo, lo.hi. Float products by FP32
 // multiply-adds (gemm_simt.cu) run at 20 to 29 of the chip's 74 TFLOP/s; this way five of the six products of a step with 16 experts x 260 rows
 // of 256 x 512 take 14 to 16 us each instead of 38 to 52, most of it the way of the operands from L2. (The first, whose signs are the ReLU mask, stays
@@ -46,9 +46,13 @@ struct FloatProduct {
 };
 enum FloatEpilogue { FE_PLAIN = 0, FE_BIAS, FE_MASK };
 
-// Three bf16 terms of a float: hi + mid + lo == v exactly, but for bits below 2^-133. (Rounding to nearest; values that would round to infinity
-// are cut instead. Infinities and NaN are their own leading term.)
-__device__ __forceinline__ void three_terms(float v, bf16 &hi, bf16 &mid, bf16 &lo) {
+// Three bf16 terms of a float times 2^16: hi + mid + lo == 2^16 v exactly, down to float's smallest bit 2^-149, since bf16's is 2^-133 (without the factor
+// values of 1e-36 had 15 bits, and ys of such activations errors of 1e-4 of its size). Values from 2^112 on, and sums of products from 2^96, leave float's range: these
+// outputs are not finite and computed again. (Rounding to nearest; values that would round to infinity are cut instead. Infinities and NaN are
+// their own leading term.)
+constexpr float F_SCALE = 0x1p16f, F_UNSCALE = 0x1p-32f;  // of an operand; of a product of two
+__device__ __forceinline__ void three_terms(float unscaled, bf16 &hi, bf16 &mid, bf16 &lo) {
+    const float v = unscaled * F_SCALE;
     const uint32_t size = __float_as_uint(v) & 0x7fffffffu;
     hi = __float2bfloat16_rn(v);
     if (size >= 0x7f7f8000u && size < 0x7f800000u) hi = __ushort_as_bfloat16((unsigned short)(__float_as_uint(v) >> 16));
@@ -415,6 +419,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) float_products_kernel(const __gri
                 add(256 + small * F_TILE, sempty_bar(small));
                 if (++small == 2) { small = 0; small_ph ^= 1u; }
             }
+#pragma unroll
+            for (int i = 0; i < 64; ++i) sums[i >> 5][i & 31] *= F_UNSCALE;
             with_product(L, t, [&](const FloatProduct &p, auto KIND_, auto EPI_) {
             constexpr int KIND = decltype(KIND_)::value, EPI = decltype(EPI_)::value;
             const int64_t row0 = (KIND == WGRAD ? t.m0 : t.row0) + quarter * 32, out0 = KIND == WGRAD ? (int64_t)t.e * p.M : 0;

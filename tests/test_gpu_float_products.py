@@ -130,3 +130,39 @@ def test_a_nan_does_not_make_a_call_slow(counts, d, h):
     clean = least_ms()
     dys[5, 3] = float("nan")
     assert least_ms() <= 10 * clean
+
+
+@pytest.mark.parametrize("of_hid,of_dys,of_w2,of_w1", [(1, 1e-36, 1, 1), (3e-37, 1, 1, 1), (1, 1e-6, 1e-30, 1), (1, 1, 1, 1e-36), (1e-30, 1e-7, 1e10, 1e-34),
+                                                       (1e20, 1e14, 1e-10, 1e-8), (1, 1e30, 1, 1e-30)])
+def test_operands_near_the_ends_of_floats_range(of_hid, of_dys, of_w2, of_w1):
+    """Operands hold their 24 bits down to float's smallest number, and products as far up as float goes."""
+    counts, d, h = [130, 0, 63, 700, 1, 257], 192, 320
+    cfg, offsets, xs, dys, W1, b1, W2, b2, ws = layer(counts, d, h, 13)
+    n, R = len(counts), sum(counts)
+    hid = torch.relu(torch.randn(R, h, device="cuda", generator=torch.Generator(device="cuda").manual_seed(4))) * of_hid
+    dys, W2, W1 = dys * of_dys, W2 * of_w2, W1 * of_w1
+    for e, got in enumerate(zip(*[[t[int(offsets[e]):int(offsets[e + 1])] if i == 0 else t[e] for e in range(n)] for i, t in
+                                  enumerate(backward(cfg, offsets, xs, hid, dys, W1, W2, ws))])):
+        r = slice(int(offsets[e]), int(offsets[e + 1]))
+        x, dy, hd, w1, w2 = (t.double() for t in (xs[r], dys[r], hid[r], W1[e], W2[e]))
+        dz = (dy @ w2.t()) * (hd > 0)
+        for i, exp in enumerate((dz @ w1.t(), x.t() @ dz, hd.t() @ dy)):
+            rms = exp.square().mean().sqrt() if exp.numel() else 0.0
+            if rms < 1e-34 * 1e-3:  # too little of float's 24 bits is left in the results themselves
+                continue
+            err = ((got[i].double() - exp).abs() / (exp.abs() + rms)).max()
+            assert err <= 1e-5, (e, i, float(rms), float(err))  # the tolerance of the float layer
+
+
+def test_a_forward_call_with_activations_near_the_least_float():
+    counts, d, h = [800, 0, 700, 1, 900], 192, 320
+    cfg, offsets, xs, dys, W1, b1, W2, b2, ws = layer(counts, d, h, 14)
+    assert B.moe_query_sizes(cfg).ws_fwd_bytes > 6 * len(counts) * d * h  # the path
+    xs, b1, b2 = xs * 1e-36, b1 * 0.0, b2 * 0.0
+    hid, ys = torch.empty(sum(counts), h, device="cuda"), torch.empty_like(xs)
+    B.moe_expert_ffn(cfg, xs, offsets, W1, b1, W2, b2, hid, ys, ws)
+    assert B.moe_check_status(ws) == 0
+    for e in (0, 2, 4):
+        r = slice(int(offsets[e]), int(offsets[e + 1]))
+        exp = hid[r].double() @ W2[e].double()
+        assert ((ys[r].double() - exp).abs() / (exp.abs() + exp.square().mean().sqrt())).max() <= 1e-5
