@@ -103,6 +103,8 @@ typedef struct moe_sizes {
     int64_t ws_bytes;     /* workspace every stage call accepts (the largest any stage needs)       */
     int64_t ws_fwd_bytes; /* workspace of moe_forward                                               */
     int64_t ws_bwd_bytes; /* workspace of moe_backward                                              */
+                          /* (all-float layers on the tensor cores: up to 8 GiB of it hold the operands'
+                             bf16 terms, 1 GiB with MOE_FLAG_RECOMPUTE_HID; larger ones have none)  */
     int64_t ctx_bytes;    /* context written by moe_forward and read by moe_backward                */
     int64_t adam_state_elems; /* floats of optimiser state of moe_expert_adam_factored: n * (3d + 3h)   */
     int64_t ws_adam_bytes;    /* workspace of moe_expert_adam_factored                                  */

@@ -580,10 +580,13 @@ struct FloatCall {
 // rows of 1024 x 1024 365, 318; 32 x 32 277, 278; 16 x 64 of 256 x 512 (1.3e8) 54.2, 56.0; 16 x 100 75.0, 68.8; 64 x 40 of 512 x 512 167, 163.
 // A step: 64 experts x 24 rows of 256 x 512 198, 203; x 32 237, 223; x 48 283, 231; 300 x 24 931, 934; 8 x 25 of 512 x 4096 339, 393;
 // 32 x 31 of 1024 x 1024 625, 603; 64 x 32 of 64 x 128 86.2, 79.0. The backward call of 8 x 64 of 64 x 128 (4.2e6) 41.0, 39.4.
+// The terms take 6 bytes of workspace a float: as much again as all other buffers of a backward call. At most 8 GiB of them, a twentieth of the memory, and 1 GiB
+// for callers that recompute hid to save memory. Larger layers keep the FP32 products, which take three and a half times as long (a backward call, ms: 8 experts x
+// 20000 rows of 1024 x 2048, 5.9 GB, by terms 15.1, by multiply-adds 53.3; 16 x 10000 of 1024 x 1024, 4.1 GB, 8.0 and 26.9).
 bool tc_float_supported(const moe_config &c, bool backward) {
-    const int64_t R = (int64_t)c.T * c.k;
+    const int64_t R = (int64_t)c.T * c.k, weights = (int64_t)c.n * c.d * c.h, most = c.flags & MOE_FLAG_RECOMPUTE_HID ? (int64_t)1 << 30 : (int64_t)8 << 30;
     if (c.act != MOE_F32 || c.d % 64 != 0 || c.h % 64 != 0) return false;
-    if ((int64_t)c.n * c.d * c.h >= (int64_t)1 << 32 || R * (c.d > c.h ? c.d : c.h) >= (int64_t)1 << 32) return false;  // quads are numbered with 31 bits
+    if (6 * (backward ? 2 * (R * ((int64_t)c.d + c.h) + weights) : R * c.h + weights) > most) return false;  // (quads are numbered with 31 bits: far below)
     return R >= (backward ? 28 : 32) * (int64_t)c.n && (double)R * c.d * c.h >= (backward ? 4.0e6 : 1.0e8);
 }
 
