@@ -23,13 +23,11 @@ constexpr int FEW_ROWS = 16, FEW_THREADS = 128, FEW_WARPS = FEW_THREADS / 32;
 struct FewRows {
     const float *A, *W;
     float *C;
-    const float *bias, *mask;
+    const float *bias, *mask;  // of rows; of transposed products
     int32_t N, K, nseg;
     int64_t w_e;
     const int32_t *offsets, *prefix;
 };
-
-__device__ __forceinline__ float few_epilogue(float v, float bias, float mask) { return mask > 0.0f ? v + bias : 0.0f; }
 
 // A tile: the rows of a segment from row0 on, by the least of 4, 8 and 16 that holds them
 struct FewTile { int32_t e, row0, rows; };
@@ -118,9 +116,7 @@ template <int LC, int WARPS> __global__ void __launch_bounds__(32 * WARPS, WARPS
             }
             const int64_t at = (int64_t)(t.row0 + r) * p.N + c;
             const float4 b = p.bias ? *reinterpret_cast<const float4 *>(p.bias + (int64_t)t.e * p.N + c) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            const float4 m = p.mask ? *reinterpret_cast<const float4 *>(p.mask + at) : make_float4(1.0f, 1.0f, 1.0f, 1.0f);
-            *reinterpret_cast<float4 *>(p.C + at) =
-                make_float4(few_epilogue(s.x, b.x, m.x), few_epilogue(s.y, b.y, m.y), few_epilogue(s.z, b.z, m.z), few_epilogue(s.w, b.w, m.w));
+            *reinterpret_cast<float4 *>(p.C + at) = make_float4(s.x + b.x, s.y + b.y, s.z + b.z, s.w + b.w);
         }
     });
 }
@@ -173,7 +169,7 @@ template <int LK, int KS> __global__ void __launch_bounds__(FEW_THREADS, 4) few_
                 const int r = f / NB, n = first + f % NB;
                 if (r >= t.rows || n >= p.N) return;
                 const int64_t at = (int64_t)(t.row0 + r) * p.N + n;
-                p.C[at] = few_epilogue(v, p.bias ? p.bias[(int64_t)t.e * p.N + n] : 0.0f, p.mask ? p.mask[at] : 1.0f);
+                p.C[at] = !p.mask || p.mask[at] > 0.0f ? v : 0.0f;
             };
             if constexpr (KS == 1) {
 #pragma unroll
@@ -195,76 +191,101 @@ template <int LK, int KS> __global__ void __launch_bounds__(FEW_THREADS, 4) few_
     });
 }
 
-// C[e] [M, N]: a thread takes sixteen rows and four columns of the gradient; LC lanes along a row
+// C[e] [M, N]: 8 TM x 64 outputs a block, TM rows and four columns a thread; sixteen rows of the segment in shared memory and the next ones on their way. A
+// block goes through its whole segment, so that where loads are uneven the longest one is the launch's time: a row of it takes 32 ns with TM = 4, 51 with 8 and 94 with 16
+// and nothing on the way meanwhile, and 31 in gemm_simt.cu. With blocks enough for all SMs all along TM = 8 reads less of shared memory (see launch_float_expert_product).
+// A backward call, us, by the float product and this way: 126 experts, 4410 rows, the longest segment 1399, of 64 x 64 112, 83; 416, 6656, 684, 64 x 128 127,
+// 103 (TM = 16: 175); 377, 25259, 2655, 704 x 448 2317, 1413; 416 x 1 row of 832 x 512 1456, 520
 struct FewGradients {
     const float *A, *B;
     float *C;
     int32_t M, N, nseg, tiles_n;
     const int32_t *offsets;
 };
-template <int LC> __global__ void __launch_bounds__(FEW_THREADS, 4) few_gradients_kernel(const FewGradients p) {
-    constexpr int G = 32 / LC, BM = FEW_WARPS * G * 16, CW = 4 * LC;
+constexpr int GRAD_N = 64;
+constexpr int grad_rows(int tm) { return FEW_WARPS * 2 * tm; }  // of a block
+template <int TM> __global__ void __launch_bounds__(FEW_THREADS, TM == 4 ? 8 : 6) few_gradients_kernel(const FewGradients p) {
+    constexpr int LC = GRAD_N / 4, G = 32 / LC, S = 2, GRAD_M = grad_rows(TM);
     wait_previous_kernel();
-    __shared__ __align__(16) float as[FEW_ROWS][BM], bs[FEW_ROWS][CW];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, e = blockIdx.y, m_at = blockIdx.x / p.tiles_n * BM, n_at = blockIdx.x % p.tiles_n * CW;
-    const int begin = p.offsets[e], end = p.offsets[e + 1];
-    const int row = (warp * G + lane / LC) * 16, col = lane % LC * 4;
-    float acc[16][4];
-#pragma unroll
-    for (int i = 0; i < 16; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0f;
-    for (int r0 = begin; r0 < end; r0 += FEW_ROWS) {
-        const int rows = min(FEW_ROWS, end - r0);
-        if (r0 > begin) __syncthreads();
-        for (int id = tid; id < rows * (BM / 4); id += FEW_THREADS) {
-            const int r = id / (BM / 4), m = id % (BM / 4) * 4;
+    __shared__ __align__(16) float as[S][FEW_ROWS][GRAD_M], bs[S][FEW_ROWS][GRAD_N];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, e = blockIdx.y, m_at = blockIdx.x / p.tiles_n * GRAD_M, n_at = blockIdx.x % p.tiles_n * GRAD_N;
+    const int begin = p.offsets[e], end = p.offsets[e + 1], blocks = (end - begin + FEW_ROWS - 1) / FEW_ROWS;
+    const int row = (warp * G + lane / LC) * TM, col = lane % LC * 4;
+    auto load = [&](int block, int s) {
+        const int r0 = begin + block * FEW_ROWS, rows = min(FEW_ROWS, end - r0);
+        for (int id = tid; id < rows * (GRAD_M / 4); id += FEW_THREADS) {
+            const int r = id / (GRAD_M / 4), m = id % (GRAD_M / 4) * 4;
             const bool live = m_at + m < p.M;
-            copy16(&as[r][m], live ? p.A + (int64_t)(r0 + r) * p.M + m_at + m : p.A, live);
+            copy16(&as[s][r][m], live ? p.A + (int64_t)(r0 + r) * p.M + m_at + m : p.A, live);
         }
         for (int id = tid; id < rows * LC; id += FEW_THREADS) {
             const int r = id / LC, n = id % LC * 4;
             const bool live = n_at + n < p.N;
-            copy16(&bs[r][n], live ? p.B + (int64_t)(r0 + r) * p.N + n_at + n : p.B, live);
+            copy16(&bs[s][r][n], live ? p.B + (int64_t)(r0 + r) * p.N + n_at + n : p.B, live);
         }
-        copies_commit();
-        copies_wait<0>();
-        __syncthreads();
-#pragma unroll 2
-        for (int r = 0; r < rows; ++r) {
-            const float4 b = *reinterpret_cast<const float4 *>(&bs[r][col]);
+    };
+    float acc[TM][4];
 #pragma unroll
-            for (int i = 0; i < 16; i += 4) {
-                const float4 a = *reinterpret_cast<const float4 *>(&as[r][row + i]);
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0f;
+#pragma unroll
+    for (int s = 0; s < S - 1; ++s) {
+        if (s < blocks) load(s, s);
+        copies_commit();
+    }
+    int s = 0;
+    for (int block = 0; block < blocks; ++block) {
+        copies_wait<S - 2>();
+        __syncthreads();  // this block is there for all, the one before is read by all
+        if (block + S - 1 < blocks) load(block + S - 1, s == 0 ? S - 1 : s - 1);
+        copies_commit();
+        const int rows = min(FEW_ROWS, end - begin - block * FEW_ROWS);
+#pragma unroll 4
+        for (int r = 0; r < rows; ++r) {
+            const float4 b = *reinterpret_cast<const float4 *>(&bs[s][r][col]);
+#pragma unroll
+            for (int i = 0; i < TM; i += 4) {
+                const float4 a = *reinterpret_cast<const float4 *>(&as[s][r][row + i]);
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    const float s = reinterpret_cast<const float *>(&a)[u];
-                    fma_two(acc[i + u][0], acc[i + u][1], s, b.x, b.y);
-                    fma_two(acc[i + u][2], acc[i + u][3], s, b.z, b.w);
+                    const float v = reinterpret_cast<const float *>(&a)[u];
+                    fma_two(acc[i + u][0], acc[i + u][1], v, b.x, b.y);
+                    fma_two(acc[i + u][2], acc[i + u][3], v, b.z, b.w);
                 }
             }
         }
+        if (++s == S) s = 0;
     }
     if (n_at + col >= p.N) return;
     float *c = p.C + ((int64_t)e * p.M + m_at + row) * p.N + n_at + col;
 #pragma unroll
-    for (int i = 0; i < 16; ++i)
+    for (int i = 0; i < TM; ++i)
         if (m_at + row + i < p.M) *reinterpret_cast<float4 *>(c + (int64_t)i * p.N) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
 }
 
-// Up to as many rows an expert as this way is the faster one. us, products of 64 experts of 200 x 520, by the float product and this way, rows an expert:
-//   rows         16 34.6, 24.4;  32 36.8, 36.0;  48 54.4, 38.0;  64 68.7, 54.1;  128 89, 83, and 50.5, 51.3 at 64 and 75, 86 at 128 into the wider side
-//   transposed   16 31.3 + 35.5, 22.5 + 22.5;  32 37.7 + 37.0, 36.0 + 31.4;  48 37.0 + 53.0, 49.4 + 43.1;  64 52.9 + 68.5, 63.0 + 54.0
-//   gradients    16 39.0 + 35.6, 13.5 + 14.4;  64 55.9 + 57.6, 36.7 + 40.6;  128 72.8 + 76.7, 66.1 + 72.3;  256 122 + 125, 128 + 141
-// Gradients of many rows need blocks besides: 8 experts of 64 x 128 with 32 rows, 16 blocks, 4.6 + 4.4, this way 5.7 + 5.8.
+int64_t grad_blocks(const SimtGemm &g) { return cdiv(g.M, grad_rows(4)) * cdiv(g.N, GRAD_N); }  // of an expert
+
+// Where this way is the faster one, by the rows an expert has on average: read off both ways' times of 780 products each (1 to 10000 rows an expert, widths of 8 to 4096,
+// equal and Zipf loads). Of the times that the rule takes, geometric means and the worst against the float product's: rows 0.62 and 1.21, transposed
+// 0.56 and 1.35, gradients 0.53 and 1.27. us, by the float product and this way:
+//   rows         64 experts of 200 x 520, 16 rows 34.6, 24.4;  48 54.4, 38.0;  but 120 x 60 of 1728 x 960 580, 818;  47 x 61 of 3136 x 1344 612, 792;
+//                narrow results of many experts: 209 x 16 of 384 x 64 19.6, 22.4;  432 x 51 of 64 x 64 14.6, 27.7;  short contractions: 134 x 31 of 64 x 1408 105, 119 (a forward call)
+//   transposed   64 of 200 x 520, 16 31.3 + 35.5, 22.5 + 22.5;  32 37.7 + 37.0, 36.0 + 31.4;  48 37.0 + 53.0, 49.4 + 43.1
+//   gradients    more than 32 rows an expert want four blocks and more an expert, or eight a SM in all: 126 x 35, the longest 1399, of 64 x 64 43, 53;
+//                one block an expert 16: 59 x 26 of 28 x 24, the longest 257, 34.8, 40.8 (a backward call)
 bool few_rows_take(const SimtGemm &g, const SegmentPlan &plan, int64_t R) {
     const bool grad = g.mode == 1;
     if (g.N % 4 != 0 || g.K % 4 != 0 || g.M % (grad ? 4 : 1) != 0 || !aligned16(g.A) || !aligned16(g.B) || !aligned16(g.C)) return false;
     if ((g.bias && !aligned16(g.bias)) || (g.mask && !aligned16(g.mask)) || g.nseg > 65535 || cdiv(g.N, 8) > 65535) return false;
-    if (g.relu || (!grad && !plan.prefix_of(FEW_ROWS))) return false;
+    if (g.relu || (!grad && (!plan.prefix_of(FEW_ROWS) || (g.sb_j == 1 ? g.mask : g.bias)))) return false;
     const int64_t n = g.nseg;
-    if (grad) return R <= 16 * n || (R <= 128 * n && n * cdiv(g.M, 64) * cdiv(g.N, 128) >= 64);
-    return R <= (g.sb_j == 1 ? 64 : 32) * n;
+    if (grad) {
+        const int64_t blocks = grad_blocks(g);
+        return R <= (blocks > 1 ? 32 : 16) * n || (R <= 64 * n && blocks > 4) || (R <= 128 * n && n * blocks >= 8 * 148);
+    }
+    if (g.sb_j != 1) return R <= 32 * n;
+    return R <= 64 * n;
 }
 
 template <int LC, int WARPS> int32_t launch_rows(const FewRows &p, int64_t tiles, cudaStream_t st) {
@@ -277,21 +298,21 @@ template <int LK, int KS> int32_t launch_transposed(const FewRows &p, int64_t ti
     MOE_LAUNCHED();
     return MOE_OK;
 }
-template <int LC> int32_t launch_gradients(FewGradients p, cudaStream_t st) {
-    constexpr int BM = FEW_WARPS * (32 / LC) * 16;
-    p.tiles_n = (int32_t)cdiv(p.N, 4 * LC);
-    launch_kernel(few_gradients_kernel<LC>, dim3((unsigned)(cdiv(p.M, BM) * p.tiles_n), (unsigned)p.nseg), FEW_THREADS, 0, st, p);
+template <int TM> int32_t launch_gradients(FewGradients p, cudaStream_t st) {
+    p.tiles_n = (int32_t)cdiv(p.N, GRAD_N);
+    launch_kernel(few_gradients_kernel<TM>, dim3((unsigned)(cdiv(p.M, grad_rows(TM)) * p.tiles_n), (unsigned)p.nseg), FEW_THREADS, 0, st, p);
     MOE_LAUNCHED();
     return MOE_OK;
 }
-
 }  // namespace
 
 int32_t launch_float_expert_product(const SimtGemm &g, const SegmentPlan &plan, int64_t R, cudaStream_t st) {
     if (R == 0 || !few_rows_take(g, plan, R)) return launch_simt_gemm(g, nullptr, st, nullptr, &plan);
     if (g.mode == 1) {
         FewGradients p = {(const float *)g.A, (const float *)g.B, (float *)g.C, (int32_t)g.M, (int32_t)g.N, g.nseg, 0, g.offsets};
-        return g.N <= 64 ? launch_gradients<16>(p, st) : launch_gradients<32>(p, st);
+        // (416 x 1 row of 832 x 512, 86528 blocks of TM = 4: a backward call 576, with TM = 8 520; 128 x 24 of 512 x 1024, 32768, 573, 535; 416 x 16 of
+        // 64 x 128, the longest 684, 3328 blocks: 103, 135)
+        return g.nseg * grad_blocks(g) >= 64 * 148 ? launch_gradients<8>(p, st) : launch_gradients<4>(p, st);
     }
     const FewRows p = {(const float *)g.A, (const float *)g.B, (float *)g.C, (const float *)g.bias, (const float *)g.mask, (int32_t)g.N, (int32_t)g.K, g.nseg, g.b_e,
                        g.offsets, plan.prefix_of(FEW_ROWS)};

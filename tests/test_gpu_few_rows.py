@@ -48,3 +48,14 @@ def test_values_that_are_no_numbers():
         for i in (1, 2, 3, 5):  # (hid: the larger of NaN and 0 is 0)
             got, exp = results[i]
             assert torch.equal(got.isnan(), exp.isnan()) and torch.equal(got.isinf(), exp.isinf()), (e, i)
+
+
+# a few long segments among short ones: blocks of sixteen rows and remainders in turn through both buffers; few blocks, and enough for the larger tiles
+@pytest.mark.parametrize("counts,d,h", [([1403] + [2, 0, 5] * 40, 64, 64), ([0, 33, 16, 48, 1, 49, 700] + [4] * 40, 96, 136), ([17, 260, 32] + [1] * 140, 392, 520),
+                                        ([65, 64, 63, 80], 72, 328), ([90] * 3 + [200], 28, 24)])
+def test_uneven_loads(counts, d, h):
+    for e, results in run(counts, d, h, d + h):
+        for i, (got, exp) in enumerate(results):
+            if exp.numel():
+                err = ((got.double() - exp).abs() / (exp.abs() + exp.square().mean().sqrt() + 1e-30)).max()
+                assert err <= 1e-5, (e, counts[e], i, float(err))  # the tolerance of the float layer
