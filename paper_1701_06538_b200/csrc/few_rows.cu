@@ -285,7 +285,8 @@ bool few_rows_take(const SimtGemm &g, const SegmentPlan &plan, int64_t R) {
         return R <= (blocks > 1 ? 32 : 16) * n || (R <= 64 * n && blocks > 4) || (R <= 128 * n && n * blocks >= 8 * 148);
     }
     if (g.sb_j != 1) return R <= 32 * n;
-    return R <= 64 * n;
+    const bool wide = g.N > 64 || n < 100;
+    return R <= (wide ? 16 : 8) * n || (wide && g.K > 64 && R <= (n * g.K * g.N < 5000000 ? 64 : 32) * n);
 }
 
 template <int LC, int WARPS> int32_t launch_rows(const FewRows &p, int64_t tiles, cudaStream_t st) {
