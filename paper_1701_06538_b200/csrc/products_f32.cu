@@ -575,11 +575,16 @@ struct FloatCall {
 
 }  // namespace
 
-// A call has to make the terms of the weights (10 bytes of traffic a float): forward, one product, from 32 rows an expert and 1e8 multiply-adds a product
-// on, backward, four products, from 28 and 4e6. us, by FP32 multiply-adds (few_rows.cu up to 64 rows) and this way. A forward call: 32 experts x 64
-// rows of 1024 x 1024 365, 318; 32 x 32 277, 278; 16 x 64 of 256 x 512 (1.3e8) 54.2, 56.0; 16 x 100 75.0, 68.8; 64 x 40 of 512 x 512 167, 163.
-// A step: 64 experts x 24 rows of 256 x 512 198, 203; x 32 237, 223; x 48 283, 231; 300 x 24 931, 934; 8 x 25 of 512 x 4096 339, 393;
-// 32 x 31 of 1024 x 1024 625, 603; 64 x 32 of 64 x 128 86.2, 79.0. The backward call of 8 x 64 of 64 x 128 (4.2e6) 41.0, 39.4.
+// A call has to make the terms (4 bytes of a float read, 6 written). Where they pay, us, by FP32 multiply-adds (few_rows.cu among them) and this way:
+// A forward call, one product: from 65 rows an expert, 1e8 multiply-adds and 16 tiles on. 256 experts x 64 rows of 256 x 512 216, 225, x 72 329, 284;
+// 32 x 40 of 256 x 512 47.1, 51.9; 16 x 50 34.3, 37.7, x 100 56.6, 48.9; 64 x 72 of 512 x 512 195, 157; 120 x 60 of 960 x 1728 1134, 1168, x 70 1674, 1420;
+// 8 x 1500 of 64 x 128 (9.8e7) 25.6, 23.8; 2 x 136 of 192 x 3072, 8 tiles, 82.7, 86.3; 6 x 144 of 64 x 2496, 10 tiles, 68.3, 72.6; 2 x 500 of 256 x 512, 18, 34.4, 33.6.
+// A backward call, four products: from 33 rows and 4e6 on. 64 x 32 of 256 x 512 105, 95, x 40 146, 100; 300 x 30 434, 390, x 40 497, 417; 8 x 30 of 512 x 4096 182,
+// 222, x 40 294, 216; 200 x 30 of 64 x 128 40.9, 45.9; 72 x 31 27.3, 29.3, x 40 39.7, 29.9; 400 x 40 of 64 x 64 57.5, 63.6. Small ones, by multiply-adds in
+// 1e6: 2.1 (4 x 64 of 64 x 128) 25.9, 26.9; 4.2 (16 x 64 of 64 x 64, 8 x 128 of 64 x 64) 25.8, 25.3 and 28.5, 27.5; 4.7 (8 x 36 of 64 x 256) 26.0, 28.8;
+// 6.3 (16 x 48 of 64 x 128) 30.3, 27.7; 8.4 (8 x 64 of 128 x 128) 27.9, 28.5, (16 x 64 of 64 x 128) 30.2, 27.6. A few tiles that are chains of many rows are the
+// exception: 1 x 20000 of 128 x 128 673, 820; 2 x 5000 205, 222; 4 x 5000 of 64 x 64 193, 228; 1 x 981 55.9, 60.9; but 1 x 512 40.4, 38.9; 1 x 3000 of 512 x 128
+// 160, 143; 19 x 2000 of 64 x 64 144, 131.
 // The terms take 6 bytes of workspace a float: as much again as all other buffers of a backward call. At most 8 GiB of them, a twentieth of the memory, and 1 GiB
 // for callers that recompute hid to save memory. Larger layers keep the FP32 products, which take three and a half times as long (a backward call, ms: 8 experts x
 // 20000 rows of 1024 x 2048, 5.9 GB, by terms 15.1, by multiply-adds 53.3; 16 x 10000 of 1024 x 1024, 4.1 GB, 8.0 and 26.9).
@@ -587,7 +592,10 @@ bool tc_float_supported(const moe_config &c, bool backward) {
     const int64_t R = (int64_t)c.T * c.k, weights = (int64_t)c.n * c.d * c.h, most = c.flags & MOE_FLAG_RECOMPUTE_HID ? (int64_t)1 << 30 : (int64_t)8 << 30;
     if (c.act != MOE_F32 || c.d % 64 != 0 || c.h % 64 != 0) return false;
     if (6 * (backward ? 2 * (R * ((int64_t)c.d + c.h) + weights) : R * c.h + weights) > most) return false;  // (quads are numbered with 31 bits: far below)
-    return R >= (backward ? 28 : 32) * (int64_t)c.n && (double)R * c.d * c.h >= (backward ? 4.0e6 : 1.0e8);
+    const double work = (double)R * c.d * c.h;
+    if (!backward) return R > 64 * (int64_t)c.n && work >= 1.0e8 && (cdiv(R, F_TILE) + c.n / 2) * cdiv(c.d, F_TILE) >= 16;
+    if (weights < 16 * 64 * 64 && R >= 700 * (int64_t)c.n) return false;
+    return R > 32 * (int64_t)c.n && work >= 4.0e6;
 }
 
 int32_t launch_float_ys(const moe_config &c, const int32_t *offsets, const void *hid, const void *W2, const void *b2, void *ys, const SegmentPlan &plan,
