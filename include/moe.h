@@ -266,7 +266,9 @@ int32_t moe_combine_bwd(const moe_config *cfg, const void *dY, const void *ys, c
 /* Back-propagation through the experts (ReLU derivative 0 at 0):
  *   db2 = sum dys, dW2 = hid^T.dys, dz = (dys.W2^T) * [hid > 0] (rounded to act), db1 = sum dz,
  *   dW1 = xs^T.dz, dxs = dz.W1^T; experts with no rows get zero gradients.
- * out: dxs [R,d], dW1 [n,d,h], db1 [n,h], dW2 [n,h,d], db2 [n,d] (all act); dz lives in ws. */
+ * out: dxs [R,d], dW1 [n,d,h], db1 [n,h], dW2 [n,h,d], db2 [n,d] (all act); dz lives in ws.
+ * dxs may be xs itself (dW1 is then formed first, in a launch of its own). Beside that and the arguments that are marked
+ * in-out, nothing is promised, here or in the other calls, for outputs that share memory with inputs. */
 int32_t moe_expert_ffn_bwd(const moe_config *cfg, const void *xs, const void *hid, const void *dys,
                            const int32_t *offsets, const void *W1, const void *W2, void *dxs, void *dW1,
                            void *db1, void *dW2, void *db2, void *ws, void *stream);

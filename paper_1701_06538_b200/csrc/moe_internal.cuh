@@ -89,6 +89,11 @@ static inline size_t act_bytes(int32_t act) { return act == MOE_BF16 ? 2 : 4; }
 static inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 static inline int64_t imin(int64_t a, int64_t b) { return a < b ? a : b; }
 static inline int64_t imax(int64_t a, int64_t b) { return a > b ? a : b; }
+// whether two buffers share memory
+static inline bool overlap(const void *a, int64_t a_bytes, const void *b, int64_t b_bytes) {
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return x < y + (uintptr_t)b_bytes && y < x + (uintptr_t)a_bytes;
+}
 static inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 31) == 0; }  // 32 bytes: the epilogues use 256-bit stores
 
 // In the place of work that rides along with a launch, where none does: the parameters and registers of the work cost the launch's own
@@ -224,7 +229,7 @@ int32_t launch_tile_prefix(const int32_t *offsets, int32_t n, int32_t bm, int32_
 
 // ----------------------------------------------------------------------------- per-call segment plan (plan.cu)
 constexpr int PLAN_HEIGHTS = 4, PLAN_COUNTERS = 8, PLAN_MAX_SORTED = 2048;
-enum PlanCounter { PLAN_HID = 0, PLAN_YS, PLAN_DZ_DW2, PLAN_DW1_DXS };  // the tiles drawn so far, by launch of expert products
+enum PlanCounter { PLAN_HID = 0, PLAN_YS, PLAN_DZ_DW2, PLAN_DW1_DXS, PLAN_DXS };  // the tiles drawn so far, by launch of expert products
 // Tensor maps of a call's expert products whose rows end with a segment, one per segment: what lies behind a segment's last row reads
 // as zero, whatever follows it in memory. ROWS: K-major operand of a row product, COLS: operand of a weight gradient
 // (contraction over the rows).

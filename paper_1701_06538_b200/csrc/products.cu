@@ -789,7 +789,7 @@ class ProductList {
     const int64_t R;
     const bool pairs, row_maps, wgrad_maps;
     const int tm;
-    int64_t tiles = 0;
+    int64_t tiles = 0, product_tiles[MAX_PRODUCTS];
     int count = 0;
     int32_t *drawn;
     ProductMaps maps;
@@ -846,6 +846,12 @@ class ProductList {
         add((int64_t)c.n * p.per_e);
         return MOE_OK;
     }
+    // of two products that were added the one: the other one has no tiles
+    void only(int which) {
+        Product &other = P.p[1 - which];
+        tiles = product_tiles[which];
+        other.tiles_n = other.per_e = 0;
+    }
     template <int SET> int32_t launch(cudaStream_t st) {
         if (tiles >= ((int64_t)1 << 31) - ((int64_t)1 << 22)) return MOE_ERR_UNSUPPORTED;
         // Pairs draw their tiles. Single CTAs do with many tiles each (4096 experts x 64 rows, 166 and more a CTA: a step 6550 us, dealt
@@ -870,7 +876,7 @@ class ProductList {
   private:
     void add(int64_t n) {
         tiles += n;
-        ++count;
+        product_tiles[count++] = n;
     }
 };
 
@@ -959,9 +965,22 @@ int32_t launch_tc_ffn_bwd(const moe_config &c, const void *xs, const void *hid, 
     MOE_TRY(by_w2.wgrad(hid, dys, c.h, c.d, dW2, MAP_HID_COLS, MAP_DYS_COLS));
     if (relu_bits) MOE_TRY(by_w2.launch<SET_DZ_DW2>(st));
     else MOE_TRY(by_w2.launch<SET_DZ_DW2_MASK>(st));
-    MOE_TRY(by_w1.wgrad(xs, dz, c.d, c.h, dW1, MAP_XS_COLS, MAP_DZ_COLS));
-    MOE_TRY(by_w1.row(&p, dz, W1, true, c.d, c.h, dxs, MAP_DZ_ROWS));
-    MOE_TRY(by_w1.launch<SET_DW1_DXS>(st));
+    auto by_w1_products = [&](ProductList &list) -> int32_t {
+        MOE_TRY(list.wgrad(xs, dz, c.d, c.h, dW1, MAP_XS_COLS, MAP_DZ_COLS));
+        return list.row(&p, dz, W1, true, c.d, c.h, dxs, MAP_DZ_ROWS);
+    };
+    MOE_TRY(by_w1_products(by_w1));
+    const int64_t xs_bytes = R * c.d * (int64_t)sizeof(bf16);
+    if (overlap(xs, xs_bytes, dxs, xs_bytes)) {  // the caller has no use for xs any more: dxs waits until dW1 has read it
+        ProductList after(c, plan, offsets, PLAN_DXS, status_word);
+        MOE_TRY(by_w1_products(after));
+        by_w1.only(0);
+        after.only(1);
+        MOE_TRY(by_w1.launch<SET_DW1_DXS>(st));
+        MOE_TRY(after.launch<SET_DW1_DXS>(st));
+    } else {
+        MOE_TRY(by_w1.launch<SET_DW1_DXS>(st));
+    }
     const BlockSums sums = {colsum, plan.prefix[0], offsets, (bf16 *)db1, c.n, c.h, tc_row_tile(c) / 32, tc_row_tile(c)};
     if (c.n >= 128 && R <= 128 * (int64_t)c.n) {
         launch_kernel(colsum_blocks_final_kernel<1024>, dim3((unsigned)c.n, (unsigned)cdiv(c.h, 1024)), 256, 0, st, sums);

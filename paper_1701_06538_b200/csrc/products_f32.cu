@@ -628,6 +628,14 @@ int32_t launch_float_ffn_bwd(const moe_config &c, const void *xs, const void *hi
     FloatLaunch<ROW_BK, FE_PLAIN, true> by_w1;
     MOE_TRY(call.wgrad(&by_w1, xs, t.xs, dz, t.dz, c.d, c.h, dW1));
     MOE_TRY(call.row(&by_w1, dz, t.dz, W1, t.W1, c.d, c.h, dxs, nullptr, nullptr, nullptr));
+    const int64_t xs_bytes = call.R * c.d * (int64_t)sizeof(float);
+    if (overlap(xs, xs_bytes, dxs, xs_bytes)) {  // the caller has no use for xs any more: dxs waits until dW1 has read it (elements that are not finite do)
+        const int32_t rows = by_w1.row.total;
+        by_w1.row.total = 0;
+        MOE_TRY(call.launch(by_w1));
+        by_w1.row.total = rows;
+        by_w1.wgrad.total = 0;
+    }
     return call.launch(by_w1);
 }
 
