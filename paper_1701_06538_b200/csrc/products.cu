@@ -52,7 +52,7 @@ constexpr Kind set_kind(int set, int i) {
     return set == SET_HID || set == SET_YS ? ROW_BMN : (set == SET_DW1_DXS) == (i == 0) ? WGRAD : ROW_BK;
 }
 // Registers a thread: as few as do without spills, so that a launch's blocks find room beside the last ones of the launch before
-constexpr int most_registers(int set) { return set == SET_HID || set == SET_YS ? 128 : 112; }
+constexpr int most_registers(int set, bool whole) { return !whole ? 168 : set == SET_HID || set == SET_YS ? 128 : 112; }
 constexpr Epilogue set_epilogue(int set, int i) {
     if (set == SET_HID) return EPI_BIAS_RELU;
     if (set == SET_YS) return EPI_BIAS;
@@ -193,31 +193,22 @@ __device__ __forceinline__ void keep_from_mask(const Product &p, int64_t row0, i
 // work (with 32-column steps the epilogue of a 256 x 256 tile took 8500 cycles, against 4900 of tensor work at K = 512).
 // Whole boxes leave as bulk tensor stores through one of the warp's 4 KiB pieces of shared memory (rows of 128 bytes, 16-byte pieces
 // swizzled by row); boxes cut by a segment end as guarded row stores.
-// release() hands the accumulator back; it is called once the box is in registers.
 struct BoxArgs {
     const CUtensorMap *tm_out;
     uint8_t *box;
-    uint32_t taddr;             // tensor-memory address of the box
     int64_t out_off, row0;      // output row of lane 0 is row0 of the matrix that starts at element out_off
     int32_t rows_valid, col0;
     int32_t map_row;            // the same row in the output's tensor map
     int64_t colsum_row;
     const bf16 *next_bias;      // of the warp's next box, or nullptr
     uint2 keep;                 // mask bits
-    bool have_acc;
 };
-template <int EPI, int BOXES, bool WHOLE, typename Release>
-__device__ __forceinline__ void epilogue_box(const Product &p, int lane, const BoxArgs &b, uint4 (&bias)[2][4], Release release) {
-    uint32_t v[2][32];
-    if (b.have_acc) {
-        tc_ld_32x32(b.taddr, v[0]);
-        tc_ld_32x32(b.taddr + 32, v[1]);
-        tc_ld_wait();
-        release();
-    } else {
-#pragma unroll
-        for (int j = 0; j < 64; ++j) v[j >> 5][j & 31] = 0u;
-    }
+__device__ __forceinline__ void load_box(uint32_t taddr, uint32_t (&v)[2][32]) {
+    tc_ld_32x32(taddr, v[0]);
+    tc_ld_32x32(taddr + 32, v[1]);
+    tc_ld_wait();
+}
+template <int EPI, int BOXES, bool WHOLE> __device__ __forceinline__ void epilogue_box(const Product &p, int lane, const BoxArgs &b, uint4 (&bias)[2][4], const uint32_t (&v)[2][32]) {
     const bool row_ok = lane < b.rows_valid, staged = b.rows_valid >= 32;
     const int64_t out_row = b.row0 + lane;
     uint8_t *mine = b.box + lane * 128;
@@ -383,6 +374,13 @@ template <bool PAIR, bool SHORT, int SET> struct TileRing {
     }
 };
 
+// Weight gradients of other widths than multiples of 64 are summed in tensor memory over 8 K blocks, 512 rows, and these sums added in registers: a tensor
+// core's accumulator drops low bits at every step of 16, over many rows more than the rounding of the result hides. Error of dW1 and dW2 against 64 bits (2-norms), as
+// sums of multiply-adds, in one accumulator and this way, in 1e-3: 60000 rows of 264 x 136 1.651 and 1.589, 1.653 and 1.596, 1.651 and 1.589; 400000 of 72 x 40 1.563
+// and 1.645, 1.705 and 1.947, 1.563 and 1.645. Tiles are 128 columns wide for it, a box a warp: a backward call of 4 experts x 15000 rows of 200 x 136 301 us, 226 this way;
+// 64 x 200 of 72 x 2056 108, 110; but 8 x 3750 of 1000 x 2008 609, 710 (by multiply-adds 9740).
+constexpr int SUM_BLOCKS = 8;
+
 // PAIR: the two CTAs' shares of a tile
 template <bool PAIR> constexpr int tile_rows() { return PAIR ? 256 : 128; }
 template <bool PAIR> constexpr int stage_bytes() { return A_BYTES + (PAIR ? 128 : BN) * BK * 2; }
@@ -393,7 +391,7 @@ template <bool PAIR, int NST> constexpr int shared_bytes() { return data_bytes<P
 // WHOLE: all widths are multiples of 64. Otherwise of eight, and one CTA: MN-major operands come in chunk by chunk through maps of the whole width, what lies
 // behind it reads as zero and is not stored.
 template <bool PAIR, int NST, int SET, bool WHOLE>
-__global__ void __maxnreg__(most_registers(SET)) expert_products_kernel(const __grid_constant__ ProductMaps maps, const __grid_constant__ Products P) {
+__global__ void __maxnreg__(most_registers(SET, WHOLE)) expert_products_kernel(const __grid_constant__ ProductMaps maps, const __grid_constant__ Products P) {
     constexpr bool SHORT = !PAIR && NST == 3;
     constexpr int RING = ring_slots<SHORT>(), BOXES = box_count<PAIR, NST>(), STAGE = stage_bytes<PAIR>(), TM = tile_rows<PAIR>();
     extern __shared__ uint8_t smem_raw[];
@@ -547,11 +545,15 @@ __global__ void __maxnreg__(most_registers(SET)) expert_products_kernel(const __
                 // K-major tile and by 16 rows of 128 bytes in an MN-major one; the sum never leaves the address field
                 constexpr uint64_t a_step = a_mn ? (16 * 128) >> 4 : 32 >> 4, b_step = b_mn ? (16 * 128) >> 4 : 32 >> 4;
                 const int tail = wgrad ? (t.row_end - t.row0) - (kblocks - 1) * BK : BK;  // rows of the last block
-                ok = mbar_wait(tempty_bar(acc), acc_ph ^ 1u, abort_flag, P.status);
-                if (!ok) return;
-                tc_fence_after();
-                const uint32_t d_tmem = tmem_base + acc * BN;
+                constexpr bool IN_PARTS = !WHOLE && wgrad;  // a sum of SUM_BLOCKS K blocks at a time
                 for (int kb = 0; kb < kblocks; ++kb) {
+                    const bool begins = IN_PARTS ? kb % SUM_BLOCKS == 0 : kb == 0;
+                    if (begins) {
+                        ok = mbar_wait(tempty_bar(acc), acc_ph ^ 1u, abort_flag, P.status);
+                        if (!ok) return;
+                        tc_fence_after();
+                    }
+                    const uint32_t d_tmem = tmem_base + acc * BN;
                     ok = mbar_wait(full_bar(s), ph, abort_flag, P.status);
                     if (!ok) break;
                     tc_fence_after();
@@ -577,21 +579,23 @@ __global__ void __maxnreg__(most_registers(SET)) expert_products_kernel(const __
 #pragma unroll
                         for (int k = 0; k < BK / 16; ++k) {
                             if (k >= ksteps) break;
-                            if (PAIR) tc_mma2_bf16(d_tmem, ad + k * a_step, bd + k * b_step, idesc, (kb > 0 || k > 0) ? 1u : 0u);
-                            else tc_mma_bf16(d_tmem, ad + k * a_step, bd + k * b_step, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+                            if (PAIR) tc_mma2_bf16(d_tmem, ad + k * a_step, bd + k * b_step, idesc, (!begins || k > 0) ? 1u : 0u);
+                            else tc_mma_bf16(d_tmem, ad + k * a_step, bd + k * b_step, idesc, (!begins || k > 0) ? 1u : 0u);
                         }
                         if (PAIR) tc_commit2(empty_bar(s));  // the stage may be refilled once these MMAs have read it
                         else tc_commit(empty_bar(s));
                     }
                     if (!PAIR) __syncwarp();
                     if (++s == NST) { s = 0; ph ^= 1u; }
+                    if (IN_PARTS ? kb % SUM_BLOCKS == SUM_BLOCKS - 1 || kb == kblocks - 1 : kb == kblocks - 1) {  // accumulator complete
+                        if (PAIR || lane == 0) {
+                            if (PAIR) tc_commit2(tfull_bar(acc));
+                            else tc_commit(tfull_bar(acc));
+                        }
+                        if (!PAIR) __syncwarp();
+                        if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
+                    }
                 }
-                if (ok && (PAIR || lane == 0)) {  // accumulator complete
-                    if (PAIR) tc_commit2(tfull_bar(acc));
-                    else tc_commit(tfull_bar(acc));
-                }
-                if (!PAIR) __syncwarp();
-                if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
               });
             }
         }
@@ -656,7 +660,6 @@ __global__ void __maxnreg__(most_registers(SET)) expert_products_kernel(const __
                 b.rows_valid = (wgrad ? p.M : t.row_end) - (int32_t)b.row0;
                 b.map_row = (int32_t)b.row0 + (wgrad ? t.e * p.M : 0);
                 b.colsum_row = PAIR ? (t.mt * 2 + (int)rank) * 4 + quarter : t.mt * 4 + quarter;
-                b.have_acc = have_acc;
                 uint4 bias[2][4];
                 const bf16 *bias_at = nullptr;
                 if (epi_bias(EPI)) {
@@ -666,11 +669,6 @@ __global__ void __maxnreg__(most_registers(SET)) expert_products_kernel(const __
                 uint2 keep[2] = {make_uint2(0u, 0u), make_uint2(0u, 0u)};
                 if (EPI == EPI_KEEP_BITS && lane < b.rows_valid) keep_load(p, b.row0 + lane, first, keep);
                 if (EPI == EPI_KEEP_MASK) keep_from_mask(p, b.row0, b.rows_valid, first, lane, boxes_at, keep);
-                if (have_acc) {  // (the loads above are in flight while the warp waits for its accumulator)
-                    ok = mbar_wait(tfull_bar(acc), acc_ph, abort_flag, P.status);
-                    if (!ok) return;
-                    tc_fence_after();
-                }
                 auto release = [&]() {  // the warp's part of the accumulator is in registers: the buffer goes back
                     tc_fence_before();
                     __syncwarp();
@@ -679,18 +677,54 @@ __global__ void __maxnreg__(most_registers(SET)) expert_products_kernel(const __
                         else mbar_arrive(tempty_bar(acc));
                     }
                 };
-                for (int u = 0; u < boxes; ++u) {
+                const uint32_t mine = tmem_base + ((uint32_t)(quarter * 32) << 16) + half * (p.tile_n / 2);
+                auto store = [&](int u, const uint32_t (&v)[2][32]) {
                     b.col0 = first + 64 * u;
-                    b.taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + half * (p.tile_n / 2) + 64 * u;
                     b.next_bias = epi_bias(EPI) && u + 1 < boxes ? bias_at + 64 : nullptr;
                     b.keep = u ? keep[1] : keep[0];
                     b.box = boxes_at + (BOXES > 1 ? turn * 4096 : 0);
                     if (b.rows_valid >= 32) turn ^= 1;  // (else nothing is stored from the box)
-                    epilogue_box<EPI, BOXES, WHOLE>(p, lane, b, bias, [&]() { if (u + 1 == boxes) release(); });
-                }
-                if (have_acc) {
-                    if (boxes == 0) release();
-                    if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
+                    epilogue_box<EPI, BOXES, WHOLE>(p, lane, b, bias, v);
+                };
+                if constexpr (!WHOLE && wgrad) {  // sums of SUM_BLOCKS K blocks, added in registers: a box a warp
+                    uint32_t v[2][32];
+                    float sum[2][32];
+#pragma unroll
+                    for (int j = 0; j < 64; ++j) sum[j >> 5][j & 31] = 0.0f;
+                    for (int r = t.row0; r < t.row_end; r += SUM_BLOCKS * BK) {
+                        ok = mbar_wait(tfull_bar(acc), acc_ph, abort_flag, P.status);
+                        if (!ok) return;
+                        tc_fence_after();
+                        load_box(mine + acc * BN, v);
+                        release();
+#pragma unroll
+                        for (int j = 0; j < 64; ++j) sum[j >> 5][j & 31] += __uint_as_float(v[j >> 5][j & 31]);
+                        if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
+                    }
+#pragma unroll
+                    for (int j = 0; j < 64; ++j) v[j >> 5][j & 31] = __float_as_uint(sum[j >> 5][j & 31]);
+                    if (boxes > 0) store(0, v);
+                } else {
+                    if (have_acc) {  // (the loads above are in flight while the warp waits for its accumulator)
+                        ok = mbar_wait(tfull_bar(acc), acc_ph, abort_flag, P.status);
+                        if (!ok) return;
+                        tc_fence_after();
+                    }
+                    for (int u = 0; u < boxes; ++u) {
+                        uint32_t v[2][32];
+                        if (have_acc) {
+                            load_box(mine + acc * BN + 64 * u, v);
+                            if (u + 1 == boxes) release();
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 64; ++j) v[j >> 5][j & 31] = 0u;
+                        }
+                        store(u, v);
+                    }
+                    if (have_acc) {
+                        if (boxes == 0) release();
+                        if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
+                    }
                 }
             });
         }
@@ -829,8 +863,8 @@ class ProductList {
     int32_t wgrad(const void *A, const void *B, int32_t M, int32_t N, void *out, SegmentMap seg_a, SegmentMap seg_b) {
         Product &p = P.p[count];
         p.N = N; p.M = M;
-        p.tile_n = BN;
-        p.tiles_n = (int32_t)cdiv(N, BN); p.per_e = (int32_t)cdiv(M, tm) * p.tiles_n;
+        p.tile_n = whole(c) ? BN : 128;  // (a box a warp, see SUM_BLOCKS)
+        p.tiles_n = (int32_t)cdiv(N, p.tile_n); p.per_e = (int32_t)cdiv(M, tm) * p.tiles_n;
         p.by_tiles_n = Divisor::of(p.tiles_n); p.by_per_e = Divisor::of(p.per_e);
         p.out = (bf16 *)out;
         if (wgrad_maps) { p.seg_a = plan.maps_of(seg_a); p.seg_b = plan.maps_of(seg_b); }
