@@ -43,7 +43,7 @@ void fill_plan(PlanArgs *a, const SegmentPlan &plan, int32_t n, int64_t R, int32
 }
 
 int32_t launch_segment_plan(const PlanArgs &a, const int32_t *offsets, cudaStream_t st) {
-    const size_t shared = plan_shared_ints(a.plan.sched ? a.n : 0) * sizeof(int32_t) + 128;  // at most 16 KiB: PLAN_MAX_SORTED
+    const size_t shared = plan_shared_ints(a.plan.sched ? a.n : 0) * sizeof(int32_t) + 128;  // at most 16 KiB: PLAN_MAX_SORTED keys
     launch_kernel(segment_plan_kernel, (unsigned)plan_blocks(a), 1024, shared, st, a, offsets);
     MOE_LAUNCHED();
     return MOE_OK;
