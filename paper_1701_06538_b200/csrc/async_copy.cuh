@@ -5,12 +5,22 @@
 
 namespace moe {
 
-__device__ __forceinline__ void copy16(void *to, const void *from, bool live) {  // else sixteen bytes of zeros (`from` is not read, but valid)
+__device__ __forceinline__ void copy16(void *to, const void *from) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(to)), "l"(from) : "memory");
+}
+__device__ __forceinline__ void copy4(void *to, const void *from) {  // the same with four bytes
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(to)), "l"(from) : "memory");
+}
+// else zeros (`from` is not read, but valid)
+__device__ __forceinline__ void copy16(void *to, const void *from, bool live) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(to)), "l"(from), "r"(live ? 16 : 0) : "memory");
 }
-__device__ __forceinline__ void copy4(void *to, const void *from, bool live) {  // the same with four bytes
+__device__ __forceinline__ void copy4(void *to, const void *from, bool live) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(to)), "l"(from), "r"(live ? 4 : 0) : "memory");
 }
+// zeros by a store: copies of zeros from one address go one by one
+__device__ __forceinline__ void zero16(void *to) { *reinterpret_cast<uint4 *>(to) = make_uint4(0u, 0u, 0u, 0u); }
+__device__ __forceinline__ void zero4(void *to) { *reinterpret_cast<uint32_t *>(to) = 0u; }
 __device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }  // all but the last N groups are there
 

@@ -215,13 +215,11 @@ template <int TM> __global__ void __launch_bounds__(FEW_THREADS, TM == 4 ? 8 : 6
         const int r0 = begin + block * FEW_ROWS, rows = min(FEW_ROWS, end - r0);
         for (int id = tid; id < rows * (GRAD_M / 4); id += FEW_THREADS) {
             const int r = id / (GRAD_M / 4), m = id % (GRAD_M / 4) * 4;
-            const bool live = m_at + m < p.M;
-            copy16(&as[s][r][m], live ? p.A + (int64_t)(r0 + r) * p.M + m_at + m : p.A, live);
+            if (m_at + m < p.M) copy16(&as[s][r][m], p.A + (int64_t)(r0 + r) * p.M + m_at + m);  // (what lies behind is computed from whatever is there and dropped)
         }
         for (int id = tid; id < rows * LC; id += FEW_THREADS) {
             const int r = id / LC, n = id % LC * 4;
-            const bool live = n_at + n < p.N;
-            copy16(&bs[s][r][n], live ? p.B + (int64_t)(r0 + r) * p.N + n_at + n : p.B, live);
+            if (n_at + n < p.N) copy16(&bs[s][r][n], p.B + (int64_t)(r0 + r) * p.N + n_at + n);
         }
     };
     float acc[TM][4];

@@ -148,7 +148,8 @@ template <int KIND, int EPI> __device__ __forceinline__ void repair_tile(const F
             const bool live_a = c < rows && k0 + k < depth;
             const float *a = !live_a ? p.A : TURN_A ? p.A + (t.row0 + c) * (int64_t)p.K + k0 + k : p.A + (int64_t)(t.row0 + k0 + k) * p.M + t.m0 + c;
             if (TURN_A) turned[0][q] = live_a ? *reinterpret_cast<const float4 *>(a) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            else copy16(as + k * R_PITCH + c, a, live_a);
+            else if (live_a) copy16(as + k * R_PITCH + c, a);
+            else zero16(as + k * R_PITCH + c);
             place(TURN_B, q, c, k);
             const bool live_b = c < cols && k0 + k < depth;
             const float *b = !live_b         ? p.B
@@ -156,7 +157,8 @@ template <int KIND, int EPI> __device__ __forceinline__ void repair_tile(const F
                              : TURN_B        ? p.B + ((int64_t)t.e * p.N + t.n0 + c) * p.K + k0 + k
                                              : p.B + ((int64_t)t.e * p.K + k0 + k) * p.N + t.n0 + c;
             if (TURN_B) turned[1][q] = live_b ? *reinterpret_cast<const float4 *>(b) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            else copy16(bs + k * R_PITCH + c, b, live_b);
+            else if (live_b) copy16(bs + k * R_PITCH + c, b);
+            else zero16(bs + k * R_PITCH + c);
         }
         copies_commit();
     };

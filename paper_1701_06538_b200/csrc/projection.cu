@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(ProjectionTile<T, BM, BN, TM, TN, BK, S>::NT, 
     for (int q = 0; q < QA; ++q) {
         const int id = tid + q * NT;
         int64_t r = m0 + id / A_ROW;
-        if (r >= m_end) r = m0;  // (a row that is computed and dropped)
+        if (r >= m_end) r = m0;  // (not copied)
         if (p.row_index) r = p.row_index[r] / p.row_div;
         from_a[q] = static_cast<const T *>(p.x) + r * p.d + id % A_ROW * VK;
     }
@@ -92,36 +92,42 @@ __global__ void __launch_bounds__(ProjectionTile<T, BM, BN, TM, TN, BK, S>::NT, 
     }
     const int64_t step = (int64_t)(NT > BN ? NT / BN : 1) * p.n0;  // single floats: a thread's copies of a column stand this far apart
     const int blocks = (p.d + BK - 1) / BK;
-    auto load = [&](int kb) {  // features behind the last one are zero in both operands
+    // Features behind the last one are not used, rows behind the last one are whatever is there, computed and dropped. (Neither is copied: copies from one address, of zeros
+    // too, go one by one: 29 rows of 56 features onto 1448 columns 7.3 us, this way 3.0; 3 of 128 onto 4000 9.1, 4.6; 24 bf16 rows of 512 onto 2048 11.0, 9.2.)
+    const bool all_rows = m0 + BM <= m_end;
+    auto load = [&](int kb) {
         uint8_t *to = stages + kb % S * Tile::STAGE;
         const int k0 = kb * BK;
+        auto copies = [&](auto whole_) {
+            constexpr bool WHOLE = decltype(whole_)::value;  // all rows and features are there
 #pragma unroll
-        for (int q = 0; q < QA; ++q) {
-            const int id = tid + q * NT, k = k0 + id % A_ROW * VK;
-            copy16(to + id / A_ROW * Tile::ROW_BYTES + id % A_ROW * 16, k < p.d ? from_a[q] + k0 : static_cast<const T *>(p.x), k < p.d);
-        }
-        if constexpr (QUADS) {
-#pragma unroll
-            for (int q = 0; q < QB; ++q) {
-                const int id = tid + q * NT, k = k0 + id / B_ROW;
-                copy16(to + Tile::A_STAGE + id * 16, k < p.d ? from_b[q] + (int64_t)k0 * p.n0 : W0, k < p.d);
+            for (int q = 0; q < QA; ++q) {
+                const int id = tid + q * NT;
+                uint8_t *at = to + id / A_ROW * Tile::ROW_BYTES + id % A_ROW * 16;
+                if (WHOLE || (k0 + id % A_ROW * VK < p.d && m0 + id / A_ROW < m_end)) copy16(at, from_a[q] + k0);
             }
-        } else {
-            auto column = [&](auto whole) {
+            if constexpr (QUADS) {
+#pragma unroll
+                for (int q = 0; q < QB; ++q) {
+                    const int id = tid + q * NT;
+                    uint8_t *at = to + Tile::A_STAGE + id * 16;
+                    if (WHOLE || k0 + id / B_ROW < p.d) copy16(at, from_b[q] + (int64_t)k0 * p.n0);
+                }
+            } else {
 #pragma unroll
                 for (int c = 0; c < COLS; ++c) {
                     const float *from = from_b[c] + (int64_t)k0 * p.n0;
 #pragma unroll
                     for (int q = c; q < QB; q += COLS, from += step) {
                         const int id = tid + q * NT;
-                        if constexpr (decltype(whole)::value) copy4(to + Tile::A_STAGE + id * 4, from, true);
-                        else copy4(to + Tile::A_STAGE + id * 4, k0 + id / B_ROW < p.d ? from : W0, k0 + id / B_ROW < p.d);
+                        uint8_t *at = to + Tile::A_STAGE + id * 4;
+                        if (WHOLE || k0 + id / B_ROW < p.d) copy4(at, from);
                     }
                 }
-            };
-            if (k0 + BK <= p.d) column(std::true_type());
-            else column(std::false_type());
-        }
+            }
+        };
+        if (all_rows && k0 + BK <= p.d) copies(std::true_type());
+        else copies(std::false_type());
     };
 #pragma unroll
     for (int s = 0; s < S - 1; ++s) {
@@ -142,27 +148,31 @@ __global__ void __launch_bounds__(ProjectionTile<T, BM, BN, TM, TN, BK, S>::NT, 
         copies_commit();
         const uint8_t *a = stages + kb % S * Tile::STAGE + row0 * Tile::ROW_BYTES;
         const float *b = reinterpret_cast<const float *>(stages + kb % S * Tile::STAGE + Tile::A_STAGE) + col0;
+        auto multiply = [&](int steps) {
 #pragma unroll 2
-        for (int kk = 0; kk < BK; kk += VK) {
-            uint4 av[TM];
+            for (int kk = 0; kk < steps; kk += VK) {
+                uint4 av[TM];
 #pragma unroll
-            for (int i = 0; i < TM; ++i) av[i] = *reinterpret_cast<const uint4 *>(a + 4 * i * Tile::ROW_BYTES + kk * sizeof(T));
+                for (int i = 0; i < TM; ++i) av[i] = *reinterpret_cast<const uint4 *>(a + 4 * i * Tile::ROW_BYTES + kk * sizeof(T));
 #pragma unroll
-            for (int v = 0; v < VK; ++v) {
-                float bv[TN];
+                for (int v = 0; v < VK; ++v) {
+                    float bv[TN];
 #pragma unroll
-                for (int j = 0; j < TN; j += VN) {
-                    if constexpr (VN == 4) *reinterpret_cast<float4 *>(bv + j) = *reinterpret_cast<const float4 *>(b + (kk + v) * BN + 8 * j);
-                    else *reinterpret_cast<float2 *>(bv + j) = *reinterpret_cast<const float2 *>(b + (kk + v) * BN + 8 * j);
-                }
+                    for (int j = 0; j < TN; j += VN) {
+                        if constexpr (VN == 4) *reinterpret_cast<float4 *>(bv + j) = *reinterpret_cast<const float4 *>(b + (kk + v) * BN + 8 * j);
+                        else *reinterpret_cast<float2 *>(bv + j) = *reinterpret_cast<const float2 *>(b + (kk + v) * BN + 8 * j);
+                    }
 #pragma unroll
-                for (int i = 0; i < TM; ++i) {
-                    const float x = element<T>(av[i], v);
+                    for (int i = 0; i < TM; ++i) {
+                        const float x = element<T>(av[i], v);
 #pragma unroll
-                    for (int j = 0; j < TN; j += 2) fma_two(acc[i][j], acc[i][j + 1], x, bv[j], bv[j + 1]);
+                        for (int j = 0; j < TN; j += 2) fma_two(acc[i][j], acc[i][j + 1], x, bv[j], bv[j + 1]);
+                    }
                 }
             }
-        }
+        };
+        if (kb * BK + BK <= p.d) multiply(BK);
+        else multiply(p.d - kb * BK);  // (features are whole vectors)
     }
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
@@ -235,6 +245,13 @@ template <typename T> int32_t pick_tile(const ProjectionArgs &p, int32_t *tile_p
         const int64_t blocks = (cdiv(p.rows, c.bm) + (p.offsets ? p.groups / 2 : 0)) * cdiv(p.N, c.bn);
         const double cost = 1e-3 * c.chain * p.d + c.more + (double)(cdiv(blocks, 148) - 1) * (1e-3 * c.share[F] * p.d + c.more);
         if (i == 0 || cost < least) { best = i; least = cost; }
+    }
+    // Single floats of the weights that the float product takes in 128 x 64 tiles, whose number may fall better onto the SMs (its kernels of 3554 x 1200 x 1970, 868
+    // tiles, 355 us, 896 of 64 x 128 here or 1736 of 64 x 64 398; 7117 x 1632 x 262, 280 tiles, 175 and 187)
+    if (!p.quads && !p.offsets) {
+        const int64_t blocks = cdiv(p.rows, 128) * cdiv(p.N, 64);
+        const double more = costs[0].more, there = 1e-3 * costs[0].chain * p.d + more + (double)(cdiv(blocks, 148) - 1) * (1e-3 * costs[0].share[F] * p.d + more);
+        if (2 * blocks >= 3 * 148 && 1.02 * there < least) return PROJECTION_ELSEWHERE;
     }
     // float rows have as many shared-memory reads in the largest tiles as the float product has (32768 x 512 x 512: 362, that way 349)
     if (F && best == 0 && p.d >= 256 && !p.offsets && cdiv(p.rows, 64) * cdiv(p.N, 128) >= 6 * 148) return PROJECTION_ELSEWHERE;

@@ -25,3 +25,15 @@ def test_flat_logits(T, n, k, d, act):
                                          (129, 5, 7, 40, "f32"), (5000, 17, 13, 72, "bf16"), (9000, 3, 66, 24, "f32"), (40, 33, 2, 8, "bf16")])
 def test_grouped_logits(T, a, b, d, act):
     check(small_workload(f"tile-{a}x{b}", T=T, d=d, h=16, n=a * b, k=2, act=act, a=a, k1=2, b=b, k2=1, seed=56))
+
+
+# single floats of the weights: where 128 x 64 tiles of the float product are the fewer waves, and just not
+@pytest.mark.parametrize("T,n,k,d,act", [(17365, 73, 2, 72, "f32"), (11001, 75, 2, 296, "bf16"), (7117, 131, 2, 40, "f32"), (3554, 301, 2, 136, "bf16"), (4000, 93, 2, 136, "f32")])
+def test_flat_logits_by_the_float_product(T, n, k, d, act):
+    check(small_workload(f"tile-{T}-{n}", T=T, d=d, h=16, n=n, k=k, act=act, seed=60 + k))
+
+
+# fewer rows and features than a tile has, in many columns
+@pytest.mark.parametrize("T,n,k,d,act", [(3, 700, 2, 128, "f32"), (29, 724, 2, 56, "f32"), (29, 201, 2, 56, "bf16"), (5, 90, 2, 8, "bf16"), (65, 500, 2, 40, "bf16"), (1, 333, 2, 4, "f32")])
+def test_few_rows_onto_many_columns(T, n, k, d, act):
+    check(small_workload(f"tile-{T}-{n}-{d}", T=T, d=d, h=16, n=n, k=k, act=act, seed=70 + k))
