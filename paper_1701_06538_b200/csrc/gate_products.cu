@@ -157,22 +157,34 @@ __global__ void __launch_bounds__(WgradTile<T, BM, BN, TM, TN, BK, S>::NT, BLOCK
             rb[q] = k < count ? (p.perm ? p.perm[begin + k] : (int32_t)(begin + k)) : -1;
         }
     };
-    auto load = [&](int kb) {  // rows behind the last one are zero in both operands
+    // rows behind the last one are zero in both operands; features and logits behind the last ones are whatever is there, computed and dropped
+    const bool whole_tile = m_at + BM <= p.d && n_at + BN <= cols;
+    auto load = [&](int kb) {
         uint8_t *to = stages + kb % S * Tile::STAGE;
+        auto copies = [&](auto whole_) {
+            constexpr bool WHOLE = decltype(whole_)::value;
 #pragma unroll
-        for (int q = 0; q < QA; ++q) {
-            const int id = tid + q * NT, m = m_at + id % A_ROW * VK;
-            const bool live = ra[q] >= 0 && m < p.d;
-            copy16(to + id * 16, live ? static_cast<const T *>(p.x) + (int64_t)(ra[q] / p.row_div) * p.d + m : static_cast<const T *>(p.x), live);
-        }
+            for (int q = 0; q < QA; ++q) {
+                const int id = tid + q * NT, m = m_at + id % A_ROW * VK;
+                if (!WHOLE && m >= p.d) continue;
+                if (WHOLE || ra[q] >= 0) copy16(to + id * 16, static_cast<const T *>(p.x) + (int64_t)(ra[q] / p.row_div) * p.d + m);
+                else zero16(to + id * 16);
+            }
 #pragma unroll
-        for (int q = 0; q < QB; ++q) {
-            const int id = tid + q * NT, c = n_at + id % B_ROW * VB;
-            const bool live = rb[q] >= 0 && c < cols;
-            const float *from = live ? p.dlogit + (int64_t)rb[q] * cols + c : p.dlogit;
-            if (QUADS) copy16(to + Tile::A_STAGE + id * 16, from, live);
-            else copy4(to + Tile::A_STAGE + id * 4, from, live);
-        }
+            for (int q = 0; q < QB; ++q) {
+                const int id = tid + q * NT, c = n_at + id % B_ROW * VB;
+                if (!WHOLE && c >= cols) continue;
+                uint8_t *at = to + Tile::A_STAGE + id * 4 * VB;
+                const float *from = p.dlogit + (int64_t)rb[q] * cols + c;
+                if (WHOLE || rb[q] >= 0) {
+                    if (QUADS) copy16(at, from);
+                    else copy4(at, from);
+                } else if (QUADS) zero16(at);
+                else zero4(at);
+            }
+        };
+        if (whole_tile && (kb + 1) * BK <= count) copies(std::true_type());
+        else copies(std::false_type());
         fetch(kb + 1);
     };
     fetch(0);
@@ -275,7 +287,7 @@ template <typename T, int BM, int BN, int TM, int TN, int BK, int S, int BLOCKS>
 //   dW: 256 x 64 x 16 4.4 4.1, 15000 x 512 x 16 22.9 15.8 (64 x 16 tiles); 1000 x 512 x 24 6.2 4.4, 2085 x 256 x 32 6.3 4.6 (32 x 32, two warps);
 //       3001 x 320 x 40 9.2 7.3, 5000 x 512 x 32 11.5 9.2, 15000 x 128 x 72 17.7 15.5 (64 x 32); but 12000 x 256 x 128 26.8 28.6, 20000 x 1024 x 40 70 75
 //       single floats (rows of logits that are no multiple of sixteen bytes): that way twice at all sizes, 3000 x 128 x 14 11.1 4.2, 8192 x 512 x 94
-//       64 29, 60000 x 256 x 10 69 35, 15000 x 256 x 650 280 161, 32768 x 512 x 510 1119 529
+//       64 29, 60000 x 256 x 10 69 35, 15000 x 256 x 650 276 153, 5000 x 512 x 1970 582 309
 bool gate_rows_supported(const GateProduct &p) {
     const int32_t cols = p.W2 ? 2 * p.n : p.n;
     if (cdiv(p.d, 16) > 65535) return false;
@@ -299,8 +311,12 @@ int32_t launch_gate_wgrad(const GateProduct &p, float *part, cudaStream_t st, Ga
     const int32_t cols = p.W2 ? 2 * p.n : p.n, splits = simt_wgrad_splits(p.d, cols, p.groups, p.rows);
     auto run = [&](auto x) {
         using T = decltype(x);
+        // few features, of which a wider tile would mostly be empty; with few slices its warps are worth more. 32000 tokens x 8 x 72 logits 18.7 us, this way
+        // 9.5, 26346 x 16 x 40 12.0, 6.0; but 3000 x 16 x 80 3.8, 5.2
+        if (p.d <= 16 && !few_blocks(p, cols, splits))
+            return cols <= 16 ? launch_wgrad<T, 16, 16, 4, 2, 32, 4, 8>(p, splits, part, st) : launch_wgrad<T, 16, 32, 4, 4, 32, 4, 8>(p, splits, part, st);
         if (cols <= 16) return launch_wgrad<T, 64, 16, 4, 2, 32, 4, 4>(p, splits, part, st);
-        if (few_blocks(p, cols, splits)) return launch_wgrad<T, 32, 32, 4, 2, 32, 4, 4>(p, splits, part, st);
+        if (few_blocks(p, cols, splits) || p.d <= 32) return launch_wgrad<T, 32, 32, 4, 2, 32, 4, 4>(p, splits, part, st);
         return launch_wgrad<T, 64, 32, 4, 4, 32, 4, 4>(p, splits, part, st);
     };
     MOE_TRY(p.act == MOE_BF16 ? run(bf16()) : run(float()));

@@ -47,3 +47,9 @@ def test_flat_step(w):
 @pytest.mark.parametrize("w", HIER, ids=lambda w: w.name)
 def test_hierarchical_step(w):
     check_hier((w,) + oracle_cached(w) + (None, None), 0)
+
+
+# weight gradients of few features in many slices: 16 features, up to 32, and just above
+@pytest.mark.parametrize("T,d,n,act", [(26346, 16, 20, "f32"), (20001, 8, 21, "bf16"), (40000, 8, 4, "f32"), (33000, 12, 7, "f32"), (20000, 24, 20, "bf16"), (20000, 32, 19, "f32"), (20000, 36, 20, "f32")])
+def test_few_features(T, d, n, act):
+    check_flat(small_workload(f"gp-features-{T}-{d}-{n}", T=T, d=d, h=64, n=n, k=2, act=act, seed=140), 0)
