@@ -585,8 +585,8 @@ struct FloatCall {
 // 222, x 40 294, 216; 200 x 30 of 64 x 128 40.9, 45.9; 72 x 31 27.3, 29.3, x 40 39.7, 29.9; 400 x 40 of 64 x 64 57.5, 63.6. Small ones, by multiply-adds in
 // 1e6: 2.1 (4 x 64 of 64 x 128) 25.9, 26.9; 4.2 (16 x 64 of 64 x 64, 8 x 128 of 64 x 64) 25.8, 25.3 and 28.5, 27.5; 4.7 (8 x 36 of 64 x 256) 26.0, 28.8;
 // 6.3 (16 x 48 of 64 x 128) 30.3, 27.7; 8.4 (8 x 64 of 128 x 128) 27.9, 28.5, (16 x 64 of 64 x 128) 30.2, 27.6. A few tiles that are chains of many rows are the
-// exception: 1 x 20000 of 128 x 128 673, 820; 2 x 5000 205, 222; 4 x 5000 of 64 x 64 193, 228; 1 x 981 55.9, 60.9; but 1 x 512 40.4, 38.9; 1 x 3000 of 512 x 128
-// 160, 143; 19 x 2000 of 64 x 64 144, 131.
+// exception: 1 x 20000 of 128 x 128 673, 820; 2 x 5000 205, 222; 4 x 5000 of 64 x 64 193, 228; 1 x 981 55.9, 60.9; 27 experts, 34799 rows, the longest segment
+// 12894, of 64 x 64 444, 547; but 1 x 512 40.4, 38.9; equal loads of 19 x 2000 of 64 x 64 144, 131; 1 x 3000 of 512 x 128 160, 143.
 // The terms take 6 bytes of workspace a float: as much again as all other buffers of a backward call. At most 8 GiB of them, a twentieth of the memory, and 1 GiB
 // for callers that recompute hid to save memory. Larger layers keep the FP32 products, which take three and a half times as long (a backward call, ms: 8 experts x
 // 20000 rows of 1024 x 2048, 5.9 GB, by terms 15.1, by multiply-adds 53.3; 16 x 10000 of 1024 x 1024, 4.1 GB, 8.0 and 26.9).
@@ -596,7 +596,7 @@ bool tc_float_supported(const moe_config &c, bool backward) {
     if (6 * (backward ? 2 * (R * ((int64_t)c.d + c.h) + weights) : R * c.h + weights) > most) return false;  // (quads are numbered with 31 bits: far below)
     const double work = (double)R * c.d * c.h;
     if (!backward) return R > 64 * (int64_t)c.n && work >= 1.0e8 && (cdiv(R, F_TILE) + c.n / 2) * cdiv(c.d, F_TILE) >= 16;
-    if (weights < 16 * 64 * 64 && R >= 700 * (int64_t)c.n) return false;
+    if (weights < 32 * 64 * 64 && R >= 700 * (int64_t)c.n) return false;
     return R > 32 * (int64_t)c.n && work >= 4.0e6;
 }
 

@@ -6,6 +6,7 @@
 // asynchronous copies several K blocks ahead, rows of x as they lie: a thread reads its rows sixteen bytes along the features at a time (eight
 // features of a bf16 row, where a transposed float tile takes eight reads), so that the shared-memory reads, which with float tiles of both
 // operands took as long as the multiply-adds, leave these the pipes. `fma.rn.f32x2` does two columns with one instruction.
+#include <math.h>
 #include <string.h>
 
 #include <type_traits>
@@ -242,7 +243,9 @@ template <typename T> int32_t pick_tile(const ProjectionArgs &p, int32_t *tile_p
     double least = 0.0;
     for (int i = 0; i < 6; ++i) {
         const ProjectionCost &c = costs[i];
-        const int64_t blocks = (cdiv(p.rows, c.bm) + (p.offsets ? p.groups / 2 : 0)) * cdiv(p.N, c.bn);
+        // (tiles of groups: half a tile more each, and as much again as their number may exceed that: 1244 rows in 32 groups, 1648 x 234, 143 tiles by the halves alone,
+        // one wave, was two: 64 x 64 tiles, 143 us a call of moe_gate, 32 x 32 110)
+        const int64_t blocks = (cdiv(p.rows, c.bm) + (p.offsets ? p.groups / 2 + (int64_t)(0.5 * sqrt((double)p.groups)) : 0)) * cdiv(p.N, c.bn);
         const double cost = 1e-3 * c.chain * p.d + c.more + (double)(cdiv(blocks, 148) - 1) * (1e-3 * c.share[F] * p.d + c.more);
         if (i == 0 || cost < least) { best = i; least = cost; }
     }
