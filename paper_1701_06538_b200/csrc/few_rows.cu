@@ -66,8 +66,9 @@ template <int LC, int WARPS> __global__ void __launch_bounds__(32 * WARPS, WARPS
         const int chunks = (p.K + 31) / 32;
         auto fetch = [&](int c) {
             const int k = c * 32 + lane;
+            const float *__restrict__ from = a + k;
 #pragma unroll
-            for (int r = 0; r < RB; ++r) next[r] = r < t.rows && k < p.K ? a[(int64_t)r * p.K + k] : 0.0f;
+            for (int r = 0; r < RB; ++r, from += p.K) next[r] = r < t.rows && k < p.K ? *from : 0.0f;  // (one address: sixteen of them were spilled)
         };
         if (warp < chunks) fetch(warp);
         for (int c = warp; c < chunks; c += WARPS) {
