@@ -545,56 +545,56 @@ __global__ void __maxnreg__(most_registers(SET, WHOLE)) expert_products_kernel(c
                 // K-major tile and by 16 rows of 128 bytes in an MN-major one; the sum never leaves the address field
                 constexpr uint64_t a_step = a_mn ? (16 * 128) >> 4 : 32 >> 4, b_step = b_mn ? (16 * 128) >> 4 : 32 >> 4;
                 const int tail = wgrad ? (t.row_end - t.row0) - (kblocks - 1) * BK : BK;  // rows of the last block
-                constexpr bool IN_PARTS = !WHOLE && wgrad;  // a sum of SUM_BLOCKS K blocks at a time
-                for (int kb = 0; kb < kblocks; ++kb) {
-                    const bool begins = IN_PARTS ? kb % SUM_BLOCKS == 0 : kb == 0;
-                    if (begins) {
-                        ok = mbar_wait(tempty_bar(acc), acc_ph ^ 1u, abort_flag, P.status);
-                        if (!ok) return;
-                        tc_fence_after();
-                    }
-                    const uint32_t d_tmem = tmem_base + acc * BN;
-                    ok = mbar_wait(full_bar(s), ph, abort_flag, P.status);
-                    if (!ok) break;
+                // parts of SUM_BLOCKS K blocks, or one
+                const int part_blocks = !WHOLE && wgrad ? SUM_BLOCKS : kblocks;
+                for (int part = 0; part < kblocks; part += part_blocks) {
+                    ok = mbar_wait(tempty_bar(acc), acc_ph ^ 1u, abort_flag, P.status);
+                    if (!ok) return;
                     tc_fence_after();
-                    const uint32_t a_src = base + s * STAGE, b_src = a_src + A_BYTES;
-                    // K steps of 16 rows to issue for this block: none that lies behind the segment's end
-                    const int ksteps = kb < kblocks - 1 || (WHOLE && !wgrad) ? BK / 16 : wgrad ? (tail + 15) / 16 : p.last_steps;
-                    if (!PAIR && wgrad && kb == kblocks - 1 && !p.seg_a && ksteps * 16 > tail) {
-                        // Without the segments' own maps (see wgrad_uses_maps) the rows behind the end, up to the end of the step that holds
-                        // it, are the next segment's: zeroed in A AND in B (0 x finite = 0 would do for finite data; both keep a
-                        // non-finite value of the next segment out of this segment's sums): 128-B lines in all 64-column
-                        // chunks, the A tile's two chunks directly followed by the B tile's four. Eight lanes a line of one chunk,
-                        // four lines at a time (as one loop over all lines, with a division for each, this was 1450 cycles a tile of 64 rows)
-                        uint8_t *z = smem + s * STAGE + (tail + (lane >> 3)) * 128 + (lane & 7) * 16;
-                        for (int r = lane >> 3; r < ksteps * 16 - tail; r += 4, z += 4 * 128)
+                    const uint32_t d_tmem = tmem_base + acc * BN;
+                    const int part_end = !WHOLE && wgrad ? min(kblocks, part + SUM_BLOCKS) : kblocks;
+                    for (int kb = part; kb < part_end; ++kb) {
+                        ok = mbar_wait(full_bar(s), ph, abort_flag, P.status);
+                        if (!ok) break;
+                        tc_fence_after();
+                        const uint32_t a_src = base + s * STAGE, b_src = a_src + A_BYTES;
+                        // K steps of 16 rows to issue for this block: none that lies behind the segment's end
+                        const int ksteps = kb < kblocks - 1 || (WHOLE && !wgrad) ? BK / 16 : wgrad ? (tail + 15) / 16 : p.last_steps;
+                        if (!PAIR && wgrad && kb == kblocks - 1 && !p.seg_a && ksteps * 16 > tail) {
+                            // Without the segments' own maps (see wgrad_uses_maps) the rows behind the end, up to the end of the step that holds
+                            // it, are the next segment's: zeroed in A AND in B (0 x finite = 0 would do for finite data; both keep a
+                            // non-finite value of the next segment out of this segment's sums): 128-B lines in all 64-column
+                            // chunks, the A tile's two chunks directly followed by the B tile's four. Eight lanes a line of one chunk,
+                            // four lines at a time (as one loop over all lines, with a division for each, this was 1450 cycles a tile of 64 rows)
+                            uint8_t *z = smem + s * STAGE + (tail + (lane >> 3)) * 128 + (lane & 7) * 16;
+                            for (int r = lane >> 3; r < ksteps * 16 - tail; r += 4, z += 4 * 128)
 #pragma unroll
-                            for (int chunk = 0; chunk < (BM + BN) / 64; ++chunk)
-                                *reinterpret_cast<uint4 *>(z + chunk * (BK * 128)) = make_uint4(0, 0, 0, 0);
-                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                        __syncwarp();
-                    }
-                    if (PAIR || lane == 0) {
-                        const uint64_t ad = a_mn ? desc_mnmajor(a_src) : desc_kmajor(a_src), bd = b_mn ? desc_mnmajor(b_src) : desc_kmajor(b_src);
-#pragma unroll
-                        for (int k = 0; k < BK / 16; ++k) {
-                            if (k >= ksteps) break;
-                            if (PAIR) tc_mma2_bf16(d_tmem, ad + k * a_step, bd + k * b_step, idesc, (!begins || k > 0) ? 1u : 0u);
-                            else tc_mma_bf16(d_tmem, ad + k * a_step, bd + k * b_step, idesc, (!begins || k > 0) ? 1u : 0u);
+                                for (int chunk = 0; chunk < (BM + BN) / 64; ++chunk)
+                                    *reinterpret_cast<uint4 *>(z + chunk * (BK * 128)) = make_uint4(0, 0, 0, 0);
+                            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                            __syncwarp();
                         }
-                        if (PAIR) tc_commit2(empty_bar(s));  // the stage may be refilled once these MMAs have read it
-                        else tc_commit(empty_bar(s));
-                    }
-                    if (!PAIR) __syncwarp();
-                    if (++s == NST) { s = 0; ph ^= 1u; }
-                    if (IN_PARTS ? kb % SUM_BLOCKS == SUM_BLOCKS - 1 || kb == kblocks - 1 : kb == kblocks - 1) {  // accumulator complete
                         if (PAIR || lane == 0) {
-                            if (PAIR) tc_commit2(tfull_bar(acc));
-                            else tc_commit(tfull_bar(acc));
+                            const uint64_t ad = a_mn ? desc_mnmajor(a_src) : desc_kmajor(a_src), bd = b_mn ? desc_mnmajor(b_src) : desc_kmajor(b_src);
+#pragma unroll
+                            for (int k = 0; k < BK / 16; ++k) {
+                                if (k >= ksteps) break;
+                                if (PAIR) tc_mma2_bf16(d_tmem, ad + k * a_step, bd + k * b_step, idesc, (kb > part || k > 0) ? 1u : 0u);
+                                else tc_mma_bf16(d_tmem, ad + k * a_step, bd + k * b_step, idesc, (kb > part || k > 0) ? 1u : 0u);
+                            }
+                            if (PAIR) tc_commit2(empty_bar(s));  // the stage may be refilled once these MMAs have read it
+                            else tc_commit(empty_bar(s));
                         }
                         if (!PAIR) __syncwarp();
-                        if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
+                        if (++s == NST) { s = 0; ph ^= 1u; }
                     }
+                    if (ok && (PAIR || lane == 0)) {  // accumulator complete
+                        if (PAIR) tc_commit2(tfull_bar(acc));
+                        else tc_commit(tfull_bar(acc));
+                    }
+                    if (!PAIR) __syncwarp();
+                    if (!ok) return;
+                    if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
                 }
               });
             }
@@ -678,13 +678,12 @@ __global__ void __maxnreg__(most_registers(SET, WHOLE)) expert_products_kernel(c
                     }
                 };
                 const uint32_t mine = tmem_base + ((uint32_t)(quarter * 32) << 16) + half * (p.tile_n / 2);
-                auto store = [&](int u, const uint32_t (&v)[2][32]) {
+                auto begin = [&](int u) {  // box u, ahead of its loads
                     b.col0 = first + 64 * u;
                     b.next_bias = epi_bias(EPI) && u + 1 < boxes ? bias_at + 64 : nullptr;
                     b.keep = u ? keep[1] : keep[0];
                     b.box = boxes_at + (BOXES > 1 ? turn * 4096 : 0);
                     if (b.rows_valid >= 32) turn ^= 1;  // (else nothing is stored from the box)
-                    epilogue_box<EPI, BOXES, WHOLE>(p, lane, b, bias, v);
                 };
                 if constexpr (!WHOLE && wgrad) {  // sums of SUM_BLOCKS K blocks, added in registers: a box a warp
                     uint32_t v[2][32];
@@ -703,7 +702,10 @@ __global__ void __maxnreg__(most_registers(SET, WHOLE)) expert_products_kernel(c
                     }
 #pragma unroll
                     for (int j = 0; j < 64; ++j) v[j >> 5][j & 31] = __float_as_uint(sum[j >> 5][j & 31]);
-                    if (boxes > 0) store(0, v);
+                    if (boxes > 0) {
+                        begin(0);
+                        epilogue_box<EPI, BOXES, WHOLE>(p, lane, b, bias, v);
+                    }
                 } else {
                     if (have_acc) {  // (the loads above are in flight while the warp waits for its accumulator)
                         ok = mbar_wait(tfull_bar(acc), acc_ph, abort_flag, P.status);
@@ -712,6 +714,7 @@ __global__ void __maxnreg__(most_registers(SET, WHOLE)) expert_products_kernel(c
                     }
                     for (int u = 0; u < boxes; ++u) {
                         uint32_t v[2][32];
+                        begin(u);
                         if (have_acc) {
                             load_box(mine + acc * BN + 64 * u, v);
                             if (u + 1 == boxes) release();
@@ -719,7 +722,7 @@ __global__ void __maxnreg__(most_registers(SET, WHOLE)) expert_products_kernel(c
 #pragma unroll
                             for (int j = 0; j < 64; ++j) v[j >> 5][j & 31] = 0u;
                         }
-                        store(u, v);
+                        epilogue_box<EPI, BOXES, WHOLE>(p, lane, b, bias, v);
                     }
                     if (have_acc) {
                         if (boxes == 0) release();
