@@ -166,3 +166,29 @@ def test_a_forward_call_with_activations_near_the_least_float():
         r = slice(int(offsets[e]), int(offsets[e + 1]))
         exp = hid[r].double() @ W2[e].double()
         assert ((ys[r].double() - exp).abs() / (exp.abs() + exp.square().mean().sqrt())).max() <= 1e-5
+
+
+@pytest.mark.parametrize("d,h,scale", [(192, 320, 1), (64, 1024, 1), (448, 64, 3)])
+def test_rows_behind_a_segment_do_not_count(d, h, scale):
+    """Every segment is followed by one whose rows are infinite, in all operands: segments around the 16-row steps, 64-row blocks and 128-row tiles, in which the rows
+    behind the end are cleared in the three terms of both operands."""
+    counts = []
+    for c in ENDS:
+        counts += [c * scale, 3]
+    counts += [900, 3]
+    cfg, offsets, xs, dys, W1, b1, W2, b2, ws = layer(counts, d, h, d + h + 1)
+    n, R = len(counts), sum(counts)
+    hid = torch.relu(torch.randn(R, h, device="cuda", generator=torch.Generator(device="cuda").manual_seed(5)))
+    assert B.moe_query_sizes(cfg).ws_bwd_bytes > 12 * n * d * h  # the path
+    for e in range(1, n, 2):
+        r = slice(int(offsets[e]), int(offsets[e + 1]))
+        xs[r], dys[r], hid[r] = float("inf"), float("inf"), float("inf")
+    dxs, dW1, dW2 = backward(cfg, offsets, xs, hid, dys, W1, W2, ws)
+    for e in range(0, n, 2):
+        r = slice(int(offsets[e]), int(offsets[e + 1]))
+        x, dy, hd, w1, w2 = (t.double() for t in (xs[r], dys[r], hid[r], W1[e], W2[e]))
+        dz = (dy @ w2.t()) * (hd > 0)
+        for i, (got, exp) in enumerate(((dxs[r], dz @ w1.t()), (dW1[e], x.t() @ dz), (dW2[e], hd.t() @ dy))):
+            if exp.numel():
+                err = ((got.double() - exp).abs() / (exp.abs() + exp.square().mean().sqrt() + 1e-30)).max()
+                assert err <= 1e-5, (e, counts[e], i, float(err))  # the tolerance of the float layer
