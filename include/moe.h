@@ -117,7 +117,7 @@ typedef struct moe_ctx_layout {
     int64_t xs, perm, inv_perm, counts, offsets;                  /* moe_dispatch outputs */
     int64_t hid, ys;                                              /* moe_expert_ffn outputs */
     int64_t importance, load, losses;                             /* moe_losses outputs   */
-    int64_t relu_bits; /* bf16 layers on the tensor cores that keep hid: [R, h/32] uint32, bit set where hid > 0 (the
+    int64_t relu_bits; /* bf16 layers whose widths are multiples of 64 and that keep hid: [R, h/32] uint32, bit set where hid > 0 (the
                           backward's ReLU mask, read instead of hid); absent otherwise */
 } moe_ctx_layout;
 

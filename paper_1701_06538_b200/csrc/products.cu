@@ -51,7 +51,8 @@ constexpr int set_size(int set) { return set == SET_HID || set == SET_YS ? 1 : 2
 constexpr Kind set_kind(int set, int i) {
     return set == SET_HID || set == SET_YS ? ROW_BMN : (set == SET_DW1_DXS) == (i == 0) ? WGRAD : ROW_BK;
 }
-// Registers a thread: as few as do without spills, so that a launch's blocks find room beside the last ones of the launch before
+// Registers a thread: as few as do without spills (but for two words of ys on SM pairs), so that a launch's blocks find room beside the last ones of the launch
+// before; odd widths have running sums in registers besides
 constexpr int most_registers(int set, bool whole) { return !whole ? 168 : set == SET_HID || set == SET_YS ? 128 : 112; }
 constexpr Epilogue set_epilogue(int set, int i) {
     if (set == SET_HID) return EPI_BIAS_RELU;

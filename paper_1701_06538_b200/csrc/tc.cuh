@@ -199,12 +199,8 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
 __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// arrive on the barrier at this shared-memory offset in the EVEN CTA of the pair
-__device__ __forceinline__ void mbar_arrive_leader(uint32_t bar) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar & PEER_BIT_MASK) : "memory");
-}
-// The same without release semantics, for handing an accumulator buffer back: the tensor-memory reads are
-// complete (tcgen05.wait::ld) and fenced (tcgen05.fence::before_thread_sync) before the arrive, and nothing
+// Arrive on the barrier at this shared-memory offset in the EVEN CTA of the pair, without release semantics, for handing an accumulator buffer
+// back: the tensor-memory reads are complete (tcgen05.wait::ld) and fenced (tcgen05.fence::before_thread_sync) before the arrive, and nothing
 // the other side reads was written through memory. A release at cluster scope would wait here for all of this
 // thread's earlier global stores (the output rows) to reach L2, several thousand cycles per tile.
 __device__ __forceinline__ void mbar_arrive_leader_relaxed(uint32_t bar) {
