@@ -254,7 +254,8 @@ template <typename T> int32_t pick_tile(const ProjectionArgs &p, int32_t *tile_p
     if (!p.quads && !p.offsets) {
         const int64_t blocks = cdiv(p.rows, 128) * cdiv(p.N, 64);
         const double more = costs[0].more, there = 1e-3 * costs[0].chain * p.d + more + (double)(cdiv(blocks, 148) - 1) * (1e-3 * costs[0].share[F] * p.d + more);
-        if (2 * blocks >= 3 * 148 && 1.02 * there < least) return PROJECTION_ELSEWHERE;
+        // (float rows in 64 x 128 tiles take 2 % longer than there with as many waves: 6040 x 896 x 986 274 us, 268)
+        if (2 * blocks >= 3 * 148 && (F && best == 0 ? 1.0 : 1.02) * there <= least) return PROJECTION_ELSEWHERE;
     }
     // float rows have as many shared-memory reads in the largest tiles as the float product has (32768 x 512 x 512: 362, that way 349)
     if (F && best == 0 && p.d >= 256 && !p.offsets && cdiv(p.rows, 64) * cdiv(p.N, 128) >= 6 * 148) return PROJECTION_ELSEWHERE;
