@@ -378,9 +378,11 @@ template <bool PAIR, bool SHORT, int SET> struct TileRing {
 // Weight gradients of other widths than multiples of 64 are summed in tensor memory over 8 K blocks, 512 rows, and these sums added in registers: a tensor
 // core's accumulator drops low bits at every step of 16, over many rows more than the rounding of the result hides. Error of dW1 and dW2 against 64 bits (2-norms), as
 // sums of multiply-adds, in one accumulator and this way, in 1e-3: 60000 rows of 264 x 136 1.651 and 1.589, 1.653 and 1.596, 1.651 and 1.589; 400000 of 72 x 40 1.563
-// and 1.645, 1.705 and 1.947, 1.563 and 1.645. Tiles are 128 columns wide for it, a box a warp: a backward call of 4 experts x 15000 rows of 200 x 136 301 us, 226 this way;
-// 64 x 200 of 72 x 2056 108, 110; but 8 x 3750 of 1000 x 2008 609, 710 (by multiply-adds 9740).
+// and 1.645, 1.705 and 1.947, 1.563 and 1.645. A warp has the sums of one box, so a tile of a longer segment is done 128 columns at a time; where segments are that
+// long on average the tiles are that wide from the start. A backward call, us, in one accumulator and this way: 4 experts x 15000 rows of 200 x 136 301, 226; 64 x 200 of
+// 72 x 2056 107, 109; 8 x 3750 of 1000 x 2008 660, 724 (by multiply-adds 9750).
 constexpr int SUM_BLOCKS = 8;
+template <bool WHOLE, Kind KIND> __device__ __forceinline__ bool in_parts(const Tile &t) { return !WHOLE && KIND == WGRAD && t.row_end - t.row0 > SUM_BLOCKS * BK; }
 
 // PAIR: the two CTAs' shares of a tile
 template <bool PAIR> constexpr int tile_rows() { return PAIR ? 256 : 128; }
@@ -449,10 +451,11 @@ __global__ void __maxnreg__(most_registers(SET, WHOLE)) expert_products_kernel(c
             while (ok && tiles.next(t)) {
               with_product<SET>(t.prod, [&](auto I_) {
                 constexpr int I = decltype(I_)::value;
-                constexpr int KIND = set_kind(SET, I);
+                constexpr Kind KIND = set_kind(SET, I);
                 const Product &p = P.p[I];
                 const CUtensorMap *tm_a = &maps.a[I], *tm_b = &maps.b[I];
-                const uint32_t bytes = PAIR ? 2 * STAGE : A_BYTES + p.tile_n * BK * 2;
+                const int width = in_parts<WHOLE, KIND>(t) ? 128 : p.tile_n;  // columns of a pass over the contraction
+                const uint32_t bytes = PAIR ? 2 * STAGE : A_BYTES + width * BK * 2;
                 auto stage = [&](auto load) {  // load(A's place, B's place, barrier) of one K block
                     ok = mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, P.status);
                     if (!ok) return;
@@ -478,19 +481,24 @@ __global__ void __maxnreg__(most_registers(SET, WHOLE)) expert_products_kernel(c
                     const bool ragged = p.seg_a && (t.row_end - t.row0) % BK != 0;
                     if (ragged) { acquire_map(p.seg_a + t.e); acquire_map(p.seg_b + t.e); }
                     const int ca = t.m0 / 64 + 2 * (int)rank, cb = t.n0 / 64 + 2 * (int)rank;
-                    for (int kb = 0; kb < kblocks && ok; ++kb) {
-                        const bool tail = ragged && kb == kblocks - 1;
-                        const int r = t.row0 + kb * BK;
-                        stage([&](uint32_t a, uint32_t b, uint32_t bar) {
-                            if (WHOLE) {
-                                load_3d(a, tail ? p.seg_a + t.e : tm_a, bar, 0, r, ca);
-                                load_3d(b, tail ? p.seg_b + t.e : tm_b, bar, 0, r, cb);
-                            } else {
-                                for (int c = 0; c < BM / 64; ++c) tma_load_2d(a + c * (BK * 128), tm_a, bar, t.m0 + 64 * c, r);
-                                for (int c = 0; c < p.tile_n / 64; ++c) tma_load_2d(b + c * (BK * 128), tm_b, bar, t.n0 + 64 * c, r);
-                            }
-                        });
-                    }
+                    auto pass = [&](int32_t n0) {
+                        for (int kb = 0; kb < kblocks && ok; ++kb) {
+                            const bool tail = ragged && kb == kblocks - 1;
+                            const int r = t.row0 + kb * BK;
+                            stage([&](uint32_t a, uint32_t b, uint32_t bar) {
+                                if (WHOLE) {
+                                    load_3d(a, tail ? p.seg_a + t.e : tm_a, bar, 0, r, ca);
+                                    load_3d(b, tail ? p.seg_b + t.e : tm_b, bar, 0, r, cb);
+                                } else {
+                                    for (int c = 0; c < BM / 64; ++c) tma_load_2d(a + c * (BK * 128), tm_a, bar, t.m0 + 64 * c, r);
+                                    for (int c = 0; c < width / 64; ++c) tma_load_2d(b + c * (BK * 128), tm_b, bar, n0 + 64 * c, r);
+                                }
+                            });
+                        }
+                    };
+                    if constexpr (WHOLE) pass(t.n0);
+                    else
+                        for (int32_t n0 = t.n0; n0 < min(t.n0 + p.tile_n, p.N) && ok; n0 += width) pass(n0);
                 } else {
                     const int kblocks = p.kblocks, row = t.row0 + 128 * (int)rank;
                     if (p.seg_a && row + 128 > t.row_end) {
@@ -534,68 +542,77 @@ __global__ void __maxnreg__(most_registers(SET, WHOLE)) expert_products_kernel(c
             Tile t;
             while (ok && tiles.next(t)) {
               with_product<SET>(t.prod, [&](auto I_) {
-                constexpr int I = decltype(I_)::value, KIND = set_kind(SET, I);
+                constexpr int I = decltype(I_)::value;
+                constexpr Kind KIND = set_kind(SET, I);
                 constexpr bool wgrad = KIND == WGRAD;
                 const Product &p = P.p[I];
                 const int kblocks = wgrad ? (t.row_end - t.row0 + BK - 1) / BK : p.kblocks;
                 if (kblocks == 0) return;  // empty segment (WGRAD): the epilogue writes zeros
                 constexpr int a_mn = wgrad ? 1 : 0, b_mn = KIND == ROW_BK ? 0 : 1;
-                // one CTA: columns behind the output's are not computed
-                const uint32_t idesc = PAIR ? make_idesc2(a_mn, b_mn) : make_idesc(a_mn, b_mn, min(p.tile_n, WHOLE ? p.N - t.n0 : (p.N - t.n0 + 15) & ~15));
                 // a K step of 16 advances the start address (low descriptor bits, in 16-byte units) by 32 bytes in a
                 // K-major tile and by 16 rows of 128 bytes in an MN-major one; the sum never leaves the address field
                 constexpr uint64_t a_step = a_mn ? (16 * 128) >> 4 : 32 >> 4, b_step = b_mn ? (16 * 128) >> 4 : 32 >> 4;
                 const int tail = wgrad ? (t.row_end - t.row0) - (kblocks - 1) * BK : BK;  // rows of the last block
-                // parts of SUM_BLOCKS K blocks, or one
-                const int part_blocks = !WHOLE && wgrad ? SUM_BLOCKS : kblocks;
-                for (int part = 0; part < kblocks; part += part_blocks) {
-                    ok = mbar_wait(tempty_bar(acc), acc_ph ^ 1u, abort_flag, P.status);
-                    if (!ok) return;
-                    tc_fence_after();
-                    const uint32_t d_tmem = tmem_base + acc * BN;
-                    const int part_end = !WHOLE && wgrad ? min(kblocks, part + SUM_BLOCKS) : kblocks;
-                    for (int kb = part; kb < part_end; ++kb) {
-                        ok = mbar_wait(full_bar(s), ph, abort_flag, P.status);
-                        if (!ok) break;
+                const bool parts = in_parts<WHOLE, KIND>(t);
+                auto pass = [&](int32_t n0, int width) {
+                    // one CTA: columns behind the output's are not computed
+                    const uint32_t idesc = PAIR ? make_idesc2(a_mn, b_mn) : make_idesc(a_mn, b_mn, min(width, WHOLE ? p.N - n0 : (p.N - n0 + 15) & ~15));
+                    const int part_blocks = parts ? SUM_BLOCKS : kblocks;
+                    for (int part = 0; part < kblocks; part += part_blocks) {
+                        ok = mbar_wait(tempty_bar(acc), acc_ph ^ 1u, abort_flag, P.status);
+                        if (!ok) return;
                         tc_fence_after();
-                        const uint32_t a_src = base + s * STAGE, b_src = a_src + A_BYTES;
-                        // K steps of 16 rows to issue for this block: none that lies behind the segment's end
-                        const int ksteps = kb < kblocks - 1 || (WHOLE && !wgrad) ? BK / 16 : wgrad ? (tail + 15) / 16 : p.last_steps;
-                        if (!PAIR && wgrad && kb == kblocks - 1 && !p.seg_a && ksteps * 16 > tail) {
-                            // Without the segments' own maps (see wgrad_uses_maps) the rows behind the end, up to the end of the step that holds
-                            // it, are the next segment's: zeroed in A AND in B (0 x finite = 0 would do for finite data; both keep a
-                            // non-finite value of the next segment out of this segment's sums): 128-B lines in all 64-column
-                            // chunks, the A tile's two chunks directly followed by the B tile's four. Eight lanes a line of one chunk,
-                            // four lines at a time (as one loop over all lines, with a division for each, this was 1450 cycles a tile of 64 rows)
-                            uint8_t *z = smem + s * STAGE + (tail + (lane >> 3)) * 128 + (lane & 7) * 16;
-                            for (int r = lane >> 3; r < ksteps * 16 - tail; r += 4, z += 4 * 128)
+                        const uint32_t d_tmem = tmem_base + acc * BN;
+                        const int part_end = parts ? min(kblocks, part + SUM_BLOCKS) : kblocks;
+                        for (int kb = part; kb < part_end; ++kb) {
+                            ok = mbar_wait(full_bar(s), ph, abort_flag, P.status);
+                            if (!ok) break;
+                            tc_fence_after();
+                            const uint32_t a_src = base + s * STAGE, b_src = a_src + A_BYTES;
+                            // K steps of 16 rows to issue for this block: none that lies behind the segment's end
+                            const int ksteps = kb < kblocks - 1 || (WHOLE && !wgrad) ? BK / 16 : wgrad ? (tail + 15) / 16 : p.last_steps;
+                            if (!PAIR && wgrad && kb == kblocks - 1 && !p.seg_a && ksteps * 16 > tail) {
+                                // Without the segments' own maps (see wgrad_uses_maps) the rows behind the end, up to the end of the step that holds
+                                // it, are the next segment's: zeroed in A AND in B (0 x finite = 0 would do for finite data; both keep a
+                                // non-finite value of the next segment out of this segment's sums): 128-B lines in all 64-column
+                                // chunks, the A tile's two chunks directly followed by the B tile's four. Eight lanes a line of one chunk,
+                                // four lines at a time (as one loop over all lines, with a division for each, this was 1450 cycles a tile of 64 rows)
+                                uint8_t *z = smem + s * STAGE + (tail + (lane >> 3)) * 128 + (lane & 7) * 16;
+                                for (int r = lane >> 3; r < ksteps * 16 - tail; r += 4, z += 4 * 128)
 #pragma unroll
-                                for (int chunk = 0; chunk < (BM + BN) / 64; ++chunk)
-                                    *reinterpret_cast<uint4 *>(z + chunk * (BK * 128)) = make_uint4(0, 0, 0, 0);
-                            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                            __syncwarp();
-                        }
-                        if (PAIR || lane == 0) {
-                            const uint64_t ad = a_mn ? desc_mnmajor(a_src) : desc_kmajor(a_src), bd = b_mn ? desc_mnmajor(b_src) : desc_kmajor(b_src);
-#pragma unroll
-                            for (int k = 0; k < BK / 16; ++k) {
-                                if (k >= ksteps) break;
-                                if (PAIR) tc_mma2_bf16(d_tmem, ad + k * a_step, bd + k * b_step, idesc, (kb > part || k > 0) ? 1u : 0u);
-                                else tc_mma_bf16(d_tmem, ad + k * a_step, bd + k * b_step, idesc, (kb > part || k > 0) ? 1u : 0u);
+                                    for (int chunk = 0; chunk < (BM + BN) / 64; ++chunk)
+                                        *reinterpret_cast<uint4 *>(z + chunk * (BK * 128)) = make_uint4(0, 0, 0, 0);
+                                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                                __syncwarp();
                             }
-                            if (PAIR) tc_commit2(empty_bar(s));  // the stage may be refilled once these MMAs have read it
-                            else tc_commit(empty_bar(s));
+                            if (PAIR || lane == 0) {
+                                const uint64_t ad = a_mn ? desc_mnmajor(a_src) : desc_kmajor(a_src), bd = b_mn ? desc_mnmajor(b_src) : desc_kmajor(b_src);
+#pragma unroll
+                                for (int k = 0; k < BK / 16; ++k) {
+                                    if (k >= ksteps) break;
+                                    if (PAIR) tc_mma2_bf16(d_tmem, ad + k * a_step, bd + k * b_step, idesc, (kb > part || k > 0) ? 1u : 0u);
+                                    else tc_mma_bf16(d_tmem, ad + k * a_step, bd + k * b_step, idesc, (kb > part || k > 0) ? 1u : 0u);
+                                }
+                                if (PAIR) tc_commit2(empty_bar(s));  // the stage may be refilled once these MMAs have read it
+                                else tc_commit(empty_bar(s));
+                            }
+                            if (!PAIR) __syncwarp();
+                            if (++s == NST) { s = 0; ph ^= 1u; }
+                        }
+                        if (ok && (PAIR || lane == 0)) {  // accumulator complete
+                            if (PAIR) tc_commit2(tfull_bar(acc));
+                            else tc_commit(tfull_bar(acc));
                         }
                         if (!PAIR) __syncwarp();
-                        if (++s == NST) { s = 0; ph ^= 1u; }
+                        if (!ok) return;
+                        if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
                     }
-                    if (ok && (PAIR || lane == 0)) {  // accumulator complete
-                        if (PAIR) tc_commit2(tfull_bar(acc));
-                        else tc_commit(tfull_bar(acc));
-                    }
-                    if (!PAIR) __syncwarp();
-                    if (!ok) return;
-                    if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
+                };
+                if constexpr (WHOLE || !wgrad) {
+                    pass(t.n0, p.tile_n);
+                } else {
+                    const int width = parts ? 128 : p.tile_n;
+                    for (int32_t n0 = t.n0; n0 < min(t.n0 + p.tile_n, p.N) && ok; n0 += width) pass(n0, width);
                 }
               });
             }
@@ -686,26 +703,29 @@ __global__ void __maxnreg__(most_registers(SET, WHOLE)) expert_products_kernel(c
                     b.box = boxes_at + (BOXES > 1 ? turn * 4096 : 0);
                     if (b.rows_valid >= 32) turn ^= 1;  // (else nothing is stored from the box)
                 };
-                if constexpr (!WHOLE && wgrad) {  // sums of SUM_BLOCKS K blocks, added in registers: a box a warp
-                    uint32_t v[2][32];
-                    float sum[2][32];
+                if (in_parts<WHOLE, set_kind(SET, I)>(t)) {  // sums of SUM_BLOCKS K blocks, added in registers: a box a warp and 128 columns
+                    for (int32_t n0 = t.n0; n0 < min(t.n0 + p.tile_n, p.N); n0 += 128) {
+                        uint32_t v[2][32];
+                        float sum[2][32];
 #pragma unroll
-                    for (int j = 0; j < 64; ++j) sum[j >> 5][j & 31] = 0.0f;
-                    for (int r = t.row0; r < t.row_end; r += SUM_BLOCKS * BK) {
-                        ok = mbar_wait(tfull_bar(acc), acc_ph, abort_flag, P.status);
-                        if (!ok) return;
-                        tc_fence_after();
-                        load_box(mine + acc * BN, v);
-                        release();
+                        for (int j = 0; j < 64; ++j) sum[j >> 5][j & 31] = 0.0f;
+                        for (int r = t.row0; r < t.row_end; r += SUM_BLOCKS * BK) {
+                            ok = mbar_wait(tfull_bar(acc), acc_ph, abort_flag, P.status);
+                            if (!ok) return;
+                            tc_fence_after();
+                            load_box(tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + half * 64, v);
+                            release();
 #pragma unroll
-                        for (int j = 0; j < 64; ++j) sum[j >> 5][j & 31] += __uint_as_float(v[j >> 5][j & 31]);
-                        if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
-                    }
+                            for (int j = 0; j < 64; ++j) sum[j >> 5][j & 31] += __uint_as_float(v[j >> 5][j & 31]);
+                            if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
+                        }
 #pragma unroll
-                    for (int j = 0; j < 64; ++j) v[j >> 5][j & 31] = __float_as_uint(sum[j >> 5][j & 31]);
-                    if (boxes > 0) {
-                        begin(0);
-                        epilogue_box<EPI, BOXES, WHOLE>(p, lane, b, bias, v);
+                        for (int j = 0; j < 64; ++j) v[j >> 5][j & 31] = __float_as_uint(sum[j >> 5][j & 31]);
+                        if (n0 + half * 64 < p.N) {
+                            begin(0);
+                            b.col0 = n0 + half * 64;
+                            epilogue_box<EPI, BOXES, WHOLE>(p, lane, b, bias, v);
+                        }
                     }
                 } else {
                     if (have_acc) {  // (the loads above are in flight while the warp waits for its accumulator)
@@ -867,7 +887,7 @@ class ProductList {
     int32_t wgrad(const void *A, const void *B, int32_t M, int32_t N, void *out, SegmentMap seg_a, SegmentMap seg_b) {
         Product &p = P.p[count];
         p.N = N; p.M = M;
-        p.tile_n = whole(c) ? BN : 128;  // (a box a warp, see SUM_BLOCKS)
+        p.tile_n = whole(c) || R < SUM_BLOCKS * BK * (int64_t)c.n ? BN : 128;  // (see SUM_BLOCKS)
         p.tiles_n = (int32_t)cdiv(N, p.tile_n); p.per_e = (int32_t)cdiv(M, tm) * p.tiles_n;
         p.by_tiles_n = Divisor::of(p.tiles_n); p.by_per_e = Divisor::of(p.per_e);
         p.out = (bf16 *)out;

@@ -22,12 +22,14 @@ def test_fused_step(flags):
     check_flat(small_workload("odd-widths", T=1100, d=104, h=280, n=6, k=2, act="bf16", seed=121), flags)
 
 
-@pytest.mark.parametrize("rows,d,h", [(400000, 72, 40), (511, 40, 72), (512, 40, 136), (513, 136, 40), (1025, 264, 200), (150000, 200, 264)])
-def test_long_weight_gradients_are_rounded_once(rows, d, h):
+@pytest.mark.parametrize("rows,d,h,short", [(400000, 72, 40, 1), (511, 40, 72, 1), (512, 40, 136, 1), (513, 136, 40, 1), (1025, 264, 200, 1), (150000, 200, 264, 1),
+                                            # few rows an expert on average: tiles 256 columns wide, of the long segment in two halves
+                                            (40000, 264, 392, 100), (513, 520, 136, 9), (1024, 136, 120, 9)])
+def test_long_weight_gradients_are_rounded_once(rows, d, h, short):
     """dW1 and dW2 of odd widths over many rows: as far from 64 bits as the rounding to bf16 alone is, within 2 %. (The operands' means are not 0: sums that grow row
     by row are what a tensor core's accumulator drops bits of; summed in one, 400000 rows were off by 1.18 times that. Sums begin anew every 512 rows.)"""
-    n = 2
-    counts = [rows, 3]
+    counts = [rows] + [3] * short
+    n = len(counts)
     R = sum(counts)
     cfg = B.make_config(R, d, h, n, 1, "bf16")
     g = torch.Generator(device="cuda").manual_seed(rows)
